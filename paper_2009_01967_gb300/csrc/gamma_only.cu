@@ -152,7 +152,9 @@ __global__ void g_gamma_kernel(int nb, int n_part, const double *__restrict__ pa
 }
 
 // Degenerate averaging for one system of any size: ranks by frequency
-// (ties by index), then one thread walks the chains |d nu| < tol.
+// (ties by index), then the thread of each chain's first mode averages the
+// chain |d nu| < tol in ascending order (one thread walking the whole list
+// took 0.17 ms for 768 modes).
 __global__ void g_rank_kernel(int nb, const double *__restrict__ nu, int *__restrict__ order) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= nb) return;
@@ -163,19 +165,15 @@ __global__ void g_rank_kernel(int nb, const double *__restrict__ nu, int *__rest
 }
 __global__ void g_degen_kernel(int nb, const double *__restrict__ nu, const int *__restrict__ order,
                                double tol, double *__restrict__ gamma) {
-    if (blockIdx.x != 0 || threadIdx.x != 0) return;
-    int start = 0;
-    for (int a = 1; a <= nb; ++a) {
-        if (a == nb || nu[order[a]] - nu[order[a - 1]] >= tol) {
-            if (a - start > 1) {
-                double t = 0.0;
-                for (int b = start; b < a; ++b) t += gamma[order[b]];
-                t /= (double)(a - start);
-                for (int b = start; b < a; ++b) gamma[order[b]] = t;
-            }
-            start = a;
-        }
-    }
+    const int a = blockIdx.x * blockDim.x + threadIdx.x;
+    if (a >= nb || (a > 0 && !(nu[order[a]] - nu[order[a - 1]] >= tol))) return;      // a starts no chain
+    int end = a + 1;
+    while (end < nb && !(nu[order[end]] - nu[order[end - 1]] >= tol)) ++end;
+    if (end - a < 2) return;
+    double t = 0.0;
+    for (int b = a; b < end; ++b) t += gamma[order[b]];
+    t /= (double)(end - a);
+    for (int b = a; b < end; ++b) gamma[order[b]] = t;
 }
 
 template <typename R>
@@ -246,7 +244,7 @@ cudaError_t launch_gamma_only(const GammaPlan &gp, const GammaDev &d, const LwPa
         g_gamma_kernel<<<counted((nb + 127) / 128), 128, 0, st>>>(nb, gp.n_part, d.partial, d.omega, pref, gamma_out);
     }
     g_rank_kernel<<<counted((nb + 127) / 128), 128, 0, st>>>(nb, d.nu, d.order);
-    g_degen_kernel<<<counted(1), 32, 0, st>>>(nb, d.nu, d.order, degen_tol_thz, gamma_out);
+    g_degen_kernel<<<counted((nb + 127) / 128), 128, 0, st>>>(nb, d.nu, d.order, degen_tol_thz, gamma_out);
     return cudaGetLastError();
 }
 

@@ -399,6 +399,20 @@ kald_status plan_system(kald_ctx *ctx, const kald_system *s, HostSystem &h) {
         h.fc3_rk[t] = rep_of(x + 6);
     }
     h.pair3_start.push_back(n3);
+    // two stable counting sorts of the (j, k) sorted groups: by k, then by class
+    const int ng = (int)h.pair3_j.size();
+    auto len_class = [&](int g) {
+        const int len = h.pair3_start[g + 1] - h.pair3_start[g];
+        return len > kYLong ? 0 : kYLong + 1 - len;
+    };
+    const std::vector<int> by_k = stable_key_order(ng, n, [&](int g) { return (long long)h.pair3_k[g]; });
+    const std::vector<int> by_class = stable_key_order(ng, kYLong + 1, [&](int x) { return (long long)len_class(by_k[x]); });
+    h.pair3_order.resize(ng);
+    h.pair3_long = 0;
+    for (int x = 0; x < ng; ++x) {
+        h.pair3_order[x] = by_k[by_class[x]];
+        h.pair3_long += len_class(h.pair3_order[x]) == 0;
+    }
     h.n_rep = n_rep;
     return KALD_OK;
 }
@@ -970,6 +984,7 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
         const size_t nn = (size_t)nb * nb;
         GammaPlan &gp = it.gp;
         gp.n_groups = (int)h.pair3_j.size();
+        gp.n_fc3 = h.fc3_i.size();
         gp.n_part = std::max(1, 2 * ctx->sm_count);
         gp.sms = std::max(1, ctx->sm_count);
         gp.omega_h.resize(nb);
@@ -982,6 +997,7 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
         if (mode == KALD_BF16_SPLIT) {
             if (h.fc3_symmetric < 0) h.fc3_symmetric = fc3_symmetric_last_two(&sys[it.x]) ? 1 : 0;
             gp.symmetric = h.fc3_symmetric;
+            gp.n_long = h.pair3_long;
             band_tiles(gp.omega_h, tc_tile(), opt->n_sigma * kTwoPi * opt->sigma_thz, gp.symmetric, gp.tiles,
                        gp.tile_start);
         }
@@ -990,7 +1006,7 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
                    scaled_bytes(h.fc3_blk, h.fc3_atoms, h, 27, 27, 0) + 2 * ws_round(sizeof(double) * nb) +
                    ws_round(sizeof(int) * nb);
         if (mode == KALD_BF16_SPLIT)
-            b += tc_gamma_scratch_bytes(nb, ctx->sm_count) + ws_round(sizeof(int2) * n_tiles + sizeof(int) * (nb + 1)) +
+            b += tc_gamma_scratch_bytes(nb, ctx->sm_count, gp.n_fc3) + bytes_of(h.pair3_order) + ws_round(sizeof(int2) * n_tiles + sizeof(int) * (nb + 1)) +
                  ws_round(sizeof(double) * n_tiles);
         else
             b += 4 * ws_round(rs * nn) + ws_round(sizeof(double) * nb * (size_t)gp.n_part);
@@ -1023,9 +1039,11 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
         gd.occ = static_cast<double *>(ws_take(ctx, sizeof(double) * nb));
         gd.E = gd.Y = gd.T = gd.PHI = nullptr;
         gd.partial = nullptr;
+        gd.group_order = nullptr;
         gd.tc_scratch = nullptr; gd.tiles_dev = nullptr; gd.partial_tc = nullptr;
         if (mode == KALD_BF16_SPLIT) {
-            gd.tc_scratch = ws_take(ctx, tc_gamma_scratch_bytes(nb, ctx->sm_count));
+            gd.tc_scratch = ws_take(ctx, tc_gamma_scratch_bytes(nb, ctx->sm_count, it.gp.n_fc3));
+            gd.group_order = upload(ctx, h.pair3_order);
             gd.tiles_dev = static_cast<int2 *>(ws_take(ctx, sizeof(int2) * n_tiles + sizeof(int) * (nb + 1)));
             gd.partial_tc = static_cast<double *>(ws_take(ctx, sizeof(double) * n_tiles));
         } else {

@@ -119,6 +119,9 @@ inline size_t ws_round(size_t b) { return (b + 255) & ~size_t(255); }
 // Pointer kind: true if `p` is device (or managed) memory usable on ctx->device.
 bool is_device_ptr(const void *p);
 
+// (j, k) groups of more blocks than this take a warp each in the Gamma-only Y build.
+constexpr int kYLong = 8;
+
 // ---- host-side plan of a system ---------------------------------------------
 struct HostSystem {
     int n_atoms = 0;
@@ -135,6 +138,10 @@ struct HostSystem {
     std::vector<double> fc2_dist;                      // [n_fc2][3] x_i - x_j - R
     // fc3 grouped by (j, k) atom pair (CSR over output pairs)
     std::vector<int> pair3_j, pair3_k, pair3_start;
+    // the groups of more than kYLong blocks first, then by falling length, each
+    // class ordered by (k, j) (the Y build of the Gamma-only tensor-core path)
+    std::vector<int> pair3_order;
+    int pair3_long = 0;
     std::vector<int> fc3_i, fc3_rj, fc3_rk;            // per block (sorted order)
     std::vector<double> fc3_blk;                       // [n_fc3][27] Phi3 (eV/A^3), grouped, not mass-scaled
     std::vector<int> fc3_atoms;                        // [n_fc3][3] (i, j, k) of each block
@@ -280,6 +287,8 @@ cudaError_t launch_mode_prep(int n, const double *nu, double omega_min_w, double
 // gamma_only.cu: Gamma-only linewidths of a system with nb > kMaxNbSmall
 struct GammaPlan {
     int n_groups = 0;
+    int n_long = 0;                  // groups with a warp of their own in the tensor-core path's Y build
+    size_t n_fc3 = 0;                // fc3 blocks
     int n_part = 0;                  // epilogue CTAs (partial sums) per mode
     std::vector<double> omega_h;     // [nb] rad/ps, 0 for a masked mode
     // tensor-core path: delta-band tiles (tm, tn) of each mode, CSR by mode
@@ -291,6 +300,7 @@ struct GammaPlan {
 };
 struct GammaDev {
     const int *group_jk, *group_start, *blk_i;   // (j, k) groups of fc3 blocks
+    const int *group_order;          // HostSystem::pair3_order (tensor-core path)
     const double *fc3;               // [n_fc3][27] Phi3 / sqrt(mi mj mk)
     const double2 *eig;              // [nb][nb] (real parts used)
     const double *nu;                // [nb] THz
@@ -315,7 +325,7 @@ int tune_gamma_batch(const GammaPlan &gp, const GammaDev &d, const LwParams &p, 
 // modes per launch of the tensor-core Gamma-only path and its scratch bytes
 int tc_gamma_batch(int nb, int sms);
 int tc_gamma_batch_max(int nb, int sms);
-size_t tc_gamma_scratch_bytes(int nb, int sms);
+size_t tc_gamma_scratch_bytes(int nb, int sms, size_t n_fc3);
 int tc_tile(void);
 cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const LwParams &p, void *scratch,
                                  const std::vector<int2> &tiles, const std::vector<int> &tile_start,

@@ -29,6 +29,8 @@
 
 #include <algorithm>
 #include <cmath>
+#include <utility>
+#include <vector>
 
 #include "kald_internal.h"
 #include "tc_common.cuh"
@@ -299,31 +301,113 @@ __global__ void split_kernel(int rows, int cols, const SRC *__restrict__ src, si
     }
 }
 
-// YT[c][b] of mode mu0 + blockIdx.y straight into its BF16 hi/lo planes
-// (plane stride plane_elems; FP64 sums).
-__global__ void ybuild_bf16_kernel(int n_groups, const int *__restrict__ group_jk,
-                                   const int *__restrict__ group_start, const int *__restrict__ blk_i,
-                                   const double *__restrict__ fc3, const double2 *__restrict__ eig, int nb,
-                                   int mu0, int ld, size_t plane_elems, __nv_bfloat16 *__restrict__ hi,
-                                   __nv_bfloat16 *__restrict__ lo) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n_groups * 9) return;
-    const double2 *eig_mu = eig + (size_t)(mu0 + blockIdx.y) * nb;
-    hi += blockIdx.y * plane_elems;
-    lo += blockIdx.y * plane_elems;
-    const int g = e / 9, bg = e % 9;
-    const int j = group_jk[2 * g], k = group_jk[2 * g + 1];
-    double acc = 0.0;
-    for (int bl = group_start[g]; bl < group_start[g + 1]; ++bl) {
-        const int i = blk_i[bl];
-        const double *f = fc3 + (size_t)27 * bl + bg;
-        acc += f[0] * eig_mu[3 * i].x + f[9] * eig_mu[3 * i + 1].x + f[18] * eig_mu[3 * i + 2].x;
+// FP32 pairs (hi, lo) of the scaled Phi3 blocks, 27 per block.
+__global__ void fc3_pair_kernel(size_t n, const double *__restrict__ src, float2 *__restrict__ out) {
+    for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < n; x += (size_t)gridDim.x * blockDim.x) {
+        const F2 v = f2_of(src[x]);
+        out[x] = make_float2(v.h, v.l);
     }
-    const float v = (float)acc;
-    const __nv_bfloat16 h = __float2bfloat16_rn(v);
+}
+// FP32 pairs of the eigenvectors with the modes contiguous: Et[d][mu], row
+// length ldm (32 x 32 tiles through shared memory).
+__global__ void __launch_bounds__(256)
+eig_pair_kernel(int nb, const double2 *__restrict__ eig, int ldm, float2 *__restrict__ Et) {
+    __shared__ float2 tile[32][33];
+    const int d0 = blockIdx.x * 32, m0 = blockIdx.y * 32;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    for (int r = ty; r < 32; r += 8)
+        if (m0 + r < nb && d0 + tx < nb) {
+            const F2 v = f2_of(eig[(size_t)(m0 + r) * nb + d0 + tx].x);
+            tile[r][tx] = make_float2(v.h, v.l);
+        }
+    __syncthreads();
+    for (int r = ty; r < 32; r += 8)
+        if (d0 + r < nb && m0 + tx < nb) Et[(size_t)(d0 + r) * ldm + m0 + tx] = tile[tx][r];
+}
+
+// acc += a b for FP32 pairs: the product to about 2^-46 of itself (FMA
+// residual plus the cross terms), the sum by Knuth's two-sum.
+__device__ __forceinline__ void pair_fma(F2 &acc, float2 a, float2 b) {
+    const float p = __fmul_rn(a.x, b.x);
+    float e = __fmaf_rn(a.x, b.x, -p);
+    e = __fmaf_rn(a.x, b.y, e);
+    e = __fmaf_rn(a.y, b.x, e);
+    const float s = __fadd_rn(acc.h, p);
+    const float v = __fsub_rn(s, acc.h);
+    const float r = __fadd_rn(__fsub_rn(acc.h, __fsub_rn(s, v)), __fsub_rn(p, v));
+    acc.h = s;
+    acc.l = __fadd_rn(acc.l, __fadd_rn(r, e));
+}
+
+// YT[c][b] of modes mu0 .. mu0 + nm - 1 straight into their BF16 hi/lo planes
+// (plane stride plane_elems).  Sums of FP32 pairs (about 46 bits), rounded
+// once to FP32 and then split.
+//
+// Bound: FP64 units.  As plain FP64 sums (one thread per output and mode, 2
+// FP64 FMA per clock and SM) this build took 173 us per launch of 18 modes of a 768-mode
+// cell, three times both GEMMs together; a pair FMA is 12 FP32 operations
+// against the 64 that one FP64 FMA costs here.  A thread takes MT modes
+// of one output, so a block's values are read once for all of them and the
+// modes of an eigenvector component are contiguous.  Groups come longest
+// first (order): the n_long longest -- the atoms paired with themselves hold
+// one block per neighbour where the others hold two or three -- take a warp
+// each, three lanes per output, so that they do not serialise the launch.
+template <int MT>
+__global__ void __launch_bounds__(256)
+ybuild_pair_kernel(int n_groups, int n_long, const int *__restrict__ order, const int *__restrict__ group_jk,
+                   const int *__restrict__ group_start, const int *__restrict__ blk_i,
+                   const float2 *__restrict__ fc3, const float2 *__restrict__ Et, int ldm, int mu0, int nm, int ld,
+                   size_t plane_elems, __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo) {
+    const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    const int m0 = blockIdx.y * MT;
+    const bool lng = gw < n_long;                      // uniform over the warp
+    const int t = lng ? 0 : (gw - n_long) * 32 + lane;
+    const int gi = lng ? gw : n_long + t / 9;
+    const int bg = lng ? lane % 9 : t % 9;
+    const bool act = gi < n_groups && (!lng || lane < 27);
+    const int g = act ? order[gi] : 0;
+    F2 acc[MT];
+#pragma unroll
+    for (int m = 0; m < MT; ++m) acc[m] = F2{0.f, 0.f};
+    if (act) {
+        const int b1 = group_start[g + 1], step = lng ? 3 : 1;
+#pragma unroll 2
+        for (int bl = group_start[g] + (lng ? lane / 9 : 0); bl < b1; bl += step) {
+            const float2 *e = Et + (size_t)(3 * __ldg(blk_i + bl)) * ldm + mu0 + m0;
+            const float2 *f = fc3 + (size_t)27 * bl + bg;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const float2 v = __ldg(f + 9 * a);
+#pragma unroll
+                for (int m = 0; m < MT; ++m) pair_fma(acc[m], v, __ldg(e + (size_t)a * ldm + m));
+            }
+        }
+    }
+    if (lng) {
+        // the three lanes of an output, in order
+#pragma unroll
+        for (int m = 0; m < MT; ++m) {
+            F2 p[2];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                p[k].h = __shfl_down_sync(0xffffffffu, acc[m].h, 9 * (k + 1));
+                p[k].l = __shfl_down_sync(0xffffffffu, acc[m].l, 9 * (k + 1));
+            }
+            acc[m] = f2_add(f2_add(acc[m], p[0]), p[1]);
+        }
+    }
+    if (!act || (lng && lane >= 9)) return;
+    const int j = group_jk[2 * g], k = group_jk[2 * g + 1];
     const size_t off = (size_t)(3 * k + bg % 3) * ld + 3 * j + bg / 3;
-    hi[off] = h;
-    lo[off] = __float2bfloat16_rn(v - __bfloat162float(h));
+#pragma unroll
+    for (int m = 0; m < MT; ++m) {
+        if (m0 + m >= nm) break;
+        const float v = __fadd_rn(acc[m].h, acc[m].l);
+        const __nv_bfloat16 h = __float2bfloat16_rn(v);
+        const size_t o = (size_t)(m0 + m) * plane_elems + off;
+        hi[o] = h;
+        lo[o] = __float2bfloat16_rn(v - __bfloat162float(h));
+    }
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -372,12 +456,19 @@ int tc_gamma_batch(int nb, int sms) {
 // Largest modes per launch the autotuner may choose (twice the default, at most 32).
 int tc_gamma_batch_max(int nb, int sms) { return std::max(1, std::min({2 * tc_gamma_batch(nb, sms), 32, nb})); }
 
-size_t tc_gamma_scratch_bytes(int nb, int sms) {
+// Modes per row of the transposed eigenvector pairs (the Y build reads up to
+// three modes past the last one).
+static int tc_ldm(int nb) { return (nb + 3 + 31) / 32 * 32; }
+
+size_t tc_gamma_scratch_bytes(int nb, int sms, size_t n_fc3) {
     const int ld = (nb + kBN - 1) / kBN * kBN;     // whole 128-column tiles per row
     const int rows = (nb + kBM - 1) / kBM * kBM;
     const size_t plane = ws_round(sizeof(__nv_bfloat16) * (size_t)rows * ld);
     // E hi/lo, then Y hi, Y lo, T hi, T lo of every mode of a batch (the largest batch)
-    return (2 + 4 * (size_t)tc_gamma_batch_max(nb, sms)) * plane + ws_round(sizeof(int) * 4);
+    // then the FP32 pairs of Phi3 and of the eigenvectors
+    return (2 + 4 * (size_t)tc_gamma_batch_max(nb, sms)) * plane + ws_round(sizeof(int) * 4) +
+           ws_round(sizeof(float2) * 27 * std::max<size_t>(n_fc3, 1)) +
+           ws_round(sizeof(float2) * (size_t)nb * tc_ldm(nb));
 }
 
 // The tensor-core pipeline for one Gamma-only system (Y build, T = E Y^T-form,
@@ -402,6 +493,14 @@ cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const L
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(err, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
+    const int ldm = tc_ldm(nb);
+    char *pairs = b + (2 + 4 * (size_t)tc_gamma_batch_max(nb, sms)) * plane + ws_round(sizeof(int) * 4);
+    float2 *fc3p = reinterpret_cast<float2 *>(pairs);
+    float2 *Et = reinterpret_cast<float2 *>(pairs + ws_round(sizeof(float2) * 27 * std::max<size_t>(gp.n_fc3, 1)));
+    const size_t nf = 27 * gp.n_fc3;
+    if (nf) fc3_pair_kernel<<<counted((unsigned)std::min<size_t>((nf + 255) / 256, 4096)), 256, 0, st>>>(nf, d.fc3, fc3p);
+    eig_pair_kernel<<<counted(dim3((nb + 31) / 32, (nb + 31) / 32)), 256, 0, st>>>(
+        nb, reinterpret_cast<const double2 *>(d.eig), ldm, Et);
     split_kernel<double2><<<counted(4096), 256, 0, st>>>(nb, nb, reinterpret_cast<const double2 *>(d.eig),
                                                 (size_t)nb, ld, Eh, El);
     // the planes of one stack are contiguous: plane_elems = plane / 2 elements apart
@@ -435,8 +534,18 @@ cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const L
         if (t1 == t0) continue;                     // no delta-band tile (masked modes)
         // Y_mu^T planes: every batch writes the same (sparse) pattern of
         // entries, so the previous batch's values are all overwritten
-        ybuild_bf16_kernel<<<counted(dim3((gp.n_groups * 9 + 255) / 256, nm)), 256, 0, st>>>(
-            gp.n_groups, d.group_jk, d.group_start, d.blk_i, d.fc3, d.eig, nb, mu0, ld, plane_elems, Yh, Yl);
+        const long long yth = 32LL * gp.n_long + 9LL * (gp.n_groups - gp.n_long);
+        const unsigned ygx = (unsigned)((yth + 255) / 256);
+        auto ybuild = [&](auto kern, int mt) {
+            kern<<<counted(dim3(ygx, (nm + mt - 1) / mt)), 256, 0, st>>>(gp.n_groups, gp.n_long, d.group_order,
+                                                                         d.group_jk, d.group_start, d.blk_i, fc3p, Et,
+                                                                         ldm, mu0, nm, ld, plane_elems, Yh, Yl);
+        };
+        // modes per thread: 4, or 3 where that leaves fewer of them unused
+        if (nm == 1) ybuild(ybuild_pair_kernel<1>, 1);
+        else if (nm == 2) ybuild(ybuild_pair_kernel<2>, 2);
+        else if ((nm + 2) / 3 * 3 < (nm + 3) / 4 * 4) ybuild(ybuild_pair_kernel<3>, 3);
+        else ybuild(ybuild_pair_kernel<4>, 4);
         EpiSplit es{Th, Tl, ld, prow};
         EpiGamma eg{};
         ProfMark p1(p.prof, KALD_PROF_TC_GEMM1, st);

@@ -1,0 +1,47 @@
+"""Edge sizes of individual kernels (GPU), against the FP64 oracle or the
+library's own FP64 path, which other tests hold to the oracle at 1e-10.
+
+Tolerances are those of the modes: 1e-5 of gamma for the FP32 and BF16-split
+linewidths (the energy windows and weights are FP32 in both), 1e-10 for FP64
+results."""
+
+import numpy as np
+import pytest
+
+import kald_inputs as ki
+from oracle import phonons as ph
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def k():
+    from paper_2009_01967_gb300 import build
+    build.build()
+    import paper_2009_01967_gb300 as kk
+    ctx = kk.Context(0)
+    yield kk, ctx
+    ctx.close()
+
+
+def _rel(a, b):
+    return np.max(np.abs(a - b) / np.maximum(np.abs(b), 1e-6 * np.abs(b).max()))
+
+
+@pytest.mark.parametrize("cell,extra", [((3, 3, 1), 0), ((9, 1, 1), 0), ((5, 2, 1), 0), ((3, 3, 1), 300)])
+def test_gamma_only_y_build(k, cell, extra):
+    """108, 108 and 120 modes (a last batch of 12, 12 and 24 of 32 modes, no
+    whole 32-mode tile of eigenvector pairs at the end); 300 random blocks add
+    groups of every length up to the warp-per-group limit and a Phi3 without
+    symmetry."""
+    kk, ctx = k
+    s = ki.fcc_supercell_system(cell, seed=5)
+    if extra:
+        s = ki.random_fc3_system(s, extra, seed=3)
+    nu, eig = ph.phonons(s, (1, 1, 1))
+    out = {}
+    for prec in ("fp64", "bf16split"):
+        opt = kk.Options(temperature_K=300.0, sigma_thz=0.1, precision=prec)
+        out[prec] = kk.kald_linewidths(ctx, [s], (1, 1, 1), nu.ravel(), eig.ravel(), opt)
+    assert abs(out["fp64"][1][1] - out["bf16split"][1][1]) <= 1e-5 * out["fp64"][1][1]
+    assert _rel(out["bf16split"][0], out["fp64"][0]) < 1e-5
