@@ -1277,27 +1277,37 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
             p.n_chunks = (nq + p.qp_chunk - 1) / p.qp_chunk;
             if (tcx) { p.qp_chunk = nq; p.n_chunks = 1; }
             if (small) {
-                p.qp_chunk = sn_chunk(nb);
+                p.qp_chunk = sn_chunk(nb, nq, ctx->sm_count);
                 p.n_chunks = (nq + p.qp_chunk - 1) / p.qp_chunk;
             }
         }
-        std::vector<int> sn_kk;
+        // the register kernel's blocks by class and atom triple, and its tables of
+        // phase sums while they stay within 16 GB and the context's limit (the
+        // kernel sums every block per pair without them)
+        std::vector<int> sn_kk, sn_start, sn_atoms;
         std::vector<int4> sn_bj, sn_bk;
-        std::vector<int2> sn_gjk;
+        std::vector<double> sn_raw;
+        size_t sn_tab = 0;
         if (small) {
+            sn_tab = sn_table_bytes(nb, nq, f32w);
+            if (sn_tab > (size_t(16) << 30) || (ctx->ws_limit && sn_tab > ctx->ws_limit / 2)) sn_tab = 0;
+            std::vector<int> order;
+            plan_sn(h, sn_tab != 0, order, sn_start);
             sn_kk.resize(3 * (size_t)nq);
             for (int q = 0; q < nq; ++q)
                 for (int c = 0; c < 3; ++c) sn_kk[3 * (size_t)q + c] = qf[3 * (size_t)q + c] * (sn_L / mesh[c]);
             sn_bj.resize(std::max<size_t>(n3, 1), make_int4(0, 0, 0, 0));
             sn_bk.resize(std::max<size_t>(n3, 1), make_int4(0, 0, 0, 0));
-            for (size_t b = 0; b < n3; ++b) {
-                const int *rj = &h.rep_int[3 * h.fc3_rj[b]], *rk = &h.rep_int[3 * h.fc3_rk[b]];
-                sn_bj[b] = make_int4(h.fc3_i[b], rj[0], rj[1], rj[2]);
-                sn_bk[b] = make_int4(rk[0], rk[1], rk[2], 0);
+            sn_raw.resize(27 * n3);
+            sn_atoms.resize(3 * n3);
+            for (size_t x = 0; x < n3; ++x) {
+                const size_t b = (size_t)order[x];
+                const int *rj = &h.rep_int[3 * (size_t)h.fc3_rj[b]], *rk = &h.rep_int[3 * (size_t)h.fc3_rk[b]];
+                sn_bj[x] = make_int4(rj[0], rj[1], rj[2], 0);
+                sn_bk[x] = make_int4(rk[0], rk[1], rk[2], 0);
+                std::copy_n(&h.fc3_blk[27 * b], 27, &sn_raw[27 * x]);
+                std::copy_n(&h.fc3_atoms[3 * b], 3, &sn_atoms[3 * x]);
             }
-            const int ng = (int)h.pair3_j.size();
-            sn_gjk.resize(std::max(1, ng));
-            for (int g = 0; g < ng; ++g) sn_gjk[g] = make_int2(h.pair3_j[g], h.pair3_k[g]);
         }
         const int tcx_b = tcx ? tcx_batch_max(nb, nq, ctx->sm_count) : 0;   // scratch for the tuner's largest batch
         // tensor-core path over the whole mesh with Phi3 symmetric under
@@ -1351,17 +1361,19 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
                 while (at <= y_n_at) y_gi[(size_t)g * (y_n_at + 1) + at++] = b1;
             }
         }
-        YSchedule ys;
-        plan_ybuild(h, ys);
+        YSchedule ys;                            // lane schedule of the CUDA-core kernel's Y build
+        if (!small && !tcx) plan_ybuild(h, ys);
         p.n_rounds = ys.n_rounds;
-        std::vector<int4> binfo(std::max<size_t>(n3, 1), make_int4(0, 0, 0, 0));
-        for (size_t b = 0; b < n3; ++b) binfo[b] = make_int4(h.fc3_i[b], h.fc3_rj[b], h.fc3_rk[b], 0);
+        if (small) p.n_rep = 0;                  // the register kernel takes its phases from roots of unity
+        std::vector<int4> binfo(small ? 1 : std::max<size_t>(n3, 1), make_int4(0, 0, 0, 0));
+        for (size_t b = 0; !small && b < n3; ++b) binfo[b] = make_int4(h.fc3_i[b], h.fc3_rj[b], h.fc3_rk[b], 0);
         const size_t c2 = f32w ? sizeof(float2) : sizeof(double2);
         size_t need = bytes_of(ys.group_jk) + bytes_of(ys.segs) + bytes_of(ys.sched) + bytes_of(binfo) +
-                      scaled_bytes(h.fc3_blk, h.fc3_atoms, h, 27, 28, f32w) +
+                      (small ? scaled_bytes(sn_raw, sn_atoms, h, 27, 28, 0)
+                             : scaled_bytes(h.fc3_blk, h.fc3_atoms, h, 27, 28, f32w)) +
                       bytes_of(h.rep_cart) + bytes_of(qc) + bytes_of(qf) +
                       2 * ws_round(sizeof(double) * nq * nb) + ws_round(c2 * nn) +
-                      ws_round(c2 * (size_t)nq * h.n_rep) +
+                      ws_round(c2 * (size_t)nq * p.n_rep) +
                       ws_round(sizeof(double) * (size_t)nqc * p.n_chunks * nb) + 2 * ws_round(16) +
                       bytes_of(qsel) + bytes_of(qrow) + bytes_of(qout);
         if (!d_nu) need += ws_round(sizeof(double) * nq * nb);
@@ -1377,8 +1389,8 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         if (!y_blk.empty())
             need += scaled_bytes(y_blk, y_atoms, h, 27, 28, 1) + bytes_of(y_gi) + bytes_of(y_rep);
         if (small)
-            need += bytes_of(sn_kk) + bytes_of(sn_bj) + bytes_of(sn_bk) + bytes_of(sn_gjk) +
-                    bytes_of(h.pair3_start) + ws_round(c2 * (2 * (size_t)sn_m0 + 1));
+            need += bytes_of(sn_kk) + bytes_of(sn_bj) + bytes_of(sn_bk) + bytes_of(sn_start) +
+                    ws_round(sizeof(double2) * (2 * (size_t)sn_m0 + 1)) + ws_round(sn_tab);
         if ((st = ws_reserve(ctx, need))) return st;
         LwDev d;
         d.group_jk = upload(ctx, ys.group_jk);
@@ -1386,7 +1398,8 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         d.sched = upload(ctx, ys.sched);
         d.blkinfo = upload(ctx, binfo);
         // Phi3 / sqrt(mi mj mk), 28 values per block (16-byte loads), in the working precision
-        d.fc3 = upload_scaled(ctx, h.fc3_blk, h.fc3_atoms, h, 27, 28, f32w);
+        d.fc3 = small ? upload_scaled(ctx, sn_raw, sn_atoms, h, 27, 28, 0)
+                      : upload_scaled(ctx, h.fc3_blk, h.fc3_atoms, h, 27, 28, f32w);
         d.rep_cart = upload(ctx, h.rep_cart);
         d.qcart = upload(ctx, qc);
         d.qfrac = upload(ctx, qf);
@@ -1396,7 +1409,7 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         d.occ = static_cast<double *>(ws_take(ctx, sizeof(double) * nq * nb));
         d.wn32 = f32w ? static_cast<float4 *>(ws_take(ctx, sizeof(float4) * (size_t)nq * nb)) : nullptr;
         d.eps_work = ws_take(ctx, c2 * nn);
-        d.chi = ws_take(ctx, c2 * (size_t)nq * h.n_rep);
+        d.chi = ws_take(ctx, c2 * (size_t)nq * p.n_rep);
         d.partial = static_cast<double *>(ws_take(ctx, sizeof(double) * (size_t)nqc * p.n_chunks * nb));
         d.qsel = upload(ctx, qsel);
         d.qrow = upload(ctx, qrow);
@@ -1450,13 +1463,13 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         SnTables sn;
         if (small) {
             sn.L = sn_L; sn.m0 = sn_m0;
-            sn.n_groups = (int)h.pair3_j.size();
             sn.kk = upload(ctx, sn_kk);
-            sn.gstart = upload(ctx, h.pair3_start);
-            sn.gjk = upload(ctx, sn_gjk);
+            sn.start = upload(ctx, sn_start);
             sn.bj = upload(ctx, sn_bj);
             sn.bk = upload(ctx, sn_bk);
-            sn.roots = ws_take(ctx, c2 * (2 * (size_t)sn_m0 + 1));
+            sn.fc3 = static_cast<const double *>(d.fc3);
+            sn.roots = static_cast<double2 *>(ws_take(ctx, sizeof(double2) * (2 * (size_t)sn_m0 + 1)));
+            sn.tab = sn_tab ? ws_take(ctx, sn_tab) : nullptr;
         }
         cudaStream_t s = ctx->stream;
         cudaError_t e = launch_lw_prep(p, d, f32w, s);

@@ -338,16 +338,18 @@ cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const L
 // q.R = 2 pi sum_d k_d n_d / N_d for q = sum_d (k_d / N_d) b_d, R = sum_d n_d a_d.
 struct SnTables {
     int L, m0;                        // root order, index offset of the table
-    int n_groups;
     const int *kk;                    // [nq][3] k_d L / N_d
-    const int *gstart;                // [n_groups + 1] blocks of each (j, k) group
-    const int2 *gjk;                  // [n_groups] atoms (j, k)
-    const int4 *bj;                   // [n_fc3] (i, Rj in cells), group order
-    const int4 *bk;                   // [n_fc3] (Rk in cells, 0)
-    void *roots;                      // [2 m0 + 1] exp(-2 pi i (t - m0) / L), working precision
+    const int *start;                 // [4 n_atoms^3 + 1] blocks of each (class, i, j, k) (plan_sn)
+    const int4 *bj, *bk;              // [n_fc3] Rj and Rk in cells, plan_sn order
+    const double *fc3;                // [n_fc3][28] Phi3 / sqrt(mi mj mk), plan_sn order
+    double2 *roots;                   // [2 m0 + 1] exp(-2 pi i (t - m0) / L)
+    void *tab;                        // phase-sum tables A, B, C [3][nq][nb^3] in the working
+                                      // precision, or NULL: every block summed per pair
 };
 bool sn_supported(int nb);
-int sn_chunk(int nb);
+int sn_chunk(int nb, int nq, int sm_count);
+size_t sn_table_bytes(int nb, int nq, int fp32);
+void plan_sn(const HostSystem &h, bool tables, std::vector<int> &order, std::vector<int> &start);
 cudaError_t launch_lw_small(const LwParams &p, const LwDev &d, const SnTables &t, int fp32, cudaStream_t st);
 
 // tc_crystal.cu: crystal linewidth sums on tensor cores (BF16 split, nb <= 96).

@@ -658,11 +658,11 @@ cudaError_t launch_lw_prep(const LwParams &p, const LwDev &d, int fp32, cudaStre
     const int grid = (int)std::min<size_t>((ne + 255) / 256, 4096);
     if (fp32) {
         wn_pair_kernel<<<counted((n + 255) / 256), 256, 0, st>>>(n, d.omega, d.occ, d.wn32);
-        chi_kernel<float2><<<counted((nc + 255) / 256), 256, 0, st>>>(p.nq, p.n_rep, d.qcart, d.rep_cart,
+        if (nc) chi_kernel<float2><<<counted((nc + 255) / 256), 256, 0, st>>>(p.nq, p.n_rep, d.qcart, d.rep_cart,
                                                              (float2 *)d.chi);
         eps_transpose_kernel<float2><<<counted(grid), 256, 0, st>>>(p.nq, p.nb, d.eig, (float2 *)d.eps_work);
     } else {
-        chi_kernel<double2><<<counted((nc + 255) / 256), 256, 0, st>>>(p.nq, p.n_rep, d.qcart, d.rep_cart,
+        if (nc) chi_kernel<double2><<<counted((nc + 255) / 256), 256, 0, st>>>(p.nq, p.n_rep, d.qcart, d.rep_cart,
                                                               (double2 *)d.chi);
         eps_transpose_kernel<double2><<<counted(grid), 256, 0, st>>>(p.nq, p.nb, d.eig, (double2 *)d.eps_work);
     }

@@ -1,6 +1,6 @@
 // Crystal linewidths of one- and two-atom cells (nb = 3 or 6; paper Eq.
 // projection_plus, gamma_operators, phase_space).  One thread per (pair,
-// mode s): the phase-summed contraction Y_s, both dense contractions
+// mode s): the contraction Y_s of the phase sums, both dense contractions
 //   T'(s', c) = sum_b eps'(b, s') Y_s(b, c),  phi(s', s'') = sum_c T'(s', c) conj(eps''(c, s''))
 // and the delta-weight epilogue run in registers (nb^2 complex values each).
 // A tensor-core tile of 128 rows would be more than 70% padding here.
@@ -9,11 +9,16 @@
 // exp(-2 pi i m / L) with m = kk(q').nj - kk(q'').nk (kk_d = k_d L / N_d,
 // L = lcm of the mesh), read from a table of roots of unity.
 //
+// Three kinds of blocks have a phase of one q-point only (Rk = 0: q', Rj = 0:
+// q'', Rj = Rk: q) and are summed once per q-point into tables.
+//
 // CTA = (q, chunk of q'), thread = (q' lane, mode s); every thread walks its
 // q' of the chunk in order, the CTA adds the lanes of each mode in order and
 // writes one FP64 partial per (q, chunk, s) for lw_finish.
 
+#include <algorithm>
 #include <type_traits>
+#include <vector>
 
 #include "kald_internal.h"
 #include "wdiff.cuh"
@@ -65,57 +70,92 @@ __device__ __forceinline__ void rfma(float2 &acc, float v, float2 e) {
     acc = __ffma2_rn(make_float2(v, v), e, acc);
 }
 
-// The 28 (27 + pad) values of one Phi3 block, as 16-byte loads.
-__device__ __forceinline__ void load_block(const float *f, float v[28]) {
-    const float4 *f4 = reinterpret_cast<const float4 *>(f);
-#pragma unroll
-    for (int x = 0; x < 7; ++x) {
-        const float4 u = __ldg(f4 + x);
-        v[4 * x] = u.x; v[4 * x + 1] = u.y; v[4 * x + 2] = u.z; v[4 * x + 3] = u.w;
-    }
-}
-__device__ __forceinline__ void load_block(const double *f, double v[28]) {
-    const double2 *f2 = reinterpret_cast<const double2 *>(f);
-#pragma unroll
-    for (int x = 0; x < 14; ++x) {
-        const double2 u = __ldg(f2 + x);
-        v[2 * x] = u.x; v[2 * x + 1] = u.y;
-    }
-}
-
 // roots[t] = exp(-2 pi i (t - m0) / L), argument reduced to [0, L) first.
-__global__ void roots_kernel(int L, int m0, int fp32, void *out) {
+__global__ void roots_kernel(int L, int m0, double2 *__restrict__ out) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t > 2 * m0) return;
     const int r = (((t - m0) % L) + L) % L;
     double sn, cs;
     sincospi(2.0 * (double)r / (double)L, &sn, &cs);
-    if (fp32) static_cast<float2 *>(out)[t] = make_float2((float)cs, (float)-sn);
-    else static_cast<double2 *>(out)[t] = make_double2(cs, -sn);
+    out[t] = make_double2(cs, -sn);
+}
+
+// Sum over the blocks of one class and atom triple (CSR key) of Phi3~[al be ga]
+// times the block's phase exp(-2 pi i m / L), m = x.nj - y.nk with x, y the
+// scaled mesh coordinates of q' and q'' (one of them zero for a table); FP64.
+__device__ __forceinline__ double2 phase_sum(const SnTables &t, int key, int v, int x0, int x1, int x2, int y0, int y1,
+                                             int y2) {
+    double2 acc = make_double2(0.0, 0.0);
+    for (int bl = t.start[key]; bl < t.start[key + 1]; ++bl) {
+        const int4 nj = __ldg(t.bj + bl), nk = __ldg(t.bk + bl);
+        const int m = x0 * nj.x + x1 * nj.y + x2 * nj.z - y0 * nk.x - y1 * nk.y - y2 * nk.z;
+        const double2 ph = __ldg(t.roots + m + t.m0);
+        const double f = __ldg(t.fc3 + (size_t)28 * bl + v);
+        acc.x = fma(f, ph.x, acc.x);
+        acc.y = fma(f, ph.y, acc.y);
+    }
+    return acc;
+}
+
+// Tables of the phase sums that depend on one q-point only, [nq][NB^3] each
+// (index (a NB + b) NB + c): A(q') of the blocks with Rk = 0, B(q'') of those
+// with Rj = 0, C(q) of those with Rj = Rk (chi(q', R) conj chi(q'', R) =
+// conj chi(q, R), q'' = q + q').  One CTA per q-point, FP64 sums.
+template <typename R, int NB>
+__global__ void __launch_bounds__(kSnThreads)
+sn_tables_kernel(int nq, SnTables t, typename Cx<R>::T *__restrict__ tab) {
+    using R2 = typename Cx<R>::T;
+    constexpr int N3 = NB * NB * NB, NA = NB / 3;
+    const int q = blockIdx.x;
+    const int k0 = t.kk[3 * q], k1 = t.kk[3 * q + 1], k2 = t.kk[3 * q + 2];
+    for (int x = threadIdx.x; x < 3 * N3; x += kSnThreads) {
+        const int cls = x / N3, e = x - cls * N3;
+        const int a = e / (NB * NB), b = (e / NB) % NB, c = e % NB;
+        const int key = cls * NA * NA * NA + ((a / 3) * NA + b / 3) * NA + c / 3;
+        const int v = 9 * (a % 3) + 3 * (b % 3) + c % 3;
+        const double2 s = cls == 0 ? phase_sum(t, key, v, k0, k1, k2, 0, 0, 0)
+                                   : phase_sum(t, key, v, 0, 0, 0, k0, k1, k2);
+        R2 o;
+        o.x = (R)s.x;
+        o.y = (R)s.y;
+        tab[((size_t)cls * nq + q) * N3 + e] = o;
+    }
 }
 
 // BTE: each thread also scatters its (q', s) rates into the three operator
 // planes (FP64 only; every plane entry has exactly one writer).
+//
+// Y_s(b, c) = sum_a eps_a(q s) W(a, b, c) with the mode-independent phase sums
+// W = A(q') + B(q'') + C(q) + the blocks whose two cell vectors are non-zero
+// and different (class 3, summed per pair).  The CTA forms W for its pairs one
+// row a at a time in shared memory; every mode of the pair reads it from there.
+//
+// Bound: FMA issue, FP32 or FP64.  Phasing every block for every (pair, mode)
+// cost 54 n_fc3 FMA (25,380 for the two-atom cell), fifteen times the two dense
+// contractions; with the tables a (pair, mode) costs 3 nb^3 complex FMA in all.
+// One call, two-atom cell, 24^3 mesh, FP32: 1367 ms before, 191 ms now.
 template <typename R, int NB, bool BTE>
 __global__ void __launch_bounds__(kSnThreads)
-sn_kernel(LwParams p, LwDev d, SnTables t, const R *__restrict__ fc3, const typename Cx<R>::T *__restrict__ epsT) {
+sn_kernel(LwParams p, LwDev d, SnTables t, const typename Cx<R>::T *__restrict__ tab,
+          const typename Cx<R>::T *__restrict__ epsT) {
     using R2 = typename Cx<R>::T;
-    constexpr int NA = NB / 3;
+    constexpr int NA = NB / 3, N2 = NB * NB, N3 = N2 * NB;
     constexpr int JPC = kSnThreads / NB;           // q' lanes per CTA
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int nroot = 2 * t.m0 + 1;
-    R2 *roots = reinterpret_cast<R2 *>(smem_raw);
-    R2 *eq = roots + nroot;                        // eps(q)^T: eq[b * NB + s]
-    double *red = reinterpret_cast<double *>(
-        (reinterpret_cast<uintptr_t>(eq + NB * NB) + 15) & ~uintptr_t(15));
+    constexpr int WP = N2 + 1;                     // row pitch of W (odd: the pairs' rows start in other banks)
+    __shared__ __align__(16) R2 W[JPC * WP];
+    __shared__ __align__(16) R2 eq[N2], Cq[N3];    // eps(q)^T: eq[b * NB + s]
+    __shared__ int qpp_sm[JPC];
+    __shared__ double red[kSnThreads];
 
     const int qi = blockIdx.x, chunk = blockIdx.y;
     const int2 qm = d.qsel[qi];
     const int q = qm.x;
     const int tid = threadIdx.x;
-    for (int x = tid; x < nroot; x += kSnThreads) roots[x] = static_cast<const R2 *>(t.roots)[x];
-    for (int x = tid; x < NB * NB; x += kSnThreads) eq[x] = epsT[(size_t)q * NB * NB + x];
-    __syncthreads();
+    const bool tabs = tab != nullptr;
+    const R2 *tabA = tab, *tabB = tab + (size_t)p.nq * N3, *tabC = tab + 2 * (size_t)p.nq * N3;
+    for (int x = tid; x < N2; x += kSnThreads) eq[x] = epsT[(size_t)q * N2 + x];
+    for (int x = tid; x < N3; x += kSnThreads)
+        if (tabs) Cq[x] = tabC[(size_t)q * N3 + x];
 
     const int jl = tid / NB, s = tid - (tid / NB) * NB;
     const bool act = jl < JPC;
@@ -127,55 +167,61 @@ sn_kernel(LwParams p, LwDev d, SnTables t, const R *__restrict__ fc3, const type
     const R sig2inv = (R)delta_param(p.shape, p.sigma_w);   // the delta shape's parameter
     const R cut = (R)p.cut_w;
     const int *kq = d.qfrac + 3 * q;
+    const int n_gen = t.start[4 * NA * NA * NA] - t.start[3 * NA * NA * NA];
     double sum = 0.0;
     unsigned long long allowed = 0;
     const int qp0 = chunk * p.qp_chunk, qp1 = min(p.nq, qp0 + p.qp_chunk);
-    for (int qp = qp0 + jl; act && w > (R)0 && qp < qp1; qp += JPC) {
-        const int *kp = d.qfrac + 3 * qp;
-        const int qpp = (((kq[0] + kp[0]) % p.mesh[0]) * p.mesh[1] + (kq[1] + kp[1]) % p.mesh[1]) * p.mesh[2] +
-                        (kq[2] + kp[2]) % p.mesh[2];
-        const int a0 = t.kk[3 * qp], a1 = t.kk[3 * qp + 1], a2 = t.kk[3 * qp + 2];
-        const int c0 = t.kk[3 * qpp], c1 = t.kk[3 * qpp + 1], c2 = t.kk[3 * qpp + 2];
-        // ---- Y_s(b, c), group by group
+    for (int qb = qp0; qb < qp1; qb += JPC) {
+        const int n_p = min(JPC, qp1 - qb);        // pairs of this pass: q' = qb ..
+        __syncthreads();                           // the last pass has read qpp_sm and W
+        if (tid < n_p) {
+            const int *kp = d.qfrac + 3 * (qb + tid);
+            qpp_sm[tid] = (((kq[0] + kp[0]) % p.mesh[0]) * p.mesh[1] + (kq[1] + kp[1]) % p.mesh[1]) * p.mesh[2] +
+                          (kq[2] + kp[2]) % p.mesh[2];
+        }
         R2 Y[NB][NB];
 #pragma unroll
         for (int b = 0; b < NB; ++b)
 #pragma unroll
             for (int c = 0; c < NB; ++c) Y[b][c].x = Y[b][c].y = (R)0;
-        for (int g = 0; g < t.n_groups; ++g) {
-            const int2 jk = t.gjk[g];
-            R2 acc[9];
-#pragma unroll
-            for (int x = 0; x < 9; ++x) acc[x].x = acc[x].y = (R)0;
-            for (int bl = t.gstart[g]; bl < t.gstart[g + 1]; ++bl) {
-                const int4 bj = __ldg(t.bj + bl), bk = __ldg(t.bk + bl);
-                const int m = a0 * bj.y + a1 * bj.z + a2 * bj.w - c0 * bk.x - c1 * bk.y - c2 * bk.z;
-                const R2 ph = roots[m + t.m0];
-                R2 e[3];
-#pragma unroll
-                for (int x = 0; x < 3; ++x) e[x] = cmul(eq[(3 * bj.x + x) * NB + s], ph);
-                R v[28];
-                load_block(fc3 + (size_t)28 * bl, v);
-#pragma unroll
-                for (int x = 0; x < 9; ++x) {
-                    rfma(acc[x], v[18 + x], e[2]);
-                    rfma(acc[x], v[9 + x], e[1]);
-                    rfma(acc[x], v[x], e[0]);
+        const int qp = qb + jl;
+        const bool run = act && jl < n_p && w > (R)0;
+#pragma unroll 1
+        for (int a = 0; a < NB; ++a) {
+            __syncthreads();
+            for (int x = tid; x < n_p * N2; x += kSnThreads) {
+                const int pj = x / N2, e = x - pj * N2;
+                const size_t r1 = (size_t)(qb + pj) * N3 + a * N2 + e, r2 = (size_t)qpp_sm[pj] * N3 + a * N2 + e;
+                R2 v;
+                v.x = v.y = (R)0;
+                if (tabs) {
+                    const R2 u1 = __ldg(tabA + r1), u2 = __ldg(tabB + r2), u3 = Cq[a * N2 + e];
+                    v.x = u1.x + u2.x + u3.x;
+                    v.y = u1.y + u2.y + u3.y;
                 }
+                if (n_gen) {
+                    const int b = e / NB, c = e - (e / NB) * NB;
+                    const int *x1 = t.kk + 3 * (qb + pj), *x2 = t.kk + 3 * qpp_sm[pj];
+                    const double2 g = phase_sum(t, 3 * NA * NA * NA + ((a / 3) * NA + b / 3) * NA + c / 3,
+                                                9 * (a % 3) + 3 * (b % 3) + c % 3, x1[0], x1[1], x1[2], x2[0], x2[1],
+                                                x2[2]);
+                    v.x += (R)g.x;
+                    v.y += (R)g.y;
+                }
+                W[pj * WP + e] = v;
             }
-            // add the group's 3x3 block at atoms (j, k) with constant register indices
+            __syncthreads();
+            if (run) {
+                const R2 ev = eq[a * NB + s];
+                const R2 *Wj = W + jl * WP;
 #pragma unroll
-            for (int ja = 0; ja < NA; ++ja)
+                for (int b = 0; b < NB; ++b)
 #pragma unroll
-                for (int ka = 0; ka < NA; ++ka)
-                    if (ja == jk.x && ka == jk.y) {
-#pragma unroll
-                        for (int x = 0; x < 9; ++x) {
-                            Y[3 * ja + x / 3][3 * ka + x % 3].x += acc[x].x;
-                            Y[3 * ja + x / 3][3 * ka + x % 3].y += acc[x].y;
-                        }
-                    }
+                    for (int c = 0; c < NB; ++c) cfma(Y[b][c], ev, Wj[b * NB + c]);
+            }
         }
+        if (!run) continue;
+        const int qpp = qpp_sm[jl];
         // ---- per s': the row T'(s', c) = sum_b eps'(b, s') Y(b, c), then
         // phi(s', s'') = sum_c T'(s', c) conj(eps''(c, s'')) and both weights
         const R2 *e1 = epsT + (size_t)qp * NB * NB;    // e1[b * NB + s']
@@ -275,13 +321,11 @@ sn_kernel(LwParams p, LwDev d, SnTables t, const R *__restrict__ fc3, const type
 template <typename R, int NB, bool BTE = false>
 cudaError_t run_sn(const LwParams &p, const LwDev &d, const SnTables &t, cudaStream_t st) {
     using R2 = typename Cx<R>::T;
-    const size_t smem = sizeof(R2) * ((size_t)(2 * t.m0 + 1) + NB * NB) + 16 + sizeof(double) * kSnThreads;
-    auto k = sn_kernel<R, NB, BTE>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    R2 *tab = static_cast<R2 *>(t.tab);
+    if (tab) sn_tables_kernel<R, NB><<<counted(p.nq), kSnThreads, 0, st>>>(p.nq, t, tab);
     ProfMark pm(p.prof, KALD_PROF_SMALL_NB, st);
-    k<<<counted(dim3(p.nqc, p.n_chunks)), kSnThreads, smem, st>>>(p, d, t, static_cast<const R *>(d.fc3),
-                                                                 static_cast<const R2 *>(d.eps_work));
+    sn_kernel<R, NB, BTE><<<counted(dim3(p.nqc, p.n_chunks)), kSnThreads, 0, st>>>(
+        p, d, t, tab, static_cast<const R2 *>(d.eps_work));
     pm.end();
     return cudaGetLastError();
 }
@@ -290,14 +334,44 @@ cudaError_t run_sn(const LwParams &p, const LwDev &d, const SnTables &t, cudaStr
 
 bool sn_supported(int nb) { return nb == 3 || nb == 6; }
 
-// q' per CTA: every thread of the CTA walks about eight of them.
-int sn_chunk(int nb) { return (kSnThreads / nb) * 8; }
+// q' per CTA: up to eight passes over the CTA's lanes, fewer where the mesh is
+// too coarse to give every SM about four CTAs.  From the mesh alone, not from the
+// q-points of a call: a q-point's sums do not depend on the call.
+int sn_chunk(int nb, int nq, int sm_count) {
+    const int lanes = kSnThreads / nb;
+    const long long rows = nq / 2 + 1, passes = (nq + lanes - 1) / lanes;
+    const long long ctas = 4LL * std::max(1, sm_count);
+    return lanes * (int)std::max(1LL, std::min(8LL, rows * passes / ctas));
+}
+size_t sn_table_bytes(int nb, int nq, int fp32) {
+    return (fp32 ? sizeof(float2) : sizeof(double2)) * 3 * (size_t)nq * nb * nb * nb;
+}
+
+// The blocks ordered by class (0: Rk = 0, 1: Rj = 0, 2: Rj = Rk, 3: the rest)
+// and, inside a class, by the atom triple (i, j, k); start [4 n_atoms^3 + 1].
+// Without tables every block is of class 3.
+void plan_sn(const HostSystem &h, bool tables, std::vector<int> &order, std::vector<int> &start) {
+    const int na = h.n_atoms, n = (int)h.fc3_i.size(), keys = 4 * na * na * na;
+    std::vector<int> key(n);
+    start.assign(keys + 1, 0);
+    for (int b = 0; b < n; ++b) {
+        const int *rj = &h.rep_int[3 * (size_t)h.fc3_rj[b]], *rk = &h.rep_int[3 * (size_t)h.fc3_rk[b]];
+        const bool zj = !rj[0] && !rj[1] && !rj[2], zk = !rk[0] && !rk[1] && !rk[2];
+        const int cls = !tables ? 3 : zk ? 0 : zj ? 1 : h.fc3_rj[b] == h.fc3_rk[b] ? 2 : 3;
+        key[b] = ((cls * na + h.fc3_i[b]) * na + h.fc3_atoms[3 * (size_t)b + 1]) * na + h.fc3_atoms[3 * (size_t)b + 2];
+        ++start[key[b] + 1];
+    }
+    for (int k = 0; k < keys; ++k) start[k + 1] += start[k];
+    std::vector<int> at(start.begin(), start.end() - 1);
+    order.resize(n);
+    for (int b = 0; b < n; ++b) order[at[key[b]]++] = b;
+}
 
 cudaError_t launch_lw_small(const LwParams &p, const LwDev &d, const SnTables &t, int fp32, cudaStream_t st) {
     if (!sn_supported(p.nb) || t.L < 1 || t.m0 < 0) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(d.allowed, 0, sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
-    roots_kernel<<<counted((2 * t.m0 + 1 + 255) / 256), 256, 0, st>>>(t.L, t.m0, fp32, t.roots);
+    roots_kernel<<<counted((2 * t.m0 + 1 + 255) / 256), 256, 0, st>>>(t.L, t.m0, t.roots);
     if (fp32) return p.nb == 3 ? run_sn<float, 3>(p, d, t, st) : run_sn<float, 6>(p, d, t, st);
     if (p.bte) return p.nb == 3 ? run_sn<double, 3, true>(p, d, t, st) : run_sn<double, 6, true>(p, d, t, st);
     return p.nb == 3 ? run_sn<double, 3>(p, d, t, st) : run_sn<double, 6>(p, d, t, st);

@@ -45,3 +45,26 @@ def test_gamma_only_y_build(k, cell, extra):
         out[prec] = kk.kald_linewidths(ctx, [s], (1, 1, 1), nu.ravel(), eig.ravel(), opt)
     assert abs(out["fp64"][1][1] - out["bf16split"][1][1]) <= 1e-5 * out["fp64"][1][1]
     assert _rel(out["bf16split"][0], out["fp64"][0]) < 1e-5
+
+
+@pytest.mark.parametrize("mesh,extra,cap", [((1, 1, 1), 40, 0), ((7, 2, 3), 40, 0), ((9, 5, 1), 0, 0),
+                                            ((4, 4, 4), 40, 1 << 20)])
+def test_register_kernel_phase_tables(k, mesh, extra, cap):
+    """Phase sums from the per-q tables: a single q-point, uneven meshes with a
+    last partial pass over the q', random blocks with two different cell
+    vectors (summed per pair), and no tables at all under a workspace cap that
+    they would not fit."""
+    from oracle import anharmonic as an
+    kk, ctx = k
+    w = ki.small_binary(mesh=mesh, sigma=0.1)
+    s = ki.random_fc3_system(w.systems[0], extra, seed=7) if extra else w.systems[0]
+    nu, eig = ph.phonons(s, mesh)
+    g_o = an.linewidths(s, mesh, nu, eig, w.T, w.sigma_thz, w.n_sigma)
+    ctx.set_workspace_limit(cap)
+    try:
+        for prec, tol in (("fp64", 1e-10), ("fp32", 1e-5)):
+            opt = kk.Options(temperature_K=w.T, sigma_thz=w.sigma_thz, n_sigma=w.n_sigma, precision=prec)
+            g, _ = kk.kald_linewidths(ctx, s, mesh, nu, eig, opt)
+            assert _rel(g.reshape(g_o.shape), g_o) < tol
+    finally:
+        ctx.set_workspace_limit(0)
