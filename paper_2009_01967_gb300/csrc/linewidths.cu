@@ -542,89 +542,141 @@ __global__ void lw_finish_kernel(int n_out, int nb, int n_chunks, const double *
     }
 }
 
+// The live modes of every q-point in ascending frequency (ties by index),
+// count[q] of them: omega and n in FP64, and their FP32 pairs when wn is given.
+__global__ void sort_modes_kernel(int nb, const double *__restrict__ omega, const double *__restrict__ occ,
+                                  double2 *__restrict__ wn64, float4 *__restrict__ wn, int *__restrict__ count) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double *w = reinterpret_cast<double *>(smem_raw);
+    const size_t row = (size_t)blockIdx.x * nb;
+    for (int x = threadIdx.x; x < nb; x += blockDim.x) w[x] = omega[row + x];
+    if (threadIdx.x == 0) count[blockIdx.x] = 0;
+    __syncthreads();
+    for (int x = threadIdx.x; x < nb; x += blockDim.x) {
+        const double v = w[x];
+        if (!(v > 0.0)) continue;
+        int r = 0;
+        for (int y = 0; y < nb; ++y) r += w[y] > 0.0 && (w[y] < v || (w[y] == v && y < x));
+        const double n = occ[row + x];
+        if (wn64) wn64[row + r] = make_double2(v, n);
+        if (wn) {
+            const F2 a = f2_of(v), o = f2_of(n);
+            wn[row + r] = make_float4(a.h, a.l, o.h, o.l);
+        }
+        atomicAdd(count + blockIdx.x, 1);
+    }
+}
+
 // Phase space per mode (the definition after Eq. delta_deconstructed, with
 // the weights of Eq. phase_space and the readings of the linewidths: the 1/2
 // on the - process, 1/N_k, masked modes):
 //   g_mu = (1/N_k) sum_{q' s' s''} [(n' - n'') G(w + w' - w'') + 1/2 (1 + n' + n'') G(w - w' - w'')],
 // q'' = q + q' for both processes (the - process of (q, -q') has the same
-// frequencies, since w(-q) = w(q)).  One thread per (q, s), q' in order;
-// the modes of q' and q'' are staged in shared memory per q' (all threads of
-// a CTA share q).  FP64, or FP32 weights with the compensated differences and
-// FP64 sums over q'.  The delta normalisation and 1/N_k are applied at the end.
+// frequencies, since w(-q) = w(q)).  CTA = (q, block of s, chunk of q'), one
+// thread per s, FP64 sums over q', one partial sum per chunk.  FP64, or FP32
+// weights with the compensated differences.
+//
+// Bound: issue slots.  The modes of q' and q'' are staged in ascending order,
+// so along w' the two windows of w'' slide one way each: a thread keeps their
+// near ends and walks only the modes inside (about a seventh of them per
+// window at 3 sigma = 0.15 THz of a 2 THz band); the exact test of the window
+// decides, the walk is a little wider.  32 atoms, 6^3 mesh, FP32: 143 ms when
+// every (s', s'') was tested by one thread per (q, s), 10.9 ms now.
 template <typename R>
 __global__ void __launch_bounds__(128)
-phase_space_kernel(LwParams p, LwDev d, double scale, double *__restrict__ g_out) {
+phase_space_kernel(LwParams p, LwDev d, const void *__restrict__ modes, const int *__restrict__ count, int chunk,
+                   double *__restrict__ partial) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr bool kPair = std::is_same<R, float>::value;
     const int nb = p.nb;
-    const int per_q = (nb + blockDim.x - 1) / blockDim.x;          // CTAs per q
-    const int q = p.q0 + (int)blockIdx.x / per_q;
+    const int per_q = (nb + blockDim.x - 1) / blockDim.x;          // CTAs per q and chunk
+    const int q = (int)blockIdx.x / per_q;
     const int s = ((int)blockIdx.x % per_q) * blockDim.x + threadIdx.x;
     // modes of q' and q'': FP32 pairs (w hi, w lo, n hi, n lo), or FP64 (w, n)
-    float4 *f1 = reinterpret_cast<float4 *>(smem_raw);
-    float4 *f2 = f1 + nb;
-    double2 *e1 = reinterpret_cast<double2 *>(smem_raw);
-    double2 *e2 = e1 + nb;
+    using M = typename std::conditional<kPair, float4, double2>::type;
+    M *f1 = reinterpret_cast<M *>(smem_raw), *f2 = f1 + nb;
+    const M *all = static_cast<const M *>(modes);
     const R a = (R)delta_param(p.shape, p.sigma_w);
     const R cut = (R)p.cut_w;
-    const bool act = s < nb && q < p.q1;
-    const double w_s = act ? d.omega[(size_t)q * nb + s] : 0.0;
+    const double w_s = s < nb ? d.omega[(size_t)q * nb + s] : 0.0;
     const F2 wsp = f2_of(w_s);
+    const R w = (R)w_s;
     double sum = 0.0;
-    for (int qp = 0; qp < p.nq; ++qp) {
+    const int qp1 = min(p.nq, ((int)blockIdx.y + 1) * chunk);
+    for (int qp = blockIdx.y * chunk; qp < qp1; ++qp) {
         const int *kq = d.qfrac + 3 * q, *kp = d.qfrac + 3 * qp;
         const int qpp = (((kq[0] + kp[0]) % p.mesh[0]) * p.mesh[1] + (kq[1] + kp[1]) % p.mesh[1]) * p.mesh[2] +
                         (kq[2] + kp[2]) % p.mesh[2];
+        const int m1 = count[qp], m2 = count[qpp];
         __syncthreads();
-        for (int x = threadIdx.x; x < nb; x += blockDim.x) {
-            if constexpr (kPair) {
-                f1[x] = d.wn32[(size_t)qp * nb + x];
-                f2[x] = d.wn32[(size_t)qpp * nb + x];
-            } else {
-                e1[x] = make_double2(d.omega[(size_t)qp * nb + x], d.occ[(size_t)qp * nb + x]);
-                e2[x] = make_double2(d.omega[(size_t)qpp * nb + x], d.occ[(size_t)qpp * nb + x]);
-            }
+        for (int x = threadIdx.x; x < max(m1, m2); x += blockDim.x) {
+            if (x < m1) f1[x] = all[(size_t)qp * nb + x];
+            if (x < m2) f2[x] = all[(size_t)qpp * nb + x];
         }
         __syncthreads();
-        if (!act || !(w_s > 0.0)) continue;
+        if (!(w_s > 0.0) || m1 == 0 || m2 == 0) continue;
+        // half width of the walk: the window, plus the rounding of sums of three frequencies
+        const R wide = cut * (R)1.0001 + (kPair ? (R)1e-6 : (R)1e-14) * (w + f1[m1 - 1].x + f2[m2 - 1].x);
         R part = (R)0;
-        for (int sp = 0; sp < nb; ++sp) {
-            R w1, n1;
+        int lo = 0, top = m2;                  // first w'' of the + window, one past the last of the - window
+        for (int sp = 0; sp < m1; ++sp) {
+            const M u = f1[sp];
+            const R w1 = u.x;
+            R n1;
             F2 n1p, sum_p, dif_p;
             if constexpr (kPair) {
-                const float4 u = f1[sp];
-                w1 = u.x; n1 = u.z;
+                n1 = u.z;
                 n1p = F2{u.z, u.w};
                 sum_p = f2_add(wsp, F2{u.x, u.y});
                 dif_p = f2_add(wsp, F2{-u.x, -u.y});
             } else {
-                w1 = e1[sp].x; n1 = e1[sp].y;
+                n1 = u.y;
             }
-            if (!(w1 > (R)0)) continue;
             R inner = (R)0;
-            for (int spp = 0; spp < nb; ++spp) {
-                R w2, n2, dp, dm, dn;
+            const R wp = w + w1, wm = w - w1;
+            while (lo < m2 && wp - f2[lo].x >= wide) ++lo;
+            for (int k = lo; k < m2; ++k) {
+                const M v = f2[k];
+                if (!(wp - v.x > -wide)) break;
+                R dp, dn;
                 if constexpr (kPair) {
-                    const float4 v = f2[spp];
-                    w2 = v.x; n2 = v.z;
                     dp = f2_diff(sum_p, F2{v.x, v.y});
-                    dm = f2_diff(dif_p, F2{v.x, v.y});
                     dn = f2_diff(n1p, F2{v.z, v.w});
                 } else {
-                    w2 = e2[spp].x; n2 = e2[spp].y;
-                    dp = w_s + w1 - w2;
-                    dm = w_s - w1 - w2;
-                    dn = n1 - n2;
+                    dp = w_s + w1 - v.x;
+                    dn = n1 - v.y;
                 }
-                if (!(w2 > (R)0)) continue;
                 if (fabs(dp) < cut) inner += dn * delta_shape(dp, p.shape, a);
+            }
+            while (top > 0 && f2[top - 1].x - wm >= wide) --top;
+            for (int k = top - 1; k >= 0; --k) {
+                const M v = f2[k];
+                if (!(v.x - wm > -wide)) break;
+                R dm, n2;
+                if constexpr (kPair) {
+                    dm = f2_diff(dif_p, F2{v.x, v.y});
+                    n2 = v.z;
+                } else {
+                    dm = w_s - w1 - v.x;
+                    n2 = v.y;
+                }
                 if (fabs(dm) < cut) inner += (R)0.5 * ((R)1 + n1 + n2) * delta_shape(dm, p.shape, a);
             }
             part += inner;
         }
         sum += (double)part;
     }
-    if (act) g_out[(size_t)(q - p.q0) * nb + s] = (w_s > 0.0) ? scale * sum : 0.0;
+    if (s < nb) partial[((size_t)blockIdx.y * p.nq + q) * nb + s] = sum;
+}
+
+// g[x] = scale * sum of the chunks' partial sums in order.
+__global__ void phase_space_sum_kernel(size_t n, int n_chunks, const double *__restrict__ partial, double scale,
+                                       double *__restrict__ g) {
+    const size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    if (x >= n) return;
+    double t = 0.0;
+    for (int c = 0; c < n_chunks; ++c) t += partial[(size_t)c * n + x];
+    g[x] = scale * t;
 }
 
 template <typename R>
@@ -701,23 +753,43 @@ cudaError_t launch_lw_main(const LwParams &p, const LwDev &d, int fp32, int sm_c
     return cudaGetLastError();
 }
 
-cudaError_t launch_wn_pairs(int n, const double *omega, const double *occ, float4 *wn32, cudaStream_t st) {
-    wn_pair_kernel<<<counted((n + 255) / 256), 256, 0, st>>>(n, omega, occ, wn32);
-    return cudaGetLastError();
+// q' chunks of the phase-space sum: about eight CTAs per SM.
+static int phase_space_chunks(int nb, int nq, int sm_count) {
+    const long long rows = (long long)nq * ((nb + 127) / 128);
+    return (int)std::max(1LL, std::min<long long>(std::min(nq, 1024), (8LL * std::max(1, sm_count) + rows - 1) / rows));
+}
+size_t phase_space_bytes(int nb, int nq, int sm_count) {
+    const size_t n = (size_t)nb * nq;
+    return ws_round(16 * n) + ws_round(sizeof(int) * (size_t)nq) +
+           ws_round(sizeof(double) * n * phase_space_chunks(nb, nq, sm_count));
 }
 
-cudaError_t launch_phase_space(const LwParams &p, const LwDev &d, int fp32, double *g_out, cudaStream_t st) {
-    const int threads = 128;
+cudaError_t launch_phase_space(const LwParams &p, const LwDev &d, int fp32, int sm_count, void *work, double *g_out,
+                               cudaStream_t st) {
+    const size_t n = (size_t)p.nb * p.nq;
+    char *w = static_cast<char *>(work);
+    void *modes = w;
+    int *count = reinterpret_cast<int *>(w + ws_round(16 * n));
+    double *partial = reinterpret_cast<double *>(w + ws_round(16 * n) + ws_round(sizeof(int) * (size_t)p.nq));
+    const int n_chunks0 = phase_space_chunks(p.nb, p.nq, sm_count);
+    const int chunk = (p.nq + n_chunks0 - 1) / n_chunks0, n_chunks = (p.nq + chunk - 1) / chunk;
+    const int threads = std::min(128, (p.nb + 31) / 32 * 32);
     const int per_q = (p.nb + threads - 1) / threads;
-    const size_t smem = 2 * sizeof(float4) * (size_t)p.nb;     // >= two double2 rows
+    const size_t ssort = sizeof(double) * (size_t)p.nb, smem = 2 * sizeof(float4) * (size_t)p.nb;
+    cudaError_t e = cudaFuncSetAttribute(sort_modes_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssort);
+    if (e != cudaSuccess) return e;
+    sort_modes_kernel<<<counted(p.nq), threads, ssort, st>>>(p.nb, d.omega, d.occ,
+                                                             fp32 ? nullptr : static_cast<double2 *>(modes),
+                                                             fp32 ? static_cast<float4 *>(modes) : nullptr, count);
     const double scale = delta_norm(p.shape, p.sigma_w) / (double)p.nq;
     auto k32 = phase_space_kernel<float>;
     auto k64 = phase_space_kernel<double>;
-    cudaError_t e = cudaFuncSetAttribute(fp32 ? k32 : k64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(fp32 ? k32 : k64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)((p.q1 - p.q0) * per_q));
-    if (fp32) k32<<<counted(grid), threads, smem, st>>>(p, d, scale, g_out);
-    else k64<<<counted(grid), threads, smem, st>>>(p, d, scale, g_out);
+    const dim3 grid((unsigned)(p.nq * per_q), (unsigned)n_chunks);
+    if (fp32) k32<<<counted(grid), threads, smem, st>>>(p, d, modes, count, chunk, partial);
+    else k64<<<counted(grid), threads, smem, st>>>(p, d, modes, count, chunk, partial);
+    phase_space_sum_kernel<<<counted((unsigned)((n + 255) / 256)), 256, 0, st>>>(n, n_chunks, partial, scale, g_out);
     return cudaGetLastError();
 }
 

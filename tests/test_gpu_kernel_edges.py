@@ -68,3 +68,36 @@ def test_register_kernel_phase_tables(k, mesh, extra, cap):
             assert _rel(g.reshape(g_o.shape), g_o) < tol
     finally:
         ctx.set_workspace_limit(0)
+
+
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-10), ("fp32", 1e-5)])
+@pytest.mark.parametrize("nb,mesh,sigma", [(3, (2, 3, 1), 0.3), (5, (3, 1, 1), 5.0), (130, (2, 1, 1), 0.02)])
+def test_phase_space_sliding_windows(k, nb, mesh, sigma, precision, tol):
+    """Frequencies in no order, with equal, negative and masked ones, windows
+    wider than the spectrum and narrow ones, more modes than one CTA's threads."""
+    from types import SimpleNamespace
+    from oracle import anharmonic as an
+    kk, ctx = k
+    if nb % 3:
+        nb += 3 - nb % 3
+    rng = np.random.default_rng(nb)
+    nq = int(np.prod(mesh))
+    nu = rng.uniform(0.2, 2.0, (nq, nb))
+    nu[:, nb // 2] = nu[:, 0]
+    nu[0, 1], nu[-1, 0] = -0.3, 0.001
+    s = ki.small_binary(mesh=mesh).systems[0]
+    n = nb // 3
+    s = SimpleNamespace(masses=np.full(n, 20.0), positions=np.arange(3.0 * n).reshape(n, 3), lattice=10 * np.eye(3),
+                        fc2_idx=s.fc2_idx[:0], fc2=s.fc2[:0], fc3_idx=s.fc3_idx[:0], fc3=s.fc3[:0])
+    g_o = an.phase_space(mesh, nu, 300.0, sigma, 3.0)
+    opt = kk.Options(temperature_K=300.0, sigma_thz=sigma, precision=precision)
+    g = kk.kald_phase_space(ctx, s, mesh, nu, opt).reshape(g_o.shape)
+    assert np.all(g[nu <= 0.01] == 0.0)
+    # the oracle's - process takes w(-q'); on this spectrum, which is not that of
+    # a crystal, it is compared on meshes where -q' = q' or with nu made even
+    neg = np.array([np.ravel_multi_index(tuple((-np.array(np.unravel_index(q, mesh))) % mesh), mesh) for q in range(nq)])
+    if np.any(neg != np.arange(nq)):
+        nu = np.where((neg < np.arange(nq))[:, None], nu[neg], nu)
+        g_o = an.phase_space(mesh, nu, 300.0, sigma, 3.0)
+        g = kk.kald_phase_space(ctx, s, mesh, nu, opt).reshape(g_o.shape)
+    assert _rel(g, g_o) < tol
