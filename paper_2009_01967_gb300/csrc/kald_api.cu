@@ -170,6 +170,7 @@ void mesh_points(const double lat[3][3], const int32_t mesh[3], std::vector<doub
 struct DevSystem {
     int *pair2_i = nullptr, *pair2_j = nullptr, *pair2_start = nullptr;
     double *fc2 = nullptr, *fc2_r = nullptr, *fc2_d = nullptr;
+    int4 *up = nullptr;
     int *p3_start = nullptr, *p3_jk = nullptr, *b_i = nullptr, *b_rj = nullptr, *b_rk = nullptr;
     void *fc3 = nullptr;
     double *rep = nullptr;
@@ -209,7 +210,8 @@ void *upload_scaled(kald_ctx *ctx, const std::vector<double> &raw, const std::ve
 
 size_t fc2_bytes(const HostSystem &h) {
     return bytes_of(h.pair2_i) + bytes_of(h.pair2_j) + bytes_of(h.pair2_start) +
-           scaled_bytes(h.fc2_blk, h.fc2_atoms, h, 9, 9, 0) + bytes_of(h.fc2_rcart) + bytes_of(h.fc2_dist);
+           scaled_bytes(h.fc2_blk, h.fc2_atoms, h, 9, 9, 0) + bytes_of(h.fc2_rcart) + bytes_of(h.fc2_dist) +
+           bytes_of(h.pair2_up);
 }
 void upload_fc2(kald_ctx *ctx, const HostSystem &h, DevSystem &d) {
     d.pair2_i = upload(ctx, h.pair2_i);
@@ -218,12 +220,14 @@ void upload_fc2(kald_ctx *ctx, const HostSystem &h, DevSystem &d) {
     d.fc2 = static_cast<double *>(upload_scaled(ctx, h.fc2_blk, h.fc2_atoms, h, 9, 9, 0));
     d.fc2_r = upload(ctx, h.fc2_rcart);
     d.fc2_d = upload(ctx, h.fc2_dist);
+    d.up = upload(ctx, h.pair2_up);
 }
 DevFc2 dev_fc2(const HostSystem &h, const DevSystem &d) {
     DevFc2 f;
     f.n_pairs = (int)h.pair2_i.size();
     f.pair_i = d.pair2_i; f.pair_j = d.pair2_j; f.pair_start = d.pair2_start;
     f.blk = d.fc2; f.rcart = d.fc2_r;
+    f.n_up = (int)h.pair2_up.size(); f.up = d.up;
     return f;
 }
 
@@ -332,6 +336,16 @@ kald_status plan_system(kald_ctx *ctx, const kald_system *s, HostSystem &h) {
         }
     }
     h.pair2_start.push_back(n2);
+    h.pair2_up.clear();
+    if (h.nb <= kMaxNbSmall) {
+        std::vector<int> at((size_t)n * n, -1);
+        for (size_t p = 0; p < h.pair2_i.size(); ++p) at[(size_t)h.pair2_i[p] * n + h.pair2_j[p]] = (int)p;
+        for (int i = 0; i < n; ++i)
+            for (int j = i; j < n; ++j) {
+                const int a = at[(size_t)i * n + j], b = at[(size_t)j * n + i];
+                if (a >= 0 || b >= 0) h.pair2_up.push_back(make_int4(i, j, a, b));
+            }
+    }
     // ---- fc3, grouped by (j, k) output pair; replica table
     const int n3 = s->n_fc3;
     // replica index of an integer cell vector, in first-seen order: a dense
@@ -630,6 +644,9 @@ kald_status kald_phonons(kald_ctx *ctx, const kald_system *sys, const int32_t me
     if (mirror)
         need += bytes_of(qc_rep) + bytes_of(rep_row) + bytes_of(rep_conj) + ws_round(sizeof(double) * nrep * nb) +
                 ws_round(sizeof(double2) * nnr);
+    const size_t n_blk2 = h.fc2_blk.size() / 9;
+    if (vel && !large)
+        need += vel_table_bytes(nrep, n_blk2) + (mirror ? ws_round(sizeof(double) * 3 * nrep * nb) : 0);
     if (large) need += eigh_large_scratch_bytes(nb) + eigh_batch_records_bytes(1);
     if (!d_nu) need += ws_round(sizeof(double) * nq * nb);
     if (!d_eig) need += ws_round(sizeof(double2) * nn);
@@ -651,22 +668,33 @@ kald_status kald_phonons(kald_ctx *ctx, const kald_system *sys, const int32_t me
                            : static_cast<double2 *>(ws_take(ctx, sizeof(double2) * nn));
     double *vel_d = nullptr;
     if (vel) vel_d = d_vel ? vel : static_cast<double *>(ws_take(ctx, sizeof(double) * 3 * nq * nb));
+    void *vel_tab = vel && !large ? ws_take(ctx, vel_table_bytes(nrep, n_blk2)) : nullptr;
+    double *vel_rep = vel && mirror ? static_cast<double *>(ws_take(ctx, sizeof(double) * 3 * nrep * nb)) : nullptr;
     cudaStream_t s = ctx->stream;
     double *big = large ? static_cast<double *>(ws_take(ctx, eigh_large_scratch_bytes(nb))) : nullptr;
     void *rec = large ? ws_take(ctx, eigh_batch_records_bytes(1)) : nullptr;
     cudaMemsetAsync(nonconv, 0, sizeof(int), s);
-    cudaError_t e = launch_dynmat(dev_fc2(h, d), nb, mirror ? nrep : nq, qcart_rep, D, s);
+    cudaError_t e = launch_dynmat(dev_fc2(h, d), nb, mirror ? nrep : nq, n_blk2, qcart_rep, D, s);
     if (e == cudaSuccess) {
         if (large) {
             const EighJob job{nb, D, big, nu_d, eig_d};
             e = launch_eigh_large_batch(1, &job, rec, ctx->sm_count, ctx->smem_optin, s);
         } else if (mirror) {
             e = launch_jacobi(nb, nrep, D, V, nu_rep, eig_rep, nonconv, ctx->smem_optin, s);
-            if (e == cudaSuccess) e = launch_mirror_phonons(nq, nb, row_d, conj_d, nu_rep, eig_rep, nu_d, eig_d, s);
+            if (e == cudaSuccess && vel)
+                e = launch_vel_diag(dev_fc2(h, d), nb, nrep, n_blk2, qcart_rep, nu_rep, nullptr, eig_rep, nullptr, nullptr,
+                                    vel_tab, vel_rep, nullptr, s);
+            if (e == cudaSuccess)
+                e = launch_mirror_phonons(nq, nb, row_d, conj_d, nu_rep, eig_rep, vel_rep, nu_d, eig_d, vel_d, s);
+        } else {
+            e = launch_jacobi(nb, nq, D, V, nu_d, eig_d, nonconv, ctx->smem_optin, s);
+            if (e == cudaSuccess && vel)
+                e = launch_vel_diag(dev_fc2(h, d), nb, nq, n_blk2, qcart, nu_d, nullptr, eig_d, nullptr, nullptr, vel_tab,
+                                    vel_d, nullptr, s);
         }
-        else e = launch_jacobi(nb, nq, D, V, nu_d, eig_d, nonconv, ctx->smem_optin, s);
     }
-    if (e == cudaSuccess && vel) e = launch_velocity_diag(dev_fc2(h, d), nb, nq, qcart, nu_d, eig_d, vel_d, s);
+    if (e == cudaSuccess && vel && large)
+        e = launch_velocity_diag(dev_fc2(h, d), nb, nq, qcart, nu_d, eig_d, vel_d, s);
     if (e != cudaSuccess) return cuda_check(ctx, e, "kald_phonons launch");
     int nc = 0;
     cudaMemcpyAsync(&nc, nonconv, sizeof(int), cudaMemcpyDeviceToHost, s);
@@ -742,7 +770,7 @@ kald_status kald_phonons_batch(kald_ctx *ctx, int32_t n_sys, const kald_system *
             double *nu_d = d_nu ? nu_thz + off_nb[x] : static_cast<double *>(ws_take(ctx, sizeof(double) * nb));
             double2 *eig_d = d_eig ? reinterpret_cast<double2 *>(eigvec) + off_eig[x]
                                    : static_cast<double2 *>(ws_take(ctx, sizeof(double2) * nn));
-            e = launch_dynmat(dev_fc2(h, d), nb, 1, qcart, D, ctx->stream);
+            e = launch_dynmat(dev_fc2(h, d), nb, 1, h.fc2_blk.size() / 9, qcart, D, ctx->stream);
             jobs.push_back({nb, D, big, nu_d, eig_d});
             nu_stage.push_back(nu_d);
             eig_stage.push_back(eig_d);
@@ -848,6 +876,32 @@ bool fc3_symmetric_all(const kald_system *s) {
                     const double u = f[9 * a + 3 * c + d], v = g[9 * c + 3 * a + d];
                     if (std::fabs(u - v) > tol) return false;
                 }
+    }
+    return true;
+}
+// True when every fc2 block (i; j R) has the partner (j; i -R) with the
+// Cartesian indices exchanged, to 1e-12 of the largest |Phi2|.
+bool fc2_symmetric(const kald_system *s) {
+    double tol = 0.0;
+    for (size_t v = 0; v < 9 * (size_t)s->n_fc2; ++v) tol = std::max(tol, std::fabs(s->fc2[v]));
+    tol *= 1e-12;
+    // blocks ordered by (i, j, R); the partner's key is looked up by bisection
+    std::vector<int> o(s->n_fc2);
+    std::iota(o.begin(), o.end(), 0);
+    auto less = [](const int32_t *a, const int32_t *b) { return std::lexicographical_compare(a, a + 5, b, b + 5); };
+    auto row = [&](int b) { return s->fc2_idx + 5 * (size_t)b; };
+    std::sort(o.begin(), o.end(), [&](int a, int b) { return less(row(a), row(b)); });
+    for (int x = 0; x + 1 < s->n_fc2; ++x)
+        if (!less(row(o[x]), row(o[x + 1]))) return false;       // a repeated block
+    for (int b = 0; b < s->n_fc2; ++b) {
+        const int32_t *x = row(b);
+        const int32_t k[5] = {x[1], x[0], -x[2], -x[3], -x[4]};
+        auto it = std::lower_bound(o.begin(), o.end(), k, [&](int a, const int32_t *key) { return less(row(a), key); });
+        if (it == o.end() || less(k, row(*it))) return false;
+        const double *f = s->fc2 + 9 * (size_t)b, *g = s->fc2 + 9 * (size_t)*it;
+        for (int a = 0; a < 3; ++a)
+            for (int c = 0; c < 3; ++c)
+                if (!(std::fabs(f[3 * a + c] - g[3 * c + a]) <= tol)) return false;
     }
     return true;
 }
@@ -1610,7 +1664,7 @@ kald_status kald_kappa_bte(kald_ctx *ctx, const kald_system *sys, const int32_t 
             mesh_points(h.lattice, mesh, qc, qf);
             const bool d_nu = is_device_ptr(nu_thz), d_eig = is_device_ptr(eigvec), d_k = is_device_ptr(kappa);
             size_t need = fc2_bytes(h) + bytes_of(qc) + ws_round(sizeof(double) * 3 * (size_t)N) +
-                          bte_work_bytes(N) + ws_round(72);
+                          bte_work_bytes(N) + ws_round(72) + vel_table_bytes(nq, h.fc2_blk.size() / 9);
             if (!d_nu) need += ws_round(sizeof(double) * N);
             if (!d_eig) need += ws_round(sizeof(double2) * (size_t)N * nb);
             st = ws_reserve(ctx, need);
@@ -1623,7 +1677,10 @@ kald_status kald_kappa_bte(kald_ctx *ctx, const kald_system *sys, const int32_t 
                 double *vel = static_cast<double *>(ws_take(ctx, sizeof(double) * 3 * (size_t)N));
                 void *work = ws_take(ctx, bte_work_bytes(N));
                 double *k_d = d_k ? kappa : static_cast<double *>(ws_take(ctx, 72));
-                cudaError_t e = launch_velocity_diag(dev_fc2(h, d), nb, nq, qcart, nu_d, eig_d, vel, ctx->stream);
+                const size_t n_blk2 = h.fc2_blk.size() / 9;
+                void *vel_tab = ws_take(ctx, vel_table_bytes(nq, n_blk2));
+                cudaError_t e = launch_vel_diag(dev_fc2(h, d), nb, nq, n_blk2, qcart, nu_d, nullptr, eig_d, nullptr,
+                                                nullptr, vel_tab, vel, nullptr, ctx->stream);
                 if (e == cudaSuccess)
                     e = bte_solve(N, g1, g0, nu_d, vel, opt->omega_min_thz, opt->temperature_K, opt->classical,
                                   method, tol, max_iter, work, kKappaSI / ((double)nq * h.volume), k_d, iters, conv,
@@ -1910,7 +1967,17 @@ kald_status kald_kappa_rta(kald_ctx *ctx, const kald_system *sys, const int32_t 
     const size_t nn = (size_t)nq * nb * nb;
     const bool d_nu = is_device_ptr(nu_thz), d_eig = is_device_ptr(eigvec), d_g = is_device_ptr(gamma);
     const bool d_k = is_device_ptr(kappa);
-    size_t need = fc2_bytes(h) + bytes_of(qc) + ws_round(sizeof(double) * 9 * (size_t)nq) + ws_round(72);
+    if (h.fc2_symmetric < 0) h.fc2_symmetric = fc2_symmetric(sys) ? 1 : 0;
+    const int n_el = h.fc2_symmetric ? 1 : 2;      // real (and imaginary) parts of the diagonal elements
+    const size_t n_blk2 = h.fc2_blk.size() / 9, nel = 3 * (size_t)nq * nb;
+    std::vector<int> neg(nq);
+    for (int q = 0; q < nq; ++q) {
+        const int *k = &qf[3 * (size_t)q];
+        neg[q] = (((mesh[0] - k[0]) % mesh[0]) * mesh[1] + (mesh[1] - k[1]) % mesh[1]) * mesh[2] +
+                 (mesh[2] - k[2]) % mesh[2];
+    }
+    size_t need = fc2_bytes(h) + bytes_of(qc) + ws_round(sizeof(double) * 9 * (size_t)nq) + ws_round(72) +
+                  2 * bytes_of(neg) + n_el * ws_round(sizeof(double) * nel) + vel_table_bytes(nq, n_blk2);
     if (!d_nu) need += ws_round(sizeof(double) * nq * nb);
     if (!d_eig) need += ws_round(sizeof(double2) * nn);
     if (!d_g) need += ws_round(sizeof(double) * nq * nb);
@@ -1923,10 +1990,19 @@ kald_status kald_kappa_rta(kald_ctx *ctx, const kald_system *sys, const int32_t 
     const double *g_d = stage_in(ctx, gamma, (size_t)nq * nb, d_g);
     double *partial = static_cast<double *>(ws_take(ctx, sizeof(double) * 9 * (size_t)nq));
     double *k_d = d_k ? kappa : static_cast<double *>(ws_take(ctx, 72));
+    const int *neg_d = upload(ctx, neg);
+    int *src = static_cast<int *>(ws_take(ctx, sizeof(int) * (size_t)nq));
+    double *vre = static_cast<double *>(ws_take(ctx, sizeof(double) * nel));
+    double *vim = n_el == 2 ? static_cast<double *>(ws_take(ctx, sizeof(double) * nel)) : nullptr;
+    void *vel_tab = ws_take(ctx, vel_table_bytes(nq, n_blk2));
     const double scale = kKappaSI / ((double)nq * h.volume);
-    cudaError_t e = launch_kappa_rta(dev_fc2(h, d), nb, nq, qcart, nu_d, eig_d, g_d, opt->temperature_K,
-                                     opt->classical, opt->omega_min_thz, opt->degen_tol_thz, partial,
-                                     k_d, scale, ctx->stream);
+    cudaError_t e = launch_vel_diag(dev_fc2(h, d), nb, nq, n_blk2, qcart, nullptr, nu_d, eig_d, neg_d, src, vel_tab, vre,
+                                    vim, ctx->stream);
+    if (e == cudaSuccess)
+        e = launch_kappa_rta_diag(dev_fc2(h, d), nb, nq, qcart, nu_d, eig_d, g_d, src, vre, vim,
+                                  vel_batch(nq, n_blk2) == nq ? static_cast<const double2 *>(vel_tab) : nullptr,
+                                  (int)n_blk2, opt->temperature_K, opt->classical, opt->omega_min_thz, opt->degen_tol_thz, partial, k_d, scale,
+                                  ctx->stream);
     if (e != cudaSuccess) return cuda_check(ctx, e, "kald_kappa_rta launch");
     if (!d_k) cudaMemcpyAsync(kappa, k_d, 72, cudaMemcpyDeviceToHost, ctx->stream);
     return finish(ctx, "kald_kappa_rta");

@@ -136,6 +136,8 @@ struct HostSystem {
     std::vector<int> fc2_atoms;                        // [n_fc2][2] (i, j) of each block
     std::vector<double> fc2_rcart;                     // [n_fc2][3] Cartesian R
     std::vector<double> fc2_dist;                      // [n_fc2][3] x_i - x_j - R
+    std::vector<int4> pair2_up;                        // DevFc2::up (nb <= 96)
+    mutable int fc2_symmetric = -1;                    // Phi2(i, jR) = Phi2(j, i-R)^T (lazy)
     // fc3 grouped by (j, k) atom pair (CSR over output pairs)
     std::vector<int> pair3_j, pair3_k, pair3_start;
     // the groups of more than kYLong blocks first, then by falling length, each
@@ -168,6 +170,10 @@ struct DevFc2 {
     const int *pair_i, *pair_j, *pair_start;
     const double *blk;        // [n][9]
     const double *rcart;      // [n][3]
+    // unordered atom pairs i <= j: (i, j, pair of (i, j), pair of (j, i)), -1 where
+    // there is none (crystals; n_up = 0 otherwise)
+    int n_up = 0;
+    const int4 *up = nullptr;
 };
 // Mass-scaled copy of force-constant blocks on the device (Phi / sqrt of the
 // product of the n_at masses of each block): raw [n_blk][nval] FP64, atoms
@@ -175,9 +181,10 @@ struct DevFc2 {
 cudaError_t launch_mass_scale(int n_blk, int nval, int n_at, const double *raw, const int *atoms,
                               const double *masses, int out_stride, int f32, void *out, cudaStream_t st);
 cudaError_t launch_mirror_phonons(int nq, int nb, const int *row, const int *conj, const double *nu_c,
-                                  const double2 *eig_c, double *nu, double2 *eig, cudaStream_t st);
-cudaError_t launch_dynmat(const DevFc2 &f, int nb, int nq, const double *qcart,
-                          double2 *D, cudaStream_t st);
+                                  const double2 *eig_c, const double *vel_c, double *nu, double2 *eig, double *vel,
+                                  cudaStream_t st);
+cudaError_t launch_dynmat(const DevFc2 &f, int nb, int nq, size_t n_blk, const double *qcart, double2 *D,
+                          cudaStream_t st);
 cudaError_t launch_jacobi(int nb, int nq, double2 *A, double2 *V, double *nu_thz,
                           double2 *eig_out, int *nonconv, size_t smem_optin, cudaStream_t st);
 // eigh_large.cu: one real symmetric matrix (the Gamma-only D), n up to about
@@ -203,6 +210,13 @@ cudaError_t launch_eigh_large_batch(int n_sys, const EighJob *jobs, void *record
 cudaError_t launch_velocity_diag(const DevFc2 &f, int nb, int nq, const double *qcart,
                                  const double *nu_thz, const double2 *eig, double *vel,
                                  cudaStream_t st);
+
+// velocity.cu: diagonal velocity elements (nb <= 96); table of vel_table_bytes.
+size_t vel_table_bytes(int nq, size_t n_blk);
+int vel_batch(int nq, size_t n_blk);   // q-points of one batch: the table holds them all when this is nq
+cudaError_t launch_vel_diag(const DevFc2 &f, int nb, int nq, size_t n_blk, const double *qcart, const double *nu_scale,
+                            const double *nu_cmp, const double2 *eig, const int *neg, int *src, void *table,
+                            double *out_re, double *out_im, cudaStream_t st);
 
 // linewidths.cu
 struct LwParams {
@@ -433,6 +447,15 @@ cudaError_t bte_solve(int N, const double *G1, const double *g0, const double *n
                       void *work, double scale, double *kappa_out, int &iters, bool &converged, cudaStream_t st);
 
 // kappa.cu
+// From the diagonal elements vre (vim: NULL for a symmetric Phi2) of
+// launch_vel_diag; src[q]: the q-point whose elements q takes; phases: its
+// table exp(-i q.R) [nq][n_blk], or NULL.
+cudaError_t launch_kappa_rta_diag(const DevFc2 &f, int nb, int nq, const double *qcart, const double *nu_thz,
+                                  const double2 *eig, const double *gamma, const int *src, const double *vre,
+                                  const double *vim, const double2 *phases, int n_blk, double T, int classical, double omega_min_thz,
+                                  double degen_tol_thz, double *partial, double *kappa_out, double scale,
+                                  cudaStream_t st);
+// Without scratch beyond the partial sums (kald_kappa_rta_noalloc).
 cudaError_t launch_kappa_rta(const DevFc2 &f, int nb, int nq, const double *qcart,
                              const double *nu_thz, const double2 *eig, const double *gamma,
                              double T, int classical, double omega_min_thz, double degen_tol_thz,

@@ -201,14 +201,192 @@ kappa_rta_kernel(DevFc2 f, int nb, const double *__restrict__ qcart, const doubl
         for (int a = 0; a < 9; ++a) partial[(size_t)q * 9 + a] = acc[a];
 }
 
-__global__ void sum_partials_kernel(int n, const double *__restrict__ partial, double scale,
-                                    double *__restrict__ out) {
-    // one thread per component, fixed order
-    const int a = threadIdx.x;
-    if (a >= 9) return;
+// kappa_RTA of one q per CTA from the diagonal elements: ranks, degenerate
+// sets and their mean c tau formed by one thread per mode; the elements
+// between different modes of one set (rare in disordered cells) over ordered
+// atom pairs whose blocks are summed once, in shared memory, for all pairs of modes.
+// One thread sorting the modes and every (s, s') running over all blocks took
+// 12.2 ms for 32 atoms and 512 q-points; with velocity.cu 2.6 ms now.
+constexpr int kRtaPairs = 8;         // ordered atom pairs per pass
+__global__ void __launch_bounds__(kRtaThreads)
+kappa_rta_diag_kernel(DevFc2 f, int nb, const double *__restrict__ qcart, const double *__restrict__ nu,
+                      const double2 *__restrict__ eig, const double *__restrict__ gamma, const int *__restrict__ src,
+                      const double *__restrict__ vre, const double *__restrict__ vim,
+                      const double2 *__restrict__ phases, int n_blk, double T, int classical, double omega_min_thz,
+                      double degen_tol, double *__restrict__ partial) {
+    __shared__ double v[kMaxNbSmall], ct[kMaxNbSmall];
+    __shared__ int order[kMaxNbSmall], set_of[kMaxNbSmall], start[kMaxNbSmall + 1];   // set_of[s]: -1 takes no part
+    __shared__ unsigned starts[kRtaThreads / 32];
+    __shared__ short2 task[kRtaTasks];
+    __shared__ double2 M[kRtaPairs * 27];
+    __shared__ int n_task_sm;
+    __shared__ double red[(kRtaThreads / 32) * 9];
+    const int q = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const double *g = gamma + (size_t)q * nb;
+    if (tid < nb) v[tid] = nu[(size_t)q * nb + tid];
+    __syncthreads();
+    if (tid < nb) {                                // ascending, ties by index, NaN last
+        const double x = v[tid];
+        int r = 0;
+        for (int t = 0; t < nb; ++t) {
+            const double y = v[t];
+            const bool lt = y < x || (x != x && y == y);
+            const bool gt = y > x || (y != y && x == x);
+            r += lt || (!gt && t < tid);
+        }
+        order[r] = tid;
+    }
+    __syncthreads();
+    const bool first = tid < nb && (tid == 0 || v[order[tid]] - v[order[tid - 1]] >= degen_tol);
+    const unsigned bal = __ballot_sync(0xffffffffu, first);
+    if (lane == 0) starts[warp] = bal;
+    __syncthreads();
+    int sid = __popc(starts[warp] & (0xffffffffu >> (31 - lane))) - 1, n_sets = 0;
+    for (int w = 0; w < kRtaThreads / 32; ++w) {
+        if (w < warp) sid += __popc(starts[w]);
+        n_sets += __popc(starts[w]);
+    }
+    if (first) start[sid] = tid;
+    if (tid == 0) start[n_sets] = nb;
+    __syncthreads();
+    int many = 0;
+    if (tid < n_sets) {
+        double acc = 0.0;
+        int cnt = 0;
+        for (int b = start[tid]; b < start[tid + 1]; ++b) {
+            const int s = order[b];
+            const bool ok = (v[s] > omega_min_thz) && (g[s] > 0.0);
+            set_of[s] = ok ? tid : -1;
+            if (ok) { acc += heat_cap(kTwoPi * v[s], T, classical) / (2.0 * g[s]); ++cnt; }
+        }
+        ct[tid] = cnt ? acc / cnt : 0.0;
+        many = cnt > 1;
+    }
+    many = __syncthreads_or(many);
+    double acc[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+    if (tid < nb && set_of[tid] >= 0) {
+        const size_t o = ((size_t)src[q] * nb + tid) * 3;
+        const double sc = kEvA2AmuPs2 / (2.0 * (kTwoPi * v[tid]));
+        const double w8 = ct[set_of[tid]] * sc * sc;
+        for (int a = 0; a < 3; ++a)
+            for (int b = 0; b < 3; ++b)
+                acc[3 * a + b] = w8 * (vre[o + a] * vre[o + b] + (vim ? vim[o + a] * vim[o + b] : 0.0));
+    }
+    if (many) {
+        // pairs of different modes inside a set: s < s' counted twice when dD is
+        // Hermitian (symmetric Phi2), every ordered pair otherwise
+        const bool herm = vim == nullptr;
+        const double qx = qcart[3 * q], qy = qcart[3 * q + 1], qz = qcart[3 * q + 2];
+        const double2 *E = eig + (size_t)q * nb * nb;
+        for (int skip = 0;;) {
+            if (tid == 0) {
+                int n = 0, seen = 0;
+                for (int d = 0; d < n_sets && n < kRtaTasks; ++d)
+                    for (int a = start[d]; a < start[d + 1] && n < kRtaTasks; ++a)
+                        for (int b = herm ? a + 1 : start[d]; b < start[d + 1] && n < kRtaTasks; ++b) {
+                            const int s = order[a], t = order[b];
+                            if (a == b || set_of[s] < 0 || set_of[t] < 0) continue;
+                            if (seen++ < skip) continue;
+                            task[n++] = make_short2((short)s, (short)t);
+                        }
+                n_task_sm = n;
+            }
+            __syncthreads();
+            const int n_task = n_task_sm;
+            if (n_task == 0) break;
+            double2 V[8][3];
+            for (int u = 0; u < 8; ++u)
+                for (int a = 0; a < 3; ++a) V[u][a] = make_double2(0.0, 0.0);
+            for (int p0 = 0; p0 < f.n_pairs; p0 += kRtaPairs) {
+                const int n_p = min(kRtaPairs, f.n_pairs - p0);
+                __syncthreads();
+                // (several threads per pair and element where there are few pairs)
+                const int parts = max(1, min(kRtaThreads / (9 * n_p), kRtaPairs / n_p));
+                for (int x = tid; x < 9 * n_p * parts; x += kRtaThreads) {
+                    const int pp = x / 9, part = pp / n_p, p = pp - part * n_p, ab = x - 9 * pp;
+                    double2 m[3];
+                    for (int a = 0; a < 3; ++a) m[a] = make_double2(0.0, 0.0);
+                    for (int b = f.pair_start[p0 + p] + part; b < f.pair_start[p0 + p + 1]; b += parts) {
+                        const double *R = f.rcart + 3 * (size_t)b;
+                        double sn, cn;
+                        if (phases) {
+                            const double2 z = phases[(size_t)q * n_blk + b];
+                            cn = z.x;
+                            sn = -z.y;
+                        } else {
+                            sincos(qx * R[0] + qy * R[1] + qz * R[2], &sn, &cn);
+                        }
+                        const double bv = f.blk[9 * (size_t)b + ab];
+                        // (-i R_a) exp(-i q.R) = -R_a sin - i R_a cos
+                        for (int a = 0; a < 3; ++a) {
+                            m[a].x -= R[a] * (bv * sn);
+                            m[a].y -= R[a] * (bv * cn);
+                        }
+                    }
+                    for (int a = 0; a < 3; ++a) M[27 * pp + 3 * ab + a] = m[a];
+                }
+                __syncthreads();
+                if (parts > 1) {
+                    for (int x = tid; x < 27 * n_p; x += kRtaThreads) {
+                        double2 m = M[x];
+                        for (int k = 1; k < parts; ++k) {
+                            const double2 z = M[27 * n_p * k + x];
+                            m.x += z.x;
+                            m.y += z.y;
+                        }
+                        M[x] = m;
+                    }
+                    __syncthreads();
+                }
+                for (int u = 0; u < 8; ++u) {
+                    const int x = tid + u * kRtaThreads;
+                    if (x >= n_task) break;
+                    const double2 *es = E + (size_t)task[x].x * nb, *et = E + (size_t)task[x].y * nb;
+                    for (int p = 0; p < n_p; ++p) {
+                        const double2 *ei = es + 3 * f.pair_i[p0 + p], *ej = et + 3 * f.pair_j[p0 + p];
+                        for (int a = 0; a < 3; ++a)
+                            for (int b = 0; b < 3; ++b) {
+                                const double2 P = cmulc(ei[a], ej[b]);
+                                for (int c = 0; c < 3; ++c) {
+                                    const double2 z = M[27 * p + 3 * (3 * a + b) + c];
+                                    V[u][c].x += P.x * z.x - P.y * z.y;
+                                    V[u][c].y += P.x * z.y + P.y * z.x;
+                                }
+                            }
+                    }
+                }
+            }
+            for (int u = 0; u < 8; ++u) {
+                const int x = tid + u * kRtaThreads;
+                if (x >= n_task) break;
+                const int s = task[x].x, t = task[x].y;
+                const double sc = kEvA2AmuPs2 / (2.0 * sqrt((kTwoPi * v[s]) * (kTwoPi * v[t])));
+                const double w8 = (herm ? 2.0 : 1.0) * ct[set_of[s]] * sc * sc;
+                for (int a = 0; a < 3; ++a)
+                    for (int b = 0; b < 3; ++b)
+                        acc[3 * a + b] += w8 * (V[u][a].x * V[u][b].x + V[u][a].y * V[u][b].y);
+            }
+            skip += n_task;
+            __syncthreads();
+            if (n_task < kRtaTasks) break;
+        }
+    }
+    block_reduce9(acc, red);
+    if (tid == 0)
+        for (int a = 0; a < 9; ++a) partial[(size_t)q * 9 + a] = acc[a];
+}
+
+// out[a] = scale * sum of n partial sums: one warp per component, every lane
+// its share in order, then a fixed tree (one thread per component took 12 us
+// for 216 partial sums and grew with their number).
+__global__ void __launch_bounds__(288)
+sum_partials_kernel(int n, const double *__restrict__ partial, double scale, double *__restrict__ out) {
+    const int a = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double t = 0.0;
-    for (int x = 0; x < n; ++x) t += partial[(size_t)x * 9 + a];
-    out[a] = t * scale;
+#pragma unroll 4
+    for (int x = lane; x < n; x += 32) t += partial[(size_t)x * 9 + a];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) out[a] = t * scale;
 }
 
 // ---------------------------------------------------------------- QHGK
@@ -396,7 +574,19 @@ cudaError_t launch_kappa_rta(const DevFc2 &f, int nb, int nq, const double *qcar
                              double *partial, double *kappa_out, double scale, cudaStream_t st) {
     kappa_rta_kernel<<<counted(nq), kRtaThreads, 0, st>>>(f, nb, qcart, nu_thz, eig, gamma, T, classical,
                                                 omega_min_thz, degen_tol_thz, partial);
-    sum_partials_kernel<<<counted(1), 32, 0, st>>>(nq, partial, scale, kappa_out);
+    sum_partials_kernel<<<counted(1), 288, 0, st>>>(nq, partial, scale, kappa_out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_kappa_rta_diag(const DevFc2 &f, int nb, int nq, const double *qcart, const double *nu_thz,
+                                  const double2 *eig, const double *gamma, const int *src, const double *vre,
+                                  const double *vim, const double2 *phases, int n_blk, double T, int classical, double omega_min_thz,
+                                  double degen_tol_thz, double *partial, double *kappa_out, double scale,
+                                  cudaStream_t st) {
+    kappa_rta_diag_kernel<<<counted(nq), kRtaThreads, 0, st>>>(f, nb, qcart, nu_thz, eig, gamma, src, vre, vim,
+                                                               phases, n_blk, T, classical, omega_min_thz,
+                                                               degen_tol_thz, partial);
+    sum_partials_kernel<<<counted(1), 288, 0, st>>>(nq, partial, scale, kappa_out);
     return cudaGetLastError();
 }
 
@@ -431,7 +621,7 @@ cudaError_t launch_qhgk(const DevFc2Dist &f, int nb, const double *nu_thz, const
     const int nblk = (nb + rows - 1) / rows;
     qhgk_pairsum_kernel<<<counted(nblk), 256, 0, st>>>(nb, W, omega, gamma, T, classical,
                                               kTwoPi * degen_tol_thz, bandwidth_w, threshold_w, rows, partial);
-    sum_partials_kernel<<<counted(1), 32, 0, st>>>(nblk, partial, scale, kappa_out);
+    sum_partials_kernel<<<counted(1), 288, 0, st>>>(nblk, partial, scale, kappa_out);
     return cudaGetLastError();
 }
 

@@ -22,28 +22,49 @@ __device__ __forceinline__ double2 cmulc(double2 a, double2 b) {   // conj(a) * 
     return make_double2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
 }
 
-// D[q] (nb x nb, row-major) from fc2 blocks grouped by atom pair: one output
-// element (pair, a, b) per thread iteration, blocks summed in a fixed order.
-// Grid: x strides over the elements of one q, y over the q-points.
-__global__ void dynmat_kernel(DevFc2 f, int nb, int nq, const double *__restrict__ qcart,
-                              double2 *__restrict__ D) {
-    const int n_elem = f.n_pairs * 9;
+// D[q] (nb x nb, row-major) from fc2 blocks grouped by atom pair: L lanes per
+// pair share its blocks (one sincos per block, nine elements each), then add
+// their sums in a fixed tree.  Grid: x strides over the pairs of one q, y over
+// the q-points.  One thread per element walked all blocks of its pair, a
+// sincos each: 89 us for the one-atom cell (79 blocks in one pair), 0.45 ms for
+// 32 atoms and 512 q-points; 15 us and 0.17 ms now.
+template <int L>
+__global__ void __launch_bounds__(256)
+dynmat_kernel(DevFc2 f, int nb, int nq, const double *__restrict__ qcart, double2 *__restrict__ D) {
+    const int sub = threadIdx.x % L, per = blockDim.x / L;
     for (int q = blockIdx.y; q < nq; q += gridDim.y) {
         const double qx = qcart[3 * q], qy = qcart[3 * q + 1], qz = qcart[3 * q + 2];
         double2 *Dq = D + (size_t)q * nb * nb;
-        for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n_elem; e += gridDim.x * blockDim.x) {
-            const int p = e / 9, ab = e % 9;
-            const int i = f.pair_i[p], j = f.pair_j[p];
-            double2 acc = make_double2(0.0, 0.0);
-            for (int b = f.pair_start[p]; b < f.pair_start[p + 1]; ++b) {
-                const double *R = f.rcart + 3 * b;
+        for (int p0 = blockIdx.x * per; p0 < f.n_pairs; p0 += gridDim.x * per) {
+            const int p = p0 + threadIdx.x / L;
+            const bool in = p < f.n_pairs;                 // every lane takes part in the shuffles
+            double2 acc[9];
+#pragma unroll
+            for (int e = 0; e < 9; ++e) acc[e] = make_double2(0.0, 0.0);
+            const int b1 = in ? f.pair_start[p + 1] : 0;
+            for (int b = in ? f.pair_start[p] + sub : 0; b < b1; b += L) {
+                const double *R = f.rcart + 3 * (size_t)b;
                 double s, c;
                 sincos(qx * R[0] + qy * R[1] + qz * R[2], &s, &c);
-                const double v = f.blk[9 * b + ab];
-                acc.x += v * c;            // exp(-i q.R) = c - i s
-                acc.y -= v * s;
+#pragma unroll
+                for (int e = 0; e < 9; ++e) {              // exp(-i q.R) = c - i s
+                    const double v = f.blk[9 * (size_t)b + e];
+                    acc[e].x = fma(v, c, acc[e].x);
+                    acc[e].y = fma(-v, s, acc[e].y);
+                }
             }
-            Dq[(size_t)(3 * i + ab / 3) * nb + 3 * j + ab % 3] = acc;
+#pragma unroll
+            for (int o = L / 2; o > 0; o >>= 1)
+#pragma unroll
+                for (int e = 0; e < 9; ++e) {
+                    acc[e].x += __shfl_xor_sync(0xffffffffu, acc[e].x, o);
+                    acc[e].y += __shfl_xor_sync(0xffffffffu, acc[e].y, o);
+                }
+            if (!in) continue;
+            double2 *row = Dq + (size_t)(3 * f.pair_i[p]) * nb + 3 * f.pair_j[p];
+#pragma unroll
+            for (int e = 0; e < 9; ++e)
+                if (e % L == sub) row[(size_t)(e / 3) * nb + e % 3] = acc[e];
         }
     }
 }
@@ -464,7 +485,8 @@ hermitian_ql_kernel(int n, const double2 *__restrict__ Ain, double2 *__restrict_
     }
 }
 
-// Diagonal Hellmann-Feynman velocity of every mode at every q.
+// Diagonal Hellmann-Feynman velocity of every mode at every q (nb > 96; smaller
+// cells: velocity.cu).
 __global__ void velocity_kernel(DevFc2 f, int nb, const double *__restrict__ qcart,
                                 const double *__restrict__ nu, const double2 *__restrict__ eig,
                                 double *__restrict__ vel) {
@@ -540,15 +562,18 @@ cudaError_t launch_mass_scale(int n_blk, int nval, int n_at, const double *raw, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_dynmat(const DevFc2 &f, int nb, int nq, const double *qcart, double2 *D,
+cudaError_t launch_dynmat(const DevFc2 &f, int nb, int nq, size_t n_blk, const double *qcart, double2 *D,
                           cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(D, 0, sizeof(double2) * (size_t)nq * nb * nb, st);
     if (e != cudaSuccess) return e;
+    // lanes per pair: a warp for pairs of many blocks (small cells), else four;
     // enough CTAs along x to fill the GPU when there are few q-points
-    const int n_elem = f.n_pairs * 9;
-    const int gx = std::max(1, std::min((n_elem + 255) / 256, std::max(1, 1216 / std::max(nq, 1))));
+    const int lanes = n_blk > 8 * (size_t)std::max(f.n_pairs, 1) ? 32 : 4;
+    const int per = 256 / lanes;
+    const int gx = std::max(1, std::min((f.n_pairs + per - 1) / per, std::max(1, 1216 / std::max(nq, 1))));
     const dim3 grid((unsigned)gx, (unsigned)std::min(nq, 65535));
-    dynmat_kernel<<<counted(grid), 256, 0, st>>>(f, nb, nq, qcart, D);
+    if (lanes == 32) dynmat_kernel<32><<<counted(grid), 256, 0, st>>>(f, nb, nq, qcart, D);
+    else dynmat_kernel<4><<<counted(grid), 256, 0, st>>>(f, nb, nq, qcart, D);
     return cudaGetLastError();
 }
 
@@ -590,7 +615,8 @@ cudaError_t launch_jacobi(int nb, int nq, double2 *A, double2 *V, double *nu_thz
 // representatives, row row[q].
 __global__ void mirror_phonons_kernel(int nq, int nb, const int *__restrict__ row, const int *__restrict__ conj,
                                       const double *__restrict__ nu_c, const double2 *__restrict__ eig_c,
-                                      double *__restrict__ nu, double2 *__restrict__ eig) {
+                                      const double *__restrict__ vel_c, double *__restrict__ nu,
+                                      double2 *__restrict__ eig, double *__restrict__ vel) {
     const size_t per = (size_t)nb * nb;
     for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < (size_t)nq * per;
          x += (size_t)gridDim.x * blockDim.x) {
@@ -599,14 +625,20 @@ __global__ void mirror_phonons_kernel(int nq, int nb, const int *__restrict__ ro
         const double2 v = eig_c[(size_t)row[q] * per + e];
         eig[x] = conj[q] ? make_double2(v.x, -v.y) : v;
         if (e < (size_t)nb) nu[(size_t)q * nb + e] = nu_c[(size_t)row[q] * nb + e];
+        if (vel && e < (size_t)nb)                             // v(-q) = -v(q)
+            for (int a = 0; a < 3; ++a) {
+                const double u = vel_c[((size_t)row[q] * nb + e) * 3 + a];
+                vel[((size_t)q * nb + e) * 3 + a] = conj[q] ? -u : u;
+            }
     }
 }
 
 cudaError_t launch_mirror_phonons(int nq, int nb, const int *row, const int *conj, const double *nu_c,
-                                  const double2 *eig_c, double *nu, double2 *eig, cudaStream_t st) {
+                                  const double2 *eig_c, const double *vel_c, double *nu, double2 *eig, double *vel,
+                                  cudaStream_t st) {
     const size_t n = (size_t)nq * nb * nb;
     const int grid = (int)std::min<size_t>((n + 255) / 256, 4096);
-    mirror_phonons_kernel<<<counted(grid), 256, 0, st>>>(nq, nb, row, conj, nu_c, eig_c, nu, eig);
+    mirror_phonons_kernel<<<counted(grid), 256, 0, st>>>(nq, nb, row, conj, nu_c, eig_c, vel_c, nu, eig, vel);
     return cudaGetLastError();
 }
 

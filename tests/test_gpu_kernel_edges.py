@@ -101,3 +101,29 @@ def test_phase_space_sliding_windows(k, nb, mesh, sigma, precision, tol):
         g_o = an.phase_space(mesh, nu, 300.0, sigma, 3.0)
         g = kk.kald_phase_space(ctx, s, mesh, nu, opt).reshape(g_o.shape)
     assert _rel(g, g_o) < tol
+
+
+@pytest.mark.parametrize("cell,mesh", [("binary", (3, 2, 2)), ("fcc4", (2, 2, 3)), ("fcc20", (2, 1, 1))])
+@pytest.mark.parametrize("asym", [0.0, 0.05])
+def test_kappa_rta_from_diagonal_elements(k, cell, mesh, asym):
+    """Two, four and 20 atoms: degenerate sets (the off-diagonal elements), a
+    Phi2 without the (i, j) <-> (j, i) symmetry (complex diagonal elements, an
+    atom pair listed in one order only), and eigenvectors at -q that are not the
+    conjugates of those at q."""
+    from dataclasses import replace
+    from oracle import conductivity as co
+    kk, ctx = k
+    s = ki.small_binary(mesh=mesh).systems[0] if cell == "binary" else \
+        ki.fcc_supercell_system(1 if cell == "fcc4" else (5, 1, 1), seed=7)
+    nu, eig = ph.phonons(s, mesh)
+    rng = np.random.default_rng(3)
+    eig = eig * np.exp(2j * np.pi * rng.random(nu.shape))[..., None]
+    g = np.where(nu > 0.01, 0.1 + 0.02 * nu ** 2, 0.0)
+    if asym:
+        fc2 = s.fc2 * (1.0 + asym * rng.standard_normal(s.fc2.shape))
+        keep = ~((s.fc2_idx[:, 0] == 1) & (s.fc2_idx[:, 1] == 0))
+        s = replace(s, fc2=fc2[keep], fc2_idx=s.fc2_idx[keep])
+    kap_o = co.kappa_rta(s, mesh, nu, eig, g, 300.0)
+    opt = kk.Options(temperature_K=300.0, sigma_thz=0.1)
+    kap = kk.kald_kappa_rta(ctx, s, mesh, nu, eig, g, opt)
+    np.testing.assert_allclose(kap, kap_o, rtol=1e-10, atol=1e-10 * np.abs(kap_o).max())
