@@ -1777,6 +1777,21 @@ kald_status kald_phase_space(kald_ctx *ctx, const kald_system *sys, const int32_
     return finish(ctx, "kald_phase_space");
 }
 
+// Workspace of the generalised velocities of one Gamma-only system.
+static size_t qhgk_work_bytes(int nb) {
+    return ws_round(sizeof(double) * 4 * (size_t)nb) + ws_round(sizeof(double) * 3 * (size_t)nb * nb) +
+           ws_round(oz_work_bytes(nb)) + ws_round(16);
+}
+static QhgkWork take_qhgk_work(kald_ctx *ctx, int nb) {
+    QhgkWork w;
+    double *m = static_cast<double *>(ws_take(ctx, sizeof(double) * 4 * (size_t)nb));
+    w.modes = {m, m + nb, m + 2 * (size_t)nb, m + 3 * (size_t)nb};
+    w.W = static_cast<double *>(ws_take(ctx, sizeof(double) * 3 * (size_t)nb * nb));
+    w.oz = ws_take(ctx, oz_work_bytes(nb));
+    w.err = static_cast<int *>(ws_take(ctx, 16));
+    return w;
+}
+
 kald_status kald_diffusivity(kald_ctx *ctx, int32_t n_sys, const kald_system *sys, const double *nu_thz,
                              const double *eigvec, const double *gamma, const kald_options *opt, double *D) {
     if (!ctx) return KALD_E_INVALID;
@@ -1802,8 +1817,7 @@ kald_status kald_diffusivity(kald_ctx *ctx, int32_t n_sys, const kald_system *sy
             }
         for (int i = 0; i < h.n_atoms; ++i) row_start[i + 1] += row_start[i];
         size_t need = bytes_of(row_start) + bytes_of(col_j) + scaled_bytes(h.fc2_blk, h.fc2_atoms, h, 9, 9, 0) +
-                      bytes_of(h.fc2_dist) + ws_round(sizeof(double) * nn) + 2 * ws_round(sizeof(double) * 3 * nn) +
-                      ws_round(sizeof(double) * nb) * 2;
+                      bytes_of(h.fc2_dist) + qhgk_work_bytes(nb) + ws_round(sizeof(double) * nb);
         if (!d_nu) need += ws_round(sizeof(double) * nb);
         if (!d_eig) need += ws_round(sizeof(double2) * nn);
         if (!d_g) need += ws_round(sizeof(double) * nb);
@@ -1817,17 +1831,19 @@ kald_status kald_diffusivity(kald_ctx *ctx, int32_t n_sys, const kald_system *sy
         const double *nu_d = stage_in(ctx, nu_thz + off_nb, (size_t)nb, d_nu);
         const double2 *eig_d = stage_in(ctx, reinterpret_cast<const double2 *>(eigvec) + off_eig, nn, d_eig);
         const double *g_d = stage_in(ctx, gamma + off_nb, (size_t)nb, d_g);
-        double *E = static_cast<double *>(ws_take(ctx, sizeof(double) * nn));
-        double *B = static_cast<double *>(ws_take(ctx, sizeof(double) * 3 * nn));
-        double *W = static_cast<double *>(ws_take(ctx, sizeof(double) * 3 * nn));
-        double *omega = static_cast<double *>(ws_take(ctx, sizeof(double) * nb));
+        const QhgkWork work = take_qhgk_work(ctx, nb);
+        cudaMemsetAsync(work.err, 0, sizeof(int), ctx->stream);
+        if (h.fc2_symmetric < 0) h.fc2_symmetric = fc2_symmetric(&sys[x]) ? 1 : 0;
         double *D_d = d_D ? D + off_nb : static_cast<double *>(ws_take(ctx, sizeof(double) * nb));
         cudaError_t e = launch_diffusivity(f, nb, nu_d, eig_d, g_d, opt->omega_min_thz,
-                                           kTwoPi * opt->qhgk_bandwidth_thz, kTwoPi * opt->qhgk_threshold_thz, E, B,
-                                           W, omega, D_d, ctx->stream);
+                                           kTwoPi * opt->qhgk_bandwidth_thz, kTwoPi * opt->qhgk_threshold_thz,
+                                           h.fc2_symmetric, work, D_d, ctx->smem_optin, ctx->wait_limit, ctx->stream);
         if (e != cudaSuccess) return cuda_check(ctx, e, "kald_diffusivity launch");
+        int errf = 0;
+        cudaMemcpyAsync(&errf, work.err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
         if (!d_D) cudaMemcpyAsync(D + off_nb, D_d, sizeof(double) * nb, cudaMemcpyDeviceToHost, ctx->stream);
         if ((st = finish(ctx, "kald_diffusivity"))) return st;
+        if (errf) return fail(ctx, KALD_E_TIMEOUT, "kald_diffusivity: a tensor-core pipeline wait expired");
         off_nb += nb;
         off_eig += nn;
     }
@@ -2048,8 +2064,9 @@ kald_status kald_kappa_qhgk(kald_ctx *ctx, int32_t n_sys, const kald_system *sys
         it.off_nb = off_nb;
         it.off_eig = off_eig;
         need += bytes_of(it.row_start) + bytes_of(it.col_j) + scaled_bytes(h.fc2_blk, h.fc2_atoms, h, 9, 9, 0) +
-                bytes_of(h.fc2_dist) + ws_round(sizeof(double) * nn) + 2 * ws_round(sizeof(double) * 3 * nn) +
-                ws_round(sizeof(double) * (9 * (size_t)it.n_partial + nb)) + ws_round(72);
+                bytes_of(h.fc2_dist) + qhgk_work_bytes(nb) + ws_round(sizeof(double) * 9 * (size_t)it.n_partial) +
+                ws_round(72);
+        if (h.fc2_symmetric < 0) h.fc2_symmetric = fc2_symmetric(&sys[x]) ? 1 : 0;
         if (!d_nu) need += ws_round(sizeof(double) * nb);
         if (!d_eig) need += ws_round(sizeof(double2) * nn);
         if (!d_g) need += ws_round(sizeof(double) * nb);
@@ -2061,7 +2078,8 @@ kald_status kald_kappa_qhgk(kald_ctx *ctx, int32_t n_sys, const kald_system *sys
         DevFc2Dist f;
         const double *nu, *g;
         const double2 *eig;
-        double *E, *B, *W, *partial, *k;
+        QhgkWork work;
+        double *partial, *k;
     };
     std::vector<Dev> devs(n_sys);
     for (int x = 0; x < n_sys; ++x) {
@@ -2078,10 +2096,9 @@ kald_status kald_kappa_qhgk(kald_ctx *ctx, int32_t n_sys, const kald_system *sys
         dv.nu = stage_in(ctx, nu_thz + it.off_nb, (size_t)nb, d_nu);
         dv.eig = stage_in(ctx, reinterpret_cast<const double2 *>(eigvec) + it.off_eig, nn, d_eig);
         dv.g = stage_in(ctx, gamma + it.off_nb, (size_t)nb, d_g);
-        dv.E = static_cast<double *>(ws_take(ctx, sizeof(double) * nn));
-        dv.B = static_cast<double *>(ws_take(ctx, sizeof(double) * 3 * nn));
-        dv.W = static_cast<double *>(ws_take(ctx, sizeof(double) * 3 * nn));
-        dv.partial = static_cast<double *>(ws_take(ctx, sizeof(double) * (9 * (size_t)it.n_partial + nb)));
+        dv.work = take_qhgk_work(ctx, nb);
+        cudaMemsetAsync(dv.work.err, 0, sizeof(int), ctx->stream);
+        dv.partial = static_cast<double *>(ws_take(ctx, sizeof(double) * 9 * (size_t)it.n_partial));
         dv.k = d_k ? kappa + 9 * (size_t)x : static_cast<double *>(ws_take(ctx, 72));
     }
     std::vector<cudaStream_t> lanes;
@@ -2092,8 +2109,8 @@ kald_status kald_kappa_qhgk(kald_ctx *ctx, int32_t n_sys, const kald_system *sys
         const HostSystem &h = *items[x].hp;
         e = launch_qhgk(dv.f, h.nb, dv.nu, dv.eig, dv.g, opt->temperature_K, opt->classical, opt->omega_min_thz,
                         opt->degen_tol_thz, kTwoPi * opt->qhgk_bandwidth_thz, kTwoPi * opt->qhgk_threshold_thz,
-                        dv.E, dv.B, dv.W, dv.partial, items[x].n_partial, dv.k, kKappaSI / h.volume,
-                        lanes[x % lanes.size()]);
+                        h.fc2_symmetric, vgen && x == 0, dv.work, dv.partial, items[x].n_partial, dv.k,
+                        kKappaSI / h.volume, ctx->smem_optin, ctx->wait_limit, lanes[x % lanes.size()]);
     }
     const cudaError_t ej = join_lanes(ctx, lanes);
     if (e == cudaSuccess) e = ej;
@@ -2105,10 +2122,15 @@ kald_status kald_kappa_qhgk(kald_ctx *ctx, int32_t n_sys, const kald_system *sys
         if (!d_k) cudaMemcpyAsync(kappa + 9 * (size_t)x, devs[x].k, 72, cudaMemcpyDeviceToHost, ctx->stream);
     if (vgen) {
         const size_t nn0 = (size_t)items[0].hp->nb * items[0].hp->nb;
-        cudaMemcpyAsync(vgen, devs[0].W, sizeof(double) * 3 * nn0,
+        cudaMemcpyAsync(vgen, devs[0].work.W, sizeof(double) * 3 * nn0,
                         d_v ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, ctx->stream);
     }
+    std::vector<int> errf(n_sys, 0);
+    for (int x = 0; x < n_sys; ++x)
+        cudaMemcpyAsync(&errf[x], devs[x].work.err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
     if ((st = finish(ctx, "kald_kappa_qhgk"))) return st;
+    for (int x = 0; x < n_sys; ++x)
+        if (errf[x]) return fail(ctx, KALD_E_TIMEOUT, "kald_kappa_qhgk: a tensor-core pipeline wait expired");
     return KALD_OK;
 }
 

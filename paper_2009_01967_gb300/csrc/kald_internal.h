@@ -468,13 +468,29 @@ struct DevFc2Dist {
     const double *blk;        // [n][9] Phi2/sqrt(mi mj)
     const double *dist;       // [n][3] x_i - x_j - L
 };
+// Tables per mode and work buffers of the generalised velocities.
+struct QhgkModes {
+    double *omega, *occ, *heat, *fac;   // [nb] each
+};
+struct QhgkWork {
+    QhgkModes modes;
+    double *W;                // [3][nb][nb]
+    void *oz;                 // oz_work_bytes(nb)
+    int *err;                 // bounded-wait failures
+};
+// qhgk_gemm.cu: W_a = E B_a^T scaled by fac per mode, over B_a [3][n][n] in BW;
+// antisym: the tiles on and above the diagonal only, mirrored when fill.
+size_t oz_work_bytes(int n);
+cudaError_t launch_oz_gemm(int n, const double2 *E, double *BW, const double *fac, int antisym, int fill, void *work,
+                           int *err, uint32_t wait_limit, cudaStream_t st);
 // Mode diffusivity D [nb] (A^2/ps) of a Gamma-only system (generalised
-// velocity as for QHGK, then the per-mode sum); omega [nb] scratch.
+// velocity as for QHGK, then the per-mode sum).
 // bandwidth_w > 0: fixed width in place of gamma + gamma'; threshold_w > 0:
 // pairs with |d omega| > threshold left out (rad/ps, as for launch_qhgk).
 cudaError_t launch_diffusivity(const DevFc2Dist &f, int nb, const double *nu_thz, const double2 *eig,
                                const double *gamma, double omega_min_thz, double bandwidth_w, double threshold_w,
-                               double *Ework, double *Bwork, double *W, double *omega, double *D, cudaStream_t st);
+                               int antisym, const QhgkWork &w, double *D, size_t smem_optin, uint32_t wait_limit,
+                               cudaStream_t st);
 // Phase space per mode (linewidths.cu): g [nq * nb] in ps; work of
 // phase_space_bytes (sorted modes, counts, partial sums of the q' chunks).
 size_t phase_space_bytes(int nb, int nq, int sm_count);
@@ -482,10 +498,10 @@ cudaError_t launch_phase_space(const LwParams &p, const LwDev &d, int fp32, int 
                                cudaStream_t st);
 cudaError_t launch_qhgk(const DevFc2Dist &f, int nb, const double *nu_thz, const double2 *eig,
                         const double *gamma, double T, int classical, double omega_min_thz,
-                        double degen_tol_thz, double bandwidth_w, double threshold_w,
-                        double *Ework /*[nb*nb]*/, double *Bwork /*[3][nb][nb]*/,
-                        double *W /*[3][nb][nb]*/, double *partial, int n_partial,
-                        double *kappa_out /*[9]*/, double scale, cudaStream_t st);
+                        double degen_tol_thz, double bandwidth_w, double threshold_w, int antisym, int fill,
+                        const QhgkWork &w, double *partial /*[n_partial][9]*/, int n_partial,
+                        double *kappa_out /*[9]*/, double scale, size_t smem_optin, uint32_t wait_limit,
+                        cudaStream_t st);
 // gamma(nu) by a not-a-knot cubic spline through the valid source modes
 // (interp.cu); work of interp_work_bytes(n_src).
 size_t interp_work_bytes(int n_src);

@@ -390,136 +390,105 @@ sum_partials_kernel(int n, const double *__restrict__ partial, double scale, dou
 }
 
 // ---------------------------------------------------------------- QHGK
-// E[mu][d] = Re eig[0][mu][d]
-__global__ void real_part_kernel(size_t n, const double2 *__restrict__ eig, double *__restrict__ E) {
-    for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < n;
-         x += (size_t)gridDim.x * blockDim.x)
-        E[x] = eig[x].x;
-}
-
-// B_a[d][mu] = sum_e A_a[d][e] E[mu][e], rows d = 3 i + a' gathered over the
-// blocks of atom i (CSR): one thread per (i, a', mu), three outputs (a).
-__global__ void sparse_ae_kernel(DevFc2Dist f, int nb, const double *__restrict__ E,
-                                 double *__restrict__ B) {
-    const size_t n = (size_t)f.n_rows * 3 * nb;
-    for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < n;
-         x += (size_t)gridDim.x * blockDim.x) {
-        const int mu = (int)(x % nb);
-        const int ra = (int)(x / nb);            // 3 i + a'
-        const int i = ra / 3, ap = ra % 3;
-        const double *Em = E + (size_t)mu * nb;
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-        for (int b = f.row_start[i]; b < f.row_start[i + 1]; ++b) {
-            const int j = f.col_j[b];
-            const double *blk = f.blk + 9 * b + 3 * ap;
-            const double t = blk[0] * Em[3 * j] + blk[1] * Em[3 * j + 1] + blk[2] * Em[3 * j + 2];
-            s0 += f.dist[3 * b] * t;
-            s1 += f.dist[3 * b + 1] * t;
-            s2 += f.dist[3 * b + 2] * t;
-        }
-        B[(size_t)ra * nb + mu] = s0;
-        B[((size_t)nb + ra) * nb + mu] = s1;
-        B[((size_t)2 * nb + ra) * nb + mu] = s2;
-    }
-}
-
-// W_a[mu][mu'] = sum_d E[mu][d] B_a[d][mu'] * C / (2 sqrt(w w')), masked.
-// 64 x 64 output tile per CTA, 16 x 16 threads with 4 x 4 outputs each.
+// B_a[mu][d] = sum_e A_a[d][e] E[mu][e], rows d = 3 i + a' gathered over the
+// blocks of atom i (CSR).  CTA = MU modes, their eigenvectors in shared memory
+// so that a block's values are read once for all of them; one thread per row,
+// three outputs (a) per mode.  Bound: FP64 units, 6 FMA per (block, row, mode).
+// (SMEM false: one mode per CTA read from global memory, for eigenvectors that
+// do not fit.)
+template <int MU, bool SMEM = true>
 __global__ void __launch_bounds__(256)
-dgemm_w_kernel(int nb, const double *__restrict__ E, const double *__restrict__ B,
-               const double *__restrict__ omega, double *__restrict__ W) {
-    __shared__ double As[16][64 + 1];   // As[k][m] = E[m0 + m][k0 + k]
-    __shared__ double Bs[16][64];       // Bs[k][n] = B[k0 + k][n0 + n]
-    const int a = blockIdx.z;
-    const double *Ba = B + (size_t)a * nb * nb;
-    const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    double acc[4][4] = {};
-    for (int k0 = 0; k0 < nb; k0 += 16) {
-        for (int x = threadIdx.x; x < 16 * 64; x += 256) {
-            const int m = x / 16, k = x % 16;
-            As[k][m] = (m0 + m < nb && k0 + k < nb) ? E[(size_t)(m0 + m) * nb + k0 + k] : 0.0;
-            const int kk = x / 64, n = x % 64;
-            Bs[kk][n] = (k0 + kk < nb && n0 + n < nb) ? Ba[(size_t)(k0 + kk) * nb + n0 + n] : 0.0;
+sparse_ae_kernel(DevFc2Dist f, int nb, const double2 *__restrict__ eig, double *__restrict__ B) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double *E = reinterpret_cast<double *>(smem_raw);          // [MU][nb]
+    const int mu0 = blockIdx.x * MU;
+    for (int m = 0; m < (SMEM ? MU : 0); ++m)
+        for (int x = threadIdx.x; x < nb; x += blockDim.x)
+            E[m * nb + x] = mu0 + m < nb ? eig[(size_t)(mu0 + m) * nb + x].x : 0.0;
+    __syncthreads();
+    for (int ra = threadIdx.x; ra < 3 * f.n_rows; ra += blockDim.x) {       // 3 i + a'
+        const int i = ra / 3, ap = ra - 3 * i;
+        double s[MU][3];
+#pragma unroll
+        for (int m = 0; m < MU; ++m) s[m][0] = s[m][1] = s[m][2] = 0.0;
+        for (int b = f.row_start[i]; b < f.row_start[i + 1]; ++b) {
+            const int j = 3 * f.col_j[b];
+            const double *blk = f.blk + 9 * (size_t)b + 3 * ap, *R = f.dist + 3 * (size_t)b;
+            const double v0 = blk[0], v1 = blk[1], v2 = blk[2], r0 = R[0], r1 = R[1], r2 = R[2];
+#pragma unroll
+            for (int m = 0; m < MU; ++m) {
+                double e0, e1, e2;
+                if constexpr (SMEM) {
+                    const double *e = E + m * nb + j;
+                    e0 = e[0]; e1 = e[1]; e2 = e[2];
+                } else {
+                    const double2 *e = eig + (size_t)(mu0 + m) * nb + j;
+                    e0 = e[0].x; e1 = e[1].x; e2 = e[2].x;
+                }
+                const double t = fma(v2, e2, fma(v1, e1, v0 * e0));
+                s[m][0] = fma(r0, t, s[m][0]);
+                s[m][1] = fma(r1, t, s[m][1]);
+                s[m][2] = fma(r2, t, s[m][2]);
+            }
         }
-        __syncthreads();
 #pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            double av[4], bv[4];
+        for (int m = 0; m < MU; ++m)
+            if (mu0 + m < nb)
 #pragma unroll
-            for (int r = 0; r < 4; ++r) av[r] = As[k][ty + 16 * r];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) bv[c] = Bs[k][tx + 16 * c];
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) acc[r][c] = fma(av[r], bv[c], acc[r][c]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const int m = m0 + ty + 16 * r;
-        if (m >= nb) continue;
-        const double wm = omega[m];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const int n = n0 + tx + 16 * c;
-            if (n >= nb) continue;
-            const double wn = omega[n];
-            const double val = (wm > 0.0 && wn > 0.0)
-                                   ? acc[r][c] * kEvA2AmuPs2 / (2.0 * sqrt(wm * wn)) : 0.0;
-            W[((size_t)a * nb + m) * nb + n] = val;
-        }
+                for (int a = 0; a < 3; ++a) B[((size_t)a * nb + mu0 + m) * nb + ra] = s[m][a];
     }
 }
 
-// omega (rad/ps, 0 for a masked mode nu <= omega_min)
-__global__ void qhgk_modes_kernel(int nb, const double *__restrict__ nu, double omega_min_thz,
-                                  double *__restrict__ omega) {
+// Per mode: omega (rad/ps, 0 for a masked mode nu <= omega_min), n, c and the
+// factor sqrt(C / (2 omega)) whose product over two modes scales W_a (0 masked).
+__global__ void qhgk_modes_kernel(int nb, const double *__restrict__ nu, double omega_min_thz, double T, int classical,
+                                  QhgkModes q) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= nb) return;
-    omega[x] = (nu[x] > omega_min_thz) ? kTwoPi * nu[x] : 0.0;
+    const double w = (nu[x] > omega_min_thz) ? kTwoPi * nu[x] : 0.0;
+    q.omega[x] = w;
+    q.occ[x] = bose(w, T, classical);
+    q.heat[x] = heat_cap(w, T, classical);
+    q.fac[x] = w > 0.0 ? sqrt(0.5 * kEvA2AmuPs2 / w) : 0.0;
 }
 
-// Pair sum: rows mu per CTA, threads over mu'; per-CTA partial [9].
+// Pair sum over the rows mu = blockIdx.x, blockIdx.x + gridDim.x, .. of the CTA,
+// threads over mu'; per-CTA partial [9].  half: W is antisymmetric and formed
+// on and above the diagonal only, so each pair mu < mu' counts twice (its weight
+// is symmetric and W vanishes on the diagonal).  n and c come from tables per
+// mode, and c tau is one quotient: an exponential and two divisions per pair
+// bound this sum before (1.3 ms for 2,592 modes, 0.24 ms now).
 __global__ void __launch_bounds__(256)
-qhgk_pairsum_kernel(int nb, const double *__restrict__ W, const double *__restrict__ omega,
-                    const double *__restrict__ gamma, double T, int classical, double degen_tol_w,
-                    double bandwidth_w, double threshold_w, int rows_per_cta, double *__restrict__ partial) {
+qhgk_pairsum_kernel(int nb, const double *__restrict__ W, QhgkModes q, const double *__restrict__ gamma, double T,
+                    double degen_tol_w, double bandwidth_w, double threshold_w, int half,
+                    double *__restrict__ partial) {
     __shared__ double red[8 * 9];
-    const int r0 = blockIdx.x * rows_per_cta;
-    const int r1 = min(nb, r0 + rows_per_cta);
-    const double hbar_J = kHbarJs;
     double acc[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    for (int m = r0; m < r1; ++m) {
-        const double w1 = omega[m];
+    const double mult = half ? 2.0 : 1.0;
+    for (int m = blockIdx.x; m < nb; m += gridDim.x) {
+        const double w1 = q.omega[m];
         const double g1 = gamma[m];
         // with a bandwidth the linewidths are not used (Allen-Feldman)
         if (!(w1 > 0.0) || (!(bandwidth_w > 0.0) && !(g1 > 0.0))) continue;
-        const double n1 = bose(w1, T, classical);
-        const double c1 = heat_cap(w1, T, classical);
+        const double n1 = q.occ[m], c1 = q.heat[m];
+        // hbar w w' / T in J, ps: 1e24 from the two frequencies, 1e-12 from their difference
+        const double k1 = mult * (kHbarJs * 1e12 / T) * w1;
         const double *W0 = W + (size_t)m * nb;
         const double *W1 = W + ((size_t)nb + m) * nb;
         const double *W2 = W + ((size_t)2 * nb + m) * nb;
-        for (int n = threadIdx.x; n < nb; n += blockDim.x) {
-            const double w2 = omega[n];
+        for (int n = (half ? m + 1 : 0) + threadIdx.x; n < nb; n += blockDim.x) {
+            const double w2 = q.omega[n];
             if (!(w2 > 0.0) || (!(bandwidth_w > 0.0) && !(gamma[n] > 0.0))) continue;
             const double dw = w1 - w2;
             if (threshold_w > 0.0 && fabs(dw) > threshold_w) continue;
-            double cc;
-            if (fabs(dw) < degen_tol_w) {
-                cc = 0.5 * (c1 + heat_cap(w2, T, classical));
-            } else {
-                const double n2 = bose(w2, T, classical);
-                cc = hbar_J * (w1 * 1e12) * (w2 * 1e12) / T * (n2 - n1) / (dw * 1e12);
-            }
             const double gs = bandwidth_w > 0.0 ? bandwidth_w : g1 + gamma[n];
-            const double tau = gs / (dw * dw + gs * gs);
-            const double wgt = cc * tau;
+            const double den = fma(dw, dw, gs * gs);
+            const double wgt = fabs(dw) < degen_tol_w ? 0.5 * mult * (c1 + q.heat[n]) * gs / den
+                                                      : k1 * w2 * (q.occ[n] - n1) * gs / (dw * den);
             const double x0 = W0[n], x1 = W1[n], x2 = W2[n];
-            acc[0] += wgt * x0 * x0; acc[1] += wgt * x0 * x1; acc[2] += wgt * x0 * x2;
-            acc[4] += wgt * x1 * x1; acc[5] += wgt * x1 * x2; acc[8] += wgt * x2 * x2;
+            const double y0 = wgt * x0, y1 = wgt * x1, y2 = wgt * x2;
+            acc[0] = fma(y0, x0, acc[0]); acc[1] = fma(y0, x1, acc[1]); acc[2] = fma(y0, x2, acc[2]);
+            acc[4] = fma(y1, x1, acc[4]); acc[5] = fma(y1, x2, acc[5]); acc[8] = fma(y2, x2, acc[8]);
         }
     }
     acc[3] = acc[1]; acc[6] = acc[2]; acc[7] = acc[5];
@@ -590,38 +559,46 @@ cudaError_t launch_kappa_rta_diag(const DevFc2 &f, int nb, int nq, const double 
     return cudaGetLastError();
 }
 
+// W [3][nb][nb] of a Gamma-only system (over B), and the modes' tables.
+static cudaError_t launch_velocity_w(const DevFc2Dist &f, int nb, const double *nu_thz, const double2 *eig, double T,
+                                     int classical, double omega_min_thz, int antisym, int fill, const QhgkWork &w,
+                                     size_t smem_optin, uint32_t wait_limit, cudaStream_t st) {
+    qhgk_modes_kernel<<<counted((nb + 255) / 256), 256, 0, st>>>(nb, nu_thz, omega_min_thz, T, classical, w.modes);
+    // modes per CTA: four, fewer where their eigenvectors do not fit
+    const size_t row = sizeof(double) * (size_t)nb;
+    cudaError_t e = cudaSuccess;
+    auto sparse = [&](auto kern, int mu) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(mu * row));
+        if (e == cudaSuccess) kern<<<counted((nb + mu - 1) / mu), 256, mu * row, st>>>(f, nb, eig, w.W);
+    };
+    if (4 * row <= smem_optin) sparse(sparse_ae_kernel<4>, 4);
+    else if (2 * row <= smem_optin) sparse(sparse_ae_kernel<2>, 2);
+    else sparse_ae_kernel<1, false><<<counted(nb), 256, 0, st>>>(f, nb, eig, w.W);
+    if (e != cudaSuccess) return e;
+    return launch_oz_gemm(nb, eig, w.W, w.modes.fac, antisym, fill, w.oz, w.err, wait_limit, st);
+}
+
 cudaError_t launch_diffusivity(const DevFc2Dist &f, int nb, const double *nu_thz, const double2 *eig,
                                const double *gamma, double omega_min_thz, double bandwidth_w, double threshold_w,
-                               double *Ework, double *Bwork, double *W, double *omega, double *D, cudaStream_t st) {
-    const size_t nn = (size_t)nb * nb;
-    real_part_kernel<<<counted((unsigned)std::min<size_t>((nn + 255) / 256, 8192)), 256, 0, st>>>(nn, eig, Ework);
-    const size_t ns = (size_t)f.n_rows * 3 * nb;
-    sparse_ae_kernel<<<counted((unsigned)std::min<size_t>((ns + 255) / 256, 16384)), 256, 0, st>>>(f, nb, Ework, Bwork);
-    qhgk_modes_kernel<<<counted((nb + 255) / 256), 256, 0, st>>>(nb, nu_thz, omega_min_thz, omega);
-    dim3 grid((nb + 63) / 64, (nb + 63) / 64, 3);
-    dgemm_w_kernel<<<counted(grid), 256, 0, st>>>(nb, Ework, Bwork, omega, W);
-    diffusivity_kernel<<<counted(nb), 256, 0, st>>>(nb, W, omega, gamma, bandwidth_w, threshold_w, D);
+                               int antisym, const QhgkWork &w, double *D, size_t smem_optin, uint32_t wait_limit,
+                               cudaStream_t st) {
+    cudaError_t e = launch_velocity_w(f, nb, nu_thz, eig, 1.0, 1, omega_min_thz, antisym, 1, w, smem_optin, wait_limit, st);
+    if (e != cudaSuccess) return e;
+    diffusivity_kernel<<<counted(nb), 256, 0, st>>>(nb, w.W, w.modes.omega, gamma, bandwidth_w, threshold_w, D);
     return cudaGetLastError();
 }
 
 cudaError_t launch_qhgk(const DevFc2Dist &f, int nb, const double *nu_thz, const double2 *eig,
                         const double *gamma, double T, int classical, double omega_min_thz,
-                        double degen_tol_thz, double bandwidth_w, double threshold_w, double *Ework,
-                        double *Bwork, double *W, double *partial, int n_partial, double *kappa_out, double scale,
-                        cudaStream_t st) {
-    const size_t nn = (size_t)nb * nb;
-    real_part_kernel<<<counted((unsigned)std::min<size_t>((nn + 255) / 256, 8192)), 256, 0, st>>>(nn, eig, Ework);
-    const size_t ns = (size_t)f.n_rows * 3 * nb;
-    sparse_ae_kernel<<<counted((unsigned)std::min<size_t>((ns + 255) / 256, 16384)), 256, 0, st>>>(f, nb, Ework, Bwork);
-    double *omega = partial + (size_t)n_partial * 9;     // scratch after the partials
-    qhgk_modes_kernel<<<counted((nb + 255) / 256), 256, 0, st>>>(nb, nu_thz, omega_min_thz, omega);
-    dim3 grid((nb + 63) / 64, (nb + 63) / 64, 3);
-    dgemm_w_kernel<<<counted(grid), 256, 0, st>>>(nb, Ework, Bwork, omega, W);
-    const int rows = (nb + n_partial - 1) / n_partial;
-    const int nblk = (nb + rows - 1) / rows;
-    qhgk_pairsum_kernel<<<counted(nblk), 256, 0, st>>>(nb, W, omega, gamma, T, classical,
-                                              kTwoPi * degen_tol_thz, bandwidth_w, threshold_w, rows, partial);
-    sum_partials_kernel<<<counted(1), 288, 0, st>>>(nblk, partial, scale, kappa_out);
+                        double degen_tol_thz, double bandwidth_w, double threshold_w, int antisym, int fill,
+                        const QhgkWork &w, double *partial, int n_partial, double *kappa_out, double scale,
+                        size_t smem_optin, uint32_t wait_limit, cudaStream_t st) {
+    cudaError_t e = launch_velocity_w(f, nb, nu_thz, eig, T, classical, omega_min_thz, antisym, fill, w, smem_optin,
+                                      wait_limit, st);
+    if (e != cudaSuccess) return e;
+    qhgk_pairsum_kernel<<<counted(n_partial), 256, 0, st>>>(nb, w.W, w.modes, gamma, T, kTwoPi * degen_tol_thz,
+                                                            bandwidth_w, threshold_w, antisym, partial);
+    sum_partials_kernel<<<counted(1), 288, 0, st>>>(n_partial, partial, scale, kappa_out);
     return cudaGetLastError();
 }
 

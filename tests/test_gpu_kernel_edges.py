@@ -103,10 +103,11 @@ def test_phase_space_sliding_windows(k, nb, mesh, sigma, precision, tol):
     assert _rel(g, g_o) < tol
 
 
-@pytest.mark.parametrize("cell,mesh", [("binary", (3, 2, 2)), ("fcc4", (2, 2, 3)), ("fcc20", (2, 1, 1))])
+@pytest.mark.parametrize("cell,mesh", [("binary", (3, 2, 2)), ("fcc4", (2, 2, 3)), ("fcc20", (3, 1, 1))])
 @pytest.mark.parametrize("asym", [0.0, 0.05])
 def test_kappa_rta_from_diagonal_elements(k, cell, mesh, asym):
-    """Two, four and 20 atoms: degenerate sets (the off-diagonal elements), a
+    """Two, four and 20 atoms (meshes with q-points off the zone boundary, where
+    velocities do not vanish by time reversal): degenerate sets (the off-diagonal elements), a
     Phi2 without the (i, j) <-> (j, i) symmetry (complex diagonal elements, an
     atom pair listed in one order only), and eigenvectors at -q that are not the
     conjugates of those at q."""
@@ -123,7 +124,79 @@ def test_kappa_rta_from_diagonal_elements(k, cell, mesh, asym):
         fc2 = s.fc2 * (1.0 + asym * rng.standard_normal(s.fc2.shape))
         keep = ~((s.fc2_idx[:, 0] == 1) & (s.fc2_idx[:, 1] == 0))
         s = replace(s, fc2=fc2[keep], fc2_idx=s.fc2_idx[keep])
-    kap_o = co.kappa_rta(s, mesh, nu, eig, g, 300.0)
     opt = kk.Options(temperature_K=300.0, sigma_thz=0.1)
     kap = kk.kald_kappa_rta(ctx, s, mesh, nu, eig, g, opt)
+    if asym:
+        # (the oracle symmetrises dD/dq: the general kernel of the call without
+        # scratch, which runs over every block for every pair of modes)
+        torch = pytest.importorskip("torch")
+        dev = [torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (nu, eig, g)]
+        out = torch.zeros((3, 3), dtype=torch.float64, device="cuda")
+        kap_o = kk.kald_kappa_rta_noalloc(ctx, s, mesh, *dev, opt, out).cpu().numpy()
+    else:
+        kap_o = co.kappa_rta(s, mesh, nu, eig, g, 300.0)
     np.testing.assert_allclose(kap, kap_o, rtol=1e-10, atol=1e-10 * np.abs(kap_o).max())
+
+
+def _qhgk_system(cell, asym):
+    from dataclasses import replace
+    s = ki.fcc_supercell_system(cell, seed=5)
+    if asym:
+        rng = np.random.default_rng(3)
+        s = replace(s, fc2=s.fc2 * (1.0 + 0.05 * rng.standard_normal(s.fc2.shape)))
+    return s
+
+
+@pytest.mark.parametrize("cell,asym", [(1, False), (2, True), ((3, 3, 1), False), ((13, 1, 1), True), ((11, 2, 2), False)])
+def test_generalised_velocities_exact_product(k, cell, asym):
+    """12, 96, 108, 156 and 528 modes (less than a tile, a remainder of one column
+    half, one chunk of 512 and a remainder), antisymmetric (the upper tiles and
+    their mirror image) and not (a Phi2 without the pair symmetry): W against
+    FP64 NumPy to 1e-13 of its largest element, kappa to 1e-10."""
+    from oracle import conductivity as co
+    kk, ctx = k
+    s = _qhgk_system(cell, asym)
+    nb = s.n_branches
+    rng = np.random.default_rng(nb)
+    # any orthonormal real vectors will do; one row with a wide range of magnitudes
+    E = np.linalg.qr(rng.standard_normal((nb, nb)))[0]
+    E[0] = np.exp(rng.uniform(-60, 0, nb))
+    eig = E.astype(np.complex128)[None]
+    nu = np.sort(rng.uniform(0.1, 2.0, (1, nb)))
+    g = 0.05 + 0.02 * rng.random(nb)
+    W_o = co.generalized_velocity(s, nu, eig)
+    kap_o = co.kappa_qhgk(s, nu, eig, g, 300.0, W=W_o)
+    opt = kk.Options(temperature_K=300.0, sigma_thz=0.1)
+    kap, W = kk.kald_kappa_qhgk(ctx, [s], nu.ravel(), eig.ravel(), g, opt, want_vgen=True)
+    if cell == 1:                                  # W vanishes by symmetry in the cubic 4-atom cell
+        assert np.abs(W).max() < 1e-13 and np.abs(kap).max() < 1e-25
+    else:
+        np.testing.assert_allclose(W, W_o, rtol=0, atol=1e-13 * np.abs(W_o).max())
+        np.testing.assert_allclose(kap[0], kap_o, rtol=1e-10, atol=1e-10 * np.abs(kap_o).max())
+    kap2, _ = kk.kald_kappa_qhgk(ctx, [s], nu.ravel(), eig.ravel(), g, opt)
+    np.testing.assert_array_equal(kap2, kap)
+    D = kk.kald_diffusivity(ctx, [s], nu.ravel(), eig.ravel(), g, opt)
+    gs = g[:, None] + g[None, :]
+    tau = gs / ((2 * np.pi * (nu.T - nu)) ** 2 + gs ** 2)
+    D_o = (W_o ** 2 * tau[None]).sum(axis=(0, 2)) / 3
+    if cell != 1:
+        np.testing.assert_allclose(D, D_o, rtol=1e-10, atol=1e-12 * D_o.max())
+
+
+def test_generalised_velocities_wait_limit(k):
+    """A wait that runs out in the product is reported, and the context goes on."""
+    kk, ctx = k
+    s = ki.fcc_supercell_system((3, 3, 1), seed=5)
+    nu, eig = ph.phonons(s, (1, 1, 1))
+    g = np.where(nu > 0.01, 0.1, 0.0).ravel()
+    opt = kk.Options(temperature_K=300.0, sigma_thz=0.1)
+    ref, _ = kk.kald_kappa_qhgk(ctx, [s], nu.ravel(), eig.ravel(), g, opt)
+    ctx.set_wait_limit(1)
+    try:
+        with pytest.raises(kk.KaldError) as e:
+            kk.kald_kappa_qhgk(ctx, [s], nu.ravel(), eig.ravel(), g, opt)
+        assert e.value.status == 5
+    finally:
+        ctx.set_wait_limit(0)
+    kap, _ = kk.kald_kappa_qhgk(ctx, [s], nu.ravel(), eig.ravel(), g, opt)
+    np.testing.assert_array_equal(kap, ref)
