@@ -196,8 +196,10 @@ uint64_t kald_kernel_launches(void);
  *   eigvec  [Nq][nb][nb][2] out, complex128, row s = eigenvector of mode s,
  *           unit norm (interleaved re, im)
  *   vel     [Nq][nb][3] out (A/ps), or NULL
- * nb <= 96: one Householder tridiagonalisation + implicit QL eigensolver per q
- * (KALD_E_NOCONV if an eigenvalue takes more than 60 QL sweeps) for the lower
+ * nb <= 96: one Householder tridiagonalisation per q, then bisection and
+ * inverse iteration (nb >= 16), or implicit QL for smaller cells and wherever
+ * the inverse iteration's residuals or norms fail their check (KALD_E_NOCONV
+ * if an eigenvalue then takes more than 60 QL sweeps), for the lower
  * index of each pair {q, -q}; the
  * other takes the same frequencies and the conjugate eigenvectors (time
  * reversal: D(-q) = conj D(q) for real Phi2).  nb > 96 is supported at Gamma only (mesh

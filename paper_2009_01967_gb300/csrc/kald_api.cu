@@ -640,7 +640,9 @@ kald_status kald_phonons(kald_ctx *ctx, const kald_system *sys, const int32_t me
     }
     const bool mirror = !large && nrep < nq;
     const size_t nnr = mirror ? (size_t)nrep * nb * nb : nn;
-    size_t need = fc2_bytes(h) + bytes_of(qc) + 2 * ws_round(sizeof(double2) * nnr) + ws_round(sizeof(int));
+    const size_t nnv = large ? 0 : (size_t)(mirror ? nrep : nq) * jacobi_scratch(nb);      // eigensolver scratch
+    size_t need = fc2_bytes(h) + bytes_of(qc) + ws_round(sizeof(double2) * nnr) + ws_round(sizeof(double2) * nnv) +
+                  ws_round(sizeof(int));
     if (mirror)
         need += bytes_of(qc_rep) + bytes_of(rep_row) + bytes_of(rep_conj) + ws_round(sizeof(double) * nrep * nb) +
                 ws_round(sizeof(double2) * nnr);
@@ -656,7 +658,7 @@ kald_status kald_phonons(kald_ctx *ctx, const kald_system *sys, const int32_t me
     upload_fc2(ctx, h, d);
     const double *qcart = upload(ctx, qc);
     double2 *D = static_cast<double2 *>(ws_take(ctx, sizeof(double2) * nnr));
-    double2 *V = static_cast<double2 *>(ws_take(ctx, sizeof(double2) * nnr));
+    double2 *V = static_cast<double2 *>(ws_take(ctx, sizeof(double2) * nnv));
     int *nonconv = static_cast<int *>(ws_take(ctx, sizeof(int)));
     const double *qcart_rep = mirror ? upload(ctx, qc_rep) : qcart;
     const int *row_d = mirror ? upload(ctx, rep_row) : nullptr;

@@ -185,6 +185,7 @@ cudaError_t launch_mirror_phonons(int nq, int nb, const int *row, const int *con
                                   cudaStream_t st);
 cudaError_t launch_dynmat(const DevFc2 &f, int nb, int nq, size_t n_blk, const double *qcart, double2 *D,
                           cudaStream_t st);
+size_t jacobi_scratch(int nb);
 cudaError_t launch_jacobi(int nb, int nq, double2 *A, double2 *V, double *nu_thz,
                           double2 *eig_out, int *nonconv, size_t smem_optin, cudaStream_t st);
 // eigh_large.cu: one real symmetric matrix (the Gamma-only D), n up to about

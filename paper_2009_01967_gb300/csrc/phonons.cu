@@ -11,6 +11,7 @@
 #include <algorithm>
 
 #include "kald_internal.h"
+#include "tridiag.cuh"
 
 namespace kald {
 namespace {
@@ -228,22 +229,48 @@ jacobi_kernel(int nb, double2 *__restrict__ Ain, double2 *__restrict__ Vt_all,
     }
 }
 
-// Householder-QL Hermitian eigensolver, one matrix per CTA (FP64), about a
+// Householder Hermitian eigensolver, one matrix per CTA (FP64), about a
 // twentieth of the Jacobi sweeps' flops:
 //  1. tridiagonalisation by complex reflectors H_k = I - tau_k v_k v_k^H
 //     (v_k[k+1] = 1, the rest stored below the subdiagonal of column k of A in
-//     shared memory); the subdiagonal beta_k is real for k < n-2, and the last
-//     one is made real by a phase on the last index;
-//  2. implicit QL with Wilkinson shifts on the real tridiagonal: thread 0 forms
-//     the rotations of each sweep, every thread applies them to its row of the
-//     real eigenvector matrix Z (shared memory, column-major);
-//  3. eigenvectors Q P Z: the phase, then the reflectors in reverse order,
-//     each thread on one column of a global scratch G[dof][j] (coalesced);
-//  4. ascending order, as the Jacobi kernel writes it.
-// Shared memory: A n*n complex, Z n*n real, d, e, tau, work, order.
-constexpr int kHqlThreads = 256;
+//     shared memory) on the lower triangle; the subdiagonal beta_k is real for
+//     k < n-2, and the last one is made real by a phase on the last index;
+//  2. n >= kHqlInvit: eigenvalues by bisection with Sturm counts, one thread
+//     each, and their vectors by inverse iteration (tridiagonal LU with partial
+//     pivoting, three solves), Gram-Schmidt along chains of eigenvalues closer
+//     than 1e-2 |T|; every residual and norm is checked, and a matrix that
+//     fails the check, like every smaller one, takes implicit QL with Wilkinson
+//     shifts (thread 0 forms the rotations of each sweep, all threads apply them
+//     to the rows of Z);
+//  3. eigenvectors Q P Z: four lanes per column hold it in registers and apply
+//     the phase and the reflectors in reverse order, reflectors from shared memory;
+//  4. ascending order.
+// Bound: the FP64 units (0.5 lanes per clock and SM sub-partition, so every
+// FP64 instruction of a warp takes 64 cycles there, whatever its active lanes)
+// and, in QL, one chain of about 26 such instructions per rotation on one
+// thread, some 8,000 rotations for n = 96: half of the 16.6 ms per matrix that
+// tridiagonalisation, QL and a back-transformation through global memory took.
+// 260 matrices of 96 x 96 (8^3 mesh): 33.3 ms before, 10.4 ms now.
+// Shared memory: A n*(n|1) complex, Z n*n real (the work vectors of step 1
+// before that), d, e, tau, lambda, work, order.
+constexpr int kHqlThreads = 384;         // four lanes per column of up to 96
+constexpr int kHqlInvit = 16;
+constexpr int kHqlRows = 24;             // rows per lane of a column
 
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+// acc += conj(a) b, acc -= a b
+__device__ __forceinline__ void cfmac(double2 &acc, double2 a, double2 b) {
+    acc.x = fma(a.x, b.x, acc.x);
+    acc.x = fma(a.y, b.y, acc.x);
+    acc.y = fma(a.x, b.y, acc.y);
+    acc.y = fma(-a.y, b.x, acc.y);
+}
+__device__ __forceinline__ void cfms(double2 &acc, double2 a, double2 b) {
+    acc.x = fma(-a.x, b.x, acc.x);
+    acc.x = fma(a.y, b.y, acc.x);
+    acc.y = fma(-a.x, b.y, acc.y);
+    acc.y = fma(-a.y, b.x, acc.y);
+}
 
 // (x, y) summed over the CTA in a fixed order; every thread gets the sum.
 __device__ double2 hql_block_sum(double2 v, double2 *red) {
@@ -260,20 +287,104 @@ __device__ double2 hql_block_sum(double2 v, double2 *red) {
 }
 
 struct HqlLayout {
-    size_t z, d, e, tau, w, red, ord, bytes;
+    size_t z, d, e, tau, lam, w, red, ord, bytes;
 };
 __host__ __device__ inline HqlLayout hql_layout(int n) {
     auto up16 = [](size_t b) { return (b + 15) & ~size_t(15); };
     HqlLayout L;
-    L.z = up16(sizeof(double2) * (size_t)n * n);
-    L.d = up16(L.z + sizeof(double) * (size_t)n * n);
+    L.z = up16(sizeof(double2) * (size_t)n * (n | 1));
+    // Z, or before it the vectors v and w and four partial products of step 1
+    const size_t z = sizeof(double) * (size_t)n * (n | 1), w1 = sizeof(double2) * 6 * (size_t)n;
+    L.d = up16(L.z + (z > w1 ? z : w1));
     L.e = up16(L.d + sizeof(double) * n);
     L.tau = up16(L.e + sizeof(double) * n);
-    L.w = up16(L.tau + sizeof(double2) * n);
+    L.lam = up16(L.tau + sizeof(double2) * n);
+    L.w = up16(L.lam + sizeof(double) * n);
     L.red = up16(L.w + sizeof(double2) * n);
     L.ord = up16(L.red + sizeof(double2) * (kHqlThreads / 32));
     L.bytes = up16(L.ord + sizeof(int) * n);
     return L;
+}
+// Global scratch per matrix in double2: the LU factors of the inverse
+// iteration (four doubles and a flag per element).
+__host__ __device__ inline size_t hql_scratch(int n) {
+    return n >= kHqlInvit ? 2 * (size_t)n * n + ((size_t)n * n + 15) / 16 : 1;
+}
+
+// Inverse iteration for eigenvalue sigma of T (diagonal d, subdiagonal e), by
+// one thread t of n: into x[0 .. n - 1] and of the
+// factors (element j at j * n + t).  Returns the residual max_j |(T - sigma) x|_j.
+__device__ double hql_invit(int n, int t, const double *__restrict__ d, const double *__restrict__ e, double sigma,
+                            double tiny, double *__restrict__ F, unsigned char *__restrict__ piv, double *__restrict__ x) {
+    const size_t S = (size_t)n, nn = S * S;
+    double *rdg = F, *u1 = F + nn, *u2 = F + 2 * nn, *ml = F + 3 * nn;
+    double cd = d[0] - sigma, cu = e[0];
+    for (int j = 0; j < n - 1; ++j) {
+        const double lj = e[j], nd = d[j + 1] - sigma, nu = (j + 1 < n - 1) ? e[j + 1] : 0.0;
+        double dj, u1j, u2j, f, ncd, ncu;
+        unsigned char pv;
+        if (fabs(cd) >= fabs(lj)) {                    // keep row j
+            f = (cd != 0.0) ? lj / cd : 0.0;
+            dj = cd; u1j = cu; u2j = 0.0; pv = 0;
+            ncd = nd - f * cu; ncu = nu;
+        } else {                                       // exchange rows j and j+1
+            f = cd / lj;
+            dj = lj; u1j = nd; u2j = nu; pv = 1;
+            ncd = cu - f * nd; ncu = -f * nu;
+        }
+        if (fabs(dj) < tiny) dj = tiny;
+        const size_t a = (size_t)j * S + t;
+        rdg[a] = 1.0 / dj;
+        u1[a] = u1j;
+        u2[a] = u2j;
+        ml[a] = f;
+        piv[a] = pv;
+        cd = ncd;
+        cu = ncu;
+    }
+    if (fabs(cd) < tiny) cd = tiny;
+    rdg[(size_t)(n - 1) * S + t] = 1.0 / cd;
+    double scale = 1.0;
+    for (int it = 0; it < 3; ++it) {
+        // start vector: deterministic, not aligned with any special direction
+        auto start = [&](int j) {
+            unsigned h = (unsigned)(j * 131 + t * 7919 + 1) * 2654435761u;
+            h ^= h >> 15;
+            return 0.75 + (double)(h & 0xffff) * (0.5 / 65536.0);
+        };
+        double cx = (it == 0) ? start(0) : x[0] * scale;
+#pragma unroll 4
+        for (int j = 0; j < n - 1; ++j) {
+            const size_t a = (size_t)j * S + t;
+            const double nx = (it == 0) ? start(j + 1) : x[j + 1] * scale;
+            const double m = ml[a];
+            const bool pv = piv[a];
+            x[j] = pv ? nx : cx;
+            cx = fma(-m, pv ? nx : cx, pv ? cx : nx);
+        }
+        x[n - 1] = cx;
+        double x1 = 0.0, x2 = 0.0, nrm = 0.0;
+#pragma unroll 4
+        for (int j = n - 1; j >= 0; --j) {
+            const size_t a = (size_t)j * S + t;
+            const double v = j < n - 1 ? (x[j] - u1[a] * x1 - u2[a] * x2) * rdg[a] : x[j] * rdg[a];
+            x[j] = v;
+            nrm = fma(v, v, nrm);
+            x2 = x1;
+            x1 = v;
+        }
+        scale = 1.0 / sqrt(nrm);
+    }
+    for (int j = 0; j < n; ++j) x[j] *= scale;
+    double res = 0.0;
+    for (int j = 0; j < n; ++j) {
+        double r = (d[j] - sigma) * x[j];
+        if (j > 0) r = fma(e[j - 1], x[j - 1], r);
+        if (j < n - 1) r = fma(e[j], x[j + 1], r);
+        r = fabs(r);
+        res = (r <= res) ? res : r;                    // (a NaN stays)
+    }
+    return res;
 }
 
 __global__ void __launch_bounds__(kHqlThreads)
@@ -281,43 +392,48 @@ hermitian_ql_kernel(int n, const double2 *__restrict__ Ain, double2 *__restrict_
                     double *__restrict__ nu_out, double2 *__restrict__ eig_out, int *nonconv) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const HqlLayout L = hql_layout(n);
-    double2 *A = reinterpret_cast<double2 *>(smem_raw);                 // [n][n] row-major
-    double *Zt = reinterpret_cast<double *>(smem_raw + L.z);            // Zt[col * n + row]
+    const int ld = n | 1;                          // odd pitch: rows and columns of A both walk distinct banks
+    double2 *A = reinterpret_cast<double2 *>(smem_raw);                 // [n][ld], lower triangle
+    const int zl = ld;
+    double *Zt = reinterpret_cast<double *>(smem_raw + L.z);            // Zt[col * zl + row]
+    double2 *vv = reinterpret_cast<double2 *>(smem_raw + L.z);          // step 1: v, w, partial products (over Zt)
+    double2 *w = vv + n, *wp = vv + 2 * n;
     double *d = reinterpret_cast<double *>(smem_raw + L.d);
     double *e = reinterpret_cast<double *>(smem_raw + L.e);
     double2 *tau = reinterpret_cast<double2 *>(smem_raw + L.tau);
-    double2 *w = reinterpret_cast<double2 *>(smem_raw + L.w);           // tridiagonalisation
-    double *rc = reinterpret_cast<double *>(smem_raw + L.w);            // QL rotations (over w)
+    double *lam = reinterpret_cast<double *>(smem_raw + L.lam);
+    double *rc = reinterpret_cast<double *>(smem_raw + L.w);            // QL rotations; e^2 in bisection
     double *rs = rc + n;
     double2 *red = reinterpret_cast<double2 *>(smem_raw + L.red);
     int *ord = reinterpret_cast<int *>(smem_raw + L.ord);
     __shared__ int ql_lo, ql_hi, ql_go, ql_fail;
+    __shared__ double g_lo, g_hi, g_tn;
 
-    const int q = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
+    const int q = blockIdx.x, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
     const double2 *Aq = Ain + (size_t)q * n * n;
-    double2 *G = G_all + (size_t)q * n * n;
+    double2 *G = G_all + (size_t)q * hql_scratch(n);
     const double2 one = make_double2(1.0, 0.0);
 
-    // the Hermitian part (D + D^dagger)/2, Z = I
+    // the Hermitian part (D + D^dagger)/2, lower triangle
     for (int x = tid; x < n * n; x += nt) {
         const int r = x / n, c = x - (x / n) * n;
+        if (c > r) continue;
         const double2 a = Aq[(size_t)r * n + c], b = Aq[(size_t)c * n + r];
-        A[x] = make_double2(0.5 * (a.x + b.x), 0.5 * (a.y - b.y));
-        Zt[x] = (r == c) ? 1.0 : 0.0;
+        A[r * ld + c] = make_double2(0.5 * (a.x + b.x), 0.5 * (a.y - b.y));
     }
     if (tid == 0) ql_fail = 0;
     __syncthreads();
 
     // ---- 1. tridiagonalisation
+    const int parts = max(1, min(4, nt / n));      // threads per row of the product
     for (int k = 0; k + 2 < n; ++k) {
-        const int m = n - k - 1;
         double2 part = make_double2(0.0, 0.0);
         for (int i = k + 2 + tid; i < n; i += nt) {
-            const double2 v = A[i * n + k];
+            const double2 v = A[i * ld + k];
             part.x += v.x * v.x + v.y * v.y;
         }
         const double xn2 = hql_block_sum(part, red).x;
-        const double2 alpha = A[(k + 1) * n + k];
+        const double2 alpha = A[(k + 1) * ld + k];
         const bool refl = !(xn2 == 0.0 && alpha.y == 0.0);
         double beta = alpha.x;
         double2 t = make_double2(0.0, 0.0);
@@ -328,38 +444,50 @@ hermitian_ql_kernel(int n, const double2 *__restrict__ Ain, double2 *__restrict_
             const double2 den = make_double2(alpha.x - beta, alpha.y);
             const double dd = den.x * den.x + den.y * den.y;
             const double2 sc = make_double2(den.x / dd, -den.y / dd);
-            for (int i = k + 2 + tid; i < n; i += nt) A[i * n + k] = cmul(A[i * n + k], sc);
+            for (int i = k + 1 + tid; i < n; i += nt) {
+                const double2 v = (i == k + 1) ? one : cmul(A[i * ld + k], sc);
+                vv[i] = v;
+                if (i > k + 1) A[i * ld + k] = v;
+            }
         }
         if (tid == 0) { tau[k] = t; e[k] = beta; }
         __syncthreads();
         if (refl) {
-            // w = tau B v with B = A[k+1.., k+1..] Hermitian: w_i = tau sum_j conj(B_ji) v_j
+            // w = tau B v with B = A[k+1.., k+1..] Hermitian, from its lower triangle
+            for (int x = tid; x < parts * n; x += nt) {
+                const int p = x / n, i = x - p * n;
+                if (i <= k) continue;
+                double2 acc = make_double2(0.0, 0.0);
+                for (int j = k + 1 + p; j < n; j += parts) {
+                    const bool low = j <= i;
+                    const double2 b = A[low ? i * ld + j : j * ld + i];
+                    cfmac(acc, make_double2(b.x, low ? -b.y : b.y), vv[j]);      // B_ij = conj(A_ji) above
+                }
+                wp[p * n + i] = acc;
+            }
+            __syncthreads();
             double2 pd = make_double2(0.0, 0.0);
             for (int i = k + 1 + tid; i < n; i += nt) {
-                double2 acc = make_double2(0.0, 0.0);
-                for (int j = k + 1; j < n; ++j) {
-                    const double2 vj = (j == k + 1) ? one : A[j * n + k];
-                    acc = cadd(acc, cmulc(A[j * n + i], vj));
-                }
-                w[i] = cmul(t, acc);
-                const double2 vi = (i == k + 1) ? one : A[i * n + k];
-                pd = cadd(pd, cmulc(w[i], vi));                  // w^H v
+                double2 acc = wp[i];
+                for (int p = 1; p < parts; ++p) acc = cadd(acc, wp[p * n + i]);
+                const double2 wi = cmul(t, acc);
+                w[i] = wi;
+                pd = cadd(pd, cmulc(wi, vv[i]));                 // w^H v
             }
             const double2 wv = hql_block_sum(pd, red);
             const double2 a2 = cmul(make_double2(-0.5 * t.x, -0.5 * t.y), wv);
-            for (int i = k + 1 + tid; i < n; i += nt) {
-                const double2 vi = (i == k + 1) ? one : A[i * n + k];
-                w[i] = cadd(w[i], cmul(a2, vi));
-            }
+            for (int i = k + 1 + tid; i < n; i += nt) w[i] = cadd(w[i], cmul(a2, vv[i]));
             __syncthreads();
-            // B -= v w^H + w v^H
-            for (int x = tid; x < m * m; x += nt) {
-                const int i = k + 1 + x / m, j = k + 1 + (x - (x / m) * m);
-                const double2 vi = (i == k + 1) ? one : A[i * n + k];
-                const double2 vj = (j == k + 1) ? one : A[j * n + k];
-                const double2 u = cadd(cmul(vi, make_double2(w[j].x, -w[j].y)),
-                                       cmul(w[i], make_double2(vj.x, -vj.y)));
-                A[i * n + j] = make_double2(A[i * n + j].x - u.x, A[i * n + j].y - u.y);
+            // B -= v w^H + w v^H, lower triangle, a row per warp
+            for (int i = k + 1 + warp; i < n; i += nw) {
+                const double2 vi = vv[i], wi = w[i];
+                for (int j = k + 1 + lane; j <= i; j += 32) {
+                    double2 b = A[i * ld + j];
+                    const double2 wj = w[j], vj = vv[j];
+                    cfms(b, vi, make_double2(wj.x, -wj.y));
+                    cfms(b, wi, make_double2(vj.x, -vj.y));
+                    A[i * ld + j] = b;
+                }
             }
             __syncthreads();
         }
@@ -367,121 +495,225 @@ hermitian_ql_kernel(int n, const double2 *__restrict__ Ain, double2 *__restrict_
     // the last subdiagonal element made real by the phase ph on index n-1
     double2 ph = one;
     if (n >= 2) {
-        const double2 sub = A[(n - 1) * n + (n - 2)];
+        const double2 sub = A[(n - 1) * ld + (n - 2)];
         const double r = hypot(sub.x, sub.y);
         if (r > 0.0) ph = make_double2(sub.x / r, sub.y / r);
         if (tid == 0) e[n - 2] = r;
     }
-    for (int i = tid; i < n; i += nt) d[i] = A[i * n + i].x;
+    for (int i = tid; i < n; i += nt) d[i] = A[i * ld + i].x;
     if (tid == 0) e[n - 1] = 0.0;
     __syncthreads();
 
-    // ---- 2. implicit QL (thread 0 forms each sweep, all threads rotate Z)
-    int l = 0, iter = 0;                           // thread 0's state
-    for (;;) {
-        if (tid == 0) {
-            ql_go = 0;
-            while (l < n) {
-                int mm = l;
-                for (; mm < n - 1; ++mm) {
-                    const double dd = fabs(d[mm]) + fabs(d[mm + 1]);
-                    if (fabs(e[mm]) <= 1.0e-16 * dd) break;
-                }
-                if (mm == l) { ++l; iter = 0; continue; }
-                if (++iter > 60) { ql_fail = 1; ++l; iter = 0; continue; }
-                double g = (d[l + 1] - d[l]) / (2.0 * e[l]);
-                double r = hypot(g, 1.0);
-                g = d[mm] - d[l] + e[l] / (g + copysign(r, g));
-                double s = 1.0, c = 1.0, p = 0.0;
-                int i = mm - 1;
-                bool early = false;
-                for (; i >= l; --i) {
-                    // one reciprocal square root per rotation: the chain of
-                    // dependent FP64 operations on thread 0 bounds this stage
-                    const double f = s * e[i], b = c * e[i];
-                    const double rr = f * f + g * g;
-                    if (rr == 0.0) {                 // deflation inside the sweep
-                        e[i + 1] = 0.0;
-                        d[i + 1] -= p;
-                        e[mm] = 0.0;
-                        early = true;
-                        break;
-                    }
-                    const double ir = rsqrt(rr);
-                    r = rr * ir;
-                    e[i + 1] = r;
-                    s = f * ir;
-                    c = g * ir;
-                    g = d[i + 1] - p;
-                    r = (d[i] - g) * s + 2.0 * c * b;
-                    p = s * r;
-                    d[i + 1] = g + p;
-                    g = c * r - b;
-                    rc[i] = c;
-                    rs[i] = s;
-                }
-                if (!early) {
-                    d[l] -= p;
-                    e[l] = g;
-                    e[mm] = 0.0;
-                }
-                ql_hi = mm - 1;
-                ql_lo = early ? i + 1 : l;
-                ql_go = 1;
-                break;
+    // ---- 2a. bisection and inverse iteration
+    bool done = false;
+    if (n >= kHqlInvit) {
+        if (warp == 0) {                           // Gershgorin interval and |T|
+            double lo = 1e300, hi = -1e300, tn = 0.0;
+            for (int i = lane; i < n; i += 32) {
+                const double r = (i > 0 ? fabs(e[i - 1]) : 0.0) + fabs(e[i]);
+                lo = fmin(lo, d[i] - r);
+                hi = fmax(hi, d[i] + r);
+                tn = fmax(tn, fabs(d[i]) + r);
+            }
+            for (int o = 16; o > 0; o >>= 1) {
+                lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+                hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+                tn = fmax(tn, __shfl_xor_sync(0xffffffffu, tn, o));
+            }
+            if (lane == 0) {
+                const double pad = 1e-12 * fmax(tn, 1e-300);
+                g_lo = lo - pad;
+                g_hi = hi + pad;
+                g_tn = tn;
             }
         }
+        for (int i = tid; i < n; i += nt) rc[i] = e[i] * e[i];
         __syncthreads();
-        if (!ql_go) break;
-        const int hi = ql_hi, lo = ql_lo;
-        for (int r = tid; r < n; r += nt)
-            for (int i = hi; i >= lo; --i) {
-                const double zi1 = Zt[(i + 1) * n + r], zi = Zt[i * n + r];
-                Zt[(i + 1) * n + r] = rs[i] * zi + rc[i] * zi1;
-                Zt[i * n + r] = rc[i] * zi - rs[i] * zi1;
+        const double tn = g_tn, eps = 2.220446049250313e-16;
+        int bad = 0;
+        if (tid < n) {
+            double lo = g_lo, hi = g_hi;
+            const double pivmin = 1e-300 + 1e-30 * tn * tn;
+            for (int it = 0; it < 80; ++it) {
+                if (hi - lo <= fmax(0.5 * eps * tn, 2.0 * eps * fmax(fabs(lo), fabs(hi)))) break;
+                const double x = 0.5 * (lo + hi);
+                if (!(x > lo && x < hi)) break;
+                if (sturm_count(n, d, rc, x, pivmin) > tid) hi = x;
+                else lo = x;
             }
-        __syncthreads();
+            const double l = 0.5 * (lo + hi);
+            lam[tid] = l;
+            double *F = reinterpret_cast<double *>(G);
+            const double res = hql_invit(n, tid, d, e, l, eps * tn, F,
+                                         reinterpret_cast<unsigned char *>(F + 4 * (size_t)n * n), Zt + (size_t)tid * zl);
+            bad = !(res <= 64.0 * eps * tn);
+        }
+        bad = __syncthreads_or(bad);
+        // right-looking Gram-Schmidt along the chains of close eigenvalues (every
+        // branch around a barrier is uniform over the CTA)
+        if (!bad) {
+            const double close = 1e-2 * tn;
+            int mine = 0;
+            for (int a = 0; a < n; ++a) {
+                if (warp == 0) {
+                    double s = 0.0;
+                    for (int j = lane; j < n; j += 32) s = fma(Zt[a * zl + j], Zt[a * zl + j], s);
+                    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                    const double sc = 1.0 / sqrt(s);
+                    if (!(s > 1e-4)) mine = 1;             // most of the vector was in the span of the earlier ones
+                    for (int j = lane; j < n; j += 32) Zt[a * zl + j] *= sc;
+                }
+                if (!(a + 1 < n && lam[a + 1] - lam[a] <= close)) continue;      // no later vector of this chain
+                if (__syncthreads_or(mine)) break;
+                int end = a + 2;
+                while (end < n && lam[end] - lam[end - 1] <= close) ++end;
+                for (int b = a + 1 + warp; b < end; b += nw) {
+                    double s = 0.0;
+                    for (int j = lane; j < n; j += 32) s = fma(Zt[a * zl + j], Zt[b * zl + j], s);
+                    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                    for (int j = lane; j < n; j += 32) Zt[b * zl + j] = fma(-s, Zt[a * zl + j], Zt[b * zl + j]);
+                }
+                __syncthreads();
+            }
+            bad = __syncthreads_or(mine);
+        }
+        done = !bad;
     }
-    if (tid == 0 && ql_fail) atomicAdd(nonconv, 1);
 
-    // ---- 3. eigenvectors Q P Z in G[dof][j]
-    for (int x = tid; x < n * n; x += nt) {
-        const int r = x / n, j = x - (x / n) * n;
-        const double z = Zt[j * n + r];
-        G[x] = (r == n - 1) ? make_double2(z * ph.x, z * ph.y) : make_double2(z, 0.0);
-    }
-    __syncthreads();
-    for (int k = n - 3; k >= 0; --k) {
-        const double2 t = tau[k];
-        if (t.x == 0.0 && t.y == 0.0) continue;
-        for (int j = tid; j < n; j += nt) {
-            double2 dot = G[(size_t)(k + 1) * n + j];
-            for (int i = k + 2; i < n; ++i) dot = cadd(dot, cmulc(A[i * n + k], G[(size_t)i * n + j]));
-            const double2 td = cmul(t, dot);
-            G[(size_t)(k + 1) * n + j] = make_double2(G[(size_t)(k + 1) * n + j].x - td.x,
-                                                      G[(size_t)(k + 1) * n + j].y - td.y);
-            for (int i = k + 2; i < n; ++i) {
-                const double2 u = cmul(A[i * n + k], td);
-                G[(size_t)i * n + j] = make_double2(G[(size_t)i * n + j].x - u.x, G[(size_t)i * n + j].y - u.y);
+    // ---- 2b. implicit QL (thread 0 forms each sweep, all threads rotate Z)
+    if (!done) {
+        for (int x = tid; x < n * n; x += nt) Zt[(x / n) * zl + x % n] = (x / n == x % n) ? 1.0 : 0.0;
+        __syncthreads();
+        int l = 0, iter = 0;                           // thread 0's state
+        for (;;) {
+            if (tid == 0) {
+                ql_go = 0;
+                while (l < n) {
+                    int mm = l;
+                    for (; mm < n - 1; ++mm) {
+                        const double dd = fabs(d[mm]) + fabs(d[mm + 1]);
+                        if (fabs(e[mm]) <= 1.0e-16 * dd) break;
+                    }
+                    if (mm == l) { ++l; iter = 0; continue; }
+                    if (++iter > 60) { ql_fail = 1; ++l; iter = 0; continue; }
+                    double g = (d[l + 1] - d[l]) / (2.0 * e[l]);
+                    double r = hypot(g, 1.0);
+                    g = d[mm] - d[l] + e[l] / (g + copysign(r, g));
+                    double s = 1.0, c = 1.0, p = 0.0;
+                    int i = mm - 1;
+                    bool early = false;
+                    for (; i >= l; --i) {
+                        // one reciprocal square root per rotation: the chain of
+                        // dependent FP64 operations on thread 0 bounds this stage
+                        const double f = s * e[i], b = c * e[i];
+                        const double rr = f * f + g * g;
+                        if (rr == 0.0) {                 // deflation inside the sweep
+                            e[i + 1] = 0.0;
+                            d[i + 1] -= p;
+                            e[mm] = 0.0;
+                            early = true;
+                            break;
+                        }
+                        const double ir = rsqrt(rr);
+                        r = rr * ir;
+                        e[i + 1] = r;
+                        s = f * ir;
+                        c = g * ir;
+                        g = d[i + 1] - p;
+                        r = (d[i] - g) * s + 2.0 * c * b;
+                        p = s * r;
+                        d[i + 1] = g + p;
+                        g = c * r - b;
+                        rc[i] = c;
+                        rs[i] = s;
+                    }
+                    if (!early) {
+                        d[l] -= p;
+                        e[l] = g;
+                        e[mm] = 0.0;
+                    }
+                    ql_hi = mm - 1;
+                    ql_lo = early ? i + 1 : l;
+                    ql_go = 1;
+                    break;
+                }
             }
+            __syncthreads();
+            if (!ql_go) break;
+            const int hi = ql_hi, lo = ql_lo;
+            for (int r = tid; r < n; r += nt)
+                for (int i = hi; i >= lo; --i) {
+                    const double zi1 = Zt[(i + 1) * zl + r], zi = Zt[i * zl + r];
+                    Zt[(i + 1) * zl + r] = rs[i] * zi + rc[i] * zi1;
+                    Zt[i * zl + r] = rc[i] * zi - rs[i] * zi1;
+                }
+            __syncthreads();
         }
+        if (tid == 0 && ql_fail) atomicAdd(nonconv, 1);
+        for (int s = tid; s < n; s += nt) lam[s] = d[s];
     }
-    // ---- 4. ascending order (ties by index), as rows of eig_out
+    // ---- ascending order (ties by index): ord[j] = row of column j in the output
+    __syncthreads();
     for (int s = tid; s < n; s += nt) {
-        const double ls = d[s];
+        const double ls = lam[s];
         int rank = 0;
         for (int t2 = 0; t2 < n; ++t2) {
-            const double lt = d[t2];
+            const double lt = lam[t2];
             rank += (lt < ls) || (lt == ls && t2 < s);
         }
-        ord[rank] = s;
+        ord[s] = rank;
         const double w2 = ls * kEvA2AmuPs2;
         nu_out[(size_t)q * n + rank] = (w2 >= 0.0 ? sqrt(w2) : -sqrt(-w2)) / kTwoPi;
     }
     __syncthreads();
-    for (int x = tid; x < n * n; x += nt) {
-        const int rk = x / n, dof = x - (x / n) * n;
-        eig_out[(size_t)q * n * n + x] = G[(size_t)dof * n + ord[rk]];
+
+    // ---- 3. eigenvectors Q P Z, four lanes per column (row 4 r + lane % 4 in register r)
+    const int rl = tid & 3;
+    for (int j0 = 0; j0 < n; j0 += nt / 4) {
+        const int j = j0 + (tid >> 2);
+        const bool in = j < n;
+        double2 g[kHqlRows];
+#pragma unroll
+        for (int r = 0; r < kHqlRows; ++r) {
+            const int i = 4 * r + rl;
+            const double z = (in && i < n) ? Zt[j * zl + i] : 0.0;
+            g[r] = (i == n - 1) ? make_double2(z * ph.x, z * ph.y) : make_double2(z, 0.0);
+        }
+        for (int k = n - 3; k >= 0; --k) {
+            const double2 t = tau[k];
+            if (t.x == 0.0 && t.y == 0.0) continue;        // uniform
+            double2 dot = make_double2(0.0, 0.0);
+#pragma unroll
+            for (int c = 0; c < kHqlRows / 4; ++c) {
+                if (16 * c + 15 <= k || 16 * c >= n) continue;            // uniform: no row past k here
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int r = 4 * c + u, i = 4 * r + rl;
+                    if (i > k && i < n) cfmac(dot, i == k + 1 ? one : A[i * ld + k], g[r]);
+                }
+            }
+            dot.x += __shfl_xor_sync(0xffffffffu, dot.x, 1);
+            dot.y += __shfl_xor_sync(0xffffffffu, dot.y, 1);
+            dot.x += __shfl_xor_sync(0xffffffffu, dot.x, 2);
+            dot.y += __shfl_xor_sync(0xffffffffu, dot.y, 2);
+            const double2 td = cmul(t, dot);
+#pragma unroll
+            for (int c = 0; c < kHqlRows / 4; ++c) {
+                if (16 * c + 15 <= k || 16 * c >= n) continue;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int r = 4 * c + u, i = 4 * r + rl;
+                    if (i > k && i < n) cfms(g[r], i == k + 1 ? one : A[i * ld + k], td);
+                }
+            }
+        }
+        // ---- 4. rows of eig_out
+        if (in) {
+            double2 *out = eig_out + ((size_t)q * n + ord[j]) * n;
+#pragma unroll
+            for (int r = 0; r < kHqlRows; ++r)
+                if (4 * r + rl < n) out[4 * r + rl] = g[r];
+        }
     }
 }
 
@@ -587,9 +819,12 @@ size_t jacobi_smem_bytes(int nb) {
     return b;
 }
 
-// Per-q Hermitian eigenpairs: the Householder-QL kernel where its shared
+// Complex values of scratch per matrix of launch_jacobi.
+size_t jacobi_scratch(int nb) { return std::max((size_t)nb * nb, hql_scratch(nb)); }
+
+// Per-q Hermitian eigenpairs: the Householder kernel where its shared
 // memory fits (nb <= 96 on GB300), the Jacobi kernel otherwise.  V is a
-// scratch of nq * nb * nb complex values.
+// scratch of nq * jacobi_scratch(nb) complex values.
 cudaError_t launch_jacobi(int nb, int nq, double2 *A, double2 *V, double *nu_thz,
                           double2 *eig_out, int *nonconv, size_t smem_optin, cudaStream_t st) {
     const size_t hsm = hql_layout(nb).bytes;
@@ -597,7 +832,8 @@ cudaError_t launch_jacobi(int nb, int nq, double2 *A, double2 *V, double *nu_thz
         cudaError_t e = cudaFuncSetAttribute(hermitian_ql_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)hsm);
         if (e != cudaSuccess) return e;
-        hermitian_ql_kernel<<<counted(nq), kHqlThreads, hsm, st>>>(nb, A, V, nu_thz, eig_out, nonconv);
+        const int threads = std::min(kHqlThreads, std::max(64, (4 * nb + 31) / 32 * 32));
+        hermitian_ql_kernel<<<counted(nq), threads, hsm, st>>>(nb, A, V, nu_thz, eig_out, nonconv);
         return cudaGetLastError();
     }
     const size_t smem = jacobi_smem_bytes(nb);

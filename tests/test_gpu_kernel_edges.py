@@ -200,3 +200,42 @@ def test_generalised_velocities_wait_limit(k):
         ctx.set_wait_limit(0)
     kap, _ = kk.kald_kappa_qhgk(ctx, [s], nu.ravel(), eig.ravel(), g, opt)
     np.testing.assert_array_equal(kap, ref)
+
+
+def _springs(n, kind):
+    """A Gamma-only n-atom system whose 3n x 3n dynamical matrix (masses 1) is a
+    given symmetric matrix: clustered, multiple and split spectra."""
+    from types import SimpleNamespace
+    nb = 3 * n
+    rng = np.random.default_rng(n)
+    Q = np.linalg.qr(rng.standard_normal((nb, nb)))[0]
+    lam = {"spread": np.linspace(0.1, 4.0, nb),
+           "multiple": np.repeat([0.5, 1.0, 1.0 + 1e-13, 3.0], (nb + 3) // 4)[:nb],
+           "clustered": 1.0 + 1e-9 * np.arange(nb) + (np.arange(nb) % 3),
+           "zero": np.zeros(nb)}.get(kind)
+    D = np.diag(np.arange(1.0, nb + 1) / nb) if kind == "diagonal" else (Q * lam) @ Q.T
+    D = 0.5 * (D + D.T)
+    idx = np.array([[i, j, 0, 0, 0] for i in range(n) for j in range(n)], np.int32)
+    fc2 = np.array([D[3 * i:3 * i + 3, 3 * j:3 * j + 3] for i in range(n) for j in range(n)])
+    s = SimpleNamespace(masses=np.ones(n), positions=rng.random((n, 3)), lattice=10 * np.eye(3), fc2_idx=idx, fc2=fc2,
+                        fc3_idx=np.zeros((0, 9), np.int32), fc3=np.zeros((0, 3, 3, 3)))
+    return s, D
+
+
+@pytest.mark.parametrize("n", [1, 5, 6, 11, 21, 32])
+@pytest.mark.parametrize("kind", ["spread", "multiple", "clustered", "zero", "diagonal"])
+def test_hermitian_eigensolver_spectra(k, n, kind):
+    """3 to 96 branches (QL below 16, inverse iteration above, 15, 18, 33, 63 and
+    96 rows): well separated, multiple and clustered eigenvalues, a zero and a
+    diagonal matrix (no reflector, T split everywhere).  Eigenvalues, residuals
+    and orthonormality to 1e-13 of |D| and of one."""
+    from oracle.units import EV_A2_AMU
+    kk, ctx = k
+    s, D = _springs(n, kind)
+    nu, eig, _ = kk.kald_phonons(ctx, s, (1, 1, 1), want_vel=False)
+    E = eig[0].T                                            # columns = modes
+    scale = max(np.abs(D).sum(axis=1).max(), 1e-30)
+    lam = np.sign(nu[0]) * (2 * np.pi * nu[0]) ** 2 / EV_A2_AMU
+    np.testing.assert_allclose(lam, np.linalg.eigvalsh(D), rtol=0, atol=1e-13 * scale)
+    np.testing.assert_allclose(E.conj().T @ E, np.eye(3 * n), rtol=0, atol=1e-13)
+    assert np.abs(D @ E - E * lam).max() <= 1e-13 * scale
