@@ -78,8 +78,8 @@ typedef enum {
  *    squared projection |phi|^2 of a momentum triple (q1, q2, q3),
  *    q1 + q2 + q3 = 0 modulo G, is the same for every order of the triple, so
  *    one projection per orbit of ordered triples under permutations and
- *    inversion feeds the linewidths of all three members (BF16-split tensor
- *    path, whole-mesh calls). */
+ *    inversion feeds the linewidths of all three members (cells of three to 32
+ *    atoms in every precision, whole-mesh calls). */
 typedef enum {
     KALD_SYM_ALL = 0,        /* every symmetry the path supports (default)    */
     KALD_SYM_INVERSION = 1,  /* time reversal only                            */

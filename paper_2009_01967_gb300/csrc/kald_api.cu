@@ -1118,7 +1118,7 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
         LwParams p{};
         p.nb = h.nb; p.nq = 1;
         p.mesh[0] = p.mesh[1] = p.mesh[2] = 1;
-        p.n_rep = 0; p.n_rounds = 0; p.qp_chunk = 1; p.n_chunks = 1;
+        p.n_rep = 0; p.qp_chunk = 1; p.n_chunks = 1;
         p.q0 = 0; p.q1 = 1;
         p.sigma_w = kTwoPi * opt->sigma_thz;
         p.cut_w = opt->n_sigma * p.sigma_w;
@@ -1151,7 +1151,7 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
         LwParams p;
         p.nb = h.nb; p.nq = 1;
         p.mesh[0] = p.mesh[1] = p.mesh[2] = 1;
-        p.n_rep = 0; p.n_rounds = 0; p.qp_chunk = 1; p.n_chunks = 1;
+        p.n_rep = 0; p.qp_chunk = 1; p.n_chunks = 1;
         p.q0 = 0; p.q1 = 1;
         p.sigma_w = kTwoPi * opt->sigma_thz;
         p.cut_w = opt->n_sigma * p.sigma_w;
@@ -1417,14 +1417,44 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
                 while (at <= y_n_at) y_gi[(size_t)g * (y_n_at + 1) + at++] = b1;
             }
         }
-        YSchedule ys;                            // lane schedule of the CUDA-core kernel's Y build
-        if (!small && !tcx) plan_ybuild(h, ys);
-        p.n_rounds = ys.n_rounds;
+        // CUDA-core kernel: terms and tables of its phase sums (tables within 16 GB
+        // and half of the context's limit), and one projection per orbit of momentum
+        // triples over the whole mesh when Phi3 is symmetric under permutations
+        const bool cc = !small && !tcx;
+        LwTermsHost lt;
+        size_t lw_tab[3] = {0, 0, 0};
+        int cc_pairs = 0;
+        if (cc) {
+            plan_lw_terms(h, true, lt);
+            size_t all = 0;
+            for (int c = 0; c < 3; ++c) {
+                lw_tab[c] = (f32w ? sizeof(float2) : sizeof(double2)) * 27 * (size_t)lt.n_slot[c] * nq;
+                all += lw_tab[c];
+            }
+            if (all > (size_t(16) << 30) || (ctx->ws_limit && all > ctx->ws_limit / 2)) {
+                plan_lw_terms(h, false, lt);
+                lw_tab[0] = lw_tab[1] = lw_tab[2] = 0;
+            }
+            if (!listed && reuse && opt->symmetry == KALD_SYM_ALL && nq > 1) {
+                if (h.fc3_perm_symmetric < 0) h.fc3_perm_symmetric = fc3_symmetric_all(&sys[x]) ? 1 : 0;
+                if (h.fc3_perm_symmetric) cc_pairs = std::max(0, orbit_pairs(mesh));
+            }
+        }
+        std::vector<int> orb_rows;
+        size_t cc_out3 = 0, cc_sums = 0;         // position sums of the mode blocks, and where their totals start
+        if (cc_pairs) {
+            const int blocks = lw_orbit_blocks(nb, cc_pairs, f32w, ctx->sm_count, ctx->smem_optin);
+            cc_sums = blocks > 1 ? 3 * (size_t)cc_pairs * nb * blocks : 0;
+            cc_out3 = 3 * (size_t)cc_pairs * nb * (blocks > 1 ? blocks + 1 : 1);
+            orb_rows.resize(nqc);
+            for (int i = 0; i < nqc; ++i) orb_rows[i] = qsel[i].x;
+            p.n_chunks = 1;
+        }
         if (small) p.n_rep = 0;                  // the register kernel takes its phases from roots of unity
         std::vector<int4> binfo(small ? 1 : std::max<size_t>(n3, 1), make_int4(0, 0, 0, 0));
         for (size_t b = 0; !small && b < n3; ++b) binfo[b] = make_int4(h.fc3_i[b], h.fc3_rj[b], h.fc3_rk[b], 0);
         const size_t c2 = f32w ? sizeof(float2) : sizeof(double2);
-        size_t need = bytes_of(ys.group_jk) + bytes_of(ys.segs) + bytes_of(ys.sched) + bytes_of(binfo) +
+        size_t need = bytes_of(binfo) +
                       (small ? scaled_bytes(sn_raw, sn_atoms, h, 27, 28, 0)
                              : scaled_bytes(h.fc3_blk, h.fc3_atoms, h, 27, 28, f32w)) +
                       bytes_of(h.rep_cart) + bytes_of(qc) + bytes_of(qf) +
@@ -1447,11 +1477,13 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         if (small)
             need += bytes_of(sn_kk) + bytes_of(sn_bj) + bytes_of(sn_bk) + bytes_of(sn_start) +
                     ws_round(sizeof(double2) * (2 * (size_t)sn_m0 + 1)) + ws_round(sn_tab);
+        if (cc)
+            need += bytes_of(lt.group) + bytes_of(lt.term_start) + bytes_of(lt.term) + bytes_of(lt.slot_start) +
+                    bytes_of(lt.slot_blk) + ws_round(lw_tab[0]) + ws_round(lw_tab[1]) + ws_round(lw_tab[2]);
+        if (cc_pairs)
+            need += bytes_of(orb_rows) + ws_round(orbit_bytes(mesh, nqc)) + ws_round(sizeof(double) * cc_out3);
         if ((st = ws_reserve(ctx, need))) return st;
         LwDev d;
-        d.group_jk = upload(ctx, ys.group_jk);
-        d.segs = upload(ctx, ys.segs);
-        d.sched = upload(ctx, ys.sched);
         d.blkinfo = upload(ctx, binfo);
         // Phi3 / sqrt(mi mj mk), 28 values per block (16-byte loads), in the working precision
         d.fc3 = small ? upload_scaled(ctx, sn_raw, sn_atoms, h, 27, 28, 0)
@@ -1528,12 +1560,37 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
             sn.tab = sn_tab ? ws_take(ctx, sn_tab) : nullptr;
         }
         cudaStream_t s = ctx->stream;
-        cudaError_t e = launch_lw_prep(p, d, f32w, s);
+        LwTerms terms;
+        OrbitPlan orb;
+        cudaError_t e = cudaSuccess;
+        if (cc) {
+            terms.group = upload(ctx, lt.group);
+            terms.term_start = upload(ctx, lt.term_start);
+            terms.term = upload(ctx, lt.term);
+            terms.slot_start = upload(ctx, lt.slot_start);
+            terms.slot_blk = upload(ctx, lt.slot_blk);
+            for (int c = 0; c < 3; ++c) {
+                terms.n_slot[c] = lt.n_slot[c];
+                terms.slot0[c] = lt.slot0[c];
+                terms.tab[c] = ws_take(ctx, lw_tab[c]);
+            }
+            if (cc_pairs) {
+                const int *rows_d = upload(ctx, orb_rows);
+                void *work = ws_take(ctx, orbit_bytes(mesh, nqc));
+                terms.out3 = static_cast<double *>(ws_take(ctx, sizeof(double) * cc_out3));
+                e = launch_orbit_plan(mesh, nqc, rows_d, d.qrow, work, orb, s);     // whole mesh: qrow[q] is q's row
+                terms.n_pairs = orb.n_pairs;
+                terms.pairs = orb.pairs;
+                terms.orbit = orb.orbit;
+            }
+        }
+        if (e == cudaSuccess) e = launch_lw_prep(p, d, f32w, s);
         if (e == cudaSuccess)
             e = small ? launch_lw_small(p, d, sn, f32w, s)
                 : tcx ? launch_lw_tensor(p, d, tg, tc_scr, tcx_b, ctx->sm_count, tc_err, s,
                                          use_sym ? &tsym : nullptr, sym_scr)
-                      : launch_lw_main(p, d, f32w, ctx->sm_count, ctx->smem_optin, s);
+                      : launch_lw_main(p, d, terms, f32w, ctx->sm_count, ctx->smem_optin, s);
+        if (e == cudaSuccess && cc_pairs) e = launch_orbit_class_sums(orb, nb, terms.out3 + cc_sums, d.partial, s);
         if (e == cudaSuccess) e = launch_lw_finish(p, d, opt->degen_tol_thz, g_d, s);
         if (e != cudaSuccess) return cuda_check(ctx, e, "kald_linewidths launch");
         unsigned long long al = 0;
@@ -1545,7 +1602,7 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         if (errf) return fail(ctx, KALD_E_TIMEOUT, "kald_linewidths: a tensor-core pipeline wait expired");
         tot += (uint64_t)nqr * nq * (uint64_t)nb * nb * nb;
         // one projection per orbit counts three times the orbit's ordered triples
-        allowed_tot += use_sym ? (al + 1) / 3 : al;
+        allowed_tot += use_sym ? (al + 1) / 3 : cc_pairs ? al / 6 : al;
         off_nb += (size_t)nq * nb;
         off_eig += nn;
     }

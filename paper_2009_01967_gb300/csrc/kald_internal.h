@@ -223,7 +223,6 @@ cudaError_t launch_vel_diag(const DevFc2 &f, int nb, int nq, size_t n_blk, const
 struct LwParams {
     int nb, nq, mesh[3];
     int n_rep;
-    int n_rounds;             // rounds of the Y-build lane schedule
     double sigma_w;           // 2 pi sigma (rad/ps)
     double cut_w;             // n_sigma * sigma_w
     int shape;                // energy-delta shape (kald_options.delta_shape)
@@ -239,18 +238,8 @@ struct LwParams {
     uint32_t wait_limit;      // polls of the tensor-core pipeline waits
     Prof *prof;               // per-launch timing (NULL: off); host pointer, never read on the device
 };
-// Y-build lane schedule (built on the host by plan_ybuild): in round r lane t
-// runs segments sched[r*kLwThreads+t] .. sched[r*kLwThreads+t+1]-1.  A segment is
-// (group, first block, end block, red): the blocks of one (j, k) atom pair,
-// or a slice of them; red > 1 marks a slice whose partial sums are added
-// across `red` aligned lanes with shuffles (a "heavy" round: every lane has
-// exactly one segment, all with the same red); group < 0 is an empty slot.
-constexpr int kLwThreads = 512;
 struct LwDev {
-    const int *group_jk;      // [n_groups][2] atoms (j, k)
-    const int4 *segs;         // [n_seg] (group, b0, b1, red)
-    const int *sched;         // [n_rounds * kLwThreads + 1]
-    const int4 *blkinfo;      // [n_fc3] (i, rep(Rj), rep(Rk), 0), schedule order
+    const int4 *blkinfo;      // [n_fc3] (i, rep(Rj), rep(Rk), 0), HostSystem order
     const void *fc3;          // [n_fc3][28] float or double, Phi3 / sqrt(mi mj mk), padded
     const double *rep_cart;   // [n_rep][3]
     const double *qcart;      // [nq][3]
@@ -281,17 +270,54 @@ struct LwDev {
     unsigned long long *allowed;   // [1] delta-allowed triplet count
     int *queue;               // [1] work counter
 };
-struct YSchedule {
-    std::vector<int> group_jk;     // [n_groups][2]
-    std::vector<int4> segs;
-    std::vector<int> sched;
-    std::vector<int> blk_order;    // schedule position -> block index of HostSystem fc3 order
-    int n_rounds = 0;
+// orbits.cu: orbits of momentum triples on a whole mesh, enumerated on the
+// device.  rows: the lower index of each pair {q, -q}, ascending; row_of [nq]: the
+// row of a q-point that has one.
+struct OrbitPlan {
+    int n_pairs = 0, n_rows = 0, nq = 0;
+    int mesh[3] = {0, 0, 0};
+    const int2 *pairs = nullptr;    // [n_pairs] (q1, q2), by row
+    const int *orbit = nullptr;     // [n_pairs] ordered triples in the orbit
+    const uint2 *bits = nullptr;    // [n_rows][words] (canonical q2, canonical ones before)
+    const int *start = nullptr;     // [n_rows + 1] first pair of a row
+    const int *rows = nullptr, *row_of = nullptr;
 };
-// Build the lane schedule of the Y-build for one planned system.
-void plan_ybuild(const HostSystem &h, YSchedule &ys);
+int orbit_pairs(const int32_t mesh[3]);           // number of orbits, -1: too many to index
+size_t orbit_bytes(const int32_t mesh[3], int n_rows);
+cudaError_t launch_orbit_plan(const int32_t mesh[3], int n_rows, const int *rows, const int *row_of, void *work,
+                              OrbitPlan &o, cudaStream_t st);
+// out [n_rows][nb]: sums of each row's q from the positions' sums out3
+// [n_pairs][3][nb] (nb <= 96) of its orbits.
+cudaError_t launch_orbit_class_sums(const OrbitPlan &o, int nb, const float *out3, double *out, cudaStream_t st);
+cudaError_t launch_orbit_class_sums(const OrbitPlan &o, int nb, const double *out3, double *out, cudaStream_t st);
+
+// The phase sums of the CUDA-core kernel (plan_lw_terms): per (j, k) group its
+// terms (i, class, slot) -- phase sums of class 0, 1 or 2 from tables per q', q''
+// or q -- or (i, 3, block), phased per pair.  n_pairs > 0: one projection per
+// orbit (pairs, orbit of an OrbitPlan, the positions' sums into out3).
+struct LwTermsHost {
+    std::vector<int> group, term_start, slot_start, slot_blk;
+    std::vector<int4> term;
+    int n_slot[3] = {0, 0, 0}, slot0[3] = {0, 0, 0};
+};
+struct LwTerms {
+    const int *group = nullptr;        // [n_atoms^2] group of (j, k), -1: none
+    const int *term_start = nullptr;   // [n_groups + 1]
+    const int4 *term = nullptr;
+    const int *slot_start = nullptr;   // blocks of each slot, the classes' slots one after another
+    const int *slot_blk = nullptr;
+    int n_slot[3] = {0, 0, 0}, slot0[3] = {0, 0, 0};
+    void *tab[3] = {nullptr, nullptr, nullptr};   // [nq][n_slot][27] complex
+    int n_pairs = 0;
+    const int2 *pairs = nullptr;
+    const int *orbit = nullptr;
+    double *out3 = nullptr;            // [n_pairs][blocks][3][nb] (lw_orbit_blocks)
+    int n_sblk = 1, s_per = 0;         // blocks of modes per item, modes per block (set by the launch)
+};
+int lw_orbit_blocks(int nb, int n_pairs, int fp32, int sm_count, size_t smem_optin);
+void plan_lw_terms(const HostSystem &h, bool tables, LwTermsHost &o);
 cudaError_t launch_lw_prep(const LwParams &p, const LwDev &d, int fp32, cudaStream_t st);
-cudaError_t launch_lw_main(const LwParams &p, const LwDev &d, int fp32, int sm_count,
+cudaError_t launch_lw_main(const LwParams &p, const LwDev &d, const LwTerms &t, int fp32, int sm_count,
                            size_t smem_optin, cudaStream_t st);
 cudaError_t launch_lw_finish(const LwParams &p, const LwDev &d, double degen_tol_thz,
                              double *gamma_out, cudaStream_t st);

@@ -17,13 +17,15 @@
 // hbar pi / (8 N_k) (eV/A^2 amu -> ps^-2)^3 / (sqrt(2 pi) sigma w) is applied
 // per mode at the end in FP64.
 //
-// Work: a persistent grid pulls items (q, chunk of q') from a device counter
-// (atomicAdd only; nothing waits).  Each item writes its own FP64 partial
-// sums, which a second kernel adds in a fixed order, so results do not
-// depend on the schedule.
+// Work: a persistent grid pulls items -- (q, chunk of q'), or one orbit of
+// momentum triples (OrbitPlan) -- from a device counter (atomicAdd only; nothing
+// waits).  Each item writes its own FP64 partial sums, which a second kernel adds
+// in a fixed order, so results do not depend on the schedule.
 
 #include <algorithm>
+#include <array>
 #include <type_traits>
+#include <vector>
 
 #include "kald_internal.h"
 #include "wdiff.cuh"
@@ -43,7 +45,7 @@ template <> __device__ __forceinline__ double2 mk<double2>(double x, double y) {
     return make_double2(x, y);
 }
 
-constexpr int kThreads = kLwThreads;   // 512: 16 warps per SM
+constexpr int kThreads = 512;          // most threads of a CTA
 constexpr int kTR = 6;                 // register tile: kTR rows (s') ...
 constexpr int kTC = 3;                 // ... by kTC columns (complex)
 
@@ -116,57 +118,119 @@ __device__ __forceinline__ R2 cmul(const R2 a, const R2 b) {
     return r;
 }
 
-// Load the 28 (27 + pad) scaled Phi3 values of one block.
-__device__ __forceinline__ void load_blk(const float *f, float v[28]) {
-    const float4 *f4 = reinterpret_cast<const float4 *>(f);
-#pragma unroll
-    for (int x = 0; x < 7; ++x) {
-        const float4 t = __ldg(f4 + x);
-        v[4 * x] = t.x; v[4 * x + 1] = t.y; v[4 * x + 2] = t.z; v[4 * x + 3] = t.w;
-    }
-}
-__device__ __forceinline__ void load_blk(const double *f, double v[28]) {
-    const double2 *f2 = reinterpret_cast<const double2 *>(f);
-#pragma unroll
-    for (int x = 0; x < 14; ++x) {
-        const double2 t = __ldg(f2 + x);
-        v[2 * x] = t.x; v[2 * x + 1] = t.y;
+// Phase sums of one q-point, [nq][slots][27] per class: the blocks of each
+// (j, k, i) whose phase depends on q' alone (class 0: Rk = 0, chi(q', Rj)), on
+// q'' alone (class 1: Rj = 0, conj chi(q'', Rk)) or on q alone (class 2:
+// Rj = Rk, conj chi(q, R)); see LwTerms.  One thread per value, sums in FP64.
+template <typename R>
+__global__ void lw_tables_kernel(int nq, int n_rep, LwTerms t, const int4 *__restrict__ blkinfo,
+                                 const R *__restrict__ fc3, const typename C2<R>::T *__restrict__ chi) {
+    using R2 = typename C2<R>::T;
+    for (int cls = 0; cls < 3; ++cls) {
+        const size_t per = (size_t)t.n_slot[cls] * 27, n = per * nq;
+        R2 *out = static_cast<R2 *>(t.tab[cls]);
+        for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < n; x += (size_t)gridDim.x * blockDim.x) {
+            const size_t q = x / per, e = x - q * per;
+            const int slot = t.slot0[cls] + (int)(e / 27), v = (int)(e % 27);
+            double re = 0.0, im = 0.0;
+            for (int y = t.slot_start[slot]; y < t.slot_start[slot + 1]; ++y) {
+                const int b = t.slot_blk[y];
+                const int4 bi = __ldg(blkinfo + b);
+                const R2 z = chi[q * n_rep + (cls == 1 ? bi.z : bi.y)];
+                const double f = (double)fc3[(size_t)28 * b + v];
+                re += f * (double)z.x;
+                im += cls == 0 ? f * (double)z.y : -f * (double)z.y;
+            }
+            out[x] = mk<R2>(re, im);
+        }
     }
 }
 
-// Shared memory layout (R2 = complex of the working precision; P = nb
-// rounded up to a multiple of kTR, Q = P + 1):
-//   Y    [P][Q]     Y(b, c) at b*P + c, then T'^T(c, s') at c*Q + s' (odd
-//                   pitch: the transposed store walks distinct banks)
-//   EpT  [P][P]     eps(q')^T            (only when operands live in smem)
-//   EppT [P][P]     conj(eps(q''))^T     (only when operands live in smem)
-//   es   [P]        eps(q, s) column
-//   chip, chipp [n_rep]    chi(q'), chi(q'')
-//   wp, np_, wpp, npp [P]  omega and n of q' / q'' (R; the hi parts for FP32)
-//   wpl, npl, wppl, nppl [P]  lo parts of the FP32 pairs (FP32 only; wdiff.cuh)
-//   red  [nb] double       per-mode sums over the item's q' (fixed order)
-//   wsum [nwarps] double   per-warp sums of the current mode
-//   tiles [kThreads] short active (s', s'') tiles of the delta band
-template <typename R, bool OPER_SMEM>
+// out [n_pairs][per]: the n_sblk mode blocks' position sums of a pair added in order.
+__global__ void lw_block_sums_kernel(size_t n, int per, int n_sblk, const double *__restrict__ out3,
+                                     double *__restrict__ out) {
+    for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < n; x += (size_t)gridDim.x * blockDim.x) {
+        const size_t pair = x / per, e = x - pair * per;
+        double v = 0.0;
+        for (int b = 0; b < n_sblk; ++b) v += out3[(pair * n_sblk + b) * per + e];
+        out[x] = v;
+    }
+}
+
+// Hits of one (s, s', s'') over the six ordered triples (p, a, b) of its three
+// modes: |w_p + w_a - w_b| or |w_p - w_a - w_b| inside the window, each formed
+// in the order in which the projection of (p, a) would form it.
+__device__ __forceinline__ unsigned window_hits6(const F2 (&w)[3], float cut) {
+    unsigned n = 0;
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+#pragma unroll
+        for (int o = 1; o < 3; ++o) {
+            const F2 a = w[(p + o) % 3], b = w[(p + 3 - o) % 3];
+            n += fabsf(f2_diff(f2_add(w[p], a), b)) < cut || fabsf(f2_diff(f2_add(w[p], f2_neg(a)), b)) < cut;
+        }
+    return n;
+}
+__device__ __forceinline__ unsigned window_hits6(const double (&w)[3], double cut) {
+    unsigned n = 0;
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+#pragma unroll
+        for (int o = 1; o < 3; ++o) {
+            const double a = w[(p + o) % 3], b = w[(p + 3 - o) % 3];
+            n += fabs(w[p] + a - b) < cut || fabs(w[p] - a - b) < cut;
+        }
+    return n;
+}
+
+// Shared memory of a CTA of sb modes and nthr threads (R2 = complex of the
+// working precision; P = nb rounded up to a multiple of kTR, Q = P + 1):
+//   Y    [sb][P][Q]  Y(b, c) at b*P + c, then T'^T(c, s') at c*Q + s' (odd
+//                    pitch: the transposed store walks distinct banks)
+//   EpT, EppT [P][P] eps(q')^T and conj(eps(q''))^T (only when they fit: oper)
+//   es   [sb][P]     eps(q, s) columns
+//   wp, np_, wpp, npp [P]     omega and n of q' / q'' (R; the hi parts for FP32)
+//   wpl, npl, wppl, nppl [P]  lo parts of the FP32 pairs (wdiff.cuh)
+//   red  [3][nb] double  the item's sums per mode (of each position of an orbit)
+//   psum [nthr], prow [nthr][6], pcol [nthr][3] double  sums of the listed tiles
+//                    (rows and columns: orbits only)
+//   tiles [nthr] int the (mode, tile) pairs the delta windows reach
+template <typename R>
+__host__ __device__ inline size_t lw_smem_bytes(int nb, int sb, int nthr, bool oper, bool orbit) {
+    const size_t P = (size_t)((nb + kTR - 1) / kTR) * kTR;
+    size_t b = 2 * sizeof(R) * (sb * P * (P + 1) + (oper ? 2 * P * P : 0) + sb * P);
+    b += sizeof(R) * 8 * P;
+    b = (b + 15) & ~size_t(15);
+    b += sizeof(double) * (3 * (size_t)nb + (size_t)nthr * (orbit ? 10 : 1));
+    b += sizeof(int) * (size_t)nthr;
+    return b + 32;
+}
+
+// Bound: FMA issue (FP64: 2 per clock and SM).  Y_s(b, c) is summed from the
+// tables of LwTerms, one thread per (mode, atom pair); both contractions run in
+// 6 x 3 register tiles, sb modes side by side so that small cells fill the CTA;
+// GEMM2 only on the tiles that a window reaches.  ORBIT: one projection per
+// orbit of momentum triples, three weights per element, the sums of all three
+// positions into out3.  Eight atoms (24 branches), 4^3 mesh, FP64: 74 ms with
+// every block phased for every mode, one mode per CTA and one q-point of each
+// pair {q, -q}; 4.8 ms now.
+template <typename R, bool OPER_SMEM, bool ORBIT>
 __global__ void __launch_bounds__(kThreads, 1)
-lw_main_kernel(LwParams p, LwDev d, const R *__restrict__ fc3,
-               const typename C2<R>::T *__restrict__ epsT_all,
-               const typename C2<R>::T *__restrict__ chi_all) {
+lw_main_kernel(LwParams p, LwDev d, LwTerms t, int SB, const R *__restrict__ fc3,
+               const typename C2<R>::T *__restrict__ epsT_all, const typename C2<R>::T *__restrict__ chi_all) {
     using R2 = typename C2<R>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int nwarps = kThreads / 32;
-    const int nb = p.nb;
+    const int nb = p.nb, nthr = blockDim.x;
     const int P = ((nb + kTR - 1) / kTR) * kTR;
-    const int Q = P + 1;
+    const int Q = P + 1, na = nb / 3, nap = P / 3;
     const int tcols = P / kTC;                       // column tiles
-    const int n_tiles = (P / kTR) * tcols;           // <= 512 for nb <= 96
+    const int n_tiles = (P / kTR) * tcols;
+    const size_t ysz = (size_t)P * Q;
     R2 *Y = reinterpret_cast<R2 *>(smem_raw);
-    R2 *EpT = Y + (size_t)P * Q;
+    R2 *EpT = Y + SB * ysz;
     R2 *EppT = OPER_SMEM ? EpT + (size_t)P * P : EpT;
     R2 *es = OPER_SMEM ? EppT + (size_t)P * P : EpT;
-    R2 *chip = es + P;
-    R2 *chipp = chip + p.n_rep;
-    R *wp = reinterpret_cast<R *>(chipp + p.n_rep);
+    R *wp = reinterpret_cast<R *>(es + SB * P);
     R *np_ = wp + P;
     R *wpp = np_ + P;
     R *npp = wpp + P;
@@ -175,33 +239,46 @@ lw_main_kernel(LwParams p, LwDev d, const R *__restrict__ fc3,
     R *wppl = npl + P;
     R *nppl = wppl + P;
     constexpr bool kPair = std::is_same<R, float>::value;
-    double *red = reinterpret_cast<double *>(
-        (reinterpret_cast<uintptr_t>(nppl + P) + 15) & ~uintptr_t(15));
-    double *wsum = red + nb;
-    short *tiles = reinterpret_cast<short *>(wsum + nwarps);
-    __shared__ int item_sm, n_act_sm, warp_cnt[nwarps];
+    double *red = reinterpret_cast<double *>((reinterpret_cast<uintptr_t>(nppl + P) + 15) & ~uintptr_t(15));
+    double *psum = red + 3 * nb;
+    double *prow = psum + nthr, *pcol = prow + 6 * (size_t)(ORBIT ? nthr : 0);
+    int *tiles = reinterpret_cast<int *>(pcol + 3 * (size_t)(ORBIT ? nthr : 0));
+    __shared__ int item_sm, n_act_sm, warp_cnt[kThreads / 32];
 
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = nthr >> 5;
     const R sig2inv = (R)delta_param(p.shape, p.sigma_w);   // the delta shape's parameter
     const R cut = (R)p.cut_w;
-    const int n_items = p.nqc * p.n_chunks;
+    // an orbit's count is formed member by member where a window's edge is near
+    // (the members' sums round differently): closer than the rounding of FP32
+    // pairs or FP64
+    const R edge = cut * (kPair ? (R)1e-4 : (R)1e-9) + (kPair ? (R)1e-5 : (R)1e-12);
+    // items: (pair or q chunk, block of modes), n_sblk blocks of s_per modes each
+    const int n_items = (ORBIT ? t.n_pairs : p.nqc * p.n_chunks) * t.n_sblk;
     unsigned long long allowed = 0;
 
     for (;;) {
         if (tid == 0) item_sm = atomicAdd(d.queue, 1);
         __syncthreads();
-        const int item = item_sm;
+        const int item_all = item_sm;
         __syncthreads();
-        if (item >= n_items) break;
-        const int qi = item / p.n_chunks;
-        const int2 qm = d.qsel[qi];
-        const int q = qm.x;
-        const int chunk = item % p.n_chunks;
-        const unsigned long long allowed0 = allowed;
-        for (int x = tid; x < nb; x += kThreads) red[x] = 0.0;
+        if (item_all >= n_items) break;
+        const int item = item_all / t.n_sblk, sblk = item_all - item * t.n_sblk;
+        const int sbeg = sblk * t.s_per, send = min(nb, sbeg + t.s_per);
+        int q, qp0, qp1, mult;
+        if (ORBIT) {
+            const int2 pr = t.pairs[item];
+            q = pr.x; qp0 = pr.y; qp1 = pr.y + 1;
+            mult = t.orbit[item];
+        } else {
+            const int2 qm = d.qsel[item / p.n_chunks];
+            q = qm.x;
+            mult = qm.y;                             // an item of q stands for -q as well when it takes q's linewidths
+            qp0 = (item % p.n_chunks) * p.qp_chunk;
+            qp1 = min(p.nq, qp0 + p.qp_chunk);
+        }
+        unsigned long long hits = 0;
+        for (int x = tid; x < 3 * nb; x += nthr) red[x] = 0.0;
 
-        const int qp0 = chunk * p.qp_chunk;
-        const int qp1 = min(p.nq, qp0 + p.qp_chunk);
         for (int qp = qp0; qp < qp1; ++qp) {
             // q'' = q + q' on the mesh
             const int *kq = d.qfrac + 3 * q, *kp = d.qfrac + 3 * qp;
@@ -210,12 +287,7 @@ lw_main_kernel(LwParams p, LwDev d, const R *__restrict__ fc3,
             const int k2 = (kq[2] + kp[2]) % p.mesh[2];
             const int qpp = (k0 * p.mesh[1] + k1) * p.mesh[2] + k2;
             __syncthreads();
-            // stage per-pair data
-            for (int x = tid; x < p.n_rep; x += kThreads) {
-                chip[x] = chi_all[(size_t)qp * p.n_rep + x];
-                chipp[x] = chi_all[(size_t)qpp * p.n_rep + x];
-            }
-            for (int x = tid; x < P; x += kThreads) {
+            for (int x = tid; x < P; x += nthr) {
                 const bool in = x < nb;
                 if constexpr (kPair) {
                     const float4 a = in ? d.wn32[(size_t)qp * nb + x] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -232,7 +304,7 @@ lw_main_kernel(LwParams p, LwDev d, const R *__restrict__ fc3,
             if (OPER_SMEM) {
                 const R2 *src1 = epsT_all + (size_t)qp * nb * nb;
                 const R2 *src2 = epsT_all + (size_t)qpp * nb * nb;
-                for (int x = tid; x < P * P; x += kThreads) {
+                for (int x = tid; x < P * P; x += nthr) {
                     const int b = x / P, s = x % P;
                     const bool in = (b < nb) && (s < nb);
                     R2 v1 = in ? src1[b * nb + s] : mk<R2>(0.0, 0.0);
@@ -242,69 +314,76 @@ lw_main_kernel(LwParams p, LwDev d, const R *__restrict__ fc3,
                     EppT[x] = v2;
                 }
             }
-            __syncthreads();
+            // the tables' rows of this pair
+            const R2 *tab[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+                tab[c] = static_cast<const R2 *>(t.tab[c]) + (size_t)(c == 0 ? qp : c == 1 ? qpp : q) * t.n_slot[c] * 27;
 
-            for (int s = 0; s < nb; ++s) {
-                const double w_s = d.omega[(size_t)q * nb + s];
-                if (w_s <= 0.0) continue;              // masked mode (uniform branch)
-                const R w = (R)w_s;
-                const F2 wsp = f2_of(w_s);             // FP32 pair of w (FP32 epilogue)
-                // ---- Y_s: zero, then the scheduled gather over fc3 blocks
-                for (int x = tid; x < P; x += kThreads)
-                    es[x] = x < nb ? epsT_all[((size_t)q * nb + x) * nb + s] : mk<R2>(0.0, 0.0);
-                for (int x = tid; x < P * P; x += kThreads) Y[x] = mk<R2>(0.0, 0.0);
+            for (int s0 = sbeg; s0 < send; s0 += SB) {
+                const int ns = min(SB, send - s0);
                 __syncthreads();
-                for (int r = 0; r < p.n_rounds; ++r) {
-                    const int g0 = d.sched[r * kThreads + tid], g1 = d.sched[r * kThreads + tid + 1];
-                    for (int sg = g0; sg < g1; ++sg) {
-                        const int4 seg = d.segs[sg];
-                        R2 acc9[9];
+                for (int x = tid; x < ns * P; x += nthr) {
+                    const int m = x / P, b = x - m * P;
+                    es[m * P + b] = b < nb ? epsT_all[((size_t)q * nb + b) * nb + s0 + m] : mk<R2>(0.0, 0.0);
+                }
+                __syncthreads();
+                // ---- Y_s(3j.., 3k..): one thread per (atom pair, mode), modes fastest;
+                // padding atoms and pairs without blocks are zero
+                for (int x = tid; x < nap * nap * ns; x += nthr) {
+                    const int jk = x / ns, m = x - jk * ns, j = jk / nap, k = jk - j * nap;
+                    R2 acc9[9];
 #pragma unroll
-                        for (int x = 0; x < 9; ++x) acc9[x] = mk<R2>(0.0, 0.0);
-                        for (int bl = seg.y; bl < seg.z; ++bl) {
-                            const int4 bi = __ldg(d.blkinfo + bl);
-                            R v[28];
-                            load_blk(fc3 + (size_t)28 * bl, v);
-                            const R2 a = chip[bi.y], b = chipp[bi.z];
-                            // P = chi(q', Rj) conj(chi(q'', Rk))
-                            R2 ph;
-                            ph.x = a.x * b.x + a.y * b.y;
-                            ph.y = a.y * b.x - a.x * b.y;
-                            const R2 e0 = cmul(es[3 * bi.x], ph);
-                            const R2 e1 = cmul(es[3 * bi.x + 1], ph);
-                            const R2 e2 = cmul(es[3 * bi.x + 2], ph);
+                    for (int e = 0; e < 9; ++e) acc9[e] = mk<R2>(0.0, 0.0);
+                    const int g = (j < na && k < na) ? __ldg(t.group + j * na + k) : -1;
+                    if (g >= 0) {
+                        const R2 *em = es + m * P;
+                        for (int y = t.term_start[g]; y < t.term_start[g + 1]; ++y) {
+                            const int4 tm = __ldg(t.term + y);               // (i, class, slot or block)
+                            const R2 *e3 = em + 3 * tm.x;
+                            if (tm.y < 3) {
+                                const R2 *w = (tm.y == 0 ? tab[0] : tm.y == 1 ? tab[1] : tab[2]) + (size_t)27 * tm.z;
 #pragma unroll
-                            for (int x = 0; x < 9; ++x) {
-                                acc9[x].x = fma(v[x], e0.x, fma(v[9 + x], e1.x, fma(v[18 + x], e2.x, acc9[x].x)));
-                                acc9[x].y = fma(v[x], e0.y, fma(v[9 + x], e1.y, fma(v[18 + x], e2.y, acc9[x].y)));
+                                for (int a = 0; a < 3; ++a) {
+                                    const R2 ev = e3[a];
+#pragma unroll
+                                    for (int e = 0; e < 9; ++e) cfma(acc9[e], ev, w[9 * a + e]);
+                                }
+                            } else {
+                                const int4 bi = __ldg(d.blkinfo + tm.z);
+                                const R2 u = chi_all[(size_t)qp * p.n_rep + bi.y], v = chi_all[(size_t)qpp * p.n_rep + bi.z];
+                                R2 ph;                                       // chi(q', Rj) conj(chi(q'', Rk))
+                                ph.x = u.x * v.x + u.y * v.y;
+                                ph.y = u.y * v.x - u.x * v.y;
+                                const R *f = fc3 + (size_t)28 * tm.z;
+#pragma unroll
+                                for (int a = 0; a < 3; ++a) {
+                                    const R2 ev = cmul(e3[a], ph);
+#pragma unroll
+                                    for (int e = 0; e < 9; ++e) {
+                                        const R fv = __ldg(f + 9 * a + e);
+                                        acc9[e].x = fma(fv, ev.x, acc9[e].x);
+                                        acc9[e].y = fma(fv, ev.y, acc9[e].y);
+                                    }
+                                }
                             }
                         }
-                        const int rr = seg.w;
-                        if (rr > 1) {                  // heavy slice: add the R lanes' partials
-                            for (int o = rr >> 1; o > 0; o >>= 1)
-#pragma unroll
-                                for (int x = 0; x < 9; ++x) {
-                                    acc9[x].x += __shfl_xor_sync(0xffffffffu, acc9[x].x, o);
-                                    acc9[x].y += __shfl_xor_sync(0xffffffffu, acc9[x].y, o);
-                                }
-                        }
-                        if (seg.x >= 0 && (rr <= 1 || (lane & (rr - 1)) == 0)) {
-                            const int j = d.group_jk[2 * seg.x], k = d.group_jk[2 * seg.x + 1];
-#pragma unroll
-                            for (int x = 0; x < 9; ++x)
-                                Y[(size_t)(3 * j + x / 3) * P + 3 * k + x % 3] = acc9[x];
-                        }
                     }
+                    R2 *Ym = Y + m * ysz + (size_t)(3 * j) * P + 3 * k;
+#pragma unroll
+                    for (int e = 0; e < 9; ++e) Ym[(e / 3) * P + e % 3] = acc9[e];
                 }
                 __syncthreads();
 
                 // ---- GEMM1: T'(s', c) = sum_b epsT'(b, s') Y(b, c), dense.
-                // A warp holds one row tile (broadcast A) over 32 column tiles.
-                const int ti = tid / tcols, tj = tid % tcols;
-                const bool active = tid < n_tiles;
+                // A warp holds one row tile (broadcast A) over its column tiles.
+                const int m1 = tid / n_tiles, tile1 = tid - m1 * n_tiles;
+                const int ti = tile1 / tcols, tj = tile1 % tcols;
+                const bool active = m1 < ns;
                 int r0 = ti * kTR, c0 = tj * kTC;
                 R2 acc[kTR][kTC];
                 if (active) {
+                    const R2 *Ym = Y + m1 * ysz;
 #pragma unroll
                     for (int r = 0; r < kTR; ++r)
 #pragma unroll
@@ -317,67 +396,71 @@ lw_main_kernel(LwParams p, LwDev d, const R *__restrict__ fc3,
                         for (int r = 0; r < kTR; ++r)
                             av[r] = (OPER_SMEM || r0 + r < nb) ? arow[r0 + r] : mk<R2>(0.0, 0.0);
 #pragma unroll
-                        for (int c = 0; c < kTC; ++c) bv[c] = Y[(size_t)b * P + c0 + c];
+                        for (int c = 0; c < kTC; ++c) bv[c] = Ym[(size_t)b * P + c0 + c];
 #pragma unroll
                         for (int r = 0; r < kTR; ++r)
 #pragma unroll
                             for (int c = 0; c < kTC; ++c) cfma(acc[r][c], av[r], bv[c]);
                     }
                 }
-                // ---- delta band: list the (s', s'') tiles that can hold an allowed pair
+                // ---- delta band: list the (mode, tile) pairs that can hold an allowed triplet
                 bool band = false;
-                if (active) {
+                const R w_1 = active ? (R)d.omega[(size_t)q * nb + s0 + m1] : (R)0;
+                if (active && w_1 > (R)0) {
                     R wlo = (R)1e30, whi = (R)-1e30, xlo = (R)1e30, xhi = (R)-1e30;
 #pragma unroll
                     for (int r = 0; r < kTR; ++r) { wlo = fmin(wlo, wp[r0 + r]); whi = fmax(whi, wp[r0 + r]); }
 #pragma unroll
                     for (int c = 0; c < kTC; ++c) { xlo = fmin(xlo, wpp[c0 + c]); xhi = fmax(xhi, wpp[c0 + c]); }
-                    // d+ = w + w' - w'' in [w + wlo - xhi, w + whi - xlo]
-                    // d- = w - w' - w'' in [w - whi - xhi, w - wlo - xlo]
+                    // w + w' - w'' in [w + wlo - xhi, w + whi - xlo]
+                    // w - w' - w'' in [w - whi - xhi, w - wlo - xlo]
+                    // w - w' + w'' in [w - whi + xlo, w - wlo + xhi] (orbits)
                     // (widened by 1e-4 of the cut so that rounding here never drops a
                     // tile that the exact per-element test below would reach)
-                    const R cb = cut * (R)1.0001;
-                    band = ((w + wlo - xhi < cb) && (w + whi - xlo > -cb)) ||
-                           ((w - whi - xhi < cb) && (w - wlo - xlo > -cb));
+                    const R cb = cut * (R)1.0001 + (kPair ? (R)1e-5 : (R)0);
+                    band = ((w_1 + wlo - xhi < cb) && (w_1 + whi - xlo > -cb)) ||
+                           ((w_1 - whi - xhi < cb) && (w_1 - wlo - xlo > -cb)) ||
+                           (ORBIT && (w_1 - whi + xlo < cb) && (w_1 - wlo + xhi > -cb));
                 }
                 const unsigned bal = __ballot_sync(0xffffffffu, band);
                 if (lane == 0) warp_cnt[warp] = __popc(bal);
                 __syncthreads();
                 if (active) {
+                    R2 *Ym = Y + m1 * ysz;
 #pragma unroll
                     for (int r = 0; r < kTR; ++r)
 #pragma unroll
                         for (int c = 0; c < kTC; ++c)
-                            Y[(size_t)(c0 + c) * Q + r0 + r] = acc[r][c];   // T'^T(c, s')
+                            Ym[(size_t)(c0 + c) * Q + r0 + r] = acc[r][c];   // T'^T(c, s')
                 }
                 if (band) {
                     int off = 0;
                     for (int w8 = 0; w8 < warp; ++w8) off += warp_cnt[w8];
-                    off += __popc(bal & ((1u << lane) - 1u));
-                    tiles[off] = (short)tid;
+                    tiles[off + __popc(bal & ((1u << lane) - 1u))] = tid;
                 }
                 if (tid == 0) {
-                    int t = 0;
-                    for (int w8 = 0; w8 < nwarps; ++w8) t += warp_cnt[w8];
-                    n_act_sm = t;
+                    int n = 0;
+                    for (int w8 = 0; w8 < nwarps; ++w8) n += warp_cnt[w8];
+                    n_act_sm = n;
                 }
                 __syncthreads();
 
-                // ---- GEMM2 + epilogue on the band tiles, K split over S lanes
+                // ---- GEMM2 + epilogue on the listed tiles, K split over S lanes
                 const int n_act = n_act_sm;
                 int S = 1;
-                while (S < 8 && n_act * S * 2 <= kThreads) S <<= 1;
-                const int per_pass = kThreads / S;
+                while (S < 8 && n_act * S * 2 <= nthr) S <<= 1;
+                const int per_pass = nthr / S;
                 const int ks = tid & (S - 1);
                 const int kc = (nb + S - 1) / S;
                 const int kb0 = ks * kc, kb1 = min(nb, kb0 + kc);
-                R part = (R)0;
                 for (int base = 0; base < n_act; base += per_pass) {
                     // every lane runs every pass (the shuffles below need the
                     // whole warp); lanes past the list do no work
                     const int ti2 = base + tid / S;
-                    const bool valid = ti2 < n_act;
-                    const int tt = valid ? (int)tiles[ti2] : 0;
+                    const bool valid = tid / S < per_pass && ti2 < n_act;
+                    const int code = valid ? tiles[ti2] : 0;
+                    const int m = code / n_tiles, tt = code - m * n_tiles;
+                    const R2 *Ym = Y + m * ysz;
                     r0 = (tt / tcols) * kTR;
                     c0 = (tt % tcols) * kTC;
 #pragma unroll
@@ -388,7 +471,7 @@ lw_main_kernel(LwParams p, LwDev d, const R *__restrict__ fc3,
                     for (int c = kb0; c < ke; ++c) {
                         R2 av[kTR], bv[kTC];
 #pragma unroll
-                        for (int r = 0; r < kTR; ++r) av[r] = Y[(size_t)c * Q + r0 + r];
+                        for (int r = 0; r < kTR; ++r) av[r] = Ym[(size_t)c * Q + r0 + r];
                         if (OPER_SMEM) {
 #pragma unroll
                             for (int k = 0; k < kTC; ++k) bv[k] = EppT[(size_t)c * P + c0 + k];
@@ -416,86 +499,148 @@ lw_main_kernel(LwParams p, LwDev d, const R *__restrict__ fc3,
                                 acc[r][c].y += __shfl_xor_sync(0xffffffffu, acc[r][c].y, o);
                             }
                     }
-                    if (valid && ks == 0) {
+                    if (!valid || ks != 0) continue;
+                    const double w_s = d.omega[(size_t)q * nb + s0 + m];
+                    const R w = (R)w_s;
+                    F2 w0p, n0p;                              // FP32 pairs of w and n of (q, s)
+                    R n0 = (R)0;
+                    if constexpr (kPair) {
+                        const float4 u = d.wn32[(size_t)q * nb + s0 + m];
+                        w0p = F2{u.x, u.y};
+                        n0p = F2{u.z, u.w};
+                        n0 = u.z;
+                    } else if (ORBIT) {
+                        n0 = d.occ[(size_t)q * nb + s0 + m];
+                    }
+                    R part = (R)0, colsum[kTC];
 #pragma unroll
-                        for (int r = 0; r < kTR; ++r) {
-                            const R w1 = wp[r0 + r], n1 = np_[r0 + r];
-                            if (w1 <= (R)0) continue;
+                    for (int c = 0; c < kTC; ++c) colsum[c] = (R)0;
+#pragma unroll
+                    for (int r = 0; r < kTR; ++r) {
+                        const R w1 = wp[r0 + r], n1 = np_[r0 + r];
+                        R rowsum = (R)0;
+                        if (w1 > (R)0) {
                             const R iw1 = (R)1 / w1;
                             F2 w1p, n1p, sp, sm;
                             if constexpr (kPair) {
                                 w1p = F2{wp[r0 + r], wpl[r0 + r]};
                                 n1p = F2{np_[r0 + r], npl[r0 + r]};
-                                sp = f2_add(wsp, w1p);
-                                sm = f2_add(wsp, f2_neg(w1p));
+                                sp = f2_add(w0p, w1p);
+                                sm = f2_add(w0p, f2_neg(w1p));
                             }
 #pragma unroll
                             for (int c = 0; c < kTC; ++c) {
                                 const R w2 = wpp[c0 + c];
                                 if (w2 <= (R)0) continue;
                                 const R n2 = npp[c0 + c];
-                                R dp, dm, dn;
+                                F2 w2p, n2p;
                                 if constexpr (kPair) {
-                                    const F2 w2p{wpp[c0 + c], wppl[c0 + c]};
+                                    w2p = F2{wpp[c0 + c], wppl[c0 + c]};
+                                    n2p = F2{npp[c0 + c], nppl[c0 + c]};
+                                }
+                                R dp, dm;
+                                if constexpr (kPair) {
                                     dp = f2_diff(sp, w2p);
                                     dm = f2_diff(sm, w2p);
-                                    dn = f2_diff(n1p, F2{npp[c0 + c], nppl[c0 + c]});
                                 } else {
                                     dp = w + w1 - w2;
                                     dm = w - w1 - w2;
-                                    dn = n1 - n2;
                                 }
-                                R gpv = (R)0, gmv = (R)0;
-                                bool hit = false;
-                                if (fabs(dp) < cut) { gpv = dn * delta_shape(dp, p.shape, sig2inv); hit = true; }
-                                if (fabs(dm) < cut) {
-                                    gmv = (R)0.5 * ((R)1 + n1 + n2) * delta_shape(dm, p.shape, sig2inv);
-                                    hit = true;
-                                }
-                                const R g = gpv + gmv;
-                                if (hit) {
-                                    ++allowed;
-                                    const R2 f = acc[r][c];
-                                    const R f2 = f.x * f.x + f.y * f.y;
-                                    part += f2 * g * iw1 / w2;
+                                const bool hp = fabs(dp) < cut, hm = fabs(dm) < cut;
+                                const R2 f = acc[r][c];
+                                const R f2 = f.x * f.x + f.y * f.y;
+                                R dn;                                        // n' - n''
+                                if constexpr (kPair) dn = f2_diff(n1p, n2p);
+                                else dn = n1 - n2;
+                                if constexpr (ORBIT) {
+                                    // positions 1 = (q, s), 2 = (q', s'), 3 = (-q'', s'')
+                                    R d2, dn02, dn01;
+                                    if constexpr (kPair) {
+                                        d2 = f2_diff(sm, f2_neg(w2p));
+                                        dn02 = f2_diff(n0p, n2p);
+                                        dn01 = f2_diff(n0p, n1p);
+                                    } else {
+                                        d2 = w - w1 + w2;
+                                        dn02 = n0 - n2;
+                                        dn01 = n0 - n1;
+                                    }
+                                    const bool h2 = fabs(d2) < cut;
+                                    const bool near_edge = fabs(fabs(dp) - cut) < edge || fabs(fabs(dm) - cut) < edge ||
+                                                           fabs(fabs(d2) - cut) < edge;
+                                    if (near_edge) {
+                                        if constexpr (kPair) hits += window_hits6({w0p, w1p, w2p}, cut);
+                                        else hits += window_hits6({w, w1, w2}, cut);
+                                    } else {
+                                        hits += 2u * ((unsigned)(hp || hm) + (unsigned)(hp || h2) + (unsigned)(hm || h2));
+                                    }
+                                    if (hp || hm || h2) {
+                                        const R e3 = hp ? delta_shape(dp, p.shape, sig2inv) : (R)0;
+                                        const R e1 = hm ? delta_shape(dm, p.shape, sig2inv) : (R)0;
+                                        const R e2 = h2 ? delta_shape(d2, p.shape, sig2inv) : (R)0;
+                                        const R iw2 = (R)1 / w2;
+                                        part += f2 * (dn * (e3 - e2) + ((R)1 + n1 + n2) * e1) * iw1 * iw2;
+                                        rowsum += f2 * (dn02 * (e3 - e1) + ((R)1 + n0 + n2) * e2) * iw2;
+                                        colsum[c] += f2 * (dn01 * (e2 - e1) + ((R)1 + n0 + n1) * e3) * iw1;
+                                    }
+                                } else if (hp || hm) {
+                                    const R gpv = hp ? dn * delta_shape(dp, p.shape, sig2inv) : (R)0;
+                                    const R gmv = hm ? (R)0.5 * ((R)1 + n1 + n2) * delta_shape(dm, p.shape, sig2inv) : (R)0;
+                                    ++hits;
+                                    part += f2 * (gpv + gmv) * iw1 / w2;
                                     if constexpr (!kPair) {
                                         if (p.bte) {
                                             // rates into the BTE operator planes (FP64 atomics;
                                             // every (q, s) row is owned by this item)
                                             const double sc = p.bte_pref / (w_s * w_s);
                                             const size_t N = (size_t)p.nq * nb;
-                                            const size_t row = ((size_t)q * nb + s) * N;
+                                            const size_t row = ((size_t)q * nb + s0 + m) * N;
                                             atomicAdd(d.g1_a + row + (size_t)qp * nb + r0 + r, sc * f2 * gpv / w2);
-                                            atomicAdd(d.g1_am + row + (size_t)d.qneg[qp] * nb + r0 + r,
-                                                      sc * f2 * gmv / w2);
-                                            atomicAdd(d.g1_b + row + (size_t)qpp * nb + c0 + c, sc * f2 * g / w1);
+                                            atomicAdd(d.g1_am + row + (size_t)d.qneg[qp] * nb + r0 + r, sc * f2 * gmv / w2);
+                                            atomicAdd(d.g1_b + row + (size_t)qpp * nb + c0 + c, sc * f2 * (gpv + gmv) / w1);
                                         }
                                     }
                                 }
                             }
                         }
+                        if (ORBIT) prow[6 * ti2 + r] = (double)(rowsum / w);     // / w of position 1
                     }
+                    psum[ti2] = (double)part;
+                    if (ORBIT)
+#pragma unroll
+                        for (int c = 0; c < kTC; ++c) pcol[3 * ti2 + c] = (double)(colsum[c] / w);
                 }
-                // block sum of this mode, added to red[s] in a fixed order
-                double pd = (double)part;
-                for (int o = 16; o > 0; o >>= 1) pd += __shfl_xor_sync(0xffffffffu, pd, o);
-                if (lane == 0) wsum[warp] = pd;
                 __syncthreads();
-                if (tid == 0) {
-                    double t = 0.0;
-                    for (int w8 = 0; w8 < nwarps; ++w8) t += wsum[w8];
-                    red[s] += t;
+                // ---- the tiles' sums per mode, in the order of the list: position 1 by the
+                // mode, 2 by the row, 3 by the column
+                for (int x = tid; x < (ORBIT ? ns + 2 * nb : ns); x += nthr) {
+                    double v = 0.0;
+                    if (x < ns) {
+                        for (int y = 0; y < n_act; ++y)
+                            if (tiles[y] / n_tiles == x) v += psum[y];
+                        red[s0 + x] += v;
+                    } else {
+                        const bool row = x < ns + nb;
+                        const int e = x - ns - (row ? 0 : nb);
+                        const int ta = row ? e / kTR : e / kTC, tb = row ? e % kTR : e % kTC;
+                        for (int y = 0; y < n_act; ++y) {
+                            const int tt = tiles[y] % n_tiles;
+                            if ((row ? tt / tcols : tt % tcols) == ta) v += row ? prow[6 * y + tb] : pcol[3 * y + tb];
+                        }
+                        red[(row ? nb : 2 * nb) + e] += v;
+                    }
                 }
             }
         }
         __syncthreads();
-        for (int s = tid; s < nb; s += kThreads)
-            d.partial[((size_t)qi * p.n_chunks + chunk) * nb + s] = red[s];
-        // an item of q stands for -q as well when it takes q's linewidths
-        allowed += (unsigned long long)(qm.y - 1) * (allowed - allowed0);
+        if (ORBIT) {
+            for (int x = tid; x < 3 * nb; x += nthr) t.out3[(size_t)item_all * 3 * nb + x] = red[x];
+        } else {
+            for (int s = sbeg + tid; s < send; s += nthr) d.partial[(size_t)item * nb + s] = red[s];
+        }
+        allowed += (unsigned long long)mult * hits;
         __syncthreads();
     }
-    // delta-allowed triplet count
+    // delta-allowed triplet count (orbits: six times it)
     for (int o = 16; o > 0; o >>= 1) allowed += __shfl_xor_sync(0xffffffffu, allowed, o);
     if (lane == 0 && allowed) atomicAdd(d.allowed, allowed);
 }
@@ -679,20 +824,6 @@ __global__ void phase_space_sum_kernel(size_t n, int n_chunks, const double *__r
     g[x] = scale * t;
 }
 
-template <typename R>
-size_t lw_smem_bytes(const LwParams &p, bool oper_smem) {
-    using R2 = typename C2<R>::T;
-    const int P = ((p.nb + kTR - 1) / kTR) * kTR;
-    size_t b = sizeof(R2) * (size_t)P * (P + 1);
-    if (oper_smem) b += 2 * sizeof(R2) * (size_t)P * P;
-    b += sizeof(R2) * (P + 2 * p.n_rep);
-    b += sizeof(R) * 8 * P;
-    b = (b + 15) & ~size_t(15);
-    b += sizeof(double) * (p.nb + kThreads / 32);
-    b += sizeof(short) * kThreads;
-    return b + 16;
-}
-
 }  // namespace
 
 cudaError_t launch_mode_prep(int n, const double *nu, double omega_min_w, double T, int classical,
@@ -721,36 +852,127 @@ cudaError_t launch_lw_prep(const LwParams &p, const LwDev &d, int fp32, cudaStre
     return cudaGetLastError();
 }
 
-cudaError_t launch_lw_main(const LwParams &p, const LwDev &d, int fp32, int sm_count,
+// Modes per pass and threads of a CTA: up to 256 threads, and two CTAs per SM in
+// shared memory where several modes run side by side.
+template <typename R>
+static void lw_shape(int nb, bool orbit, size_t smem_optin, int &sb, int &nthr) {
+    const int P = (nb + kTR - 1) / kTR * kTR, n_tiles = (P / kTR) * (P / kTC);
+    const size_t half = (smem_optin - 4096) / 2;
+    auto threads = [&](int m) { return (m * n_tiles + 31) / 32 * 32; };
+    sb = std::max(1, std::min(nb, 256 / n_tiles));
+    while (sb > 1 && lw_smem_bytes<R>(nb, sb, threads(sb), true, orbit) > half) --sb;
+    nthr = threads(sb);
+}
+// Blocks of modes per pair or q chunk: one, or as many as give every SM about
+// eight items on a coarse mesh (from the mesh, not from the q-points of a call).
+static int lw_mode_blocks(int nb, int sb, long long n_base, int sm_count) {
+    const long long want = 8LL * std::max(1, sm_count);
+    return (int)std::max(1LL, std::min<long long>((nb + sb - 1) / sb, (want + n_base - 1) / std::max(1LL, n_base)));
+}
+// Mode blocks of an orbit run (the caller's out3 holds [n_pairs][blocks][3][nb],
+// and [n_pairs][3][nb] after it when there are several).
+int lw_orbit_blocks(int nb, int n_pairs, int fp32, int sm_count, size_t smem_optin) {
+    int sb, nthr;
+    if (fp32) lw_shape<float>(nb, true, smem_optin, sb, nthr);
+    else lw_shape<double>(nb, true, smem_optin, sb, nthr);
+    return lw_mode_blocks(nb, sb, n_pairs, sm_count);
+}
+
+template <typename R, bool ORBIT>
+static cudaError_t run_lw_main(const LwParams &p, const LwDev &d, LwTerms t, int sm_count, size_t smem_optin,
+                               cudaStream_t st) {
+    using R2 = typename C2<R>::T;
+    int sb, nthr;
+    lw_shape<R>(p.nb, ORBIT, smem_optin, sb, nthr);
+    // the eigenvectors in shared memory where they fit
+    const bool oper = lw_smem_bytes<R>(p.nb, sb, nthr, true, ORBIT) <= smem_optin;
+    const size_t smem = lw_smem_bytes<R>(p.nb, sb, nthr, oper, ORBIT);
+    if (smem > smem_optin || nthr > kThreads) return cudaErrorInvalidValue;
+    auto k = oper ? lw_main_kernel<R, true, ORBIT> : lw_main_kernel<R, false, ORBIT>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    int per_sm = 1;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, nthr, smem);
+    if (e != cudaSuccess) return e;
+    const size_t nt = (size_t)std::max({t.n_slot[0], t.n_slot[1], t.n_slot[2]}) * 27 * p.nq;
+    if (nt)
+        lw_tables_kernel<R><<<counted((unsigned)std::min<size_t>((nt + 255) / 256, 16384)), 256, 0, st>>>(
+            p.nq, p.n_rep, t, d.blkinfo, static_cast<const R *>(d.fc3), static_cast<const R2 *>(d.chi));
+    const int n_batch = (p.nb + sb - 1) / sb;
+    t.n_sblk = ORBIT ? lw_mode_blocks(p.nb, sb, t.n_pairs, sm_count)
+                     : lw_mode_blocks(p.nb, sb, (long long)(p.nq / 2 + 1) * p.n_chunks, sm_count);
+    t.s_per = (n_batch + t.n_sblk - 1) / t.n_sblk * sb;
+    const long long n_items = (ORBIT ? t.n_pairs : (long long)p.nqc * p.n_chunks) * t.n_sblk;
+    if (n_items > 0x7fffffffLL - (1 << 20)) return cudaErrorInvalidValue;
+    const int grid = (int)std::max(1LL, std::min<long long>(n_items, (long long)sm_count * std::max(1, per_sm)));
+    ProfMark pm(p.prof, KALD_PROF_LW_MAIN, st);
+    k<<<counted(grid), nthr, smem, st>>>(p, d, t, sb, static_cast<const R *>(d.fc3), static_cast<const R2 *>(d.eps_work),
+                                         static_cast<const R2 *>(d.chi));
+    pm.end();
+    if (ORBIT && t.n_sblk > 1) {
+        const size_t n = (size_t)t.n_pairs * 3 * p.nb;
+        lw_block_sums_kernel<<<counted((unsigned)std::min<size_t>((n + 255) / 256, 4096)), 256, 0, st>>>(
+            n, 3 * p.nb, t.n_sblk, t.out3, t.out3 + n * t.n_sblk);
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_lw_main(const LwParams &p, const LwDev &d, const LwTerms &t, int fp32, int sm_count,
                            size_t smem_optin, cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(d.queue, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(d.allowed, 0, sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
-    const int n_items = p.nqc * p.n_chunks;
-    const int grid = std::max(1, std::min(n_items, sm_count));
-    if (fp32) {
-        const size_t smem = lw_smem_bytes<float>(p, true);
-        if (smem > smem_optin) return cudaErrorInvalidValue;
-        auto k = lw_main_kernel<float, true>;
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        ProfMark pm(p.prof, KALD_PROF_LW_MAIN, st);
-        k<<<counted(grid), kThreads, smem, st>>>(p, d, (const float *)d.fc3, (const float2 *)d.eps_work,
-                                        (const float2 *)d.chi);
-        pm.end();
-    } else {
-        const size_t smem = lw_smem_bytes<double>(p, false);
-        if (smem > smem_optin) return cudaErrorInvalidValue;
-        auto k = lw_main_kernel<double, false>;
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        ProfMark pm(p.prof, KALD_PROF_LW_MAIN, st);
-        k<<<counted(grid), kThreads, smem, st>>>(p, d, (const double *)d.fc3, (const double2 *)d.eps_work,
-                                        (const double2 *)d.chi);
-        pm.end();
+    if (t.n_pairs)
+        return fp32 ? run_lw_main<float, true>(p, d, t, sm_count, smem_optin, st)
+                    : run_lw_main<double, true>(p, d, t, sm_count, smem_optin, st);
+    return fp32 ? run_lw_main<float, false>(p, d, t, sm_count, smem_optin, st)
+                : run_lw_main<double, false>(p, d, t, sm_count, smem_optin, st);
+}
+
+// The fc3 blocks by group (j, k), class and home atom i: one table slot per
+// (group, class < 3, i), one term per slot and per block of class 3 (every block
+// without tables).
+void plan_lw_terms(const HostSystem &h, bool tables, LwTermsHost &o) {
+    const int na = h.n_atoms, ng = (int)h.pair3_j.size();
+    o.group.assign((size_t)na * na, -1);
+    o.term_start.assign(1, 0);
+    o.term.clear();
+    std::vector<std::vector<int>> slots[3];               // block lists, class by class
+    for (int g = 0; g < ng; ++g) {
+        o.group[(size_t)h.pair3_j[g] * na + h.pair3_k[g]] = g;
+        std::vector<std::array<int, 3>> key;              // (class, i, block), the blocks of a slot in order
+        for (int b = h.pair3_start[g]; b < h.pair3_start[g + 1]; ++b) {
+            const int *rj = &h.rep_int[3 * (size_t)h.fc3_rj[b]], *rk = &h.rep_int[3 * (size_t)h.fc3_rk[b]];
+            const bool zj = !rj[0] && !rj[1] && !rj[2], zk = !rk[0] && !rk[1] && !rk[2];
+            const int cls = !tables ? 3 : zk ? 0 : zj ? 1 : h.fc3_rj[b] == h.fc3_rk[b] ? 2 : 3;
+            key.push_back({cls, h.fc3_i[b], b});
+        }
+        std::sort(key.begin(), key.end());
+        for (size_t x = 0; x < key.size(); ++x) {
+            const int cls = key[x][0], i = key[x][1], b = key[x][2];
+            if (cls == 3) {
+                o.term.push_back(make_int4(i, 3, b, 0));
+            } else {
+                if (x == 0 || key[x - 1][0] != cls || key[x - 1][1] != i) {
+                    o.term.push_back(make_int4(i, cls, (int)slots[cls].size(), 0));
+                    slots[cls].emplace_back();
+                }
+                slots[cls].back().push_back(b);
+            }
+        }
+        o.term_start.push_back((int)o.term.size());
     }
-    return cudaGetLastError();
+    o.slot_start.assign(1, 0);
+    o.slot_blk.clear();
+    for (int c = 0; c < 3; ++c) {
+        o.n_slot[c] = (int)slots[c].size();
+        o.slot0[c] = (int)o.slot_start.size() - 1;
+        for (const auto &v : slots[c]) {
+            o.slot_blk.insert(o.slot_blk.end(), v.begin(), v.end());
+            o.slot_start.push_back((int)o.slot_blk.size());
+        }
+    }
 }
 
 // q' chunks of the phase-space sum: about eight CTAs per SM.

@@ -239,3 +239,31 @@ def test_hermitian_eigensolver_spectra(k, n, kind):
     np.testing.assert_allclose(lam, np.linalg.eigvalsh(D), rtol=0, atol=1e-13 * scale)
     np.testing.assert_allclose(E.conj().T @ E, np.eye(3 * n), rtol=0, atol=1e-13)
     assert np.abs(D @ E - E * lam).max() <= 1e-13 * scale
+
+
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-10), ("fp32", 1e-5)])
+@pytest.mark.parametrize("cell,mesh,extra,cap", [((1, 1, 1), (3, 4, 2), 0, 0), ((1, 1, 1), (2, 2, 1), 80, 0),
+                                                 ((2, 1, 1), (3, 3, 1), 0, 0), ((3, 1, 1), (2, 1, 2), 0, 1 << 23),
+                                                 ((5, 1, 1), (2, 1, 1), 60, 0)])
+def test_cuda_core_kernel_orbits_and_tables(k, cell, mesh, extra, cap, precision, tol):
+    """Four to 20 atoms (12 to 60 branches): one projection per orbit of momentum
+    triples for a symmetric Phi3, every pair for one with random blocks (their own
+    phase class), no tables under a workspace cap; the same sums and the same
+    delta-allowed count with no symmetry at all."""
+    from oracle import anharmonic as an
+    kk, ctx = k
+    s = ki.fcc_supercell_system(cell, seed=7)
+    if extra:
+        s = ki.random_fc3_system(s, extra, seed=9)
+    nu, eig = ph.phonons(s, mesh)
+    g_o = an.linewidths(s, mesh, nu, eig, 300.0, 0.1, 3.0)
+    count = {}
+    ctx.set_workspace_limit(cap)
+    try:
+        for sym in ("all", "inversion", "none"):
+            opt = kk.Options(temperature_K=300.0, sigma_thz=0.1, precision=precision, symmetry=sym)
+            g, count[sym] = kk.kald_linewidths(ctx, s, mesh, nu, eig, opt)
+            assert _rel(g.reshape(g_o.shape), g_o) < tol
+    finally:
+        ctx.set_workspace_limit(0)
+    assert count["all"] == count["inversion"] == count["none"]
