@@ -1366,19 +1366,20 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
             }
         }
         const int tcx_b = tcx ? tcx_batch_max(nb, nq, ctx->sm_count) : 0;   // scratch for the tuner's largest batch
-        // tensor-core path over the whole mesh with Phi3 symmetric under
+        // cells of three or more atoms over the whole mesh with Phi3 symmetric under
         // permutations: one projection per orbit of momentum triples
-        TcxSymHost symh;
-        bool use_sym = false;
-        if (tcx && !listed && reuse && opt->symmetry == KALD_SYM_ALL && nq > 1) {
+        int orb_pairs = 0;
+        std::vector<int> orb_rows;
+        if (!small && !listed && reuse && opt->symmetry == KALD_SYM_ALL && nq > 1) {
             if (h.fc3_perm_symmetric < 0) h.fc3_perm_symmetric = fc3_symmetric_all(&sys[x]) ? 1 : 0;
-            if (h.fc3_perm_symmetric) {
-                std::vector<int> self_inv(nqc);
-                for (int i = 0; i < nqc; ++i) self_inv[i] = qsel[i].y == 1 ? 1 : 0;
-                plan_tcx_sym(mesh, qf, qrow, self_inv, symh);       // qrow[q]: class row (whole mesh)
-                use_sym = !symh.pairs.empty();
+            if (h.fc3_perm_symmetric) orb_pairs = std::max(0, orbit_pairs(mesh));
+            if (orb_pairs) {
+                orb_rows.resize(nqc);
+                for (int i = 0; i < nqc; ++i) orb_rows[i] = qsel[i].x;
             }
         }
+        const bool use_sym = tcx && orb_pairs;
+        const int cc_pairs = tcx ? 0 : orb_pairs;
         // tensor-core path: the fc3 blocks in (j, k) group order, the groups
         // split over the gather CTAs
         std::vector<int2> tc_gjk;
@@ -1395,7 +1396,7 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         std::vector<int> y_atoms, y_gi;
         std::vector<int2> y_rep;
         const int y_n_at = nb / 3;
-        if (tcx && nb % 3 == 0) {
+        if (tcx && nb % 3 == 0 && tcx_y_wanted(n3, h.pair3_j.size())) {
             const int n_groups = (int)h.pair3_j.size();
             y_blk.resize(27 * std::max<size_t>(n3, 1), 0.0);
             y_atoms.resize(3 * std::max<size_t>(n3, 1), 0);
@@ -1423,7 +1424,6 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         const bool cc = !small && !tcx;
         LwTermsHost lt;
         size_t lw_tab[3] = {0, 0, 0};
-        int cc_pairs = 0;
         if (cc) {
             plan_lw_terms(h, true, lt);
             size_t all = 0;
@@ -1435,19 +1435,12 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
                 plan_lw_terms(h, false, lt);
                 lw_tab[0] = lw_tab[1] = lw_tab[2] = 0;
             }
-            if (!listed && reuse && opt->symmetry == KALD_SYM_ALL && nq > 1) {
-                if (h.fc3_perm_symmetric < 0) h.fc3_perm_symmetric = fc3_symmetric_all(&sys[x]) ? 1 : 0;
-                if (h.fc3_perm_symmetric) cc_pairs = std::max(0, orbit_pairs(mesh));
-            }
         }
-        std::vector<int> orb_rows;
         size_t cc_out3 = 0, cc_sums = 0;         // position sums of the mode blocks, and where their totals start
         if (cc_pairs) {
             const int blocks = lw_orbit_blocks(nb, cc_pairs, f32w, ctx->sm_count, ctx->smem_optin);
             cc_sums = blocks > 1 ? 3 * (size_t)cc_pairs * nb * blocks : 0;
             cc_out3 = 3 * (size_t)cc_pairs * nb * (blocks > 1 ? blocks + 1 : 1);
-            orb_rows.resize(nqc);
-            for (int i = 0; i < nqc; ++i) orb_rows[i] = qsel[i].x;
             p.n_chunks = 1;
         }
         if (small) p.n_rep = 0;                  // the register kernel takes its phases from roots of unity
@@ -1469,9 +1462,7 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         if (tcx)
             need += ws_round(tcx_scratch_bytes(nb, nq, tcx_b)) + ws_round(16) + bytes_of(tc_gjk) +
                     bytes_of(tc_part_start) + bytes_of(tc_glist) + bytes_of(h.pair3_start);
-        if (use_sym)
-            need += ws_round(tcx_sym_bytes(nb, tcx_b, (int)symh.pairs.size())) + bytes_of(symh.pairs) +
-                    bytes_of(symh.orbit) + bytes_of(symh.cls_start) + bytes_of(symh.ent) + bytes_of(symh.fac);
+        if (use_sym) need += ws_round(tcx_sym_bytes(nb, tcx_b, orb_pairs));
         if (!y_blk.empty())
             need += scaled_bytes(y_blk, y_atoms, h, 27, 28, 1) + bytes_of(y_gi) + bytes_of(y_rep);
         if (small)
@@ -1480,8 +1471,7 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         if (cc)
             need += bytes_of(lt.group) + bytes_of(lt.term_start) + bytes_of(lt.term) + bytes_of(lt.slot_start) +
                     bytes_of(lt.slot_blk) + ws_round(lw_tab[0]) + ws_round(lw_tab[1]) + ws_round(lw_tab[2]);
-        if (cc_pairs)
-            need += bytes_of(orb_rows) + ws_round(orbit_bytes(mesh, nqc)) + ws_round(sizeof(double) * cc_out3);
+        if (orb_pairs) need += bytes_of(orb_rows) + ws_round(orbit_bytes(mesh, nqc)) + ws_round(sizeof(double) * cc_out3);
         if ((st = ws_reserve(ctx, need))) return st;
         LwDev d;
         d.blkinfo = upload(ctx, binfo);
@@ -1511,18 +1501,7 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         double *g_d = d_g ? gamma + off_nb : static_cast<double *>(ws_take(ctx, sizeof(double) * nqr * nb));
         void *tc_scr = tcx ? ws_take(ctx, tcx_scratch_bytes(nb, nq, tcx_b)) : nullptr;
         int *tc_err = tcx ? static_cast<int *>(ws_take(ctx, 16)) : nullptr;
-        TcxSym tsym;
-        void *sym_scr = nullptr;
-        if (use_sym) {
-            tsym.n_pairs = (int)symh.pairs.size();
-            tsym.n_cls = nqc;
-            tsym.plist = upload(ctx, symh.pairs);
-            tsym.porb = upload(ctx, symh.orbit);
-            tsym.cls_start = upload(ctx, symh.cls_start);
-            tsym.ent = upload(ctx, symh.ent);
-            tsym.fac = upload(ctx, symh.fac);
-            sym_scr = ws_take(ctx, tcx_sym_bytes(nb, tcx_b, tsym.n_pairs));
-        }
+        void *sym_scr = use_sym ? ws_take(ctx, tcx_sym_bytes(nb, tcx_b, orb_pairs)) : nullptr;
         TcxGroups tg;
         if (tcx) {
             tg.n_groups = (int)h.pair3_j.size();
@@ -1574,21 +1553,23 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
                 terms.slot0[c] = lt.slot0[c];
                 terms.tab[c] = ws_take(ctx, lw_tab[c]);
             }
-            if (cc_pairs) {
-                const int *rows_d = upload(ctx, orb_rows);
-                void *work = ws_take(ctx, orbit_bytes(mesh, nqc));
-                terms.out3 = static_cast<double *>(ws_take(ctx, sizeof(double) * cc_out3));
-                e = launch_orbit_plan(mesh, nqc, rows_d, d.qrow, work, orb, s);     // whole mesh: qrow[q] is q's row
-                terms.n_pairs = orb.n_pairs;
-                terms.pairs = orb.pairs;
-                terms.orbit = orb.orbit;
-            }
+            if (cc_pairs) terms.out3 = static_cast<double *>(ws_take(ctx, sizeof(double) * cc_out3));
+        }
+        if (orb_pairs) {
+            const int *rows_d = upload(ctx, orb_rows);
+            void *work = ws_take(ctx, orbit_bytes(mesh, nqc));
+            e = launch_orbit_plan(mesh, nqc, rows_d, d.qrow, work, orb, s);     // whole mesh: qrow[q] is q's row
+        }
+        if (cc_pairs) {
+            terms.n_pairs = orb.n_pairs;
+            terms.pairs = orb.pairs;
+            terms.orbit = orb.orbit;
         }
         if (e == cudaSuccess) e = launch_lw_prep(p, d, f32w, s);
         if (e == cudaSuccess)
             e = small ? launch_lw_small(p, d, sn, f32w, s)
                 : tcx ? launch_lw_tensor(p, d, tg, tc_scr, tcx_b, ctx->sm_count, tc_err, s,
-                                         use_sym ? &tsym : nullptr, sym_scr)
+                                         use_sym ? &orb : nullptr, sym_scr)
                       : launch_lw_main(p, d, terms, f32w, ctx->sm_count, ctx->smem_optin, s);
         if (e == cudaSuccess && cc_pairs) e = launch_orbit_class_sums(orb, nb, terms.out3 + cc_sums, d.partial, s);
         if (e == cudaSuccess) e = launch_lw_finish(p, d, opt->degen_tol_thz, g_d, s);

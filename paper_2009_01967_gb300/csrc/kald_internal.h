@@ -417,28 +417,7 @@ struct TcxGroups {
     const int4 *blkinfo = nullptr;    // [n_fc3] (i, rep(Rj), rep(Rk), 0), group order
     const float *fc3 = nullptr;       // [n_fc3][28] Phi3 / sqrt(mi mj mk), FP32, padded
 };
-// One projection per orbit of momentum triples (q1, q2, q3 = -(q1 + q2))
-// under permutations and inversion (Phi3 symmetric under permutations of its
-// indices, whole-mesh call): the pairs (q1, q2) of the canonical triples (the
-// lexicographically smallest ordered triple of each orbit), their orbit sizes,
-// and per inversion class {q, -q} the CSR of (3 pair + position, factor)
-// entries whose position holds a member of the class; factor = orbit size / 12
-// times 2 for a class with -q = q.
-struct TcxSymHost {
-    std::vector<int2> pairs;
-    std::vector<int> orbit;
-    std::vector<int> cls_start, ent;
-    std::vector<double> fac;
-};
-// qcls[q] = class row of q (rows 0 .. n_cls - 1), self_inv[row] = 1 where -q = q.
-void plan_tcx_sym(const int32_t mesh[3], const std::vector<int> &qf, const std::vector<int> &qcls,
-                  const std::vector<int> &self_inv, TcxSymHost &out);
-struct TcxSym {
-    int n_pairs = 0, n_cls = 0;
-    const int2 *plist = nullptr;
-    const int *porb = nullptr, *cls_start = nullptr, *ent = nullptr;
-    const double *fac = nullptr;
-};
+bool tcx_y_wanted(size_t n_fc3, size_t n_groups);   // the phase sum on tensor cores is considered
 size_t tcx_sym_bytes(int nb, int batch, int n_pairs);
 bool tcx_supported(int nb);           // 65 <= nb <= 96 (one tile width, N = K = 192)
 int tcx_half(int nb);
@@ -448,7 +427,7 @@ int tcx_parts(int n_groups);
 void plan_tcx_parts(const HostSystem &h, int n_parts, std::vector<int> &part_start, std::vector<int> &glist);
 size_t tcx_scratch_bytes(int nb, int nq, int batch);
 cudaError_t launch_lw_tensor(const LwParams &p, const LwDev &d, const TcxGroups &g, void *scratch, int batch,
-                             int sms, int *err, cudaStream_t st, const TcxSym *sym = nullptr,
+                             int sms, int *err, cudaStream_t st, const OrbitPlan *sym = nullptr,
                              void *sym_scratch = nullptr);
 
 // ifc.cu: finite-difference force constants of a pair potential.  Neighbours

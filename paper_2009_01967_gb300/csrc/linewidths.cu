@@ -647,43 +647,48 @@ lw_main_kernel(LwParams p, LwDev d, LwTerms t, int SB, const R *__restrict__ fc3
 
 // gamma = pref / w * sum over chunks; then average over degenerate sets.
 // Row j of gamma is q-point qout[j], j < n_out; its sums are in row qrow[j]
-// of partial (those of q itself, or of -q).
-__global__ void lw_finish_kernel(int n_out, int nb, int n_chunks, const double *__restrict__ partial,
-                                 const int *__restrict__ qout, const int *__restrict__ qrow,
-                                 const double *__restrict__ omega, const double *__restrict__ nu, double pref,
-                                 double degen_tol, double *__restrict__ gamma) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n_out) return;
-    const int q = qout[j];
-    double *g = gamma + (size_t)j * nb;
+// of partial (those of q itself, or of -q).  One CTA per row, one thread per
+// mode: the sums and the rank of each mode, then the thread of each set's first
+// mode averages it in ascending order (a thread per row sorting its modes took
+// 0.11 ms for 64 q-points of 96 modes).
+__global__ void __launch_bounds__(kMaxNbSmall)
+lw_finish_kernel(int nb, int n_chunks, const double *__restrict__ partial, const int *__restrict__ qout,
+                 const int *__restrict__ qrow, const double *__restrict__ omega, const double *__restrict__ nu, double pref,
+                 double degen_tol, double *__restrict__ gamma) {
+    __shared__ double v[kMaxNbSmall], gs[kMaxNbSmall];
+    __shared__ int order[kMaxNbSmall];
+    const int j = blockIdx.x, s = threadIdx.x, q = qout[j];
     const size_t row = (size_t)qrow[j];
-    for (int s = 0; s < nb; ++s) {
+    if (s < nb) {
         double t = 0.0;
+#pragma unroll 4
         for (int c = 0; c < n_chunks; ++c) t += partial[(row * n_chunks + c) * nb + s];
         const double w = omega[(size_t)q * nb + s];
-        g[s] = (w > 0.0) ? pref * t / w : 0.0;
+        gs[s] = (w > 0.0) ? pref * t / w : 0.0;
+        v[s] = nu[(size_t)q * nb + s];
     }
-    // degenerate sets: chains of |d nu| < tol in ascending order of nu
-    int order[kMaxNbSmall];
-    const double *v = nu + (size_t)q * nb;
-    for (int s = 0; s < nb; ++s) order[s] = s;
-    for (int a = 1; a < nb; ++a) {             // insertion sort (stable)
-        const int x = order[a];
-        int b = a - 1;
-        while (b >= 0 && v[order[b]] > v[x]) { order[b + 1] = order[b]; --b; }
-        order[b + 1] = x;
-    }
-    int start = 0;
-    for (int a = 1; a <= nb; ++a) {
-        if (a == nb || v[order[a]] - v[order[a - 1]] >= degen_tol) {
-            if (a - start > 1) {
-                double t = 0.0;
-                for (int b = start; b < a; ++b) t += g[order[b]];
-                t /= (double)(a - start);
-                for (int b = start; b < a; ++b) g[order[b]] = t;
-            }
-            start = a;
+    __syncthreads();
+    if (s < nb) {                                  // ascending, ties by index, NaN last
+        const double x = v[s];
+        int r = 0;
+        for (int t = 0; t < nb; ++t) {
+            const double y = v[t];
+            const bool lt = y < x || (x != x && y == y);
+            const bool gt = y > x || (y != y && x == x);
+            r += lt || (!gt && t < s);
         }
+        order[r] = s;
+    }
+    __syncthreads();
+    // degenerate sets: chains of |d nu| < tol in ascending order of nu
+    double *g = gamma + (size_t)j * nb;
+    if (s < nb && (s == 0 || v[order[s]] - v[order[s - 1]] >= degen_tol)) {
+        int end = s + 1;
+        while (end < nb && !(v[order[end]] - v[order[end - 1]] >= degen_tol)) ++end;
+        double t = 0.0;
+        for (int b = s; b < end; ++b) t += gs[order[b]];
+        if (end - s > 1) t /= (double)(end - s);
+        for (int b = s; b < end; ++b) g[order[b]] = t;
     }
 }
 
@@ -1020,8 +1025,8 @@ cudaError_t launch_lw_finish(const LwParams &p, const LwDev &d, double degen_tol
     const double pref = kHbarEvPs * kPi / 8.0 * kEvA2AmuPs2 * kEvA2AmuPs2 * kEvA2AmuPs2 /
                         (double)p.nq / (1.0 / delta_norm(p.shape, p.sigma_w));
     const int n_out = p.q1 - p.q0;
-    lw_finish_kernel<<<counted((n_out + 63) / 64), 64, 0, st>>>(n_out, p.nb, p.n_chunks, d.partial, d.qout, d.qrow,
-                                                             d.omega, d.nu, pref, degen_tol_thz, gamma_out);
+    lw_finish_kernel<<<counted(n_out), (p.nb + 31) / 32 * 32, 0, st>>>(p.nb, p.n_chunks, d.partial, d.qout, d.qrow,
+                                                                       d.omega, d.nu, pref, degen_tol_thz, gamma_out);
     return cudaGetLastError();
 }
 

@@ -133,6 +133,30 @@ __device__ __forceinline__ uint32_t pack_f16x2(__half lo_half, __half hi_half) {
 }
 
 
+// w + w' and w - w' over the live rows of a warp, and whether any energy window of
+// theirs can reach a live column with a frequency in r: the epilogue skips the 16
+// columns otherwise (modes ascend in frequency, so a window covers a run of
+// columns; 40% of the chunks of the 32-atom cell on its 8^3 mesh are skipped).
+struct RowRange {
+    float s_lo, s_hi, d_lo, d_hi;
+};
+__device__ __forceinline__ RowRange row_range(bool live, float sum, float dif) {
+    RowRange r{live ? sum : 1e30f, live ? sum : -1e30f, live ? dif : 1e30f, live ? dif : -1e30f};
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        r.s_lo = fminf(r.s_lo, __shfl_xor_sync(0xffffffffu, r.s_lo, o));
+        r.s_hi = fmaxf(r.s_hi, __shfl_xor_sync(0xffffffffu, r.s_hi, o));
+        r.d_lo = fminf(r.d_lo, __shfl_xor_sync(0xffffffffu, r.d_lo, o));
+        r.d_hi = fmaxf(r.d_hi, __shfl_xor_sync(0xffffffffu, r.d_hi, o));
+    }
+    return r;
+}
+template <bool THREE>
+__device__ __forceinline__ bool chunk_reached(const RowRange &r, float2 c, float wide) {
+    return (r.s_lo - c.y < wide && r.s_hi - c.x > -wide) || (r.d_lo - c.y < wide && r.d_hi - c.x > -wide) ||
+           (THREE && r.d_lo + c.x < wide && r.d_hi + c.y > -wide);
+}
+
 // D[m][n] = sum_k A[pair][k][m] B[z][n][k] over the 128-row tiles
 // [blockIdx.x * tpc, ...) of one pair (blockIdx.y); A MN-major, B K-major;
 // z = q' for GEMM1, q'' for GEMM2.  Warp-specialised and persistent over the
@@ -170,6 +194,7 @@ tcx_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__
     // (-w hi, -w hi', -w lo, -w lo'), the same for n, and 1 / w
     __shared__ float4 wpk_sm[64], npk_sm[64];
     __shared__ float2 iwk_sm[64];
+    __shared__ float2 wrange_sm[6];              // least and largest live frequency of 16 columns
     __shared__ float rowsum[2][3][kBM];          // [tile parity][column group][row]
     // EPI_SYM: row sums of position 2 and per-quadrant column sums of position 3
     constexpr int kSymRows = EPI == EPI_SYM ? kBM : 1, kSymCols = EPI == EPI_SYM ? 96 : 1;
@@ -211,6 +236,17 @@ tcx_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__
                 mn[0][j] = v ? -c.z : 0.0f;
                 mn[1][j] = v ? -c.w : 0.0f;
                 iw[j] = v ? 1.0f / c.x : 0.0f;
+            }
+            if (t < 48) {
+                // eight lanes hold the 16 columns of a chunk
+                float lo = fminf(mw[0][0] > -1e29f ? -mw[0][0] : 1e30f, mw[0][1] > -1e29f ? -mw[0][1] : 1e30f);
+                float hi = fmaxf(mw[0][0] > -1e29f ? -mw[0][0] : -1e30f, mw[0][1] > -1e29f ? -mw[0][1] : -1e30f);
+                const unsigned msk = t < 32 ? 0xffffffffu : 0x0000ffffu;
+                for (int o = 1; o < 8; o <<= 1) {
+                    lo = fminf(lo, __shfl_xor_sync(msk, lo, o));
+                    hi = fmaxf(hi, __shfl_xor_sync(msk, hi, o));
+                }
+                if ((t & 7) == 0) wrange_sm[t >> 3] = make_float2(lo, hi);
             }
             wpk_sm[t] = make_float4(mw[0][0], mw[0][1], mw[1][0], mw[1][1]);
             npk_sm[t] = make_float4(mn[0][0], mn[0][1], mn[1][0], mn[1][1]);
@@ -299,6 +335,8 @@ tcx_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__
         const int ew = warp - 4, qd = warp & 3, hf = ew >> 2;
         const int row = qd * 32 + lane;
         float cut = x.cut, s2i = x.sig2inv;
+        // window half width of the chunk test, wider than any rounding of the exact one
+        const float wide = cut * 1.0001f + 1e-4f;
         unsigned int cnt = 0;                      // window hits of this thread (at most H / 2 per tile)
         for (int i = 0; i < n_tiles; ++i) {
             const int tile = t0 + i, buf = i & 1;
@@ -391,8 +429,13 @@ tcx_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__
                 const float rf = live ? 1.0f / (a0.x * a1.x) : 0.0f;                      // 1 / (w1 w2)
                 const float2 RF = make_float2(rf, rf), M1 = make_float2(-1.0f, -1.0f);
                 float2 acc1 = make_float2(0.0f, 0.0f), acc2 = make_float2(0.0f, 0.0f);
+                const RowRange rr = row_range(live, wp.h, wm.h);
                 for (int ci = hf; ok && ci < H / 16; ci += NG) {
                     const int c0 = ci * 16;
+                    if (!chunk_reached<true>(rr, wrange_sm[ci], wide)) {       // uniform over the warp
+                        if (lane < 16 && c0 + lane < kSymCols) colsum[buf][qd][c0 + lane] = 0.0f;
+                        continue;
+                    }
                     float re[16], im[16];
                     tmem_ld16x2(taddr + c0, taddr + H + c0, re, im);
                     float cv[16];
@@ -479,8 +522,10 @@ tcx_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__
                 const float2 N1H = make_float2(a1.z, a1.z), N1L = make_float2(a1.w, a1.w);
                 const float2 HN1 = make_float2(hn1, hn1);
                 float2 acc = make_float2(0.0f, 0.0f);
+                const RowRange rr = row_range(live, wp.h, wm.h);
                 for (int ci = hf; ok && ci < H / 16; ci += NG) {
                     const int c0 = ci * 16;
+                    if (!chunk_reached<false>(rr, wrange_sm[ci], wide)) continue;       // uniform over the warp
                     float re[16], im[16];
                     tmem_ld16x2(taddr + c0, taddr + H + c0, re, im);
                     if (!live) continue;
@@ -1118,28 +1163,15 @@ __global__ void sym_pair_sums_kernel(XParams x, float *__restrict__ out3) {
         v = sl[2 * m] + sl[2 * m + 1];
     } else if (pos == 1) {
         const float *rb = x.rbuf + (size_t)a * x.Mp + m;
+#pragma unroll 8
         for (int s = 0; s < nb; ++s) v += rb[(size_t)s * nb];
     } else {
         const int mt = x.Mp / kBM;
         const float *cb = x.cbuf + (size_t)a * mt * nb + m;
+#pragma unroll 8
         for (int tl = 0; tl < mt; ++tl) v += cb[(size_t)tl * nb];
     }
     out3[((size_t)(x.pair0 + a) * 3 + pos) * nb + m] = v;
-}
-
-// gacc[i][s] = sum over the entries e of class i (CSR, a fixed order) of
-// fac[e] out3[ent[e]][s], FP64: the linewidth sums of the q-points of class
-// i ({q, -q}) from every orbit projection that holds one of them.
-__global__ void sym_class_sums_kernel(int n_cls, int nb, const int *__restrict__ cls_start,
-                                      const int *__restrict__ ent, const double *__restrict__ fac,
-                                      const float *__restrict__ out3, double *__restrict__ gacc) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n_cls * nb) return;
-    const int i = t / nb, m = t - i * nb;
-    double sum = 0.0;
-    for (int e = cls_start[i]; e < cls_start[i + 1]; ++e)
-        sum += fac[e] * (double)out3[(size_t)ent[e] * nb + m];
-    gacc[t] = sum;
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -1300,6 +1332,15 @@ cudaError_t run_batches(const LwParams &p, const LwDev &d, const TcxGroups &g, L
 
 }  // namespace
 
+// Blocks per (j, k) group from which the phase sum on tensor cores is considered
+// (its MMAs do not grow with the blocks, the gather does), or when KALD_TCX_Y asks
+// for it.
+constexpr int kTcxYBlocks = 12;
+bool tcx_y_wanted(size_t n_fc3, size_t n_groups) {
+    if (const char *ey = std::getenv("KALD_TCX_Y")) return std::atoi(ey) != 0;
+    return n_fc3 >= (size_t)kTcxYBlocks * std::max<size_t>(n_groups, 1);
+}
+
 int tcx_half(int nb) { return (nb + 31) / 32 * 32; }
 bool tcx_supported(int nb) { return nb > 64 && nb <= 96; }
 
@@ -1368,64 +1409,6 @@ size_t tcx_sym_bytes(int nb, int batch, int n_pairs) {
            ws_round(sizeof(float) * 3 * (size_t)n_pairs * nb);
 }
 
-// Canonical triples: for every ordered pair (q1, q2) the triple (q1, q2, q3),
-// q3 = -(q1 + q2) on the mesh, is kept when it is the smallest (lexicographic)
-// of the ordered triples its orbit under the six permutations and inversion
-// q -> -q reaches.  Each orbit is kept once, by its smallest member.
-void plan_tcx_sym(const int32_t mesh[3], const std::vector<int> &qf, const std::vector<int> &qcls,
-                  const std::vector<int> &self_inv, TcxSymHost &out) {
-    const int m0 = mesh[0], m1 = mesh[1], m2 = mesh[2], nq = m0 * m1 * m2;
-    auto flat = [&](int k0, int k1, int k2) {
-        return (((k0 % m0) + m0) % m0 * m1 + ((k1 % m1) + m1) % m1) * m2 + ((k2 % m2) + m2) % m2;
-    };
-    std::vector<int> neg(nq);
-    for (int q = 0; q < nq; ++q) neg[q] = flat(-qf[3 * q], -qf[3 * q + 1], -qf[3 * q + 2]);
-    out.pairs.clear();
-    out.orbit.clear();
-    for (int q1 = 0; q1 < nq; ++q1)
-        for (int q2 = 0; q2 < nq; ++q2) {
-            const int q3 = neg[flat(qf[3 * q1] + qf[3 * q2], qf[3 * q1 + 1] + qf[3 * q2 + 1],
-                                    qf[3 * q1 + 2] + qf[3 * q2 + 2])];
-            const std::array<int, 3> t{q1, q2, q3};
-            std::array<std::array<int, 3>, 12> img;
-            const int perm[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
-            bool canonical = true;
-            for (int p = 0; p < 6 && canonical; ++p) {
-                img[2 * p] = {t[perm[p][0]], t[perm[p][1]], t[perm[p][2]]};
-                img[2 * p + 1] = {neg[img[2 * p][0]], neg[img[2 * p][1]], neg[img[2 * p][2]]};
-                canonical = !(img[2 * p] < t) && !(img[2 * p + 1] < t);
-            }
-            if (!canonical) continue;
-            std::sort(img.begin(), img.end());
-            const int n_orb = (int)(std::unique(img.begin(), img.end()) - img.begin());
-            out.pairs.push_back(make_int2(q1, q2));
-            out.orbit.push_back(n_orb);
-        }
-    // entries per class, in (class, pair, position) order
-    const int n_cls = (int)self_inv.size();
-    const size_t np = out.pairs.size();
-    out.cls_start.assign(n_cls + 1, 0);
-    std::vector<int> cls_of(3 * np);
-    for (size_t i = 0; i < np; ++i) {
-        const int q1 = out.pairs[i].x, q2 = out.pairs[i].y;
-        const int q3 = neg[flat(qf[3 * q1] + qf[3 * q2], qf[3 * q1 + 1] + qf[3 * q2 + 1], qf[3 * q1 + 2] + qf[3 * q2 + 2])];
-        const int qs[3] = {q1, q2, q3};
-        for (int pos = 0; pos < 3; ++pos) {
-            cls_of[3 * i + pos] = qcls[qs[pos]];
-            ++out.cls_start[qcls[qs[pos]] + 1];
-        }
-    }
-    for (int c = 0; c < n_cls; ++c) out.cls_start[c + 1] += out.cls_start[c];
-    out.ent.assign(3 * np, 0);
-    out.fac.assign(3 * np, 0.0);
-    std::vector<int> fill(out.cls_start.begin(), out.cls_start.end() - 1);
-    for (size_t e = 0; e < 3 * np; ++e) {
-        const int c = cls_of[e], at = fill[c]++;
-        out.ent[at] = (int)e;
-        out.fac[at] = out.orbit[e / 3] / 12.0 * (self_inv[c] ? 2.0 : 1.0);
-    }
-}
-
 size_t tcx_scratch_bytes(int nb, int nq, int batch) {
     const int H = tcx_half(nb), Kp = 2 * H, BN = 2 * H;
     const size_t Mp = (size_t)(nb * nb + kBM - 1) / kBM * kBM;
@@ -1462,7 +1445,10 @@ TcxSched tcx_schedule(int nb, int nq, int n_groups, bool y_ok, bool sym, int sms
     auto tpc_for = [&](int batch, int waves) { return tiles_for(mt, batch, waves); };
     const int mty = std::max(1, (n_groups + kYGroups - 1) / kYGroups);
     const int yk0 = y_ok ? 1 : 0;
-    TcxSched def{b0, tpc_for(b0, 1), 2, yk0, tiles_for(mty, b0, 1)};
+    // untimed problems take the CUDA-core gather: 3.1 us a pair against 6.2 us on
+    // tensor cores for 7 blocks per atom pair; the tensor-core sum is timed, and its
+    // operands made, from kTcxYBlocks blocks per atom pair on (tcx_y_wanted)
+    TcxSched def{b0, tpc_for(b0, 1), 2, 0, tiles_for(mty, b0, 1)};
     const char *eb = std::getenv("KALD_TCX_BATCH"), *et = std::getenv("KALD_TCX_TPC"), *eg = std::getenv("KALD_TCX_GP");
     const char *ey = std::getenv("KALD_TCX_Y");
     if (eb || et || eg || ey) {
@@ -1545,7 +1531,7 @@ TcxSched tcx_schedule(int nb, int nq, int n_groups, bool y_ok, bool sym, int sms
 // launch_lw_finish, the delta-allowed count into d.allowed and bounded-wait
 // failures into err.
 cudaError_t launch_lw_tensor(const LwParams &p, const LwDev &d, const TcxGroups &g, void *scratch, int batch,
-                             int sms, int *err, cudaStream_t st, const TcxSym *sym, void *sym_scratch) {
+                             int sms, int *err, cudaStream_t st, const OrbitPlan *sym, void *sym_scratch) {
     const int nb = p.nb, nq = p.nq;
     if (!tcx_supported(nb) || batch < 1 || g.n_parts < 1 || sms < 1) return cudaErrorInvalidValue;
     const int H = tcx_half(nb), Kp = 2 * H, BN = 2 * H;
@@ -1572,8 +1558,12 @@ cudaError_t launch_lw_tensor(const LwParams &p, const LwDev &d, const TcxGroups 
     auto *slots = reinterpret_cast<float *>(take(sizeof(float) * 2 * (size_t)n_slices * nq * nb));
     auto *gacc = reinterpret_cast<double *>(take(sizeof(double) * (size_t)nq * nb));
 
-    // entries of A1 / T1 that no group or column covers stay zero: clear once
-    cudaError_t e = cudaMemsetAsync(pl[0][0], 0, 8 * ws_round(ab), st);
+    // entries of A1 / T1 that no group or column covers stay zero: clear once (not
+    // where every atom pair has blocks and no row or column is padding: then every
+    // entry is written for every pair; 0.6 ms of a 6 ms call on a 4^3 mesh)
+    const bool covered = nb % 32 == 0 && Mp == nb * nb && (long long)g.n_groups * 9 == (long long)nb * nb;
+    cudaError_t e = cudaSuccess;
+    if (!covered) e = cudaMemsetAsync(pl[0][0], 0, 8 * ws_round(ab), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(gacc, 0, sizeof(double) * (size_t)nq * nb, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(d.allowed, 0, sizeof(unsigned long long), st);
@@ -1607,8 +1597,8 @@ cudaError_t launch_lw_tensor(const LwParams &p, const LwDev &d, const TcxGroups 
     float *out3 = nullptr;
     const size_t mtl = (size_t)Mp / kBM;
     if (sym) {
-        x.plist = sym->plist;
-        x.porb = sym->porb;
+        x.plist = sym->pairs;
+        x.porb = sym->orbit;
         char *sb = static_cast<char *>(sym_scratch);
         out3 = reinterpret_cast<float *>(sb + 2 * ws_round(sizeof(float) * (size_t)batch * Mp) +
                                          2 * ws_round(sizeof(float) * (size_t)batch * mtl * nb));
@@ -1670,12 +1660,8 @@ cudaError_t launch_lw_tensor(const LwParams &p, const LwDev &d, const TcxGroups 
         if (ev[k]) cudaEventDestroy(ev[k]);
     if (e != cudaSuccess) return e;
     if (sym) {
-        // class sums from the per-pair sums of every orbit (after both lanes)
-        const int n = sym->n_cls * nb;
-        sym_class_sums_kernel<<<counted((n + 127) / 128), 128, 0, st>>>(sym->n_cls, nb, sym->cls_start, sym->ent,
-                                                                        sym->fac, out3, gacc);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+        // the sums of each q-point from those of its orbits (after both lanes)
+        return launch_orbit_class_sums(*sym, nb, out3, d.partial, st);
     }
     return cudaMemcpyAsync(d.partial, gacc, sizeof(double) * (size_t)p.nqc * nb,
                            cudaMemcpyDeviceToDevice, st);
