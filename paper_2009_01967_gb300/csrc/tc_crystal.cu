@@ -176,7 +176,7 @@ template <int EPI> struct Warps {
     static constexpr int kThreads = 32 * (4 + kEpi);
 };
 
-template <int EPI, int BN, int PB>
+template <int EPI, int BN, int PB, int SHAPE>
 __global__ void __launch_bounds__(Warps<EPI>::kThreads, 1)
 tcx_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ CUtensorMap mAl,
                 const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CUtensorMap mBm,
@@ -188,13 +188,14 @@ tcx_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__
     unsigned char *sB = base;                      // [kb][piece][BN rows x 128 B]
     unsigned char *sA = base + C::kBBytes;         // [stage][hi, lo][two 64-row atoms]
     __shared__ __align__(8) uint64_t bfull, afull[kStages], aempty[kStages], tfull[2], tempty[2], drain;
+    __shared__ __align__(8) uint64_t rfull[2], rfree[2];       // the sums of a tile parity: written, reduced
     __shared__ uint32_t tmem_base_sm;
     __shared__ int fail_sm;
     // columns of q'' in pairs (2u, 2u + 1) for the packed FP32x2 epilogue:
     // (-w hi, -w hi', -w lo, -w lo'), the same for n, and 1 / w
     __shared__ float4 wpk_sm[64], npk_sm[64];
     __shared__ float2 iwk_sm[64];
-    __shared__ float2 wrange_sm[6];              // least and largest live frequency of 16 columns
+    __shared__ float2 wrange_sm[12];             // least and largest live frequency of 8 columns
     __shared__ float rowsum[2][3][kBM];          // [tile parity][column group][row]
     // EPI_SYM: row sums of position 2 and per-quadrant column sums of position 3
     constexpr int kSymRows = EPI == EPI_SYM ? kBM : 1, kSymCols = EPI == EPI_SYM ? 96 : 1;
@@ -217,7 +218,12 @@ tcx_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__
     if (threadIdx.x == 0) {
         mbar_init(&bfull, 1);
         for (int s = 0; s < kStages; ++s) { mbar_init(&afull[s], 1); mbar_init(&aempty[s], 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(&tfull[b], 1); mbar_init(&tempty[b], NE); }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&tfull[b], 1);
+            mbar_init(&tempty[b], NE);
+            mbar_init(&rfull[b], NE);
+            mbar_init(&rfree[b], 2);
+        }
         mbar_init(&drain, 1);
         fail_sm = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -238,15 +244,15 @@ tcx_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__
                 iw[j] = v ? 1.0f / c.x : 0.0f;
             }
             if (t < 48) {
-                // eight lanes hold the 16 columns of a chunk
+                // four lanes hold the 8 columns of a chunk
                 float lo = fminf(mw[0][0] > -1e29f ? -mw[0][0] : 1e30f, mw[0][1] > -1e29f ? -mw[0][1] : 1e30f);
                 float hi = fmaxf(mw[0][0] > -1e29f ? -mw[0][0] : -1e30f, mw[0][1] > -1e29f ? -mw[0][1] : -1e30f);
                 const unsigned msk = t < 32 ? 0xffffffffu : 0x0000ffffu;
-                for (int o = 1; o < 8; o <<= 1) {
+                for (int o = 1; o < 4; o <<= 1) {
                     lo = fminf(lo, __shfl_xor_sync(msk, lo, o));
                     hi = fmaxf(hi, __shfl_xor_sync(msk, hi, o));
                 }
-                if ((t & 7) == 0) wrange_sm[t >> 3] = make_float2(lo, hi);
+                if ((t & 3) == 0) wrange_sm[t >> 2] = make_float2(lo, hi);
             }
             wpk_sm[t] = make_float4(mw[0][0], mw[0][1], mw[1][0], mw[1][1]);
             npk_sm[t] = make_float4(mn[0][0], mn[0][1], mn[1][0], mn[1][1]);
@@ -331,13 +337,9 @@ tcx_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__
             }
             mma_commit(&drain);                    // every MMA of this thread done
         }
-    } else if (warp >= 4) {
+    } else if (warp >= 4 && EPI == EPI_T) {
         const int ew = warp - 4, qd = warp & 3, hf = ew >> 2;
         const int row = qd * 32 + lane;
-        float cut = x.cut, s2i = x.sig2inv;
-        // window half width of the chunk test, wider than any rounding of the exact one
-        const float wide = cut * 1.0001f + 1e-4f;
-        unsigned int cnt = 0;                      // window hits of this thread (at most H / 2 per tile)
         for (int i = 0; i < n_tiles; ++i) {
             const int tile = t0 + i, buf = i & 1;
             bool ok = !*(volatile int *)&fail_sm && mbar_wait(&tfull[buf], (i >> 1) & 1, x.wait_limit);
@@ -345,102 +347,135 @@ tcx_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             if (!ok) fail_sm = 1;
             const uint32_t taddr = tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)(buf * (C::kTmemCols / 2));
-            const int r = tile * kBM + row;            // (c, s) for GEMM1, (s, s') for GEMM2
+            const int r = tile * kBM + row;            // (c, s)
             const bool rv = r < nb * nb;
             const int r_hi = r / nb, r_lo = r - r_hi * nb;
-            if (EPI == EPI_T) {
-                const int c = r_hi, s = r_lo;
-                const bool vec = (nb % 8) == 0;
-                // nb a multiple of 32 (so H = nb and nb^2 = Mp): every warp's 32 rows
-                // are valid and share c, with consecutive s
-                const bool pairs = (nb % 32) == 0 && H == nb && x.Mp == nb * nb;
-                for (int ci = hf; ok && ci < BN / 32; ci += NG) {
-                    const int c0 = ci * 32;
-                    float v[32];
-                    tmem_ld32(taddr + c0, v);
-                    if (!rv) continue;
-                    const int part = c0 >= H ? 1 : 0;   // H is a multiple of 32
-                    const int sp0 = c0 - part * H;
-                    if (sp0 >= nb) continue;
-                    const size_t off = ((size_t)a * x.Kp + part * H + c) * x.Mp + (size_t)s * nb + sp0;
-                    if (pairs) {
-                        uint32_t hw[16], lw[16];
+            const int c = r_hi, s = r_lo;
+            const bool vec = (nb % 8) == 0;
+            // nb a multiple of 32 (so H = nb and nb^2 = Mp): every warp's 32 rows
+            // are valid and share c, with consecutive s
+            const bool pairs = (nb % 32) == 0 && H == nb && x.Mp == nb * nb;
+            for (int ci = hf; ok && ci < BN / 32; ci += NG) {
+                const int c0 = ci * 32;
+                float v[32];
+                tmem_ld32(taddr + c0, v);
+                if (!rv) continue;
+                const int part = c0 >= H ? 1 : 0;   // H is a multiple of 32
+                const int sp0 = c0 - part * H;
+                if (sp0 >= nb) continue;
+                const size_t off = ((size_t)a * x.Kp + part * H + c) * x.Mp + (size_t)s * nb + sp0;
+                if (pairs) {
+                    uint32_t hw[16], lw[16];
 #pragma unroll
-                        for (int e = 0; e < 16; ++e) {
-                            const float f0 = v[2 * e], f1 = v[2 * e + 1];
+                    for (int e = 0; e < 16; ++e) {
+                        const float f0 = v[2 * e], f1 = v[2 * e + 1];
+                        const __nv_bfloat16 h0 = __float2bfloat16_rn(f0), h1 = __float2bfloat16_rn(f1);
+                        hw[e] = pack_bf16x2(h0, h1);
+                        lw[e] = pack_bf16x2(__float2bfloat16_rn(f0 - __bfloat162float(h0)),
+                                            __float2bfloat16_rn(f1 - __bfloat162float(h1)));
+                    }
+                    const size_t rs = sizeof(__nv_bfloat16) * (size_t)nb;
+                    st_rowpair_v8(reinterpret_cast<char *>(x.t1h + off), rs, hw, lane & 1);
+                    st_rowpair_v8(reinterpret_cast<char *>(x.t1l + off), rs, lw, lane & 1);
+                } else if (vec && sp0 + 32 <= nb) {
+                    uint4 *ph = reinterpret_cast<uint4 *>(x.t1h + off);
+                    uint4 *pl = reinterpret_cast<uint4 *>(x.t1l + off);
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) {
+                        uint32_t hw[4], lw[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const float f0 = v[8 * g + 2 * e], f1 = v[8 * g + 2 * e + 1];
                             const __nv_bfloat16 h0 = __float2bfloat16_rn(f0), h1 = __float2bfloat16_rn(f1);
                             hw[e] = pack_bf16x2(h0, h1);
                             lw[e] = pack_bf16x2(__float2bfloat16_rn(f0 - __bfloat162float(h0)),
                                                 __float2bfloat16_rn(f1 - __bfloat162float(h1)));
                         }
-                        const size_t rs = sizeof(__nv_bfloat16) * (size_t)nb;
-                        st_rowpair_v8(reinterpret_cast<char *>(x.t1h + off), rs, hw, lane & 1);
-                        st_rowpair_v8(reinterpret_cast<char *>(x.t1l + off), rs, lw, lane & 1);
-                    } else if (vec && sp0 + 32 <= nb) {
-                        uint4 *ph = reinterpret_cast<uint4 *>(x.t1h + off);
-                        uint4 *pl = reinterpret_cast<uint4 *>(x.t1l + off);
+                        ph[g] = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+                        pl[g] = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+                    }
+                } else {
 #pragma unroll
-                        for (int g = 0; g < 4; ++g) {
-                            uint32_t hw[4], lw[4];
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const float f0 = v[8 * g + 2 * e], f1 = v[8 * g + 2 * e + 1];
-                                const __nv_bfloat16 h0 = __float2bfloat16_rn(f0), h1 = __float2bfloat16_rn(f1);
-                                hw[e] = pack_bf16x2(h0, h1);
-                                lw[e] = pack_bf16x2(__float2bfloat16_rn(f0 - __bfloat162float(h0)),
-                                                    __float2bfloat16_rn(f1 - __bfloat162float(h1)));
-                            }
-                            ph[g] = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-                            pl[g] = make_uint4(lw[0], lw[1], lw[2], lw[3]);
-                        }
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) {
-                            if (sp0 + e >= nb) continue;
-                            const __nv_bfloat16 h = __float2bfloat16_rn(v[e]);
-                            x.t1h[off + e] = h;
-                            x.t1l[off + e] = __float2bfloat16_rn(v[e] - __bfloat162float(h));
-                        }
+                    for (int e = 0; e < 32; ++e) {
+                        if (sp0 + e >= nb) continue;
+                        const __nv_bfloat16 h = __float2bfloat16_rn(v[e]);
+                        x.t1h[off + e] = h;
+                        x.t1l[off + e] = __float2bfloat16_rn(v[e] - __bfloat162float(h));
                     }
                 }
-            } else if (EPI == EPI_SYM) {
-                // positions 1 = (q, s), 2 = (q', s'), 3 = (-q'', s'') of the triple;
-                // w3 = w(q''), n3 = n(q'').  With D1 = G(w2 + w3 - w1),
-                // D2 = G(w1 + w3 - w2), D3 = G(w1 + w2 - w3) (Gaussian, or the
-                // chosen shape, inside the window), each position p takes
-                //   F1 = (n2 - n3)(D3 - D2) + (1 + n2 + n3) D1
-                //   F2 = (n1 - n3)(D3 - D1) + (1 + n1 + n3) D2
-                //   F3 = (n1 - n2)(D2 - D1) + (1 + n1 + n2) D3
-                // times |phi|^2 / (w of the other two positions).
-                const int s = r_hi, sp = r_lo;
-                const float4 a0 = rv ? x.wn[(size_t)q * nb + s] : make_float4(0.f, 0.f, 0.f, 0.f);
-                const float4 a1 = rv ? x.wn[(size_t)qp * nb + sp] : make_float4(0.f, 0.f, 0.f, 0.f);
-                const bool live = rv && a0.x > 0.0f && a1.x > 0.0f;
-                const F2 wp = f2_add(F2{a0.x, a0.y}, F2{a1.x, a1.y});     // w1 + w2
-                const F2 wm = f2_add(F2{a0.x, a0.y}, F2{-a1.x, -a1.y});   // w1 - w2
-                const float2 WPH = make_float2(wp.h, wp.h), WPL = make_float2(wp.l, wp.l);
-                const float2 WMH = make_float2(wm.h, wm.h), WML = make_float2(wm.l, wm.l);
-                const float2 N2H = make_float2(a1.z, a1.z), N2L = make_float2(a1.w, a1.w);
-                const float2 N1H = make_float2(a0.z, a0.z), N1L = make_float2(a0.w, a0.w);
-                const float2 K2 = make_float2(1.0f + a1.z, 1.0f + a1.z), K1 = make_float2(1.0f + a0.z, 1.0f + a0.z);
-                const float n12 = __fadd_rn(__fsub_rn(a0.z, a1.z), __fsub_rn(a0.w, a1.w));   // n1 - n2
-                const float2 N12 = make_float2(n12, n12);
-                const float2 S12 = make_float2(1.0f + a0.z + a1.z, 1.0f + a0.z + a1.z);
-                const float rf = live ? 1.0f / (a0.x * a1.x) : 0.0f;                      // 1 / (w1 w2)
-                const float2 RF = make_float2(rf, rf), M1 = make_float2(-1.0f, -1.0f);
-                float2 acc1 = make_float2(0.0f, 0.0f), acc2 = make_float2(0.0f, 0.0f);
-                const RowRange rr = row_range(live, wp.h, wm.h);
-                for (int ci = hf; ok && ci < H / 16; ci += NG) {
-                    const int c0 = ci * 16;
-                    if (!chunk_reached<true>(rr, wrange_sm[ci], wide)) {       // uniform over the warp
-                        if (lane < 16 && c0 + lane < kSymCols) colsum[buf][qd][c0 + lane] = 0.0f;
-                        continue;
-                    }
-                    float re[16], im[16];
-                    tmem_ld16x2(taddr + c0, taddr + H + c0, re, im);
-                    float cv[16];
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&tempty[buf]);
+        }
+    } else if (warp >= 4) {
+        // ---- GEMM2: |phi|^2, windows and weights.  Warp (quadrant qd, group hf): rows
+        // 32 qd .. of the tile; the three groups of a quadrant deal its reached chunks
+        // of 8 columns among themselves.  The sums go to shared memory; warps 2 and 3
+        // reduce them while these warps are in the next tile.
+        const int ew = warp - 4, qd = warp & 3, hf = ew >> 2;
+        const int row = qd * 32 + lane;
+        const float cut = x.cut, s2i = delta_param2(SHAPE, x.sig2inv);
+        // window half width of the chunk test, wider than any rounding of the exact one
+        const float wide = cut * 1.0001f + 1e-4f;
+        const float2 M1 = make_float2(-1.0f, -1.0f);
+        float2 cnt2 = make_float2(0.0f, 0.0f);         // window hits of this thread (exact: far below 2^24)
+        auto load_row = [&](int tile, float4 &a0, float4 &a1) {
+            const int r = tile * kBM + row, s = r / nb;
+            const bool rv = r < nb * nb;
+            a0 = rv ? __ldg(x.wn + (size_t)q * nb + s) : make_float4(0.f, 0.f, 0.f, 0.f);
+            a1 = rv ? __ldg(x.wn + (size_t)qp * nb + (r - s * nb)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        };
+        float4 a0n, a1n;                               // the next tile's rows, loaded one tile ahead
+        load_row(t0, a0n, a1n);
+        for (int i = 0; i < n_tiles; ++i) {
+            const int tile = t0 + i, buf = i & 1;
+            const float4 a0 = a0n, a1 = a1n;
+            if (i + 1 < n_tiles) load_row(tile + 1, a0n, a1n);
+            const bool live = a0.x > 0.0f && a1.x > 0.0f;
+            // w1 + w2 and w1 - w2 as FP32 pairs; a dead row is out of every window's reach
+            const F2 wp = live ? f2_add(F2{a0.x, a0.y}, F2{a1.x, a1.y}) : F2{4e30f, 0.f};
+            const F2 wm = live ? f2_add(F2{a0.x, a0.y}, F2{-a1.x, -a1.y}) : F2{4e30f, 0.f};
+            const RowRange rr = row_range(live, wp.h, wm.h);
+            const unsigned chunks =
+                __ballot_sync(0xffffffffu, lane < H / 8 && chunk_reached<EPI == EPI_SYM>(rr, wrange_sm[min(lane, 11)], wide));
+            const float2 WPH = make_float2(wp.h, wp.h), WPL = make_float2(wp.l, wp.l);
+            const float2 WMH = make_float2(wm.h, wm.h), WML = make_float2(wm.l, wm.l);
+            const float2 N2H = make_float2(a1.z, a1.z), N2L = make_float2(a1.w, a1.w);
+            // the tile's accumulator, and the sums' buffer of this parity
+            bool ok = !*(volatile int *)&fail_sm && mbar_wait(&tfull[buf], (i >> 1) & 1, x.wait_limit) &&
+                      (i < 2 || mbar_wait(&rfree[buf], ((i >> 1) - 1) & 1, x.wait_limit));
+            ok = __all_sync(0xffffffffu, ok);
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            if (!ok) {
+                fail_sm = 1;
+                break;
+            }
+            const uint32_t taddr = tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)(buf * (C::kTmemCols / 2));
+            float2 acc1 = make_float2(0.0f, 0.0f), acc2 = make_float2(0.0f, 0.0f);
+            int rank = 0;
+            for (unsigned left = chunks; left; left &= left - 1) {
+                if (rank++ % NG != hf) continue;       // uniform over the warp
+                const int c0 = 8 * (__ffs(left) - 1);
+                float re[8], im[8];
+                tmem_ld8x2(taddr + c0, taddr + H + c0, re, im);
+                if constexpr (EPI == EPI_SYM) {
+                    // positions 1 = (q, s), 2 = (q', s'), 3 = (-q'', s'') of the triple;
+                    // w3 = w(q''), n3 = n(q'').  With D1 = G(w2 + w3 - w1),
+                    // D2 = G(w1 + w3 - w2), D3 = G(w1 + w2 - w3) inside the window, each
+                    // position p takes
+                    //   F1 = (n2 - n3)(D3 - D2) + (1 + n2 + n3) D1
+                    //   F2 = (n1 - n3)(D3 - D1) + (1 + n1 + n3) D2
+                    //   F3 = (n1 - n2)(D2 - D1) + (1 + n1 + n2) D3
+                    // times |phi|^2 / (w of the other two positions).
+                    const float2 N1H = make_float2(a0.z, a0.z), N1L = make_float2(a0.w, a0.w);
+                    const float2 K2 = make_float2(1.0f + a1.z, 1.0f + a1.z), K1 = make_float2(1.0f + a0.z, 1.0f + a0.z);
+                    const float n12 = __fadd_rn(__fsub_rn(a0.z, a1.z), __fsub_rn(a0.w, a1.w));   // n1 - n2
+                    const float2 N12 = make_float2(n12, n12);
+                    const float2 S12 = make_float2(1.0f + a0.z + a1.z, 1.0f + a0.z + a1.z);
+                    float cv[8];
 #pragma unroll
-                    for (int k = 0; k < 16; k += 2) {
+                    for (int k = 0; k < 8; k += 2) {
                         const int u = (c0 + k) >> 1;
                         const float4 cw = wpk_sm[u], cn = npk_sm[u];
                         const float2 mwh = make_float2(cw.x, cw.y), mwl = make_float2(cw.z, cw.w);
@@ -448,167 +483,149 @@ tcx_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__
                         const float2 d3 = __fadd2_rn(__fadd2_rn(WPH, mwh), __fadd2_rn(WPL, mwl));   // w1 + w2 - w3
                         const float2 d1 = __fadd2_rn(__fadd2_rn(WMH, mwh), __fadd2_rn(WML, mwl));   // w1 - w2 - w3
                         const float2 d2 = __fadd2_rn(__ffma2_rn(M1, mwh, WMH), __ffma2_rn(M1, mwl, WML));   // w1 - w2 + w3
+                        const float2 m3 = make_float2(fabsf(d3.x) < cut ? 1.0f : 0.0f, fabsf(d3.y) < cut ? 1.0f : 0.0f);
+                        const float2 m1 = make_float2(fabsf(d1.x) < cut ? 1.0f : 0.0f, fabsf(d1.y) < cut ? 1.0f : 0.0f);
+                        const float2 m2 = make_float2(fabsf(d2.x) < cut ? 1.0f : 0.0f, fabsf(d2.y) < cut ? 1.0f : 0.0f);
+                        const float2 e1 = __fmul2_rn(delta_shape2<SHAPE>(d1, s2i), m1);
+                        const float2 e2 = __fmul2_rn(delta_shape2<SHAPE>(d2, s2i), m2);
+                        const float2 e3 = __fmul2_rn(delta_shape2<SHAPE>(d3, s2i), m3);
                         const float2 n23 = __fadd2_rn(__fadd2_rn(N2H, mnh), __fadd2_rn(N2L, mnl));  // n2 - n3
                         const float2 n13 = __fadd2_rn(__fadd2_rn(N1H, mnh), __fadd2_rn(N1L, mnl));  // n1 - n3
                         const float2 s23 = __ffma2_rn(M1, mnh, K2);                                 // 1 + n2 + n3
                         const float2 s13 = __ffma2_rn(M1, mnh, K1);                                 // 1 + n1 + n3
-                        float2 e1 = delta_shape2(d1, x.shape, s2i), e2 = delta_shape2(d2, x.shape, s2i);
-                        float2 e3 = delta_shape2(d3, x.shape, s2i);
-                        const bool h1x = fabsf(d1.x) < cut, h1y = fabsf(d1.y) < cut;
-                        const bool h2x = fabsf(d2.x) < cut, h2y = fabsf(d2.y) < cut;
-                        const bool h3x = fabsf(d3.x) < cut, h3y = fabsf(d3.y) < cut;
-                        e1.x = h1x ? e1.x : 0.0f; e1.y = h1y ? e1.y : 0.0f;
-                        e2.x = h2x ? e2.x : 0.0f; e2.y = h2y ? e2.y : 0.0f;
-                        e3.x = h3x ? e3.x : 0.0f; e3.y = h3y ? e3.y : 0.0f;
-                        const float2 f1 = __ffma2_rn(n23, __fadd2_rn(e3, __fmul2_rn(M1, e2)), __fmul2_rn(s23, e1));
-                        const float2 f2 = __ffma2_rn(n13, __fadd2_rn(e3, __fmul2_rn(M1, e1)), __fmul2_rn(s13, e2));
-                        const float2 f3 = __ffma2_rn(N12, __fadd2_rn(e2, __fmul2_rn(M1, e1)), __fmul2_rn(S12, e3));
+                        const float2 f1 = __ffma2_rn(n23, __ffma2_rn(M1, e2, e3), __fmul2_rn(s23, e1));
+                        const float2 f2 = __ffma2_rn(n13, __ffma2_rn(M1, e1, e3), __fmul2_rn(s13, e2));
+                        const float2 f3 = __ffma2_rn(N12, __ffma2_rn(M1, e1, e2), __fmul2_rn(S12, e3));
                         const float2 r2 = make_float2(re[k], re[k + 1]), i2 = make_float2(im[k], im[k + 1]);
                         const float2 p2 = live ? __ffma2_rn(r2, r2, __fmul2_rn(i2, i2)) : make_float2(0.0f, 0.0f);
                         const float2 pw = __fmul2_rn(p2, iwk_sm[u]);                                // |phi|^2 / w3
                         acc1 = __ffma2_rn(pw, f1, acc1);
                         acc2 = __ffma2_rn(pw, f2, acc2);
-                        const float2 c3 = __fmul2_rn(__fmul2_rn(p2, f3), RF);
+                        const float2 c3 = __fmul2_rn(p2, f3);
                         cv[k] = c3.x;
                         cv[k + 1] = c3.y;
-                        if (live)
-                            cnt += (unsigned)((h1x || h2x) + (h2x || h3x) + (h1x || h3x)) +
-                                   (unsigned)((h1y || h2y) + (h2y || h3y) + (h1y || h3y));
+                        // pairs of windows with a hit: 0, 2, 3, 3 of three for 0 .. 3 hits
+                        const float2 nh = __fadd2_rn(__fadd2_rn(m1, m2), m3), nn = __fadd2_rn(nh, nh);
+                        cnt2 = __fadd2_rn(cnt2, make_float2(fminf(nn.x, 3.0f), fminf(nn.y, 3.0f)));
                     }
-                    // column sums over the warp's 32 rows: halving exchanges, then
-                    // lanes 2c and 2c + 1 hold column c of the chunk
+                    // column sums of p2 f3 / (w1 w2) over the warp's 32 rows: halving
+                    // exchanges, then the four lanes of a column
+                    const float rf = live ? 1.0f / (a0.x * a1.x) : 0.0f;
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
+                    for (int y = 0; y < 8; ++y) cv[y] *= rf;
+#pragma unroll
+                    for (int y = 0; y < 4; ++y) {
                         const bool up = lane & 16;
-                        const float give = up ? cv[i] : cv[i + 8], keep = up ? cv[i + 8] : cv[i];
-                        cv[i] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+                        const float give = up ? cv[y] : cv[y + 4], keep = up ? cv[y + 4] : cv[y];
+                        cv[y] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
                     }
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
+                    for (int y = 0; y < 2; ++y) {
                         const bool up = lane & 8;
-                        const float give = up ? cv[i] : cv[i + 4], keep = up ? cv[i + 4] : cv[i];
-                        cv[i] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
-                    }
-#pragma unroll
-                    for (int i = 0; i < 2; ++i) {
-                        const bool up = lane & 4;
-                        const float give = up ? cv[i] : cv[i + 2], keep = up ? cv[i + 2] : cv[i];
-                        cv[i] = keep + __shfl_xor_sync(0xffffffffu, give, 4);
+                        const float give = up ? cv[y] : cv[y + 2], keep = up ? cv[y + 2] : cv[y];
+                        cv[y] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
                     }
                     {
-                        const bool up = lane & 2;
+                        const bool up = lane & 4;
                         const float give = up ? cv[0] : cv[1], keep = up ? cv[1] : cv[0];
-                        cv[0] = keep + __shfl_xor_sync(0xffffffffu, give, 2);
+                        cv[0] = keep + __shfl_xor_sync(0xffffffffu, give, 4);
                     }
+                    cv[0] += __shfl_xor_sync(0xffffffffu, cv[0], 2);
                     cv[0] += __shfl_xor_sync(0xffffffffu, cv[0], 1);
-                    const int col = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
-                    if ((lane & 1) == 0 && c0 + col < kSymCols) colsum[buf][qd][c0 + col] = cv[0];
-                }
-                rowsum[buf][hf][row] = live ? (acc1.x + acc1.y) / a1.x : 0.0f;      // / w2
-                rowsum_b[buf][hf][row] = live ? (acc2.x + acc2.y) / a0.x : 0.0f;    // / w1
-            } else {
-                const int s = r_hi, sp = r_lo;
-                const float4 a0 = rv ? x.wn[(size_t)q * nb + s] : make_float4(0.f, 0.f, 0.f, 0.f);
-                const float4 a1 = rv ? x.wn[(size_t)qp * nb + sp] : make_float4(0.f, 0.f, 0.f, 0.f);
-                const bool live = rv && a0.x > 0.0f && a1.x > 0.0f;
-                const float w1 = a1.x;
-                // w + w' and w - w' as FP32 pairs; n' as a pair (wdiff.cuh)
-                const F2 wp = f2_add(F2{a0.x, a0.y}, F2{a1.x, a1.y});
-                const F2 wm = f2_add(F2{a0.x, a0.y}, F2{-a1.x, -a1.y});
-                const float hn1 = 0.5f * (1.0f + a1.z);
-                // the same differences as f2_diff, two columns per packed FP32x2 operation
-                const float2 WPH = make_float2(wp.h, wp.h), WPL = make_float2(wp.l, wp.l);
-                const float2 WMH = make_float2(wm.h, wm.h), WML = make_float2(wm.l, wm.l);
-                const float2 N1H = make_float2(a1.z, a1.z), N1L = make_float2(a1.w, a1.w);
-                const float2 HN1 = make_float2(hn1, hn1);
-                float2 acc = make_float2(0.0f, 0.0f);
-                const RowRange rr = row_range(live, wp.h, wm.h);
-                for (int ci = hf; ok && ci < H / 16; ci += NG) {
-                    const int c0 = ci * 16;
-                    if (!chunk_reached<false>(rr, wrange_sm[ci], wide)) continue;       // uniform over the warp
-                    float re[16], im[16];
-                    tmem_ld16x2(taddr + c0, taddr + H + c0, re, im);
-                    if (!live) continue;
+                    const int col = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+                    if ((lane & 3) == 0) colsum[buf][qd][c0 + col] = cv[0];
+                } else {
+                    const float hn1 = 0.5f * (1.0f + a1.z);
+                    const float2 HN1 = make_float2(hn1, hn1);
 #pragma unroll
-                    for (int k = 0; k < 16; k += 2) {
+                    for (int k = 0; k < 8; k += 2) {
                         const int u = (c0 + k) >> 1;
                         const float4 cw = wpk_sm[u], cn = npk_sm[u];
                         const float2 mwh = make_float2(cw.x, cw.y), mwl = make_float2(cw.z, cw.w);
                         const float2 mnh = make_float2(cn.x, cn.y), mnl = make_float2(cn.z, cn.w);
                         const float2 dp = __fadd2_rn(__fadd2_rn(WPH, mwh), __fadd2_rn(WPL, mwl));
                         const float2 dm = __fadd2_rn(__fadd2_rn(WMH, mwh), __fadd2_rn(WML, mwl));
-                        const float2 nd = __fadd2_rn(__fadd2_rn(N1H, mnh), __fadd2_rn(N1L, mnl));   // n' - n''
+                        const float2 mp = make_float2(fabsf(dp.x) < cut ? 1.0f : 0.0f, fabsf(dp.y) < cut ? 1.0f : 0.0f);
+                        const float2 mm = make_float2(fabsf(dm.x) < cut ? 1.0f : 0.0f, fabsf(dm.y) < cut ? 1.0f : 0.0f);
+                        const float2 nd = __fadd2_rn(__fadd2_rn(N2H, mnh), __fadd2_rn(N2L, mnl));   // n' - n''
                         const float2 gc = __ffma2_rn(make_float2(-0.5f, -0.5f), mnh, HN1);          // (1 + n' + n'') / 2
-                        const float2 ep = delta_shape2(dp, x.shape, s2i), em = delta_shape2(dm, x.shape, s2i);
-                        const bool hp0 = fabsf(dp.x) < cut, hp1 = fabsf(dp.y) < cut;
-                        const bool hm0 = fabsf(dm.x) < cut, hm1 = fabsf(dm.y) < cut;
-                        float2 gp = __fmul2_rn(nd, ep), gm = __fmul2_rn(gc, em);
-                        gp.x = hp0 ? gp.x : 0.0f;
-                        gp.y = hp1 ? gp.y : 0.0f;
-                        gm.x = hm0 ? gm.x : 0.0f;
-                        gm.y = hm1 ? gm.y : 0.0f;
+                        const float2 gp = __fmul2_rn(nd, __fmul2_rn(delta_shape2<SHAPE>(dp, s2i), mp));
+                        const float2 gm = __fmul2_rn(gc, __fmul2_rn(delta_shape2<SHAPE>(dm, s2i), mm));
                         const float2 r2 = make_float2(re[k], re[k + 1]), i2 = make_float2(im[k], im[k + 1]);
-                        const float2 p2 = __ffma2_rn(r2, r2, __fmul2_rn(i2, i2));
-                        acc = __ffma2_rn(__fmul2_rn(p2, __fadd2_rn(gp, gm)), iwk_sm[u], acc);
-                        cnt += ((hp0 || hm0) ? 1u : 0u) + ((hp1 || hm1) ? 1u : 0u);
+                        const float2 p2 = live ? __ffma2_rn(r2, r2, __fmul2_rn(i2, i2)) : make_float2(0.0f, 0.0f);
+                        acc1 = __ffma2_rn(__fmul2_rn(p2, __fadd2_rn(gp, gm)), iwk_sm[u], acc1);
+                        cnt2 = __fadd2_rn(cnt2, make_float2(fmaxf(mp.x, mm.x), fmaxf(mp.y, mm.y)));
                     }
                 }
-                rowsum[buf][hf][row] = live ? (acc.x + acc.y) / w1 : 0.0f;
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            rowsum[buf][hf][row] = live ? (acc1.x + acc1.y) / a1.x : 0.0f;              // / w2
+            if constexpr (EPI == EPI_SYM) {
+                rowsum_b[buf][hf][row] = live ? (acc2.x + acc2.y) / a0.x : 0.0f;        // / w1
+                if (hf == 0)                           // columns no row of this quadrant reaches
+                    for (int c = lane; c < H; c += 32)
+                        if (!((chunks >> (c >> 3)) & 1u)) colsum[buf][qd][c] = 0.0f;
+            }
             __syncwarp();
-            if (lane == 0) mbar_arrive(&tempty[buf]);
-            if (EPI != EPI_T) {
-                // per-mode sums over the tile's rows: mode segment j goes to warp
-                // 4 + (j % 4), lanes take rows 32 apart, then a fixed shuffle tree.
-                // (The buffer of this tile parity is rewritten two tiles later,
-                // after the next named barrier.)
-                named_sync(1, NE * 32);
-                if (EPI == EPI_SYM && hf == 0 && ok) {
-                    // position 2: the tile's row sums; position 3: its column sums
-                    if (r < nb * nb) {
-                        float v = 0.0f;
+            if (lane == 0) {
+                mbar_arrive(&tempty[buf]);
+                mbar_arrive(&rfull[buf]);
+            }
+        }
+        // EPI_PHI: the count of -q too, where -q takes q's linewidths;
+        // EPI_SYM: three times the count of the orbit's ordered triples
+        const unsigned long long mult = EPI == EPI_SYM ? (unsigned long long)x.porb[x.pair0 + a]
+                                                       : (unsigned long long)x.qsel[row_of(x, a)].y;
+        unsigned long long c64 = (unsigned long long)(cnt2.x + cnt2.y) * mult;
+        for (int o = 16; o > 0; o >>= 1) c64 += __shfl_xor_sync(0xffffffffu, c64, o);
+        if (lane == 0 && c64) atomicAdd(x.allowed, c64);
+    } else if (EPI != EPI_T) {
+        // ---- warps 2 and 3: the tile's sums, in a fixed order
+        const int rw = warp - 2;
+        for (int i = 0; i < n_tiles; ++i) {
+            const int tile = t0 + i, buf = i & 1;
+            bool ok = !*(volatile int *)&fail_sm && mbar_wait(&rfull[buf], (i >> 1) & 1, x.wait_limit);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) {
+                fail_sm = 1;
+                break;
+            }
+            const int rt = tile * kBM, re = min(nb * nb, rt + kBM);
+            if (EPI == EPI_SYM) {
+                // position 2: the tile's row sums; position 3: its column sums
+                for (int row = rw * 64 + lane; row < rw * 64 + 64; row += 32) {
+                    if (rt + row >= re) continue;
+                    float v = 0.0f;
 #pragma unroll
-                        for (int gq = 0; gq < NG; ++gq) v += rowsum_b[buf][gq][row];
-                        x.rbuf[(size_t)a * x.Mp + r] = v;
-                    }
-                    if (row < nb) {
-                        const float v = ((colsum[buf][0][row] + colsum[buf][1][row]) + colsum[buf][2][row]) +
-                                        colsum[buf][3][row];
-                        x.cbuf[((size_t)a * mt + tile) * nb + row] = v;
-                    }
+                    for (int gq = 0; gq < NG; ++gq) v += rowsum_b[buf][gq][row];
+                    x.rbuf[(size_t)a * x.Mp + rt + row] = v;
                 }
-                if (hf == 0 && ok) {
-                    const int rt = tile * kBM, re = min(nb * nb, rt + kBM);
-                    if (rt < re) {
-                        const int s_lo = rt / nb, s_hi = (re - 1) / nb;
-                        float *sl = EPI == EPI_SYM ? x.slots + (size_t)a * nb * 2
-                                                   : x.slots + ((size_t)(row_of(x, a) % x.n_slices) * x.nq + qp) * nb * 2;
-                        for (int sm = s_lo + qd; sm <= s_hi; sm += 4) {
-                            const int b0 = max(rt, sm * nb), b1 = min(re, (sm + 1) * nb);
-                            float v = 0.0f;
-                            for (int rr = b0 + lane; rr < b1; rr += 32)
+                for (int c = rw * 48 + lane; c < min(nb, rw * 48 + 48); c += 32)
+                    x.cbuf[((size_t)a * mt + tile) * nb + c] =
+                        ((colsum[buf][0][c] + colsum[buf][1][c]) + colsum[buf][2][c]) + colsum[buf][3][c];
+            }
+            // per-mode sums over the tile's rows: mode segment j goes to warp 2 + (j % 2),
+            // lanes take rows 32 apart, then a fixed shuffle tree
+            if (rt < re) {
+                const int s_lo = rt / nb, s_hi = (re - 1) / nb;
+                float *sl = EPI == EPI_SYM ? x.slots + (size_t)a * nb * 2
+                                           : x.slots + ((size_t)(row_of(x, a) % x.n_slices) * x.nq + qp) * nb * 2;
+                for (int sm = s_lo + rw; sm <= s_hi; sm += 2) {
+                    const int b0 = max(rt, sm * nb), b1 = min(re, (sm + 1) * nb);
+                    float v = 0.0f;
+                    for (int r2 = b0 + lane; r2 < b1; r2 += 32)
 #pragma unroll
-                                for (int gq = 0; gq < NG; ++gq) v += rowsum[buf][gq][rr - rt];
-                            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                            if (lane == 0) {
-                                const bool first = b0 == sm * nb;
-                                sl[2 * sm + (first ? 0 : 1)] = v;
-                                if (first && b1 == (sm + 1) * nb) sl[2 * sm + 1] = 0.0f;   // no continuation
-                            }
-                        }
+                        for (int gq = 0; gq < NG; ++gq) v += rowsum[buf][gq][r2 - rt];
+                    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                    if (lane == 0) {
+                        const bool first = b0 == sm * nb;
+                        sl[2 * sm + (first ? 0 : 1)] = v;
+                        if (first && b1 == (sm + 1) * nb) sl[2 * sm + 1] = 0.0f;   // no continuation
                     }
                 }
             }
-        }
-        if (EPI != EPI_T) {
-            // EPI_PHI: the count of -q too, where -q takes q's linewidths;
-            // EPI_SYM: three times the count of the orbit's ordered triples
-            const unsigned long long mult = EPI == EPI_SYM ? (unsigned long long)x.porb[x.pair0 + a]
-                                                           : (unsigned long long)x.qsel[row_of(x, a)].y;
-            unsigned long long c64 = (unsigned long long)cnt * mult;
-            for (int o = 16; o > 0; o >>= 1) c64 += __shfl_xor_sync(0xffffffffu, c64, o);
-            if (lane == 0 && c64) atomicAdd(x.allowed, c64);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&rfree[buf]);
         }
     }
     __syncthreads();
@@ -1238,13 +1255,13 @@ size_t tcx_y_bytes(int nb, int n_rep) {
 }
 bool tcx_y_fits(int nb, int n_rep) { return nb % 3 == 0 && tcx_y_bytes(nb, n_rep) <= kSmemOptin; }
 
-template <int BN, int PB>
+template <int BN, int PB, int SHAPE>
 cudaError_t run_batches(const LwParams &p, const LwDev &d, const TcxGroups &g, Lane *lanes, TcxSched sc,
                         long long pbeg, long long pend, bool reduce, double *gacc, int *err, float *out3) {
     const int batch = sc.batch, tpc = sc.tpc;
     const bool sym = lanes[0].x.plist != nullptr;
-    auto k1 = tcx_gemm_kernel<EPI_T, BN, PB>;
-    auto k2 = sym ? tcx_gemm_kernel<EPI_SYM, BN, PB> : tcx_gemm_kernel<EPI_PHI, BN, PB>;
+    auto k1 = tcx_gemm_kernel<EPI_T, BN, PB, 0>;
+    auto k2 = sym ? tcx_gemm_kernel<EPI_SYM, BN, PB, SHAPE> : tcx_gemm_kernel<EPI_PHI, BN, PB, SHAPE>;
     constexpr int smem = Cfg<BN, PB>::kSmem;
     cudaError_t e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -1641,7 +1658,9 @@ cudaError_t launch_lw_tensor(const LwParams &p, const LwDev &d, const TcxGroups 
         lanes[0].st = st; lanes[0].done[0] = ev[0]; lanes[0].done[1] = ev[1];
         lanes[1].st = aux; lanes[1].done[0] = ev[2]; lanes[1].done[1] = ev[3];
         auto run = [&](TcxSched sc, long long b0, long long b1, bool reduce) -> cudaError_t {
-            return run_batches<192, 2>(p, d, g, lanes, sc, b0, b1, reduce, gacc, err, out3);
+            return p.shape == kDeltaGauss     ? run_batches<192, 2, kDeltaGauss>(p, d, g, lanes, sc, b0, b1, reduce, gacc, err, out3)
+                   : p.shape == kDeltaLorentz ? run_batches<192, 2, kDeltaLorentz>(p, d, g, lanes, sc, b0, b1, reduce, gacc, err, out3)
+                                              : run_batches<192, 2, kDeltaTriangle>(p, d, g, lanes, sc, b0, b1, reduce, gacc, err, out3);
         };
         // pairs of the projected q-points, or the orbit pairs
         const long long pbeg = 0, pend = sym ? (long long)sym->n_pairs : (long long)p.nqc * nq;

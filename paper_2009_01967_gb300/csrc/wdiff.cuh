@@ -61,19 +61,30 @@ __device__ __forceinline__ float delta_shape(float d, int shape, float a) {
     if (shape == kDeltaLorentz) return 1.0f / fmaf(d * d, a, 1.0f);
     return fmaxf(0.0f, 1.0f - fabsf(d) * a);
 }
-// The same on a pair of values (packed FP32x2 arithmetic; per component the
-// operations and their rounding are those of delta_shape).
-__device__ __forceinline__ float2 delta_shape2(float2 d, int shape, float a) {
+// The same on a pair of values for a shape fixed at compile time (packed FP32x2
+// arithmetic, no branch between the columns of an epilogue); a from
+// delta_param2: the Gaussian's carries log2 e, so that the exponential is one
+// ex2 (one rounding less than exp).
+__device__ __forceinline__ float ex2_approx(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float delta_param2(int shape, float a) {
+    return shape == kDeltaGauss ? a * 1.44269504088896340736f : a;
+}
+template <int SHAPE>
+__device__ __forceinline__ float2 delta_shape2(float2 d, float a) {
+    if constexpr (SHAPE == kDeltaTriangle)
+        return make_float2(fmaxf(0.0f, 1.0f - fabsf(d.x) * a), fmaxf(0.0f, 1.0f - fabsf(d.y) * a));
     const float2 d2 = __fmul2_rn(d, d);
-    if (shape == kDeltaGauss) {
+    if constexpr (SHAPE == kDeltaGauss) {
         const float2 x = __fmul2_rn(d2, make_float2(-a, -a));
-        return make_float2(__expf(x.x), __expf(x.y));
-    }
-    if (shape == kDeltaLorentz) {
+        return make_float2(ex2_approx(x.x), ex2_approx(x.y));
+    } else {
         const float2 x = __ffma2_rn(d2, make_float2(a, a), make_float2(1.0f, 1.0f));
         return make_float2(1.0f / x.x, 1.0f / x.y);
     }
-    return make_float2(fmaxf(0.0f, 1.0f - fabsf(d.x) * a), fmaxf(0.0f, 1.0f - fabsf(d.y) * a));
 }
 __device__ __forceinline__ double delta_shape(double d, int shape, double a) {
     if (shape == kDeltaGauss) return exp(-d * d * a);
