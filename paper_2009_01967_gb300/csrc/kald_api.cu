@@ -1231,6 +1231,7 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
             return st;
     }
     size_t off_nb = 0, off_eig = 0;
+    int lean = 0;            // where the workspace cannot be had: 1 without tables, 2 without orbits as well
     for (int x = 0; x < n_sys; ++x) {
         std::shared_ptr<const HostSystem> hp;
         if ((st = plan_system_cached(ctx, &sys[x], hp))) return st;
@@ -1338,7 +1339,7 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
             }
         }
         // the register kernel's blocks by class and atom triple, and its tables of
-        // phase sums while they stay within 16 GB and the context's limit (the
+        // phase sums while they stay within 16 GB and what the context may take (the
         // kernel sums every block per pair without them)
         std::vector<int> sn_kk, sn_start, sn_atoms;
         std::vector<int4> sn_bj, sn_bk;
@@ -1346,7 +1347,7 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         size_t sn_tab = 0;
         if (small) {
             sn_tab = sn_table_bytes(nb, nq, f32w);
-            if (sn_tab > (size_t(16) << 30) || (ctx->ws_limit && sn_tab > ctx->ws_limit / 2)) sn_tab = 0;
+            if (lean || sn_tab > (size_t(16) << 30)) sn_tab = 0;
             std::vector<int> order;
             plan_sn(h, sn_tab != 0, order, sn_start);
             sn_kk.resize(3 * (size_t)nq);
@@ -1370,7 +1371,7 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         // permutations: one projection per orbit of momentum triples
         int orb_pairs = 0;
         std::vector<int> orb_rows;
-        if (!small && !listed && reuse && opt->symmetry == KALD_SYM_ALL && nq > 1) {
+        if (!small && !listed && reuse && opt->symmetry == KALD_SYM_ALL && nq > 1 && lean < 2) {
             if (h.fc3_perm_symmetric < 0) h.fc3_perm_symmetric = fc3_symmetric_all(&sys[x]) ? 1 : 0;
             if (h.fc3_perm_symmetric) orb_pairs = std::max(0, orbit_pairs(mesh));
             if (orb_pairs) {
@@ -1383,13 +1384,10 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         // tensor-core path: the fc3 blocks in (j, k) group order, the groups
         // split over the gather CTAs
         std::vector<int2> tc_gjk;
-        std::vector<int> tc_part_start, tc_glist;
         if (tcx) {
             const int n_groups = (int)h.pair3_j.size();
             tc_gjk.resize(std::max(1, n_groups));
             for (int g = 0; g < n_groups; ++g) tc_gjk[g] = make_int2(h.pair3_j[g], h.pair3_k[g]);
-            plan_tcx_parts(h, tcx_parts(n_groups), tc_part_start, tc_glist);
-            if (tc_glist.empty()) tc_glist.push_back(0);
         }
         // tensor-core phase sum: the blocks of each group ordered by the home atom i
         std::vector<double> y_blk;
@@ -1418,24 +1416,47 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
                 while (at <= y_n_at) y_gi[(size_t)g * (y_n_at + 1) + at++] = b1;
             }
         }
-        // CUDA-core kernel: terms and tables of its phase sums (tables within 16 GB
-        // and half of the context's limit), and one projection per orbit of momentum
-        // triples over the whole mesh when Phi3 is symmetric under permutations
+        // terms and tables of the phase sums (the CUDA-core kernel and the tensor-core
+        // path's gather), the tables within 16 GB and what the context may take
         const bool cc = !small && !tcx;
-        LwTermsHost lt;
+        std::shared_ptr<const LwTermsHost> ltp;
+        std::shared_ptr<const TcxPlanHost> tpp;
         size_t lw_tab[3] = {0, 0, 0};
-        if (cc) {
-            plan_lw_terms(h, true, lt);
+        size_t tc_yc = 0;
+        auto terms_of = [&](bool tables) {
+            auto n = std::make_shared<LwTermsHost>();
+            plan_lw_terms(h, tables, *n);
+            return n;
+        };
+        if (!small) {
+            if (!h.lw_terms) h.lw_terms = terms_of(true);      // with the system's plan
+            ltp = h.lw_terms;
             size_t all = 0;
             for (int c = 0; c < 3; ++c) {
-                lw_tab[c] = (f32w ? sizeof(float2) : sizeof(double2)) * 27 * (size_t)lt.n_slot[c] * nq;
+                lw_tab[c] = (f32w ? sizeof(float2) : sizeof(double2)) * 27 * (size_t)ltp->n_slot[c] * nq;
                 all += lw_tab[c];
             }
-            if (all > (size_t(16) << 30) || (ctx->ws_limit && all > ctx->ws_limit / 2)) {
-                plan_lw_terms(h, false, lt);
+            if (tcx) all += sizeof(float2) * 9 * (size_t)nq * nb * std::min<size_t>(ltp->n_slot[2] / 3, h.pair3_j.size());
+            if (lean || all > (size_t(16) << 30)) {
+                ltp = terms_of(false);
                 lw_tab[0] = lw_tab[1] = lw_tab[2] = 0;
             }
         }
+        if (tcx) {
+            if (ltp != h.lw_terms || !h.tcx_plan) {
+                auto n = std::make_shared<TcxPlanHost>();
+                plan_tcx_gather(h, *ltp, *n);
+                if (ltp == h.lw_terms) h.tcx_plan = n;
+                tpp = n;
+            } else {
+                tpp = h.tcx_plan;
+            }
+            tc_yc = sizeof(float2) * 9 * (size_t)nq * nb * (tpp->cterm_start.size() - 1);
+        }
+        const LwTermsHost no_terms;
+        const TcxPlanHost no_plan;
+        const LwTermsHost &lt = ltp ? *ltp : no_terms;
+        const TcxPlanHost &tp = tpp ? *tpp : no_plan;
         size_t cc_out3 = 0, cc_sums = 0;         // position sums of the mode blocks, and where their totals start
         if (cc_pairs) {
             const int blocks = lw_orbit_blocks(nb, cc_pairs, f32w, ctx->sm_count, ctx->smem_optin);
@@ -1460,19 +1481,28 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         if (!d_g) need += ws_round(sizeof(double) * nqr * nb);
         if (f32w) need += ws_round(sizeof(float4) * (size_t)nq * nb);
         if (tcx)
-            need += ws_round(tcx_scratch_bytes(nb, nq, tcx_b)) + ws_round(16) + bytes_of(tc_gjk) +
-                    bytes_of(tc_part_start) + bytes_of(tc_glist) + bytes_of(h.pair3_start);
+            need += ws_round(tcx_scratch_bytes(nb, nq, tcx_b)) + ws_round(16) + bytes_of(tc_gjk);
         if (use_sym) need += ws_round(tcx_sym_bytes(nb, tcx_b, orb_pairs));
         if (!y_blk.empty())
             need += scaled_bytes(y_blk, y_atoms, h, 27, 28, 1) + bytes_of(y_gi) + bytes_of(y_rep);
         if (small)
             need += bytes_of(sn_kk) + bytes_of(sn_bj) + bytes_of(sn_bk) + bytes_of(sn_start) +
                     ws_round(sizeof(double2) * (2 * (size_t)sn_m0 + 1)) + ws_round(sn_tab);
-        if (cc)
-            need += bytes_of(lt.group) + bytes_of(lt.term_start) + bytes_of(lt.term) + bytes_of(lt.slot_start) +
-                    bytes_of(lt.slot_blk) + ws_round(lw_tab[0]) + ws_round(lw_tab[1]) + ws_round(lw_tab[2]);
+        if (!small)
+            need += (cc ? bytes_of(lt.group) + bytes_of(lt.term_start) + bytes_of(lt.term) : 0) +
+                    bytes_of(lt.slot_start) + bytes_of(lt.slot_blk) + ws_round(lw_tab[0]) + ws_round(lw_tab[1]) + ws_round(lw_tab[2]);
+        if (tcx)
+            need += bytes_of(tp.term_start) + bytes_of(tp.list_start) + bytes_of(tp.glist) + bytes_of(tp.blk) +
+                    bytes_of(tp.term) + bytes_of(tp.cterm_start) + bytes_of(tp.cterm) +
+                    ws_round(tc_yc);
         if (orb_pairs) need += bytes_of(orb_rows) + ws_round(orbit_bytes(mesh, nqc)) + ws_round(sizeof(double) * cc_out3);
-        if ((st = ws_reserve(ctx, need))) return st;
+        if ((st = ws_reserve(ctx, need))) {
+            if (st != KALD_E_NOMEM || lean == 2) return st;
+            ++lean;
+            --x;
+            continue;
+        }
+        lean = 0;
         LwDev d;
         d.blkinfo = upload(ctx, binfo);
         // Phi3 / sqrt(mi mj mk), 28 values per block (16-byte loads), in the working precision
@@ -1505,16 +1535,15 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         TcxGroups tg;
         if (tcx) {
             tg.n_groups = (int)h.pair3_j.size();
-            tg.n_parts = (int)tc_part_start.size() - 1;
-            for (int x = 0; x < tg.n_parts; ++x) {
-                int nbk = 0;
-                for (int gi = tc_part_start[x]; gi < tc_part_start[x + 1]; ++gi)
-                    nbk += h.pair3_start[tc_glist[gi] + 1] - h.pair3_start[tc_glist[gi]];
-                tg.max_part_blocks = std::max(tg.max_part_blocks, nbk);
-            }
-            tg.part_start = upload(ctx, tc_part_start);
-            tg.glist = upload(ctx, tc_glist);
-            tg.gstart = upload(ctx, h.pair3_start);
+            tg.term_start = upload(ctx, tp.term_start);
+            tg.list_start = upload(ctx, tp.list_start);
+            tg.glist = upload(ctx, tp.glist);
+            tg.tblk = upload(ctx, tp.blk);
+            tg.term = upload(ctx, tp.term);
+            tg.n_cg = (int)tp.cterm_start.size() - 1;
+            tg.cterm_start = upload(ctx, tp.cterm_start);
+            tg.cterm = upload(ctx, tp.cterm);
+            tg.yc = static_cast<float2 *>(ws_take(ctx, tc_yc));
             tg.gjk = upload(ctx, tc_gjk);
             tg.blkinfo = d.blkinfo;               // group order (HostSystem order)
             tg.fc3 = static_cast<const float *>(d.fc3);
@@ -1542,10 +1571,12 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         LwTerms terms;
         OrbitPlan orb;
         cudaError_t e = cudaSuccess;
-        if (cc) {
-            terms.group = upload(ctx, lt.group);
-            terms.term_start = upload(ctx, lt.term_start);
-            terms.term = upload(ctx, lt.term);
+        if (!small) {
+            if (cc) {
+                terms.group = upload(ctx, lt.group);
+                terms.term_start = upload(ctx, lt.term_start);
+                terms.term = upload(ctx, lt.term);
+            }
             terms.slot_start = upload(ctx, lt.slot_start);
             terms.slot_blk = upload(ctx, lt.slot_blk);
             for (int c = 0; c < 3; ++c) {
@@ -1566,6 +1597,14 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
             terms.orbit = orb.orbit;
         }
         if (e == cudaSuccess) e = launch_lw_prep(p, d, f32w, s);
+        if (tcx) {
+            for (int c = 0; c < 3; ++c) {
+                tg.tab[c] = static_cast<const float2 *>(terms.tab[c]);
+                tg.n_slot[c] = terms.n_slot[c];
+            }
+            if (e == cudaSuccess)
+                e = launch_lw_tables_f32(nq, p.n_rep, terms, d.blkinfo, tg.fc3, static_cast<const float2 *>(d.chi), s);
+        }
         if (e == cudaSuccess)
             e = small ? launch_lw_small(p, d, sn, f32w, s)
                 : tcx ? launch_lw_tensor(p, d, tg, tc_scr, tcx_b, ctx->sm_count, tc_err, s,

@@ -123,6 +123,8 @@ bool is_device_ptr(const void *p);
 constexpr int kYLong = 8;
 
 // ---- host-side plan of a system ---------------------------------------------
+struct LwTermsHost;
+struct TcxPlanHost;
 struct HostSystem {
     int n_atoms = 0;
     int nb = 0;
@@ -153,6 +155,8 @@ struct HostSystem {
     int n_rep = 0;
     mutable int fc3_symmetric = -1;                    // Phi3 symmetric in its last two indices (lazy)
     mutable int fc3_perm_symmetric = -1;               // ... under every permutation of its indices (lazy)
+    mutable std::shared_ptr<const LwTermsHost> lw_terms;   // plan_lw_terms with tables (lazy)
+    mutable std::shared_ptr<const TcxPlanHost> tcx_plan;   // plan_tcx_gather of those terms (lazy)
 };
 
 // Validate and plan one kald_system (host).  Returns KALD_OK or an error.
@@ -316,6 +320,8 @@ struct LwTerms {
 };
 int lw_orbit_blocks(int nb, int n_pairs, int fp32, int sm_count, size_t smem_optin);
 void plan_lw_terms(const HostSystem &h, bool tables, LwTermsHost &o);
+cudaError_t launch_lw_tables_f32(int nq, int n_rep, const LwTerms &t, const int4 *blkinfo, const float *fc3,
+                                 const float2 *chi, cudaStream_t st);
 cudaError_t launch_lw_prep(const LwParams &p, const LwDev &d, int fp32, cudaStream_t st);
 cudaError_t launch_lw_main(const LwParams &p, const LwDev &d, const LwTerms &t, int fp32, int sm_count,
                            size_t smem_optin, cudaStream_t st);
@@ -395,7 +401,7 @@ cudaError_t launch_lw_small(const LwParams &p, const LwDev &d, const SnTables &t
 
 // tc_crystal.cu: crystal linewidth sums on tensor cores (BF16 split, nb <= 96).
 // The gather runs over the fc3 blocks grouped by (j, k) atom pair (the order
-// of HostSystem), the groups split over CTAs by plan_tcx_parts.
+// of HostSystem), the groups dealt to the gather's warps by plan_tcx_gather.
 // Tables of the tensor-core phase sum (tcx_y_kernel): the fc3 blocks of each
 // (j, k) group ordered by the home atom i.
 struct TcxYTables {
@@ -408,23 +414,37 @@ struct TcxYTables {
 };
 struct TcxGroups {
     TcxYTables y;                     // the same blocks for the tensor-core phase sum
-    int n_groups = 0, n_parts = 0;
-    int max_part_blocks = 0;          // most fc3 blocks in one part (shared-memory staging)
-    const int *part_start = nullptr;  // [n_parts + 1] into glist
-    const int *glist = nullptr;       // group ids, part by part
-    const int *gstart = nullptr;      // [n_groups + 1] blocks of each group (CSR)
+    int n_groups = 0;
     const int2 *gjk = nullptr;        // [n_groups] atoms (j, k)
     const int4 *blkinfo = nullptr;    // [n_fc3] (i, rep(Rj), rep(Rk), 0), group order
     const float *fc3 = nullptr;       // [n_fc3][28] Phi3 / sqrt(mi mj mk), FP32, padded
+    const float2 *tab[3] = {nullptr, nullptr, nullptr};   // [nq][n_slot][27] phase sums per class
+    int n_slot[3] = {0, 0, 0};
+    // the gather's lists: see TcxPlanHost
+    const int *term_start = nullptr, *list_start = nullptr, *glist = nullptr, *tblk = nullptr;
+    const int4 *term = nullptr;
+    int n_cg = 0;
+    const int *cterm_start = nullptr;
+    const int2 *cterm = nullptr;
+    float2 *yc = nullptr;             // [nq][n_cg][9][nb]
 };
+// Lists of the gather.  Terms of list x: term[term_start[x]..], each (i, class, slot
+// or start in blk, blocks), class 0..2 (a table's slot), 3 (blocks blk[..]) or 4
+// (nothing to add), plus 8 at the last term of a group; the list's groups in order:
+// glist[list_start[x]..], each j + (k << 8) + ((c + 1) << 16), c the index of the group
+// among those with many class-2 terms (-1: not one of them); cterm (i, slot) their terms.
+struct TcxPlanHost {
+    std::vector<int> term_start, list_start, glist, blk, cterm_start;
+    std::vector<int4> term;
+    std::vector<int2> cterm;
+};
+void plan_tcx_gather(const HostSystem &h, const LwTermsHost &lt, TcxPlanHost &o);
 bool tcx_y_wanted(size_t n_fc3, size_t n_groups);   // the phase sum on tensor cores is considered
 size_t tcx_sym_bytes(int nb, int batch, int n_pairs);
 bool tcx_supported(int nb);           // 65 <= nb <= 96 (one tile width, N = K = 192)
 int tcx_half(int nb);
 int tcx_batch(int nb, int nq, int sm_count);
 int tcx_batch_max(int nb, int nq, int sm_count);
-int tcx_parts(int n_groups);
-void plan_tcx_parts(const HostSystem &h, int n_parts, std::vector<int> &part_start, std::vector<int> &glist);
 size_t tcx_scratch_bytes(int nb, int nq, int batch);
 cudaError_t launch_lw_tensor(const LwParams &p, const LwDev &d, const TcxGroups &g, void *scratch, int batch,
                              int sms, int *err, cudaStream_t st, const OrbitPlan *sym = nullptr,

@@ -857,6 +857,20 @@ cudaError_t launch_lw_prep(const LwParams &p, const LwDev &d, int fp32, cudaStre
     return cudaGetLastError();
 }
 
+template <typename R>
+static void run_lw_tables(int nq, int n_rep, const LwTerms &t, const int4 *blkinfo, const R *fc3,
+                          const typename C2<R>::T *chi, cudaStream_t st) {
+    const size_t nt = (size_t)std::max({t.n_slot[0], t.n_slot[1], t.n_slot[2]}) * 27 * nq;
+    if (nt)
+        lw_tables_kernel<R><<<counted((unsigned)std::min<size_t>((nt + 255) / 256, 16384)), 256, 0, st>>>(nq, n_rep, t,
+                                                                                                         blkinfo, fc3, chi);
+}
+cudaError_t launch_lw_tables_f32(int nq, int n_rep, const LwTerms &t, const int4 *blkinfo, const float *fc3,
+                                 const float2 *chi, cudaStream_t st) {
+    run_lw_tables<float>(nq, n_rep, t, blkinfo, fc3, chi, st);
+    return cudaGetLastError();
+}
+
 // Modes per pass and threads of a CTA: up to 256 threads, and two CTAs per SM in
 // shared memory where several modes run side by side.
 template <typename R>
@@ -899,10 +913,7 @@ static cudaError_t run_lw_main(const LwParams &p, const LwDev &d, LwTerms t, int
     int per_sm = 1;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, nthr, smem);
     if (e != cudaSuccess) return e;
-    const size_t nt = (size_t)std::max({t.n_slot[0], t.n_slot[1], t.n_slot[2]}) * 27 * p.nq;
-    if (nt)
-        lw_tables_kernel<R><<<counted((unsigned)std::min<size_t>((nt + 255) / 256, 16384)), 256, 0, st>>>(
-            p.nq, p.n_rep, t, d.blkinfo, static_cast<const R *>(d.fc3), static_cast<const R2 *>(d.chi));
+    run_lw_tables<R>(p.nq, p.n_rep, t, d.blkinfo, static_cast<const R *>(d.fc3), static_cast<const R2 *>(d.chi), st);
     const int n_batch = (p.nb + sb - 1) / sb;
     t.n_sblk = ORBIT ? lw_mode_blocks(p.nb, sb, t.n_pairs, sm_count)
                      : lw_mode_blocks(p.nb, sb, (long long)(p.nq / 2 + 1) * p.n_chunks, sm_count);
@@ -947,12 +958,25 @@ void plan_lw_terms(const HostSystem &h, bool tables, LwTermsHost &o) {
     for (int g = 0; g < ng; ++g) {
         o.group[(size_t)h.pair3_j[g] * na + h.pair3_k[g]] = g;
         std::vector<std::array<int, 3>> key;              // (class, i, block), the blocks of a slot in order
-        for (int b = h.pair3_start[g]; b < h.pair3_start[g + 1]; ++b) {
-            const int *rj = &h.rep_int[3 * (size_t)h.fc3_rj[b]], *rk = &h.rep_int[3 * (size_t)h.fc3_rk[b]];
-            const bool zj = !rj[0] && !rj[1] && !rj[2], zk = !rk[0] && !rk[1] && !rk[2];
-            const int cls = !tables ? 3 : zk ? 0 : zj ? 1 : h.fc3_rj[b] == h.fc3_rk[b] ? 2 : 3;
-            key.push_back({cls, h.fc3_i[b], b});
-        }
+        std::vector<unsigned char> has(na, 0);            // classes in use, per i
+        for (int pass = 0; pass < 2; ++pass)
+            for (int b = h.pair3_start[g]; b < h.pair3_start[g + 1]; ++b) {
+                const int *rj = &h.rep_int[3 * (size_t)h.fc3_rj[b]], *rk = &h.rep_int[3 * (size_t)h.fc3_rk[b]];
+                const bool zj = !rj[0] && !rj[1] && !rj[2], zk = !rk[0] && !rk[1] && !rk[2];
+                const int i = h.fc3_i[b];
+                // a block with both at home has no phase: it joins a slot of its (i, j, k)
+                // where there is one (class 2 where there is none and j = k: those blocks
+                // are the ones that take many i)
+                if (tables && pass == (zj && zk ? 0 : 1)) continue;
+                if (!tables && pass) continue;
+                const int cls = !tables      ? 3
+                                : zj && zk   ? (has[i] & 1 ? 0 : has[i] & 2 ? 1 : has[i] & 4 || h.pair3_j[g] == h.pair3_k[g] ? 2 : 0)
+                                : zk         ? 0
+                                : zj         ? 1
+                                : h.fc3_rj[b] == h.fc3_rk[b] ? 2 : 3;
+                has[i] |= cls < 3 ? 1 << cls : 0;
+                key.push_back({cls, i, b});
+            }
         std::sort(key.begin(), key.end());
         for (size_t x = 0; x < key.size(); ++x) {
             const int cls = key[x][0], i = key[x][1], b = key[x][2];

@@ -1,7 +1,7 @@
 // Orbits of momentum triples (q1, q2, q3), q1 + q2 + q3 = 0 on the mesh, under
 // the six permutations and inversion, enumerated on the GPU, and the sums of the
 // linewidths from one projection per orbit (Eq. gamma_operators with Phi3
-// symmetric under permutations; see TcxSymHost's formulas in tc_crystal.cu).
+// symmetric under permutations).
 //
 // An orbit is represented by its lexicographically smallest ordered triple; its
 // first member is then the lower index of a pair {q, -q} (a row).  Rows keep a

@@ -20,8 +20,8 @@
 //     |phi|^2 / (w' w'') [ (n' - n'') G(w + w' - w'') + 1/2 (1 + n' + n'') G(w - w' - w'') ]
 //   with the same FP32 window test and Gaussian as the CUDA-core kernel, the
 //   energy and occupation differences formed from FP32 pairs (wdiff.cuh).
-// A1 and T1 are stored MN-major (rows contiguous), so the gather (one thread
-// per mode s) and the GEMM1 epilogue (32 consecutive s' per thread) write
+// A1 and T1 are stored MN-major (rows contiguous), so the gather (lanes over the
+// modes s) and the GEMM1 epilogue (32 consecutive s' per thread) write
 // whole runs; the B operands are K-major.  GEMM2's epilogue sums each mode's
 // rows (s, s') of a tile in a fixed order (FP32) into one of two slots per
 // (pair, mode); a mode spans at most two tiles (nb <= 96).  Once every pair
@@ -650,122 +650,200 @@ tcx_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__
     }
 }
 
-// Phase-summed contraction over the home index (gather), CTA = (group part,
-// P consecutive pairs of the batch with the same q), thread = mode s of q:
-//   Y_s(3j + beta, 3k + gamma) = sum over the blocks (i; j Rj; k Rk) of the
-//     atom pair (j, k) of sum_alpha Phi3~[alpha beta gamma] eps_{3i+alpha}(q s)
-//     chi(q', Rj) conj(chi(q'', Rk)),
-// in FP32; a block (the same address in all lanes) and eps(q) are read once
-// for the P pairs, which differ only in the phase.  Y is written to A1 as
-// BF16 hi/lo: for a fixed (b, c) the lanes of a warp cover consecutive rows
-// m = c nb + s.
-template <int P>
+// Zeros into the entries of the operand planes (plane apart by `stride`; [batch][Kp][Mp]
+// each) that no pair writes: rows nb.. of both halves, columns nb nb.. of the others.
+// One CTA per row.  (Clearing the planes whole took 0.64 ms of a 3.75 ms call on 4^3.)
 __global__ void __launch_bounds__(128)
-ycx_gather_kernel(XParams x, TcxGroups g, const float2 *__restrict__ epsT_all,
-                  const float2 *__restrict__ chi_all, int n_rep, __nv_bfloat16 *__restrict__ a1h,
-                  __nv_bfloat16 *__restrict__ a1l) {
-    // shared memory: the part's blocks (7 float4 of Phi3 + one int4 each, in
-    // processing order), then chi(q', R), chi(q'', R) of the P pairs
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    float4 *f_sm = reinterpret_cast<float4 *>(smem_raw);
-    int4 *b_sm = reinterpret_cast<int4 *>(f_sm + 7 * (size_t)g.max_part_blocks);
-    float2 *chi_sm = reinterpret_cast<float2 *>(b_sm + g.max_part_blocks);
-    const int part = blockIdx.x, a0 = blockIdx.y * P;
-    int q = 0;
-    for (int p = 0; p < P; ++p) {
-        int qp, qpp;
-        pair_of(x, a0 + p, q, qp, qpp);
-        for (int t = threadIdx.x; t < n_rep; t += blockDim.x) {
-            chi_sm[(2 * p) * n_rep + t] = chi_all[(size_t)qp * n_rep + t];
-            chi_sm[(2 * p + 1) * n_rep + t] = chi_all[(size_t)qpp * n_rep + t];
-        }
+clear_padding_kernel(int nb, int H, int Mp, size_t stride, __nv_bfloat16 *__restrict__ planes) {
+    const int r = blockIdx.x;
+    __nv_bfloat16 *row = planes + blockIdx.z * stride + ((size_t)blockIdx.y * 2 * H + r) * Mp;
+    const bool pad = (r < H ? r : r - H) >= nb;
+    if (pad) {
+        for (int t = threadIdx.x; t < Mp / 8; t += blockDim.x) reinterpret_cast<uint4 *>(row)[t] = make_uint4(0, 0, 0, 0);
+    } else {
+        for (int t = nb * nb + threadIdx.x; t < Mp; t += blockDim.x) row[t] = __float2bfloat16_rn(0.f);
     }
-    {
-        int off = 0;
-        for (int gi = g.part_start[part]; gi < g.part_start[part + 1]; ++gi) {
-            const int gr = g.glist[gi];
-            const int b0 = g.gstart[gr], n = g.gstart[gr + 1] - b0;
-            const float4 *src = reinterpret_cast<const float4 *>(g.fc3) + 7 * (size_t)b0;
-            for (int t = threadIdx.x; t < 7 * n; t += blockDim.x) f_sm[7 * (size_t)off + t] = __ldg(src + t);
-            for (int t = threadIdx.x; t < n; t += blockDim.x) b_sm[off + t] = __ldg(g.blkinfo + b0 + t);
-            off += n;
-        }
-    }
-    __syncthreads();
-    const int nb = x.nb, s = threadIdx.x;
+}
+
+// Y_s(3j + beta, 3k + gamma) of the class-2 terms (blocks with Rj = Rk, whose phase
+// depends on q alone) for the projected q-points: yc[q][c][9][nb], c the index of
+// the group among those with such terms.  One thread per mode.
+__global__ void __launch_bounds__(96)
+ycx_same_kernel(int nb, int nq, TcxGroups g, const int2 *__restrict__ qsel, const float2 *__restrict__ epsT_all) {
+    const int c = blockIdx.y, q = qsel ? qsel[blockIdx.x].x : blockIdx.x, s = threadIdx.x;
     if (s >= nb) return;
-    const float2 *eps = epsT_all + (size_t)q * nb * nb;      // eps(q)(row, s) at row * nb + s
-    int lb = 0;                                    // block index in shared memory
-    for (int gi = g.part_start[part]; gi < g.part_start[part + 1]; ++gi) {
-        const int gr = g.glist[gi];
-        const int2 jk = g.gjk[gr];
-        const int lb_end = lb + g.gstart[gr + 1] - g.gstart[gr];
-        float2 acc[P][9];
+    const float2 *eps = epsT_all + (size_t)q * nb * nb + s;
+    const float2 *tab = g.tab[2] + (size_t)q * g.n_slot[2] * 27;
+    float2 acc[9];
 #pragma unroll
-        for (int p = 0; p < P; ++p)
+    for (int e = 0; e < 9; ++e) acc[e] = make_float2(0.f, 0.f);
+    for (int t = g.cterm_start[c]; t < g.cterm_start[c + 1]; ++t) {
+        const int2 tm = __ldg(g.cterm + t);                    // (i, slot)
 #pragma unroll
-            for (int t = 0; t < 9; ++t) acc[p][t] = make_float2(0.f, 0.f);
-        // the next block's indices and eps row are loaded one block ahead
-        int4 bi_n = make_int4(0, 0, 0, 0);
-        float2 u_n[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-        if (lb < lb_end) {
-            bi_n = b_sm[lb];
+        for (int al = 0; al < 3; ++al) {
+            const float2 u = __ldg(eps + (size_t)(3 * tm.x + al) * nb);
 #pragma unroll
-            for (int t = 0; t < 3; ++t) u_n[t] = __ldg(eps + (size_t)(3 * bi_n.x + t) * nb + s);
+            for (int e = 0; e < 9; ++e) {
+                const float2 w = __ldg(tab + (size_t)27 * tm.y + 9 * al + e);
+                acc[e] = __ffma2_rn(make_float2(u.x, u.x), w, acc[e]);
+                acc[e] = __ffma2_rn(make_float2(-u.y, u.y), make_float2(w.y, w.x), acc[e]);
+            }
         }
-        for (; lb < lb_end; ++lb) {
-            const int4 bi = bi_n;
-            float2 u[3];
+    }
 #pragma unroll
-            for (int t = 0; t < 3; ++t) u[t] = u_n[t];
-            if (lb + 1 < lb_end) {
-                bi_n = b_sm[lb + 1];
-#pragma unroll
-                for (int t = 0; t < 3; ++t) u_n[t] = __ldg(eps + (size_t)(3 * bi_n.x + t) * nb + s);
-            }
-            const float4 *f4 = f_sm + 7 * (size_t)lb;
-            float v[28];
-#pragma unroll
-            for (int t = 0; t < 7; ++t) {
-                const float4 w4 = f4[t];
-                v[4 * t] = w4.x; v[4 * t + 1] = w4.y; v[4 * t + 2] = w4.z; v[4 * t + 3] = w4.w;
-            }
-#pragma unroll
-            for (int p = 0; p < P; ++p) {
-                const float2 c1 = chi_sm[(2 * p) * n_rep + bi.y], c2 = chi_sm[(2 * p + 1) * n_rep + bi.z];
-                // ph = c1 conj(c2), e = u ph: complex products as packed FP32x2 operations
-                const float2 ph = __ffma2_rn(make_float2(c1.y, -c1.x), make_float2(c2.y, c2.y),
-                                             __fmul2_rn(make_float2(c1.x, c1.y), make_float2(c2.x, c2.x)));
-                float2 e[3];
-#pragma unroll
-                for (int t = 0; t < 3; ++t)
-                    e[t] = __ffma2_rn(make_float2(-u[t].y, u[t].y), make_float2(ph.y, ph.x),
-                                      __fmul2_rn(make_float2(u[t].x, u[t].x), ph));
-                // complex += real * complex as packed FP32x2 FMAs
-#pragma unroll
-                for (int t = 0; t < 9; ++t) {
-                    acc[p][t] = __ffma2_rn(make_float2(v[18 + t], v[18 + t]), e[2], acc[p][t]);
-                    acc[p][t] = __ffma2_rn(make_float2(v[9 + t], v[9 + t]), e[1], acc[p][t]);
-                    acc[p][t] = __ffma2_rn(make_float2(v[t], v[t]), e[0], acc[p][t]);
+    for (int e = 0; e < 9; ++e) g.yc[(((size_t)q * g.n_cg + c) * 9 + e) * nb + s] = acc[e];
+}
+
+// Phase-summed contraction over the home index (gather), three modes per lane
+// (2 l, 2 l + 1, 64 + l), CTA = (part of the (j, k) groups, pair), each warp
+// walking its own list of groups:
+//   Y_s(3j + beta, 3k + gamma) = sum over the group's terms (i) of
+//     sum_alpha eps_{3i+alpha}(q s) W_i[alpha beta gamma],
+// W_i the phase sums of the blocks of (i, j, k): from the per-q tables of class 0
+// (Rk = 0, of q'), 1 (Rj = 0, of q'') and 2 (Rj = Rk, of q), or of the blocks
+// themselves with their phases (class 3, summed by the lanes of the 27 values).
+// Groups with three or more class-2 terms take the sum of those from yc.  FP32;
+// Y goes to A1 as BF16 hi/lo: for a fixed (b, c) the lanes of a warp cover
+// consecutive rows m = c nb + s.
+//
+// Bound: issue (FFMA2 and the conversions of the epilogue) and the 7 MB written per
+// pair.  Phasing every block for every mode (35 packed FMAs per block and mode) took
+// 275 us per 76 pairs of the 32-atom cell, 7520 blocks each; 1920 terms are left
+// here, a term's 27 values are read once for 96 modes, and eps(q) stands in shared
+// memory: 143 us (issue 51%, DRAM 43%).
+//
+// Four parts of eight warps: two CTAs per SM in one wave of a batch of sms / 2 pairs.
+constexpr int kGatherWarps = 8, kGatherParts = 4, kGatherPitch = 96;
+__global__ void __launch_bounds__(32 * kGatherWarps, 2)
+ycx_gather_kernel(XParams x, TcxGroups g, const float2 *__restrict__ epsT_all, const float2 *__restrict__ chi_all,
+                  int n_rep, __nv_bfloat16 *__restrict__ a1h, __nv_bfloat16 *__restrict__ a1l) {
+    // eps(q)(row, s) at row * 96 + s (columns nb.. are zero), then two terms' values
+    // (Re, Im, -Im, Re) per warp
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    float2 *eps_sm = reinterpret_cast<float2 *>(smem_raw);
+    const int part = blockIdx.x, a = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int q, qp, qpp;
+    pair_of(x, a, q, qp, qpp);
+    const int nb = x.nb, s0 = 2 * lane, s2 = 64 + lane;        // modes s0, s0 + 1 and s2
+    float4 *wbuf = reinterpret_cast<float4 *>(eps_sm + nb * kGatherPitch) + warp * 2 * 27;
+    const float2 *eps = epsT_all + (size_t)q * nb * nb;        // eps(q)(row, s) at row * nb + s
+    for (int t = threadIdx.x; t < nb * kGatherPitch; t += 32 * kGatherWarps) {
+        const int r = t / kGatherPitch, s = t - r * kGatherPitch;
+        const unsigned dst = smem_u32(eps_sm + t);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;"
+                     :: "r"(dst), "l"(eps + (size_t)r * nb + (s < nb ? s : 0)), "r"(s < nb ? 8 : 0) : "memory");
+    }
+    const int list = part * kGatherWarps + warp;
+    const int t0 = g.term_start[list], t1 = g.term_start[list + 1];
+    const int *gl = g.glist + g.list_start[list];
+    const bool even = (nb & 1) == 0, in2 = s2 < nb;            // (nb > 64: s0 + 1 < nb)
+    // a term's value of this lane (lanes 0..26)
+    auto load_w = [&](const int4 tm) {
+        float2 w = make_float2(0.f, 0.f);
+        const int cls = tm.y & 7;
+        if (lane < 27) {
+            if (cls < 3) {
+                const float2 *tab = cls == 0 ? g.tab[0] : cls == 1 ? g.tab[1] : g.tab[2];
+                const int n = cls == 0 ? g.n_slot[0] : cls == 1 ? g.n_slot[1] : g.n_slot[2];
+                w = __ldg(tab + 27 * ((size_t)(cls == 0 ? qp : cls == 1 ? qpp : q) * n + tm.z) + lane);
+            } else if (cls == 3) {
+                for (int y = tm.z; y < tm.z + tm.w; ++y) {
+                    const int b = __ldg(g.tblk + y);
+                    const int4 bi = __ldg(g.blkinfo + b);
+                    const float2 u = __ldg(chi_all + (size_t)qp * n_rep + bi.y);
+                    const float2 v = __ldg(chi_all + (size_t)qpp * n_rep + bi.z);
+                    const float f = __ldg(g.fc3 + (size_t)28 * b + lane);
+                    w.x += f * (u.x * v.x + u.y * v.y);        // chi(q', Rj) conj chi(q'', Rk)
+                    w.y += f * (u.y * v.x - u.x * v.y);
                 }
             }
         }
+        return w;
+    };
+    float2 acc[9][3];
 #pragma unroll
-        for (int p = 0; p < P; ++p) {
-            const size_t pbase = (size_t)(a0 + p) * x.Kp * x.Mp;
+    for (int e = 0; e < 9; ++e)
 #pragma unroll
-            for (int t = 0; t < 9; ++t) {
-                const int b = 3 * jk.x + t / 3, c = 3 * jk.y + t % 3;
-                const size_t o_re = pbase + (size_t)b * x.Mp + (size_t)c * nb + s;
-                const size_t o_im = o_re + (size_t)x.H * x.Mp;
-                const __nv_bfloat16 hr = __float2bfloat16_rn(acc[p][t].x), hm = __float2bfloat16_rn(acc[p][t].y);
-                a1h[o_re] = hr;
-                a1l[o_re] = __float2bfloat16_rn(acc[p][t].x - __bfloat162float(hr));
-                a1h[o_im] = hm;
-                a1l[o_im] = __float2bfloat16_rn(acc[p][t].y - __bfloat162float(hm));
+        for (int m = 0; m < 3; ++m) acc[e][m] = make_float2(0.f, 0.f);
+    const int4 none = make_int4(0, 4, 0, 0);
+    int4 tm = t0 < t1 ? __ldg(g.term + t0) : none, tn = t0 + 1 < t1 ? __ldg(g.term + t0 + 1) : none;
+    float2 w = load_w(tm);
+    int gi = t0 < t1 ? __ldg(gl) : 0;                          // the group under way
+    const size_t pbase = (size_t)a * x.Kp * x.Mp, im_off = (size_t)x.H * x.Mp;
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    for (int t = t0; t < t1; ++t) {
+        const int4 cur = tm;
+        float4 *wb = wbuf + (t & 1) * 27;
+        if (lane < 27) wb[lane] = make_float4(w.x, w.y, -w.y, w.x);
+        __syncwarp();
+        tm = tn;                                               // the next term's values, in flight during this one
+        w = load_w(tm);
+        tn = t + 2 < t1 ? __ldg(g.term + t + 2) : none;
+        if ((cur.y & 7) != 4) {
+            const float2 *er = eps_sm + 3 * cur.x * kGatherPitch;
+#pragma unroll
+            for (int al = 0; al < 3; ++al) {
+                const float4 e01 = *reinterpret_cast<const float4 *>(er + al * kGatherPitch + s0);
+                const float2 e2 = er[al * kGatherPitch + s2];
+                const float2 e[3] = {make_float2(e01.x, e01.y), make_float2(e01.z, e01.w), e2};
+#pragma unroll
+                for (int el = 0; el < 9; ++el) {
+                    const float4 v = wb[9 * al + el];
+#pragma unroll
+                    for (int m = 0; m < 3; ++m) {
+                        acc[el][m] = __ffma2_rn(make_float2(e[m].x, e[m].x), make_float2(v.x, v.y), acc[el][m]);
+                        acc[el][m] = __ffma2_rn(make_float2(e[m].y, e[m].y), make_float2(v.z, v.w), acc[el][m]);
+                    }
+                }
             }
         }
+        if (!(cur.y & 8)) continue;
+        const int c2 = (gi >> 16) - 1;                         // the group is complete
+        const size_t o0 = pbase + (size_t)3 * (gi & 255) * x.Mp + (size_t)3 * (gi >> 8 & 255) * nb;
+        if (t + 1 < t1) gi = __ldg(++gl);
+        if (c2 >= 0) {
+            const float2 *yc = g.yc + ((size_t)q * g.n_cg + c2) * 9 * nb;
+#pragma unroll
+            for (int el = 0; el < 9; ++el)
+#pragma unroll
+                for (int m = 0; m < 3; ++m)
+                    if (m < 2 || in2) {
+                        const float2 u = __ldg(yc + el * nb + (m < 2 ? s0 + m : s2));
+                        acc[el][m].x += u.x;
+                        acc[el][m].y += u.y;
+                    }
+        }
+#pragma unroll
+        for (int el = 0; el < 9; ++el) {
+            const size_t o = o0 + (size_t)(el / 3) * x.Mp + (el % 3) * nb;
+#pragma unroll
+            for (int z = 0; z < 2; ++z) {
+                float v[3];
+#pragma unroll
+                for (int m = 0; m < 3; ++m) v[m] = z ? acc[el][m].y : acc[el][m].x;
+                const __nv_bfloat162 h01 = __floats2bfloat162_rn(v[0], v[1]);
+                const float2 b01 = __bfloat1622float2(h01);
+                const __nv_bfloat162 l01 = __floats2bfloat162_rn(v[0] - b01.x, v[1] - b01.y);
+                const __nv_bfloat16 h2 = __float2bfloat16_rn(v[2]);
+                const __nv_bfloat16 l2 = __float2bfloat16_rn(v[2] - __bfloat162float(h2));
+                __nv_bfloat16 *ph = a1h + o + z * im_off, *pl = a1l + o + z * im_off;
+                if (even) {
+                    *reinterpret_cast<__nv_bfloat162 *>(ph + s0) = h01;
+                    *reinterpret_cast<__nv_bfloat162 *>(pl + s0) = l01;
+                } else {
+                    ph[s0] = h01.x; ph[s0 + 1] = h01.y;
+                    pl[s0] = l01.x; pl[s0 + 1] = l01.y;
+                }
+                if (in2) { ph[s2] = h2; pl[s2] = l2; }
+            }
+#pragma unroll
+            for (int m = 0; m < 3; ++m) acc[el][m] = make_float2(0.f, 0.f);
+        }
     }
+}
+static size_t gather_smem(int nb) {
+    return sizeof(float2) * (size_t)nb * kGatherPitch + sizeof(float4) * kGatherWarps * 2 * 27;
 }
 
 // Phase sum on tensor cores: per pair, the home-index contraction
@@ -1238,11 +1316,11 @@ struct Lane {
 // Batch i starts only after batch i - 3 (the other lane) has finished, which
 // bounds the q values in flight (see tcx_slices).
 // Schedule of the batched pipeline: pairs per launch, row tiles per GEMM CTA,
-// pairs per gather CTA.  The arithmetic of every (pair, mode) is the same for
+// the phase-sum kernel.  The arithmetic of every (pair, mode) is the same for
 // any schedule (fixed-order sums per tile row), so the schedule changes only
 // the time.
 struct TcxSched {
-    int batch, tpc, gp;
+    int batch, tpc;
     int yk;                        // phase sum: 1 tensor cores (tcx_y_kernel), 0 CUDA cores
     int tpy;                       // row tiles per tcx_y_kernel CTA
 };
@@ -1267,23 +1345,8 @@ cudaError_t run_batches(const LwParams &p, const LwDev &d, const TcxGroups &g, L
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     const int nb = p.nb;
-    const int gthreads = (nb + 31) / 32 * 32;
-    const size_t gsmem = sizeof(float2) * 2 * (size_t)std::max(1, p.n_rep);   // per pair
-    const size_t gblk = (7 * sizeof(float4) + sizeof(int4)) * (size_t)std::max(1, g.max_part_blocks);
-    e = cudaFuncSetAttribute(ycx_gather_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(gblk + gsmem));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(ycx_gather_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(gblk + 2 * gsmem));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(ycx_gather_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(gblk + 4 * gsmem));
-    if (e != cudaSuccess) return e;
     const int mt = lanes[0].x.Mp / kBM;
     const int gx = (mt + tpc - 1) / tpc;
-    // pairs per gather CTA (1, 2 or 4): the CTA's pairs must share q, so gp
-    // divides nq and the batch (and the first pair is a multiple of nq); the
-    // orbit pairs of EPI_SYM take one pair per CTA
-    const int gp = (!sym && sc.gp > 1 && p.nq % sc.gp == 0 && batch % sc.gp == 0) ? sc.gp : 1;
     const float2 *ew = static_cast<const float2 *>(d.eps_work), *cw = static_cast<const float2 *>(d.chi);
     // tensor-core phase sum: row tiles of kYGroups groups, about one wave of CTAs per launch
     const bool yk = sc.yk && tcx_y_fits(nb, p.n_rep) && g.y.n_groups > 0;
@@ -1309,15 +1372,10 @@ cudaError_t run_batches(const LwParams &p, const LwDev &d, const TcxGroups &g, L
             const int tpy = std::max(1, std::min(sc.tpy, mty));
             tcx_y_kernel<BN, PB><<<counted(dim3((mty + tpy - 1) / tpy, x.n_pairs)), kYThreads, ysmem, L.st>>>(
                 L.maps[10], L.maps[11], L.maps[12], x, g.y, cw, p.n_rep, L.wscale, L.a1h, L.a1l, tpy, err);
-        } else if (gp == 4)
-            ycx_gather_kernel<4><<<counted(dim3(g.n_parts, x.n_pairs / 4)), gthreads, gblk + 4 * gsmem, L.st>>>(
+        } else {
+            ycx_gather_kernel<<<counted(dim3(kGatherParts, x.n_pairs)), 32 * kGatherWarps, gather_smem(nb), L.st>>>(
                 x, g, ew, cw, p.n_rep, L.a1h, L.a1l);
-        else if (gp == 2)
-            ycx_gather_kernel<2><<<counted(dim3(g.n_parts, x.n_pairs / 2)), gthreads, gblk + 2 * gsmem, L.st>>>(
-                x, g, ew, cw, p.n_rep, L.a1h, L.a1l);
-        else
-            ycx_gather_kernel<1><<<counted(dim3(g.n_parts, x.n_pairs)), gthreads, gblk + gsmem, L.st>>>(
-                x, g, ew, cw, p.n_rep, L.a1h, L.a1l);
+        }
         pg.end();
         ProfMark p1(p.prof, KALD_PROF_TCX_GEMM1, L.st);
         k1<<<counted(dim3(gx, x.n_pairs)), Warps<EPI_T>::kThreads, smem, L.st>>>(L.maps[0], L.maps[1], L.maps[2], L.maps[3],
@@ -1368,8 +1426,7 @@ bool tcx_supported(int nb) { return nb > 64 && nb <= 96; }
 static int tcx_slices(int nq, int batch) { return (4 * batch + nq - 1) / nq + 2; }
 
 int tcx_batch(int nb, int nq, int sm_count) {
-    // pairs per launch, a multiple of 4 (the gather takes up to 4 pairs per
-    // CTA): with two or more row tiles per pair, half an SM count of pairs,
+    // pairs per launch, a multiple of 4: with two or more row tiles per pair, half an SM count of pairs,
     // so that two CTAs per pair (half the tiles each) fill one wave; with a
     // single tile, sixteen pairs per SM.  KALD_TCX_BATCH overrides (tuning).
     const long long total = (long long)nq * nq;
@@ -1389,32 +1446,78 @@ int tcx_batch_max(int nb, int nq, int sm_count) {
     return (int)std::max(1LL, std::min<long long>(2LL * tcx_batch(nb, nq, sm_count), total));
 }
 
-int tcx_parts(int n_groups) { return std::max(1, std::min(n_groups, 128)); }
-
-// Longest-processing-time partition of the (j, k) groups over n_parts CTAs
-// (weight = blocks + a constant for the 36 stores of a group).
-void plan_tcx_parts(const HostSystem &h, int n_parts, std::vector<int> &part_start, std::vector<int> &glist) {
-    const int n_groups = (int)h.pair3_j.size();
-    std::vector<int> order(n_groups);
-    for (int gr = 0; gr < n_groups; ++gr) order[gr] = gr;
-    auto weight = [&](int gr) { return h.pair3_start[gr + 1] - h.pair3_start[gr] + 4; };
+// The gather's lists (see TcxPlanHost): the groups dealt to the warps of its parts,
+// heaviest first, each to the warp with the least work so far (a term's 162 packed
+// FMAs weigh about three quarters of a group's stores and conversions).
+void plan_tcx_gather(const HostSystem &h, const LwTermsHost &lt, TcxPlanHost &o) {
+    const int ng = (int)lt.term_start.size() - 1;
+    std::vector<std::vector<int4>> terms(ng);
+    std::vector<int> group_c(ng, -1);
+    o.cterm_start.assign(1, 0);
+    o.cterm.clear();
+    o.blk.clear();
+    for (int g = 0; g < ng; ++g) {
+        int n2 = 0;
+        for (int y = lt.term_start[g]; y < lt.term_start[g + 1]; ++y) n2 += lt.term[y].y == 2;
+        for (int y = lt.term_start[g]; y < lt.term_start[g + 1]; ++y) {
+            const int4 t = lt.term[y];                         // (i, class, slot or block, 0)
+            if (t.y == 2 && n2 >= 3) {                         // (two cost what reading their sum does)
+                o.cterm.push_back(make_int2(t.x, t.z));
+            } else if (t.y == 3) {
+                if (terms[g].empty() || terms[g].back().y != 3 || terms[g].back().x != t.x)
+                    terms[g].push_back(make_int4(t.x, 3, (int)o.blk.size(), 0));
+                o.blk.push_back(t.z);
+                terms[g].back().w += 1;
+            } else {
+                terms[g].push_back(t);
+            }
+        }
+        if (n2 >= 3) {
+            group_c[g] = (int)o.cterm_start.size() - 1;
+            o.cterm_start.push_back((int)o.cterm.size());
+        }
+    }
+    std::vector<int> code(ng);
+    std::vector<unsigned char> has((size_t)h.n_atoms * h.n_atoms, 0);
+    for (int g = 0; g < ng; ++g) {
+        code[g] = h.pair3_j[g] + (h.pair3_k[g] << 8) + ((group_c[g] + 1) << 16);
+        has[(size_t)h.pair3_j[g] * h.n_atoms + h.pair3_k[g]] = 1;
+    }
+    for (int j = 0; j < h.n_atoms; ++j)                        // atom pairs without blocks: zeros
+        for (int k = 0; k < h.n_atoms; ++k)
+            if (!has[(size_t)j * h.n_atoms + k]) code.push_back(j + (k << 8));
+    const int n_all = (int)code.size();
+    terms.resize(n_all);
+    for (auto &t : terms) {
+        if (t.empty()) t.push_back(make_int4(0, 4, 0, 0));
+        t.back().y |= 8;
+    }
+    const int n_lists = kGatherParts * kGatherWarps;
+    std::vector<int> order(n_all);
+    for (int g = 0; g < n_all; ++g) order[g] = g;
+    auto weight = [&](int g) { return 3 * (int)terms[g].size() + 4; };
     std::stable_sort(order.begin(), order.end(), [&](int u, int v) { return weight(u) > weight(v); });
     typedef std::pair<long long, int> Load;
     std::priority_queue<Load, std::vector<Load>, std::greater<Load>> heap;
-    for (int x = 0; x < n_parts; ++x) heap.push(Load(0, x));
-    std::vector<std::vector<int>> parts(n_parts);
-    for (int gr : order) {
+    for (int x = 0; x < n_lists; ++x) heap.push(Load(0, x));
+    std::vector<std::vector<int>> lists(n_lists);
+    for (int g : order) {
         Load l = heap.top();
         heap.pop();
-        parts[l.second].push_back(gr);
-        l.first += weight(gr);
+        lists[l.second].push_back(g);
+        l.first += weight(g);
         heap.push(l);
     }
-    part_start.assign(1, 0);
-    glist.clear();
-    for (int x = 0; x < n_parts; ++x) {
-        glist.insert(glist.end(), parts[x].begin(), parts[x].end());
-        part_start.push_back((int)glist.size());
+    o.term_start.assign(1, 0);
+    o.list_start.assign(1, 0);
+    o.term.clear();
+    o.glist.clear();
+    for (auto &l : lists) {
+        std::sort(l.begin(), l.end());                         // neighbouring rows of A1 and of the tables
+        for (int g : l) o.term.insert(o.term.end(), terms[g].begin(), terms[g].end());
+        for (int g : l) o.glist.push_back(code[g]);
+        o.term_start.push_back((int)o.term.size());
+        o.list_start.push_back((int)o.glist.size());
     }
 }
 
@@ -1438,12 +1541,12 @@ size_t tcx_scratch_bytes(int nb, int nq, int batch) {
 // Autotuner of the crystal pipeline's schedule.  Candidates: pairs per launch
 // b/8, b/4, b/2, b and 2b (b = tcx_batch, the hand-set default), row tiles per GEMM
 // CTA for one and for two waves of CTAs, the phase sum on tensor cores or on
-// CUDA cores (one, two or four pairs per gather CTA).  The first call for a (nb, nq,
+// CUDA cores.  The first call for a (nb, nq,
 // fc3 groups, SM count) times every candidate twice on the same first pairs of
 // the workload (both lanes, no reduction: the slots these runs write are
 // written again by the real run, and the counters are reset), keeps the
 // fastest for the rest of the process, and the real run uses it.
-// Any of KALD_TCX_BATCH, KALD_TCX_TPC, KALD_TCX_GP, KALD_TCX_Y (0: CUDA-core phase sum)
+// Any of KALD_TCX_BATCH, KALD_TCX_TPC, KALD_TCX_Y (0: CUDA-core phase sum)
 // fixes the schedule instead.
 // Problems too small to time (fewer than two samples of pairs) take the default.
 static std::mutex g_tune_mu;
@@ -1462,18 +1565,20 @@ TcxSched tcx_schedule(int nb, int nq, int n_groups, bool y_ok, bool sym, int sms
     auto tpc_for = [&](int batch, int waves) { return tiles_for(mt, batch, waves); };
     const int mty = std::max(1, (n_groups + kYGroups - 1) / kYGroups);
     const int yk0 = y_ok ? 1 : 0;
-    // untimed problems take the CUDA-core gather: 3.1 us a pair against 6.2 us on
+    // untimed problems take the CUDA-core gather: 1.9 us a pair against 6.2 us on
     // tensor cores for 7 blocks per atom pair; the tensor-core sum is timed, and its
-    // operands made, from kTcxYBlocks blocks per atom pair on (tcx_y_wanted)
-    TcxSched def{b0, tpc_for(b0, 1), 2, 0, tiles_for(mty, b0, 1)};
-    const char *eb = std::getenv("KALD_TCX_BATCH"), *et = std::getenv("KALD_TCX_TPC"), *eg = std::getenv("KALD_TCX_GP");
+    // operands made, from kTcxYBlocks blocks per atom pair on (tcx_y_wanted).  Fewer
+    // than eight batches leave the two lanes uneven and take half of a batch at once:
+    // 32 atoms on 4^3 (about 400 pairs) 3.53 against 3.73 ms, on 8^3 170 against 166.
+    const int bd = pend - pbeg < 8LL * b0 ? std::max(1, b0 / 2) : b0;
+    TcxSched def{bd, tpc_for(bd, 1), 0, tiles_for(mty, bd, 1)};
+    const char *eb = std::getenv("KALD_TCX_BATCH"), *et = std::getenv("KALD_TCX_TPC");
     const char *ey = std::getenv("KALD_TCX_Y");
-    if (eb || et || eg || ey) {
+    if (eb || et || ey) {
         if (eb && std::atoi(eb) > 0) def.batch = std::min(std::atoi(eb), batch_max);
         def.tpc = tpc_for(def.batch, 1);
         def.tpy = tiles_for(mty, def.batch, 1);
         if (et && std::atoi(et) > 0) def.tpc = std::min(std::atoi(et), mt);
-        if (eg) def.gp = std::atoi(eg);
         if (ey) def.yk = std::atoi(ey) != 0 ? yk0 : 0;
         return def;
     }
@@ -1490,16 +1595,13 @@ TcxSched tcx_schedule(int nb, int nq, int n_groups, bool y_ok, bool sym, int sms
     const auto even = [](int b) { return std::max(2, b / 2 * 2); };
     for (int batch : {even(b0 / 8), even(b0 / 4), std::max(1, b0 / 2), b0, std::min(2 * b0, batch_max)})
         for (int waves : {1, 2})
-            for (int yk = yk0; yk >= 0; --yk)
-                for (int gp : {1, 2, 4}) {
-                    if (sym && gp > 1) continue;              // one orbit pair per gather CTA
-                    // (pairs per gather CTA only matters for the CUDA-core phase sum)
-                    const TcxSched c{batch, tpc_for(batch, waves), yk ? 1 : gp, yk, tiles_for(mty, batch, waves)};
-                    bool dup = false;
-                    for (const TcxSched &x : cand)
-                        dup |= x.batch == c.batch && x.tpc == c.tpc && x.gp == c.gp && x.yk == c.yk && x.tpy == c.tpy;
-                    if (!dup) cand.push_back(c);
-                }
+            for (int yk = yk0; yk >= 0; --yk) {
+                const TcxSched c{batch, tpc_for(batch, waves), yk, tiles_for(mty, batch, waves)};
+                bool dup = false;
+                for (const TcxSched &x : cand)
+                    dup |= x.batch == c.batch && x.tpc == c.tpc && x.yk == c.yk && x.tpy == c.tpy;
+                if (!dup) cand.push_back(c);
+            }
     const long long sample = 4LL * std::min(2 * b0, batch_max);
     if (pend - pbeg < 2 * sample) return def;
     cudaEvent_t t0 = nullptr, t1 = nullptr;
@@ -1550,7 +1652,7 @@ TcxSched tcx_schedule(int nb, int nq, int n_groups, bool y_ok, bool sym, int sms
 cudaError_t launch_lw_tensor(const LwParams &p, const LwDev &d, const TcxGroups &g, void *scratch, int batch,
                              int sms, int *err, cudaStream_t st, const OrbitPlan *sym, void *sym_scratch) {
     const int nb = p.nb, nq = p.nq;
-    if (!tcx_supported(nb) || batch < 1 || g.n_parts < 1 || sms < 1) return cudaErrorInvalidValue;
+    if (!tcx_supported(nb) || batch < 1 || sms < 1) return cudaErrorInvalidValue;
     const int H = tcx_half(nb), Kp = 2 * H, BN = 2 * H;
     const int Mp = (nb * nb + kBM - 1) / kBM * kBM;
     char *b = static_cast<char *>(scratch);
@@ -1575,12 +1677,14 @@ cudaError_t launch_lw_tensor(const LwParams &p, const LwDev &d, const TcxGroups 
     auto *slots = reinterpret_cast<float *>(take(sizeof(float) * 2 * (size_t)n_slices * nq * nb));
     auto *gacc = reinterpret_cast<double *>(take(sizeof(double) * (size_t)nq * nb));
 
-    // entries of A1 / T1 that no group or column covers stay zero: clear once (not
-    // where every atom pair has blocks and no row or column is padding: then every
-    // entry is written for every pair; 0.6 ms of a 6 ms call on a 4^3 mesh)
-    const bool covered = nb % 32 == 0 && Mp == nb * nb && (long long)g.n_groups * 9 == (long long)nb * nb;
+    // padding of A1 / T1 stays zero: cleared once (the gather writes every atom pair;
+    // the tensor-core phase sum only those with blocks)
     cudaError_t e = cudaSuccess;
-    if (!covered) e = cudaMemsetAsync(pl[0][0], 0, 8 * ws_round(ab), st);
+    if (g.y.fc3 && (long long)g.n_groups * 9 != (long long)nb * nb)
+        e = cudaMemsetAsync(pl[0][0], 0, 8 * ws_round(ab), st);
+    else if (nb < H || nb * nb < Mp)
+        clear_padding_kernel<<<counted(dim3(Kp, (unsigned)batch, 8)), 128, 0, st>>>(nb, H, Mp, ws_round(ab) / 2, pl[0][0]);
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemsetAsync(gacc, 0, sizeof(double) * (size_t)nq * nb, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(d.allowed, 0, sizeof(unsigned long long), st);
@@ -1592,6 +1696,13 @@ cudaError_t launch_lw_tensor(const LwParams &p, const LwDev &d, const TcxGroups 
         embed_b0_kernel<<<counted(eg), 256, 0, st>>>(nq, nb, H, d.eig, b0h, b0l);
         y_scale_kernel<<<counted(1), 1024, 0, st>>>(g.y, wscale);
     }
+
+    cudaError_t ge = cudaFuncSetAttribute(ycx_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)gather_smem(nb));
+    if (ge != cudaSuccess) return ge;
+    if (g.n_cg)       // (an orbit's pair starts at any q of the mesh)
+        ycx_same_kernel<<<counted(dim3(sym ? nq : p.nqc, g.n_cg)), 96, 0, st>>>(
+            nb, nq, g, sym ? nullptr : d.qsel, static_cast<const float2 *>(d.eps_work));
 
     XParams x;
     x.nb = nb; x.H = H; x.Kp = Kp; x.Mp = Mp;

@@ -267,3 +267,67 @@ def test_cuda_core_kernel_orbits_and_tables(k, cell, mesh, extra, cap, precision
     finally:
         ctx.set_workspace_limit(0)
     assert count["all"] == count["inversion"] == count["none"]
+
+
+@pytest.mark.parametrize("cell,mesh,extra,tables", [((5, 5, 1), (2, 1, 1), 0, True), ((5, 5, 1), (3, 1, 2), 3000, True),
+                                                    ((23, 1, 1), (1, 3, 1), 40, True), ((4, 2, 3), (2, 2, 1), 40, True),
+                                                    ((4, 4, 2), (2, 1, 1), 0, False), ((4, 4, 2), (2, 1, 1), 40, False),
+                                                    ((4, 4, 2), (1, 1, 1), 0, True)])
+def test_tensor_core_gather(k, cell, mesh, extra, tables):
+    """The phase sum of the BF16-split crystal path for 69, 72, 75 (odd rows) and 96
+    branches: terms of all classes, random blocks (alone and several per atom
+    triple), one q-point, and no tables at the smallest workspace the call takes;
+    gamma and the delta-allowed count against the FP64 mode."""
+    from kald_inputs.configs import A_FCC
+    from kald_inputs.lattice import fcc_primitive
+    from kald_inputs.lj import lj_system
+    kk, ctx = k
+    lat = fcc_primitive(A_FCC)[0]
+    at = np.array(list(np.ndindex(*cell)))
+    s = lj_system(lat * np.array(cell)[:, None], at @ lat, np.where(np.arange(len(at)) % 3 == 1, 60.0, 39.948))
+    if extra:
+        s = ki.random_fc3_system(s, extra, seed=4)
+    nu, eig = ph.phonons(s, mesh)
+    opt = {p: kk.Options(temperature_K=300.0, sigma_thz=0.1, precision=p) for p in ("fp64", "bf16split")}
+    ref, cnt = kk.kald_linewidths(ctx, [s], mesh, nu.ravel(), eig.ravel(), opt["fp64"])
+    if not tables:
+        ctx.set_workspace_limit(_smallest_workspace(kk, ctx, s, mesh, nu, eig, opt["bf16split"]))
+    try:
+        got, cnt2 = kk.kald_linewidths(ctx, [s], mesh, nu.ravel(), eig.ravel(), opt["bf16split"])
+    finally:
+        ctx.set_workspace_limit(0)
+    assert abs(cnt[1] - cnt2[1]) <= 1e-5 * cnt[1]
+    assert _rel(got, ref) < 1e-5
+
+
+def _smallest_workspace(kk, ctx, s, mesh, nu, eig, opt):
+    """Bytes the call asks for when it cannot have what it would like."""
+    import re
+    ctx.set_workspace_limit(1)
+    try:
+        with pytest.raises(kk.KaldError) as e:
+            kk.kald_linewidths(ctx, [s], mesh, nu.ravel(), eig.ravel(), opt)
+        return int(re.search(r"needs (\d+) bytes", str(e.value)).group(1))
+    finally:
+        ctx.set_workspace_limit(0)
+
+
+@pytest.mark.parametrize("cell,mesh,precision", [((1, 1, 1), (3, 3, 2), "fp64"), ((2, 1, 1), (2, 3, 1), "fp32"),
+                                                 (None, (5, 5, 4), "fp64"), (None, (5, 5, 4), "fp32")])
+def test_linewidths_at_the_smallest_workspace(k, cell, mesh, precision):
+    """Under a workspace cap at which the tables or the orbits do not fit, the call
+    does without them and gives the same linewidths and count."""
+    kk, ctx = k
+    s = ki.fcc_supercell_system(cell, seed=7) if cell else ki.small_binary().systems[0]
+    nu, eig = ph.phonons(s, mesh)
+    opt = kk.Options(temperature_K=300.0, sigma_thz=0.1, precision=precision)
+    ref, cnt = kk.kald_linewidths(ctx, [s], mesh, nu.ravel(), eig.ravel(), opt)
+    least = _smallest_workspace(kk, ctx, s, mesh, nu, eig, opt)
+    for cap in (least, least + least // 8, 2 * least):
+        ctx.set_workspace_limit(cap)
+        try:
+            got, cnt2 = kk.kald_linewidths(ctx, [s], mesh, nu.ravel(), eig.ravel(), opt)
+        finally:
+            ctx.set_workspace_limit(0)
+        assert list(cnt) == list(cnt2)
+        assert _rel(got, ref) < (1e-10 if precision == "fp64" else 1e-5)
