@@ -5,15 +5,18 @@
 // computes a result on the host.
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <exception>
 #include <functional>
 #include <map>
+#include <mutex>
 #include <numeric>
 #include <array>
+#include <thread>
 #include <tuple>
-#include <unordered_map>
 
 #include "kald_internal.h"
 #include "wdiff.cuh"
@@ -272,6 +275,39 @@ static std::vector<int> stable_key_order(int n, long long n_keys, const std::fun
     return o;
 }
 
+// f(x) for x in [0, n), dealt over host threads (the caller's among them) that end
+// with the call: up to 16, and one per 2 MB of the `bytes` that f goes through in all
+// (starting a thread costs some 40 us, in which one hashes half a megabyte).  An
+// exception of f reaches the caller.
+template <typename F>
+static void parallel_for(size_t n, size_t bytes, F &&f) {
+    const size_t nt = std::min<size_t>({n, std::max(1u, std::thread::hardware_concurrency()), 16, 1 + (bytes >> 21)});
+    std::atomic<size_t> next{0};
+    std::exception_ptr err;
+    std::mutex mu;
+    auto work = [&] {
+        for (size_t x; (x = next.fetch_add(1)) < n;) {
+            try {
+                f(x);
+            } catch (...) {
+                std::lock_guard<std::mutex> lock(mu);
+                if (!err) err = std::current_exception();
+                next = n;
+            }
+        }
+    };
+    std::vector<std::thread> others;
+    try {
+        others.reserve(nt);
+        for (size_t k = 1; k < nt; ++k) others.emplace_back(work);
+    } catch (...) {
+        // no more threads to be had: those that run do the work
+    }
+    work();
+    for (std::thread &o : others) o.join();
+    if (err) std::rethrow_exception(err);
+}
+
 kald_status plan_system(kald_ctx *ctx, const kald_system *s, HostSystem &h) {
     if (!s) return fail(ctx, KALD_E_INVALID, "system is NULL");
     const int n = s->n_atoms;
@@ -466,50 +502,105 @@ struct Hash2 {
     }
 };
 
+// Plans of n systems through the cache.  The content of all of them is hashed in
+// pieces of 256 KB, and the systems that the cache does not hold are planned, on the
+// host's threads: a 500-atom system is 30 MB of force constants, which one thread
+// hashes in 7 ms (in every call) and plans in 25 ms.  Twelve new systems of 108 to 500
+// atoms through phonons, linewidths and conductivity: 755 -> 451 ms.
+kald_status plan_systems_cached(kald_ctx *ctx, int n, const kald_system *sys,
+                                std::vector<std::shared_ptr<const HostSystem>> &out) {
+    out.assign(n, nullptr);
+    struct Piece {
+        const char *p;
+        size_t n;
+        int sys;
+    };
+    constexpr size_t kPiece = size_t(256) << 10;
+    std::vector<Piece> pieces;
+    size_t total = 0;
+    for (int x = 0; x < n; ++x) {
+        const kald_system *s = sys + x;
+        if (s->n_atoms <= 0 || s->n_fc2 < 0 || s->n_fc3 < 0 || !s->masses || !s->positions ||
+            (s->n_fc2 && (!s->fc2 || !s->fc2_idx)) || (s->n_fc3 && (!s->fc3 || !s->fc3_idx)) ||
+            is_device_ptr(s->masses) || is_device_ptr(s->positions) || is_device_ptr(s->fc2) ||
+            is_device_ptr(s->fc3) || is_device_ptr(s->fc2_idx) || is_device_ptr(s->fc3_idx)) {
+            HostSystem h;                              // reports the error
+            return plan_system(ctx, s, h);
+        }
+        auto add = [&](const void *p, size_t bytes) {
+            total += bytes;
+            for (size_t o = 0; o < bytes; o += kPiece)
+                pieces.push_back({static_cast<const char *>(p) + o, std::min(kPiece, bytes - o), x});
+        };
+        add(&s->lattice[0][0], sizeof(double) * 9);
+        add(s->masses, sizeof(double) * (size_t)s->n_atoms);
+        add(s->positions, sizeof(double) * 3 * (size_t)s->n_atoms);
+        add(s->fc2_idx, sizeof(int32_t) * 5 * (size_t)s->n_fc2);
+        add(s->fc2, sizeof(double) * 9 * (size_t)s->n_fc2);
+        add(s->fc3_idx, sizeof(int32_t) * 9 * (size_t)s->n_fc3);
+        add(s->fc3, sizeof(double) * 27 * (size_t)s->n_fc3);
+    }
+    std::vector<Hash2> ph(pieces.size());
+    auto hash_piece = [&](size_t y) { ph[y].bytes(pieces[y].p, pieces[y].n); };
+    parallel_for(pieces.size(), total, hash_piece);
+    std::vector<Hash2> hs(n);
+    for (int x = 0; x < n; ++x) {
+        hs[x].word((uint64_t)sys[x].n_atoms);
+        hs[x].word((uint64_t)sys[x].n_fc2);
+        hs[x].word((uint64_t)sys[x].n_fc3);
+    }
+    for (size_t y = 0; y < pieces.size(); ++y) {
+        hs[pieces[y].sys].word(ph[y].a);
+        hs[pieces[y].sys].word(ph[y].b);
+    }
+    std::vector<int> todo;                             // first of each content that the cache does not hold
+    std::vector<int> same(n, -1);
+    for (int x = 0; x < n; ++x) {
+        for (const auto &p : ctx->plans)
+            if (p.k0 == hs[x].a && p.k1 == hs[x].b) out[x] = p.h;
+        if (out[x]) continue;
+        for (int y : todo)
+            if (hs[y].a == hs[x].a && hs[y].b == hs[x].b) same[x] = y;
+        if (same[x] < 0) todo.push_back(x);
+    }
+    std::vector<std::shared_ptr<HostSystem>> made(todo.size());
+    std::vector<kald_ctx> errs(todo.size());           // (for the messages)
+    std::vector<kald_status> sts(todo.size(), KALD_OK);
+    // the largest first, so that none is left to run alone at the end
+    std::vector<int> order(todo.size());
+    std::iota(order.begin(), order.end(), 0);
+    std::stable_sort(order.begin(), order.end(), [&](int u, int v) { return sys[todo[u]].n_fc3 > sys[todo[v]].n_fc3; });
+    parallel_for(todo.size(), total, [&](size_t z) {
+        const int y = order[z];
+        made[y] = std::make_shared<HostSystem>();
+        sts[y] = plan_system(&errs[y], &sys[todo[y]], *made[y]);
+    });
+    for (size_t y = 0; y < todo.size(); ++y)
+        if (sts[y]) return fail(ctx, sts[y], errs[y].err);
+    for (size_t y = 0; y < todo.size(); ++y) {
+        const std::shared_ptr<HostSystem> &h = made[y];
+        const size_t bytes = sizeof(double) * (h->fc3_blk.size() + h->fc2_blk.size() + 6 * h->fc2_rcart.size()) +
+                             sizeof(int) * (7 * h->fc3_i.size() + h->fc2_atoms.size());
+        // keep at most 32 plans and 1 GB of them, dropping the oldest
+        size_t held = bytes;
+        for (const auto &p : ctx->plans) held += p.bytes;
+        while (!ctx->plans.empty() && (ctx->plans.size() >= 32 || held > (size_t(1) << 30))) {
+            held -= ctx->plans.front().bytes;
+            ctx->plans.erase(ctx->plans.begin());
+        }
+        ctx->plans.push_back({hs[todo[y]].a, hs[todo[y]].b, h, bytes});
+        out[todo[y]] = h;
+    }
+    for (int x = 0; x < n; ++x)
+        if (same[x] >= 0) out[x] = out[same[x]];
+    return KALD_OK;
+}
 kald_status plan_system_cached(kald_ctx *ctx, const kald_system *s, std::shared_ptr<const HostSystem> &out) {
     if (!s) return fail(ctx, KALD_E_INVALID, "system is NULL");
-    if (s->n_atoms <= 0 || s->n_fc2 < 0 || s->n_fc3 < 0 || !s->masses || !s->positions ||
-        (s->n_fc2 && (!s->fc2 || !s->fc2_idx)) || (s->n_fc3 && (!s->fc3 || !s->fc3_idx)) ||
-        is_device_ptr(s->masses) || is_device_ptr(s->positions) || is_device_ptr(s->fc2) ||
-        is_device_ptr(s->fc3) || is_device_ptr(s->fc2_idx) || is_device_ptr(s->fc3_idx)) {
-        HostSystem h;                              // reports the error
-        return plan_system(ctx, s, h);
-    }
-    Hash2 hs;
-    hs.word((uint64_t)s->n_atoms);
-    hs.word((uint64_t)s->n_fc2);
-    hs.word((uint64_t)s->n_fc3);
-    hs.bytes(&s->lattice[0][0], sizeof(double) * 9);
-    hs.bytes(s->masses, sizeof(double) * (size_t)s->n_atoms);
-    hs.bytes(s->positions, sizeof(double) * 3 * (size_t)s->n_atoms);
-    if (s->n_fc2) {
-        hs.bytes(s->fc2_idx, sizeof(int32_t) * 5 * (size_t)s->n_fc2);
-        hs.bytes(s->fc2, sizeof(double) * 9 * (size_t)s->n_fc2);
-    }
-    if (s->n_fc3) {
-        hs.bytes(s->fc3_idx, sizeof(int32_t) * 9 * (size_t)s->n_fc3);
-        hs.bytes(s->fc3, sizeof(double) * 27 * (size_t)s->n_fc3);
-    }
-    for (size_t x = 0; x < ctx->plans.size(); ++x)
-        if (ctx->plans[x].k0 == hs.a && ctx->plans[x].k1 == hs.b) {
-            out = ctx->plans[x].h;
-            return KALD_OK;
-        }
-    auto h = std::make_shared<HostSystem>();
-    kald_status st = plan_system(ctx, s, *h);
-    if (st) return st;
-    const size_t bytes = sizeof(double) * (h->fc3_blk.size() + h->fc2_blk.size() + 6 * h->fc2_rcart.size()) +
-                         sizeof(int) * (7 * h->fc3_i.size() + h->fc2_atoms.size());
-    // keep at most 32 plans and 1 GB of them, dropping the oldest
-    size_t total = bytes;
-    for (const auto &p : ctx->plans) total += p.bytes;
-    while (!ctx->plans.empty() && (ctx->plans.size() >= 32 || total > (size_t(1) << 30))) {
-        total -= ctx->plans.front().bytes;
-        ctx->plans.erase(ctx->plans.begin());
-    }
-    ctx->plans.push_back({hs.a, hs.b, h, bytes});
-    out = h;
-    return KALD_OK;
+    std::vector<std::shared_ptr<const HostSystem>> v;
+    const kald_status st = plan_systems_cached(ctx, 1, s, v);
+    if (!st) out = v[0];
+    return st;
 }
 
 std::atomic<unsigned long long> g_launches{0};
@@ -718,12 +809,12 @@ kald_status kald_phonons_batch(kald_ctx *ctx, int32_t n_sys, const kald_system *
     if (n_sys <= 0 || !sys) return fail(ctx, KALD_E_INVALID, "n_sys must be > 0");
     if (!nu_thz || !eigvec) return fail(ctx, KALD_E_INVALID, "nu_thz/eigvec NULL");
     const int32_t gamma_mesh[3] = {1, 1, 1};
-    std::vector<std::shared_ptr<const HostSystem>> hp(n_sys);
+    std::vector<std::shared_ptr<const HostSystem>> hp;
     std::vector<size_t> off_nb(n_sys), off_eig(n_sys);
     size_t on = 0, oe = 0;
     std::vector<int> large;
+    if ((st = plan_systems_cached(ctx, n_sys, sys, hp))) return st;
     for (int x = 0; x < n_sys; ++x) {
-        if ((st = plan_system_cached(ctx, &sys[x], hp[x]))) return st;
         const int nb = hp[x]->nb;
         off_nb[x] = on;
         off_eig[x] = oe;
@@ -801,36 +892,53 @@ kald_status kald_phonons_batch(kald_ctx *ctx, int32_t n_sys, const kald_system *
 
 namespace kald {
 namespace {
+// Blocks of fc3 by their nine indices (the first of several alike): open addressing,
+// at most half full.
+struct Fc3Index {
+    const kald_system *s;
+    std::vector<int> slot;
+    size_t mask;
+    static size_t hash(const int32_t *a) {
+        size_t h = 1469598103934665603ull;
+        for (int x = 0; x < 9; ++x) h = (h ^ (size_t)(uint32_t)a[x]) * 1099511628211ull;
+        return h ^ (h >> 32);
+    }
+    explicit Fc3Index(const kald_system *sys) : s(sys) {
+        size_t n = 16;
+        while (n < 2 * (size_t)s->n_fc3) n *= 2;
+        slot.assign(n, -1);
+        mask = n - 1;
+        for (int b = 0; b < s->n_fc3; ++b) {
+            const int32_t *k = s->fc3_idx + 9 * (size_t)b;
+            size_t y = hash(k) & mask;
+            while (slot[y] >= 0 && !std::equal(k, k + 9, s->fc3_idx + 9 * (size_t)slot[y])) y = (y + 1) & mask;
+            if (slot[y] < 0) slot[y] = b;
+        }
+    }
+    int find(const int32_t *k) const {
+        size_t y = hash(k) & mask;
+        while (slot[y] >= 0 && !std::equal(k, k + 9, s->fc3_idx + 9 * (size_t)slot[y])) y = (y + 1) & mask;
+        return slot[y];
+    }
+};
+
 // True when every fc3 block (i; j Rj; k Rk) has the partner (i; k Rk; j Rj)
 // with the last two Cartesian indices exchanged, to 1e-12 of the largest
 // |Phi3| (then Y_mu and phi are symmetric and the tensor-core path computes
 // only the upper triangle).
 bool fc3_symmetric_last_two(const kald_system *s) {
-    struct H {
-        size_t operator()(const std::array<int, 9> &a) const {
-            size_t h = 1469598103934665603ull;
-            for (int v : a) h = (h ^ (size_t)(uint32_t)v) * 1099511628211ull;
-            return h;
-        }
-    };
-    std::unordered_map<std::array<int, 9>, int, H> idx;
-    idx.reserve((size_t)s->n_fc3 * 2);
+    const Fc3Index idx(s);
     // entries agree to 1e-12 of the largest |Phi3| (the self blocks (i; i; i)
     // are sums that cancel to rounding noise, so no per-entry relative test)
     double tol = 0.0;
     for (size_t v = 0; v < 27 * (size_t)s->n_fc3; ++v) tol = std::max(tol, std::fabs(s->fc3[v]));
     tol *= 1e-12;
     for (int b = 0; b < s->n_fc3; ++b) {
-        std::array<int, 9> k;
-        for (int x = 0; x < 9; ++x) k[x] = s->fc3_idx[9 * (size_t)b + x];
-        idx.emplace(k, b);
-    }
-    for (int b = 0; b < s->n_fc3; ++b) {
         const int32_t *x = s->fc3_idx + 9 * (size_t)b;
-        const std::array<int, 9> k = {x[0], x[5], x[6], x[7], x[8], x[1], x[2], x[3], x[4]};
-        auto it = idx.find(k);
-        if (it == idx.end()) return false;
-        const double *f = s->fc3 + 27 * (size_t)b, *g = s->fc3 + 27 * (size_t)it->second;
+        const int32_t k[9] = {x[0], x[5], x[6], x[7], x[8], x[1], x[2], x[3], x[4]};
+        const int at = idx.find(k);
+        if (at < 0) return false;
+        const double *f = s->fc3 + 27 * (size_t)b, *g = s->fc3 + 27 * (size_t)at;
         for (int a = 0; a < 3; ++a)
             for (int c = 0; c < 3; ++c)
                 for (int d = 0; d < 3; ++d) {
@@ -847,31 +955,18 @@ bool fc3_symmetric_last_two(const kald_system *s) {
 // |Phi3|.  The two exchanges generate all six permutations.
 bool fc3_symmetric_all(const kald_system *s) {
     if (!fc3_symmetric_last_two(s)) return false;
-    struct H {
-        size_t operator()(const std::array<int, 9> &a) const {
-            size_t h = 1469598103934665603ull;
-            for (int v : a) h = (h ^ (size_t)(uint32_t)v) * 1099511628211ull;
-            return h;
-        }
-    };
-    std::unordered_map<std::array<int, 9>, int, H> idx;
-    idx.reserve((size_t)s->n_fc3 * 2);
+    const Fc3Index idx(s);
     // entries agree to 1e-12 of the largest |Phi3| (the self blocks (i; i; i)
     // are sums that cancel to rounding noise, so no per-entry relative test)
     double tol = 0.0;
     for (size_t v = 0; v < 27 * (size_t)s->n_fc3; ++v) tol = std::max(tol, std::fabs(s->fc3[v]));
     tol *= 1e-12;
     for (int b = 0; b < s->n_fc3; ++b) {
-        std::array<int, 9> k;
-        for (int x = 0; x < 9; ++x) k[x] = s->fc3_idx[9 * (size_t)b + x];
-        idx.emplace(k, b);
-    }
-    for (int b = 0; b < s->n_fc3; ++b) {
         const int32_t *x = s->fc3_idx + 9 * (size_t)b;
-        const std::array<int, 9> k = {x[1], x[0], -x[2], -x[3], -x[4], x[5], x[6] - x[2], x[7] - x[3], x[8] - x[4]};
-        auto it = idx.find(k);
-        if (it == idx.end()) return false;
-        const double *f = s->fc3 + 27 * (size_t)b, *g = s->fc3 + 27 * (size_t)it->second;
+        const int32_t k[9] = {x[1], x[0], -x[2], -x[3], -x[4], x[5], x[6] - x[2], x[7] - x[3], x[8] - x[4]};
+        const int at = idx.find(k);
+        if (at < 0) return false;
+        const double *f = s->fc3 + 27 * (size_t)b, *g = s->fc3 + 27 * (size_t)at;
         for (int a = 0; a < 3; ++a)
             for (int c = 0; c < 3; ++c)
                 for (int d = 0; d < 3; ++d) {
@@ -1001,7 +1096,8 @@ static cudaError_t join_lanes(kald_ctx *ctx, const std::vector<cudaStream_t> &la
 // over concurrent lane streams (so that small supercells share the GPU), and
 // the call synchronises once at the end.  Each system's arithmetic is the same
 // as when it is computed alone, so the results do not depend on the batch.
-static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system *sys, const double *nu_thz,
+static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system *sys,
+                                    const std::vector<std::shared_ptr<const HostSystem>> &hps, const double *nu_thz,
                                     const double *eigvec, const kald_options *opt, double *gamma, bool d_nu,
                                     bool d_eig, bool d_g, uint64_t &tot, uint64_t &allowed_tot) {
     kald_status st;
@@ -1017,10 +1113,8 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
     std::vector<Item> items;
     size_t off_nb = 0, off_eig = 0, total_modes = 0;
     for (int x = 0; x < n_sys; ++x) {
-        std::shared_ptr<const HostSystem> hp;
-        if ((st = plan_system_cached(ctx, &sys[x], hp))) return st;
-        const int nb = hp->nb;
-        if (nb > kMaxNbSmall) items.push_back({x, hp, GammaPlan(), {}, off_nb, off_eig, 0});
+        const int nb = hps[x]->nb;
+        if (nb > kMaxNbSmall) items.push_back({x, hps[x], GammaPlan(), {}, off_nb, off_eig, 0});
         off_nb += nb;
         off_eig += (size_t)nb * nb;
     }
@@ -1034,6 +1128,20 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
         std::copy(nu_thz, nu_thz + total_modes, nu_all.begin());
     }
     size_t need = ws_round(32 * items.size());
+    if (mode == KALD_BF16_SPLIT) {
+        size_t bytes = 0;
+        std::vector<int> unknown;                      // (a plan may stand for several systems)
+        for (size_t y = 0; y < items.size(); ++y) {
+            bool first = items[y].hp->fc3_symmetric < 0;
+            for (int z : unknown) first = first && items[z].hp != items[y].hp;
+            if (first) unknown.push_back((int)y);
+            if (first) bytes += sizeof(double) * items[y].hp->fc3_blk.size();
+        }
+        parallel_for(unknown.size(), bytes, [&](size_t z) {
+            const Item &it = items[unknown[z]];
+            it.hp->fc3_symmetric = fc3_symmetric_last_two(&sys[it.x]) ? 1 : 0;
+        });
+    }
     for (Item &it : items) {
         const HostSystem &h = *it.hp;
         const int nb = h.nb;
@@ -1051,7 +1159,6 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
         it.gjk.resize(2 * (size_t)gp.n_groups);
         for (int g = 0; g < gp.n_groups; ++g) { it.gjk[2 * g] = h.pair3_j[g]; it.gjk[2 * g + 1] = h.pair3_k[g]; }
         if (mode == KALD_BF16_SPLIT) {
-            if (h.fc3_symmetric < 0) h.fc3_symmetric = fc3_symmetric_last_two(&sys[it.x]) ? 1 : 0;
             gp.symmetric = h.fc3_symmetric;
             gp.n_long = h.pair3_long;
             band_tiles(gp.omega_h, tc_tile(), opt->n_sigma * kTwoPi * opt->sigma_thz, gp.symmetric, gp.tiles,
@@ -1224,9 +1331,11 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
     const bool d_nu = is_device_ptr(nu_thz), d_eig = is_device_ptr(eigvec), d_g = is_device_ptr(gamma);
     const int fp32 = opt->precision == KALD_FP32;
     uint64_t tot = 0, allowed_tot = 0;
+    std::vector<std::shared_ptr<const HostSystem>> hps;   // one q-point: all at once; else one by one
     if (nq_mesh == 1) {
         // every Gamma-only supercell (nb > 96) of the call in one launch sequence
-        if ((st = gamma_only_batch(ctx, n_sys, sys, nu_thz, eigvec, opt, gamma, d_nu, d_eig, d_g, tot,
+        if ((st = plan_systems_cached(ctx, n_sys, sys, hps))) return st;
+        if ((st = gamma_only_batch(ctx, n_sys, sys, hps, nu_thz, eigvec, opt, gamma, d_nu, d_eig, d_g, tot,
                                    allowed_tot)))
             return st;
     }
@@ -1234,7 +1343,8 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
     int lean = 0;            // where the workspace cannot be had: 1 without tables, 2 without orbits as well
     for (int x = 0; x < n_sys; ++x) {
         std::shared_ptr<const HostSystem> hp;
-        if ((st = plan_system_cached(ctx, &sys[x], hp))) return st;
+        if (nq_mesh == 1) hp = hps[x];
+        else if ((st = plan_system_cached(ctx, &sys[x], hp))) return st;
         const HostSystem &h = *hp;
         const int nb = h.nb;
         if (nb > kMaxNbSmall && nq_mesh != 1)
@@ -2124,9 +2234,24 @@ kald_status kald_kappa_qhgk(kald_ctx *ctx, int32_t n_sys, const kald_system *sys
     };
     std::vector<Item> items(n_sys);
     size_t need = 0, off_nb = 0, off_eig = 0;
+    std::vector<std::shared_ptr<const HostSystem>> hps;
+    if ((st = plan_systems_cached(ctx, n_sys, sys, hps))) return st;
+    {
+        size_t bytes = 0;
+        std::vector<int> unknown;                      // (a plan may stand for several systems)
+        for (int x = 0; x < n_sys; ++x) {
+            bool first = hps[x]->fc2_symmetric < 0;
+            for (int z : unknown) first = first && hps[z] != hps[x];
+            if (first) unknown.push_back(x);
+            if (first) bytes += 8 * sizeof(double) * hps[x]->fc2_blk.size();   // (it sorts)
+        }
+        parallel_for(unknown.size(), bytes, [&](size_t z) {
+            hps[unknown[z]]->fc2_symmetric = fc2_symmetric(&sys[unknown[z]]) ? 1 : 0;
+        });
+    }
     for (int x = 0; x < n_sys; ++x) {
         Item &it = items[x];
-        if ((st = plan_system_cached(ctx, &sys[x], it.hp))) return st;
+        it.hp = hps[x];
         const HostSystem &h = *it.hp;
         const int nb = h.nb;
         const size_t nn = (size_t)nb * nb;
@@ -2145,7 +2270,6 @@ kald_status kald_kappa_qhgk(kald_ctx *ctx, int32_t n_sys, const kald_system *sys
         need += bytes_of(it.row_start) + bytes_of(it.col_j) + scaled_bytes(h.fc2_blk, h.fc2_atoms, h, 9, 9, 0) +
                 bytes_of(h.fc2_dist) + qhgk_work_bytes(nb) + ws_round(sizeof(double) * 9 * (size_t)it.n_partial) +
                 ws_round(72);
-        if (h.fc2_symmetric < 0) h.fc2_symmetric = fc2_symmetric(&sys[x]) ? 1 : 0;
         if (!d_nu) need += ws_round(sizeof(double) * nb);
         if (!d_eig) need += ws_round(sizeof(double2) * nn);
         if (!d_g) need += ws_round(sizeof(double) * nb);

@@ -331,3 +331,28 @@ def test_linewidths_at_the_smallest_workspace(k, cell, mesh, precision):
             ctx.set_workspace_limit(0)
         assert list(cnt) == list(cnt2)
         assert _rel(got, ref) < (1e-10 if precision == "fp64" else 1e-5)
+
+
+def test_batch_plans_equal_single_calls(k):
+    """A batch whose systems repeat, some hashed on several threads (more than a
+    megabyte of force constants), gives what each system gives alone, from new and
+    from kept plans; a faulty system in it is refused with its own message."""
+    kk, ctx = k
+    big, small = ki.fcc_supercell_system((4, 4, 3), seed=1), ki.fcc_supercell_system((3, 3, 1), seed=2)
+    systems = [small, big, ki.random_fc3_system(small, 30, seed=3), big, small]
+    opt = kk.Options(temperature_K=300.0, sigma_thz=0.1, precision="bf16split")
+    ph1 = [ph.phonons(s, (1, 1, 1)) for s in (big, small)]
+    by = [1, 0, 1, 0, 1]
+    nu, eig = (np.concatenate([ph1[b][c].ravel() for b in by]) for c in (0, 1))
+    with kk.Context(0) as fresh:
+        runs = [kk.kald_linewidths(fresh, systems, (1, 1, 1), nu, eig, opt) for _ in range(2)]
+    alone = [kk.kald_linewidths(ctx, [s], (1, 1, 1), ph1[b][0].ravel(), ph1[b][1].ravel(), opt)
+             for s, b in zip(systems, by)]
+    for g, cnt in runs:
+        np.testing.assert_array_equal(np.asarray(g).ravel(), np.concatenate([np.asarray(a[0]).ravel() for a in alone]))
+        assert cnt[1] == sum(a[1][1] for a in alone)
+    bad = ki.fcc_supercell_system((3, 3, 1), seed=2)
+    bad.fc3_idx[5, 0] = bad.n_atoms
+    nu3, eig3 = (np.tile(ph1[1][c].ravel(), 3) for c in (0, 1))
+    with pytest.raises(kk.KaldError, match="fc3_idx"):
+        kk.kald_linewidths(ctx, [small, bad, small], (1, 1, 1), nu3, eig3, opt)
