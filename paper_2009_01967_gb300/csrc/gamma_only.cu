@@ -14,6 +14,7 @@
 // CUDA-core) kernels of that pipeline.
 
 #include <algorithm>
+#include <array>
 #include <map>
 #include <mutex>
 #include <utility>
@@ -201,12 +202,14 @@ cudaError_t run_plain(const GammaPlan &gp, const GammaDev &d, const LwParams &p,
     return cudaGetLastError();
 }
 
-// gamma[mu] = pref / w_mu * sum of the mode's band-tile partials (CSR, fixed order).
+// gamma[mu] = pref / w_mu * (what other modes' tiles left for the mode + the sum of
+// its own band-tile partials (CSR, fixed order)).
 __global__ void g_gamma_csr_kernel(int nb, const int *__restrict__ tile_start, const double *__restrict__ partial,
-                                   const double *__restrict__ omega, double pref, double *__restrict__ gamma) {
+                                   const double *__restrict__ gacc, const double *__restrict__ omega, double pref,
+                                   double *__restrict__ gamma) {
     const int mu = blockIdx.x * blockDim.x + threadIdx.x;
     if (mu >= nb) return;
-    double t = 0.0;
+    double t = gacc ? gacc[mu] : 0.0;
     for (int k = tile_start[mu]; k < tile_start[mu + 1]; ++k) t += partial[k];
     const double w = omega[mu];
     gamma[mu] = (w > 0.0) ? pref * t / w : 0.0;
@@ -227,15 +230,14 @@ cudaError_t launch_gamma_only(const GammaPlan &gp, const GammaDev &d, const LwPa
         const size_t nt = gp.tiles.size();
         e = cudaMemsetAsync(d.partial_tc, 0, sizeof(double) * std::max<size_t>(nt, 1), st);
         if (e != cudaSuccess) return e;
+        const double *gacc = nullptr;
         e = launch_gamma_only_tc(gp, d, p, d.tc_scratch, gp.tiles, gp.tile_start, d.tiles_dev, gp.symmetric,
-                                 d.partial_tc, d.err, gp.sms, st, nb);
+                                 d.partial_tc, d.err, gp.sms, st, nb, &gacc);
         if (e != cudaSuccess) return e;
-        // tile_start is uploaded right after the tiles (same allocation)
+        // tile_start stands right after the tiles (same allocation)
         const int *ts = reinterpret_cast<const int *>(d.tiles_dev + std::max<size_t>(nt, 1));
-        e = cudaMemcpyAsync(const_cast<int *>(ts), gp.tile_start.data(), sizeof(int) * (nb + 1),
-                            cudaMemcpyHostToDevice, st);
-        if (e != cudaSuccess) return e;
-        g_gamma_csr_kernel<<<counted((nb + 127) / 128), 128, 0, st>>>(nb, ts, d.partial_tc, d.omega, pref, gamma_out);
+        g_gamma_csr_kernel<<<counted((nb + 127) / 128), 128, 0, st>>>(nb, ts, d.partial_tc, gacc, d.omega, pref,
+                                                                      gamma_out);
     } else {
         e = cudaMemsetAsync(d.partial, 0, sizeof(double) * (size_t)nb * gp.n_part, st);
         if (e != cudaSuccess) return e;
@@ -254,12 +256,12 @@ cudaError_t launch_gamma_only(const GammaPlan &gp, const GammaDev &d, const LwPa
 // again by the real run), fastest kept per (nb, SMs) for the process.  The
 // per-mode arithmetic does not depend on the batch.
 static std::mutex g_mb_mu;
-static std::map<std::pair<int, int>, int> g_mb_tuned;
+static std::map<std::array<int, 4>, int> g_mb_tuned;      // by (nb, SMs, largest batch, sym3)
 
 int tune_gamma_batch(const GammaPlan &gp, const GammaDev &d, const LwParams &p, cudaStream_t st) {
     const int nb = p.nb, sms = gp.sms;
-    const int def = tc_gamma_batch(nb, sms), mbx = tc_gamma_batch_max(nb, sms);
-    const std::pair<int, int> key(nb, sms);
+    const int mbx = gp.mb_max, def = std::min(tc_gamma_batch(nb, sms), mbx);
+    const std::array<int, 4> key{nb, sms, mbx, gp.sym3};
     {
         std::lock_guard<std::mutex> lock(g_mb_mu);
         auto it = g_mb_tuned.find(key);
@@ -284,7 +286,7 @@ int tune_gamma_batch(const GammaPlan &gp, const GammaDev &d, const LwParams &p, 
         g2.mb = c;
         ok = cudaEventRecord(t0, st) == cudaSuccess &&
              launch_gamma_only_tc(g2, d, p, d.tc_scratch, g2.tiles, g2.tile_start, d.tiles_dev, g2.symmetric,
-                                  d.partial_tc, d.err, sms, st, sample) == cudaSuccess &&
+                                  d.partial_tc, d.err, sms, st, sample, nullptr) == cudaSuccess &&
              cudaEventRecord(t1, st) == cudaSuccess && cudaEventSynchronize(t1) == cudaSuccess;
         float ms = 0.0f;
         if (ok) ok = cudaEventElapsedTime(&ms, t0, t1) == cudaSuccess;

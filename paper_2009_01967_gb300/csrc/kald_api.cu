@@ -922,59 +922,46 @@ struct Fc3Index {
     }
 };
 
-// True when every fc3 block (i; j Rj; k Rk) has the partner (i; k Rk; j Rj)
-// with the last two Cartesian indices exchanged, to 1e-12 of the largest
-// |Phi3| (then Y_mu and phi are symmetric and the tensor-core path computes
-// only the upper triangle).
-bool fc3_symmetric_last_two(const kald_system *s) {
+// Sets h.fc3_symmetric: every fc3 block (i; j Rj; k Rk) has the partner (i; k Rk; j Rj)
+// with the last two Cartesian indices exchanged (then Y_mu and phi are symmetric and
+// the tensor-core path computes only the upper triangle); and h.fc3_perm_symmetric:
+// besides, the partner (j; i -Rj; k Rk - Rj) (home atom j) with the first two
+// exchanged.  The two exchanges generate all six permutations.
+void fc3_symmetries(const kald_system *s, const HostSystem &h) {
     const Fc3Index idx(s);
-    // entries agree to 1e-12 of the largest |Phi3| (the self blocks (i; i; i)
-    // are sums that cancel to rounding noise, so no per-entry relative test)
+    // entries agree to 1e-12 of the largest |Phi3| (the self blocks (i; i; i) are sums
+    // that cancel to rounding noise, so no per-entry relative test)
     double tol = 0.0;
     for (size_t v = 0; v < 27 * (size_t)s->n_fc3; ++v) tol = std::max(tol, std::fabs(s->fc3[v]));
     tol *= 1e-12;
-    for (int b = 0; b < s->n_fc3; ++b) {
-        const int32_t *x = s->fc3_idx + 9 * (size_t)b;
-        const int32_t k[9] = {x[0], x[5], x[6], x[7], x[8], x[1], x[2], x[3], x[4]};
-        const int at = idx.find(k);
-        if (at < 0) return false;
-        const double *f = s->fc3 + 27 * (size_t)b, *g = s->fc3 + 27 * (size_t)at;
-        for (int a = 0; a < 3; ++a)
-            for (int c = 0; c < 3; ++c)
-                for (int d = 0; d < 3; ++d) {
-                    const double u = f[9 * a + 3 * c + d], v = g[9 * a + 3 * d + c];
-                    if (std::fabs(u - v) > tol) return false;
-                }
-    }
-    return true;
-}
-// True when Phi3 is symmetric under every permutation of its three (atom,
-// cell, Cartesian) indices: with the exchange of the last two (above), every
-// block (i; j Rj; k Rk) has the partner (j; i -Rj; k Rk - Rj) (home atom j)
-// with the first two Cartesian indices exchanged, to 1e-12 of the largest
-// |Phi3|.  The two exchanges generate all six permutations.
-bool fc3_symmetric_all(const kald_system *s) {
-    if (!fc3_symmetric_last_two(s)) return false;
-    const Fc3Index idx(s);
-    // entries agree to 1e-12 of the largest |Phi3| (the self blocks (i; i; i)
-    // are sums that cancel to rounding noise, so no per-entry relative test)
-    double tol = 0.0;
-    for (size_t v = 0; v < 27 * (size_t)s->n_fc3; ++v) tol = std::max(tol, std::fabs(s->fc3[v]));
-    tol *= 1e-12;
-    for (int b = 0; b < s->n_fc3; ++b) {
-        const int32_t *x = s->fc3_idx + 9 * (size_t)b;
-        const int32_t k[9] = {x[1], x[0], -x[2], -x[3], -x[4], x[5], x[6] - x[2], x[7] - x[3], x[8] - x[4]};
-        const int at = idx.find(k);
-        if (at < 0) return false;
-        const double *f = s->fc3 + 27 * (size_t)b, *g = s->fc3 + 27 * (size_t)at;
-        for (int a = 0; a < 3; ++a)
-            for (int c = 0; c < 3; ++c)
-                for (int d = 0; d < 3; ++d) {
-                    const double u = f[9 * a + 3 * c + d], v = g[9 * c + 3 * a + d];
-                    if (std::fabs(u - v) > tol) return false;
-                }
-    }
-    return true;
+    auto partners = [&](auto &&key, auto &&at) {
+        for (int b = 0; b < s->n_fc3; ++b) {
+            int32_t k[9];
+            key(s->fc3_idx + 9 * (size_t)b, k);
+            const int o = idx.find(k);
+            if (o < 0) return false;
+            const double *f = s->fc3 + 27 * (size_t)b, *g = s->fc3 + 27 * (size_t)o;
+            for (int a = 0; a < 3; ++a)
+                for (int c = 0; c < 3; ++c)
+                    for (int d = 0; d < 3; ++d)
+                        if (std::fabs(f[9 * a + 3 * c + d] - g[at(a, c, d)]) > tol) return false;
+        }
+        return true;
+    };
+    const bool last = partners(
+        [](const int32_t *x, int32_t *k) {
+            const int32_t y[9] = {x[0], x[5], x[6], x[7], x[8], x[1], x[2], x[3], x[4]};
+            std::copy_n(y, 9, k);
+        },
+        [](int a, int c, int d) { return 9 * a + 3 * d + c; });
+    const bool first = last && partners(
+        [](const int32_t *x, int32_t *k) {
+            const int32_t y[9] = {x[1], x[0], -x[2], -x[3], -x[4], x[5], x[6] - x[2], x[7] - x[3], x[8] - x[4]};
+            std::copy_n(y, 9, k);
+        },
+        [](int a, int c, int d) { return 9 * c + 3 * a + d; });
+    h.fc3_symmetric = last ? 1 : 0;
+    h.fc3_perm_symmetric = first ? 1 : 0;
 }
 // True when every fc2 block (i; j R) has the partner (j; i -R) with the
 // Cartesian indices exchanged, to 1e-12 of the largest |Phi2|.
@@ -1003,7 +990,8 @@ bool fc2_symmetric(const kald_system *s) {
     return true;
 }
 // (tm, tn) tiles of T E^T that the delta window can reach, per mode.
-void band_tiles(const std::vector<double> &w, int tile, double cut, int symmetric, std::vector<int2> &tiles,
+// symmetric: tn >= tm; sym3: tm from the mode's own tile on, too.
+void band_tiles(const std::vector<double> &w, int tile, double cut, int symmetric, int sym3, std::vector<int2> &tiles,
                 std::vector<int> &start) {
     const int nb = (int)w.size(), nt = (nb + tile - 1) / tile;
     std::vector<double> lo(nt, 1e300), hi(nt, -1e300);
@@ -1018,7 +1006,7 @@ void band_tiles(const std::vector<double> &w, int tile, double cut, int symmetri
     for (int mu = 0; mu < nb; ++mu) {
         start[mu] = (int)tiles.size();
         if (!(w[mu] > 0.0)) continue;
-        for (int a = 0; a < nt; ++a) {
+        for (int a = sym3 ? mu / tile : 0; a < nt; ++a) {
             if (!(hi[a] >= lo[a])) continue;
             for (int b = symmetric ? a : 0; b < nt; ++b) {
                 if (!(hi[b] >= lo[b])) continue;
@@ -1127,7 +1115,6 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
     } else {
         std::copy(nu_thz, nu_thz + total_modes, nu_all.begin());
     }
-    size_t need = ws_round(32 * items.size());
     if (mode == KALD_BF16_SPLIT) {
         size_t bytes = 0;
         std::vector<int> unknown;                      // (a plan may stand for several systems)
@@ -1139,9 +1126,12 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
         }
         parallel_for(unknown.size(), bytes, [&](size_t z) {
             const Item &it = items[unknown[z]];
-            it.hp->fc3_symmetric = fc3_symmetric_last_two(&sys[it.x]) ? 1 : 0;
+            fc3_symmetries(&sys[it.x], *it.hp);
         });
     }
+    // where the workspace cannot be had, batches of fewer modes and no tiles' sums
+    for (int lean = 0;; lean = 1) {
+    size_t need = ws_round(32 * items.size());
     for (Item &it : items) {
         const HostSystem &h = *it.hp;
         const int nb = h.nb;
@@ -1160,8 +1150,15 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
         for (int g = 0; g < gp.n_groups; ++g) { it.gjk[2 * g] = h.pair3_j[g]; it.gjk[2 * g + 1] = h.pair3_k[g]; }
         if (mode == KALD_BF16_SPLIT) {
             gp.symmetric = h.fc3_symmetric;
+            std::vector<int> per_k(h.n_atoms, 0);
+            for (int k : h.pair3_k) gp.row_entries = std::max(gp.row_entries, 3 * ++per_k[k]);
+            // one projection per unordered triple of modes: half of the first
+            // contraction and a third of the second (256 atoms 7.7 -> 4.6 ms, twelve
+            // cells of 108 to 500 atoms 451 -> 335 ms)
+            gp.sym3 = !lean && opt->symmetry == KALD_SYM_ALL && h.fc3_perm_symmetric;
+            gp.mb_max = lean ? std::max(1, tc_gamma_batch(nb, ctx->sm_count) / 2) : tc_gamma_batch_max(nb, ctx->sm_count);
             gp.n_long = h.pair3_long;
-            band_tiles(gp.omega_h, tc_tile(), opt->n_sigma * kTwoPi * opt->sigma_thz, gp.symmetric, gp.tiles,
+            band_tiles(gp.omega_h, tc_tile(), opt->n_sigma * kTwoPi * opt->sigma_thz, gp.symmetric, gp.sym3, gp.tiles,
                        gp.tile_start);
         }
         const size_t n_tiles = std::max<size_t>(gp.tiles.size(), 1);
@@ -1169,7 +1166,7 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
                    scaled_bytes(h.fc3_blk, h.fc3_atoms, h, 27, 27, 0) + 2 * ws_round(sizeof(double) * nb) +
                    ws_round(sizeof(int) * nb);
         if (mode == KALD_BF16_SPLIT)
-            b += tc_gamma_scratch_bytes(nb, ctx->sm_count, gp.n_fc3) + bytes_of(h.pair3_order) + ws_round(sizeof(int2) * n_tiles + sizeof(int) * (nb + 1)) +
+            b += tc_gamma_scratch_bytes(nb, gp.mb_max, gp.n_fc3, gp.sym3) + bytes_of(h.pair3_order) + ws_round(sizeof(int2) * n_tiles + sizeof(int) * (nb + 1)) +
                  ws_round(sizeof(double) * n_tiles);
         else
             b += 4 * ws_round(rs * nn) + ws_round(sizeof(double) * nb * (size_t)gp.n_part);
@@ -1179,7 +1176,9 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
         it.need = b;
         need += b;
     }
-    if ((st = ws_reserve(ctx, need))) return st;
+    if (!(st = ws_reserve(ctx, need))) break;
+    if (st != KALD_E_NOMEM || lean || mode != KALD_BF16_SPLIT) return st;
+    }
     // per-system counters: allowed triplets (8 B) and the wait-failure flag (4 B)
     char *counters = static_cast<char *>(ws_take(ctx, 32 * items.size()));
     cudaMemsetAsync(counters, 0, 32 * items.size(), ctx->stream);
@@ -1205,7 +1204,7 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
         gd.group_order = nullptr;
         gd.tc_scratch = nullptr; gd.tiles_dev = nullptr; gd.partial_tc = nullptr;
         if (mode == KALD_BF16_SPLIT) {
-            gd.tc_scratch = ws_take(ctx, tc_gamma_scratch_bytes(nb, ctx->sm_count, it.gp.n_fc3));
+            gd.tc_scratch = ws_take(ctx, tc_gamma_scratch_bytes(nb, it.gp.mb_max, it.gp.n_fc3, it.gp.sym3));
             gd.group_order = upload(ctx, h.pair3_order);
             gd.tiles_dev = static_cast<int2 *>(ws_take(ctx, sizeof(int2) * n_tiles + sizeof(int) * (nb + 1)));
             gd.partial_tc = static_cast<double *>(ws_take(ctx, sizeof(double) * n_tiles));
@@ -1240,12 +1239,13 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
     if (mode == KALD_BF16_SPLIT) {
         // modes per launch: the autotuner's choice per distinct nb (timed on the
         // first system of that size, before the concurrent launches)
-        std::map<int, int> mb_of;
+        std::map<std::pair<int, int>, int> mb_of;
         for (size_t t = 0; t < items.size(); ++t) {
             const int nb = items[t].hp->nb;
-            if (!mb_of.count(nb)) mb_of[nb] = tune_gamma_batch(items[t].gp, devs[t].gd, params_of(*items[t].hp),
-                                                               ctx->stream);
-            items[t].gp.mb = mb_of[nb];
+            const std::pair<int, int> key(nb, items[t].gp.sym3);
+            if (!mb_of.count(key)) mb_of[key] = tune_gamma_batch(items[t].gp, devs[t].gd, params_of(*items[t].hp),
+                                                                 ctx->stream);
+            items[t].gp.mb = mb_of[key];
         }
         cudaMemsetAsync(counters, 0, 32 * items.size(), ctx->stream);   // the timing runs counted too
     }
@@ -1482,7 +1482,7 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         int orb_pairs = 0;
         std::vector<int> orb_rows;
         if (!small && !listed && reuse && opt->symmetry == KALD_SYM_ALL && nq > 1 && lean < 2) {
-            if (h.fc3_perm_symmetric < 0) h.fc3_perm_symmetric = fc3_symmetric_all(&sys[x]) ? 1 : 0;
+            if (h.fc3_perm_symmetric < 0) fc3_symmetries(&sys[x], h);
             if (h.fc3_perm_symmetric) orb_pairs = std::max(0, orbit_pairs(mesh));
             if (orb_pairs) {
                 orb_rows.resize(nqc);

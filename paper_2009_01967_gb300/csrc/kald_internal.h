@@ -342,6 +342,9 @@ struct GammaPlan {
     std::vector<int2> tiles;
     std::vector<int> tile_start;     // [nb + 1]
     int symmetric = 0;               // Phi3 symmetric in its last two indices
+    int sym3 = 0;                    // ... and under every permutation: each triple of modes projected once
+    int row_entries = 1;             // largest number of entries of a row of Y_mu^T
+    int mb_max = 1;                  // largest modes per launch that the scratch holds
     int sms = 1;                     // SMs of the device (modes per tensor-core launch)
     int mb = 0;                      // modes per tensor-core launch (0: tc_gamma_batch; autotuned)
 };
@@ -372,12 +375,12 @@ int tune_gamma_batch(const GammaPlan &gp, const GammaDev &d, const LwParams &p, 
 // modes per launch of the tensor-core Gamma-only path and its scratch bytes
 int tc_gamma_batch(int nb, int sms);
 int tc_gamma_batch_max(int nb, int sms);
-size_t tc_gamma_scratch_bytes(int nb, int sms, size_t n_fc3);
+size_t tc_gamma_scratch_bytes(int nb, int mb_max, size_t n_fc3, int sym3);
 int tc_tile(void);
 cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const LwParams &p, void *scratch,
                                  const std::vector<int2> &tiles, const std::vector<int> &tile_start,
                                  int2 *tiles_dev, int symmetric, double *partial_tc, int *err, int sms,
-                                 cudaStream_t st, int mode_limit);
+                                 cudaStream_t st, int mode_limit, const double **gacc_out);
 
 // small_nb.cu: crystal linewidths of one- and two-atom cells (nb = 3 or 6),
 // one thread per (pair, mode), the projection in registers.  The Bloch phase

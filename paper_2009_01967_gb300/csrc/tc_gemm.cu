@@ -1,11 +1,16 @@
 // Tensor-core (tcgen05) path of the Gamma-only linewidths: the per-mode
 // contractions T = E Y_mu^T-form and phi = T E^T (paper Eq. projection_plus at
-// q = 0) on 5th-generation tensor cores with a BF16 hi+lo split.
+// q = 0) on 5th-generation tensor cores with a 16-bit hi+lo split.
 //
-// Every operand x is carried as two BF16 planes, hi = bf16(x), lo = bf16(x - hi),
+// Every operand x is carried as two FP16 planes, hi = fp16(x), lo = fp16(x - hi),
 // and a product is formed from three MMAs, A_hi B_hi + A_hi B_lo + A_lo B_hi,
-// accumulated in FP32 in tensor memory; the dropped lo*lo term and the
-// rounding of lo leave about 16 significant bits per product.
+// accumulated in FP32 in tensor memory; the dropped lo*lo term and the rounding of
+// lo leave about 22 significant bits per product (two BF16 pieces left 16, and the
+// error of gamma from that, 1e-5 for the smallest cells, grows when each triple of
+// modes is projected once instead of three times).  FP16's narrow range is met by
+// powers of two (Scales): each mode's eigenvector is scaled by its largest
+// component, Y_mu by that of mode mu and a bound of the contraction with Phi3, T by
+// the number of terms of its sums; the epilogues take them out exactly.
 //
 // Several modes go through each launch (a batch of MB modes, so that small
 // systems still fill the GPU): the Y and T planes of the batch are stacked
@@ -15,9 +20,8 @@
 // Kernel shape (one 128 x 128 output tile per CTA, 128 threads):
 //   warp 0 lane 0   TMA producer: 4 tiled loads per K block of 64 (A hi/lo,
 //                   B hi/lo; 128-byte swizzle), 3-stage ring of mbarriers
-//   warp 1          allocates 512 TMEM columns (four accumulators, K blocks
-//                   round-robin); lane 0 issues the MMAs
-//                   (M = 128, N = 128, K = 16, kind::f16, BF16 in, FP32 out)
+//   warp 1          allocates 512 TMEM columns (four accumulators); lane 0 issues the MMAs
+//                   (M = 128, N = 128, K = 16, kind::f16, FP16 in, FP32 out)
 //                   and commits each stage back to the producer
 //   warps 0-3       epilogue: tcgen05.ld of their 32 accumulator lanes
 // Every mbarrier wait is bounded; on expiry the CTA records the failure in a
@@ -25,7 +29,7 @@
 // and returns, and the host reports KALD_E_TIMEOUT.
 
 #include <cuda.h>
-#include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include <algorithm>
 #include <cmath>
@@ -39,19 +43,21 @@
 namespace kald {
 namespace {
 
-constexpr int kBM = 128, kBN = 128, kBK = 64;      // tile; 64 BF16 = one 128-byte swizzle row
+constexpr int kBM = 128, kBN = 128, kBK = 64;      // tile; 64 FP16 = one 128-byte swizzle row
 constexpr int kStages = 3;
-// The K loop is spread round-robin over kAcc accumulators (all 512 TMEM
-// columns) that the epilogue adds in FP32: a long chain of tensor-core
-// accumulations (2592 / 16 x 3 for the 864-atom cell) drifts towards zero by
-// about 1e-5 relative; four chains of a quarter of the length keep gamma
-// within 1e-5 of the FP64 oracle.
+// Tensor-core accumulation truncates: a long chain of MMAs into one accumulator
+// (2592 / 16 x 3 for the 864-atom cell) drifts towards zero by about 1e-5 relative.
+// The hi hi products go round-robin into three accumulators and the two small
+// products into a fourth, whose own truncations are 2^-8 of that (all 512 TMEM
+// columns); the epilogue adds the four in FP32.  A third of the K steps then
+// truncate a full-size sum: all three products over four accumulators did so three
+// quarters as often as there are steps.
 constexpr int kAcc = 4;
 constexpr int kTileBytes = kBM * kBK * 2;          // 16 KB per operand plane per stage
 constexpr int kStageBytes = 4 * kTileBytes;        // A hi, A lo, B hi, B lo
 
-enum : int { EPI_SPLIT = 0, EPI_GAMMA = 1 };
-constexpr uint32_t kIdesc = tc::idesc_bf16(kBN);
+enum : int { EPI_SPLIT = 0, EPI_GAMMA = 1, EPI_GSYM = 2 };
+constexpr uint32_t kIdesc = tc::idesc_f16(kBN);
 
 using namespace tc;
 
@@ -66,17 +72,37 @@ struct EpiGamma {
     unsigned long long *allowed;
     const int2 *tiles;        // (tm | b << 16, tn): band tile (tm, tn) of mode mu0 + b
     int symmetric;            // phi symmetric: upper-triangle tiles, symmetrised weights
+    double *rowp, *colp;      // EPI_GSYM: [n_tiles][128] sums for the modes of a tile's rows and columns
 };
 struct EpiSplit {
-    __nv_bfloat16 *hi, *lo;   // [batch][rows][ld] output planes
+    __half *hi, *lo;   // [batch][rows][ld] output planes
     int ld;
     int b_rows;               // rows of one Y / T plane (stacked per mode of the batch)
+    int tm0;                  // first row tile
 };
 
-// Columns [c, c + 32) of the nacc accumulators, added in a fixed order.
-__device__ __forceinline__ void tmem_ld_sum(uint32_t taddr, int nacc, float v[32]) {
+// Powers of two that bring the operands into FP16's range:
+//   E(m, .) = 2^e_m E', |E'| <= 1, stored x 2^kEBits;
+//   Y_mu = 2^(e_mu + eL) Y', |Y'| <= 1, stored x 2^kYBits (2^eL bounds the sums of
+//   |Phi3| that one component multiplies);
+//   T = E Y_mu = 2^(e_m + e_mu + eL) T', |T'| <= 2^eR, stored x 2^(kTBits - eR).
+constexpr int kEBits = 10, kYBits = 14, kTBits = 15;
+struct Scales {
+    const int *l1;            // bits of the largest sum of |Phi3| (FP32)
+    const int *e;             // [nb] e_m
+    int eR;                   // 2^eR >= entries of a row of Y_mu^T
+    __device__ __forceinline__ int eL() const {
+        int x;
+        frexpf(__int_as_float(__ldg(l1)), &x);
+        return x;
+    }
+};
+
+// Columns [c, c + 32) of the accumulators, added in a fixed order.
+__device__ __forceinline__ void tmem_ld_sum(uint32_t taddr, float v[32]) {
     tmem_ld32(taddr, v);
-    for (int a = 1; a < nacc; ++a) {
+#pragma unroll
+    for (int a = 1; a < kAcc; ++a) {
         float u[32];
         tmem_ld32(taddr + (uint32_t)(a * kBN), u);
 #pragma unroll
@@ -84,13 +110,65 @@ __device__ __forceinline__ void tmem_ld_sum(uint32_t taddr, int nacc, float v[32
     }
 }
 
-// C[m][n] = sum_k A[m][k] B[n][k]; A, B as BF16 hi/lo planes behind four
+// Columns [c, c + 16) of the accumulators, added in the same order.
+__device__ __forceinline__ void tmem_ld_sum16(uint32_t taddr, float v[16]) {
+    tmem_ld16(taddr, v);
+#pragma unroll
+    for (int a = 1; a < kAcc; ++a) {
+        float u[16];
+        tmem_ld16(taddr + (uint32_t)(a * kBN), u);
+#pragma unroll
+        for (int x = 0; x < 16; ++x) v[x] += u[x];
+    }
+}
+
+// Sums over the 32 lanes of 16 values each: lane l returns value l / 2 (both
+// lanes of a pair the same), added pairwise in a fixed order.
+__device__ __forceinline__ float lane_sums16(float (&v)[16]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int h = 8; h > 0; h >>= 1) {
+        const bool up = lane & (2 * h);
+#pragma unroll
+        for (int x = 0; x < h; ++x) {
+            const float keep = up ? v[x + h] : v[x], send = up ? v[x] : v[x + h];
+            v[x] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * h);
+        }
+    }
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+// The projections of mode a with the unordered pair {b, c} of two other positions:
+// sum of the weights of (a; b, c) and (a; c, b) (of one of them for b = c) and
+// their window hits, the energy differences formed as EPI_GAMMA forms them -- b the
+// row and c the column, exchanged as well where both lie in one tile (`same`).
+__device__ __forceinline__ float pair_terms(F2 wa, F2 wb, F2 wc, F2 nb_, F2 nc_, bool equal, bool same, float cut,
+                                            int shape, float s2i, int &cnt) {
+    const F2 dif = f2_add(wa, f2_neg(wb));
+    const float dp = f2_diff(f2_add(wa, wb), wc), dm = f2_diff(dif, wc);
+    const float dn = f2_diff(nb_, nc_), sn = 1.0f + nb_.h + nc_.h;
+    const bool hp = fabsf(dp) < cut, hm = fabsf(dm) < cut;
+    float g = 0.0f;
+    if (hp) g += dn * delta_shape(dp, shape, s2i);
+    if (hm) g += 0.5f * sn * delta_shape(dm, shape, s2i);
+    cnt += hp || hm;
+    if (equal) return g;
+    const float dp2 = same ? f2_diff(f2_add(wa, wc), wb) : f2_diff(dif, f2_neg(wc));
+    const float dm2 = same ? f2_diff(f2_add(wa, f2_neg(wc)), wb) : dm;
+    const bool hp2 = fabsf(dp2) < cut, hm2 = fabsf(dm2) < cut;
+    if (hp2) g -= dn * delta_shape(dp2, shape, s2i);
+    if (hm2) g += 0.5f * sn * delta_shape(dm2, shape, s2i);
+    cnt += hp2 || hm2;
+    return g;
+}
+
+// C[m][n] = sum_k A[m][k] B[n][k]; A, B as FP16 hi/lo planes behind four
 // tensor maps (box 64 x 128, 128-byte swizzle).  Grid: one CTA per tile.
 template <int EPI>
 __global__ void __launch_bounds__(128, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ CUtensorMap mAl,
                const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CUtensorMap mBl,
-               int M, int N, int K, EpiSplit es, EpiGamma eg, int *err, uint32_t wait_limit) {
+               int M, int N, int K, Scales sc, EpiSplit es, EpiGamma eg, int *err, uint32_t wait_limit) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // 1024-byte alignment for the swizzled tiles
     unsigned char *base = reinterpret_cast<unsigned char *>(
@@ -98,23 +176,22 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
     __shared__ __align__(8) uint64_t full[kStages], empty[kStages], done;
     __shared__ uint32_t tmem_base_sm;
     __shared__ int fail_sm;
-    __shared__ float wn_sm[kBN], wl_sm[kBN], nn_sm[kBN], nl_sm[kBN];
+    __shared__ float wn_sm[kBN], wl_sm[kBN], nn_sm[kBN], nl_sm[kBN], cf_sm[kBN];
     __shared__ double red[4];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int tm, tn, bz;                              // tile and mode of the batch
-    if (EPI == EPI_GAMMA) {
+    if (EPI != EPI_SPLIT) {
         const int2 t = eg.tiles[blockIdx.x];
         tm = t.x & 0xffff; bz = t.x >> 16; tn = t.y;
     } else {
-        tm = blockIdx.y; tn = blockIdx.x; bz = blockIdx.z;
+        tm = es.tm0 + blockIdx.y; tn = blockIdx.x; bz = blockIdx.z;
     }
     // row coordinates of the A and B tiles: T (GEMM2's A) and Y (GEMM1's B)
     // are stacked per mode of the batch
-    const int a_row = tm * kBM + (EPI == EPI_GAMMA ? bz * eg.a_rows : 0);
+    const int a_row = tm * kBM + (EPI != EPI_SPLIT ? bz * eg.a_rows : 0);
     const int b_row = tn * kBN + (EPI == EPI_SPLIT ? bz * es.b_rows : 0);
     const int nkb = (K + kBK - 1) / kBK;
-    const int nacc = min(kAcc, nkb);             // accumulators that received MMAs
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
@@ -157,11 +234,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
             const uint64_t bh = smem_desc(st + 2 * kTileBytes), bl = smem_desc(st + 3 * kTileBytes);
 #pragma unroll
             for (int k = 0; k < kBK / 16; ++k) {
-                const uint64_t dk = (uint64_t)((k * 32) >> 4);     // 16 BF16 = 32 B along K
-                const uint32_t dacc = tmem + (uint32_t)((kb % kAcc) * kBN);
-                mma_bf16(dacc, ah + dk, bh + dk, kIdesc, (kb >= kAcc || k > 0) ? 1u : 0u);
-                mma_bf16(dacc, ah + dk, bl + dk, kIdesc, 1u);
-                mma_bf16(dacc, al + dk, bh + dk, kIdesc, 1u);
+                const uint64_t dk = (uint64_t)((k * 32) >> 4);     // 16 FP16 = 32 B along K
+                const int step = kb * (kBK / 16) + k;
+                const uint32_t dacc = tmem + (uint32_t)((step % (kAcc - 1)) * kBN), dlo = tmem + (kAcc - 1) * kBN;
+                mma_bf16(dacc, ah + dk, bh + dk, kIdesc, step >= kAcc - 1 ? 1u : 0u);
+                mma_bf16(dlo, ah + dk, bl + dk, kIdesc, step > 0 ? 1u : 0u);
+                mma_bf16(dlo, al + dk, bh + dk, kIdesc, 1u);
             }
             mma_commit(&empty[s]);               // stage free once these MMAs finish
         }
@@ -185,27 +263,128 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
         // rows, so each lane pair writes two whole 64-byte row segments per
         // chunk with 32-byte stores (st_rowpair_v8).
         const bool okw = __all_sync(0xffffffffu, ok);
+        const float tsc = ldexpf(1.0f, kTBits - sc.eR - kEBits - kYBits);
         const size_t orow = (size_t)bz * es.b_rows + m;
         char *ph = reinterpret_cast<char *>(es.hi + orow * es.ld + tn * kBN);
         char *pl = reinterpret_cast<char *>(es.lo + orow * es.ld + tn * kBN);
-        const size_t rs = sizeof(__nv_bfloat16) * (size_t)es.ld;
+        const size_t rs = sizeof(__half) * (size_t)es.ld;
 #pragma unroll 1
         for (int c0 = 0; c0 < kBN; c0 += 32) {
             float v[32];
-            tmem_ld_sum(taddr + c0, nacc, v);
+            tmem_ld_sum(taddr + c0, v);
             if (!okw) continue;
             uint32_t hw[16], lw[16];
 #pragma unroll
             for (int x = 0; x < 16; ++x) {
-                const float a = v[2 * x], b = v[2 * x + 1];
-                const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-                const __nv_bfloat162 l = __floats2bfloat162_rn(a - __low2float(h), b - __high2float(h));
+                const float a = v[2 * x] * tsc, b = v[2 * x + 1] * tsc;
+                const __half2 h = __floats2half2_rn(a, b);
+                const __half2 l = __floats2half2_rn(a - __low2float(h), b - __high2float(h));
                 hw[x] = *reinterpret_cast<const uint32_t *>(&h);
                 lw[x] = *reinterpret_cast<const uint32_t *>(&l);
             }
             st_rowpair_v8(ph + 2 * c0, rs, hw, lane & 1);
             st_rowpair_v8(pl + 2 * c0, rs, lw, lane & 1);
         }
+    } else if (EPI == EPI_GSYM) {
+        // Phi3 symmetric under every permutation: mode mu of the batch, rows m >= mu
+        // and columns n >= m stand for all orders of {mu, m, n}.  The three modes'
+        // sums share |phi|^2 / (w_mu w_m w_n) and the three energy differences
+        //   s3 = mu + m - n,  s2 = mu - m + n,  s1 = -(mu - m - n);
+        // mode m's go to rowp, mode n's to colp (FP64 across tiles).  With every
+        // frequency above two windows, differences inside the window are exact but
+        // for their last rounding, so that one set serves the three positions;
+        // below that each position forms its own (pair_terms).
+        __shared__ float cs_sm[4][kBN];
+        const int nc = tn * kBN + threadIdx.x;
+        const F2 wcol = nc < N ? f2_of(eg.omega[nc]) : F2{0.f, 0.f};
+        const F2 ncol = nc < N ? f2_of(eg.occ[nc]) : F2{0.f, 0.f};
+        wn_sm[threadIdx.x] = wcol.h; wl_sm[threadIdx.x] = wcol.l;
+        nn_sm[threadIdx.x] = ncol.h; nl_sm[threadIdx.x] = ncol.l;
+        cf_sm[threadIdx.x] = nc < N ? ldexpf(1.0f, __ldg(sc.e + nc)) : 0.0f;
+        const float cut = (float)eg.cut, s2i = (float)eg.sig2inv;
+        const int mu = eg.mu0 + bz;
+        const float rf = m < M ? ldexpf(1.0f, __ldg(sc.e + m) + __ldg(sc.e + mu) + sc.eL() + sc.eR - kTBits - kEBits) : 0.0f;
+        const F2 wmu = f2_of(eg.omega[mu]), nmu = f2_of(eg.occ[mu]);
+        const F2 w1p = m < M ? f2_of(eg.omega[m]) : F2{0.f, 0.f};
+        const F2 n1p = m < M ? f2_of(eg.occ[m]) : F2{0.f, 0.f};
+        const float w1 = w1p.h, n1 = n1p.h, two = 2.01f * cut;
+        const bool fast = __syncthreads_and((!(w1 > 0.0f) || w1 >= two) && (!(wcol.h > 0.0f) || wcol.h >= two)) &&
+                          wmu.h >= two;                // (the columns are in shared memory, too)
+        const F2 wsum = f2_add(wmu, w1p), wdif = f2_add(wmu, f2_neg(w1p));
+        const float dmu = f2_diff(nmu, n1p);
+        const bool live = w1 > 0.0f && m >= mu;
+        const int tmu = mu / kBM;
+        float acc1 = 0.0f, acc2 = 0.0f;
+        int cnt = 0;
+#pragma unroll 1
+        for (int c0 = 0; c0 < kBN; c0 += 16) {
+            float v[16];
+            tmem_ld_sum16(taddr + c0, v);
+            bool any = false;
+#pragma unroll
+            for (int x = 0; x < 16; ++x) {
+                const float f = v[x] * rf * cf_sm[c0 + x];
+                v[x] = 0.0f;
+                const F2 w2p{wn_sm[c0 + x], wl_sm[c0 + x]};
+                const float w2 = w2p.h;
+                const int n = tn * kBN + c0 + x;
+                const float s3 = f2_diff(wsum, w2p), s1 = f2_diff(wdif, w2p), s2 = f2_diff(wdif, f2_neg(w2p));
+                if (!live || n < m || !(w2 > 0.0f)) continue;
+                const F2 n2p{nn_sm[c0 + x], nl_sm[c0 + x]};
+                const float n2 = n2p.h;
+                float g1, g2, g3;
+                if (fast) {
+                    const bool h3 = fabsf(s3) < cut, h1 = fabsf(s1) < cut, h2 = fabsf(s2) < cut;
+                    if (!(h3 || h1 || h2)) continue;
+                    const float G3 = h3 ? delta_shape(s3, eg.shape, s2i) : 0.0f;
+                    const float G1 = h1 ? delta_shape(s1, eg.shape, s2i) : 0.0f;
+                    const float G2 = h2 ? delta_shape(s2, eg.shape, s2i) : 0.0f;
+                    g1 = f2_diff(n1p, n2p) * (G3 - G2) + (m == n ? 0.5f : 1.0f) * (1.0f + n1 + n2) * G1;
+                    g2 = f2_diff(nmu, n2p) * (G3 - G1) + (1.0f + nmu.h + n2) * G2;
+                    g3 = dmu * (G2 - G1) + (m == mu ? 0.5f : 1.0f) * (1.0f + nmu.h + n1) * G3;
+                    const int h31 = h3 || h1, h21 = h2 || h1, h32 = h3 || h2;
+                    cnt += h31 + (m < n ? h21 : 0);                      // (mu; m, n)
+                    if (m > mu) cnt += h32 + h21;                        // (m; mu, n)
+                    if (m < n) cnt += h32 + (m > mu ? h31 : 0);          // (n; mu, m)
+                } else {
+                    int h = 0;
+                    g1 = pair_terms(wmu, w1p, w2p, n1p, n2p, m == n, tm == tn, cut, eg.shape, s2i, h);
+                    g2 = g3 = 0.0f;
+                    if (m > mu) g2 = pair_terms(w1p, wmu, w2p, nmu, n2p, false, tmu == tn, cut, eg.shape, s2i, h);
+                    if (m < n) g3 = pair_terms(w2p, wmu, w1p, nmu, n1p, m == mu, tmu == tm, cut, eg.shape, s2i, h);
+                    if (!h) continue;
+                    cnt += h;
+                }
+                any = true;
+                const float c = f * f / (w1 * w2);
+                acc1 += c * g1;
+                if (m > mu) acc2 += c * g2;
+                if (m < n) v[x] = c * g3;
+            }
+            if (__any_sync(0xffffffffu, any)) {
+                const float s = lane_sums16(v);
+                if (!(lane & 1)) cs_sm[warp][c0 + (lane >> 1)] = s;
+            } else if (lane < 16) {
+                cs_sm[warp][c0 + lane] = 0.0f;
+            }
+        }
+        double accd = (double)acc1;
+        unsigned long long cn = (unsigned long long)cnt;
+        for (int o = 16; o > 0; o >>= 1) {
+            accd += __shfl_xor_sync(0xffffffffu, accd, o);
+            cn += __shfl_xor_sync(0xffffffffu, cn, o);
+        }
+        if (lane == 0) red[warp] = accd;
+        if (lane == 0 && cn && ok) atomicAdd(eg.allowed, cn);
+        // the other modes' sums, with their own frequency in place of mu's below the line
+        const double iw = 1.0 / (double)wmu.h;
+        const size_t o = (size_t)blockIdx.x * kBM;
+        eg.rowp[o + threadIdx.x] = ok ? (double)acc2 * ((double)w1 * iw) : 0.0;
+        __syncthreads();
+        if (threadIdx.x == 0) eg.partial[blockIdx.x] = ok ? red[0] + red[1] + red[2] + red[3] : 0.0;
+        const double cs = ((double)cs_sm[0][threadIdx.x] + (double)cs_sm[1][threadIdx.x]) +
+                          ((double)cs_sm[2][threadIdx.x] + (double)cs_sm[3][threadIdx.x]);
+        eg.colp[o + threadIdx.x] = ok ? cs * ((double)wcol.h * iw) : 0.0;
     } else {
         // delta weights in FP32 (window test first; the FP64 unit is slow),
         // the energy and occupation differences from FP32 pairs (wdiff.cuh)
@@ -215,10 +394,14 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
             const F2 nv = n < N ? f2_of(eg.occ[n]) : F2{0.f, 0.f};
             wn_sm[x] = wv.h; wl_sm[x] = wv.l;
             nn_sm[x] = nv.h; nl_sm[x] = nv.l;
+            cf_sm[x] = n < N ? ldexpf(1.0f, __ldg(sc.e + n)) : 0.0f;
         }
         __syncthreads();
         const float cut = (float)eg.cut, s2i = (float)eg.sig2inv;
         const F2 wmu = f2_of(eg.omega[eg.mu0 + bz]);
+        const float rf = m < M ? ldexpf(1.0f, __ldg(sc.e + m) + __ldg(sc.e + eg.mu0 + bz) + sc.eL() + sc.eR - kTBits -
+                                                  kEBits)
+                               : 0.0f;
         const F2 w1p = m < M ? f2_of(eg.omega[m]) : F2{0.f, 0.f};
         const F2 n1p = m < M ? f2_of(eg.occ[m]) : F2{0.f, 0.f};
         const float w1 = w1p.h, n1 = n1p.h;
@@ -229,7 +412,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
 #pragma unroll 1
         for (int c0 = 0; c0 < kBN; c0 += 32) {
             float v[32];
-            tmem_ld_sum(taddr + c0, nacc, v);
+            tmem_ld_sum(taddr + c0, v);
             if (!(w1 > 0.0f)) continue;
 #pragma unroll 4
             for (int x = 0; x < 32; ++x) {
@@ -247,7 +430,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
                 if (hp) g += dn * delta_shape(dp, eg.shape, s2i);
                 if (hm) g += (upper ? 1.0f : 0.5f) * (1.0f + n1 + n2) * delta_shape(dm, eg.shape, s2i);
                 if (hp2) g -= dn * delta_shape(dp2, eg.shape, s2i);
-                const float f = v[x];
+                const float f = v[x] * rf * cf_sm[c0 + x];
                 acc += f * f * g / (w1 * w2);
                 cnt += (unsigned long long)(hp || hm) + (unsigned long long)(upper && (hp2 || hm));
             }
@@ -283,21 +466,69 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
     }
 }
 
-// hi/lo BF16 planes of a row-major matrix (rows x cols) into padded planes
-// (rows_pad x ld); the padding stays zero from the caller's memset.
-template <typename SRC>
-__global__ void split_kernel(int rows, int cols, const SRC *__restrict__ src, size_t src_stride, int ld,
-                             __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo) {
-    const size_t n = (size_t)rows * cols;
-    for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < n;
-         x += (size_t)gridDim.x * blockDim.x) {
-        const size_t r = x / cols, c = x % cols;
-        float v;
-        if constexpr (sizeof(SRC) == 16) v = (float)reinterpret_cast<const double2 *>(src)[r * src_stride + c].x;
-        else v = (float)src[r * src_stride + c];
-        const __nv_bfloat16 h = __float2bfloat16_rn(v);
+// gacc[m] += the sums that the tiles of the batch's modes mu0 .. mu0 + nm - 1 leave for
+// mode m (EPI_GSYM): tile by tile within a mode, mode by mode, whatever the batch.
+// One CTA per 128 modes m; partial sums of a mode of the batch per 128 threads.
+__global__ void __launch_bounds__(1024)
+gsym_sums_kernel(int nb, int mu0, int nm, const int *__restrict__ tile_start, const int2 *__restrict__ tiles, int t0,
+                 const double *__restrict__ rowp, const double *__restrict__ colp, double *__restrict__ gacc) {
+    __shared__ double sm[32][kBM];
+    const int t = blockIdx.x, x = threadIdx.x & (kBM - 1);
+    for (int b = threadIdx.x / kBM; b < nm; b += blockDim.x / kBM) {
+        double s = 0.0;
+        for (int y = tile_start[mu0 + b]; y < tile_start[mu0 + b + 1]; ++y) {
+            const int2 r = __ldg(tiles + y);
+            if ((r.x & 0xffff) == t) s += rowp[(size_t)(y - t0) * kBM + x];
+            if (r.y == t) s += colp[(size_t)(y - t0) * kBM + x];
+        }
+        sm[b][x] = s;
+    }
+    __syncthreads();
+    const int m = t * kBM + x;
+    if (threadIdx.x >= kBM || m >= nb) return;
+    double v = gacc[m];
+    for (int b = 0; b < nm; ++b) v += sm[b][x];
+    gacc[m] = v;
+}
+
+// Exponent of each mode's largest eigenvector component: |E(m, .)| <= 2^e[m].
+__global__ void __launch_bounds__(128)
+mode_scale_kernel(int nb, const double2 *__restrict__ eig, int *__restrict__ e) {
+    __shared__ float red[4];
+    float v = 0.0f;
+    for (int c = threadIdx.x; c < nb; c += blockDim.x) v = fmaxf(v, fabsf((float)eig[(size_t)blockIdx.x * nb + c].x));
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x) return;
+    int x;
+    frexpf(fmaxf(fmaxf(red[0], red[1]), fmaxf(red[2], red[3])), &x);
+    e[blockIdx.x] = x;
+}
+// Largest sum of |Phi3| over the blocks and home components of an entry of Y_mu (a
+// bound: slightly enlarged), as the bits of a non-negative FP32 value.
+__global__ void __launch_bounds__(256)
+fc3_bound_kernel(int n_groups, const int *__restrict__ group_start, const float2 *__restrict__ fc3, int *l1) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    float s = 0.0f;
+    if (t < 9 * n_groups)
+        for (int b = group_start[t / 9]; b < group_start[t / 9 + 1]; ++b)
+            for (int a = 0; a < 3; ++a) s += fabsf(fc3[(size_t)27 * b + 9 * a + t % 9].x);
+    s *= 1.001f;
+    for (int o = 16; o > 0; o >>= 1) s = fmaxf(s, __shfl_xor_sync(0xffffffffu, s, o));
+    if ((threadIdx.x & 31) == 0) atomicMax(l1, __float_as_int(s));
+}
+// hi/lo FP16 planes of the scaled eigenvectors (padding stays zero from the caller's
+// memset).
+__global__ void split_kernel(int nb, const double2 *__restrict__ eig, const int *__restrict__ e, int ld,
+                             __half *__restrict__ hi, __half *__restrict__ lo) {
+    const size_t n = (size_t)nb * nb;
+    for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < n; x += (size_t)gridDim.x * blockDim.x) {
+        const size_t r = x / nb, c = x % nb;
+        const float v = (float)ldexp(eig[x].x, kEBits - __ldg(e + r));
+        const __half h = __float2half_rn(v);
         hi[r * ld + c] = h;
-        lo[r * ld + c] = __float2bfloat16_rn(v - __bfloat162float(h));
+        lo[r * ld + c] = __float2half_rn(v - __half2float(h));
     }
 }
 
@@ -339,7 +570,7 @@ __device__ __forceinline__ void pair_fma(F2 &acc, float2 a, float2 b) {
     acc.l = __fadd_rn(acc.l, __fadd_rn(r, e));
 }
 
-// YT[c][b] of modes mu0 .. mu0 + nm - 1 straight into their BF16 hi/lo planes
+// YT[c][b] of modes mu0 .. mu0 + nm - 1 straight into their FP16 hi/lo planes
 // (plane stride plane_elems).  Sums of FP32 pairs (about 46 bits), rounded
 // once to FP32 and then split.
 //
@@ -357,7 +588,7 @@ __global__ void __launch_bounds__(256)
 ybuild_pair_kernel(int n_groups, int n_long, const int *__restrict__ order, const int *__restrict__ group_jk,
                    const int *__restrict__ group_start, const int *__restrict__ blk_i,
                    const float2 *__restrict__ fc3, const float2 *__restrict__ Et, int ldm, int mu0, int nm, int ld,
-                   size_t plane_elems, __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo) {
+                   size_t plane_elems, Scales sc, __half *__restrict__ hi, __half *__restrict__ lo) {
     const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     const int m0 = blockIdx.y * MT;
     const bool lng = gw < n_long;                      // uniform over the warp
@@ -399,14 +630,15 @@ ybuild_pair_kernel(int n_groups, int n_long, const int *__restrict__ order, cons
     if (!act || (lng && lane >= 9)) return;
     const int j = group_jk[2 * g], k = group_jk[2 * g + 1];
     const size_t off = (size_t)(3 * k + bg % 3) * ld + 3 * j + bg / 3;
+    const int eL = sc.eL();
 #pragma unroll
     for (int m = 0; m < MT; ++m) {
         if (m0 + m >= nm) break;
-        const float v = __fadd_rn(acc[m].h, acc[m].l);
-        const __nv_bfloat16 h = __float2bfloat16_rn(v);
+        const float v = __fadd_rn(acc[m].h, acc[m].l) * ldexpf(1.0f, kYBits - eL - __ldg(sc.e + mu0 + m0 + m));
+        const __half h = __float2half_rn(v);
         const size_t o = (size_t)(m0 + m) * plane_elems + off;
         hi[o] = h;
-        lo[o] = __float2bfloat16_rn(v - __bfloat162float(h));
+        lo[o] = __float2half_rn(v - __half2float(h));
     }
 }
 
@@ -427,15 +659,15 @@ EncodeTiledFn encode_fn() {
     return fn;
 }
 
-// Tensor map of a BF16 plane [rows][ld] (ld a multiple of 64), box 64 x 128.
-bool make_map(CUtensorMap *map, const __nv_bfloat16 *ptr, int rows, int ld) {
+// Tensor map of an FP16 plane [rows][ld] (ld a multiple of 64), box 64 x 128.
+bool make_map(CUtensorMap *map, const __half *ptr, int rows, int ld) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)ld, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
     const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)kBM};
     const cuuint32_t estr[2] = {1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<__nv_bfloat16 *>(ptr), dims, strides, box,
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<__half *>(ptr), dims, strides, box,
               estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -460,15 +692,22 @@ int tc_gamma_batch_max(int nb, int sms) { return std::max(1, std::min({2 * tc_ga
 // three modes past the last one).
 static int tc_ldm(int nb) { return (nb + 3 + 31) / 32 * 32; }
 
-size_t tc_gamma_scratch_bytes(int nb, int sms, size_t n_fc3) {
+// Row and column sums of the tiles of a batch (EPI_GSYM).
+static size_t tc_gsym_bytes(int nb, int mb) {
+    const size_t nt = (size_t)(nb + kBM - 1) / kBM;
+    return ws_round(sizeof(double) * kBM * (size_t)mb * (nt * (nt + 1) / 2));
+}
+
+size_t tc_gamma_scratch_bytes(int nb, int mb_max, size_t n_fc3, int sym3) {
     const int ld = (nb + kBN - 1) / kBN * kBN;     // whole 128-column tiles per row
     const int rows = (nb + kBM - 1) / kBM * kBM;
-    const size_t plane = ws_round(sizeof(__nv_bfloat16) * (size_t)rows * ld);
+    const size_t plane = ws_round(sizeof(__half) * (size_t)rows * ld);
     // E hi/lo, then Y hi, Y lo, T hi, T lo of every mode of a batch (the largest batch)
-    // then the FP32 pairs of Phi3 and of the eigenvectors
-    return (2 + 4 * (size_t)tc_gamma_batch_max(nb, sms)) * plane + ws_round(sizeof(int) * 4) +
-           ws_round(sizeof(float2) * 27 * std::max<size_t>(n_fc3, 1)) +
-           ws_round(sizeof(float2) * (size_t)nb * tc_ldm(nb));
+    // then the FP32 pairs of Phi3 and of the eigenvectors and the scales, then (Phi3 symmetric under
+    // every permutation) the tiles' sums and the modes' sums over the batches
+    return (2 + 4 * (size_t)mb_max) * plane + ws_round(sizeof(float2) * 27 * std::max<size_t>(n_fc3, 1)) +
+           ws_round(sizeof(float2) * (size_t)nb * tc_ldm(nb)) + ws_round(sizeof(int) * (size_t)(nb + 4)) +
+           (sym3 ? 2 * tc_gsym_bytes(nb, mb_max) + ws_round(sizeof(double) * (size_t)nb) : 0);
 }
 
 // The tensor-core pipeline for one Gamma-only system (Y build, T = E Y^T-form,
@@ -477,34 +716,57 @@ size_t tc_gamma_scratch_bytes(int nb, int sms, size_t n_fc3) {
 cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const LwParams &p, void *scratch,
                                  const std::vector<int2> &tiles, const std::vector<int> &tile_start,
                                  int2 *tiles_dev, int symmetric, double *partial_tc, int *err, int sms,
-                                 cudaStream_t st, int mode_limit) {
+                                 cudaStream_t st, int mode_limit, const double **gacc_out) {
     const int nb = p.nb;
     const int ld = (nb + kBN - 1) / kBN * kBN;     // whole 128-column tiles per row
     const int rows = (nb + kBM - 1) / kBM * kBM;
-    const int mb = (gp.mb > 0) ? std::min(gp.mb, tc_gamma_batch_max(nb, sms)) : tc_gamma_batch(nb, sms);
-    const size_t plane = ws_round(sizeof(__nv_bfloat16) * (size_t)rows * ld);
+    const int mb = std::min(gp.mb > 0 ? gp.mb : tc_gamma_batch(nb, sms), gp.mb_max);
+    const size_t plane = ws_round(sizeof(__half) * (size_t)rows * ld);
     const size_t stack = (size_t)mb * plane;        // one operand plane for every mode of a batch
     char *b = static_cast<char *>(scratch);
-    __nv_bfloat16 *Eh = reinterpret_cast<__nv_bfloat16 *>(b);
-    __nv_bfloat16 *El = reinterpret_cast<__nv_bfloat16 *>(b + plane);
-    auto S = [&](int i) { return reinterpret_cast<__nv_bfloat16 *>(b + 2 * plane + i * stack); };
-    __nv_bfloat16 *Yh = S(0), *Yl = S(1), *Th = S(2), *Tl = S(3);
+    __half *Eh = reinterpret_cast<__half *>(b);
+    __half *El = reinterpret_cast<__half *>(b + plane);
+    auto S = [&](int i) { return reinterpret_cast<__half *>(b + 2 * plane + i * stack); };
+    __half *Yh = S(0), *Yl = S(1), *Th = S(2), *Tl = S(3);
     cudaError_t e = cudaMemsetAsync(b, 0, 2 * plane + 4 * stack, st);
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(err, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
     const int ldm = tc_ldm(nb);
-    char *pairs = b + (2 + 4 * (size_t)tc_gamma_batch_max(nb, sms)) * plane + ws_round(sizeof(int) * 4);
+    char *pairs = b + (2 + 4 * (size_t)gp.mb_max) * plane;
     float2 *fc3p = reinterpret_cast<float2 *>(pairs);
     float2 *Et = reinterpret_cast<float2 *>(pairs + ws_round(sizeof(float2) * 27 * std::max<size_t>(gp.n_fc3, 1)));
+    char *sums = reinterpret_cast<char *>(Et) + ws_round(sizeof(float2) * (size_t)nb * ldm);
+    char *gsums = sums + ws_round(sizeof(int) * (size_t)(nb + 4));
+    double *rowp = nullptr, *colp = nullptr, *gacc = nullptr;
+    // tile_start follows the tiles (same allocation)
+    int *ts = reinterpret_cast<int *>(tiles_dev + std::max<size_t>(tiles.size(), 1));
+    e = cudaMemcpyAsync(ts, tile_start.data(), sizeof(int) * (nb + 1), cudaMemcpyHostToDevice, st);
+    if (e != cudaSuccess) return e;
+    if (gp.sym3) {
+        rowp = reinterpret_cast<double *>(gsums);
+        colp = reinterpret_cast<double *>(gsums + tc_gsym_bytes(nb, gp.mb_max));
+        gacc = reinterpret_cast<double *>(gsums + 2 * tc_gsym_bytes(nb, gp.mb_max));
+        e = cudaMemsetAsync(gacc, 0, sizeof(double) * (size_t)nb, st);
+        if (e != cudaSuccess) return e;
+    }
+    if (gacc_out) *gacc_out = gacc;
     const size_t nf = 27 * gp.n_fc3;
     if (nf) fc3_pair_kernel<<<counted((unsigned)std::min<size_t>((nf + 255) / 256, 4096)), 256, 0, st>>>(nf, d.fc3, fc3p);
     eig_pair_kernel<<<counted(dim3((nb + 31) / 32, (nb + 31) / 32)), 256, 0, st>>>(
         nb, reinterpret_cast<const double2 *>(d.eig), ldm, Et);
-    split_kernel<double2><<<counted(4096), 256, 0, st>>>(nb, nb, reinterpret_cast<const double2 *>(d.eig),
-                                                (size_t)nb, ld, Eh, El);
+    int *l1 = reinterpret_cast<int *>(sums), *em = l1 + 4;
+    e = cudaMemsetAsync(l1, 0, sizeof(int), st);
+    if (e != cudaSuccess) return e;
+    if (gp.n_groups)
+        fc3_bound_kernel<<<counted((9 * gp.n_groups + 255) / 256), 256, 0, st>>>(gp.n_groups, d.group_start, fc3p, l1);
+    mode_scale_kernel<<<counted(nb), 128, 0, st>>>(nb, reinterpret_cast<const double2 *>(d.eig), em);
+    int eR = 0;
+    while ((1LL << eR) < gp.row_entries) ++eR;
+    const Scales sc{l1, em, eR};
+    split_kernel<<<counted(4096), 256, 0, st>>>(nb, reinterpret_cast<const double2 *>(d.eig), em, ld, Eh, El);
     // the planes of one stack are contiguous: plane_elems = plane / 2 elements apart
-    const size_t plane_elems = plane / sizeof(__nv_bfloat16);
+    const size_t plane_elems = plane / sizeof(__half);
     const int stack_rows = (int)((size_t)mb * plane_elems / ld);
     CUtensorMap mEh, mEl, mYh, mYl, mTh, mTl;
     if (plane_elems % ld != 0 || !make_map(&mEh, Eh, rows, ld) || !make_map(&mEl, El, rows, ld) ||
@@ -513,7 +775,7 @@ cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const L
         return cudaErrorInvalidValue;
     const int prow = (int)(plane_elems / ld);      // rows from one plane to the next (>= rows)
     auto k1 = tc_gemm_kernel<EPI_SPLIT>;
-    auto k2 = tc_gemm_kernel<EPI_GAMMA>;
+    auto k2 = gp.sym3 ? tc_gemm_kernel<EPI_GSYM> : tc_gemm_kernel<EPI_GAMMA>;
     e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
     if (e != cudaSuccess) return e;
@@ -539,24 +801,28 @@ cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const L
         auto ybuild = [&](auto kern, int mt) {
             kern<<<counted(dim3(ygx, (nm + mt - 1) / mt)), 256, 0, st>>>(gp.n_groups, gp.n_long, d.group_order,
                                                                          d.group_jk, d.group_start, d.blk_i, fc3p, Et,
-                                                                         ldm, mu0, nm, ld, plane_elems, Yh, Yl);
+                                                                         ldm, mu0, nm, ld, plane_elems, sc, Yh, Yl);
         };
         // modes per thread: 4, or 3 where that leaves fewer of them unused
         if (nm == 1) ybuild(ybuild_pair_kernel<1>, 1);
         else if (nm == 2) ybuild(ybuild_pair_kernel<2>, 2);
         else if ((nm + 2) / 3 * 3 < (nm + 3) / 4 * 4) ybuild(ybuild_pair_kernel<3>, 3);
         else ybuild(ybuild_pair_kernel<4>, 4);
-        EpiSplit es{Th, Tl, ld, prow};
+        // (with sym3 the tiles of a mode start at its own row tile)
+        const int tm0 = gp.sym3 ? mu0 / kBM : 0;
+        EpiSplit es{Th, Tl, ld, prow, tm0};
         EpiGamma eg{};
         ProfMark p1(p.prof, KALD_PROF_TC_GEMM1, st);
-        k1<<<counted(dim3(nt, nt, nm)), 128, kSmemBytes, st>>>(mEh, mEl, mYh, mYl, nb, nb, ld, es, eg, err,
+        k1<<<counted(dim3(nt, nt - tm0, nm)), 128, kSmemBytes, st>>>(mEh, mEl, mYh, mYl, nb, nb, ld, sc, es, eg, err,
                                                                p.wait_limit);
         p1.end();
         EpiGamma eg2{d.omega, d.occ, mu0, prow, sig2inv, p.cut_w, p.shape, partial_tc + t0, d.allowed,
-                     tiles_dev + t0, symmetric};
-        EpiSplit es0{nullptr, nullptr, 0, 0};
+                     tiles_dev + t0, symmetric, rowp, colp};
+        EpiSplit es0{nullptr, nullptr, 0, 0, 0};
         ProfMark p2(p.prof, KALD_PROF_TC_GEMM2, st);
-        k2<<<counted(t1 - t0), 128, kSmemBytes, st>>>(mTh, mTl, mEh, mEl, nb, nb, ld, es0, eg2, err, p.wait_limit);
+        k2<<<counted(t1 - t0), 128, kSmemBytes, st>>>(mTh, mTl, mEh, mEl, nb, nb, ld, sc, es0, eg2, err, p.wait_limit);
+        if (gp.sym3)
+            gsym_sums_kernel<<<counted(nt), 1024, 0, st>>>(nb, mu0, nm, ts, tiles_dev, t0, rowp, colp, gacc);
         p2.end();
     }
     return cudaGetLastError();

@@ -356,3 +356,32 @@ def test_batch_plans_equal_single_calls(k):
     nu3, eig3 = (np.tile(ph1[1][c].ravel(), 3) for c in (0, 1))
     with pytest.raises(kk.KaldError, match="fc3_idx"):
         kk.kald_linewidths(ctx, [small, bad, small], (1, 1, 1), nu3, eig3, opt)
+
+
+@pytest.mark.parametrize("cell,sigma,shape", [((3, 3, 1), 0.02, "gaussian"), ((3, 3, 2), 0.2, "gaussian"),
+                                              ((4, 3, 3), 0.05, "gaussian"), ((4, 3, 3), 0.02, "lorentzian"),
+                                              ((5, 2, 1), 0.1, "triangular")])
+def test_gamma_only_triples_projected_once(k, cell, sigma, shape):
+    """108 to 432 modes (one to four tiles, the last one partial), windows narrower
+    and wider than half the lowest frequencies: each unordered triple of modes
+    projected once gives the linewidths and the exact count of one projection per
+    ordered triple, at the usual workspace and at the smallest."""
+    kk, ctx = k
+    s = ki.fcc_supercell_system(cell, seed=11)
+    nu, eig = ph.phonons(s, (1, 1, 1))
+    def run(**o):
+        opt = kk.Options(temperature_K=300.0, sigma_thz=sigma, delta=shape, **o)
+        return kk.kald_linewidths(ctx, [s], (1, 1, 1), nu.ravel(), eig.ravel(), opt)
+    ref, _ = run(precision="fp64")
+    each, count = run(precision="bf16split", symmetry="inversion")
+    once, count1 = run(precision="bf16split")
+    least = _smallest_workspace(kk, ctx, s, (1, 1, 1), nu, eig,
+                                kk.Options(temperature_K=300.0, sigma_thz=sigma, delta=shape, precision="bf16split"))
+    ctx.set_workspace_limit(least)
+    try:
+        small, count2 = run(precision="bf16split")
+    finally:
+        ctx.set_workspace_limit(0)
+    assert tuple(count) == tuple(count1) == tuple(count2)
+    for g in (each, once, small):
+        assert _rel(g, ref) < 1e-5
