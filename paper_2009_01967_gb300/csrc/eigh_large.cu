@@ -13,7 +13,7 @@
 //      next reflector) in the same pass.  v_k is kept in row k right of the
 //      diagonal (contiguous, read by the back-transformation).
 //   2. Gershgorin interval and |T| on the device, then multisection with
-//      Sturm counts (number of negative pivots of T - x I), one warp per
+//      Sturm counts (number of negative pivots of T - x I), eight lanes per
 //      eigenvalue, to an interval of max(eps |T|, 2 eps |lambda|).
 //   3. Inverse iteration: (T - lambda_i I) x = b solved by tridiagonal LU with
 //      partial pivoting (a zero pivot is replaced by eps |T|), three solves;
@@ -35,8 +35,8 @@
 // reflector k goes into one launch whose CTAs are dealt over the systems in
 // proportion to their remaining rows (cta_start).  Every value is computed by
 // the same threads in the same order as in a solve of the system alone (row
-// dot products by one warp, block sums over a fixed 512 threads, one warp per
-// eigenvalue or vector), so the batch does not change any result.
+// dot products by one warp, block sums over a fixed 512 threads, eight lanes per
+// eigenvalue, one warp per vector), so the batch does not change any result.
 
 #include <algorithm>
 #include <cmath>
@@ -273,11 +273,17 @@ gersh_kernel(const EighSys *__restrict__ sysv) {
 }
 
 // Step 2b: eigenvalue i (ascending) from Sturm counts (tridiag.cuh).
-// Multisection, one warp per eigenvalue: each round the 32 lanes take the
-// Sturm count at the 32 interior points that split the bracket [lo, hi] into
-// 33 equal parts, and the bracket shrinks to the part where the count first
-// exceeds i (lambda_i < x there).  About 11 rounds reach an interval of
+// Multisection, kBisectLanes lanes per eigenvalue: each round they take the Sturm
+// counts at the 8 interior points that split the bracket [lo, hi] into 9 equal
+// parts, and the bracket shrinks to the part where the count first exceeds i
+// (lambda_i < x there).  About 17 rounds reach an interval of
 // max(eps |T|, 2 eps |lambda|).
+//
+// Bound: the FP64 units (three operations per step of a count).  A whole warp per
+// eigenvalue took 11 rounds of 32 counts; eight lanes take 17 of 8, 2.6 times
+// fewer, and four eigenvalues share a warp.  With the rare steps out of the loop as
+// well (sturm_rescale), twelve systems of 324 to 1500 rows 73 -> 12.6 ms.
+constexpr int kBisectLanes = 8;
 __global__ void __launch_bounds__(128)
 bisect_kernel(const EighSys *__restrict__ sysv) {
     const EighSys &S = sysv[blockIdx.y];
@@ -286,25 +292,30 @@ bisect_kernel(const EighSys *__restrict__ sysv) {
     const double *__restrict__ e2 = S.e2;
     const double *__restrict__ g = S.g;
     double *__restrict__ lam = S.lam;
-    const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    const int lane = threadIdx.x & 31;
-    if (i >= n) return;                                // whole warps
-    double lo = g[0], hi = g[1];
+    const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) / kBisectLanes);
+    const int lane = threadIdx.x & (kBisectLanes - 1), grp = (threadIdx.x & 31) / kBisectLanes * kBisectLanes;
+    if (i - grp / kBisectLanes >= n) return;           // whole warps
     const double atol = kEps * g[2], pivmin = g[3];
-    for (int it = 0; it < 64; ++it) {
-        if (hi - lo <= fmax(atol, 2.0 * kEps * fmax(fabs(lo), fabs(hi)))) break;
-        const double x = lo + (hi - lo) * ((double)(lane + 1) / 33.0);
-        const unsigned above = __ballot_sync(0xffffffffu, sturm_count(n, d, e2, x, pivmin) > i);
-        const int f = above ? __ffs(above) - 1 : 32;   // first point above lambda_i
-        const double xf = __shfl_sync(0xffffffffu, x, min(f, 31));
-        const double xp = __shfl_sync(0xffffffffu, x, max(f - 1, 0));
+    double lo = g[0], hi = g[1];
+    bool run = i < n;
+    for (int it = 0; it < 96; ++it) {
+        run = run && !(hi - lo <= fmax(atol, 2.0 * kEps * fmax(fabs(lo), fabs(hi))));
+        if (!__any_sync(0xffffffffu, run)) break;
+        const double x = lo + (hi - lo) * ((double)(lane + 1) / (kBisectLanes + 1.0));
+        const unsigned above = __ballot_sync(0xffffffffu, sturm_count(n, d, e2, x, pivmin) > i) >> grp &
+                               ((1u << kBisectLanes) - 1u);
+        const int f = above ? __ffs(above) - 1 : kBisectLanes;   // first point above lambda_i
+        const double xf = __shfl_sync(0xffffffffu, x, grp + min(f, kBisectLanes - 1));
+        const double xp = __shfl_sync(0xffffffffu, x, grp + max(f - 1, 0));
         const double nlo = (f == 0) ? lo : xp;
-        const double nhi = (f == 32) ? hi : xf;
-        if (nlo <= lo && nhi >= hi) break;            // bracket at machine resolution
-        lo = nlo;
-        hi = nhi;
+        const double nhi = (f == kBisectLanes) ? hi : xf;
+        run = run && !(nlo <= lo && nhi >= hi);        // else: bracket at machine resolution
+        if (run) {
+            lo = nlo;
+            hi = nhi;
+        }
     }
-    if (lane == 0) lam[i] = 0.5 * (lo + hi);
+    if (i < n && lane == 0) lam[i] = 0.5 * (lo + hi);
 }
 
 // Step 3: inverse iteration, one thread per eigenvalue t.  LU factors of
@@ -566,7 +577,7 @@ cudaError_t launch_eigh_large_batch(int n_sys, const EighJob *jobs, void *record
         tri_step_kernel<<<counted(c), kTriThreads, tri_smem, st>>>(dev, map, k);
     }
     gersh_kernel<<<counted(dim3(1, n_sys)), 1024, 0, st>>>(dev);
-    bisect_kernel<<<counted(dim3((unsigned)((n_max + 3) / 4), n_sys)), 128, 0, st>>>(dev);
+    bisect_kernel<<<counted(dim3((unsigned)((n_max * kBisectLanes + 127) / 128), n_sys)), 128, 0, st>>>(dev);
     invit_kernel<<<counted(dim3((unsigned)((n_max + 31) / 32), n_sys)), 32, 0, st>>>(dev);
     mgs_kernel<<<counted(dim3((unsigned)n_max, n_sys)), 256, 0, st>>>(dev);
     // vectors per CTA: about one CTA per SM for the largest system, within the
