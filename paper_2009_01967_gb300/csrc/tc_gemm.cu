@@ -17,7 +17,9 @@
 // (plane b at rows b * rows .. ), GEMM1 takes the mode from blockIdx.z and
 // GEMM2 from its tile record.
 //
-// Kernel shape (one 128 x 128 output tile per CTA, 128 threads):
+// Kernel shape (one 128 x 128 output tile per CTA, 128 threads; 512 for the triples'
+// weights, four warps per 32 rows, since nothing overlaps an epilogue here: with 128
+// threads it took 35 of that product's 50 ms for twelve cells of 324 to 1500 modes):
 //   warp 0 lane 0   TMA producer: 4 tiled loads per K block of 64 (A hi/lo,
 //                   B hi/lo; 128-byte swizzle), 3-stage ring of mbarriers
 //   warp 1          allocates 512 TMEM columns (four accumulators); lane 0 issues the MMAs
@@ -164,8 +166,9 @@ __device__ __forceinline__ float pair_terms(F2 wa, F2 wb, F2 wc, F2 nb_, F2 nc_,
 
 // C[m][n] = sum_k A[m][k] B[n][k]; A, B as FP16 hi/lo planes behind four
 // tensor maps (box 64 x 128, 128-byte swizzle).  Grid: one CTA per tile.
+constexpr int gemm_threads(int epi) { return epi == EPI_GSYM ? 512 : 128; }
 template <int EPI>
-__global__ void __launch_bounds__(128, 1)
+__global__ void __launch_bounds__(gemm_threads(EPI), 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ CUtensorMap mAl,
                const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CUtensorMap mBl,
                int M, int N, int K, Scales sc, EpiSplit es, EpiGamma eg, int *err, uint32_t wait_limit) {
@@ -177,7 +180,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
     __shared__ uint32_t tmem_base_sm;
     __shared__ int fail_sm;
     __shared__ float wn_sm[kBN], wl_sm[kBN], nn_sm[kBN], nl_sm[kBN], cf_sm[kBN];
-    __shared__ double red[4];
+    __shared__ double red[gemm_threads(EPI) / 32];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int tm, tn, bz;                              // tile and mode of the batch
@@ -253,9 +256,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
         ok = false;
         if (threadIdx.x == 0) atomicOr(err, 1);
     }
-    const int row = warp * 32 + lane;            // accumulator lane = tile row
+    const int quad = warp & 3;                   // the 32 lanes a warp may read
+    const int row = quad * 32 + lane;            // accumulator lane = tile row
     const int m = tm * kBM + row;
-    const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
+    const uint32_t taddr = tmem + ((uint32_t)(quad * 32) << 16);
     if (EPI == EPI_SPLIT) {
         // whole tile: rows and columns past M, N hold exact zeros (their A rows
         // / B rows are zero padding) and the planes are allocated to the padded
@@ -294,13 +298,16 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
         // frequency above two windows, differences inside the window are exact but
         // for their last rounding, so that one set serves the three positions;
         // below that each position forms its own (pair_terms).
-        __shared__ float cs_sm[4][kBN];
-        const int nc = tn * kBN + threadIdx.x;
+        constexpr int kCols = kBN / 4;                   // columns of a warp
+        __shared__ float cs_sm[4][kBN], rs_sm[4][kBM];
+        const int tc = threadIdx.x & (kBN - 1), nc = tn * kBN + tc;
         const F2 wcol = nc < N ? f2_of(eg.omega[nc]) : F2{0.f, 0.f};
-        const F2 ncol = nc < N ? f2_of(eg.occ[nc]) : F2{0.f, 0.f};
-        wn_sm[threadIdx.x] = wcol.h; wl_sm[threadIdx.x] = wcol.l;
-        nn_sm[threadIdx.x] = ncol.h; nl_sm[threadIdx.x] = ncol.l;
-        cf_sm[threadIdx.x] = nc < N ? ldexpf(1.0f, __ldg(sc.e + nc)) : 0.0f;
+        if (threadIdx.x < kBN) {
+            const F2 ncol = nc < N ? f2_of(eg.occ[nc]) : F2{0.f, 0.f};
+            wn_sm[tc] = wcol.h; wl_sm[tc] = wcol.l;
+            nn_sm[tc] = ncol.h; nl_sm[tc] = ncol.l;
+            cf_sm[tc] = nc < N ? ldexpf(1.0f, __ldg(sc.e + nc)) : 0.0f;
+        }
         const float cut = (float)eg.cut, s2i = (float)eg.sig2inv;
         const int mu = eg.mu0 + bz;
         const float rf = m < M ? ldexpf(1.0f, __ldg(sc.e + m) + __ldg(sc.e + mu) + sc.eL() + sc.eR - kTBits - kEBits) : 0.0f;
@@ -316,8 +323,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
         const int tmu = mu / kBM;
         float acc1 = 0.0f, acc2 = 0.0f;
         int cnt = 0;
+        const int cq = warp >> 2;
 #pragma unroll 1
-        for (int c0 = 0; c0 < kBN; c0 += 16) {
+        for (int c0 = cq * kCols; c0 < (cq + 1) * kCols; c0 += 16) {
             float v[16];
             tmem_ld_sum16(taddr + c0, v);
             bool any = false;
@@ -363,9 +371,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
             }
             if (__any_sync(0xffffffffu, any)) {
                 const float s = lane_sums16(v);
-                if (!(lane & 1)) cs_sm[warp][c0 + (lane >> 1)] = s;
+                if (!(lane & 1)) cs_sm[quad][c0 + (lane >> 1)] = s;
             } else if (lane < 16) {
-                cs_sm[warp][c0 + lane] = 0.0f;
+                cs_sm[quad][c0 + lane] = 0.0f;
             }
         }
         double accd = (double)acc1;
@@ -376,15 +384,21 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
         }
         if (lane == 0) red[warp] = accd;
         if (lane == 0 && cn && ok) atomicAdd(eg.allowed, cn);
+        rs_sm[cq][row] = acc2;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double s = 0.0;
+            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
+            eg.partial[blockIdx.x] = ok ? s : 0.0;
+        }
         // the other modes' sums, with their own frequency in place of mu's below the line
         const double iw = 1.0 / (double)wmu.h;
         const size_t o = (size_t)blockIdx.x * kBM;
-        eg.rowp[o + threadIdx.x] = ok ? (double)acc2 * ((double)w1 * iw) : 0.0;
-        __syncthreads();
-        if (threadIdx.x == 0) eg.partial[blockIdx.x] = ok ? red[0] + red[1] + red[2] + red[3] : 0.0;
-        const double cs = ((double)cs_sm[0][threadIdx.x] + (double)cs_sm[1][threadIdx.x]) +
-                          ((double)cs_sm[2][threadIdx.x] + (double)cs_sm[3][threadIdx.x]);
-        eg.colp[o + threadIdx.x] = ok ? cs * ((double)wcol.h * iw) : 0.0;
+        auto sum4 = [&](const float (&v)[4][kBM], int x) {
+            return ((double)v[0][x] + (double)v[1][x]) + ((double)v[2][x] + (double)v[3][x]);
+        };
+        if (warp < 4) eg.rowp[o + row] = ok ? sum4(rs_sm, row) * ((double)w1 * iw) : 0.0;
+        else if (warp < 8) eg.colp[o + tc] = ok ? sum4(cs_sm, tc) * ((double)wcol.h * iw) : 0.0;
     } else {
         // delta weights in FP32 (window test first; the FP64 unit is slow),
         // the energy and occupation differences from FP32 pairs (wdiff.cuh)
@@ -820,7 +834,7 @@ cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const L
                      tiles_dev + t0, symmetric, rowp, colp};
         EpiSplit es0{nullptr, nullptr, 0, 0, 0};
         ProfMark p2(p.prof, KALD_PROF_TC_GEMM2, st);
-        k2<<<counted(t1 - t0), 128, kSmemBytes, st>>>(mTh, mTl, mEh, mEl, nb, nb, ld, sc, es0, eg2, err, p.wait_limit);
+        k2<<<counted(t1 - t0), gp.sym3 ? gemm_threads(EPI_GSYM) : 128, kSmemBytes, st>>>(mTh, mTl, mEh, mEl, nb, nb, ld, sc, es0, eg2, err, p.wait_limit);
         if (gp.sym3)
             gsym_sums_kernel<<<counted(nt), 1024, 0, st>>>(nb, mu0, nm, ts, tiles_dev, t0, rowp, colp, gacc);
         p2.end();
