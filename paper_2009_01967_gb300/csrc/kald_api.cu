@@ -281,7 +281,8 @@ static std::vector<int> stable_key_order(int n, long long n_keys, const std::fun
 // exception of f reaches the caller.
 template <typename F>
 static void parallel_for(size_t n, size_t bytes, F &&f) {
-    const size_t nt = std::min<size_t>({n, std::max(1u, std::thread::hardware_concurrency()), 16, 1 + (bytes >> 21)});
+    size_t nt = std::min<size_t>({n, 16, 1 + (bytes >> 21)});
+    if (nt > 1) nt = std::min<size_t>(nt, std::max(1u, std::thread::hardware_concurrency()));   // (reads a file)
     std::atomic<size_t> next{0};
     std::exception_ptr err;
     std::mutex mu;
@@ -1477,20 +1478,23 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
             }
         }
         const int tcx_b = tcx ? tcx_batch_max(nb, nq, ctx->sm_count) : 0;   // scratch for the tuner's largest batch
-        // cells of three or more atoms over the whole mesh with Phi3 symmetric under
-        // permutations: one projection per orbit of momentum triples
+        // the whole mesh with Phi3 symmetric under permutations: one projection per
+        // orbit of momentum triples (the register kernel: while its sums stay within 16 GB)
         int orb_pairs = 0;
         std::vector<int> orb_rows;
-        if (!small && !listed && reuse && opt->symmetry == KALD_SYM_ALL && nq > 1 && lean < 2) {
+        if (!listed && reuse && opt->symmetry == KALD_SYM_ALL && nq > 1 && lean < 2) {
             if (h.fc3_perm_symmetric < 0) fc3_symmetries(&sys[x], h);
             if (h.fc3_perm_symmetric) orb_pairs = std::max(0, orbit_pairs(mesh));
+            if (small && sn_orbit_bytes(nb, orb_pairs, f32w) > (size_t(16) << 30)) orb_pairs = 0;
             if (orb_pairs) {
                 orb_rows.resize(nqc);
                 for (int i = 0; i < nqc; ++i) orb_rows[i] = qsel[i].x;
             }
         }
         const bool use_sym = tcx && orb_pairs;
-        const int cc_pairs = tcx ? 0 : orb_pairs;
+        const int cc_pairs = tcx || small ? 0 : orb_pairs;
+        const size_t sn_out3 = small && orb_pairs ? sn_orbit_work(nb, nq, orb_pairs, f32w) : 0;
+        if (sn_out3) p.n_chunks = 1;
         // tensor-core path: the fc3 blocks in (j, k) group order, the groups
         // split over the gather CTAs
         std::vector<int2> tc_gjk;
@@ -1605,7 +1609,8 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
             need += bytes_of(tp.term_start) + bytes_of(tp.list_start) + bytes_of(tp.glist) + bytes_of(tp.blk) +
                     bytes_of(tp.term) + bytes_of(tp.cterm_start) + bytes_of(tp.cterm) +
                     ws_round(tc_yc);
-        if (orb_pairs) need += bytes_of(orb_rows) + ws_round(orbit_bytes(mesh, nqc)) + ws_round(sizeof(double) * cc_out3);
+        if (orb_pairs) need += bytes_of(orb_rows) + ws_round(orbit_bytes(mesh, nqc)) + ws_round(sizeof(double) * cc_out3) +
+                           ws_round(sn_out3);
         if ((st = ws_reserve(ctx, need))) {
             if (st != KALD_E_NOMEM || lean == 2) return st;
             ++lean;
@@ -1716,7 +1721,8 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
                 e = launch_lw_tables_f32(nq, p.n_rep, terms, d.blkinfo, tg.fc3, static_cast<const float2 *>(d.chi), s);
         }
         if (e == cudaSuccess)
-            e = small ? launch_lw_small(p, d, sn, f32w, s)
+            e = small ? launch_lw_small(p, d, sn, f32w, orb_pairs ? &orb : nullptr,
+                                        sn_out3 ? ws_take(ctx, sn_out3) : nullptr, ctx->sm_count, s)
                 : tcx ? launch_lw_tensor(p, d, tg, tc_scr, tcx_b, ctx->sm_count, tc_err, s,
                                          use_sym ? &orb : nullptr, sym_scr)
                       : launch_lw_main(p, d, terms, f32w, ctx->sm_count, ctx->smem_optin, s);
@@ -1732,7 +1738,7 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         if (errf) return fail(ctx, KALD_E_TIMEOUT, "kald_linewidths: a tensor-core pipeline wait expired");
         tot += (uint64_t)nqr * nq * (uint64_t)nb * nb * nb;
         // one projection per orbit counts three times the orbit's ordered triples
-        allowed_tot += use_sym ? (al + 1) / 3 : cc_pairs ? al / 6 : al;
+        allowed_tot += use_sym ? (al + 1) / 3 : orb_pairs ? al / 6 : al;
         off_nb += (size_t)nq * nb;
         off_eig += nn;
     }

@@ -400,7 +400,13 @@ bool sn_supported(int nb);
 int sn_chunk(int nb, int nq, int sm_count);
 size_t sn_table_bytes(int nb, int nq, int fp32);
 void plan_sn(const HostSystem &h, bool tables, std::vector<int> &order, std::vector<int> &start);
-cudaError_t launch_lw_small(const LwParams &p, const LwDev &d, const SnTables &t, int fp32, cudaStream_t st);
+// orb: one projection per orbit (Phi3 symmetric under permutations, the whole mesh),
+// the positions' sums through out3 (sn_orbit_work bytes).
+size_t sn_orbit_bytes(int nb, int n_pairs, int fp32);
+size_t sn_orbit_work(int nb, int nq, int n_pairs, int fp32);
+struct OrbitPlan;
+cudaError_t launch_lw_small(const LwParams &p, const LwDev &d, const SnTables &t, int fp32, const OrbitPlan *orb,
+                            void *out3, int sms, cudaStream_t st);
 
 // tc_crystal.cu: crystal linewidth sums on tensor cores (BF16 split, nb <= 96).
 // The gather runs over the fc3 blocks grouped by (j, k) atom pair (the order

@@ -157,32 +157,6 @@ __global__ void lw_block_sums_kernel(size_t n, int per, int n_sblk, const double
     }
 }
 
-// Hits of one (s, s', s'') over the six ordered triples (p, a, b) of its three
-// modes: |w_p + w_a - w_b| or |w_p - w_a - w_b| inside the window, each formed
-// in the order in which the projection of (p, a) would form it.
-__device__ __forceinline__ unsigned window_hits6(const F2 (&w)[3], float cut) {
-    unsigned n = 0;
-#pragma unroll
-    for (int p = 0; p < 3; ++p)
-#pragma unroll
-        for (int o = 1; o < 3; ++o) {
-            const F2 a = w[(p + o) % 3], b = w[(p + 3 - o) % 3];
-            n += fabsf(f2_diff(f2_add(w[p], a), b)) < cut || fabsf(f2_diff(f2_add(w[p], f2_neg(a)), b)) < cut;
-        }
-    return n;
-}
-__device__ __forceinline__ unsigned window_hits6(const double (&w)[3], double cut) {
-    unsigned n = 0;
-#pragma unroll
-    for (int p = 0; p < 3; ++p)
-#pragma unroll
-        for (int o = 1; o < 3; ++o) {
-            const double a = w[(p + o) % 3], b = w[(p + 3 - o) % 3];
-            n += fabs(w[p] + a - b) < cut || fabs(w[p] - a - b) < cut;
-        }
-    return n;
-}
-
 // Shared memory of a CTA of sb modes and nthr threads (R2 = complex of the
 // working precision; P = nb rounded up to a multiple of kTR, Q = P + 1):
 //   Y    [sb][P][Q]  Y(b, c) at b*P + c, then T'^T(c, s') at c*Q + s' (odd

@@ -51,6 +51,32 @@ __device__ __forceinline__ float f2_diff(F2 a, F2 b) {
     return __fadd_rn(__fsub_rn(a.h, b.h), __fsub_rn(a.l, b.l));
 }
 
+// Hits of one (s, s', s'') over the six ordered triples (p, a, b) of its three
+// modes: |w_p + w_a - w_b| or |w_p - w_a - w_b| inside the window, each formed
+// in the order in which the projection of (p, a) would form it.
+__device__ __forceinline__ unsigned window_hits6(const F2 (&w)[3], float cut) {
+    unsigned n = 0;
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+#pragma unroll
+        for (int o = 1; o < 3; ++o) {
+            const F2 a = w[(p + o) % 3], b = w[(p + 3 - o) % 3];
+            n += fabsf(f2_diff(f2_add(w[p], a), b)) < cut || fabsf(f2_diff(f2_add(w[p], f2_neg(a)), b)) < cut;
+        }
+    return n;
+}
+__device__ __forceinline__ unsigned window_hits6(const double (&w)[3], double cut) {
+    unsigned n = 0;
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+#pragma unroll
+        for (int o = 1; o < 3; ++o) {
+            const double a = w[(p + o) % 3], b = w[(p + 3 - o) % 3];
+            n += fabs(w[p] + a - b) < cut || fabs(w[p] - a - b) < cut;
+        }
+    return n;
+}
+
 // Energy-delta shapes of the epilogues, without their normalisation (applied
 // per mode at the end, delta_norm): 0 Gaussian exp(-a d^2), a = 1/(2 sigma^2);
 // 1 Lorentzian 1/(1 + a d^2), a = 1/sigma^2; 2 triangle max(0, 1 - a |d|),

@@ -385,3 +385,24 @@ def test_gamma_only_triples_projected_once(k, cell, sigma, shape):
     assert tuple(count) == tuple(count1) == tuple(count2)
     for g in (each, once, small):
         assert _rel(g, ref) < 1e-5
+
+
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-10), ("fp32", 1e-5)])
+@pytest.mark.parametrize("atoms,mesh,sigma", [(2, (2, 1, 1), 0.2), (2, (3, 3, 3), 0.1), (2, (5, 4, 2), 0.05),
+                                              (1, (4, 4, 4), 0.2), (1, (7, 3, 1), 0.1)])
+def test_register_kernel_orbits(k, atoms, mesh, sigma, precision, tol):
+    """One- and two-atom cells, meshes with and without self-inverse and 3 q = 0
+    points, fewer and more orbits than a pass holds: one projection per orbit gives
+    the linewidths of the oracle and the exact count of one projection per pair."""
+    from oracle import anharmonic as an
+    kk, ctx = k
+    w = ki.small_binary(mesh=mesh, sigma=sigma) if atoms == 2 else ki.small_fcc_prim(mesh=mesh, sigma=sigma)
+    s = w.systems[0]
+    nu, eig = ph.phonons(s, mesh)
+    g_o = an.linewidths(s, mesh, nu, eig, w.T, sigma, 3.0)
+    count = {}
+    for sym in ("all", "inversion", "none"):
+        opt = kk.Options(temperature_K=w.T, sigma_thz=sigma, precision=precision, symmetry=sym)
+        g, count[sym] = kk.kald_linewidths(ctx, s, mesh, nu, eig, opt)
+        assert _rel(g.reshape(g_o.shape), g_o) < tol
+    assert count["all"] == count["inversion"] == count["none"]
