@@ -156,13 +156,24 @@ __global__ void g_gamma_kernel(int nb, int n_part, const double *__restrict__ pa
 // (ties by index), then the thread of each chain's first mode averages the
 // chain |d nu| < tol in ascending order (one thread walking the whole list
 // took 0.17 ms for 768 modes).
+// (compared as integers that order like the values: the FP64 unit took 96 us for 768
+// modes; NaN sorts by its bits, and -0 with 0)
+__device__ __forceinline__ long long sort_key(double x) {
+    const long long b = __double_as_longlong(x + 0.0);
+    return b < 0 ? (long long)(0x8000000000000000ull) - b : b;
+}
 __global__ void g_rank_kernel(int nb, const double *__restrict__ nu, int *__restrict__ order) {
+    __shared__ long long key[128];
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nb) return;
-    const double v = nu[s];
+    const long long v = s < nb ? sort_key(nu[s]) : 0;
     int r = 0;
-    for (int t = 0; t < nb; ++t) r += (nu[t] < v) || (nu[t] == v && t < s);
-    order[r] = s;
+    for (int t0 = 0; t0 < nb; t0 += 128) {
+        __syncthreads();
+        if (t0 + threadIdx.x < nb) key[threadIdx.x] = sort_key(nu[t0 + threadIdx.x]);
+        __syncthreads();
+        for (int t = 0; t < min(128, nb - t0); ++t) r += key[t] < v || (key[t] == v && t0 + t < s);
+    }
+    if (s < nb) order[r] = s;
 }
 __global__ void g_degen_kernel(int nb, const double *__restrict__ nu, const int *__restrict__ order,
                                double tol, double *__restrict__ gamma) {
@@ -260,7 +271,7 @@ static std::map<std::array<int, 4>, int> g_mb_tuned;      // by (nb, SMs, larges
 
 int tune_gamma_batch(const GammaPlan &gp, const GammaDev &d, const LwParams &p, cudaStream_t st) {
     const int nb = p.nb, sms = gp.sms;
-    const int mbx = gp.mb_max, def = std::min(tc_gamma_batch(nb, sms), mbx);
+    const int mbx = gp.mb_max, def = std::min(tc_gamma_batch(nb, sms, gp.sym3), mbx);
     const std::array<int, 4> key{nb, sms, mbx, gp.sym3};
     {
         std::lock_guard<std::mutex> lock(g_mb_mu);

@@ -1157,7 +1157,8 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
             // contraction and a third of the second (256 atoms 7.7 -> 4.6 ms, twelve
             // cells of 108 to 500 atoms 451 -> 335 ms)
             gp.sym3 = !lean && opt->symmetry == KALD_SYM_ALL && h.fc3_perm_symmetric;
-            gp.mb_max = lean ? std::max(1, tc_gamma_batch(nb, ctx->sm_count) / 2) : tc_gamma_batch_max(nb, ctx->sm_count);
+            gp.mb_max = lean ? std::max(1, tc_gamma_batch(nb, ctx->sm_count, 0) / 2)
+                             : tc_gamma_batch_max(nb, ctx->sm_count, gp.sym3);
             gp.n_long = h.pair3_long;
             band_tiles(gp.omega_h, tc_tile(), opt->n_sigma * kTwoPi * opt->sigma_thz, gp.symmetric, gp.sym3, gp.tiles,
                        gp.tile_start);

@@ -373,8 +373,8 @@ cudaError_t launch_gamma_only(const GammaPlan &gp, const GammaDev &d, const LwPa
 // before that).  The timing runs use the system's own buffers.
 int tune_gamma_batch(const GammaPlan &gp, const GammaDev &d, const LwParams &p, cudaStream_t st);
 // modes per launch of the tensor-core Gamma-only path and its scratch bytes
-int tc_gamma_batch(int nb, int sms);
-int tc_gamma_batch_max(int nb, int sms);
+int tc_gamma_batch(int nb, int sms, int sym3);
+int tc_gamma_batch_max(int nb, int sms, int sym3);
 size_t tc_gamma_scratch_bytes(int nb, int mb_max, size_t n_fc3, int sym3);
 int tc_tile(void);
 cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const LwParams &p, void *scratch,
