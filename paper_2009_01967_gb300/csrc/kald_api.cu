@@ -1943,16 +1943,21 @@ kald_status kald_phase_space(kald_ctx *ctx, const kald_system *sys, const int32_
     const bool d_nu = is_device_ptr(nu_thz), d_g = is_device_ptr(g);
     const int f32 = opt->precision != KALD_FP64;
     const size_t nm = (size_t)nq * nb;
-    size_t need = bytes_of(qf) + 2 * ws_round(sizeof(double) * nm) + ws_round(phase_space_bytes(nb, nq, ctx->sm_count));
-    if (!d_nu) need += ws_round(sizeof(double) * nm);
-    if (!d_g) need += ws_round(sizeof(double) * nm);
-    if ((st = ws_reserve(ctx, need))) return st;
+    int lean = 0;            // where the workspace cannot be had: no chunks
+    for (;; lean = 1) {
+        size_t need = bytes_of(qf) + 2 * ws_round(sizeof(double) * nm) +
+                      ws_round(phase_space_bytes(nb, nq, ctx->sm_count, lean));
+        if (!d_nu) need += ws_round(sizeof(double) * nm);
+        if (!d_g) need += ws_round(sizeof(double) * nm);
+        if (!(st = ws_reserve(ctx, need))) break;
+        if (st != KALD_E_NOMEM || lean) return st;
+    }
     LwDev d{};
     d.qfrac = upload(ctx, qf);
     d.nu = stage_in(ctx, nu_thz, nm, d_nu);
     d.omega = static_cast<double *>(ws_take(ctx, sizeof(double) * nm));
     d.occ = static_cast<double *>(ws_take(ctx, sizeof(double) * nm));
-    void *work = ws_take(ctx, phase_space_bytes(nb, nq, ctx->sm_count));
+    void *work = ws_take(ctx, phase_space_bytes(nb, nq, ctx->sm_count, lean));
     double *g_d = d_g ? g : static_cast<double *>(ws_take(ctx, sizeof(double) * nm));
     LwParams p{};
     p.nb = nb; p.nq = nq;
@@ -1967,7 +1972,7 @@ kald_status kald_phase_space(kald_ctx *ctx, const kald_system *sys, const int32_
     p.wait_limit = ctx->wait_limit;
     p.prof = &ctx->prof;
     cudaError_t e = launch_mode_prep((int)nm, d.nu, p.omega_min_w, p.T, p.classical, d.omega, d.occ, ctx->stream);
-    if (e == cudaSuccess) e = launch_phase_space(p, d, f32, ctx->sm_count, work, g_d, ctx->stream);
+    if (e == cudaSuccess) e = launch_phase_space(p, d, f32, ctx->sm_count, work, lean, g_d, ctx->stream);
     if (e != cudaSuccess) return cuda_check(ctx, e, "kald_phase_space launch");
     if (!d_g) cudaMemcpyAsync(g, g_d, sizeof(double) * nm, cudaMemcpyDeviceToHost, ctx->stream);
     return finish(ctx, "kald_phase_space");

@@ -528,9 +528,9 @@ cudaError_t launch_diffusivity(const DevFc2Dist &f, int nb, const double *nu_thz
                                cudaStream_t st);
 // Phase space per mode (linewidths.cu): g [nq * nb] in ps; work of
 // phase_space_bytes (sorted modes, counts, partial sums of the q' chunks).
-size_t phase_space_bytes(int nb, int nq, int sm_count);
-cudaError_t launch_phase_space(const LwParams &p, const LwDev &d, int fp32, int sm_count, void *work, double *g_out,
-                               cudaStream_t st);
+size_t phase_space_bytes(int nb, int nq, int sm_count, int lean);
+cudaError_t launch_phase_space(const LwParams &p, const LwDev &d, int fp32, int sm_count, void *work, int lean,
+                               double *g_out, cudaStream_t st);
 cudaError_t launch_qhgk(const DevFc2Dist &f, int nb, const double *nu_thz, const double2 *eig,
                         const double *gamma, double T, int classical, double omega_min_thz,
                         double degen_tol_thz, double bandwidth_w, double threshold_w, int antisym, int fill,

@@ -666,19 +666,25 @@ lw_finish_kernel(int nb, int n_chunks, const double *__restrict__ partial, const
     }
 }
 
-// The live modes of every q-point in ascending frequency (ties by index),
-// count[q] of them: omega and n in FP64, and their FP32 pairs when wn is given.
+// The live modes of every q-point in ascending frequency (ties by index), then
+// kNoMode as frequency: omega and n in FP64, or their FP32 pairs when wn is given.
+constexpr float kNoMode = 1e30f;
 __global__ void sort_modes_kernel(int nb, const double *__restrict__ omega, const double *__restrict__ occ,
-                                  double2 *__restrict__ wn64, float4 *__restrict__ wn, int *__restrict__ count) {
+                                  double2 *__restrict__ wn64, float4 *__restrict__ wn) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *w = reinterpret_cast<double *>(smem_raw);
     const size_t row = (size_t)blockIdx.x * nb;
     for (int x = threadIdx.x; x < nb; x += blockDim.x) w[x] = omega[row + x];
-    if (threadIdx.x == 0) count[blockIdx.x] = 0;
     __syncthreads();
     for (int x = threadIdx.x; x < nb; x += blockDim.x) {
         const double v = w[x];
-        if (!(v > 0.0)) continue;
+        if (!(v > 0.0)) {                                // behind the live ones, in any order
+            int r = nb - 1;
+            for (int y = 0; y < x; ++y) r -= !(w[y] > 0.0);
+            if (wn64) wn64[row + r] = make_double2(kNoMode, 0.0);
+            if (wn) wn[row + r] = make_float4(kNoMode, 0.f, 0.f, 0.f);
+            continue;
+        }
         int r = 0;
         for (int y = 0; y < nb; ++y) r += w[y] > 0.0 && (w[y] < v || (w[y] == v && y < x));
         const double n = occ[row + x];
@@ -687,8 +693,40 @@ __global__ void sort_modes_kernel(int nb, const double *__restrict__ omega, cons
             const F2 a = f2_of(v), o = f2_of(n);
             wn[row + r] = make_float4(a.h, a.l, o.h, o.l);
         }
-        atomicAdd(count + blockIdx.x, 1);
     }
+}
+
+// -q of a mesh point.
+__device__ __forceinline__ int neg_point(const int *__restrict__ k, const int (&mesh)[3]) {
+    const int a = k[0] ? mesh[0] - k[0] : 0, b = k[1] ? mesh[1] - k[1] : 0, c = k[2] ? mesh[2] - k[2] : 0;
+    return (a * mesh[1] + b) * mesh[2] + c;
+}
+// *differ |= 1 unless every q-point has the frequencies of -q, to 4e-13 of its largest
+// (two diagonalisations of D(q) and of its conjugate agree to some 1e-14; the sums of
+// -q are then those of q to 1e-10).
+template <typename M>
+__global__ void __launch_bounds__(128)
+mirror_check_kernel(LwParams p, const int *__restrict__ qfrac, const M *__restrict__ modes, int *__restrict__ differ) {
+    __shared__ double top[4];
+    const int q = blockIdx.x, m = neg_point(qfrac + 3 * q, p.mesh);
+    if (m <= q) return;
+    auto freq = [&](int k, int x) {
+        const M a = modes[(size_t)k * p.nb + x];
+        if constexpr (std::is_same<M, float4>::value) return (double)a.x + (double)a.y;
+        else return a.x;
+    };
+    double mx = 0.0;
+    for (int x = threadIdx.x; x < p.nb; x += blockDim.x) {
+        const double w = freq(q, x);
+        if (w < (double)kNoMode) mx = fmax(mx, w);
+    }
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((threadIdx.x & 31) == 0) top[threadIdx.x >> 5] = mx;
+    __syncthreads();
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) mx = fmax(mx, top[w]);
+    bool d = false;
+    for (int x = threadIdx.x; x < p.nb; x += blockDim.x) d |= !(fabs(freq(q, x) - freq(m, x)) <= 4e-13 * mx);
+    if (__syncthreads_or(d) && threadIdx.x == 0) atomicOr(differ, 1);
 }
 
 // Phase space per mode (the definition after Eq. delta_deconstructed, with
@@ -696,7 +734,8 @@ __global__ void sort_modes_kernel(int nb, const double *__restrict__ omega, cons
 // on the - process, 1/N_k, masked modes):
 //   g_mu = (1/N_k) sum_{q' s' s''} [(n' - n'') G(w + w' - w'') + 1/2 (1 + n' + n'') G(w - w' - w'')],
 // q'' = q + q' for both processes (the - process of (q, -q') has the same
-// frequencies, since w(-q) = w(q)).  CTA = (q, block of s, chunk of q'), one
+// frequencies, since w(-q) = w(q)); where the input says so (mirror_check_kernel), one
+// q-point of each pair {q, -q}.  CTA = (q, block of s, chunk of q'), one
 // thread per s, FP64 sums over q', one partial sum per chunk.  FP64, or FP32
 // weights with the compensated differences.
 //
@@ -705,16 +744,17 @@ __global__ void sort_modes_kernel(int nb, const double *__restrict__ omega, cons
 // near ends and walks only the modes inside (about a seventh of them per
 // window at 3 sigma = 0.15 THz of a 2 THz band); the exact test of the window
 // decides, the walk is a little wider.  32 atoms, 6^3 mesh, FP32: 143 ms when
-// every (s', s'') was tested by one thread per (q, s), 10.9 ms now.
+// every (s', s'') was tested by one thread per (q, s), 5.3 ms now (half of the q-points).
 template <typename R>
 __global__ void __launch_bounds__(128)
-phase_space_kernel(LwParams p, LwDev d, const void *__restrict__ modes, const int *__restrict__ count, int chunk,
+phase_space_kernel(LwParams p, LwDev d, const void *__restrict__ modes, const int *__restrict__ differ, int chunk,
                    double *__restrict__ partial) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr bool kPair = std::is_same<R, float>::value;
     const int nb = p.nb;
     const int per_q = (nb + blockDim.x - 1) / blockDim.x;          // CTAs per q and chunk
     const int q = (int)blockIdx.x / per_q;
+    if (differ && *differ == 0 && neg_point(d.qfrac + 3 * q, p.mesh) < q) return;   // -q's sums are taken
     const int s = ((int)blockIdx.x % per_q) * blockDim.x + threadIdx.x;
     // modes of q' and q'': FP32 pairs (w hi, w lo, n hi, n lo), or FP64 (w, n)
     using M = typename std::conditional<kPair, float4, double2>::type;
@@ -731,13 +771,21 @@ phase_space_kernel(LwParams p, LwDev d, const void *__restrict__ modes, const in
         const int *kq = d.qfrac + 3 * q, *kp = d.qfrac + 3 * qp;
         const int qpp = (((kq[0] + kp[0]) % p.mesh[0]) * p.mesh[1] + (kq[1] + kp[1]) % p.mesh[1]) * p.mesh[2] +
                         (kq[2] + kp[2]) % p.mesh[2];
-        const int m1 = count[qp], m2 = count[qpp];
+        int m1 = 0, m2 = 0;                    // live modes of q' and q''
         __syncthreads();
-        for (int x = threadIdx.x; x < max(m1, m2); x += blockDim.x) {
-            if (x < m1) f1[x] = all[(size_t)qp * nb + x];
-            if (x < m2) f2[x] = all[(size_t)qpp * nb + x];
+        for (int x0 = 0; x0 < nb; x0 += blockDim.x) {
+            const int x = x0 + threadIdx.x;
+            bool l1 = false, l2 = false;
+            if (x < nb) {
+                const M a1 = all[(size_t)qp * nb + x], a2 = all[(size_t)qpp * nb + x];
+                f1[x] = a1;
+                f2[x] = a2;
+                l1 = a1.x < (R)kNoMode;
+                l2 = a2.x < (R)kNoMode;
+            }
+            m1 += __syncthreads_count(l1);
+            m2 += __syncthreads_count(l2);
         }
-        __syncthreads();
         if (!(w_s > 0.0) || m1 == 0 || m2 == 0) continue;
         // half width of the walk: the window, plus the rounding of sums of three frequencies
         const R wide = cut * (R)1.0001 + (kPair ? (R)1e-6 : (R)1e-14) * (w + f1[m1 - 1].x + f2[m2 - 1].x);
@@ -793,13 +841,30 @@ phase_space_kernel(LwParams p, LwDev d, const void *__restrict__ modes, const in
     if (s < nb) partial[((size_t)blockIdx.y * p.nq + q) * nb + s] = sum;
 }
 
-// g[x] = scale * sum of the chunks' partial sums in order.
-__global__ void phase_space_sum_kernel(size_t n, int n_chunks, const double *__restrict__ partial, double scale,
-                                       double *__restrict__ g) {
-    const size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+// g[x] = scale * sum of the chunks' partial sums in order (partial may be g); for a
+// q-point left out, those of -q's mode of the same frequency.
+__global__ void phase_space_sum_kernel(LwParams p, const int *__restrict__ qfrac, const double *__restrict__ omega,
+                                       const int *__restrict__ differ, int n_chunks, const double *partial, double scale,
+                                       double *g) {
+    const size_t n = (size_t)p.nq * p.nb, x = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     if (x >= n) return;
+    size_t y = x;
+    if (differ && *differ == 0) {
+        const int q = (int)(x / p.nb), m = neg_point(qfrac + 3 * q, p.mesh);
+        if (m < q) {
+            const double w = omega[x];
+            double best = 1e300;
+            for (size_t z = (size_t)m * p.nb; z < (size_t)(m + 1) * p.nb; ++z) {
+                const double e = fabs(omega[z] - w);
+                if (e < best) {
+                    best = e;
+                    y = z;
+                }
+            }
+        }
+    }
     double t = 0.0;
-    for (int c = 0; c < n_chunks; ++c) t += partial[(size_t)c * n + x];
+    for (int c = 0; c < n_chunks; ++c) t += partial[(size_t)c * n + y];
     g[x] = scale * t;
 }
 
@@ -978,43 +1043,53 @@ void plan_lw_terms(const HostSystem &h, bool tables, LwTermsHost &o) {
     }
 }
 
-// q' chunks of the phase-space sum: about eight CTAs per SM.
+// q' chunks of the phase-space sum: about 26 CTAs per SM, two waves of three warps each
+// (eight left the SMs uneven: 6.9 ms where 26 take 5.3 for 32 atoms on 6^3).
 static int phase_space_chunks(int nb, int nq, int sm_count) {
-    const long long rows = (long long)nq * ((nb + 127) / 128);
-    return (int)std::max(1LL, std::min<long long>(std::min(nq, 1024), (8LL * std::max(1, sm_count) + rows - 1) / rows));
+    const long long rows = (long long)(nq / 2 + 1) * ((nb + 127) / 128);      // (half of the q-points as a rule)
+    return (int)std::max(1LL, std::min<long long>(std::min(nq, 1024), (26LL * std::max(1, sm_count) + rows - 1) / rows));
 }
-size_t phase_space_bytes(int nb, int nq, int sm_count) {
+// (lean: the sorted modes alone, one chunk straight into the result)
+size_t phase_space_bytes(int nb, int nq, int sm_count, int lean) {
     const size_t n = (size_t)nb * nq;
-    return ws_round(16 * n) + ws_round(sizeof(int) * (size_t)nq) +
-           ws_round(sizeof(double) * n * phase_space_chunks(nb, nq, sm_count));
+    return ws_round(16 * n) +
+           (lean ? 0 : ws_round(sizeof(int)) + ws_round(sizeof(double) * n * phase_space_chunks(nb, nq, sm_count)));
 }
 
-cudaError_t launch_phase_space(const LwParams &p, const LwDev &d, int fp32, int sm_count, void *work, double *g_out,
-                               cudaStream_t st) {
+cudaError_t launch_phase_space(const LwParams &p, const LwDev &d, int fp32, int sm_count, void *work, int lean,
+                               double *g_out, cudaStream_t st) {
     const size_t n = (size_t)p.nb * p.nq;
     char *w = static_cast<char *>(work);
     void *modes = w;
-    int *count = reinterpret_cast<int *>(w + ws_round(16 * n));
-    double *partial = reinterpret_cast<double *>(w + ws_round(16 * n) + ws_round(sizeof(int) * (size_t)p.nq));
-    const int n_chunks0 = phase_space_chunks(p.nb, p.nq, sm_count);
+    int *differ = lean ? nullptr : reinterpret_cast<int *>(w + ws_round(16 * n));
+    double *partial = lean ? g_out : reinterpret_cast<double *>(w + ws_round(16 * n) + ws_round(sizeof(int)));
+    const int n_chunks0 = lean ? 1 : phase_space_chunks(p.nb, p.nq, sm_count);
     const int chunk = (p.nq + n_chunks0 - 1) / n_chunks0, n_chunks = (p.nq + chunk - 1) / chunk;
     const int threads = std::min(128, (p.nb + 31) / 32 * 32);
     const int per_q = (p.nb + threads - 1) / threads;
     const size_t ssort = sizeof(double) * (size_t)p.nb, smem = 2 * sizeof(float4) * (size_t)p.nb;
     cudaError_t e = cudaFuncSetAttribute(sort_modes_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssort);
     if (e != cudaSuccess) return e;
-    sort_modes_kernel<<<counted(p.nq), threads, ssort, st>>>(p.nb, d.omega, d.occ,
-                                                             fp32 ? nullptr : static_cast<double2 *>(modes),
-                                                             fp32 ? static_cast<float4 *>(modes) : nullptr, count);
+    auto *wn64 = static_cast<double2 *>(modes);
+    auto *wn32 = static_cast<float4 *>(modes);
+    sort_modes_kernel<<<counted(p.nq), threads, ssort, st>>>(p.nb, d.omega, d.occ, fp32 ? nullptr : wn64,
+                                                             fp32 ? wn32 : nullptr);
+    if (differ) {
+        e = cudaMemsetAsync(differ, 0, sizeof(int), st);
+        if (e != cudaSuccess) return e;
+        if (fp32) mirror_check_kernel<float4><<<counted(p.nq), threads, 0, st>>>(p, d.qfrac, wn32, differ);
+        else mirror_check_kernel<double2><<<counted(p.nq), threads, 0, st>>>(p, d.qfrac, wn64, differ);
+    }
     const double scale = delta_norm(p.shape, p.sigma_w) / (double)p.nq;
     auto k32 = phase_space_kernel<float>;
     auto k64 = phase_space_kernel<double>;
     e = cudaFuncSetAttribute(fp32 ? k32 : k64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)(p.nq * per_q), (unsigned)n_chunks);
-    if (fp32) k32<<<counted(grid), threads, smem, st>>>(p, d, modes, count, chunk, partial);
-    else k64<<<counted(grid), threads, smem, st>>>(p, d, modes, count, chunk, partial);
-    phase_space_sum_kernel<<<counted((unsigned)((n + 255) / 256)), 256, 0, st>>>(n, n_chunks, partial, scale, g_out);
+    if (fp32) k32<<<counted(grid), threads, smem, st>>>(p, d, modes, differ, chunk, partial);
+    else k64<<<counted(grid), threads, smem, st>>>(p, d, modes, differ, chunk, partial);
+    phase_space_sum_kernel<<<counted((unsigned)((n + 255) / 256)), 256, 0, st>>>(p, d.qfrac, d.omega, differ, n_chunks,
+                                                                               partial, scale, g_out);
     return cudaGetLastError();
 }
 

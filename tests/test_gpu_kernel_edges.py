@@ -406,3 +406,35 @@ def test_register_kernel_orbits(k, atoms, mesh, sigma, precision, tol):
         g, count[sym] = kk.kald_linewidths(ctx, s, mesh, nu, eig, opt)
         assert _rel(g.reshape(g_o.shape), g_o) < tol
     assert count["all"] == count["inversion"] == count["none"]
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("mesh", [(4, 3, 2), (1, 5, 1)])
+@pytest.mark.parametrize("change", [0.0, 1e-14, 1e-3])
+def test_phase_space_of_mirrored_frequencies(k, mesh, change, precision):
+    """Frequencies of -q equal to those of q, to rounding, or not: the sums of one
+    q-point of each pair, or of both, are those of the smallest workspace, where
+    every q-point is summed by itself (1e-10: 4e-13 of the largest frequency moves a
+    Gaussian weight by 3 w_max / sigma times that; FP32 1e-5 of the mode)."""
+    import re
+    kk, ctx = k
+    s = ki.small_binary(mesh=mesh).systems[0]
+    nq, nb = int(np.prod(mesh)), 6
+    rng = np.random.default_rng(3)
+    nu = rng.uniform(0.3, 2.0, (nq, nb))
+    neg = np.array([np.ravel_multi_index(tuple((-np.array(np.unravel_index(q, mesh))) % mesh), mesh) for q in range(nq)])
+    nu = np.where((neg < np.arange(nq))[:, None], nu[neg], nu)
+    last = int(np.flatnonzero(neg < np.arange(nq))[-1])
+    nu[last, 3] *= 1.0 + change
+    opt = kk.Options(temperature_K=300.0, sigma_thz=0.05, precision=precision)
+    g = kk.kald_phase_space(ctx, s, mesh, nu, opt)
+    ctx.set_workspace_limit(1)
+    try:
+        with pytest.raises(kk.KaldError) as e:
+            kk.kald_phase_space(ctx, s, mesh, nu, opt)
+        ctx.set_workspace_limit(int(re.search(r"needs (\d+) bytes", str(e.value)).group(1)))
+        ref = kk.kald_phase_space(ctx, s, mesh, nu, opt)
+    finally:
+        ctx.set_workspace_limit(0)
+    assert np.max(np.abs(g - ref)) <= (1e-10 if precision == "fp64" else 1e-5) * np.max(np.abs(ref))
+    assert np.all(np.asarray(ref) > 0)
