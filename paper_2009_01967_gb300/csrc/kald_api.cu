@@ -1168,7 +1168,7 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
                    scaled_bytes(h.fc3_blk, h.fc3_atoms, h, 27, 27, 0) + 2 * ws_round(sizeof(double) * nb) +
                    ws_round(sizeof(int) * nb);
         if (mode == KALD_BF16_SPLIT)
-            b += tc_gamma_scratch_bytes(nb, gp.mb_max, gp.n_fc3, gp.sym3) + bytes_of(h.pair3_order) + ws_round(sizeof(int2) * n_tiles + sizeof(int) * (nb + 1)) +
+            b += tc_gamma_scratch_bytes(nb, gp.mb_max, gp.n_fc3, gp.sym3, gp.tiles.size()) + bytes_of(h.pair3_order) + ws_round(sizeof(int2) * n_tiles + sizeof(int) * (nb + 1)) +
                  ws_round(sizeof(double) * n_tiles);
         else
             b += 4 * ws_round(rs * nn) + ws_round(sizeof(double) * nb * (size_t)gp.n_part);
@@ -1206,7 +1206,8 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
         gd.group_order = nullptr;
         gd.tc_scratch = nullptr; gd.tiles_dev = nullptr; gd.partial_tc = nullptr;
         if (mode == KALD_BF16_SPLIT) {
-            gd.tc_scratch = ws_take(ctx, tc_gamma_scratch_bytes(nb, it.gp.mb_max, it.gp.n_fc3, it.gp.sym3));
+            gd.tc_scratch = ws_take(ctx, tc_gamma_scratch_bytes(nb, it.gp.mb_max, it.gp.n_fc3, it.gp.sym3,
+                                                                it.gp.tiles.size()));
             gd.group_order = upload(ctx, h.pair3_order);
             gd.tiles_dev = static_cast<int2 *>(ws_take(ctx, sizeof(int2) * n_tiles + sizeof(int) * (nb + 1)));
             gd.partial_tc = static_cast<double *>(ws_take(ctx, sizeof(double) * n_tiles));

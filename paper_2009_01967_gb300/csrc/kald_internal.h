@@ -375,7 +375,7 @@ int tune_gamma_batch(const GammaPlan &gp, const GammaDev &d, const LwParams &p, 
 // modes per launch of the tensor-core Gamma-only path and its scratch bytes
 int tc_gamma_batch(int nb, int sms, int sym3);
 int tc_gamma_batch_max(int nb, int sms, int sym3);
-size_t tc_gamma_scratch_bytes(int nb, int mb_max, size_t n_fc3, int sym3);
+size_t tc_gamma_scratch_bytes(int nb, int mb_max, size_t n_fc3, int sym3, size_t n_tiles);
 int tc_tile(void);
 cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const LwParams &p, void *scratch,
                                  const std::vector<int2> &tiles, const std::vector<int> &tile_start,

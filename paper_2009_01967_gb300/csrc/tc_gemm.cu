@@ -481,33 +481,32 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
     }
 }
 
-// gacc[m] += the sums that the tiles of the batch's modes mu0 .. mu0 + nm - 1 leave for
-// mode m (EPI_GSYM): tile by tile within a mode, mode by mode, whatever the batch.
-// One CTA per 128 modes m; partial sums of a mode of the batch per 128 threads.
-__global__ void __launch_bounds__(1024)
-gsym_sums_kernel(int nb, int mu0, int nm, const int *__restrict__ tile_start, const int2 *__restrict__ tiles, int t0,
-                 const double *__restrict__ rowp, const double *__restrict__ colp, double *__restrict__ gacc) {
-    __shared__ double sm[32][kBM];
-    const int t = blockIdx.x, x = threadIdx.x & (kBM - 1), m = t * kBM + x;
-    const bool own = threadIdx.x < kBM && m < nb;
-    double v = own ? gacc[m] : 0.0;
-    for (int b0 = 0; b0 < nm; b0 += 32) {
-        const int b1 = min(nm, b0 + 32);
-        for (int b = b0 + threadIdx.x / kBM; b < b1; b += blockDim.x / kBM) {
-            double s = 0.0;
-            for (int y = tile_start[mu0 + b]; y < tile_start[mu0 + b + 1]; ++y) {
-                const int2 r = __ldg(tiles + y);
-                if ((r.x & 0xffff) == t) s += rowp[(size_t)(y - t0) * kBM + x];
-                if (r.y == t) s += colp[(size_t)(y - t0) * kBM + x];
-            }
-            sm[b - b0][x] = s;
-        }
-        __syncthreads();
-        if (own)
-            for (int b = b0; b < b1; ++b) v += sm[b - b0][x];
-        __syncthreads();
+// What the tiles leave for the modes of their rows and columns (EPI_GSYM), added in a
+// fixed order: part[c][m] the sums from the tiles of modes kSumModes c .., tile by tile,
+// for mode m; then gacc[m] over the c.  (One kernel per batch of modes that added to
+// gacc took 13 us each: a 256-atom cell 3.42 ms, 3.15 so.)
+constexpr int kSumModes = 8;
+__global__ void __launch_bounds__(kBM)
+gsym_part_kernel(int nb, const int *__restrict__ tile_start, const int2 *__restrict__ tiles,
+                 const double *__restrict__ rowp, const double *__restrict__ colp, double *__restrict__ part) {
+    const int t = blockIdx.x, x = threadIdx.x, mu0 = blockIdx.y * kSumModes, m = t * kBM + x;
+    const int y1 = tile_start[min(nb, mu0 + kSumModes)];
+    double s = 0.0;
+#pragma unroll 4
+    for (int y = tile_start[mu0]; y < y1; ++y) {
+        const int2 r = __ldg(tiles + y);
+        if ((r.x & 0xffff) == t) s += rowp[(size_t)y * kBM + x];
+        if (r.y == t) s += colp[(size_t)y * kBM + x];
     }
-    if (own) gacc[m] = v;
+    if (m < nb) part[(size_t)blockIdx.y * nb + m] = s;
+}
+__global__ void gsym_sums_kernel(int nb, int n_part, const double *__restrict__ part, double *__restrict__ gacc) {
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m >= nb) return;
+    double s = 0.0;
+#pragma unroll 8
+    for (int c = 0; c < n_part; ++c) s += part[(size_t)c * nb + m];
+    gacc[m] = s;
 }
 
 // Exponent of each mode's largest eigenvector component: |E(m, .)| <= 2^e[m].
@@ -717,22 +716,20 @@ int tc_gamma_batch_max(int nb, int sms, int sym3) {
 // three modes past the last one).
 static int tc_ldm(int nb) { return (nb + 3 + 31) / 32 * 32; }
 
-// Row and column sums of the tiles of a batch (EPI_GSYM).
-static size_t tc_gsym_bytes(int nb, int mb) {
-    const size_t nt = (size_t)(nb + kBM - 1) / kBM;
-    return ws_round(sizeof(double) * kBM * (size_t)mb * (nt * (nt + 1) / 2));
-}
+// Row (or column) sums of the tiles, and the parts of the modes' sums (EPI_GSYM).
+static size_t tc_gsym_bytes(size_t n_tiles) { return ws_round(sizeof(double) * kBM * std::max<size_t>(n_tiles, 1)); }
+static int tc_gsym_parts(int nb) { return (nb + kSumModes - 1) / kSumModes; }
 
-size_t tc_gamma_scratch_bytes(int nb, int mb_max, size_t n_fc3, int sym3) {
+size_t tc_gamma_scratch_bytes(int nb, int mb_max, size_t n_fc3, int sym3, size_t n_tiles) {
     const int ld = (nb + kBN - 1) / kBN * kBN;     // whole 128-column tiles per row
     const int rows = (nb + kBM - 1) / kBM * kBM;
     const size_t plane = ws_round(sizeof(__half) * (size_t)rows * ld);
     // E hi/lo, then Y hi, Y lo, T hi, T lo of every mode of a batch (the largest batch)
     // then the FP32 pairs of Phi3 and of the eigenvectors and the scales, then (Phi3 symmetric under
-    // every permutation) the tiles' sums and the modes' sums over the batches
+    // every permutation) the tiles' sums and the modes' sums
     return (2 + 4 * (size_t)mb_max) * plane + ws_round(sizeof(float2) * 27 * std::max<size_t>(n_fc3, 1)) +
            ws_round(sizeof(float2) * (size_t)nb * tc_ldm(nb)) + ws_round(sizeof(int) * (size_t)(nb + 4)) +
-           (sym3 ? 2 * tc_gsym_bytes(nb, mb_max) + ws_round(sizeof(double) * (size_t)nb) : 0);
+           (sym3 ? 2 * tc_gsym_bytes(n_tiles) + ws_round(sizeof(double) * (size_t)nb * (1 + tc_gsym_parts(nb))) : 0);
 }
 
 // The tensor-core pipeline for one Gamma-only system (Y build, T = E Y^T-form,
@@ -770,10 +767,8 @@ cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const L
     if (e != cudaSuccess) return e;
     if (gp.sym3) {
         rowp = reinterpret_cast<double *>(gsums);
-        colp = reinterpret_cast<double *>(gsums + tc_gsym_bytes(nb, gp.mb_max));
-        gacc = reinterpret_cast<double *>(gsums + 2 * tc_gsym_bytes(nb, gp.mb_max));
-        e = cudaMemsetAsync(gacc, 0, sizeof(double) * (size_t)nb, st);
-        if (e != cudaSuccess) return e;
+        colp = reinterpret_cast<double *>(gsums + tc_gsym_bytes(tiles.size()));
+        gacc = reinterpret_cast<double *>(gsums + 2 * tc_gsym_bytes(tiles.size()));
     }
     if (gacc_out) *gacc_out = gacc;
     const size_t nf = 27 * gp.n_fc3;
@@ -842,13 +837,17 @@ cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const L
                                                                p.wait_limit);
         p1.end();
         EpiGamma eg2{d.omega, d.occ, mu0, prow, sig2inv, p.cut_w, p.shape, partial_tc + t0, d.allowed,
-                     tiles_dev + t0, symmetric, rowp, colp};
+                     tiles_dev + t0, symmetric, rowp ? rowp + (size_t)t0 * kBM : nullptr,
+                     colp ? colp + (size_t)t0 * kBM : nullptr};
         EpiSplit es0{nullptr, nullptr, 0, 0, 0};
         ProfMark p2(p.prof, KALD_PROF_TC_GEMM2, st);
         k2<<<counted(t1 - t0), gp.sym3 ? gemm_threads(EPI_GSYM) : 128, kSmemBytes, st>>>(mTh, mTl, mEh, mEl, nb, nb, ld, sc, es0, eg2, err, p.wait_limit);
-        if (gp.sym3)
-            gsym_sums_kernel<<<counted(nt), 1024, 0, st>>>(nb, mu0, nm, ts, tiles_dev, t0, rowp, colp, gacc);
         p2.end();
+    }
+    if (gp.sym3 && gacc_out) {
+        double *part = gacc + nb;
+        gsym_part_kernel<<<counted(dim3(nt, tc_gsym_parts(nb))), kBM, 0, st>>>(nb, ts, tiles_dev, rowp, colp, part);
+        gsym_sums_kernel<<<counted((nb + 63) / 64), 64, 0, st>>>(nb, tc_gsym_parts(nb), part, gacc);
     }
     return cudaGetLastError();
 }
