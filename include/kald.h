@@ -57,11 +57,12 @@ typedef enum {
     KALD_FP32 = 1,           /* projection + delta epilogue in FP32 on CUDA
                                 cores, FP64 accumulation across q'            */
     KALD_BF16_SPLIT = 2      /* the two dense projection contractions on
-                                tcgen05 tensor cores with BF16 hi+lo operands
-                                (three MMAs per product) and FP32
-                                accumulation; the Bloch-phase gather (crystals)
-                                and the delta epilogue in FP32, sums over q'
-                                and modes in FP64.  Crystals (nb <= 96) and
+                                tcgen05 tensor cores with 16-bit hi+lo operands
+                                (BF16 for crystals, FP16 with power-of-two
+                                scales for Gamma-only systems; three MMAs per
+                                product) and FP32 accumulation; the Bloch-phase
+                                gather (crystals) and the delta epilogue in
+                                FP32, sums over q' and modes in FP64.  Crystals (nb <= 96) and
                                 Gamma-only systems.                           */
 } kald_precision;
 
@@ -78,8 +79,10 @@ typedef enum {
  *    squared projection |phi|^2 of a momentum triple (q1, q2, q3),
  *    q1 + q2 + q3 = 0 modulo G, is the same for every order of the triple, so
  *    one projection per orbit of ordered triples under permutations and
- *    inversion feeds the linewidths of all three members (cells of three to 32
- *    atoms in every precision, whole-mesh calls). */
+ *    inversion feeds the linewidths of all three members (cells of up to 32
+ *    atoms in every precision, whole-mesh calls).  Gamma-only systems with
+ *    KALD_BF16_SPLIT project each unordered triple of modes once (this one needs
+ *    no averaging). */
 typedef enum {
     KALD_SYM_ALL = 0,        /* every symmetry the path supports (default)    */
     KALD_SYM_INVERSION = 1,  /* time reversal only                            */
@@ -155,7 +158,8 @@ kald_status kald_set_stream(kald_ctx *ctx, void *stream);
 kald_status kald_set_wait_limit(kald_ctx *ctx, uint32_t polls);
 
 /* Cap the context's device workspace at `bytes` (0: no cap).  A later call
- * that would need more returns KALD_E_NOMEM without allocating; the cap also
+ * that would like more goes without its tables and large batches, and one
+ * that needs more returns KALD_E_NOMEM without allocating; the cap also
  * lets a caller bound the library's device memory.  No counterpart in the
  * paper. */
 kald_status kald_set_workspace_limit(kald_ctx *ctx, uint64_t bytes);
@@ -351,7 +355,9 @@ kald_status kald_kappa_rta(kald_ctx *ctx, const kald_system *sys, const int32_t 
  *   tau_{mu mu'} = (g + g') / ((w - w')^2 + (g + g')^2).
  *   eigvec  real eigenvectors (imaginary parts must be zero)
  *   kappa   [n_sys][3][3] out
- *   vgen    [3][nb][nb] out (W_a in A/ps, system 0 only) or NULL */
+ *   vgen    [3][nb][nb] out (W_a in A/ps, system 0 only) or NULL
+ * W_a is a product of exact slices on the tensor cores: a pipeline wait that
+ * expires returns KALD_E_TIMEOUT (also from kald_diffusivity). */
 kald_status kald_kappa_qhgk(kald_ctx *ctx, int32_t n_sys, const kald_system *sys,
                             const double *nu_thz, const double *eigvec, const double *gamma,
                             const kald_options *opt, double *kappa, double *vgen);

@@ -1538,7 +1538,7 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         std::shared_ptr<const LwTermsHost> ltp;
         std::shared_ptr<const TcxPlanHost> tpp;
         size_t lw_tab[3] = {0, 0, 0};
-        size_t tc_yc = 0;
+        size_t lw_yc = 0;
         auto terms_of = [&](bool tables) {
             auto n = std::make_shared<LwTermsHost>();
             plan_lw_terms(h, tables, *n);
@@ -1552,10 +1552,11 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
                 lw_tab[c] = (f32w ? sizeof(float2) : sizeof(double2)) * 27 * (size_t)ltp->n_slot[c] * nq;
                 all += lw_tab[c];
             }
-            if (tcx) all += sizeof(float2) * 9 * (size_t)nq * nb * std::min<size_t>(ltp->n_slot[2] / 3, h.pair3_j.size());
+            lw_yc = (f32w ? sizeof(float2) : sizeof(double2)) * 9 * (size_t)nq * nb * (ltp->cterm_start.size() - 1);
+            all += lw_yc;
             if (lean || all > (size_t(16) << 30)) {
                 ltp = terms_of(false);
-                lw_tab[0] = lw_tab[1] = lw_tab[2] = 0;
+                lw_tab[0] = lw_tab[1] = lw_tab[2] = lw_yc = 0;
             }
         }
         if (tcx) {
@@ -1567,7 +1568,6 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
             } else {
                 tpp = h.tcx_plan;
             }
-            tc_yc = sizeof(float2) * 9 * (size_t)nq * nb * (tpp->cterm_start.size() - 1);
         }
         const LwTermsHost no_terms;
         const TcxPlanHost no_plan;
@@ -1605,12 +1605,12 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
             need += bytes_of(sn_kk) + bytes_of(sn_bj) + bytes_of(sn_bk) + bytes_of(sn_start) +
                     ws_round(sizeof(double2) * (2 * (size_t)sn_m0 + 1)) + ws_round(sn_tab);
         if (!small)
-            need += (cc ? bytes_of(lt.group) + bytes_of(lt.term_start) + bytes_of(lt.term) : 0) +
-                    bytes_of(lt.slot_start) + bytes_of(lt.slot_blk) + ws_round(lw_tab[0]) + ws_round(lw_tab[1]) + ws_round(lw_tab[2]);
+            need += (cc ? bytes_of(lt.group) + bytes_of(lt.term_start) + bytes_of(lt.term) + bytes_of(lt.group_c) : 0) +
+                    bytes_of(lt.slot_start) + bytes_of(lt.slot_blk) + bytes_of(lt.cterm_start) + bytes_of(lt.cterm) +
+                    ws_round(lw_yc) + ws_round(lw_tab[0]) + ws_round(lw_tab[1]) + ws_round(lw_tab[2]);
         if (tcx)
             need += bytes_of(tp.term_start) + bytes_of(tp.list_start) + bytes_of(tp.glist) + bytes_of(tp.blk) +
-                    bytes_of(tp.term) + bytes_of(tp.cterm_start) + bytes_of(tp.cterm) +
-                    ws_round(tc_yc);
+                    bytes_of(tp.term);
         if (orb_pairs) need += bytes_of(orb_rows) + ws_round(orbit_bytes(mesh, nqc)) + ws_round(sizeof(double) * cc_out3) +
                            ws_round(sn_out3);
         if ((st = ws_reserve(ctx, need))) {
@@ -1657,10 +1657,6 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
             tg.glist = upload(ctx, tp.glist);
             tg.tblk = upload(ctx, tp.blk);
             tg.term = upload(ctx, tp.term);
-            tg.n_cg = (int)tp.cterm_start.size() - 1;
-            tg.cterm_start = upload(ctx, tp.cterm_start);
-            tg.cterm = upload(ctx, tp.cterm);
-            tg.yc = static_cast<float2 *>(ws_take(ctx, tc_yc));
             tg.gjk = upload(ctx, tc_gjk);
             tg.blkinfo = d.blkinfo;               // group order (HostSystem order)
             tg.fc3 = static_cast<const float *>(d.fc3);
@@ -1693,7 +1689,12 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
                 terms.group = upload(ctx, lt.group);
                 terms.term_start = upload(ctx, lt.term_start);
                 terms.term = upload(ctx, lt.term);
+                terms.group_c = upload(ctx, lt.group_c);
             }
+            terms.n_cg = (int)lt.cterm_start.size() - 1;
+            terms.cterm_start = upload(ctx, lt.cterm_start);
+            terms.cterm = upload(ctx, lt.cterm);
+            terms.yc = ws_take(ctx, lw_yc);
             terms.slot_start = upload(ctx, lt.slot_start);
             terms.slot_blk = upload(ctx, lt.slot_blk);
             for (int c = 0; c < 3; ++c) {
@@ -1721,6 +1722,10 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
             }
             if (e == cudaSuccess)
                 e = launch_lw_tables_f32(nq, p.n_rep, terms, d.blkinfo, tg.fc3, static_cast<const float2 *>(d.chi), s);
+            tg.n_cg = terms.n_cg;
+            tg.yc = static_cast<const float2 *>(terms.yc);
+            if (e == cudaSuccess)     // (an orbit's pair starts at any q of the mesh)
+                e = launch_lw_same(nb, nq, terms, use_sym ? nq : nqc, use_sym ? nullptr : d.qsel, d.eps_work, 1, s);
         }
         if (e == cudaSuccess)
             e = small ? launch_lw_small(p, d, sn, f32w, orb_pairs ? &orb : nullptr,

@@ -303,6 +303,10 @@ struct LwTermsHost {
     std::vector<int> group, term_start, slot_start, slot_blk;
     std::vector<int4> term;
     int n_slot[3] = {0, 0, 0}, slot0[3] = {0, 0, 0};
+    // groups with three or more class-2 terms: their index (-1: none) and those terms
+    // (i, slot), which are not among the others (launch_lw_same sums them per q)
+    std::vector<int> group_c, cterm_start;
+    std::vector<int2> cterm;
 };
 struct LwTerms {
     const int *group = nullptr;        // [n_atoms^2] group of (j, k), -1: none
@@ -312,6 +316,10 @@ struct LwTerms {
     const int *slot_blk = nullptr;
     int n_slot[3] = {0, 0, 0}, slot0[3] = {0, 0, 0};
     void *tab[3] = {nullptr, nullptr, nullptr};   // [nq][n_slot][27] complex
+    int n_cg = 0;
+    const int *group_c = nullptr, *cterm_start = nullptr;
+    const int2 *cterm = nullptr;
+    void *yc = nullptr;                // [nq][n_cg][9][nb] complex
     int n_pairs = 0;
     const int2 *pairs = nullptr;
     const int *orbit = nullptr;
@@ -322,6 +330,10 @@ int lw_orbit_blocks(int nb, int n_pairs, int fp32, int sm_count, size_t smem_opt
 void plan_lw_terms(const HostSystem &h, bool tables, LwTermsHost &o);
 cudaError_t launch_lw_tables_f32(int nq, int n_rep, const LwTerms &t, const int4 *blkinfo, const float *fc3,
                                  const float2 *chi, cudaStream_t st);
+// Y_s(3j + beta, 3k + gamma) of the class-2 terms set apart, into t.yc, for the n_rows
+// q-points rows[.].x (rows null: q-points 0 .. n_rows - 1).
+cudaError_t launch_lw_same(int nb, int nq, const LwTerms &t, int n_rows, const int2 *rows, const void *epsT, int fp32,
+                           cudaStream_t st);
 cudaError_t launch_lw_prep(const LwParams &p, const LwDev &d, int fp32, cudaStream_t st);
 cudaError_t launch_lw_main(const LwParams &p, const LwDev &d, const LwTerms &t, int fp32, int sm_count,
                            size_t smem_optin, cudaStream_t st);
@@ -433,19 +445,15 @@ struct TcxGroups {
     const int *term_start = nullptr, *list_start = nullptr, *glist = nullptr, *tblk = nullptr;
     const int4 *term = nullptr;
     int n_cg = 0;
-    const int *cterm_start = nullptr;
-    const int2 *cterm = nullptr;
-    float2 *yc = nullptr;             // [nq][n_cg][9][nb]
+    const float2 *yc = nullptr;       // [nq][n_cg][9][nb] (LwTerms::yc)
 };
 // Lists of the gather.  Terms of list x: term[term_start[x]..], each (i, class, slot
 // or start in blk, blocks), class 0..2 (a table's slot), 3 (blocks blk[..]) or 4
 // (nothing to add), plus 8 at the last term of a group; the list's groups in order:
-// glist[list_start[x]..], each j + (k << 8) + ((c + 1) << 16), c the index of the group
-// among those with many class-2 terms (-1: not one of them); cterm (i, slot) their terms.
+// glist[list_start[x]..], each j + (k << 8) + ((c + 1) << 16), c = LwTermsHost::group_c.
 struct TcxPlanHost {
-    std::vector<int> term_start, list_start, glist, blk, cterm_start;
+    std::vector<int> term_start, list_start, glist, blk;
     std::vector<int4> term;
-    std::vector<int2> cterm;
 };
 void plan_tcx_gather(const HostSystem &h, const LwTermsHost &lt, TcxPlanHost &o);
 bool tcx_y_wanted(size_t n_fc3, size_t n_groups);   // the phase sum on tensor cores is considered

@@ -146,6 +146,32 @@ __global__ void lw_tables_kernel(int nq, int n_rep, LwTerms t, const int4 *__res
     }
 }
 
+// One thread per mode, CTA = (row, group set apart).
+template <typename R>
+__global__ void __launch_bounds__(kMaxNbSmall)
+lw_same_kernel(int nb, LwTerms t, const int2 *__restrict__ rows, const typename C2<R>::T *__restrict__ epsT_all) {
+    using R2 = typename C2<R>::T;
+    const int c = blockIdx.y, q = rows ? rows[blockIdx.x].x : blockIdx.x, s = threadIdx.x;
+    if (s >= nb) return;
+    const R2 *eps = epsT_all + (size_t)q * nb * nb + s;
+    const R2 *tab = static_cast<const R2 *>(t.tab[2]) + (size_t)q * t.n_slot[2] * 27;
+    R2 acc[9];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) acc[e] = mk<R2>(0.0, 0.0);
+    for (int y = t.cterm_start[c]; y < t.cterm_start[c + 1]; ++y) {
+        const int2 tm = __ldg(t.cterm + y);                    // (i, slot)
+#pragma unroll
+        for (int al = 0; al < 3; ++al) {
+            const R2 u = eps[(size_t)(3 * tm.x + al) * nb];
+#pragma unroll
+            for (int e = 0; e < 9; ++e) cfma(acc[e], u, tab[(size_t)27 * tm.y + 9 * al + e]);
+        }
+    }
+    R2 *yc = static_cast<R2 *>(t.yc) + ((size_t)q * t.n_cg + c) * 9 * nb + s;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) yc[(size_t)e * nb] = acc[e];
+}
+
 // out [n_pairs][per]: the n_sblk mode blocks' position sums of a pair added in order.
 __global__ void lw_block_sums_kernel(size_t n, int per, int n_sblk, const double *__restrict__ out3,
                                      double *__restrict__ out) {
@@ -311,6 +337,12 @@ lw_main_kernel(LwParams p, LwDev d, LwTerms t, int SB, const R *__restrict__ fc3
                     for (int e = 0; e < 9; ++e) acc9[e] = mk<R2>(0.0, 0.0);
                     const int g = (j < na && k < na) ? __ldg(t.group + j * na + k) : -1;
                     if (g >= 0) {
+                        const int c2 = __ldg(t.group_c + g);
+                        if (c2 >= 0) {
+                            const R2 *yc = static_cast<const R2 *>(t.yc) + ((size_t)q * t.n_cg + c2) * 9 * nb + s0 + m;
+#pragma unroll
+                            for (int e = 0; e < 9; ++e) acc9[e] = yc[(size_t)e * nb];
+                        }
                         const R2 *em = es + m * P;
                         for (int y = t.term_start[g]; y < t.term_start[g + 1]; ++y) {
                             const int4 tm = __ldg(t.term + y);               // (i, class, slot or block)
@@ -904,6 +936,15 @@ static void run_lw_tables(int nq, int n_rep, const LwTerms &t, const int4 *blkin
         lw_tables_kernel<R><<<counted((unsigned)std::min<size_t>((nt + 255) / 256, 16384)), 256, 0, st>>>(nq, n_rep, t,
                                                                                                          blkinfo, fc3, chi);
 }
+cudaError_t launch_lw_same(int nb, int nq, const LwTerms &t, int n_rows, const int2 *rows, const void *epsT, int fp32,
+                           cudaStream_t st) {
+    if (!t.n_cg || !n_rows) return cudaSuccess;
+    const dim3 grid(rows ? n_rows : nq, t.n_cg);
+    const int threads = (nb + 31) / 32 * 32;
+    if (fp32) lw_same_kernel<float><<<counted(grid), threads, 0, st>>>(nb, t, rows, static_cast<const float2 *>(epsT));
+    else lw_same_kernel<double><<<counted(grid), threads, 0, st>>>(nb, t, rows, static_cast<const double2 *>(epsT));
+    return cudaGetLastError();
+}
 cudaError_t launch_lw_tables_f32(int nq, int n_rep, const LwTerms &t, const int4 *blkinfo, const float *fc3,
                                  const float2 *chi, cudaStream_t st) {
     run_lw_tables<float>(nq, n_rep, t, blkinfo, fc3, chi, st);
@@ -953,6 +994,9 @@ static cudaError_t run_lw_main(const LwParams &p, const LwDev &d, LwTerms t, int
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, nthr, smem);
     if (e != cudaSuccess) return e;
     run_lw_tables<R>(p.nq, p.n_rep, t, d.blkinfo, static_cast<const R *>(d.fc3), static_cast<const R2 *>(d.chi), st);
+    // (an orbit's pair starts at any q of the mesh)
+    e = launch_lw_same(p.nb, p.nq, t, ORBIT ? p.nq : p.nqc, ORBIT ? nullptr : d.qsel, d.eps_work, sizeof(R) == 4, st);
+    if (e != cudaSuccess) return e;
     const int n_batch = (p.nb + sb - 1) / sb;
     t.n_sblk = ORBIT ? lw_mode_blocks(p.nb, sb, t.n_pairs, sm_count)
                      : lw_mode_blocks(p.nb, sb, (long long)(p.nq / 2 + 1) * p.n_chunks, sm_count);
@@ -993,6 +1037,9 @@ void plan_lw_terms(const HostSystem &h, bool tables, LwTermsHost &o) {
     o.group.assign((size_t)na * na, -1);
     o.term_start.assign(1, 0);
     o.term.clear();
+    o.group_c.clear();
+    o.cterm_start.assign(1, 0);
+    o.cterm.clear();
     std::vector<std::vector<int>> slots[3];               // block lists, class by class
     for (int g = 0; g < ng; ++g) {
         o.group[(size_t)h.pair3_j[g] * na + h.pair3_k[g]] = g;
@@ -1028,6 +1075,19 @@ void plan_lw_terms(const HostSystem &h, bool tables, LwTermsHost &o) {
                 }
                 slots[cls].back().push_back(b);
             }
+        }
+        // many class-2 terms are summed per q-point, not per pair (an atom paired with
+        // itself has one per neighbour: a single thread walks a group's terms); two cost
+        // what reading their sum does
+        const size_t t0 = (size_t)o.term_start.back();
+        const auto is2 = [](const int4 &t) { return t.y == 2; };
+        const bool many = std::count_if(o.term.begin() + t0, o.term.end(), is2) >= 3;
+        o.group_c.push_back(many ? (int)o.cterm_start.size() - 1 : -1);
+        if (many) {
+            for (size_t y = t0; y < o.term.size(); ++y)
+                if (is2(o.term[y])) o.cterm.push_back(make_int2(o.term[y].x, o.term[y].z));
+            o.term.erase(std::remove_if(o.term.begin() + t0, o.term.end(), is2), o.term.end());
+            o.cterm_start.push_back((int)o.cterm.size());
         }
         o.term_start.push_back((int)o.term.size());
     }

@@ -665,35 +665,6 @@ clear_padding_kernel(int nb, int H, int Mp, size_t stride, __nv_bfloat16 *__rest
     }
 }
 
-// Y_s(3j + beta, 3k + gamma) of the class-2 terms (blocks with Rj = Rk, whose phase
-// depends on q alone) for the projected q-points: yc[q][c][9][nb], c the index of
-// the group among those with such terms.  One thread per mode.
-__global__ void __launch_bounds__(96)
-ycx_same_kernel(int nb, int nq, TcxGroups g, const int2 *__restrict__ qsel, const float2 *__restrict__ epsT_all) {
-    const int c = blockIdx.y, q = qsel ? qsel[blockIdx.x].x : blockIdx.x, s = threadIdx.x;
-    if (s >= nb) return;
-    const float2 *eps = epsT_all + (size_t)q * nb * nb + s;
-    const float2 *tab = g.tab[2] + (size_t)q * g.n_slot[2] * 27;
-    float2 acc[9];
-#pragma unroll
-    for (int e = 0; e < 9; ++e) acc[e] = make_float2(0.f, 0.f);
-    for (int t = g.cterm_start[c]; t < g.cterm_start[c + 1]; ++t) {
-        const int2 tm = __ldg(g.cterm + t);                    // (i, slot)
-#pragma unroll
-        for (int al = 0; al < 3; ++al) {
-            const float2 u = __ldg(eps + (size_t)(3 * tm.x + al) * nb);
-#pragma unroll
-            for (int e = 0; e < 9; ++e) {
-                const float2 w = __ldg(tab + (size_t)27 * tm.y + 9 * al + e);
-                acc[e] = __ffma2_rn(make_float2(u.x, u.x), w, acc[e]);
-                acc[e] = __ffma2_rn(make_float2(-u.y, u.y), make_float2(w.y, w.x), acc[e]);
-            }
-        }
-    }
-#pragma unroll
-    for (int e = 0; e < 9; ++e) g.yc[(((size_t)q * g.n_cg + c) * 9 + e) * nb + s] = acc[e];
-}
-
 // Phase-summed contraction over the home index (gather), three modes per lane
 // (2 l, 2 l + 1, 64 + l), CTA = (part of the (j, k) groups, pair), each warp
 // walking its own list of groups:
@@ -702,7 +673,7 @@ ycx_same_kernel(int nb, int nq, TcxGroups g, const int2 *__restrict__ qsel, cons
 // W_i the phase sums of the blocks of (i, j, k): from the per-q tables of class 0
 // (Rk = 0, of q'), 1 (Rj = 0, of q'') and 2 (Rj = Rk, of q), or of the blocks
 // themselves with their phases (class 3, summed by the lanes of the 27 values).
-// Groups with three or more class-2 terms take the sum of those from yc.  FP32;
+// Groups with many class-2 terms take the sum of those from yc.  FP32;
 // Y goes to A1 as BF16 hi/lo: for a fixed (b, c) the lanes of a warp cover
 // consecutive rows m = c nb + s.
 //
@@ -1452,18 +1423,11 @@ int tcx_batch_max(int nb, int nq, int sm_count) {
 void plan_tcx_gather(const HostSystem &h, const LwTermsHost &lt, TcxPlanHost &o) {
     const int ng = (int)lt.term_start.size() - 1;
     std::vector<std::vector<int4>> terms(ng);
-    std::vector<int> group_c(ng, -1);
-    o.cterm_start.assign(1, 0);
-    o.cterm.clear();
     o.blk.clear();
     for (int g = 0; g < ng; ++g) {
-        int n2 = 0;
-        for (int y = lt.term_start[g]; y < lt.term_start[g + 1]; ++y) n2 += lt.term[y].y == 2;
         for (int y = lt.term_start[g]; y < lt.term_start[g + 1]; ++y) {
             const int4 t = lt.term[y];                         // (i, class, slot or block, 0)
-            if (t.y == 2 && n2 >= 3) {                         // (two cost what reading their sum does)
-                o.cterm.push_back(make_int2(t.x, t.z));
-            } else if (t.y == 3) {
+            if (t.y == 3) {
                 if (terms[g].empty() || terms[g].back().y != 3 || terms[g].back().x != t.x)
                     terms[g].push_back(make_int4(t.x, 3, (int)o.blk.size(), 0));
                 o.blk.push_back(t.z);
@@ -1472,15 +1436,11 @@ void plan_tcx_gather(const HostSystem &h, const LwTermsHost &lt, TcxPlanHost &o)
                 terms[g].push_back(t);
             }
         }
-        if (n2 >= 3) {
-            group_c[g] = (int)o.cterm_start.size() - 1;
-            o.cterm_start.push_back((int)o.cterm.size());
-        }
     }
     std::vector<int> code(ng);
     std::vector<unsigned char> has((size_t)h.n_atoms * h.n_atoms, 0);
     for (int g = 0; g < ng; ++g) {
-        code[g] = h.pair3_j[g] + (h.pair3_k[g] << 8) + ((group_c[g] + 1) << 16);
+        code[g] = h.pair3_j[g] + (h.pair3_k[g] << 8) + ((lt.group_c[g] + 1) << 16);
         has[(size_t)h.pair3_j[g] * h.n_atoms + h.pair3_k[g]] = 1;
     }
     for (int j = 0; j < h.n_atoms; ++j)                        // atom pairs without blocks: zeros
@@ -1700,9 +1660,6 @@ cudaError_t launch_lw_tensor(const LwParams &p, const LwDev &d, const TcxGroups 
     cudaError_t ge = cudaFuncSetAttribute(ycx_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)gather_smem(nb));
     if (ge != cudaSuccess) return ge;
-    if (g.n_cg)       // (an orbit's pair starts at any q of the mesh)
-        ycx_same_kernel<<<counted(dim3(sym ? nq : p.nqc, g.n_cg)), 96, 0, st>>>(
-            nb, nq, g, sym ? nullptr : d.qsel, static_cast<const float2 *>(d.eps_work));
 
     XParams x;
     x.nb = nb; x.H = H; x.Kp = Kp; x.Mp = Mp;
