@@ -162,40 +162,30 @@ def shard_plan(mesh, n_sys: int, world: int, rank: int) -> dict:
 
 def orbit_pairs(mesh) -> int:
     """Number of orbits of ordered momentum triples (q1, q2, -(q1 + q2)) under
-    the six permutations and inversion q -> -q: the projections the tensor
-    path makes when Phi3 is symmetric under permutations (host counting)."""
-    m = np.asarray(mesh, dtype=np.int64)
-    nq = int(np.prod(m))
-    k = np.stack(np.meshgrid(*[np.arange(x) for x in m], indexing="ij"), -1).reshape(-1, 3)
-
-    def flat(v):
-        v = np.mod(v, m)
-        return (v[..., 0] * m[1] + v[..., 1]) * m[2] + v[..., 2]
-    q1, q2 = np.meshgrid(np.arange(nq), np.arange(nq), indexing="ij")
-    q1, q2 = q1.ravel(), q2.ravel()
-    q3 = flat(-(k[q1] + k[q2]))
-    neg = flat(-k)
-    code = lambda a, b, c: (a * nq + b) * nq + c
-    t = code(q1, q2, q3)
-    lowest = np.ones(t.shape, dtype=bool)
-    for a, b, c in ((q1, q2, q3), (q1, q3, q2), (q2, q1, q3), (q2, q3, q1), (q3, q1, q2), (q3, q2, q1)):
-        lowest &= t <= code(a, b, c)
-        lowest &= t <= code(neg[a], neg[b], neg[c])
-    return int(np.sum(lowest))
+    the six permutations and inversion q -> -q: the projections made when Phi3 is
+    symmetric under permutations.  Burnside's lemma over the twelve operations:
+    the identity fixes N^2 pairs, inversion s^2 (s q-points with -q = q), each
+    exchange N, with inversion N, the two 3-cycles the q with 3 q = 0 each, with
+    inversion q = 0 alone."""
+    n = s = c = 1
+    for m in mesh:
+        n *= int(m)
+        s *= 2 if m % 2 == 0 else 1
+        c *= 3 if m % 3 == 0 else 1
+    return (n * n + s * s + 6 * n + 2 * c + 2) // 12
 
 
 def projected_pairs(mesh, plan: dict, opt, nb: int) -> int:
     """(q, q') projections per step on this rank: one per orbit of momentum
-    triples on the BF16-split tensor path over the whole mesh (Phi3 of a pair
-    potential is symmetric under permutations); else the inversion classes
+    triples over the whole mesh (Phi3 of a pair potential is symmetric under
+    permutations); else the inversion classes
     {q, -q} of its q-points times the mesh (time reversal, when symmetry is not
     "none" and degenerate averaging is on); else its q-points times the mesh."""
     nq = int(np.prod(mesh))
     qs = plan["q"] if plan["kind"] == "qlist" else list(range(nq))
     if nq == 1 or opt.symmetry == "none" or not opt.degen_tol_thz > 0:
         return len(qs) * nq
-    if (opt.symmetry == "all" and opt.precision == "bf16split" and 65 <= nb <= 96
-            and plan["kind"] != "qlist"):
+    if opt.symmetry == "all" and plan["kind"] != "qlist":
         return orbit_pairs(mesh)
     mine = set(qs)
     return sum(1 for c in inversion_classes(mesh) if mine.intersection(c)) * nq
@@ -292,8 +282,9 @@ TRAFFIC_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of tcx_gemm_
                   "timed launches")
 
 
-def _gamma_only_band_tiles(om, cut, tile=128, symmetric=True):
-    """Delta-band (tm, tn) tiles of every valid mode, as the library lists them."""
+def _gamma_only_band_tiles(om, cut, tile=128, symmetric=True, once=False):
+    """Delta-band (tm, tn) tiles of every valid mode, as the library lists them
+    (`once`: each triple of modes projected once, tm from the mode's own tile on)."""
     b = len(om)
     nt = -(-b // tile)
     lo = np.full(nt, np.inf)
@@ -307,8 +298,9 @@ def _gamma_only_band_tiles(om, cut, tile=128, symmetric=True):
         return ((ww + lo[a] - hi[c] < cut) and (ww + hi[a] - lo[c] > -cut)) or \
                ((ww - hi[a] - hi[c] < cut) and (ww - lo[a] - lo[c] > -cut))
     n_tiles = 0
-    for ww in om[om > 0]:
-        for a in range(nt):
+    for mu in np.flatnonzero(om > 0):
+        ww = om[mu]
+        for a in range(mu // tile if once else 0, nt):
             for c in range(a if symmetric else 0, nt):
                 if hi[a] >= lo[a] and hi[c] >= lo[c] and (band(ww, a, c) or (symmetric and c != a and band(ww, c, a))):
                     n_tiles += 1
@@ -324,7 +316,6 @@ def roofline_of(args, w, nbs, nu_c, opt, prof, steps, allowed, pairs_step=None):
     sm_max = float(peaks.get("sm_max_mhz", 2070.0))
     fp32_peak = 152 * 128 * 2 * sm_max * 1e6 / 1e12          # TFLOP/s, FMA = 2 flops
     nq = w.n_q
-    s = w.systems[0]
     nb = nbs[0]
     offs = np.cumsum([0] + [nq * b for b in nbs])
     gamma_only = nq == 1
@@ -339,13 +330,14 @@ def roofline_of(args, w, nbs, nu_c, opt, prof, steps, allowed, pairs_step=None):
             for x, b in enumerate(nbs):
                 nu_x = nu_c[offs[x]:offs[x + 1]]
                 om = np.where(nu_x > opt.omega_min_thz, 2 * np.pi * nu_x, 0.0)
-                n_valid = int(np.sum(om > 0))
-                n_tiles = _gamma_only_band_tiles(om, cut)
+                once = opt.symmetry == "all"                 # each unordered triple of modes
+                n_tiles = _gamma_only_band_tiles(om, cut, once=once)
                 nt, ld = -(-b // 128), -(-b // 128) * 128
-                alg += n_valid * 2.0 * b ** 3 + n_tiles * 2.0 * 128 * 128 * b
-                exe += 3 * 2.0 * 128 * 128 * ld * (n_valid * nt * nt + n_tiles)
-            alg_note = ("per valid mode 2 nb^3 (T = E Y) plus 2 x 128 x 128 x nb per delta-band tile of "
-                        "phi = T E^T; executed: 3 BF16 MMAs per product on 128-padded tiles")
+                tm0 = np.flatnonzero(om > 0) // 128 if once else np.zeros(int(np.sum(om > 0)), int)
+                alg += float(np.sum(2.0 * b * b * (b - 128.0 * tm0))) + n_tiles * 2.0 * 128 * 128 * b
+                exe += 3 * 2.0 * 128 * 128 * ld * (float(np.sum(nt * (nt - tm0))) + n_tiles)
+            alg_note = ("per valid mode 2 nb^2 x the rows from its own 128-row tile on (T = E Y) plus 2 x 128 x 128 x nb "
+                        "per delta-band tile of phi = T E^T; executed: 3 FP16 MMAs per product on 128-padded tiles")
         else:
             names = ("tcx_gemm1", "tcx_gemm2")
             kernel = "tcx_gemm_kernel (GEMM1 T' = eps'^T Y_s, GEMM2 phi = T' conj(eps'') + delta epilogue)"
@@ -362,24 +354,23 @@ def roofline_of(args, w, nbs, nu_c, opt, prof, steps, allowed, pairs_step=None):
         executed = exe
     elif small:
         names = ("small_nb",)
-        kernel = "sn_kernel (one- and two-atom cells: phase sum, both contractions and the epilogue in registers)"
+        kernel = ("sn_orbit32_kernel / sn_orbit_kernel / sn_kernel (one- and two-atom cells: phase sums from tables, "
+                  "both contractions and the epilogue in registers)")
         n_valid = int(np.sum(nu_c > opt.omega_min_thz))
-        n_fc3 = s.fc3.shape[0]
-        alg = n_valid * nq * (108.0 * n_fc3 + 8.0 * nb ** 3) + allowed * 8.0 * nb
-        alg_note = "per (mode, q'): 108 n_fc3 (phase-summed first-index contraction) + 8 nb^3 (T'), 8 nb per allowed phi"
+        alg = n_valid * nq * 16.0 * nb ** 3 + allowed * 8.0 * nb
+        alg_note = "per (pair, mode): 8 nb^3 (first-index contraction with the phase sums) + 8 nb^3 (T'), 8 nb per allowed phi"
         peak = fp32_peak if args.precision != "fp64" else fp32_peak / 64.0
         bound, peak_note = "alu", "152 SMs x 128 FP32 lanes x 2 flop x sm_max_mhz" + ("" if args.precision != "fp64" else " / 64 (FP64)")
     else:
         names = ("lw_main",) if not gamma_only else ()
         kernel = "lw_main_kernel" if not gamma_only else "g_gemm_nt_kernel"
         n_valid = int(np.sum(nu_c > opt.omega_min_thz))
-        n_fc3 = s.fc3.shape[0]
         if gamma_only:
             alg = sum(4.0 * b ** 3 * int(np.sum(nu_c[offs[x]:offs[x + 1]] > opt.omega_min_thz))
                       for x, b in enumerate(nbs))
         else:
-            alg = n_valid * nq * (20.0 * n_fc3 + 8.0 * nb ** 3) + allowed * 8.0 * nb
-        alg_note = "Y build + T' per (mode, q'), phi at delta-allowed pairs"
+            alg = n_valid * nq * 8.0 * nb ** 3 + allowed * 8.0 * nb
+        alg_note = "T' per (mode, q'), phi at delta-allowed pairs (the phase sums come from tables)"
         peak = fp32_peak if args.precision == "fp32" else fp32_peak / 64.0
         bound, peak_note = "alu", "152 SMs x 128 FP32 lanes x 2 flop x sm_max_mhz" + ("" if args.precision == "fp32" else " / 64 (FP64)")
     ms = sum(prof.get(n, (0.0, 0))[0] for n in names)
