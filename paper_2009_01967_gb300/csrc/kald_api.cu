@@ -211,26 +211,27 @@ void *upload_scaled(kald_ctx *ctx, const std::vector<double> &raw, const std::ve
     return out;
 }
 
+size_t up_bytes(const HostSystem &h) { return h.pair2_up.empty() ? 0 : bytes_of(h.pair2_up); }
 size_t fc2_bytes(const HostSystem &h) {
     return bytes_of(h.pair2_i) + bytes_of(h.pair2_j) + bytes_of(h.pair2_start) +
            scaled_bytes(h.fc2_blk, h.fc2_atoms, h, 9, 9, 0) + bytes_of(h.fc2_rcart) + bytes_of(h.fc2_dist) +
-           bytes_of(h.pair2_up);
+           up_bytes(h);
 }
-void upload_fc2(kald_ctx *ctx, const HostSystem &h, DevSystem &d) {
+void upload_fc2(kald_ctx *ctx, const HostSystem &h, DevSystem &d, bool up = true) {
     d.pair2_i = upload(ctx, h.pair2_i);
     d.pair2_j = upload(ctx, h.pair2_j);
     d.pair2_start = upload(ctx, h.pair2_start);
     d.fc2 = static_cast<double *>(upload_scaled(ctx, h.fc2_blk, h.fc2_atoms, h, 9, 9, 0));
     d.fc2_r = upload(ctx, h.fc2_rcart);
     d.fc2_d = upload(ctx, h.fc2_dist);
-    d.up = upload(ctx, h.pair2_up);
+    d.up = up && !h.pair2_up.empty() ? upload(ctx, h.pair2_up) : nullptr;
 }
 DevFc2 dev_fc2(const HostSystem &h, const DevSystem &d) {
     DevFc2 f;
     f.n_pairs = (int)h.pair2_i.size();
     f.pair_i = d.pair2_i; f.pair_j = d.pair2_j; f.pair_start = d.pair2_start;
     f.blk = d.fc2; f.rcart = d.fc2_r;
-    f.n_up = (int)h.pair2_up.size(); f.up = d.up;
+    f.n_up = d.up ? (int)h.pair2_up.size() : 0; f.up = d.up;
     return f;
 }
 
@@ -732,20 +733,35 @@ kald_status kald_phonons(kald_ctx *ctx, const kald_system *sys, const int32_t me
     }
     const bool mirror = !large && nrep < nq;
     const size_t nnr = mirror ? (size_t)nrep * nb * nb : nn;
-    const size_t nnv = large ? 0 : (size_t)(mirror ? nrep : nq) * jacobi_scratch(nb);      // eigensolver scratch
-    size_t need = fc2_bytes(h) + bytes_of(qc) + ws_round(sizeof(double2) * nnr) + ws_round(sizeof(double2) * nnv) +
-                  ws_round(sizeof(int));
+    const int nqe = mirror ? nrep : nq;              // q-points solved
+    const size_t n_blk2 = h.fc2_blk.size() / 9;
+    size_t nnv = large ? 0 : (size_t)nqe * jacobi_scratch(nb);      // eigensolver scratch
+    int qbatch = nqe;                                // q-points per eigensolver launch
+    size_t need = fc2_bytes(h) + bytes_of(qc) + ws_round(sizeof(double2) * nnr) + ws_round(sizeof(int));
     if (mirror)
         need += bytes_of(qc_rep) + bytes_of(rep_row) + bytes_of(rep_conj) + ws_round(sizeof(double) * nrep * nb) +
                 ws_round(sizeof(double2) * nnr);
-    const size_t n_blk2 = h.fc2_blk.size() / 9;
-    if (vel && !large)
-        need += vel_table_bytes(nrep, n_blk2) + (mirror ? ws_round(sizeof(double) * 3 * nrep * nb) : 0);
+    const size_t vel_bytes = vel && !large ? vel_table_bytes(nqe, n_blk2) : 0;
+    const size_t vrep_bytes = vel && mirror ? ws_round(sizeof(double) * 3 * nrep * nb) : 0;
     if (large) need += eigh_large_scratch_bytes(nb) + eigh_batch_records_bytes(1);
     if (!d_nu) need += ws_round(sizeof(double) * nq * nb);
     if (!d_eig) need += ws_round(sizeof(double2) * nn);
     if (vel && !d_vel) need += ws_round(sizeof(double) * 3 * nq * nb);
-    if ((st = ws_reserve(ctx, need))) return st;
+    // lean: where the workspace cannot be had, the eigensolver takes the q-points in
+    // batches whose scratch is that of plain matrices, and the velocities' table and
+    // half of the mesh's velocities stand where the matrices were (D, then V)
+    bool lean = false;
+    if ((st = ws_reserve(ctx, need + ws_round(sizeof(double2) * nnv) + vel_bytes + vrep_bytes)) == KALD_E_NOMEM && !large) {
+        lean = true;
+        const size_t up = up_bytes(h) / sizeof(double2) + 16, plain = (size_t)nqe * nb * nb;
+        qbatch = (int)std::max<size_t>(1, std::min<size_t>(nqe, (plain - std::min(plain, up)) / jacobi_scratch(nb)));
+        nnv = (size_t)qbatch * jacobi_scratch(nb);
+        const size_t later = vrep_bytes + (vel ? sizeof(double2) * n_blk2 : 0);     // after the eigensolver
+        const size_t held = ws_round(sizeof(double2) * nnr);
+        if (later > held) nnv = std::max(nnv, (later - held + sizeof(double2) - 1) / sizeof(double2));
+        st = ws_reserve(ctx, need + ws_round(sizeof(double2) * nnv));
+    }
+    if (st) return st;
     DevSystem d;
     upload_fc2(ctx, h, d);
     const double *qcart = upload(ctx, qc);
@@ -762,8 +778,27 @@ kald_status kald_phonons(kald_ctx *ctx, const kald_system *sys, const int32_t me
                            : static_cast<double2 *>(ws_take(ctx, sizeof(double2) * nn));
     double *vel_d = nullptr;
     if (vel) vel_d = d_vel ? vel : static_cast<double *>(ws_take(ctx, sizeof(double) * 3 * nq * nb));
-    void *vel_tab = vel && !large ? ws_take(ctx, vel_table_bytes(nrep, n_blk2)) : nullptr;
-    double *vel_rep = vel && mirror ? static_cast<double *>(ws_take(ctx, sizeof(double) * 3 * nrep * nb)) : nullptr;
+    void *vel_tab = nullptr;
+    double *vel_rep = nullptr;
+    size_t vel_room = vel_bytes;
+    if (lean) {
+        char *dv = reinterpret_cast<char *>(D);      // D and V are neighbours
+        vel_rep = vrep_bytes ? reinterpret_cast<double *>(dv) : nullptr;
+        vel_tab = dv + vrep_bytes;
+        vel_room = ws_round(sizeof(double2) * nnr) + ws_round(sizeof(double2) * nnv) - vrep_bytes;
+    } else {
+        vel_tab = vel_bytes ? ws_take(ctx, vel_bytes) : nullptr;
+        vel_rep = vrep_bytes ? static_cast<double *>(ws_take(ctx, vrep_bytes)) : nullptr;
+    }
+    auto solve = [&](double *nu_o, double2 *eig_o, cudaStream_t st_) {
+        cudaError_t r = cudaSuccess;
+        for (int q0 = 0; q0 < nqe && r == cudaSuccess; q0 += qbatch) {
+            const size_t o = (size_t)q0 * nb;
+            r = launch_jacobi(nb, std::min(qbatch, nqe - q0), D + o * nb, V, nu_o + o, eig_o + o * nb, nonconv,
+                              ctx->smem_optin, st_);
+        }
+        return r;
+    };
     cudaStream_t s = ctx->stream;
     double *big = large ? static_cast<double *>(ws_take(ctx, eigh_large_scratch_bytes(nb))) : nullptr;
     void *rec = large ? ws_take(ctx, eigh_batch_records_bytes(1)) : nullptr;
@@ -774,17 +809,17 @@ kald_status kald_phonons(kald_ctx *ctx, const kald_system *sys, const int32_t me
             const EighJob job{nb, D, big, nu_d, eig_d};
             e = launch_eigh_large_batch(1, &job, rec, ctx->sm_count, ctx->smem_optin, s);
         } else if (mirror) {
-            e = launch_jacobi(nb, nrep, D, V, nu_rep, eig_rep, nonconv, ctx->smem_optin, s);
+            e = solve(nu_rep, eig_rep, s);
             if (e == cudaSuccess && vel)
                 e = launch_vel_diag(dev_fc2(h, d), nb, nrep, n_blk2, qcart_rep, nu_rep, nullptr, eig_rep, nullptr, nullptr,
-                                    vel_tab, vel_rep, nullptr, s);
+                                    vel_tab, vel_room, vel_rep, nullptr, s);
             if (e == cudaSuccess)
                 e = launch_mirror_phonons(nq, nb, row_d, conj_d, nu_rep, eig_rep, vel_rep, nu_d, eig_d, vel_d, s);
         } else {
-            e = launch_jacobi(nb, nq, D, V, nu_d, eig_d, nonconv, ctx->smem_optin, s);
+            e = solve(nu_d, eig_d, s);
             if (e == cudaSuccess && vel)
                 e = launch_vel_diag(dev_fc2(h, d), nb, nq, n_blk2, qcart, nu_d, nullptr, eig_d, nullptr, nullptr, vel_tab,
-                                    vel_d, nullptr, s);
+                                    vel_room, vel_d, nullptr, s);
         }
     }
     if (e == cudaSuccess && vel && large)
@@ -1445,6 +1480,10 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
             int nch = (int)std::max(1LL, std::min<long long>(nq, (want + n_full - 1) / n_full));
             p.qp_chunk = (nq + nch - 1) / nch;
             p.n_chunks = (nq + p.qp_chunk - 1) / p.qp_chunk;
+            if (lean == 2) {                     // (half of the partial sums: the terms' lists take less)
+                p.qp_chunk = std::min(nq, 2 * p.qp_chunk);
+                p.n_chunks = (nq + p.qp_chunk - 1) / p.qp_chunk;
+            }
             if (tcx) { p.qp_chunk = nq; p.n_chunks = 1; }
             if (small) {
                 p.qp_chunk = sn_chunk(nb, nq, ctx->sm_count);
@@ -1865,11 +1904,19 @@ kald_status kald_kappa_bte(kald_ctx *ctx, const kald_system *sys, const int32_t 
             std::vector<int> qf;
             mesh_points(h.lattice, mesh, qc, qf);
             const bool d_nu = is_device_ptr(nu_thz), d_eig = is_device_ptr(eigvec), d_k = is_device_ptr(kappa);
+            const size_t n_blk2 = h.fc2_blk.size() / 9;
+            size_t vel_bytes = vel_table_bytes(nq, n_blk2);
             size_t need = fc2_bytes(h) + bytes_of(qc) + ws_round(sizeof(double) * 3 * (size_t)N) +
-                          bte_work_bytes(N) + ws_round(72) + vel_table_bytes(nq, h.fc2_blk.size() / 9);
+                          bte_work_bytes(N) + ws_round(72);
             if (!d_nu) need += ws_round(sizeof(double) * N);
             if (!d_eig) need += ws_round(sizeof(double2) * (size_t)N * nb);
-            st = ws_reserve(ctx, need);
+            // lean: the velocities' table in the solver's vectors, which come after it
+            bool lean = false;
+            if ((st = ws_reserve(ctx, need + vel_bytes)) == KALD_E_NOMEM &&
+                sizeof(double2) * n_blk2 <= bte_work_bytes(N)) {
+                lean = true;
+                st = ws_reserve(ctx, need);
+            }
             if (st == KALD_OK) {
                 DevSystem d;
                 upload_fc2(ctx, h, d);
@@ -1879,10 +1926,10 @@ kald_status kald_kappa_bte(kald_ctx *ctx, const kald_system *sys, const int32_t 
                 double *vel = static_cast<double *>(ws_take(ctx, sizeof(double) * 3 * (size_t)N));
                 void *work = ws_take(ctx, bte_work_bytes(N));
                 double *k_d = d_k ? kappa : static_cast<double *>(ws_take(ctx, 72));
-                const size_t n_blk2 = h.fc2_blk.size() / 9;
-                void *vel_tab = ws_take(ctx, vel_table_bytes(nq, n_blk2));
+                void *vel_tab = lean ? work : ws_take(ctx, vel_bytes);
                 cudaError_t e = launch_vel_diag(dev_fc2(h, d), nb, nq, n_blk2, qcart, nu_d, nullptr, eig_d, nullptr,
-                                                nullptr, vel_tab, vel, nullptr, ctx->stream);
+                                                nullptr, vel_tab, lean ? bte_work_bytes(N) : vel_bytes, vel, nullptr,
+                                                ctx->stream);
                 if (e == cudaSuccess)
                     e = bte_solve(N, g1, g0, nu_d, vel, opt->omega_min_thz, opt->temperature_K, opt->classical,
                                   method, tol, max_iter, work, kKappaSI / ((double)nq * h.volume), k_d, iters, conv,
@@ -1985,16 +2032,17 @@ kald_status kald_phase_space(kald_ctx *ctx, const kald_system *sys, const int32_
 }
 
 // Workspace of the generalised velocities of one Gamma-only system.
-static size_t qhgk_work_bytes(int nb) {
+static size_t qhgk_work_bytes(int nb, int dirs) {
     return ws_round(sizeof(double) * 4 * (size_t)nb) + ws_round(sizeof(double) * 3 * (size_t)nb * nb) +
-           ws_round(oz_work_bytes(nb)) + ws_round(16);
+           ws_round(oz_work_bytes(nb, dirs)) + ws_round(16);
 }
-static QhgkWork take_qhgk_work(kald_ctx *ctx, int nb) {
+static QhgkWork take_qhgk_work(kald_ctx *ctx, int nb, int dirs) {
     QhgkWork w;
     double *m = static_cast<double *>(ws_take(ctx, sizeof(double) * 4 * (size_t)nb));
     w.modes = {m, m + nb, m + 2 * (size_t)nb, m + 3 * (size_t)nb};
     w.W = static_cast<double *>(ws_take(ctx, sizeof(double) * 3 * (size_t)nb * nb));
-    w.oz = ws_take(ctx, oz_work_bytes(nb));
+    w.oz = ws_take(ctx, oz_work_bytes(nb, dirs));
+    w.dirs = dirs;
     w.err = static_cast<int *>(ws_take(ctx, 16));
     return w;
 }
@@ -2023,12 +2071,16 @@ kald_status kald_diffusivity(kald_ctx *ctx, int32_t n_sys, const kald_system *sy
                 row_start[h.pair2_i[pp] + 1]++;
             }
         for (int i = 0; i < h.n_atoms; ++i) row_start[i + 1] += row_start[i];
-        size_t need = bytes_of(row_start) + bytes_of(col_j) + scaled_bytes(h.fc2_blk, h.fc2_atoms, h, 9, 9, 0) +
-                      bytes_of(h.fc2_dist) + qhgk_work_bytes(nb) + ws_round(sizeof(double) * nb);
-        if (!d_nu) need += ws_round(sizeof(double) * nb);
-        if (!d_eig) need += ws_round(sizeof(double2) * nn);
-        if (!d_g) need += ws_round(sizeof(double) * nb);
-        if ((st = ws_reserve(ctx, need))) return st;
+        int dirs = 3;                // one direction at a time where the workspace cannot be had
+        for (;; dirs = 1) {
+            size_t need = bytes_of(row_start) + bytes_of(col_j) + scaled_bytes(h.fc2_blk, h.fc2_atoms, h, 9, 9, 0) +
+                          bytes_of(h.fc2_dist) + qhgk_work_bytes(nb, dirs) + ws_round(sizeof(double) * nb);
+            if (!d_nu) need += ws_round(sizeof(double) * nb);
+            if (!d_eig) need += ws_round(sizeof(double2) * nn);
+            if (!d_g) need += ws_round(sizeof(double) * nb);
+            if (!(st = ws_reserve(ctx, need))) break;
+            if (st != KALD_E_NOMEM || dirs == 1) return st;
+        }
         DevFc2Dist f;
         f.n_rows = h.n_atoms;
         f.row_start = upload(ctx, row_start);
@@ -2038,7 +2090,7 @@ kald_status kald_diffusivity(kald_ctx *ctx, int32_t n_sys, const kald_system *sy
         const double *nu_d = stage_in(ctx, nu_thz + off_nb, (size_t)nb, d_nu);
         const double2 *eig_d = stage_in(ctx, reinterpret_cast<const double2 *>(eigvec) + off_eig, nn, d_eig);
         const double *g_d = stage_in(ctx, gamma + off_nb, (size_t)nb, d_g);
-        const QhgkWork work = take_qhgk_work(ctx, nb);
+        const QhgkWork work = take_qhgk_work(ctx, nb, dirs);
         cudaMemsetAsync(work.err, 0, sizeof(int), ctx->stream);
         if (h.fc2_symmetric < 0) h.fc2_symmetric = fc2_symmetric(&sys[x]) ? 1 : 0;
         double *D_d = d_D ? D + off_nb : static_cast<double *>(ws_take(ctx, sizeof(double) * nb));
@@ -2199,28 +2251,43 @@ kald_status kald_kappa_rta(kald_ctx *ctx, const kald_system *sys, const int32_t 
         neg[q] = (((mesh[0] - k[0]) % mesh[0]) * mesh[1] + (mesh[1] - k[1]) % mesh[1]) * mesh[2] +
                  (mesh[2] - k[2]) % mesh[2];
     }
-    size_t need = fc2_bytes(h) + bytes_of(qc) + ws_round(sizeof(double) * 9 * (size_t)nq) + ws_round(72) +
-                  2 * bytes_of(neg) + n_el * ws_round(sizeof(double) * nel) + vel_table_bytes(nq, n_blk2);
+    // lean: where the workspace cannot be had, the kernel that needs no velocities
+    const size_t extra = 2 * bytes_of(neg) + n_el * ws_round(sizeof(double) * nel) + vel_table_bytes(nq, n_blk2) +
+                         up_bytes(h);
+    size_t need = fc2_bytes(h) - up_bytes(h) + bytes_of(qc) + ws_round(sizeof(double) * 9 * (size_t)nq) + ws_round(72);
     if (!d_nu) need += ws_round(sizeof(double) * nq * nb);
     if (!d_eig) need += ws_round(sizeof(double2) * nn);
     if (!d_g) need += ws_round(sizeof(double) * nq * nb);
-    if ((st = ws_reserve(ctx, need))) return st;
+    bool lean = false;
+    if ((st = ws_reserve(ctx, need + extra)) == KALD_E_NOMEM) {
+        lean = true;
+        st = ws_reserve(ctx, need);
+    }
+    if (st) return st;
     DevSystem d;
-    upload_fc2(ctx, h, d);
+    upload_fc2(ctx, h, d, !lean);
     const double *qcart = upload(ctx, qc);
     const double *nu_d = stage_in(ctx, nu_thz, (size_t)nq * nb, d_nu);
     const double2 *eig_d = stage_in(ctx, reinterpret_cast<const double2 *>(eigvec), nn, d_eig);
     const double *g_d = stage_in(ctx, gamma, (size_t)nq * nb, d_g);
     double *partial = static_cast<double *>(ws_take(ctx, sizeof(double) * 9 * (size_t)nq));
     double *k_d = d_k ? kappa : static_cast<double *>(ws_take(ctx, 72));
+    const double scale = kKappaSI / ((double)nq * h.volume);
+    if (lean) {
+        const cudaError_t e = launch_kappa_rta(dev_fc2(h, d), nb, nq, qcart, nu_d, eig_d, g_d, opt->temperature_K,
+                                               opt->classical, opt->omega_min_thz, opt->degen_tol_thz, partial, k_d, scale,
+                                               ctx->stream);
+        if (e != cudaSuccess) return cuda_check(ctx, e, "kald_kappa_rta launch");
+        if (!d_k) cudaMemcpyAsync(kappa, k_d, 72, cudaMemcpyDeviceToHost, ctx->stream);
+        return finish(ctx, "kald_kappa_rta");
+    }
     const int *neg_d = upload(ctx, neg);
     int *src = static_cast<int *>(ws_take(ctx, sizeof(int) * (size_t)nq));
     double *vre = static_cast<double *>(ws_take(ctx, sizeof(double) * nel));
     double *vim = n_el == 2 ? static_cast<double *>(ws_take(ctx, sizeof(double) * nel)) : nullptr;
     void *vel_tab = ws_take(ctx, vel_table_bytes(nq, n_blk2));
-    const double scale = kKappaSI / ((double)nq * h.volume);
-    cudaError_t e = launch_vel_diag(dev_fc2(h, d), nb, nq, n_blk2, qcart, nullptr, nu_d, eig_d, neg_d, src, vel_tab, vre,
-                                    vim, ctx->stream);
+    cudaError_t e = launch_vel_diag(dev_fc2(h, d), nb, nq, n_blk2, qcart, nullptr, nu_d, eig_d, neg_d, src, vel_tab,
+                                    vel_table_bytes(nq, n_blk2), vre, vim, ctx->stream);
     if (e == cudaSuccess)
         e = launch_kappa_rta_diag(dev_fc2(h, d), nb, nq, qcart, nu_d, eig_d, g_d, src, vre, vim,
                                   vel_batch(nq, n_blk2) == nq ? static_cast<const double2 *>(vel_tab) : nullptr,
@@ -2251,7 +2318,7 @@ kald_status kald_kappa_qhgk(kald_ctx *ctx, int32_t n_sys, const kald_system *sys
         int n_partial;
     };
     std::vector<Item> items(n_sys);
-    size_t need = 0, off_nb = 0, off_eig = 0;
+    size_t need = 0, saved = 0, off_nb = 0, off_eig = 0;
     std::vector<std::shared_ptr<const HostSystem>> hps;
     if ((st = plan_systems_cached(ctx, n_sys, sys, hps))) return st;
     {
@@ -2286,15 +2353,21 @@ kald_status kald_kappa_qhgk(kald_ctx *ctx, int32_t n_sys, const kald_system *sys
         it.off_nb = off_nb;
         it.off_eig = off_eig;
         need += bytes_of(it.row_start) + bytes_of(it.col_j) + scaled_bytes(h.fc2_blk, h.fc2_atoms, h, 9, 9, 0) +
-                bytes_of(h.fc2_dist) + qhgk_work_bytes(nb) + ws_round(sizeof(double) * 9 * (size_t)it.n_partial) +
+                bytes_of(h.fc2_dist) + qhgk_work_bytes(nb, 3) + ws_round(sizeof(double) * 9 * (size_t)it.n_partial) +
                 ws_round(72);
+        saved += qhgk_work_bytes(nb, 3) - qhgk_work_bytes(nb, 1);
         if (!d_nu) need += ws_round(sizeof(double) * nb);
         if (!d_eig) need += ws_round(sizeof(double2) * nn);
         if (!d_g) need += ws_round(sizeof(double) * nb);
         off_nb += nb;
         off_eig += nn;
     }
-    if ((st = ws_reserve(ctx, need))) return st;
+    int dirs = 3;                    // one direction at a time where the workspace cannot be had
+    if ((st = ws_reserve(ctx, need)) == KALD_E_NOMEM) {
+        dirs = 1;
+        st = ws_reserve(ctx, need - saved);
+    }
+    if (st) return st;
     struct Dev {
         DevFc2Dist f;
         const double *nu, *g;
@@ -2317,7 +2390,7 @@ kald_status kald_kappa_qhgk(kald_ctx *ctx, int32_t n_sys, const kald_system *sys
         dv.nu = stage_in(ctx, nu_thz + it.off_nb, (size_t)nb, d_nu);
         dv.eig = stage_in(ctx, reinterpret_cast<const double2 *>(eigvec) + it.off_eig, nn, d_eig);
         dv.g = stage_in(ctx, gamma + it.off_nb, (size_t)nb, d_g);
-        dv.work = take_qhgk_work(ctx, nb);
+        dv.work = take_qhgk_work(ctx, nb, dirs);
         cudaMemsetAsync(dv.work.err, 0, sizeof(int), ctx->stream);
         dv.partial = static_cast<double *>(ws_take(ctx, sizeof(double) * 9 * (size_t)it.n_partial));
         dv.k = d_k ? kappa + 9 * (size_t)x : static_cast<double *>(ws_take(ctx, 72));

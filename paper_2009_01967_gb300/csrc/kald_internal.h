@@ -220,7 +220,7 @@ cudaError_t launch_velocity_diag(const DevFc2 &f, int nb, int nq, const double *
 size_t vel_table_bytes(int nq, size_t n_blk);
 int vel_batch(int nq, size_t n_blk);   // q-points of one batch: the table holds them all when this is nq
 cudaError_t launch_vel_diag(const DevFc2 &f, int nb, int nq, size_t n_blk, const double *qcart, const double *nu_scale,
-                            const double *nu_cmp, const double2 *eig, const int *neg, int *src, void *table,
+                            const double *nu_cmp, const double2 *eig, const int *neg, int *src, void *table, size_t table_bytes,
                             double *out_re, double *out_im, cudaStream_t st);
 
 // linewidths.cu
@@ -518,14 +518,15 @@ struct QhgkModes {
 struct QhgkWork {
     QhgkModes modes;
     double *W;                // [3][nb][nb]
-    void *oz;                 // oz_work_bytes(nb)
+    void *oz;                 // oz_work_bytes(nb, dirs)
+    int dirs;                 // directions whose slices are held at once: 3, or 1
     int *err;                 // bounded-wait failures
 };
 // qhgk_gemm.cu: W_a = E B_a^T scaled by fac per mode, over B_a [3][n][n] in BW;
 // antisym: the tiles on and above the diagonal only, mirrored when fill.
-size_t oz_work_bytes(int n);
+size_t oz_work_bytes(int n, int dirs);
 cudaError_t launch_oz_gemm(int n, const double2 *E, double *BW, const double *fac, int antisym, int fill, void *work,
-                           int *err, uint32_t wait_limit, cudaStream_t st);
+                           int dirs, int *err, uint32_t wait_limit, cudaStream_t st);
 // Mode diffusivity D [nb] (A^2/ps) of a Gamma-only system (generalised
 // velocity as for QHGK, then the per-mode sum).
 // bandwidth_w > 0: fixed width in place of gamma + gamma'; threshold_w > 0:

@@ -575,7 +575,7 @@ static cudaError_t launch_velocity_w(const DevFc2Dist &f, int nb, const double *
     else if (2 * row <= smem_optin) sparse(sparse_ae_kernel<2>, 2);
     else sparse_ae_kernel<1, false><<<counted(nb), 256, 0, st>>>(f, nb, eig, w.W);
     if (e != cudaSuccess) return e;
-    return launch_oz_gemm(nb, eig, w.W, w.modes.fac, antisym, fill, w.oz, w.err, wait_limit, st);
+    return launch_oz_gemm(nb, eig, w.W, w.modes.fac, antisym, fill, w.oz, w.dirs, w.err, wait_limit, st);
 }
 
 cudaError_t launch_diffusivity(const DevFc2Dist &f, int nb, const double *nu_thz, const double2 *eig,

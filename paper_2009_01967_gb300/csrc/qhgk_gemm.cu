@@ -283,26 +283,30 @@ bool oz_map(CUtensorMap *map, const void *ptr, int ld, int rows, int planes, int
 
 }  // namespace
 
-size_t oz_work_bytes(int n) {
-    return ws_round(kOz * oz_plane(n)) + ws_round(3 * kOz * oz_plane(n)) + ws_round(sizeof(double) * 4 * (size_t)n);
+size_t oz_work_bytes(int n, int dirs) {
+    return ws_round(kOz * oz_plane(n)) + ws_round(dirs * kOz * oz_plane(n)) + ws_round(sizeof(double) * 4 * (size_t)n);
 }
 
 cudaError_t launch_oz_gemm(int n, const double2 *E, double *BW, const double *fac, int antisym, int fill, void *work,
-                           int *err, uint32_t wait_limit, cudaStream_t st) {
+                           int dirs, int *err, uint32_t wait_limit, cudaStream_t st) {
     char *w = static_cast<char *>(work);
     auto *pa = reinterpret_cast<__nv_bfloat16 *>(w);
     auto *pb = reinterpret_cast<__nv_bfloat16 *>(w + ws_round(kOz * oz_plane(n)));
-    double *sa = reinterpret_cast<double *>(w + ws_round(kOz * oz_plane(n)) + ws_round(3 * kOz * oz_plane(n)));
+    double *sa = reinterpret_cast<double *>(w + ws_round(kOz * oz_plane(n)) + ws_round(dirs * kOz * oz_plane(n)));
     double *sb = sa + n;
     const int rows = oz_rows(n), ld = oz_ld(n);
     oz_slice_kernel<double2><<<counted(dim3(rows, 1)), 256, 0, st>>>(n, rows, ld, E, fac, pa, sa);
-    oz_slice_kernel<double><<<counted(dim3(rows, 3)), 256, 0, st>>>(n, rows, ld, BW, fac, pb, sb);
     CUtensorMap mA, mB;
-    if (!oz_map(&mA, pa, ld, rows, kOz, kOzBM) || !oz_map(&mB, pb, ld, rows, 3 * kOz, kOzBN)) return cudaErrorInvalidValue;
+    if (!oz_map(&mA, pa, ld, rows, kOz, kOzBM) || !oz_map(&mB, pb, ld, rows, dirs * kOz, kOzBN))
+        return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzSmem);
     if (e != cudaSuccess) return e;
-    oz_gemm_kernel<<<counted(dim3((n + kOzBN - 1) / kOzBN, rows / kOzBM, 3)), kOzThreads, kOzSmem, st>>>(
-        mA, mB, n, ld / kOzBK, antisym, sa, sb, BW, err, wait_limit);
+    for (int d = 0; d < 3; d += dirs) {            // all at once, or one by one in a small workspace
+        double *bw = BW + (size_t)d * n * n;
+        oz_slice_kernel<double><<<counted(dim3(rows, dirs)), 256, 0, st>>>(n, rows, ld, bw, fac, pb, sb);
+        oz_gemm_kernel<<<counted(dim3((n + kOzBN - 1) / kOzBN, rows / kOzBM, dirs)), kOzThreads, kOzSmem, st>>>(
+            mA, mB, n, ld / kOzBK, antisym, sa, sb, bw, err, wait_limit);
+    }
     if (antisym && fill) {
         const unsigned nt = (unsigned)((n + 31) / 32);
         antisym_fill_kernel<<<counted(dim3(nt, nt, 3)), 256, 0, st>>>(n, BW);

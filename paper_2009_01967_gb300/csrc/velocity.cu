@@ -209,7 +209,7 @@ size_t vel_table_bytes(int nq, size_t n_blk) {
 
 cudaError_t launch_vel_diag(const DevFc2 &f, int nb, int nq, size_t n_blk, const double *qcart, const double *nu_scale,
                             const double *nu_cmp, const double2 *eig, const int *neg, int *src, void *table,
-                            double *out_re, double *out_im, cudaStream_t st) {
+                            size_t table_bytes, double *out_re, double *out_im, cudaStream_t st) {
     const int nbp = (nb + 31) / 32 * 32, groups = std::min(384 / nbp, 4);
     const size_t smem = vel_smem(nb, groups);
     auto k0 = vel_kernel<false>;
@@ -217,7 +217,7 @@ cudaError_t launch_vel_diag(const DevFc2 &f, int nb, int nq, size_t n_blk, const
     cudaError_t e = cudaFuncSetAttribute(out_im ? k1 : k0, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     double2 *ph = static_cast<double2 *>(table);
-    const int batch = vel_batch(nq, n_blk);
+    const int batch = (int)std::max<size_t>(1, std::min<size_t>(nq, table_bytes / (sizeof(double2) * std::max<size_t>(n_blk, 1))));
     for (int q0 = 0; q0 < nq; q0 += batch) {
         const int n = std::min(batch, nq - q0);
         const size_t np = (size_t)n * n_blk;

@@ -438,3 +438,61 @@ def test_phase_space_of_mirrored_frequencies(k, mesh, change, precision):
         ctx.set_workspace_limit(0)
     assert np.max(np.abs(g - ref)) <= (1e-10 if precision == "fp64" else 1e-5) * np.max(np.abs(ref))
     assert np.all(np.asarray(ref) > 0)
+
+
+@pytest.mark.parametrize("cell,mesh", [((1, 1, 1), (3, 4, 2)), ((2, 2, 2), (2, 1, 1)), ((2, 1, 1), (1, 1, 1)),
+                                       (None, (5, 3, 1))])
+def test_phonons_and_conductivity_at_the_smallest_workspace(k, cell, mesh):
+    """The eigensolver in batches, the velocities' table and the mirrored velocities in
+    the matrices' place, the conductivity without stored velocities: what a call gives
+    with the workspace it would like (one- to 32-atom cells, meshes with and without
+    mirrored points)."""
+    kk, ctx = k
+    s = ki.fcc_supercell_system(cell, seed=7) if cell else ki.small_binary().systems[0]
+    opt = kk.Options(temperature_K=300.0, sigma_thz=0.1)
+
+    def least(f):
+        import re
+        ctx.set_workspace_limit(1)
+        with pytest.raises(kk.KaldError) as e:
+            f()
+        ctx.set_workspace_limit(int(re.search(r"needs (\d+) bytes", str(e.value)).group(1)))
+
+    try:
+        nu, eig, vel = kk.kald_phonons(ctx, s, mesh)
+        least(lambda: kk.kald_phonons(ctx, s, mesh))
+        nu2, eig2, vel2 = kk.kald_phonons(ctx, s, mesh)
+        np.testing.assert_array_equal(nu, nu2)
+        np.testing.assert_array_equal(eig, eig2)
+        np.testing.assert_array_equal(vel, vel2)
+        ctx.set_workspace_limit(0)
+        g = np.where(nu > 0.01, 0.1, 0.0).ravel()
+        kappa = kk.kald_kappa_rta(ctx, s, mesh, nu, eig, g, opt)
+        least(lambda: kk.kald_kappa_rta(ctx, s, mesh, nu, eig, g, opt))
+        kappa2 = kk.kald_kappa_rta(ctx, s, mesh, nu, eig, g, opt)
+    finally:
+        ctx.set_workspace_limit(0)
+    np.testing.assert_allclose(kappa2, kappa, rtol=1e-9, atol=1e-11 * np.abs(kappa).max() + 1e-30)
+
+
+@pytest.mark.parametrize("cell", [(3, 3, 1), (4, 4, 2)])
+def test_generalised_velocities_one_direction_at_a_time(k, cell):
+    """108 and 384 modes: one direction's slices at a time, bit for bit."""
+    import re
+    kk, ctx = k
+    s = ki.fcc_supercell_system(cell, seed=5)
+    nu, eig = ph.phonons(s, (1, 1, 1))
+    g = np.where(nu > 0.01, 0.1, 0.0).ravel()
+    opt = kk.Options(temperature_K=300.0, sigma_thz=0.1)
+    for call in (lambda: kk.kald_kappa_qhgk(ctx, [s], nu.ravel(), eig.ravel(), g, opt)[0],
+                 lambda: kk.kald_diffusivity(ctx, [s], nu.ravel(), eig.ravel(), g, opt)):
+        ref = call()
+        ctx.set_workspace_limit(1)
+        try:
+            with pytest.raises(kk.KaldError) as e:
+                call()
+            ctx.set_workspace_limit(int(re.search(r"needs (\d+) bytes", str(e.value)).group(1)))
+            got = call()
+        finally:
+            ctx.set_workspace_limit(0)
+        np.testing.assert_array_equal(got, ref)
