@@ -213,7 +213,7 @@ __host__ __device__ inline size_t lw_smem_bytes(int nb, int sb, int nthr, bool o
 // orbit of momentum triples, three weights per element, the sums of all three
 // positions into out3.  Eight atoms (24 branches), 4^3 mesh, FP64: 74 ms with
 // every block phased for every mode, one mode per CTA and one q-point of each
-// pair {q, -q}; 4.8 ms now.
+// pair {q, -q}; 3.3 ms now.
 template <typename R, bool OPER_SMEM, bool ORBIT>
 __global__ void __launch_bounds__(kThreads, 1)
 lw_main_kernel(LwParams p, LwDev d, LwTerms t, int SB, const R *__restrict__ fc3,

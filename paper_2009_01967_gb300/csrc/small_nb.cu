@@ -172,7 +172,7 @@ sn_tables_kernel(int nq, SnTables t, typename Cx<R>::T *__restrict__ tab) {
 // Bound: FMA issue, FP32 or FP64.  Phasing every block for every (pair, mode)
 // cost 54 n_fc3 FMA (25,380 for the two-atom cell), fifteen times the two dense
 // contractions; with the tables a (pair, mode) costs 3 nb^3 complex FMA in all.
-// One call, two-atom cell, 24^3 mesh, FP32: 1367 ms before, 191 ms now.
+// One call, two-atom cell, 24^3 mesh, FP32: 1367 ms before, 191 ms (34 with orbits).
 template <typename R, int NB, bool BTE>
 __global__ void __launch_bounds__(kSnThreads)
 sn_kernel(LwParams p, LwDev d, SnTables t, const typename Cx<R>::T *__restrict__ tab,
