@@ -574,6 +574,7 @@ kald_status plan_systems_cached(kald_ctx *ctx, int n, const kald_system *sys,
     std::stable_sort(order.begin(), order.end(), [&](int u, int v) { return sys[todo[u]].n_fc3 > sys[todo[v]].n_fc3; });
     parallel_for(todo.size(), total, [&](size_t z) {
         const int y = order[z];
+        cudaSetDevice(ctx->device);                    // (a new thread's is 0; pointers are looked up)
         made[y] = std::make_shared<HostSystem>();
         sts[y] = plan_system(&errs[y], &sys[todo[y]], *made[y]);
     });
@@ -1137,7 +1138,7 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
     std::vector<Item> items;
     size_t off_nb = 0, off_eig = 0, total_modes = 0;
     for (int x = 0; x < n_sys; ++x) {
-        const int nb = hps[x]->nb;
+        const int nb = 3 * sys[x].n_atoms;
         if (nb > kMaxNbSmall) items.push_back({x, hps[x], GammaPlan(), {}, off_nb, off_eig, 0});
         off_nb += nb;
         off_eig += (size_t)nb * nb;
@@ -1372,7 +1373,12 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
     std::vector<std::shared_ptr<const HostSystem>> hps;   // one q-point: all at once; else one by one
     if (nq_mesh == 1) {
         // every Gamma-only supercell (nb > 96) of the call in one launch sequence
-        if ((st = plan_systems_cached(ctx, n_sys, sys, hps))) return st;
+        // (64 at a time; the plans of small cells are made again one by one below)
+        std::vector<std::shared_ptr<const HostSystem>> some;
+        for (int x0 = 0; x0 < n_sys; x0 += 64) {
+            if ((st = plan_systems_cached(ctx, std::min(64, n_sys - x0), sys + x0, some))) return st;
+            for (auto &p : some) hps.push_back(p->nb > kMaxNbSmall || n_sys <= 64 ? p : nullptr);
+        }
         if ((st = gamma_only_batch(ctx, n_sys, sys, hps, nu_thz, eigvec, opt, gamma, d_nu, d_eig, d_g, tot,
                                    allowed_tot)))
             return st;
@@ -1381,7 +1387,7 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
     int lean = 0;            // where the workspace cannot be had: 1 without tables, 2 without orbits as well
     for (int x = 0; x < n_sys; ++x) {
         std::shared_ptr<const HostSystem> hp;
-        if (nq_mesh == 1) hp = hps[x];
+        if (nq_mesh == 1 && hps[x]) hp = hps[x];
         else if ((st = plan_system_cached(ctx, &sys[x], hp))) return st;
         const HostSystem &h = *hp;
         const int nb = h.nb;

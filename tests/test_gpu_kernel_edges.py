@@ -496,3 +496,20 @@ def test_generalised_velocities_one_direction_at_a_time(k, cell):
         finally:
             ctx.set_workspace_limit(0)
         np.testing.assert_array_equal(got, ref)
+
+
+def test_more_systems_than_are_planned_at_once(k):
+    """66 Gamma-only systems (64 are planned together), small cells around a large one:
+    the linewidths of each alone, bit for bit."""
+    kk, ctx = k
+    small = [ki.fcc_supercell_system((1, 1, 1), seed=i) for i in range(3)]
+    big = ki.fcc_supercell_system((3, 3, 1), seed=9)
+    systems = [small[i % 3] for i in range(65)]
+    systems.insert(40, big)
+    opt = kk.Options(temperature_K=300.0, sigma_thz=0.2, precision="bf16split")
+    ph1 = {id(s): ph.phonons(s, (1, 1, 1)) for s in small + [big]}
+    alone = {id(s): kk.kald_linewidths(ctx, [s], (1, 1, 1), ph1[id(s)][0].ravel(), ph1[id(s)][1].ravel(), opt)[0]
+             for s in small + [big]}
+    nu, eig = (np.concatenate([ph1[id(s)][c].ravel() for s in systems]) for c in (0, 1))
+    got, _ = kk.kald_linewidths(ctx, systems, (1, 1, 1), nu, eig, opt)
+    np.testing.assert_array_equal(got, np.concatenate([np.asarray(alone[id(s)]).ravel() for s in systems]))
