@@ -929,12 +929,12 @@ kald_status kald_phonons_batch(kald_ctx *ctx, int32_t n_sys, const kald_system *
 
 namespace kald {
 namespace {
-// Blocks of fc3 by their nine indices (the first of several alike): open addressing,
-// at most half full.
+// Blocks of fc3 by their nine indices: open addressing, at most half full.
 struct Fc3Index {
     const kald_system *s;
     std::vector<int> slot;
     size_t mask;
+    bool repeated = false;                   // some indices are listed more than once
     static size_t hash(const int32_t *a) {
         size_t h = 1469598103934665603ull;
         for (int x = 0; x < 9; ++x) h = (h ^ (size_t)(uint32_t)a[x]) * 1099511628211ull;
@@ -950,6 +950,7 @@ struct Fc3Index {
             size_t y = hash(k) & mask;
             while (slot[y] >= 0 && !std::equal(k, k + 9, s->fc3_idx + 9 * (size_t)slot[y])) y = (y + 1) & mask;
             if (slot[y] < 0) slot[y] = b;
+            else repeated = true;
         }
     }
     int find(const int32_t *k) const {
@@ -963,9 +964,15 @@ struct Fc3Index {
 // with the last two Cartesian indices exchanged (then Y_mu and phi are symmetric and
 // the tensor-core path computes only the upper triangle); and h.fc3_perm_symmetric:
 // besides, the partner (j; i -Rj; k Rk - Rj) (home atom j) with the first two
-// exchanged.  The two exchanges generate all six permutations.
+// exchanged.  The two exchanges generate all six permutations.  A Phi3 that lists some
+// indices more than once has neither: every listed block is added, and the comparison
+// of single blocks says nothing about the sums.
 void fc3_symmetries(const kald_system *s, const HostSystem &h) {
     const Fc3Index idx(s);
+    if (idx.repeated) {
+        h.fc3_symmetric = h.fc3_perm_symmetric = 0;
+        return;
+    }
     // entries agree to 1e-12 of the largest |Phi3| (the self blocks (i; i; i) are sums
     // that cancel to rounding noise, so no per-entry relative test)
     double tol = 0.0;

@@ -513,3 +513,29 @@ def test_more_systems_than_are_planned_at_once(k):
     nu, eig = (np.concatenate([ph1[id(s)][c].ravel() for s in systems]) for c in (0, 1))
     got, _ = kk.kald_linewidths(ctx, systems, (1, 1, 1), nu, eig, opt)
     np.testing.assert_array_equal(got, np.concatenate([np.asarray(alone[id(s)]).ravel() for s in systems]))
+
+
+@pytest.mark.parametrize("cell,mesh,precision", [(None, (3, 3, 3), "fp64"), (None, (3, 3, 3), "fp32"),
+                                                 ((1, 1, 1), (3, 2, 2), "fp64"), ((2, 2, 2), (2, 1, 1), "bf16split"),
+                                                 ((3, 3, 1), (1, 1, 1), "bf16split")])
+def test_repeated_blocks_are_added(k, cell, mesh, precision):
+    """A Phi3 block listed twice counts twice, so that Phi3 is not symmetric under
+    permutations although every single block has its partners: the linewidths are
+    those of the same Phi3 with the two blocks added into one, which no symmetry check
+    takes for symmetric (two, four and 32 atoms, and a Gamma-only cell)."""
+    from dataclasses import replace
+    kk, ctx = k
+    s = ki.fcc_supercell_system(cell, seed=7) if cell else ki.small_binary().systems[0]
+    nu, eig = ph.phonons(s, mesh)
+    pair = np.any(s.fc3_idx[:, 2:5] != 0, axis=1) | np.any(s.fc3_idx[:, 6:9] != 0, axis=1)
+    b = int(np.argmax(np.where(pair, np.abs(s.fc3).max(axis=(1, 2, 3)), 0.0)))
+    fc3 = s.fc3.copy()
+    fc3[b] *= 2.0
+    added = replace(s, fc3=fc3)
+    twice = replace(s, fc3=np.concatenate([s.fc3, s.fc3[b:b + 1]]),
+                    fc3_idx=np.concatenate([s.fc3_idx, s.fc3_idx[b:b + 1]]))
+    ref, _ = kk.kald_linewidths(ctx, [added], mesh, nu.ravel(), eig.ravel(),
+                                kk.Options(temperature_K=300.0, sigma_thz=0.1, precision="fp64", symmetry="none"))
+    got, _ = kk.kald_linewidths(ctx, [twice], mesh, nu.ravel(), eig.ravel(),
+                                kk.Options(temperature_K=300.0, sigma_thz=0.1, precision=precision))
+    assert _rel(got, ref) < (1e-10 if precision == "fp64" else 1e-5)
