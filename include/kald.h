@@ -59,7 +59,8 @@ typedef enum {
     KALD_BF16_SPLIT = 2      /* the two dense projection contractions on
                                 tcgen05 tensor cores with 16-bit hi+lo operands
                                 (BF16 for crystals, FP16 with power-of-two
-                                scales for Gamma-only systems; three MMAs per
+                                scales per atom, mode and operand, taken from
+                                the data, for Gamma-only systems; three MMAs per
                                 product) and FP32 accumulation; the Bloch-phase
                                 gather (crystals) and the delta epilogue in
                                 FP32, sums over q' and modes in FP64.  Crystals (nb <= 96) and

@@ -191,20 +191,25 @@ size_t bytes_of(const std::vector<T> &v) { return ws_round(sizeof(T) * std::max<
 // Mass-scaled force constants on the device: the raw blocks, their atoms and
 // the masses are uploaded and a kernel divides each block by the square root
 // of its masses' product (launch_mass_scale); out_stride >= nval, f32 selects
-// an FP32 copy.  scaled_bytes() is the workspace this takes.
+// an FP32 copy; in place where neither changes the layout.  scaled_bytes() is the
+// workspace this takes.
 size_t scaled_bytes(const std::vector<double> &raw, const std::vector<int> &atoms, const HostSystem &h,
                     int nval, int out_stride, int f32) {
     const size_t nblk = raw.size() / nval;
     return bytes_of(raw) + bytes_of(atoms) + bytes_of(h.masses) +
-           ws_round((f32 ? sizeof(float) : sizeof(double)) * std::max<size_t>(nblk, 1) * out_stride);
+           (out_stride == nval && !f32
+                ? 0
+                : ws_round((f32 ? sizeof(float) : sizeof(double)) * std::max<size_t>(nblk, 1) * out_stride));
 }
 void *upload_scaled(kald_ctx *ctx, const std::vector<double> &raw, const std::vector<int> &atoms,
                     const HostSystem &h, int nval, int out_stride, int f32) {
     const size_t nblk = raw.size() / nval;
-    const double *r = upload(ctx, raw);
+    double *r = upload(ctx, raw);
     const int *a = upload(ctx, atoms);
     const double *m = upload(ctx, h.masses);
-    void *out = ws_take(ctx, (f32 ? sizeof(float) : sizeof(double)) * std::max<size_t>(nblk, 1) * out_stride);
+    void *out = out_stride == nval && !f32
+                    ? r
+                    : ws_take(ctx, (f32 ? sizeof(float) : sizeof(double)) * std::max<size_t>(nblk, 1) * out_stride);
     // (a launch error surfaces at the call's final status check)
     launch_mass_scale((int)nblk, nval, (int)(atoms.size() / std::max<size_t>(nblk, 1)), r, a, m, out_stride, f32,
                       out, ctx->stream);
@@ -464,6 +469,15 @@ kald_status plan_system(kald_ctx *ctx, const kald_system *s, HostSystem &h) {
     for (int x = 0; x < ng; ++x) {
         h.pair3_order[x] = by_k[by_class[x]];
         h.pair3_long += len_class(h.pair3_order[x]) == 0;
+    }
+    h.pair3_kstart.assign(n + 1, 0);
+    for (int g = 0; g < ng; ++g) ++h.pair3_kstart[h.pair3_k[g] + 1];
+    for (int k = 0; k < n; ++k) h.pair3_kstart[k + 1] += h.pair3_kstart[k];
+    h.pair3_at.resize(ng);
+    std::vector<int> at(h.pair3_kstart.begin(), h.pair3_kstart.end() - 1);
+    for (int x = 0; x < ng; ++x) {
+        const int g = h.pair3_order[x];
+        h.pair3_at[at[h.pair3_k[g]]++] = make_int2(x, h.pair3_j[g]);
     }
     h.n_rep = n_rep;
     return KALD_OK;
@@ -1211,7 +1225,9 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
                    scaled_bytes(h.fc3_blk, h.fc3_atoms, h, 27, 27, 0) + 2 * ws_round(sizeof(double) * nb) +
                    ws_round(sizeof(int) * nb);
         if (mode == KALD_BF16_SPLIT)
-            b += tc_gamma_scratch_bytes(nb, gp.mb_max, gp.n_fc3, gp.sym3, gp.tiles.size()) + bytes_of(h.pair3_order) + ws_round(sizeof(int2) * n_tiles + sizeof(int) * (nb + 1)) +
+            b += tc_gamma_scratch_bytes(nb, gp.mb_max, gp.n_fc3, gp.sym3, gp.tiles.size()) + bytes_of(h.pair3_order) +
+                 bytes_of(h.pair3_kstart) + bytes_of(h.pair3_at) +
+                 ws_round(sizeof(int2) * n_tiles + sizeof(int) * (nb + 1)) +
                  ws_round(sizeof(double) * n_tiles);
         else
             b += 4 * ws_round(rs * nn) + ws_round(sizeof(double) * nb * (size_t)gp.n_part);
@@ -1246,12 +1262,15 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
         gd.occ = static_cast<double *>(ws_take(ctx, sizeof(double) * nb));
         gd.E = gd.Y = gd.T = gd.PHI = nullptr;
         gd.partial = nullptr;
-        gd.group_order = nullptr;
+        gd.group_order = gd.k_start = nullptr;
+        gd.k_at = nullptr;
         gd.tc_scratch = nullptr; gd.tiles_dev = nullptr; gd.partial_tc = nullptr;
         if (mode == KALD_BF16_SPLIT) {
             gd.tc_scratch = ws_take(ctx, tc_gamma_scratch_bytes(nb, it.gp.mb_max, it.gp.n_fc3, it.gp.sym3,
                                                                 it.gp.tiles.size()));
             gd.group_order = upload(ctx, h.pair3_order);
+            gd.k_start = upload(ctx, h.pair3_kstart);
+            gd.k_at = upload(ctx, h.pair3_at);
             gd.tiles_dev = static_cast<int2 *>(ws_take(ctx, sizeof(int2) * n_tiles + sizeof(int) * (nb + 1)));
             gd.partial_tc = static_cast<double *>(ws_take(ctx, sizeof(double) * n_tiles));
         } else {

@@ -146,6 +146,9 @@ struct HostSystem {
     // class ordered by (k, j) (the Y build of the Gamma-only tensor-core path)
     std::vector<int> pair3_order;
     int pair3_long = 0;
+    // the groups of each k: (place in pair3_order, j)
+    std::vector<int> pair3_kstart;
+    std::vector<int2> pair3_at;
     std::vector<int> fc3_i, fc3_rj, fc3_rk;            // per block (sorted order)
     std::vector<double> fc3_blk;                       // [n_fc3][27] Phi3 (eV/A^3), grouped, not mass-scaled
     std::vector<int> fc3_atoms;                        // [n_fc3][3] (i, j, k) of each block
@@ -363,6 +366,8 @@ struct GammaPlan {
 struct GammaDev {
     const int *group_jk, *group_start, *blk_i;   // (j, k) groups of fc3 blocks
     const int *group_order;          // HostSystem::pair3_order (tensor-core path)
+    const int *k_start;              // HostSystem::pair3_kstart, pair3_at (tensor-core path)
+    const int2 *k_at;
     const double *fc3;               // [n_fc3][27] Phi3 / sqrt(mi mj mk)
     const double2 *eig;              // [nb][nb] (real parts used)
     const double *nu;                // [nb] THz

@@ -764,7 +764,7 @@ __global__ void velocity_kernel(DevFc2 f, int nb, const double *__restrict__ qca
 // block's atoms), e < nval, and zero padding up to out_stride; FP64, or
 // rounded to FP32 when f32.  One thread per output value; out may alias raw
 // when the strides agree.
-__global__ void mass_scale_kernel(int n_blk, int nval, int n_at, const double *__restrict__ raw,
+__global__ void mass_scale_kernel(int n_blk, int nval, int n_at, const double *raw,
                                   const int *__restrict__ atoms, const double *__restrict__ masses,
                                   int out_stride, int f32, void *out) {
     const size_t n = (size_t)n_blk * out_stride;

@@ -8,9 +8,9 @@
 // lo leave about 22 significant bits per product (two BF16 pieces left 16, and the
 // error of gamma from that, 1e-5 for the smallest cells, grows when each triple of
 // modes is projected once instead of three times).  FP16's narrow range is met by
-// powers of two (Scales): each mode's eigenvector is scaled by its largest
-// component, Y_mu by that of mode mu and a bound of the contraction with Phi3, T by
-// the number of terms of its sums; the epilogues take them out exactly.
+// powers of two (Scales): each atom by how strongly Phi3 holds it, each mode's
+// eigenvector by its largest component, Y_mu by its largest element as built, T by
+// the norms of its two factors; the epilogues take them out exactly.
 //
 // Several modes go through each launch (a batch of MB modes, so that small
 // systems still fill the GPU): the Y and T planes of the batch are stacked
@@ -84,21 +84,39 @@ struct EpiSplit {
     int tm0;                  // first row tile
 };
 
-// Powers of two that bring the operands into FP16's range:
-//   E(m, .) = 2^e_m E', |E'| <= 1, stored x 2^kEBits;
-//   Y_mu = 2^(e_mu + eL) Y', |Y'| <= 1, stored x 2^kYBits (2^eL bounds the sums of
-//   |Phi3| that one component multiplies);
-//   T = E Y_mu = 2^(e_m + e_mu + eL) T', |T'| <= 2^eR, stored x 2^(kTBits - eR).
-constexpr int kEBits = 10, kYBits = 14, kTBits = 15;
+// Powers of two that bring the operands into FP16's range.  With k the exponents of
+// the atoms (atom_scale_kernel), E^(m, b) = 2^k_b E(m, b) and
+// Y^_mu(c, b) = 2^(-k_b - k_c) Y_mu(c, b), whose contractions over b and c are those
+// of E and Y:
+//   E^(m, .) = 2^e_m E', |E'| <= 1 and |E'|_2 <= 2^h_m, stored x 2^kEBits;
+//   Y^_mu = 2^y_mu Y', |Y'| <= 1 (y_mu from its largest element), stored x 2^kYBits;
+//   T^ = E^ Y^_mu = 2^(e_m + y_mu) T', |T'| <= 2^(h_m + hR) (Cauchy-Schwarz: the rows
+//   of Y_mu have at most 4^hR entries), stored x 2^(kTBits - h_m - hR).
+// FP16's step is 2^-24, so an element keeps the 16 bits of two BF16 pieces down to
+// 2^-23 of the largest one of its row of E or of its Y_mu, and to some 2^-16 of a
+// usual one of T.  The scales therefore follow what is measured: Y_mu per mode, since
+// the strong couplings inside a molecule cancel for the modes that move it as a whole,
+// and the atoms, since a mode may extend over parts whose Phi3 differs by orders of
+// magnitude.  With one exponent for the whole Phi3 the modes of the weaker part lost
+// 3e-4 of gamma where its Phi3 is 2^-16 of the stronger part's, 4e-3 at 2^-20 and 0.3
+// at 2^-24; 4e-7 now, as in a uniform cell, and 2e-6 for modes mixed of the two parts
+// at 2^-24 (216 modes).  The passes this takes: 256 atoms 2.88 -> 3.14 ms.
+constexpr int kEBits = 15, kYBits = 15, kTBits = 15;
 struct Scales {
-    const int *l1;            // bits of the largest sum of |Phi3| (FP32)
-    const int *e;             // [nb] e_m
-    int eR;                   // 2^eR >= entries of a row of Y_mu^T
-    __device__ __forceinline__ int eL() const {
+    const int *e, *h;         // [nb] e_m, h_m
+    const int *ymax;          // [nb] bits of the largest |Y^_mu| (FP32)
+    int hR;
+    __device__ __forceinline__ int y(int mu) const {
         int x;
-        frexpf(__int_as_float(__ldg(l1)), &x);
+        frexpf(__int_as_float(__ldg(ymax + mu)), &x);
         return x;
     }
+    // what takes an accumulator of the second contraction to phi, for row m of mode mu
+    // and for column n
+    __device__ __forceinline__ float row(int m, int mu) const {
+        return ldexpf(1.0f, __ldg(e + m) + __ldg(h + m) + y(mu) + hR - kTBits - kEBits);
+    }
+    __device__ __forceinline__ float col(int n) const { return ldexpf(1.0f, __ldg(e + n)); }
 };
 
 // Columns [c, c + 32) of the accumulators, added in a fixed order.
@@ -268,7 +286,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
         // rows, so each lane pair writes two whole 64-byte row segments per
         // chunk with 32-byte stores (st_rowpair_v8).
         const bool okw = __all_sync(0xffffffffu, ok);
-        const float tsc = ldexpf(1.0f, kTBits - sc.eR - kEBits - kYBits);
+        const float tsc = ldexpf(1.0f, kTBits - (m < M ? __ldg(sc.h + m) : 0) - sc.hR - kEBits - kYBits);
         const size_t orow = (size_t)bz * es.b_rows + m;
         char *ph = reinterpret_cast<char *>(es.hi + orow * es.ld + tn * kBN);
         char *pl = reinterpret_cast<char *>(es.lo + orow * es.ld + tn * kBN);
@@ -307,11 +325,11 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
             const F2 ncol = nc < N ? f2_of(eg.occ[nc]) : F2{0.f, 0.f};
             wn_sm[tc] = wcol.h; wl_sm[tc] = wcol.l;
             nn_sm[tc] = ncol.h; nl_sm[tc] = ncol.l;
-            cf_sm[tc] = nc < N ? ldexpf(1.0f, __ldg(sc.e + nc)) : 0.0f;
+            cf_sm[tc] = nc < N ? sc.col(nc) : 0.0f;
         }
         const float cut = (float)eg.cut, s2i = (float)eg.sig2inv;
         const int mu = eg.mu0 + bz;
-        const float rf = m < M ? ldexpf(1.0f, __ldg(sc.e + m) + __ldg(sc.e + mu) + sc.eL() + sc.eR - kTBits - kEBits) : 0.0f;
+        const float rf = m < M ? sc.row(m, mu) : 0.0f;
         const F2 wmu = f2_of(eg.omega[mu]), nmu = f2_of(eg.occ[mu]);
         const F2 w1p = m < M ? f2_of(eg.omega[m]) : F2{0.f, 0.f};
         const F2 n1p = m < M ? f2_of(eg.occ[m]) : F2{0.f, 0.f};
@@ -409,14 +427,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
             const F2 nv = n < N ? f2_of(eg.occ[n]) : F2{0.f, 0.f};
             wn_sm[x] = wv.h; wl_sm[x] = wv.l;
             nn_sm[x] = nv.h; nl_sm[x] = nv.l;
-            cf_sm[x] = n < N ? ldexpf(1.0f, __ldg(sc.e + n)) : 0.0f;
+            cf_sm[x] = n < N ? sc.col(n) : 0.0f;
         }
         __syncthreads();
         const float cut = (float)eg.cut, s2i = (float)eg.sig2inv;
         const F2 wmu = f2_of(eg.omega[eg.mu0 + bz]);
-        const float rf = m < M ? ldexpf(1.0f, __ldg(sc.e + m) + __ldg(sc.e + eg.mu0 + bz) + sc.eL() + sc.eR - kTBits -
-                                                  kEBits)
-                               : 0.0f;
+        const float rf = m < M ? sc.row(m, eg.mu0 + bz) : 0.0f;
         const F2 w1p = m < M ? f2_of(eg.omega[m]) : F2{0.f, 0.f};
         const F2 n1p = m < M ? f2_of(eg.occ[m]) : F2{0.f, 0.f};
         const float w1 = w1p.h, n1 = n1p.h;
@@ -509,41 +525,81 @@ __global__ void gsym_sums_kernel(int nb, int n_part, const double *__restrict__ 
     gacc[m] = s;
 }
 
-// Exponent of each mode's largest eigenvector component: |E(m, .)| <= 2^e[m].
+// Bits of the largest |Phi3| (FP32) of the blocks of each atom, in s.  A warp per (j, k)
+// group, a lane per block.
+__global__ void __launch_bounds__(256)
+atom_strength_kernel(int n_groups, const int *__restrict__ group_start, const int *__restrict__ group_jk,
+                     const int *__restrict__ blk_i, const float2 *__restrict__ fc3, unsigned *s) {
+    const int g = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (g >= n_groups) return;                         // whole warps
+    auto put = [&](int atom, unsigned v) {
+        if (v > __ldcg(s + atom)) atomicMax(s + atom, v);
+    };
+    unsigned top = 0;
+    for (int b = group_start[g] + lane; b < group_start[g + 1]; b += 32) {
+        float m = 0.0f;
+#pragma unroll
+        for (int x = 0; x < 27; ++x) m = fmaxf(m, fabsf(__ldg(fc3 + (size_t)27 * b + x).x));
+        put(__ldg(blk_i + b), __float_as_uint(m));
+        top = max(top, __float_as_uint(m));
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    if (lane < 2) put(group_jk[2 * g + lane], top);
+}
+// Exponents of the atoms: a third of how far their Phi3 is below the largest one, so
+// that Phi3 2^(-k_i - k_j - k_k) is of one size throughout.  One CTA.
+__global__ void __launch_bounds__(256)
+atom_scale_kernel(int n_at, const unsigned *__restrict__ s, int *__restrict__ k) {
+    __shared__ unsigned top;
+    if (threadIdx.x == 0) top = 0;
+    __syncthreads();
+    unsigned m = 0;
+    for (int a = threadIdx.x; a < n_at; a += blockDim.x) m = max(m, s[a]);
+    atomicMax(&top, m);
+    __syncthreads();
+    int x0;
+    frexpf(__uint_as_float(top), &x0);
+    for (int a = threadIdx.x; a < n_at; a += blockDim.x) {
+        int x = -256;                                  // (no Phi3 at all: the least)
+        if (s[a]) frexpf(__uint_as_float(s[a]), &x);
+        k[a] = max(-30, min(0, (x - x0 - 1) / 3));
+    }
+}
+// Exponents of each mode: |E^(m, .)| <= 2^e[m], its norm <= 2^(e[m] + h[m]).
 __global__ void __launch_bounds__(128)
-mode_scale_kernel(int nb, const double2 *__restrict__ eig, int *__restrict__ e) {
-    __shared__ float red[4];
-    float v = 0.0f;
-    for (int c = threadIdx.x; c < nb; c += blockDim.x) v = fmaxf(v, fabsf((float)eig[(size_t)blockIdx.x * nb + c].x));
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+mode_scale_kernel(int nb, const double2 *__restrict__ eig, const int *__restrict__ k, int *__restrict__ e,
+                  int *__restrict__ h) {
+    __shared__ float red[2][4];
+    float v = 0.0f, n2 = 0.0f;
+    for (int c = threadIdx.x; c < nb; c += blockDim.x) {
+        const float x = fabsf(ldexpf((float)eig[(size_t)blockIdx.x * nb + c].x, __ldg(k + c / 3)));
+        v = fmaxf(v, x);
+        n2 = fmaf(x, x, n2);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+        n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        red[0][threadIdx.x >> 5] = v;
+        red[1][threadIdx.x >> 5] = n2;
+    }
     __syncthreads();
     if (threadIdx.x) return;
-    int x;
-    frexpf(fmaxf(fmaxf(red[0], red[1]), fmaxf(red[2], red[3])), &x);
+    int x, y;
+    frexpf(fmaxf(fmaxf(red[0][0], red[0][1]), fmaxf(red[0][2], red[0][3])), &x);
+    frexpf(1.001f * sqrtf(red[1][0] + red[1][1] + red[1][2] + red[1][3]), &y);
     e[blockIdx.x] = x;
-}
-// Largest sum of |Phi3| over the blocks and home components of an entry of Y_mu (a
-// bound: slightly enlarged), as the bits of a non-negative FP32 value.
-__global__ void __launch_bounds__(256)
-fc3_bound_kernel(int n_groups, const int *__restrict__ group_start, const float2 *__restrict__ fc3, int *l1) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    float s = 0.0f;
-    if (t < 9 * n_groups)
-        for (int b = group_start[t / 9]; b < group_start[t / 9 + 1]; ++b)
-            for (int a = 0; a < 3; ++a) s += fabsf(fc3[(size_t)27 * b + 9 * a + t % 9].x);
-    s *= 1.001f;
-    for (int o = 16; o > 0; o >>= 1) s = fmaxf(s, __shfl_xor_sync(0xffffffffu, s, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(l1, __float_as_int(s));
+    h[blockIdx.x] = max(0, y - x);
 }
 // hi/lo FP16 planes of the scaled eigenvectors (padding stays zero from the caller's
 // memset).
-__global__ void split_kernel(int nb, const double2 *__restrict__ eig, const int *__restrict__ e, int ld,
-                             __half *__restrict__ hi, __half *__restrict__ lo) {
+__global__ void split_kernel(int nb, const double2 *__restrict__ eig, const int *__restrict__ k,
+                             const int *__restrict__ e, int ld, __half *__restrict__ hi, __half *__restrict__ lo) {
     const size_t n = (size_t)nb * nb;
     for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < n; x += (size_t)gridDim.x * blockDim.x) {
         const size_t r = x / nb, c = x % nb;
-        const float v = (float)ldexp(eig[x].x, kEBits - __ldg(e + r));
+        const float v = (float)ldexp(eig[x].x, kEBits - __ldg(e + r) + __ldg(k + c / 3));
         const __half h = __float2half_rn(v);
         hi[r * ld + c] = h;
         lo[r * ld + c] = __float2half_rn(v - __half2float(h));
@@ -588,9 +644,10 @@ __device__ __forceinline__ void pair_fma(F2 &acc, float2 a, float2 b) {
     acc.l = __fadd_rn(acc.l, __fadd_rn(r, e));
 }
 
-// YT[c][b] of modes mu0 .. mu0 + nm - 1 straight into their FP16 hi/lo planes
-// (plane stride plane_elems).  Sums of FP32 pairs (about 46 bits), rounded
-// once to FP32 and then split.
+// Y^_mu(c, b) of modes mu0 .. mu0 + nm - 1, in FP32 by entry: out[m][9 group + 3 (b % 3) +
+// c % 3], groups in `order`, and the bits of each mode's largest one in ymax.  Sums of
+// FP32 pairs (about 46 bits), rounded once.  y_store_kernel makes the planes:
+// their scale is known when the whole Y_mu is.
 //
 // Bound: FP64 units.  As plain FP64 sums (one thread per output and mode, 2
 // FP64 FMA per clock and SM) this build took 173 us per launch of 18 modes of a 768-mode
@@ -605,8 +662,9 @@ template <int MT>
 __global__ void __launch_bounds__(256)
 ybuild_pair_kernel(int n_groups, int n_long, const int *__restrict__ order, const int *__restrict__ group_jk,
                    const int *__restrict__ group_start, const int *__restrict__ blk_i,
-                   const float2 *__restrict__ fc3, const float2 *__restrict__ Et, int ldm, int mu0, int nm, int ld,
-                   size_t plane_elems, Scales sc, __half *__restrict__ hi, __half *__restrict__ lo) {
+                   const float2 *__restrict__ fc3, const float2 *__restrict__ Et, int ldm, int mu0, int nm,
+                   const int *__restrict__ kx, float *__restrict__ out, unsigned *ymax) {
+    __shared__ unsigned top_sm[8][MT];
     const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     const int m0 = blockIdx.y * MT;
     const bool lng = gw < n_long;                      // uniform over the warp
@@ -615,6 +673,8 @@ ybuild_pair_kernel(int n_groups, int n_long, const int *__restrict__ order, cons
     const int bg = lng ? lane % 9 : t % 9;
     const bool act = gi < n_groups && (!lng || lane < 27);
     const int g = act ? order[gi] : 0;
+    const bool put = act && !(lng && lane >= 9);
+    const int ks = put ? __ldg(kx + __ldg(group_jk + 2 * g)) + __ldg(kx + __ldg(group_jk + 2 * g + 1)) : 0;
     F2 acc[MT];
 #pragma unroll
     for (int m = 0; m < MT; ++m) acc[m] = F2{0.f, 0.f};
@@ -645,18 +705,68 @@ ybuild_pair_kernel(int n_groups, int n_long, const int *__restrict__ order, cons
             acc[m] = f2_add(f2_add(acc[m], p[0]), p[1]);
         }
     }
-    if (!act || (lng && lane >= 9)) return;
-    const int j = group_jk[2 * g], k = group_jk[2 * g + 1];
-    const size_t off = (size_t)(3 * k + bg % 3) * ld + 3 * j + bg / 3;
-    const int eL = sc.eL();
 #pragma unroll
     for (int m = 0; m < MT; ++m) {
-        if (m0 + m >= nm) break;
-        const float v = __fadd_rn(acc[m].h, acc[m].l) * ldexpf(1.0f, kYBits - eL - __ldg(sc.e + mu0 + m0 + m));
-        const __half h = __float2half_rn(v);
-        const size_t o = (size_t)(m0 + m) * plane_elems + off;
-        hi[o] = h;
-        lo[o] = __float2half_rn(v - __half2float(h));
+        const float v = put ? ldexpf(__fadd_rn(acc[m].h, acc[m].l), -ks) : 0.0f;
+        if (put && m0 + m < nm) out[(size_t)(m0 + m) * 9 * n_groups + 9 * gi + bg] = v;
+        const unsigned t1 = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(v)));
+        if (lane == 0) top_sm[threadIdx.x >> 5][m] = t1;
+    }
+    __syncthreads();
+    if (threadIdx.x < MT && m0 + (int)threadIdx.x < nm) {
+        unsigned t1 = 0;
+        for (int w = 0; w < 8; ++w) t1 = max(t1, top_sm[w][threadIdx.x]);
+        atomicMax(ymax + mu0 + m0 + threadIdx.x, t1);
+    }
+}
+
+// The rows c = 3 k .. 3 k + 2 of the scaled Y of up to kYStoreModes modes, hi/lo planes
+// (plane stride plane_elems): CTA = (k, modes), its groups (place in `order`, j) at
+// k_at[k_start[k]] ..
+//
+// Bound: latency, then the writes.  Whole rows, assembled in shared memory, zeros and
+// all: storing the entries where they belong, two bytes each, made the memory fetch and
+// write back a 32-byte sector for every three of them.
+constexpr int kYStoreModes = 4, kYStoreCols = 768;
+__global__ void __launch_bounds__(256)
+y_store_kernel(int n_groups, const int *__restrict__ k_start, const int2 *__restrict__ k_at,
+               const float *__restrict__ y, int mu0, int nm, int ld, size_t plane_elems, Scales sc,
+               __half *__restrict__ hi, __half *__restrict__ lo) {
+    __shared__ __align__(16) __half row[kYStoreModes][2][3][kYStoreCols];
+    const int k = blockIdx.x, m0 = blockIdx.y * kYStoreModes, n_m = min(kYStoreModes, nm - m0);
+    const int s0 = k_start[k], n_e = 9 * (k_start[k + 1] - s0);
+    int sh[kYStoreModes];
+#pragma unroll
+    for (int m = 0; m < kYStoreModes; ++m) sh[m] = kYBits - sc.y(mu0 + m0 + min(m, n_m - 1));
+    for (int c0 = 0; c0 < ld; c0 += kYStoreCols) {
+        const int w8 = min(kYStoreCols, ld - c0) / 8;             // (ld is a multiple of 128)
+        __syncthreads();
+        for (int x = threadIdx.x; x < (int)sizeof(row) / 16; x += 256)
+            reinterpret_cast<uint4 *>(row)[x] = make_uint4(0, 0, 0, 0);
+        __syncthreads();
+        for (int x = threadIdx.x; x < n_e; x += 256) {
+            const int p = x / 9, bg = x - 9 * p;
+            const int2 a = __ldg(k_at + s0 + p);
+            const int c = 3 * a.y + bg / 3 - c0;
+            if (c < 0 || c >= kYStoreCols) continue;
+            float v[kYStoreModes];
+#pragma unroll
+            for (int m = 0; m < kYStoreModes; ++m)
+                v[m] = __ldg(y + (size_t)(m0 + min(m, n_m - 1)) * 9 * n_groups + 9 * a.x + bg);
+#pragma unroll
+            for (int m = 0; m < kYStoreModes; ++m) {
+                const float s = ldexpf(v[m], sh[m]);
+                const __half h = __float2half_rn(s);
+                row[m][0][bg % 3][c] = h;
+                row[m][1][bg % 3][c] = __float2half_rn(s - __half2float(h));
+            }
+        }
+        __syncthreads();
+        for (int x = threadIdx.x; x < n_m * 6 * w8; x += 256) {
+            const int r = x / w8, z = x - r * w8, m = r / 6, pl = r / 3 % 2, g = r % 3;
+            __half *out = (pl ? lo : hi) + (size_t)(m0 + m) * plane_elems + (size_t)(3 * k + g) * ld + c0;
+            reinterpret_cast<uint4 *>(out)[z] = reinterpret_cast<const uint4 *>(row[m][pl][g])[z];
+        }
     }
 }
 
@@ -720,6 +830,9 @@ static int tc_ldm(int nb) { return (nb + 3 + 31) / 32 * 32; }
 static size_t tc_gsym_bytes(size_t n_tiles) { return ws_round(sizeof(double) * kBM * std::max<size_t>(n_tiles, 1)); }
 static int tc_gsym_parts(int nb) { return (nb + kSumModes - 1) / kSumModes; }
 
+// e, h and ymax of the modes, the strengths and the exponents of the atoms.
+static size_t tc_scale_ints(int nb) { return 3 * (size_t)nb + 2 * (size_t)((nb + 2) / 3); }
+
 size_t tc_gamma_scratch_bytes(int nb, int mb_max, size_t n_fc3, int sym3, size_t n_tiles) {
     const int ld = (nb + kBN - 1) / kBN * kBN;     // whole 128-column tiles per row
     const int rows = (nb + kBM - 1) / kBM * kBM;
@@ -728,7 +841,7 @@ size_t tc_gamma_scratch_bytes(int nb, int mb_max, size_t n_fc3, int sym3, size_t
     // then the FP32 pairs of Phi3 and of the eigenvectors and the scales, then (Phi3 symmetric under
     // every permutation) the tiles' sums and the modes' sums
     return (2 + 4 * (size_t)mb_max) * plane + ws_round(sizeof(float2) * 27 * std::max<size_t>(n_fc3, 1)) +
-           ws_round(sizeof(float2) * (size_t)nb * tc_ldm(nb)) + ws_round(sizeof(int) * (size_t)(nb + 4)) +
+           ws_round(sizeof(float2) * (size_t)nb * tc_ldm(nb)) + ws_round(sizeof(int) * tc_scale_ints(nb)) +
            (sym3 ? 2 * tc_gsym_bytes(n_tiles) + ws_round(sizeof(double) * (size_t)nb * (1 + tc_gsym_parts(nb))) : 0);
 }
 
@@ -750,7 +863,7 @@ cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const L
     __half *El = reinterpret_cast<__half *>(b + plane);
     auto S = [&](int i) { return reinterpret_cast<__half *>(b + 2 * plane + i * stack); };
     __half *Yh = S(0), *Yl = S(1), *Th = S(2), *Tl = S(3);
-    cudaError_t e = cudaMemsetAsync(b, 0, 2 * plane + 4 * stack, st);
+    cudaError_t e = cudaMemsetAsync(b, 0, 2 * plane + 2 * stack, st);       // E and Y
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(err, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
@@ -759,7 +872,7 @@ cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const L
     float2 *fc3p = reinterpret_cast<float2 *>(pairs);
     float2 *Et = reinterpret_cast<float2 *>(pairs + ws_round(sizeof(float2) * 27 * std::max<size_t>(gp.n_fc3, 1)));
     char *sums = reinterpret_cast<char *>(Et) + ws_round(sizeof(float2) * (size_t)nb * ldm);
-    char *gsums = sums + ws_round(sizeof(int) * (size_t)(nb + 4));
+    char *gsums = sums + ws_round(sizeof(int) * tc_scale_ints(nb));
     double *rowp = nullptr, *colp = nullptr, *gacc = nullptr;
     // tile_start follows the tiles (same allocation)
     int *ts = reinterpret_cast<int *>(tiles_dev + std::max<size_t>(tiles.size(), 1));
@@ -775,16 +888,21 @@ cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const L
     if (nf) fc3_pair_kernel<<<counted((unsigned)std::min<size_t>((nf + 255) / 256, 4096)), 256, 0, st>>>(nf, d.fc3, fc3p);
     eig_pair_kernel<<<counted(dim3((nb + 31) / 32, (nb + 31) / 32)), 256, 0, st>>>(
         nb, reinterpret_cast<const double2 *>(d.eig), ldm, Et);
-    int *l1 = reinterpret_cast<int *>(sums), *em = l1 + 4;
-    e = cudaMemsetAsync(l1, 0, sizeof(int), st);
+    const int n_at = nb / 3;
+    int *em = reinterpret_cast<int *>(sums), *hm = em + nb, *ymax = hm + nb, *kx = ymax + nb;
+    unsigned *strength = reinterpret_cast<unsigned *>(kx + n_at);
+    e = cudaMemsetAsync(ymax, 0, sizeof(int) * (size_t)nb, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(strength, 0, sizeof(int) * (size_t)n_at, st);
     if (e != cudaSuccess) return e;
     if (gp.n_groups)
-        fc3_bound_kernel<<<counted((9 * gp.n_groups + 255) / 256), 256, 0, st>>>(gp.n_groups, d.group_start, fc3p, l1);
-    mode_scale_kernel<<<counted(nb), 128, 0, st>>>(nb, reinterpret_cast<const double2 *>(d.eig), em);
-    int eR = 0;
-    while ((1LL << eR) < gp.row_entries) ++eR;
-    const Scales sc{l1, em, eR};
-    split_kernel<<<counted(4096), 256, 0, st>>>(nb, reinterpret_cast<const double2 *>(d.eig), em, ld, Eh, El);
+        atom_strength_kernel<<<counted((gp.n_groups + 7) / 8), 256, 0, st>>>(gp.n_groups, d.group_start, d.group_jk,
+                                                                            d.blk_i, fc3p, strength);
+    atom_scale_kernel<<<counted(1), 256, 0, st>>>(n_at, strength, kx);
+    mode_scale_kernel<<<counted(nb), 128, 0, st>>>(nb, reinterpret_cast<const double2 *>(d.eig), kx, em, hm);
+    int hR = 0;
+    while ((1LL << (2 * hR)) < gp.row_entries) ++hR;
+    const Scales sc{em, hm, ymax, hR};
+    split_kernel<<<counted(4096), 256, 0, st>>>(nb, reinterpret_cast<const double2 *>(d.eig), kx, em, ld, Eh, El);
     // the planes of one stack are contiguous: plane_elems = plane / 2 elements apart
     const size_t plane_elems = plane / sizeof(__half);
     const int stack_rows = (int)((size_t)mb * plane_elems / ld);
@@ -814,20 +932,25 @@ cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const L
         const int nm = std::min(mb, nb - mu0);
         const int t0 = tile_start[mu0], t1 = tile_start[mu0 + nm];
         if (t1 == t0) continue;                     // no delta-band tile (masked modes)
-        // Y_mu^T planes: every batch writes the same (sparse) pattern of
-        // entries, so the previous batch's values are all overwritten
+        // the entries of Y stand in the T planes before they are scaled (9 n_groups <=
+        // nb^2 FP32 values per mode there, and the first contraction writes every tile
+        // that the second reads)
+        float *yf = reinterpret_cast<float *>(Th);
         const long long yth = 32LL * gp.n_long + 9LL * (gp.n_groups - gp.n_long);
         const unsigned ygx = (unsigned)((yth + 255) / 256);
         auto ybuild = [&](auto kern, int mt) {
             kern<<<counted(dim3(ygx, (nm + mt - 1) / mt)), 256, 0, st>>>(gp.n_groups, gp.n_long, d.group_order,
                                                                          d.group_jk, d.group_start, d.blk_i, fc3p, Et,
-                                                                         ldm, mu0, nm, ld, plane_elems, sc, Yh, Yl);
+                                                                         ldm, mu0, nm, kx, yf,
+                                                                         reinterpret_cast<unsigned *>(ymax));
         };
         // modes per thread: 4, or 3 where that leaves fewer of them unused
         if (nm == 1) ybuild(ybuild_pair_kernel<1>, 1);
         else if (nm == 2) ybuild(ybuild_pair_kernel<2>, 2);
         else if ((nm + 2) / 3 * 3 < (nm + 3) / 4 * 4) ybuild(ybuild_pair_kernel<3>, 3);
         else ybuild(ybuild_pair_kernel<4>, 4);
+        y_store_kernel<<<counted(dim3(n_at, (nm + kYStoreModes - 1) / kYStoreModes)), 256, 0, st>>>(
+            gp.n_groups, d.k_start, d.k_at, yf, mu0, nm, ld, plane_elems, sc, Yh, Yl);
         // (with sym3 the tiles of a mode start at its own row tile)
         const int tm0 = gp.sym3 ? mu0 / kBM : 0;
         EpiSplit es{Th, Tl, ld, prow, tm0};

@@ -539,3 +539,59 @@ def test_repeated_blocks_are_added(k, cell, mesh, precision):
     got, _ = kk.kald_linewidths(ctx, [twice], mesh, nu.ravel(), eig.ravel(),
                                 kk.Options(temperature_K=300.0, sigma_thz=0.1, precision=precision))
     assert _rel(got, ref) < (1e-10 if precision == "fp64" else 1e-5)
+
+
+def _two_parts(cell, ratio, mix):
+    """Two copies of a cell in one, the second with Phi2 0.81 and Phi3 `ratio` times the
+    first's and no force between them (nor a mode of one in a degenerate set with one of
+    the other, whose linewidths would be averaged); with `mix`, pairs of modes of the two (of nearly
+    one frequency) rotated into each other and given their mean frequency."""
+    from dataclasses import replace
+    a = ki.fcc_supercell_system(cell, seed=5)
+    n = a.n_atoms
+    i2, i3 = a.fc2_idx.copy(), a.fc3_idx.copy()
+    i2[:, :2] += n
+    i3[:, [0, 1, 5]] += n
+    s = replace(a, masses=np.tile(a.masses, 2), positions=np.concatenate([a.positions, a.positions + 1.3]),
+                fc2_idx=np.concatenate([a.fc2_idx, i2]), fc2=np.concatenate([a.fc2, 0.81 * a.fc2]),
+                fc3_idx=np.concatenate([a.fc3_idx, i3]), fc3=np.concatenate([a.fc3, ratio * a.fc3]))
+    nu, eig = ph.phonons(a, (1, 1, 1))
+    nb = 3 * n
+    nu2 = np.concatenate([nu[0], 0.9 * nu[0]])
+    E = np.zeros((2 * nb, 2 * nb))
+    E[:nb, :nb] = E[nb:, nb:] = eig[0].real
+    part = np.repeat([0, 1], nb)
+    if mix:
+        # every fourth mode of the first part from the 10th with the mode of the second nearest to it
+        left = set(range(nb + 10, 2 * nb))
+        for m in range(10, nb, 4):
+            o = min(left, key=lambda x: abs(nu2[x] - nu2[m]))
+            left.remove(o)
+            E[m], E[o] = (E[m] + E[o]) / np.sqrt(2), (E[m] - E[o]) / np.sqrt(2)
+            nu2[m] = nu2[o] = 0.5 * (nu2[m] + nu2[o])
+            nu2[o] += 1e-3                           # (not a degenerate set)
+            part[[m, o]] = 2
+    order = np.argsort(nu2, kind="stable")
+    other = (part[order][1:] != part[order][:-1]) & (nu2[order][1:] > 0.01)
+    assert np.diff(nu2[order])[other].min() > 1e-5
+    return s, nu2[order][None], E[order].astype(complex)[None], part[order]
+
+
+@pytest.mark.parametrize("symmetry", ["all", "inversion"])
+@pytest.mark.parametrize("mix", [False, True])
+@pytest.mark.parametrize("log_ratio", [0, 12, 20, 24])
+def test_gamma_only_split_of_unlike_parts(k, log_ratio, mix, symmetry):
+    """A part whose Phi3 is up to 2^24 times weaker than the rest of the cell keeps the
+    linewidths of its modes (gamma 2^48 times smaller: each part is compared with its own
+    largest) to the 1e-5 of the mode, as do modes that extend over both parts; each triple
+    of modes projected once and three times."""
+    kk, ctx = k
+    s, nu, eig, part = _two_parts((3, 3, 1), 2.0 ** -log_ratio, mix)
+    out = {}
+    for prec in ("fp64", "bf16split"):
+        opt = kk.Options(temperature_K=300.0, sigma_thz=0.1, precision=prec, symmetry=symmetry)
+        out[prec] = kk.kald_linewidths(ctx, [s], (1, 1, 1), nu.ravel(), eig.ravel(), opt)
+    assert abs(out["fp64"][1][1] - out["bf16split"][1][1]) <= 1e-5 * out["fp64"][1][1]
+    ref, got = (np.asarray(out[p][0]).ravel() for p in ("fp64", "bf16split"))
+    for x in set(part):
+        assert _rel(got[part == x], ref[part == x]) < 1e-5
