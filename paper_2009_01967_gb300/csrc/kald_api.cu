@@ -1644,13 +1644,8 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
         const TcxPlanHost no_plan;
         const LwTermsHost &lt = ltp ? *ltp : no_terms;
         const TcxPlanHost &tp = tpp ? *tpp : no_plan;
-        size_t cc_out3 = 0, cc_sums = 0;         // position sums of the mode blocks, and where their totals start
-        if (cc_pairs) {
-            const int blocks = lw_orbit_blocks(nb, cc_pairs, f32w, ctx->sm_count, ctx->smem_optin);
-            cc_sums = blocks > 1 ? 3 * (size_t)cc_pairs * nb * blocks : 0;
-            cc_out3 = 3 * (size_t)cc_pairs * nb * (blocks > 1 ? blocks + 1 : 1);
-            p.n_chunks = 1;
-        }
+        const size_t cc_out3 = cc_pairs ? lw_orbit_sums(nb, cc_pairs, f32w, ctx->sm_count, ctx->smem_optin) : 0;
+        if (cc_pairs) p.n_chunks = 1;
         if (small) p.n_rep = 0;                  // the register kernel takes its phases from roots of unity
         std::vector<int4> binfo(small ? 1 : std::max<size_t>(n3, 1), make_int4(0, 0, 0, 0));
         for (size_t b = 0; !small && b < n3; ++b) binfo[b] = make_int4(h.fc3_i[b], h.fc3_rj[b], h.fc3_rk[b], 0);
@@ -1784,6 +1779,7 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
             terms.n_pairs = orb.n_pairs;
             terms.pairs = orb.pairs;
             terms.orbit = orb.orbit;
+            terms.plan = &orb;
         }
         if (e == cudaSuccess) e = launch_lw_prep(p, d, f32w, s);
         if (tcx) {
@@ -1804,7 +1800,6 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
                 : tcx ? launch_lw_tensor(p, d, tg, tc_scr, tcx_b, ctx->sm_count, tc_err, s,
                                          use_sym ? &orb : nullptr, sym_scr)
                       : launch_lw_main(p, d, terms, f32w, ctx->sm_count, ctx->smem_optin, s);
-        if (e == cudaSuccess && cc_pairs) e = launch_orbit_class_sums(orb, nb, terms.out3 + cc_sums, d.partial, s);
         if (e == cudaSuccess) e = launch_lw_finish(p, d, opt->degen_tol_thz, g_d, s);
         if (e != cudaSuccess) return cuda_check(ctx, e, "kald_linewidths launch");
         unsigned long long al = 0;

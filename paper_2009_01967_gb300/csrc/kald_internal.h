@@ -297,11 +297,15 @@ cudaError_t launch_orbit_plan(const int32_t mesh[3], int n_rows, const int *rows
 // [n_pairs][3][nb] (nb <= 96) of its orbits.
 cudaError_t launch_orbit_class_sums(const OrbitPlan &o, int nb, const float *out3, double *out, cudaStream_t st);
 cudaError_t launch_orbit_class_sums(const OrbitPlan &o, int nb, const double *out3, double *out, cudaStream_t st);
+// The same from the orbits p0 .. p1 - 1 (out3 from p0 on), added to out when p0 > 0.
+cudaError_t launch_orbit_class_sums(const OrbitPlan &o, int nb, int p0, int p1, const double *out3, double *out,
+                                    cudaStream_t st);
 
 // The phase sums of the CUDA-core kernel (plan_lw_terms): per (j, k) group its
 // terms (i, class, slot) -- phase sums of class 0, 1 or 2 from tables per q', q''
 // or q -- or (i, 3, block), phased per pair.  n_pairs > 0: one projection per
-// orbit (pairs, orbit of an OrbitPlan, the positions' sums into out3).
+// orbit (pairs, orbit of the OrbitPlan `plan`), the positions' sums through out3 into
+// LwDev::partial.
 struct LwTermsHost {
     std::vector<int> group, term_start, slot_start, slot_blk;
     std::vector<int4> term;
@@ -326,10 +330,11 @@ struct LwTerms {
     int n_pairs = 0;
     const int2 *pairs = nullptr;
     const int *orbit = nullptr;
-    double *out3 = nullptr;            // [n_pairs][blocks][3][nb] (lw_orbit_blocks)
+    double *out3 = nullptr;            // lw_orbit_sums values: [pairs of a launch][blocks][3][nb] ..
+    const OrbitPlan *plan = nullptr;
     int n_sblk = 1, s_per = 0;         // blocks of modes per item, modes per block (set by the launch)
 };
-int lw_orbit_blocks(int nb, int n_pairs, int fp32, int sm_count, size_t smem_optin);
+size_t lw_orbit_sums(int nb, int n_pairs, int fp32, int sm_count, size_t smem_optin);
 void plan_lw_terms(const HostSystem &h, bool tables, LwTermsHost &o);
 cudaError_t launch_lw_tables_f32(int nq, int n_rep, const LwTerms &t, const int4 *blkinfo, const float *fc3,
                                  const float2 *chi, cudaStream_t st);

@@ -144,13 +144,14 @@ orbit_fill_kernel(Mesh3 m, int nq, int words, const int *__restrict__ rows, cons
 }
 
 // out[i][s] = 1/2 sum over q2 of the sums of q = rows[i] in the orbit of
-// (q, q2, -(q + q2)): out3[pair][place][s] (FP64 here; a fixed order: every lane
-// group its q2 in steps, then the groups in order).  CTA = row, threads (group, s).
+// (q, q2, -(q + q2)): out3[pair - p0][place][s] (FP64 here; a fixed order: every lane
+// group its q2 in steps, then the groups in order), of the pairs p0 .. p1 - 1 alone;
+// `add`: on top of what out holds.  CTA = row, threads (group, s).
 template <typename T>
 __global__ void __launch_bounds__(256)
 orbit_class_sums_kernel(Mesh3 m, int nq, int nb, int words, const int *__restrict__ rows, const int *__restrict__ row_of,
-                        const uint2 *__restrict__ bits, const int *__restrict__ start, const T *__restrict__ out3,
-                        double *__restrict__ out) {
+                        const uint2 *__restrict__ bits, const int *__restrict__ start, int p0, int p1, int add,
+                        const T *__restrict__ out3, double *__restrict__ out) {
     __shared__ int ent[256];
     __shared__ double red[256];
     const int i = blockIdx.x, q = rows[i], tid = threadIdx.x;
@@ -165,18 +166,21 @@ orbit_class_sums_kernel(Mesh3 m, int nq, int nb, int words, const int *__restric
             const int c1 = (int)(key / (unsigned)nq), c2 = (int)(key - (unsigned long long)c1 * nq);
             const int r = row_of[c1];
             const uint2 w = bits[(size_t)r * words + (c2 >> 5)];
-            ent[tid] = 3 * (start[r] + (int)w.y + __popc(w.x & ((1u << (c2 & 31)) - 1u))) + place;
+            const int pair = start[r] + (int)w.y + __popc(w.x & ((1u << (c2 & 31)) - 1u));
+            ent[tid] = pair >= p0 && pair < p1 ? 3 * (pair - p0) + place : -1;
         }
         __syncthreads();
         if (g < groups)
-            for (int x = g; x < min(256, nq - q0); x += groups) sum += (double)out3[(size_t)ent[x] * nb + s];
+            for (int x = g; x < min(256, nq - q0); x += groups)
+                if (ent[x] >= 0) sum += (double)out3[(size_t)ent[x] * nb + s];
     }
     red[tid] = sum;
     __syncthreads();
     if (tid < nb) {
         double t = 0.0;
         for (int x = 0; x < groups; ++x) t += red[x * nb + tid];
-        out[(size_t)i * nb + tid] = 0.5 * t;
+        double *o = out + (size_t)i * nb + tid;
+        *o = (add ? *o : 0.0) + 0.5 * t;
     }
 }
 
@@ -234,17 +238,21 @@ cudaError_t launch_orbit_plan(const int32_t mesh[3], int n_rows, const int *rows
 }
 
 template <typename T>
-static cudaError_t class_sums(const OrbitPlan &o, int nb, const T *out3, double *out, cudaStream_t st) {
+static cudaError_t class_sums(const OrbitPlan &o, int nb, int p0, int p1, const T *out3, double *out, cudaStream_t st) {
     const Mesh3 m{o.mesh[0], o.mesh[1], o.mesh[2]};
     orbit_class_sums_kernel<T><<<counted(o.n_rows), 256, 0, st>>>(m, o.nq, nb, orbit_words(o.nq), o.rows, o.row_of, o.bits,
-                                                                  o.start, out3, out);
+                                                                  o.start, p0, p1, p0 > 0, out3, out);
     return cudaGetLastError();
 }
 cudaError_t launch_orbit_class_sums(const OrbitPlan &o, int nb, const float *out3, double *out, cudaStream_t st) {
-    return class_sums(o, nb, out3, out, st);
+    return class_sums(o, nb, 0, o.n_pairs, out3, out, st);
 }
 cudaError_t launch_orbit_class_sums(const OrbitPlan &o, int nb, const double *out3, double *out, cudaStream_t st) {
-    return class_sums(o, nb, out3, out, st);
+    return class_sums(o, nb, 0, o.n_pairs, out3, out, st);
+}
+cudaError_t launch_orbit_class_sums(const OrbitPlan &o, int nb, int p0, int p1, const double *out3, double *out,
+                                    cudaStream_t st) {
+    return class_sums(o, nb, p0, p1, out3, out, st);
 }
 
 }  // namespace kald

@@ -595,3 +595,31 @@ def test_gamma_only_split_of_unlike_parts(k, log_ratio, mix, symmetry):
     ref, got = (np.asarray(out[p][0]).ravel() for p in ("fp64", "bf16split"))
     for x in set(part):
         assert _rel(got[part == x], ref[part == x]) < 1e-5
+
+
+def test_orbit_sums_of_a_dense_mesh(k):
+    """Three atoms on 20^3: 5.3 million orbits whose positions' sums would take 1.15 GB.
+    They are projected in several launches, so that the context holds less than a GB for
+    them all with everything else (256 MB of sums, 0.4 GB of tables and orbits), and the
+    linewidths are those of single q-points, which use time reversal only."""
+    torch = pytest.importorskip("torch")
+    from kald_inputs.configs import A_FCC
+    from kald_inputs.lattice import fcc_primitive
+    from kald_inputs.lj import lj_system
+    kk, _ = k
+    lat = fcc_primitive(A_FCC)[0]
+    s = lj_system(lat * np.array([3, 1, 1])[:, None], np.arange(3)[:, None] * lat[:1], [39.948, 60.0, 39.948])
+    mesh = (20, 20, 20)
+    opt = kk.Options(temperature_K=300.0, sigma_thz=0.1, precision="fp64")
+    with kk.Context(0) as ctx:
+        nu, eig, _ = kk.kald_phonons(ctx, s, mesh, want_vel=False)
+        qs = [1, 777, 4210, 7999]
+        ref, _ = kk.kald_linewidths_qlist(ctx, s, mesh, nu.ravel(), eig.ravel(), opt, qs)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    with kk.Context(0) as ctx:
+        g, _ = kk.kald_linewidths(ctx, s, mesh, nu.ravel(), eig.ravel(), opt)
+        held = free - torch.cuda.mem_get_info()[0]
+    assert held < 1 << 30
+    g = np.asarray(g).reshape(8000, 9)[qs]
+    assert _rel(g, np.asarray(ref).reshape(g.shape)) < 1e-10
