@@ -529,7 +529,7 @@ struct QhgkWork {
     QhgkModes modes;
     double *W;                // [3][nb][nb]
     void *oz;                 // oz_work_bytes(nb, dirs)
-    int dirs;                 // directions whose slices are held at once: 3, or 1
+    int dirs;                 // directions whose slices are held at once: 3, or 1 (and 128 rows)
     int *err;                 // bounded-wait failures
 };
 // qhgk_gemm.cu: W_a = E B_a^T scaled by fac per mode, over B_a [3][n][n] in BW;

@@ -50,19 +50,19 @@ __device__ __forceinline__ uint64_t smem_desc64(const void *p) {
     return ((a >> 4) & 0x3FFFull) | (1ull << 16) | ((uint64_t)(512 >> 4) << 32) | (1ull << 46) | (4ull << 61);
 }
 
-// Digits of one row per CTA: src row (stride in elements of T; the real part of
-// a double2) -> planes [kOz][rows][ld], zero past n and for rows past n.  The
-// row's scale: 2^(exponent) x fac[row] (NaN when the row holds a value that is
-// not finite, so that the product does not hide it).
+// Digits of one row per CTA, row r0 + blockIdx.x: src row (stride in elements of T; the
+// real part of a double2) -> row blockIdx.x of the planes [kOz][rows][ld], zero past n
+// and for rows past n.  The row's scale: 2^(exponent) x fac[row] (NaN when the row holds
+// a value that is not finite, so that the product does not hide it).
 template <typename T>
 __global__ void __launch_bounds__(256)
-oz_slice_kernel(int n, int rows, int ld, const T *__restrict__ src_all, const double *__restrict__ fac,
+oz_slice_kernel(int n, int r0, int rows, int ld, const T *__restrict__ src_all, const double *__restrict__ fac,
                 __nv_bfloat16 *__restrict__ out_all, double *__restrict__ scale_all) {
     __shared__ double red[8];
     __shared__ int bad;
-    const int row = blockIdx.x, dir = blockIdx.y, tid = threadIdx.x;
+    const int row = r0 + blockIdx.x, dir = blockIdx.y, tid = threadIdx.x;
     const T *src = src_all + ((size_t)dir * n + row) * n;
-    __nv_bfloat16 *out = out_all + ((size_t)dir * kOz * rows + row) * ld;
+    __nv_bfloat16 *out = out_all + ((size_t)dir * kOz * rows + blockIdx.x) * ld;
     const size_t plane = (size_t)rows * ld;
     auto val = [&](int c) {
         if constexpr (sizeof(T) == 16) return src[c].x;
@@ -106,9 +106,11 @@ oz_slice_kernel(int n, int rows, int ld, const T *__restrict__ src_all, const do
     }
 }
 
+// The rows [128 tm0, 128 (tm0 + gridDim.y)) of W; mA holds their digits from row 0 on.
+// (What a box reaches past the planes' rows and columns is zero.)
 __global__ void __launch_bounds__(kOzThreads, 1)
 oz_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB, int n, int n_st,
-               int antisym, const double *__restrict__ sa, const double *__restrict__ sb, double *__restrict__ W,
+               int tm0, int antisym, const double *__restrict__ sa, const double *__restrict__ sb, double *__restrict__ W,
                int *err, uint32_t wait_limit) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *base = reinterpret_cast<unsigned char *>(
@@ -116,7 +118,7 @@ oz_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ C
     __shared__ __align__(8) uint64_t full[2], empty[2], tfull, tempty, drain;
     __shared__ uint32_t tmem_base_sm;
     __shared__ int fail_sm;
-    const int tn = blockIdx.x, tm = blockIdx.y, dir = blockIdx.z;
+    const int tn = blockIdx.x, tm = tm0 + blockIdx.y, dir = blockIdx.z;
     if (antisym && (tn + 1) * kOzBN <= tm * kOzBM) return;       // below the diagonal
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr int spc = kOzChunk / kOzBK;                         // stages per chunk
@@ -148,7 +150,7 @@ oz_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ C
                 if (*(volatile int *)&fail_sm) break;
                 unsigned char *st = base + (size_t)s * kOzStage;
                 mbar_expect_tx(&full[s], kOzStage);
-                tma_load_3d(st, &mA, &full[s], it * kOzBK, tm * kOzBM, 0);
+                tma_load_3d(st, &mA, &full[s], it * kOzBK, (int)blockIdx.y * kOzBM, 0);
                 tma_load_3d(st + kOz * kOzA, &mB, &full[s], it * kOzBK, tn * kOzBN, dir * kOz);
                 ++issued;
             }
@@ -252,9 +254,10 @@ antisym_fill_kernel(int n, double *__restrict__ W_all) {
         if (c0 + r < n && r0 + tx < n && c0 + r > r0 + tx) W[(size_t)(c0 + r) * n + r0 + tx] = -tile[tx][r];
 }
 
-int oz_rows(int n) { return (n + kOzBM - 1) / kOzBM * kOzBM; }
-int oz_ld(int n) { return (n + kOzBK - 1) / kOzBK * kOzBK; }
-size_t oz_plane(int n) { return sizeof(__nv_bfloat16) * (size_t)oz_rows(n) * oz_ld(n); }
+int oz_ld(int n) { return (n + 7) / 8 * 8; }          // (16-byte rows)
+size_t oz_planes(int n, int rows) { return sizeof(__nv_bfloat16) * kOz * (size_t)rows * oz_ld(n); }
+// Rows of E whose digits are held at once: all of them, or those of one row of tiles.
+int oz_rows(int n, int dirs) { return dirs == 3 ? n : std::min(n, kOzBM); }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
@@ -284,28 +287,33 @@ bool oz_map(CUtensorMap *map, const void *ptr, int ld, int rows, int planes, int
 }  // namespace
 
 size_t oz_work_bytes(int n, int dirs) {
-    return ws_round(kOz * oz_plane(n)) + ws_round(dirs * kOz * oz_plane(n)) + ws_round(sizeof(double) * 4 * (size_t)n);
+    return ws_round(oz_planes(n, oz_rows(n, dirs))) + ws_round(dirs * oz_planes(n, n)) +
+           ws_round(sizeof(double) * 4 * (size_t)n);
 }
 
 cudaError_t launch_oz_gemm(int n, const double2 *E, double *BW, const double *fac, int antisym, int fill, void *work,
                            int dirs, int *err, uint32_t wait_limit, cudaStream_t st) {
+    const int rows = oz_rows(n, dirs), ld = oz_ld(n);
     char *w = static_cast<char *>(work);
     auto *pa = reinterpret_cast<__nv_bfloat16 *>(w);
-    auto *pb = reinterpret_cast<__nv_bfloat16 *>(w + ws_round(kOz * oz_plane(n)));
-    double *sa = reinterpret_cast<double *>(w + ws_round(kOz * oz_plane(n)) + ws_round(dirs * kOz * oz_plane(n)));
+    auto *pb = reinterpret_cast<__nv_bfloat16 *>(w + ws_round(oz_planes(n, rows)));
+    double *sa = reinterpret_cast<double *>(w + ws_round(oz_planes(n, rows)) + ws_round(dirs * oz_planes(n, n)));
     double *sb = sa + n;
-    const int rows = oz_rows(n), ld = oz_ld(n);
-    oz_slice_kernel<double2><<<counted(dim3(rows, 1)), 256, 0, st>>>(n, rows, ld, E, fac, pa, sa);
     CUtensorMap mA, mB;
-    if (!oz_map(&mA, pa, ld, rows, kOz, kOzBM) || !oz_map(&mB, pb, ld, rows, dirs * kOz, kOzBN))
+    if (!oz_map(&mA, pa, ld, rows, kOz, kOzBM) || !oz_map(&mB, pb, ld, n, dirs * kOz, kOzBN))
         return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzSmem);
     if (e != cudaSuccess) return e;
-    for (int d = 0; d < 3; d += dirs) {            // all at once, or one by one in a small workspace
+    // all directions and rows at once, or one direction and 128 rows in a small workspace
+    const int n_tm = (n + kOzBM - 1) / kOzBM, tms = (rows + kOzBM - 1) / kOzBM;
+    for (int d = 0; d < 3; d += dirs) {
         double *bw = BW + (size_t)d * n * n;
-        oz_slice_kernel<double><<<counted(dim3(rows, dirs)), 256, 0, st>>>(n, rows, ld, bw, fac, pb, sb);
-        oz_gemm_kernel<<<counted(dim3((n + kOzBN - 1) / kOzBN, rows / kOzBM, dirs)), kOzThreads, kOzSmem, st>>>(
-            mA, mB, n, ld / kOzBK, antisym, sa, sb, bw, err, wait_limit);
+        oz_slice_kernel<double><<<counted(dim3(n, dirs)), 256, 0, st>>>(n, 0, n, ld, bw, fac, pb, sb);
+        for (int tm = 0; tm < n_tm; tm += tms) {
+            oz_slice_kernel<double2><<<counted(dim3(rows, 1)), 256, 0, st>>>(n, tm * kOzBM, rows, ld, E, fac, pa, sa);
+            oz_gemm_kernel<<<counted(dim3((n + kOzBN - 1) / kOzBN, tms, dirs)), kOzThreads, kOzSmem, st>>>(
+                mA, mB, n, (n + kOzBK - 1) / kOzBK, tm, antisym, sa, sb, bw, err, wait_limit);
+        }
     }
     if (antisym && fill) {
         const unsigned nt = (unsigned)((n + 31) / 32);

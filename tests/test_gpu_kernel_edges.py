@@ -623,3 +623,32 @@ def test_orbit_sums_of_a_dense_mesh(k):
     assert held < 1 << 30
     g = np.asarray(g).reshape(8000, 9)[qs]
     assert _rel(g, np.asarray(ref).reshape(g.shape)) < 1e-10
+
+
+@pytest.mark.parametrize("cell", [(1, 1, 1), (3, 3, 1), (11, 1, 1), (5, 3, 3)])
+def test_generalised_velocities_workspace(k, cell):
+    """12, 108, 132 and 540 modes (whole tiles and small remainders): the smallest
+    workspace of the calls is no more than that of the product in FP64 matrices would be
+    (E, three B and three W, the blocks as given and mass-scaled)."""
+    import re
+    torch = pytest.importorskip("torch")
+    kk, ctx = k
+    s = ki.fcc_supercell_system(cell, seed=5)
+    nb, n2 = s.n_branches, len(s.fc2)
+    up = lambda *b: sum(-(-x // 256) * 256 for x in b)
+    fc2 = up(4 * (s.n_atoms + 1), 4 * n2, 72 * n2, 8 * n2, 8 * s.n_atoms, 72 * n2, 24 * n2)
+    mats = up(8 * nb * nb, 24 * nb * nb, 24 * nb * nb)
+    n_partial = min(nb, 4 * torch.cuda.get_device_properties(0).multi_processor_count)
+    nu, eig = ph.phonons(s, (1, 1, 1))
+    dev = [torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (nu.ravel(), eig.ravel(), np.full(nb, 0.1))]
+    opt = kk.Options(temperature_K=300.0, sigma_thz=0.1)
+    for call, rest in ((lambda: kk.kald_diffusivity(ctx, [s], *dev, opt, torch.zeros(nb, dtype=torch.float64).cuda()),
+                        up(8 * nb) * 2),
+                       (lambda: kk.kald_kappa_qhgk(ctx, [s], *dev, opt), up(8 * (9 * n_partial + nb), 72))):
+        ctx.set_workspace_limit(1)
+        try:
+            with pytest.raises(kk.KaldError) as e:
+                call()
+        finally:
+            ctx.set_workspace_limit(0)
+        assert int(re.search(r"needs (\d+) bytes", str(e.value)).group(1)) <= fc2 + mats + rest
