@@ -421,9 +421,10 @@ lw_main_kernel(LwParams p, LwDev d, LwTerms t, int SB, const R *__restrict__ fc3
                     // w + w' - w'' in [w + wlo - xhi, w + whi - xlo]
                     // w - w' - w'' in [w - whi - xhi, w - wlo - xlo]
                     // w - w' + w'' in [w - whi + xlo, w - wlo + xhi] (orbits)
-                    // (widened by 1e-4 of the cut so that rounding here never drops a
-                    // tile that the exact per-element test below would reach)
-                    const R cb = cut * (R)1.0001 + (kPair ? (R)1e-5 : (R)0);
+                    // (widened by 1e-4 of the cut and the rounding of sums of three
+                    // frequencies, so that no tile is dropped here that the exact
+                    // per-element test below would reach)
+                    const R cb = cut * (R)1.0001 + (kPair ? (R)1e-6 : (R)1e-14) * (w_1 + whi + xhi);
                     band = ((w_1 + wlo - xhi < cb) && (w_1 + whi - xlo > -cb)) ||
                            ((w_1 - whi - xhi < cb) && (w_1 - wlo - xlo > -cb)) ||
                            (ORBIT && (w_1 - whi + xlo < cb) && (w_1 - wlo + xhi > -cb));

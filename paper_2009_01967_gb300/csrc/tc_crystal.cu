@@ -134,9 +134,9 @@ __device__ __forceinline__ uint32_t pack_f16x2(__half lo_half, __half hi_half) {
 
 
 // w + w' and w - w' over the live rows of a warp, and whether any energy window of
-// theirs can reach a live column with a frequency in r: the epilogue skips the 16
-// columns otherwise (modes ascend in frequency, so a window covers a run of
-// columns; 40% of the chunks of the 32-atom cell on its 8^3 mesh are skipped).
+// theirs can reach a live column with a frequency in c: the epilogue skips the 8 columns
+// otherwise (modes ascend in frequency, so a window covers a run of columns).  The window
+// is widened by the roundings of the sums of three frequencies.
 struct RowRange {
     float s_lo, s_hi, d_lo, d_hi;
 };
@@ -152,7 +152,8 @@ __device__ __forceinline__ RowRange row_range(bool live, float sum, float dif) {
     return r;
 }
 template <bool THREE>
-__device__ __forceinline__ bool chunk_reached(const RowRange &r, float2 c, float wide) {
+__device__ __forceinline__ bool chunk_reached(const RowRange &r, float2 c, float cut) {
+    const float wide = cut * 1.0001f + 1e-6f * (r.s_hi + c.y);
     return (r.s_lo - c.y < wide && r.s_hi - c.x > -wide) || (r.d_lo - c.y < wide && r.d_hi - c.x > -wide) ||
            (THREE && r.d_lo + c.x < wide && r.d_hi + c.y > -wide);
 }
@@ -416,8 +417,6 @@ tcx_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__
         const int ew = warp - 4, qd = warp & 3, hf = ew >> 2;
         const int row = qd * 32 + lane;
         const float cut = x.cut, s2i = delta_param2(SHAPE, x.sig2inv);
-        // window half width of the chunk test, wider than any rounding of the exact one
-        const float wide = cut * 1.0001f + 1e-4f;
         const float2 M1 = make_float2(-1.0f, -1.0f);
         float2 cnt2 = make_float2(0.0f, 0.0f);         // window hits of this thread (exact: far below 2^24)
         auto load_row = [&](int tile, float4 &a0, float4 &a1) {
@@ -438,7 +437,7 @@ tcx_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__
             const F2 wm = live ? f2_add(F2{a0.x, a0.y}, F2{-a1.x, -a1.y}) : F2{4e30f, 0.f};
             const RowRange rr = row_range(live, wp.h, wm.h);
             const unsigned chunks =
-                __ballot_sync(0xffffffffu, lane < H / 8 && chunk_reached<EPI == EPI_SYM>(rr, wrange_sm[min(lane, 11)], wide));
+                __ballot_sync(0xffffffffu, lane < H / 8 && chunk_reached<EPI == EPI_SYM>(rr, wrange_sm[min(lane, 11)], cut));
             const float2 WPH = make_float2(wp.h, wp.h), WPL = make_float2(wp.l, wp.l);
             const float2 WMH = make_float2(wm.h, wm.h), WML = make_float2(wm.l, wm.l);
             const float2 N2H = make_float2(a1.z, a1.z), N2L = make_float2(a1.w, a1.w);

@@ -652,3 +652,25 @@ def test_generalised_velocities_workspace(k, cell):
         finally:
             ctx.set_workspace_limit(0)
         assert int(re.search(r"needs (\d+) bytes", str(e.value)).group(1)) <= fc2 + mats + rest
+
+
+@pytest.mark.parametrize("symmetry", ["all", "none"])
+@pytest.mark.parametrize("cell,mesh,precision", [(None, (2, 1, 1), "fp32"), ((1, 1, 1), (2, 1, 1), "fp32"),
+                                                 ((3, 1, 1), (1, 1, 1), "fp64"), ((2, 2, 2), (2, 1, 1), "bf16split")])
+def test_window_edges_at_high_frequencies(k, cell, mesh, precision, symmetry):
+    """Two frequencies f1 of 200 to 300 THz and f2, |2 f1 - f2| inside the window of a
+    0.004 THz delta by 1e-5 of its width, where a rounding of FP32 sums of the
+    frequencies is 1e-4 rad/ps: the coarse tests of whole tiles drop none of the triplets,
+    (f1, f1, f2) and (f2, f1, f1), that the exact test takes."""
+    kk, ctx = k
+    s = ki.fcc_supercell_system(cell, seed=7) if cell else ki.small_binary().systems[0]
+    _, eig = ph.phonons(s, mesh)
+    nb, nq = s.n_branches, int(np.prod(mesh))
+    n1 = nb // 2
+    opt = kk.Options(temperature_K=300.0, sigma_thz=0.004, precision=precision, symmetry=symmetry)
+    for x in np.random.default_rng(nb).uniform(200.0, 300.0, 24):
+        for sign in (1.0, -1.0):
+            nu = np.full((nq, nb), x)
+            nu[:, n1:] = 2.0 * x + sign * 0.012 * (1.0 - 1e-5)
+            _, count = kk.kald_linewidths(ctx, s, mesh, nu, eig, opt)
+            assert count[1] == nq * nq * 2 * n1 * n1 * (nb - n1)
