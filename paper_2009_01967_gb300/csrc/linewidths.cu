@@ -734,9 +734,11 @@ __device__ __forceinline__ int neg_point(const int *__restrict__ k, const int (&
     const int a = k[0] ? mesh[0] - k[0] : 0, b = k[1] ? mesh[1] - k[1] : 0, c = k[2] ? mesh[2] - k[2] : 0;
     return (a * mesh[1] + b) * mesh[2] + c;
 }
-// *differ |= 1 unless every q-point has the frequencies of -q, to 4e-13 of its largest
-// (two diagonalisations of D(q) and of its conjugate agree to some 1e-14; the sums of
-// -q are then those of q to 1e-10).
+// *differ |= 1 unless every q-point has the frequencies w of -q, to 4e-13 of its largest
+// (two diagonalisations of D(q) and of its conjugate agree to some 1e-14), 5e-12 sigma
+// and 1e-11 w.  The sums of -q are then those of q to 1e-10: three frequencies change a
+// Gaussian weight inside n_sigma sigma by 3 n_sigma / sigma times their difference (5e-11
+// at 3 sigma) and an occupation of n >> 1 by a part in 1e11.
 template <typename M>
 __global__ void __launch_bounds__(128)
 mirror_check_kernel(LwParams p, const int *__restrict__ qfrac, const M *__restrict__ modes, int *__restrict__ differ) {
@@ -758,7 +760,10 @@ mirror_check_kernel(LwParams p, const int *__restrict__ qfrac, const M *__restri
     __syncthreads();
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) mx = fmax(mx, top[w]);
     bool d = false;
-    for (int x = threadIdx.x; x < p.nb; x += blockDim.x) d |= !(fabs(freq(q, x) - freq(m, x)) <= 4e-13 * mx);
+    for (int x = threadIdx.x; x < p.nb; x += blockDim.x) {
+        const double w = freq(q, x);
+        d |= !(fabs(w - freq(m, x)) <= fmin(fmin(4e-13 * mx, 5e-12 * p.sigma_w), 1e-11 * w));
+    }
     if (__syncthreads_or(d) && threadIdx.x == 0) atomicOr(differ, 1);
 }
 

@@ -674,3 +674,34 @@ def test_window_edges_at_high_frequencies(k, cell, mesh, precision, symmetry):
             nu[:, n1:] = 2.0 * x + sign * 0.012 * (1.0 - 1e-5)
             _, count = kk.kald_linewidths(ctx, s, mesh, nu, eig, opt)
             assert count[1] == nq * nq * 2 * n1 * n1 * (nb - n1)
+
+
+@pytest.mark.parametrize("top,sigma,change", [(50.0, 0.05, 3e-13), (20.0, 0.01, 3e-13), (50.0, 0.05, 4e-15), (2.0, 20.0, 3e-13)])
+def test_phase_space_mirrored_within_the_window(k, top, sigma, change):
+    """Spectra much wider than the delta, and a delta wider than the spectrum: frequencies
+    of -q that differ from those of q by `change` of the largest change no sum by more
+    than 1e-10, whether those of q are taken for both or not (the smallest workspace sums
+    every q-point by itself)."""
+    import re
+    kk, ctx = k
+    mesh, nb = (4, 3, 2), 6
+    s = ki.small_binary(mesh=mesh).systems[0]
+    nq = int(np.prod(mesh))
+    rng = np.random.default_rng(5)
+    nu = np.sort(rng.uniform(0.02, top, (nq, nb)), axis=1)
+    nu[:, 0], nu[:, -1] = 0.011, top
+    neg = np.array([np.ravel_multi_index(tuple((-np.array(np.unravel_index(q, mesh))) % mesh), mesh) for q in range(nq)])
+    # triplets at every place of the window: the middle modes of every q near half of the top
+    nu[:, 2:5] = 0.5 * top + sigma * rng.uniform(-1.0, 1.0, (nq, 3))
+    nu = np.where((neg < np.arange(nq))[:, None], nu[neg] + change * top * rng.choice([-1.0, 1.0], (nq, nb)), nu)
+    opt = kk.Options(temperature_K=300.0, sigma_thz=sigma, precision="fp64")
+    g = kk.kald_phase_space(ctx, s, mesh, nu, opt)
+    ctx.set_workspace_limit(1)
+    try:
+        with pytest.raises(kk.KaldError) as e:
+            kk.kald_phase_space(ctx, s, mesh, nu, opt)
+        ctx.set_workspace_limit(int(re.search(r"needs (\d+) bytes", str(e.value)).group(1)))
+        ref = kk.kald_phase_space(ctx, s, mesh, nu, opt)
+    finally:
+        ctx.set_workspace_limit(0)
+    assert np.max(np.abs(g - ref)) <= 1e-10 * np.max(np.abs(ref))
