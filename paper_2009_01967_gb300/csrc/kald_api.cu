@@ -620,6 +620,18 @@ kald_status plan_system_cached(kald_ctx *ctx, const kald_system *s, std::shared_
     return st;
 }
 
+// Plans of systems[which[from]] .. , up to 64 of them, into hps (by system).
+static kald_status plan_some(kald_ctx *ctx, const kald_system *systems, const std::vector<int> &which, size_t from,
+                             std::vector<std::shared_ptr<const HostSystem>> &hps) {
+    const size_t n = std::min<size_t>(64, which.size() - from);
+    std::vector<kald_system> s(n);
+    for (size_t k = 0; k < n; ++k) s[k] = systems[which[from + k]];
+    std::vector<std::shared_ptr<const HostSystem>> out;
+    const kald_status st = plan_systems_cached(ctx, (int)n, s.data(), out);
+    for (size_t k = 0; !st && k < n; ++k) hps[which[from + k]] = out[k];
+    return st;
+}
+
 std::atomic<unsigned long long> g_launches{0};
 
 }  // namespace kald
@@ -703,16 +715,10 @@ kald_status kald_profile_read(kald_ctx *ctx, int kernel, double *total_ms, uint6
     return KALD_OK;
 }
 
-kald_status kald_phonons(kald_ctx *ctx, const kald_system *sys, const int32_t mesh[3],
-                         double *nu_thz, double *eigvec, double *vel) {
-    if (!ctx) return KALD_E_INVALID;
-    kald_status st = set_device(ctx);
-    if (st) return st;
-    if ((st = check_mesh(ctx, mesh))) return st;
-    if (!nu_thz || !eigvec) return fail(ctx, KALD_E_INVALID, "nu_thz/eigvec NULL");
-    std::shared_ptr<const HostSystem> hp;
-    if ((st = plan_system_cached(ctx, sys, hp))) return st;
-    const HostSystem &h = *hp;
+// Phonons of a planned system (kald_phonons).
+static kald_status phonons_impl(kald_ctx *ctx, const HostSystem &h, const int32_t mesh[3], double *nu_thz,
+                                double *eigvec, double *vel) {
+    kald_status st;
     const int nb = h.nb;
     const bool large = nb > kMaxNbSmall;
     if (large && (mesh[0] != 1 || mesh[1] != 1 || mesh[2] != 1))
@@ -852,6 +858,18 @@ kald_status kald_phonons(kald_ctx *ctx, const kald_system *sys, const int32_t me
     return KALD_OK;
 }
 
+kald_status kald_phonons(kald_ctx *ctx, const kald_system *sys, const int32_t mesh[3],
+                         double *nu_thz, double *eigvec, double *vel) {
+    if (!ctx) return KALD_E_INVALID;
+    kald_status st = set_device(ctx);
+    if (st) return st;
+    if ((st = check_mesh(ctx, mesh))) return st;
+    if (!nu_thz || !eigvec) return fail(ctx, KALD_E_INVALID, "nu_thz/eigvec NULL");
+    std::shared_ptr<const HostSystem> hp;
+    if ((st = plan_system_cached(ctx, sys, hp))) return st;
+    return phonons_impl(ctx, *hp, mesh, nu_thz, eigvec, vel);
+}
+
 kald_status kald_phonons_batch(kald_ctx *ctx, int32_t n_sys, const kald_system *sys, double *nu_thz,
                                double *eigvec) {
     if (!ctx) return KALD_E_INVALID;
@@ -860,32 +878,34 @@ kald_status kald_phonons_batch(kald_ctx *ctx, int32_t n_sys, const kald_system *
     if (n_sys <= 0 || !sys) return fail(ctx, KALD_E_INVALID, "n_sys must be > 0");
     if (!nu_thz || !eigvec) return fail(ctx, KALD_E_INVALID, "nu_thz/eigvec NULL");
     const int32_t gamma_mesh[3] = {1, 1, 1};
-    std::vector<std::shared_ptr<const HostSystem>> hp;
+    std::vector<std::shared_ptr<const HostSystem>> hp(n_sys);
     std::vector<size_t> off_nb(n_sys), off_eig(n_sys);
     size_t on = 0, oe = 0;
-    std::vector<int> large;
-    if ((st = plan_systems_cached(ctx, n_sys, sys, hp))) return st;
+    std::vector<int> large, small;
     for (int x = 0; x < n_sys; ++x) {
-        const int nb = hp[x]->nb;
+        if (sys[x].n_atoms <= 0) return fail(ctx, KALD_E_INVALID, "n_atoms must be > 0");
+        const int nb = 3 * sys[x].n_atoms;
         off_nb[x] = on;
         off_eig[x] = oe;
         on += nb;
         oe += (size_t)nb * nb;
-        if (nb > kMaxNbSmall) {
-            if (!eigh_large_supported(nb, ctx->smem_optin))
-                return fail(ctx, KALD_E_UNSUPPORTED, "kald_phonons_batch: cell too large for the Gamma-only eigensolver");
-            large.push_back(x);
-        }
+        if (nb > kMaxNbSmall && !eigh_large_supported(nb, ctx->smem_optin))
+            return fail(ctx, KALD_E_UNSUPPORTED, "kald_phonons_batch: cell too large for the Gamma-only eigensolver");
+        (nb > kMaxNbSmall ? large : small).push_back(x);
     }
     const bool d_nu = is_device_ptr(nu_thz), d_eig = is_device_ptr(eigvec);
-    // cells of nb <= 96: the per-q path, one call each
-    for (int x = 0; x < n_sys; ++x)
-        if (hp[x]->nb <= kMaxNbSmall &&
-            (st = kald_phonons(ctx, &sys[x], gamma_mesh, nu_thz + off_nb[x], eigvec + 2 * off_eig[x], nullptr)))
+    // cells of nb <= 96: the per-q path, one call each (planned 64 at a time, as the
+    // others are: planning them all first and again one by one went past the plans kept)
+    for (size_t c = 0; c < small.size(); ++c) {
+        const int x = small[c];
+        if (c % 64 == 0 && (st = plan_some(ctx, sys, small, c, hp))) return st;
+        if ((st = phonons_impl(ctx, *hp[x], gamma_mesh, nu_thz + off_nb[x], eigvec + 2 * off_eig[x], nullptr)))
             return st;
-    if (large.empty()) return KALD_OK;
+        hp[x] = nullptr;
+    }
     for (size_t c = 0; c < large.size(); c += 64) {
         const size_t c1 = std::min(large.size(), c + 64);
+        if ((st = plan_some(ctx, sys, large, c, hp))) return st;
         const std::vector<double> q0(3, 0.0);
         size_t need = eigh_batch_records_bytes((int)(c1 - c));
         for (size_t t = c; t < c1; ++t) {
@@ -937,6 +957,7 @@ kald_status kald_phonons_batch(kald_ctx *ctx, int32_t n_sys, const kald_system *
                                 cudaMemcpyDeviceToHost, ctx->stream);
         }
         if ((st = finish(ctx, "kald_phonons_batch"))) return st;
+        for (size_t t = c; t < c1; ++t) hp[large[t]] = nullptr;
     }
     return KALD_OK;
 }
@@ -1396,25 +1417,32 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
     const bool d_nu = is_device_ptr(nu_thz), d_eig = is_device_ptr(eigvec), d_g = is_device_ptr(gamma);
     const int fp32 = opt->precision == KALD_FP32;
     uint64_t tot = 0, allowed_tot = 0;
-    std::vector<std::shared_ptr<const HostSystem>> hps;   // one q-point: all at once; else one by one
+    std::vector<std::shared_ptr<const HostSystem>> hps(n_sys);
+    std::vector<int> cells;                              // those of nb <= 96 of a Gamma-only call
     if (nq_mesh == 1) {
         // every Gamma-only supercell (nb > 96) of the call in one launch sequence
-        // (64 at a time; the plans of small cells are made again one by one below)
-        std::vector<std::shared_ptr<const HostSystem>> some;
-        for (int x0 = 0; x0 < n_sys; x0 += 64) {
-            if ((st = plan_systems_cached(ctx, std::min(64, n_sys - x0), sys + x0, some))) return st;
-            for (auto &p : some) hps.push_back(p->nb > kMaxNbSmall || n_sys <= 64 ? p : nullptr);
+        std::vector<int> large;
+        for (int x = 0; x < n_sys; ++x) {
+            if (sys[x].n_atoms <= 0) return fail(ctx, KALD_E_INVALID, "n_atoms must be > 0");
+            (3 * sys[x].n_atoms > kMaxNbSmall ? large : cells).push_back(x);
         }
+        for (size_t c = 0; c < large.size(); c += 64)
+            if ((st = plan_some(ctx, sys, large, c, hps))) return st;
         if ((st = gamma_only_batch(ctx, n_sys, sys, hps, nu_thz, eigvec, opt, gamma, d_nu, d_eig, d_g, tot,
                                    allowed_tot)))
             return st;
     }
+    size_t n_cells = 0;                                  // cells planned so far, 64 at a time
     size_t off_nb = 0, off_eig = 0;
     int lean = 0;            // where the workspace cannot be had: 1 without tables, 2 without orbits as well
     for (int x = 0; x < n_sys; ++x) {
-        std::shared_ptr<const HostSystem> hp;
-        if (nq_mesh == 1 && hps[x]) hp = hps[x];
-        else if ((st = plan_system_cached(ctx, &sys[x], hp))) return st;
+        if (!hps[x] && nq_mesh != 1) {
+            if ((st = plan_system_cached(ctx, &sys[x], hps[x]))) return st;
+        } else if (!hps[x]) {
+            if ((st = plan_some(ctx, sys, cells, n_cells, hps))) return st;
+            n_cells += 64;
+        }
+        const std::shared_ptr<const HostSystem> hp = hps[x];
         const HostSystem &h = *hp;
         const int nb = h.nb;
         if (nb > kMaxNbSmall && nq_mesh != 1)
@@ -1686,6 +1714,7 @@ static kald_status linewidths_impl(kald_ctx *ctx, int32_t n_sys, const kald_syst
             continue;
         }
         lean = 0;
+        hps[x] = nullptr;                                // (hp holds the plan to the end of this pass)
         LwDev d;
         d.blkinfo = upload(ctx, binfo);
         // Phi3 / sqrt(mi mj mk), 28 values per block (16-byte loads), in the working precision

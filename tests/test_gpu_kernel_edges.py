@@ -705,3 +705,25 @@ def test_phase_space_mirrored_within_the_window(k, top, sigma, change):
     finally:
         ctx.set_workspace_limit(0)
     assert np.max(np.abs(g - ref)) <= 1e-10 * np.max(np.abs(ref))
+
+
+def test_phonons_of_more_systems_than_are_planned_at_once(k):
+    """70 Gamma-only systems, all different, large ones among small ones at both ends of
+    the 64 that are planned together: the phonons of each alone, bit for bit."""
+    from dataclasses import replace
+    kk, ctx = k
+    base, big = ki.fcc_supercell_system((1, 1, 1), seed=3), ki.fcc_supercell_system((3, 3, 1), seed=9)
+    systems = [replace(big if x in (0, 31, 64, 69) else base, masses=(big if x in (0, 31, 64, 69) else base).masses + 0.01 * x)
+               for x in range(70)]
+    nu, eig = kk.kald_phonons_batch(ctx, systems)
+    o = e = 0
+    for s in systems:
+        nb = s.n_branches
+        nu1, eig1, _ = kk.kald_phonons(ctx, s, (1, 1, 1), want_vel=False)
+        np.testing.assert_array_equal(np.asarray(nu).ravel()[o:o + nb], nu1.ravel())
+        np.testing.assert_array_equal(np.asarray(eig).ravel()[e:e + nb * nb], eig1.ravel())
+        o += nb
+        e += nb * nb
+    bad = replace(base, masses=-base.masses)
+    with pytest.raises(kk.KaldError, match="masses"):
+        kk.kald_phonons_batch(ctx, systems[:66] + [bad])
