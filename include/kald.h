@@ -76,8 +76,8 @@ typedef enum {
  *    conjugate of that of (q, q', q'') and w(-q) = w(q); one q-point of each
  *    pair {q, -q} is projected and the other takes its averaged linewidths.
  *  - Permutation (Eq. gamma_operators with Phi3 symmetric under permutations
- *    of its three indices, checked on the host to 1e-12 of max |Phi3|; a Phi3
- *    that lists some block indices more than once -- such blocks are added --
+ *    of its three indices, checked on the host to 1e-12 of the largest |Phi3|
+ *    of the block's atoms, the smallest of the three; a Phi3 that lists some block indices more than once -- such blocks are added --
  *    is taken as not symmetric): the
  *    squared projection |phi|^2 of a momentum triple (q1, q2, q3),
  *    q1 + q2 + q3 = 0 modulo G, is the same for every order of the triple, so

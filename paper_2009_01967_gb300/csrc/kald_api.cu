@@ -1008,11 +1008,17 @@ void fc3_symmetries(const kald_system *s, const HostSystem &h) {
         h.fc3_symmetric = h.fc3_perm_symmetric = 0;
         return;
     }
-    // entries agree to 1e-12 of the largest |Phi3| (the self blocks (i; i; i) are sums
-    // that cancel to rounding noise, so no per-entry relative test)
-    double tol = 0.0;
-    for (size_t v = 0; v < 27 * (size_t)s->n_fc3; ++v) tol = std::max(tol, std::fabs(s->fc3[v]));
-    tol *= 1e-12;
+    // entries agree to 1e-12 of the largest |Phi3| of the atoms' blocks, the atom's of the
+    // block that has the smallest (the self blocks (i; i; i) are sums that cancel to
+    // rounding noise, so no per-entry relative test; and a weakly anharmonic part of a
+    // cell is not measured by the rest of it)
+    std::vector<double> top(s->n_atoms, 0.0);
+    for (int b = 0; b < s->n_fc3; ++b) {
+        const int32_t *x = s->fc3_idx + 9 * (size_t)b;
+        double m = 0.0;
+        for (int v = 0; v < 27; ++v) m = std::max(m, std::fabs(s->fc3[27 * (size_t)b + v]));
+        for (int a : {x[0], x[1], x[5]}) top[a] = std::max(top[a], m);
+    }
     auto partners = [&](auto &&key, auto &&at) {
         for (int b = 0; b < s->n_fc3; ++b) {
             int32_t k[9];
@@ -1020,6 +1026,8 @@ void fc3_symmetries(const kald_system *s, const HostSystem &h) {
             const int o = idx.find(k);
             if (o < 0) return false;
             const double *f = s->fc3 + 27 * (size_t)b, *g = s->fc3 + 27 * (size_t)o;
+            const int32_t *x = s->fc3_idx + 9 * (size_t)b;
+            const double tol = 1e-12 * std::min({top[x[0]], top[x[1]], top[x[5]]});
             for (int a = 0; a < 3; ++a)
                 for (int c = 0; c < 3; ++c)
                     for (int d = 0; d < 3; ++d)
@@ -1043,11 +1051,15 @@ void fc3_symmetries(const kald_system *s, const HostSystem &h) {
     h.fc3_perm_symmetric = first ? 1 : 0;
 }
 // True when every fc2 block (i; j R) has the partner (j; i -R) with the
-// Cartesian indices exchanged, to 1e-12 of the largest |Phi2|.
+// Cartesian indices exchanged, to 1e-12 of the largest |Phi2| of the blocks of i or of
+// j, whichever is less.
 bool fc2_symmetric(const kald_system *s) {
-    double tol = 0.0;
-    for (size_t v = 0; v < 9 * (size_t)s->n_fc2; ++v) tol = std::max(tol, std::fabs(s->fc2[v]));
-    tol *= 1e-12;
+    std::vector<double> top(s->n_atoms, 0.0);
+    for (int b = 0; b < s->n_fc2; ++b) {
+        double m = 0.0;
+        for (int v = 0; v < 9; ++v) m = std::max(m, std::fabs(s->fc2[9 * (size_t)b + v]));
+        for (int a : {s->fc2_idx[5 * (size_t)b], s->fc2_idx[5 * (size_t)b + 1]}) top[a] = std::max(top[a], m);
+    }
     // blocks ordered by (i, j, R); the partner's key is looked up by bisection
     std::vector<int> o(s->n_fc2);
     std::iota(o.begin(), o.end(), 0);
@@ -1062,6 +1074,7 @@ bool fc2_symmetric(const kald_system *s) {
         auto it = std::lower_bound(o.begin(), o.end(), k, [&](int a, const int32_t *key) { return less(row(a), key); });
         if (it == o.end() || less(k, row(*it))) return false;
         const double *f = s->fc2 + 9 * (size_t)b, *g = s->fc2 + 9 * (size_t)*it;
+        const double tol = 1e-12 * std::min(top[x[0]], top[x[1]]);
         for (int a = 0; a < 3; ++a)
             for (int c = 0; c < 3; ++c)
                 if (!(std::fabs(f[3 * a + c] - g[3 * c + a]) <= tol)) return false;

@@ -727,3 +727,40 @@ def test_phonons_of_more_systems_than_are_planned_at_once(k):
     bad = replace(base, masses=-base.masses)
     with pytest.raises(kk.KaldError, match="masses"):
         kk.kald_phonons_batch(ctx, systems[:66] + [bad])
+
+
+def test_symmetry_of_a_weak_part(k):
+    """A part of a cell whose force constants are 2^-30 (Phi3) and 2^-24 (Phi2) of the
+    other's and lack the symmetry by 1e-4 and 1e-5 of themselves, less than 1e-12 of the
+    largest: neither is taken as symmetric, and the part's linewidths and generalised
+    velocities are those of its own force constants (1e-10 of the part's largest)."""
+    from dataclasses import replace
+    from oracle import conductivity as co
+    kk, ctx = k
+    rng = np.random.default_rng(3)
+    s, _, _, _ = _two_parts((1, 1, 1), 2.0 ** -30, False)
+    n = s.n_atoms // 2
+    weak = s.fc3_idx[:, 0] >= n
+    s = replace(s, fc3=np.where(weak[:, None, None, None], s.fc3 * (1.0 + 1e-4 * rng.standard_normal(s.fc3.shape)), s.fc3))
+    mesh = (2, 2, 1)
+    nu, eig = ph.phonons(s, mesh)
+    of_weak = (np.abs(eig[:, :, 3 * n:]) ** 2).sum(-1).ravel() > 0.5
+    g = [np.asarray(kk.kald_linewidths(ctx, s, mesh, nu, eig, kk.Options(temperature_K=300.0, sigma_thz=0.1, precision="fp64",
+                                                                         symmetry=sym))[0]).ravel()
+         for sym in ("all", "none")]
+    for part in (of_weak, ~of_weak):
+        assert _rel(g[0][part], g[1][part]) < 1e-10
+
+    s, _, _, _ = _two_parts((2, 2, 1), 1.0, False)
+    n = s.n_atoms // 2
+    weak = (s.fc2_idx[:, 0] >= n)[:, None, None]
+    s = replace(s, fc2=np.where(weak, 2.0 ** -24 * s.fc2 * (1.0 + 1e-5 * rng.standard_normal(s.fc2.shape)), s.fc2))
+    # any orthonormal modes, each on one part
+    E = np.zeros((6 * n, 6 * n))
+    E[:3 * n, :3 * n], E[3 * n:, 3 * n:] = (np.linalg.qr(rng.standard_normal((3 * n, 3 * n)))[0] for _ in range(2))
+    eig = E.astype(complex)[None]
+    nu = np.sort(rng.uniform(0.1, 2.0, (1, 6 * n)))
+    W_o = co.generalized_velocity(s, nu, eig)[:, 3 * n:, 3 * n:]
+    _, W = kk.kald_kappa_qhgk(ctx, [s], nu.ravel(), eig.ravel(), np.full(6 * n, 0.1),
+                              kk.Options(temperature_K=300.0, sigma_thz=0.1), want_vgen=True)
+    np.testing.assert_allclose(W[:, 3 * n:, 3 * n:], W_o, rtol=0, atol=1e-10 * np.abs(W_o).max())
