@@ -343,11 +343,10 @@ def roofline_of(args, w, nbs, nu_c, opt, prof, steps, allowed, pairs_step=None):
             kernel = "tcx_gemm_kernel (GEMM1 T' = eps'^T Y_s, GEMM2 phi = T' conj(eps'') + delta epilogue)"
             H = -(-nb // 32) * 32
             mt = -(-(nb * nb) // 128)
-            n_mma = 5 if H <= 64 else 3
             alg = nq * nq * 2 * 8.0 * nb ** 4              # two complex nb^4 contractions per pair
-            exe = nq * nq * 2.0 * mt * n_mma * 2.0 * 128 * (2 * H) * (2 * H)
+            exe = nq * nq * 2.0 * mt * 3 * 2.0 * 128 * (2 * H) * (2 * H)
             alg_note = ("two dense complex contractions of nb^4 per momentum-conserving pair (8 flop per "
-                        "complex MAC); executed: 3 BF16 MMAs per product (5 when nb <= 64)")
+                        "complex MAC); executed: 3 BF16 MMAs per product")
         peak = float(peaks.get("bf16_tflops_sustained", 1700.0))
         bound, peak_note = "tensor", ("MEASURED_PEAKS.json bf16_tflops_sustained (cuBLAS bf16 in a power-capped "
                                       "loop; the kernels run inside a seconds-long step), of measured")

@@ -47,13 +47,6 @@ template <> struct Cx<double> { using T = double2; };
 
 constexpr int kSnThreads = 256;
 
-template <typename R2>
-__device__ __forceinline__ R2 cmul(R2 a, R2 b) {
-    R2 r;
-    r.x = a.x * b.x - a.y * b.y;
-    r.y = a.x * b.y + a.y * b.x;
-    return r;
-}
 // FP64: scalar FMAs; FP32: packed FP32x2 FMAs (two lanes of the complex
 // value per instruction).
 __device__ __forceinline__ void cfma(double2 &acc, double2 a, double2 b) {      // acc += a b

@@ -5,9 +5,8 @@
 // The two dense complex contractions of every (pair, mode s),
 //   T'(s', c)       = sum_b eps'(b, s') Y_s(b, c)
 //   phi(s, s', s'') = sum_c T'(s', c) conj(eps''(c, s'')),
-// run as real GEMMs on BF16 pieces with FP32 accumulation in tensor memory:
-// the data operand (Y, T') as hi + lo, the eigenvector operand as hi + lo
-// (three MMAs per product) or, for nb <= 64, hi + mid + lo (five MMAs).
+// run as real GEMMs on BF16 hi + lo pieces of both operands (three MMAs per
+// product) with FP32 accumulation in tensor memory.
 // With H = nb rounded up to 32, K' = 2H (k' < H: real part of index b or c,
 // k' >= H: imaginary part) and the row count M = nb^2 padded to a multiple
 // of 128:
@@ -54,18 +53,17 @@ using namespace tc;
 constexpr int kBM = 128, kBK = 64, kAK = 32, kStages = 4;
 enum : int { EPI_T = 0, EPI_PHI = 1, EPI_SYM = 2 };
 
-// BN = N = K' = 2H (64, 128 or 192; crystals have nb <= 96); PB = BF16
-// pieces of the eigenvector operand B (3 where the resident copy fits in
-// shared memory, else 2).
-template <int BN, int PB> struct Cfg {
-    static constexpr int kNkb = BN / kBK;                  // K blocks of B
-    static constexpr int kNks = BN / kAK;                  // A stages per tile
+// kBN = N = K' = 2H (65 to 96 branches, H = 96).
+constexpr int kBN = 192;
+struct Cfg {
+    static constexpr int kNkb = kBN / kBK;                 // K blocks of B
+    static constexpr int kNks = kBN / kAK;                 // A stages per tile
     static constexpr int kABytes = kBM * kAK * 2;          // one A plane per stage (two 64-row halves)
-    static constexpr int kBBlk = BN * kBK * 2;             // one B plane of one K block
-    static constexpr int kBBytes = kNkb * PB * kBBlk;      // resident B, all pieces
+    static constexpr int kBBlk = kBN * kBK * 2;            // one B plane of one K block
+    static constexpr int kBBytes = kNkb * 2 * kBBlk;       // resident B, hi and lo
     static constexpr int kStageBytes = 2 * kABytes;
     static constexpr int kSmem = kBBytes + kStages * kStageBytes + 1024;
-    static constexpr int kTmemCols = 2 * BN <= 128 ? 128 : 2 * BN <= 256 ? 256 : 512;   // two accumulators
+    static constexpr int kTmemCols = 512;                  // two accumulators
 };
 
 struct XParams {
@@ -79,7 +77,6 @@ struct XParams {
     __nv_bfloat16 *t1h, *t1l; // GEMM1 output [pairs][Kp][Mp]
     const float4 *wn;         // [nq][nb] FP32 pairs (w hi, w lo, n hi, n lo); w = 0 when masked
     float sig2inv, cut;       // delta-shape parameter (delta_param), window half width
-    int shape;                // energy-delta shape
     int n_slices;             // q-slices of slots (a batch spans fewer q values)
     float *slots;             // GEMM2 output [n_slices][nq (q')][nb][2]: per-mode sums over the
                               // mode's rows in its first tile (0) and in the next tile (1)
@@ -177,16 +174,16 @@ template <int EPI> struct Warps {
     static constexpr int kThreads = 32 * (4 + kEpi);
 };
 
-template <int EPI, int BN, int PB, int SHAPE>
+template <int EPI, int SHAPE>
 __global__ void __launch_bounds__(Warps<EPI>::kThreads, 1)
 tcx_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ CUtensorMap mAl,
-                const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CUtensorMap mBm,
-                const __grid_constant__ CUtensorMap mBl, XParams x, int tpc, int *err) {
-    using C = Cfg<BN, PB>;
+                const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CUtensorMap mBl, XParams x, int tpc,
+                int *err) {
+    using C = Cfg;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *base = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    unsigned char *sB = base;                      // [kb][piece][BN rows x 128 B]
+    unsigned char *sB = base;                      // [kb][hi, lo][kBN rows x 128 B]
     unsigned char *sA = base + C::kBBytes;         // [stage][hi, lo][two 64-row atoms]
     __shared__ __align__(8) uint64_t bfull, afull[kStages], aempty[kStages], tfull[2], tempty[2], drain;
     __shared__ __align__(8) uint64_t rfull[2], rfree[2];       // the sums of a tile parity: written, reduced
@@ -211,7 +208,7 @@ tcx_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__
     const int n_tiles = max(0, t1 - t0);
     const int nb = x.nb, H = x.H;
     constexpr int nkb = C::kNkb, nks = C::kNks;
-    constexpr uint32_t idesc = idesc_bf16(BN) | (1u << 15);     // A MN-major
+    constexpr uint32_t idesc = idesc_bf16(kBN) | (1u << 15);     // A MN-major
     int q, qp, qpp;
     pair_of(x, a, q, qp, qpp);
     const int bz = (EPI == EPI_T) ? qp : qpp;
@@ -275,9 +272,8 @@ tcx_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__
         if (lane == 0) {
             mbar_expect_tx(&bfull, C::kBBytes);
             for (int kb = 0; kb < nkb; ++kb) {
-                tma_load_3d(sB + (PB * kb) * C::kBBlk, &mBh, &bfull, kb * kBK, 0, bz);
-                if (PB == 3) tma_load_3d(sB + (PB * kb + 1) * C::kBBlk, &mBm, &bfull, kb * kBK, 0, bz);
-                tma_load_3d(sB + (PB * kb + PB - 1) * C::kBBlk, &mBl, &bfull, kb * kBK, 0, bz);
+                tma_load_3d(sB + 2 * kb * C::kBBlk, &mBh, &bfull, kb * kBK, 0, bz);
+                tma_load_3d(sB + (2 * kb + 1) * C::kBBlk, &mBl, &bfull, kb * kBK, 0, bz);
             }
             int it = 0;
             for (int tile = t0; tile < t1; ++tile) {
@@ -316,20 +312,14 @@ tcx_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__
                     unsigned char *st = sA + (size_t)s * C::kStageBytes;
                     const int kb = ks * kAK / kBK, k0 = (ks * kAK % kBK) / 16;   // B block, K16 step in it
                     const uint64_t ah = smem_desc_mn(st), al = smem_desc_mn(st + C::kABytes);
-                    const uint64_t bh = smem_desc(sB + (PB * kb) * C::kBBlk);
-                    const uint64_t bm = smem_desc(sB + (PB * kb + 1) * C::kBBlk);
-                    const uint64_t bl = smem_desc(sB + (PB * kb + PB - 1) * C::kBBlk);
+                    const uint64_t bh = smem_desc(sB + 2 * kb * C::kBBlk), bl = smem_desc(sB + (2 * kb + 1) * C::kBBlk);
 #pragma unroll
                     for (int k = 0; k < kAK / 16; ++k) {
                         const uint64_t da = (uint64_t)((k * 2048) >> 4), db = (uint64_t)(((k0 + k) * 32) >> 4);
-                        // a b = (ah + al)(bh [+ bm] + bl) without the smallest terms
+                        // a b = (ah + al)(bh + bl) without the smallest term
                         mma_bf16(d, ah + da, bh + db, idesc, (ks > 0 || k > 0) ? 1u : 0u);
                         mma_bf16(d, ah + da, bl + db, idesc, 1u);
                         mma_bf16(d, al + da, bh + db, idesc, 1u);
-                        if (PB == 3) {
-                            mma_bf16(d, ah + da, bm + db, idesc, 1u);
-                            mma_bf16(d, al + da, bm + db, idesc, 1u);
-                        }
                     }
                     mma_commit(&aempty[s]);
                 }
@@ -356,7 +346,7 @@ tcx_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__
             // nb a multiple of 32 (so H = nb and nb^2 = Mp): every warp's 32 rows
             // are valid and share c, with consecutive s
             const bool pairs = (nb % 32) == 0 && H == nb && x.Mp == nb * nb;
-            for (int ci = hf; ok && ci < BN / 32; ci += NG) {
+            for (int ci = hf; ok && ci < kBN / 32; ci += NG) {
                 const int c0 = ci * 32;
                 float v[32];
                 tmem_ld32(taddr + c0, v);
@@ -839,14 +829,14 @@ static size_t gather_smem(int nb) {
 // barriers whether or not a wait failed.
 constexpr int kYGroups = 14, kYThreads = 512, kYBuilders = 192, kYStages = 2;
 
-template <int BN, int PB> struct CfgY {
-    static constexpr int kNkb = BN / kBK;                  // K blocks (K = BN = 2H)
+struct CfgY {
+    static constexpr int kNkb = kBN / kBK;                 // K blocks (K = kBN = 2H)
     static constexpr int kAPlane = kBM * kBK * 2;          // one piece of one stage (16 KB)
     static constexpr int kStageBytes = 2 * kAPlane;        // hi + lo
-    static constexpr int kBBytes = Cfg<BN, PB>::kBBytes;
-    static constexpr int kBBlk = Cfg<BN, PB>::kBBlk;
+    static constexpr int kBBytes = Cfg::kBBytes;
+    static constexpr int kBBlk = Cfg::kBBlk;
     static constexpr int kFixed = kBBytes + kYStages * kStageBytes + 1024;
-    static constexpr int kTmemCols = Cfg<BN, PB>::kTmemCols;
+    static constexpr int kTmemCols = Cfg::kTmemCols;
 };
 // dynamic shared memory of tcx_y_kernel: fixed part + chi of q', q'' + the
 // tile's (group, i) block table
@@ -854,17 +844,15 @@ __host__ __device__ inline size_t tcx_y_smem(int fixed, int n_rep, int n_at) {
     return (size_t)fixed + sizeof(float2) * 2 * (size_t)n_rep + sizeof(int) * (size_t)kYGroups * (n_at + 1);
 }
 
-template <int BN, int PB>
 __global__ void __launch_bounds__(kYThreads, 1)
-tcx_y_kernel(const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CUtensorMap mBm,
-             const __grid_constant__ CUtensorMap mBl, XParams x, TcxYTables yt, const float2 *__restrict__ chi_all,
-             int n_rep, const float *__restrict__ wscale, __nv_bfloat16 *__restrict__ a1h,
-             __nv_bfloat16 *__restrict__ a1l, int tpc, int *err) {
-    using C = CfgY<BN, PB>;
+tcx_y_kernel(const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CUtensorMap mBl, XParams x, TcxYTables yt,
+             const float2 *__restrict__ chi_all, int n_rep, const float *__restrict__ wscale,
+             __nv_bfloat16 *__restrict__ a1h, __nv_bfloat16 *__restrict__ a1l, int tpc, int *err) {
+    using C = CfgY;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *base = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    unsigned char *sB = base;                              // [kb][piece][BN rows x 128 B]
+    unsigned char *sB = base;                              // [kb][hi, lo][kBN rows x 128 B]
     unsigned char *sA = base + C::kBBytes;                 // [stage][hi, lo][128 rows x 128 B]
     float2 *chi_sm = reinterpret_cast<float2 *>(sA + kYStages * C::kStageBytes);   // chi(q', .), chi(q'', .)
     int *gi_sm = reinterpret_cast<int *>(chi_sm + 2 * n_rep);                     // [kYGroups][n_at + 1]
@@ -879,7 +867,7 @@ tcx_y_kernel(const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CU
     const int n_tiles = max(0, t1 - t0);
     const int nb = x.nb, H = x.H, n_at = yt.n_at, ld = n_at + 1;
     constexpr int nkb = C::kNkb;
-    constexpr uint32_t idesc = idesc_f16(BN);              // FP16 operands, both K-major
+    constexpr uint32_t idesc = idesc_f16(kBN);              // FP16 operands, both K-major
     int q, qp, qpp;
     pair_of(x, a, q, qp, qpp);
     const bool builder = warp == 2 || warp == 3 || warp >= 12;
@@ -917,9 +905,8 @@ tcx_y_kernel(const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CU
         if (lane == 0 && n_tiles > 0) {
             mbar_expect_tx(&bfull, C::kBBytes);
             for (int kb = 0; kb < nkb; ++kb) {
-                tma_load_3d(sB + (PB * kb) * C::kBBlk, &mBh, &bfull, kb * kBK, 0, q);
-                if (PB == 3) tma_load_3d(sB + (PB * kb + 1) * C::kBBlk, &mBm, &bfull, kb * kBK, 0, q);
-                tma_load_3d(sB + (PB * kb + PB - 1) * C::kBBlk, &mBl, &bfull, kb * kBK, 0, q);
+                tma_load_3d(sB + 2 * kb * C::kBBlk, &mBh, &bfull, kb * kBK, 0, q);
+                tma_load_3d(sB + (2 * kb + 1) * C::kBBlk, &mBl, &bfull, kb * kBK, 0, q);
             }
             b_issued = true;
         }
@@ -942,19 +929,13 @@ tcx_y_kernel(const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CU
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     unsigned char *st = sA + (size_t)s * C::kStageBytes;
                     const uint64_t ah = smem_desc(st), al = smem_desc(st + C::kAPlane);
-                    const uint64_t bh = smem_desc(sB + (PB * kb) * C::kBBlk);
-                    const uint64_t bm = smem_desc(sB + (PB * kb + 1) * C::kBBlk);
-                    const uint64_t bl = smem_desc(sB + (PB * kb + PB - 1) * C::kBBlk);
+                    const uint64_t bh = smem_desc(sB + 2 * kb * C::kBBlk), bl = smem_desc(sB + (2 * kb + 1) * C::kBBlk);
 #pragma unroll
                     for (int k = 0; k < kBK / 16; ++k) {
                         const uint64_t dk = (uint64_t)((k * 32) >> 4);
                         mma_bf16(d, ah + dk, bh + dk, idesc, (kb > 0 || k > 0) ? 1u : 0u);
                         mma_bf16(d, ah + dk, bl + dk, idesc, 1u);
                         mma_bf16(d, al + dk, bh + dk, idesc, 1u);
-                        if (PB == 3) {
-                            mma_bf16(d, ah + dk, bm + dk, idesc, 1u);
-                            mma_bf16(d, al + dk, bm + dk, idesc, 1u);
-                        }
                     }
                     mma_commit(&aempty[s]);
                 }
@@ -1049,7 +1030,7 @@ tcx_y_kernel(const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CU
                 b = 3 * jk.x + t / 3;
                 c = 3 * jk.y + t % 3;
             }
-            for (int ci = hf; ok && ci < BN / 32; ci += 2) {
+            for (int ci = hf; ok && ci < kBN / 32; ci += 2) {
                 const int c0 = ci * 32;
                 float v[32];
                 tmem_ld32(taddr + c0, v);
@@ -1107,11 +1088,9 @@ tcx_y_kernel(const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CU
     }
 }
 
-// B1 (which = 0) and B2 (which = 1) of every q, [nq][2H][2H] K-major, as
-// BF16 pieces: hi + lo, or hi + mid + lo when mid is given.
+// B1 (which = 0) and B2 (which = 1) of every q, [nq][2H][2H] K-major, as BF16 hi + lo.
 __global__ void embed_kernel(int nq, int nb, int H, const double2 *__restrict__ eig, int which,
-                             __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ mid,
-                             __nv_bfloat16 *__restrict__ lo) {
+                             __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo) {
     const int Kp = 2 * H, BN = 2 * H;
     const size_t n = (size_t)nq * BN * Kp;
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n;
@@ -1128,15 +1107,8 @@ __global__ void embed_kernel(int nq, int nb, int H, const double2 *__restrict__ 
             else v = (float)(im_row ? (im_col ? e.x : -e.y) : (im_col ? e.y : e.x));
         }
         const __nv_bfloat16 h = __float2bfloat16_rn(v);
-        const float r = v - __bfloat162float(h);
         hi[t] = h;
-        if (mid) {
-            const __nv_bfloat16 m = __float2bfloat16_rn(r);
-            mid[t] = m;
-            lo[t] = __float2bfloat16_rn(r - __bfloat162float(m));
-        } else {
-            lo[t] = __float2bfloat16_rn(r);
-        }
+        lo[t] = __float2bfloat16_rn(v - __bfloat162float(h));
     }
 }
 
@@ -1275,7 +1247,7 @@ struct Lane {
     cudaStream_t st;
     cudaEvent_t done[2];           // after GEMM2 of the lane's batches, alternately
     XParams x;
-    CUtensorMap maps[13];          // A1 hi/lo, B1 h/m/l, T1 hi/lo, B2 h/m/l, B0 h/l/l (FP16)
+    CUtensorMap maps[10];          // A1, B1, T1, B2, B0 (FP16), hi and lo each
     __nv_bfloat16 *a1h, *a1l;
     const float *wscale;           // scales of the tensor-core phase sum (y_scale_kernel)
 };
@@ -1299,18 +1271,18 @@ struct TcxSched {
 // stages, the phase tables and one tile's block table) is within the opt-in limit.
 constexpr size_t kSmemOptin = 232448 - 2048;   // less the kernel's static shared memory
 size_t tcx_y_bytes(int nb, int n_rep) {
-    return tcx_y_smem(CfgY<192, 2>::kFixed, std::max(1, n_rep), nb / 3);
+    return tcx_y_smem(CfgY::kFixed, std::max(1, n_rep), nb / 3);
 }
 bool tcx_y_fits(int nb, int n_rep) { return nb % 3 == 0 && tcx_y_bytes(nb, n_rep) <= kSmemOptin; }
 
-template <int BN, int PB, int SHAPE>
+template <int SHAPE>
 cudaError_t run_batches(const LwParams &p, const LwDev &d, const TcxGroups &g, Lane *lanes, TcxSched sc,
                         long long pbeg, long long pend, bool reduce, double *gacc, int *err, float *out3) {
     const int batch = sc.batch, tpc = sc.tpc;
     const bool sym = lanes[0].x.plist != nullptr;
-    auto k1 = tcx_gemm_kernel<EPI_T, BN, PB, 0>;
-    auto k2 = sym ? tcx_gemm_kernel<EPI_SYM, BN, PB, SHAPE> : tcx_gemm_kernel<EPI_PHI, BN, PB, SHAPE>;
-    constexpr int smem = Cfg<BN, PB>::kSmem;
+    auto k1 = tcx_gemm_kernel<EPI_T, 0>;
+    auto k2 = sym ? tcx_gemm_kernel<EPI_SYM, SHAPE> : tcx_gemm_kernel<EPI_PHI, SHAPE>;
+    constexpr int smem = Cfg::kSmem;
     cudaError_t e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
@@ -1321,9 +1293,9 @@ cudaError_t run_batches(const LwParams &p, const LwDev &d, const TcxGroups &g, L
     // tensor-core phase sum: row tiles of kYGroups groups, about one wave of CTAs per launch
     const bool yk = sc.yk && tcx_y_fits(nb, p.n_rep) && g.y.n_groups > 0;
     const int mty = (g.y.n_groups + kYGroups - 1) / kYGroups;
-    const size_t ysmem = tcx_y_smem(CfgY<BN, PB>::kFixed, std::max(1, p.n_rep), nb / 3);
+    const size_t ysmem = tcx_y_smem(CfgY::kFixed, std::max(1, p.n_rep), nb / 3);
     if (yk) {
-        e = cudaFuncSetAttribute(tcx_y_kernel<BN, PB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ysmem);
+        e = cudaFuncSetAttribute(tcx_y_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ysmem);
         if (e != cudaSuccess) return e;
     }
     long long i = 0;
@@ -1340,8 +1312,8 @@ cudaError_t run_batches(const LwParams &p, const LwDev &d, const TcxGroups &g, L
         ProfMark pg(p.prof, KALD_PROF_TCX_GATHER, L.st);
         if (yk) {
             const int tpy = std::max(1, std::min(sc.tpy, mty));
-            tcx_y_kernel<BN, PB><<<counted(dim3((mty + tpy - 1) / tpy, x.n_pairs)), kYThreads, ysmem, L.st>>>(
-                L.maps[10], L.maps[11], L.maps[12], x, g.y, cw, p.n_rep, L.wscale, L.a1h, L.a1l, tpy, err);
+            tcx_y_kernel<<<counted(dim3((mty + tpy - 1) / tpy, x.n_pairs)), kYThreads, ysmem, L.st>>>(
+                L.maps[8], L.maps[9], x, g.y, cw, p.n_rep, L.wscale, L.a1h, L.a1l, tpy, err);
         } else {
             ycx_gather_kernel<<<counted(dim3(kGatherParts, x.n_pairs)), 32 * kGatherWarps, gather_smem(nb), L.st>>>(
                 x, g, ew, cw, p.n_rep, L.a1h, L.a1l);
@@ -1349,11 +1321,11 @@ cudaError_t run_batches(const LwParams &p, const LwDev &d, const TcxGroups &g, L
         pg.end();
         ProfMark p1(p.prof, KALD_PROF_TCX_GEMM1, L.st);
         k1<<<counted(dim3(gx, x.n_pairs)), Warps<EPI_T>::kThreads, smem, L.st>>>(L.maps[0], L.maps[1], L.maps[2], L.maps[3],
-                                                                    L.maps[4], x, tpc, err);
+                                                                                 x, tpc, err);
         p1.end();
         ProfMark p2(p.prof, KALD_PROF_TCX_GEMM2, L.st);
-        k2<<<counted(dim3(gx, x.n_pairs)), Warps<EPI_PHI>::kThreads, smem, L.st>>>(L.maps[5], L.maps[6], L.maps[7], L.maps[8],
-                                                                    L.maps[9], x, tpc, err);
+        k2<<<counted(dim3(gx, x.n_pairs)), Warps<EPI_PHI>::kThreads, smem, L.st>>>(L.maps[4], L.maps[5], L.maps[6],
+                                                                                   L.maps[7], x, tpc, err);
         p2.end();
         if (sym) {
             const int nt = (3 * p.nb + 31) / 32 * 32;
@@ -1493,7 +1465,7 @@ size_t tcx_scratch_bytes(int nb, int nq, int batch) {
     const size_t Mp = (size_t)(nb * nb + kBM - 1) / kBM * kBM;
     const size_t eb = ws_round(sizeof(__nv_bfloat16) * (size_t)nq * BN * Kp);
     const size_t ab = ws_round(sizeof(__nv_bfloat16) * (size_t)batch * Kp * Mp);
-    return 8 * eb + 8 * ab + ws_round(16) + ws_round(sizeof(float) * 2 * (size_t)tcx_slices(nq, batch) * nq * nb) +
+    return 6 * eb + 8 * ab + ws_round(16) + ws_round(sizeof(float) * 2 * (size_t)tcx_slices(nq, batch) * nq * nb) +
            ws_round(sizeof(double) * (size_t)nq * nb);
 }
 
@@ -1619,15 +1591,12 @@ cudaError_t launch_lw_tensor(const LwParams &p, const LwDev &d, const TcxGroups 
     auto take = [&](size_t bytes) { char *r = b + off; off += ws_round(bytes); return r; };
     const size_t eb = sizeof(__nv_bfloat16) * (size_t)nq * BN * Kp;
     auto *b1h = reinterpret_cast<__nv_bfloat16 *>(take(eb));
-    auto *b1m = reinterpret_cast<__nv_bfloat16 *>(take(eb));
     auto *b1l = reinterpret_cast<__nv_bfloat16 *>(take(eb));
     auto *b2h = reinterpret_cast<__nv_bfloat16 *>(take(eb));
-    auto *b2m = reinterpret_cast<__nv_bfloat16 *>(take(eb));
     auto *b2l = reinterpret_cast<__nv_bfloat16 *>(take(eb));
     auto *b0h = reinterpret_cast<__half *>(take(eb));
     auto *b0l = reinterpret_cast<__half *>(take(eb));
     auto *wscale = reinterpret_cast<float *>(take(16));
-    const bool three = BN <= 128;          // three pieces of B fit in shared memory
     const size_t ab = sizeof(__nv_bfloat16) * (size_t)batch * Kp * Mp;
     __nv_bfloat16 *pl[2][4];                       // per lane: A1 hi, A1 lo, T1 hi, T1 lo
     for (int l = 0; l < 2; ++l)
@@ -1649,8 +1618,8 @@ cudaError_t launch_lw_tensor(const LwParams &p, const LwDev &d, const TcxGroups 
     if (e == cudaSuccess) e = cudaMemsetAsync(d.allowed, 0, sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
     const int eg = (int)std::min<size_t>(((size_t)nq * BN * Kp + 255) / 256, 4096);
-    embed_kernel<<<counted(eg), 256, 0, st>>>(nq, nb, H, d.eig, 0, b1h, three ? b1m : nullptr, b1l);
-    embed_kernel<<<counted(eg), 256, 0, st>>>(nq, nb, H, d.eig, 1, b2h, three ? b2m : nullptr, b2l);
+    embed_kernel<<<counted(eg), 256, 0, st>>>(nq, nb, H, d.eig, 0, b1h, b1l);
+    embed_kernel<<<counted(eg), 256, 0, st>>>(nq, nb, H, d.eig, 1, b2h, b2l);
     if (g.y.fc3) {
         embed_b0_kernel<<<counted(eg), 256, 0, st>>>(nq, nb, H, d.eig, b0h, b0l);
         y_scale_kernel<<<counted(1), 1024, 0, st>>>(g.y, wscale);
@@ -1669,7 +1638,6 @@ cudaError_t launch_lw_tensor(const LwParams &p, const LwDev &d, const TcxGroups 
     x.t1h = nullptr; x.t1l = nullptr;
     x.wn = d.wn32;
     x.sig2inv = (float)delta_param(p.shape, p.sigma_w);
-    x.shape = p.shape;
     x.cut = (float)p.cut_w;
     x.n_slices = n_slices;
     x.slots = slots;
@@ -1703,16 +1671,13 @@ cudaError_t launch_lw_tensor(const LwParams &p, const LwDev &d, const TcxGroups 
         L.a1h = pl[l][0]; L.a1l = pl[l][1];
         L.wscale = wscale;
         L.x.t1h = pl[l][2]; L.x.t1l = pl[l][3];
-        if (!make_map3(&L.maps[0], pl[l][0], Mp, Kp, batch, kAK) ||
-            !make_map3(&L.maps[1], pl[l][1], Mp, Kp, batch, kAK) || !make_map3(&L.maps[2], b1h, Kp, BN, nq, BN) ||
-            !make_map3(&L.maps[3], b1m, Kp, BN, nq, BN) || !make_map3(&L.maps[4], b1l, Kp, BN, nq, BN) ||
-            !make_map3(&L.maps[5], pl[l][2], Mp, Kp, batch, kAK) ||
-            !make_map3(&L.maps[6], pl[l][3], Mp, Kp, batch, kAK) || !make_map3(&L.maps[7], b2h, Kp, BN, nq, BN) ||
-            !make_map3(&L.maps[8], b2m, Kp, BN, nq, BN) || !make_map3(&L.maps[9], b2l, Kp, BN, nq, BN) ||
-            !make_map3(&L.maps[10], b0h, Kp, BN, nq, BN, CU_TENSOR_MAP_DATA_TYPE_FLOAT16) ||
-            !make_map3(&L.maps[11], b0l, Kp, BN, nq, BN, CU_TENSOR_MAP_DATA_TYPE_FLOAT16) ||
-            !make_map3(&L.maps[12], b0l, Kp, BN, nq, BN, CU_TENSOR_MAP_DATA_TYPE_FLOAT16))
-            return cudaErrorInvalidValue;
+        for (int k = 0; k < 2; ++k)
+            if (!make_map3(&L.maps[k], pl[l][k], Mp, Kp, batch, kAK) ||
+                !make_map3(&L.maps[2 + k], k ? b1l : b1h, Kp, BN, nq, BN) ||
+                !make_map3(&L.maps[4 + k], pl[l][2 + k], Mp, Kp, batch, kAK) ||
+                !make_map3(&L.maps[6 + k], k ? b2l : b2h, Kp, BN, nq, BN) ||
+                !make_map3(&L.maps[8 + k], k ? b0l : b0h, Kp, BN, nq, BN, CU_TENSOR_MAP_DATA_TYPE_FLOAT16))
+                return cudaErrorInvalidValue;
     }
     // second lane: its own stream, forked from and joined back into st
     cudaStream_t aux = nullptr;
@@ -1725,9 +1690,9 @@ cudaError_t launch_lw_tensor(const LwParams &p, const LwDev &d, const TcxGroups 
         lanes[0].st = st; lanes[0].done[0] = ev[0]; lanes[0].done[1] = ev[1];
         lanes[1].st = aux; lanes[1].done[0] = ev[2]; lanes[1].done[1] = ev[3];
         auto run = [&](TcxSched sc, long long b0, long long b1, bool reduce) -> cudaError_t {
-            return p.shape == kDeltaGauss     ? run_batches<192, 2, kDeltaGauss>(p, d, g, lanes, sc, b0, b1, reduce, gacc, err, out3)
-                   : p.shape == kDeltaLorentz ? run_batches<192, 2, kDeltaLorentz>(p, d, g, lanes, sc, b0, b1, reduce, gacc, err, out3)
-                                              : run_batches<192, 2, kDeltaTriangle>(p, d, g, lanes, sc, b0, b1, reduce, gacc, err, out3);
+            return p.shape == kDeltaGauss     ? run_batches<kDeltaGauss>(p, d, g, lanes, sc, b0, b1, reduce, gacc, err, out3)
+                   : p.shape == kDeltaLorentz ? run_batches<kDeltaLorentz>(p, d, g, lanes, sc, b0, b1, reduce, gacc, err, out3)
+                                              : run_batches<kDeltaTriangle>(p, d, g, lanes, sc, b0, b1, reduce, gacc, err, out3);
         };
         // pairs of the projected q-points, or the orbit pairs
         const long long pbeg = 0, pend = sym ? (long long)sym->n_pairs : (long long)p.nqc * nq;
