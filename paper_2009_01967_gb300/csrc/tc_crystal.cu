@@ -820,10 +820,11 @@ static size_t gather_smem(int nb) {
 // exactly as the CUDA-core gather does.  Both operands of this contraction
 // are FP16 hi + lo pieces (11-bit significands: a pair carries a value to
 // about 2^-22 of itself, where BF16 pieces carry 2^-18) scaled by powers of
-// two that keep them in FP16 range: B0 = 2^14 eps (|eps| <= 1) and W times
-// wscale[0] = 2^(14 - e), e = exponent of a bound on |W| (max over entries
-// of the sum of |Phi3~| over their blocks, the phases having modulus one);
-// the epilogue multiplies by wscale[1] = 2^-14 / wscale[0] (exact).  Roles: warp 0 loads B0
+// two that keep them in FP16 range: B0 = 2^14 eps (|eps| <= 1) and the rows of a
+// group times 2^(14 - e), e = exponent of a bound on |W| there (max over entries
+// of the sum of |Phi3~| over their blocks, the phases having modulus one); the
+// epilogue takes both out (exact).  One exponent for all groups lost the linewidths
+// of a part whose Phi3 is far below the rest's.  Roles: warp 0 loads B0
 // (TMA), warp 1 issues the MMAs, warps 4..11 run the epilogue, warps 2, 3 and
 // 12..15 build.  Every wait is bounded; the builders pass the same named
 // barriers whether or not a wait failed.
@@ -945,7 +946,6 @@ tcx_y_kernel(const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CU
             mma_commit(&drain);
         }
     } else if (builder) {
-        const float sw = __ldg(wscale);
         int it = 0;
         for (int i = 0; i < n_tiles; ++i) {
             const int g0 = (t0 + i) * kYGroups, ng = min(kYGroups, yt.n_groups - g0);
@@ -964,6 +964,7 @@ tcx_y_kernel(const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CU
                 const int i_lo = a_lo / 3, n_i = a_hi > a_lo ? (a_hi - 1) / 3 - i_lo + 1 : 0;
                 for (int item = bt; item < ng * n_i; item += kYBuilders) {
                     const int g = item / n_i, ia = i_lo + item % n_i;
+                    const float sw = __ldg(wscale + 2 * (g0 + g));
                     float2 acc[3][9];
 #pragma unroll
                     for (int al = 0; al < 3; ++al)
@@ -1013,7 +1014,6 @@ tcx_y_kernel(const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CU
         const int ew = warp - 4, qd = warp & 3, hf = ew >> 2;
         const int row = qd * 32 + lane;
         const bool vec = (nb % 8) == 0;
-        const float unscale = __ldg(wscale + 1);
         for (int i = 0; i < n_tiles; ++i) {
             const int buf = i & 1;
             bool ok = !*(volatile int *)&fail_sm && mbar_wait(&tfull[buf], (i >> 1) & 1, x.wait_limit);
@@ -1024,7 +1024,9 @@ tcx_y_kernel(const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CU
             const int g0 = (t0 + i) * kYGroups, ng = min(kYGroups, yt.n_groups - g0);
             const bool rv = row < 9 * ng;
             int b = 0, c = 0;
+            float unscale = 0.0f;
             if (rv) {
+                unscale = __ldg(wscale + 2 * (g0 + row / 9) + 1);
                 const int2 jk = __ldg(yt.gjk + g0 + row / 9);
                 const int t = row % 9;
                 b = 3 * jk.x + t / 3;
@@ -1136,15 +1138,13 @@ __global__ void embed_b0_kernel(int nq, int nb, int H, const double2 *__restrict
     }
 }
 
-// wscale[0] = 2^(14 - e), e the exponent of max over (group, i, alpha beta
-// gamma) of the sum of |Phi3~[alpha beta gamma]| over the blocks of (group,
-// i) (a bound on |W|); wscale[1] = 2^-14 / wscale[0].  One block.
-__global__ void y_scale_kernel(TcxYTables yt, float *__restrict__ wscale) {
-    __shared__ float red[32];
-    const int ld = yt.n_at + 1;
+// wscale[2 g] = 2^(14 - e), e the exponent of max over (i, alpha beta gamma) of the sum
+// of |Phi3~[alpha beta gamma]| over the blocks of (group g, i) (a bound on |W| in the
+// group's rows); wscale[2 g + 1] = 2^-14 / wscale[2 g].  One warp per group, a lane per i.
+__global__ void __launch_bounds__(32) y_scale_kernel(TcxYTables yt, float *__restrict__ wscale) {
+    const int g = blockIdx.x, ld = yt.n_at + 1;
     float m = 0.0f;
-    for (int item = threadIdx.x; item < yt.n_groups * yt.n_at; item += blockDim.x) {
-        const int g = item / yt.n_at, i = item % yt.n_at;
+    for (int i = threadIdx.x; i < yt.n_at; i += 32) {
         float sum[27];
 #pragma unroll
         for (int t = 0; t < 27; ++t) sum[t] = 0.0f;
@@ -1157,14 +1157,11 @@ __global__ void y_scale_kernel(TcxYTables yt, float *__restrict__ wscale) {
         for (int t = 0; t < 27; ++t) m = fmaxf(m, sum[t]);
     }
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-    __syncthreads();
     if (threadIdx.x == 0) {
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmaxf(m, red[w]);
         // bound * 1.0001 absorbs the rounding of the FP32 sums
         const int e = m > 0.0f ? ilogbf(m * 1.0001f) : 0;
-        wscale[0] = ldexpf(1.0f, 14 - e);
-        wscale[1] = ldexpf(1.0f, e - 28);
+        wscale[2 * g] = ldexpf(1.0f, 14 - e);
+        wscale[2 * g + 1] = ldexpf(1.0f, e - 28);
     }
 }
 
@@ -1460,12 +1457,15 @@ size_t tcx_sym_bytes(int nb, int batch, int n_pairs) {
            ws_round(sizeof(float) * 3 * (size_t)n_pairs * nb);
 }
 
+// Two scales per (j, k) group.
+static size_t tcx_wscale_bytes(int nb) { return sizeof(float) * 2 * (size_t)(nb / 3) * (nb / 3); }
+
 size_t tcx_scratch_bytes(int nb, int nq, int batch) {
     const int H = tcx_half(nb), Kp = 2 * H, BN = 2 * H;
     const size_t Mp = (size_t)(nb * nb + kBM - 1) / kBM * kBM;
     const size_t eb = ws_round(sizeof(__nv_bfloat16) * (size_t)nq * BN * Kp);
     const size_t ab = ws_round(sizeof(__nv_bfloat16) * (size_t)batch * Kp * Mp);
-    return 6 * eb + 8 * ab + ws_round(16) + ws_round(sizeof(float) * 2 * (size_t)tcx_slices(nq, batch) * nq * nb) +
+    return 6 * eb + 8 * ab + ws_round(tcx_wscale_bytes(nb)) + ws_round(sizeof(float) * 2 * (size_t)tcx_slices(nq, batch) * nq * nb) +
            ws_round(sizeof(double) * (size_t)nq * nb);
 }
 
@@ -1596,7 +1596,7 @@ cudaError_t launch_lw_tensor(const LwParams &p, const LwDev &d, const TcxGroups 
     auto *b2l = reinterpret_cast<__nv_bfloat16 *>(take(eb));
     auto *b0h = reinterpret_cast<__half *>(take(eb));
     auto *b0l = reinterpret_cast<__half *>(take(eb));
-    auto *wscale = reinterpret_cast<float *>(take(16));
+    auto *wscale = reinterpret_cast<float *>(take(tcx_wscale_bytes(nb)));
     const size_t ab = sizeof(__nv_bfloat16) * (size_t)batch * Kp * Mp;
     __nv_bfloat16 *pl[2][4];                       // per lane: A1 hi, A1 lo, T1 hi, T1 lo
     for (int l = 0; l < 2; ++l)
@@ -1622,7 +1622,7 @@ cudaError_t launch_lw_tensor(const LwParams &p, const LwDev &d, const TcxGroups 
     embed_kernel<<<counted(eg), 256, 0, st>>>(nq, nb, H, d.eig, 1, b2h, b2l);
     if (g.y.fc3) {
         embed_b0_kernel<<<counted(eg), 256, 0, st>>>(nq, nb, H, d.eig, b0h, b0l);
-        y_scale_kernel<<<counted(1), 1024, 0, st>>>(g.y, wscale);
+        y_scale_kernel<<<counted(std::max(1, g.y.n_groups)), 32, 0, st>>>(g.y, wscale);
     }
 
     cudaError_t ge = cudaFuncSetAttribute(ycx_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,

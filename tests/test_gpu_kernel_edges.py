@@ -764,3 +764,22 @@ def test_symmetry_of_a_weak_part(k):
     _, W = kk.kald_kappa_qhgk(ctx, [s], nu.ravel(), eig.ravel(), np.full(6 * n, 0.1),
                               kk.Options(temperature_K=300.0, sigma_thz=0.1), want_vgen=True)
     np.testing.assert_allclose(W[:, 3 * n:, 3 * n:], W_o, rtol=0, atol=1e-10 * np.abs(W_o).max())
+
+
+@pytest.mark.parametrize("phase_sum", ["0", "1"])
+@pytest.mark.parametrize("log_ratio", [20, 24])
+def test_crystal_split_of_unlike_parts(k, log_ratio, phase_sum, monkeypatch):
+    """72 branches, half of them on a part whose Phi3 is 2^20 or 2^24 times weaker, with
+    the phase sum on CUDA cores and on tensor cores: a power of two in a part's Phi3 is
+    exact in every operand, so the part's linewidths are those of the same cell with
+    parts of one strength times its square, to the rounding of FP32 sums."""
+    kk, ctx = k
+    monkeypatch.setenv("KALD_TCX_Y", phase_sum)
+    mesh = (3, 1, 1)
+    opt = kk.Options(temperature_K=300.0, sigma_thz=0.1, precision="bf16split")
+    alike, unlike = (_two_parts((3, 1, 1), r, False)[0] for r in (1.0, 2.0 ** -log_ratio))
+    nu, eig = ph.phonons(alike, mesh)
+    weak = (np.abs(eig[:, :, 36:]) ** 2).sum(-1).ravel() > 0.5
+    ref, got = (np.asarray(kk.kald_linewidths(ctx, s, mesh, nu, eig, opt)[0]).ravel() for s in (alike, unlike))
+    assert _rel(got[weak] * 4.0 ** log_ratio, ref[weak]) < 1e-6
+    assert _rel(got[~weak], ref[~weak]) < 1e-6
