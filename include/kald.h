@@ -359,8 +359,11 @@ kald_status kald_kappa_rta(kald_ctx *ctx, const kald_system *sys, const int32_t 
  *   eigvec  real eigenvectors (imaginary parts must be zero)
  *   kappa   [n_sys][3][3] out
  *   vgen    [3][nb][nb] out (W_a in A/ps, system 0 only) or NULL
- * W_a is a product of exact slices on the tensor cores: a pipeline wait that
- * expires returns KALD_E_TIMEOUT (also from kald_diffusivity). */
+ * W_a is a product of fixed-point slices on the tensor cores, 55 bits from the
+ * largest element of each row of E and of A_a E: its error is that of an FP64
+ * product relative to the row maxima (some 1e-15 of the largest |W_a|), so that
+ * elements far below it are not exact to their own last bits.  A pipeline wait
+ * that expires returns KALD_E_TIMEOUT (also from kald_diffusivity). */
 kald_status kald_kappa_qhgk(kald_ctx *ctx, int32_t n_sys, const kald_system *sys,
                             const double *nu_thz, const double *eigvec, const double *gamma,
                             const kald_options *opt, double *kappa, double *vgen);

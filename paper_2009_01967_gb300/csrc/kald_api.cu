@@ -854,7 +854,7 @@ static kald_status phonons_impl(kald_ctx *ctx, const HostSystem &h, const int32_
     if ((st = finish(ctx, "kald_phonons"))) return st;
     if (nc)
         return fail(ctx, KALD_E_NOCONV,
-                    "Jacobi eigensolver did not converge at " + std::to_string(nc) + " q-points");
+                    "eigensolver did not converge at " + std::to_string(nc) + " q-points");
     return KALD_OK;
 }
 

@@ -782,7 +782,7 @@ mirror_check_kernel(LwParams p, const int *__restrict__ qfrac, const M *__restri
 // near ends and walks only the modes inside (about a seventh of them per
 // window at 3 sigma = 0.15 THz of a 2 THz band); the exact test of the window
 // decides, the walk is a little wider.  32 atoms, 6^3 mesh, FP32: 143 ms when
-// every (s', s'') was tested by one thread per (q, s), 5.3 ms now (half of the q-points).
+// every (s', s'') was tested by one thread per (q, s), 5.5 ms now (half of the q-points).
 template <typename R>
 __global__ void __launch_bounds__(128)
 phase_space_kernel(LwParams p, LwDev d, const void *__restrict__ modes, const int *__restrict__ differ, int chunk,

@@ -13,8 +13,15 @@
 // kOzChunk = 512 values of d sum to at most 2^24, so that the FP32 accumulators
 // hold them exactly.  After every chunk the epilogue adds the eight levels
 // into two 64-bit integers per element (levels 0-3 and 4-7), and only the end
-// converts to FP64.  Levels above 7 are dropped: 2^-56 of the product of the
-// row maxima, below the rounding of an FP64 sum of this length.
+// converts to FP64.  What is lost: each operand's rounding, 2^-56 of its row's
+// largest element, and the levels above 7, of which the first holds seven digit
+// products of up to 2^-56 of the product of the row maxima for every d -- together
+// at most about 9 n 2^-56 of that product (2^-42 for 2,592 modes), and some
+// sqrt(n) of it as a rule: 2e-15 to 4e-15 of the product of the row maxima for 324
+// and 768 modes, where FP64 sums have 2e-15 to 1e-14.  It is relative to the rows'
+// largest elements, not to sum |E B|: an element between two modes whose vectors
+// hardly overlap carries the absolute error of its rows (5e-14 of sum |E B| for
+// elements spread over e^-20, where an FP64 sum has 2e-15).
 //
 // Bound: L2 to shared memory, 98 KB per stage of 32 values of d (36 digit
 // pairs, 1,152 MMA cycles).  The FP64 units made the same product the time of
