@@ -16,7 +16,7 @@
 // converts to FP64.  What is lost: each operand's rounding, 2^-56 of its row's
 // largest element, and the levels above 7, of which the first holds seven digit
 // products of up to 2^-56 of the product of the row maxima for every d -- together
-// at most about 9 n 2^-56 of that product (2^-42 for 2,592 modes), and some
+// at most about 9 n 2^-56 of that product (3e-13 for 2,592 modes), and some
 // sqrt(n) of it as a rule: 2e-15 to 4e-15 of the product of the row maxima for 324
 // and 768 modes, where FP64 sums have 2e-15 to 1e-14.  It is relative to the rows'
 // largest elements, not to sum |E B|: an element between two modes whose vectors
