@@ -464,20 +464,18 @@ kald_status plan_system(kald_ctx *ctx, const kald_system *s, HostSystem &h) {
     };
     const std::vector<int> by_k = stable_key_order(ng, n, [&](int g) { return (long long)h.pair3_k[g]; });
     const std::vector<int> by_class = stable_key_order(ng, kYLong + 1, [&](int x) { return (long long)len_class(by_k[x]); });
-    h.pair3_order.resize(ng);
-    h.pair3_long = 0;
-    for (int x = 0; x < ng; ++x) {
-        h.pair3_order[x] = by_k[by_class[x]];
-        h.pair3_long += len_class(h.pair3_order[x]) == 0;
+    h.pair3_kstart.assign(n + 1, make_int2(0, 0));
+    for (int g = 0; g < ng; ++g) {
+        h.pair3_kstart[h.pair3_k[g] + 1].x += 1;
+        h.pair3_kstart[h.pair3_k[g]].y += len_class(g) == 0;
     }
-    h.pair3_kstart.assign(n + 1, 0);
-    for (int g = 0; g < ng; ++g) ++h.pair3_kstart[h.pair3_k[g] + 1];
-    for (int k = 0; k < n; ++k) h.pair3_kstart[k + 1] += h.pair3_kstart[k];
-    h.pair3_at.resize(ng);
-    std::vector<int> at(h.pair3_kstart.begin(), h.pair3_kstart.end() - 1);
+    for (int k = 0; k < n; ++k) h.pair3_kstart[k + 1].x += h.pair3_kstart[k].x;
+    h.pair3_grp.resize(ng);
+    std::vector<int> at(n);
+    for (int k = 0; k < n; ++k) at[k] = h.pair3_kstart[k].x;
     for (int x = 0; x < ng; ++x) {
-        const int g = h.pair3_order[x];
-        h.pair3_at[at[h.pair3_k[g]]++] = make_int2(x, h.pair3_j[g]);
+        const int g = by_k[by_class[x]];
+        h.pair3_grp[at[h.pair3_k[g]]++] = make_int4(h.pair3_start[g], h.pair3_start[g + 1], h.pair3_j[g], 0);
     }
     h.n_rep = n_rep;
     return KALD_OK;
@@ -1250,7 +1248,6 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
             gp.sym3 = !lean && opt->symmetry == KALD_SYM_ALL && h.fc3_perm_symmetric;
             gp.mb_max = lean ? std::max(1, tc_gamma_batch(nb, ctx->sm_count, 0) / 2)
                              : tc_gamma_batch_max(nb, ctx->sm_count, gp.sym3);
-            gp.n_long = h.pair3_long;
             band_tiles(gp.omega_h, tc_tile(), opt->n_sigma * kTwoPi * opt->sigma_thz, gp.symmetric, gp.sym3, gp.tiles,
                        gp.tile_start);
         }
@@ -1259,8 +1256,8 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
                    scaled_bytes(h.fc3_blk, h.fc3_atoms, h, 27, 27, 0) + 2 * ws_round(sizeof(double) * nb) +
                    ws_round(sizeof(int) * nb);
         if (mode == KALD_BF16_SPLIT)
-            b += tc_gamma_scratch_bytes(nb, gp.mb_max, gp.n_fc3, gp.sym3, gp.tiles.size()) + bytes_of(h.pair3_order) +
-                 bytes_of(h.pair3_kstart) + bytes_of(h.pair3_at) +
+            b += tc_gamma_scratch_bytes(nb, gp.mb_max, gp.n_fc3, gp.sym3, gp.tiles.size()) +
+                 bytes_of(h.pair3_kstart) + bytes_of(h.pair3_grp) +
                  ws_round(sizeof(int2) * n_tiles + sizeof(int) * (nb + 1)) +
                  ws_round(sizeof(double) * n_tiles);
         else
@@ -1296,15 +1293,14 @@ static kald_status gamma_only_batch(kald_ctx *ctx, int n_sys, const kald_system 
         gd.occ = static_cast<double *>(ws_take(ctx, sizeof(double) * nb));
         gd.E = gd.Y = gd.T = gd.PHI = nullptr;
         gd.partial = nullptr;
-        gd.group_order = gd.k_start = nullptr;
-        gd.k_at = nullptr;
+        gd.k_start = nullptr;
+        gd.k_grp = nullptr;
         gd.tc_scratch = nullptr; gd.tiles_dev = nullptr; gd.partial_tc = nullptr;
         if (mode == KALD_BF16_SPLIT) {
             gd.tc_scratch = ws_take(ctx, tc_gamma_scratch_bytes(nb, it.gp.mb_max, it.gp.n_fc3, it.gp.sym3,
                                                                 it.gp.tiles.size()));
-            gd.group_order = upload(ctx, h.pair3_order);
             gd.k_start = upload(ctx, h.pair3_kstart);
-            gd.k_at = upload(ctx, h.pair3_at);
+            gd.k_grp = upload(ctx, h.pair3_grp);
             gd.tiles_dev = static_cast<int2 *>(ws_take(ctx, sizeof(int2) * n_tiles + sizeof(int) * (nb + 1)));
             gd.partial_tc = static_cast<double *>(ws_take(ctx, sizeof(double) * n_tiles));
         } else {

@@ -142,13 +142,11 @@ struct HostSystem {
     mutable int fc2_symmetric = -1;                    // Phi2(i, jR) = Phi2(j, i-R)^T (lazy)
     // fc3 grouped by (j, k) atom pair (CSR over output pairs)
     std::vector<int> pair3_j, pair3_k, pair3_start;
-    // the groups of more than kYLong blocks first, then by falling length, each
-    // class ordered by (k, j) (the Y build of the Gamma-only tensor-core path)
-    std::vector<int> pair3_order;
-    int pair3_long = 0;
-    // the groups of each k: (place in pair3_order, j)
-    std::vector<int> pair3_kstart;
-    std::vector<int2> pair3_at;
+    // the groups of each k (first block, end, j, 0), those of more than kYLong blocks
+    // first, then by falling length, and where each k's begin with how many of the long
+    // ones it has (the Y build of the Gamma-only tensor-core path)
+    std::vector<int2> pair3_kstart;
+    std::vector<int4> pair3_grp;
     std::vector<int> fc3_i, fc3_rj, fc3_rk;            // per block (sorted order)
     std::vector<double> fc3_blk;                       // [n_fc3][27] Phi3 (eV/A^3), grouped, not mass-scaled
     std::vector<int> fc3_atoms;                        // [n_fc3][3] (i, j, k) of each block
@@ -354,7 +352,6 @@ cudaError_t launch_mode_prep(int n, const double *nu, double omega_min_w, double
 // gamma_only.cu: Gamma-only linewidths of a system with nb > kMaxNbSmall
 struct GammaPlan {
     int n_groups = 0;
-    int n_long = 0;                  // groups with a warp of their own in the tensor-core path's Y build
     size_t n_fc3 = 0;                // fc3 blocks
     int n_part = 0;                  // epilogue CTAs (partial sums) per mode
     std::vector<double> omega_h;     // [nb] rad/ps, 0 for a masked mode
@@ -370,9 +367,8 @@ struct GammaPlan {
 };
 struct GammaDev {
     const int *group_jk, *group_start, *blk_i;   // (j, k) groups of fc3 blocks
-    const int *group_order;          // HostSystem::pair3_order (tensor-core path)
-    const int *k_start;              // HostSystem::pair3_kstart, pair3_at (tensor-core path)
-    const int2 *k_at;
+    const int2 *k_start;             // HostSystem::pair3_kstart, pair3_grp (tensor-core path)
+    const int4 *k_grp;
     const double *fc3;               // [n_fc3][27] Phi3 / sqrt(mi mj mk)
     const double2 *eig;              // [nb][nb] (real parts used)
     const double *nu;                // [nb] THz

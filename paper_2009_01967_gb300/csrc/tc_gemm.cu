@@ -82,6 +82,8 @@ struct EpiSplit {
     int ld;
     int b_rows;               // rows of one Y / T plane (stacked per mode of the batch)
     int tm0;                  // first row tile
+    int mu0;                  // first mode of the batch
+    const int *yk;            // [batch][N / 3] exponents of the rows of Y (ybuild_rows_kernel)
 };
 
 // Powers of two that bring the operands into FP16's range.  With k the exponents of
@@ -89,27 +91,28 @@ struct EpiSplit {
 // Y^_mu(c, b) = 2^(-k_b - k_c) Y_mu(c, b), whose contractions over b and c are those
 // of E and Y:
 //   E^(m, .) = 2^e_m E', |E'| <= 1 and |E'|_2 <= 2^h_m, stored x 2^kEBits;
-//   Y^_mu = 2^y_mu Y', |Y'| <= 1 (y_mu from its largest element), stored x 2^kYBits;
+//   Y^_mu(c, .) = 2^y_mu,k Y', |Y'| <= 1 (the largest element of the rows of c's atom
+//   k), stored x 2^kYBits; y_mu = max over k;
 //   T^ = E^ Y^_mu = 2^(e_m + y_mu) T', |T'| <= 2^(h_m + hR) (Cauchy-Schwarz: the rows
 //   of Y_mu have at most 4^hR entries), stored x 2^(kTBits - h_m - hR).
 // FP16's step is 2^-24, so an element keeps the 16 bits of two BF16 pieces down to
-// 2^-23 of the largest one of its row of E or of its Y_mu, and to some 2^-16 of a
+// 2^-23 of the largest one of its row of E or rows of Y_mu, and to some 2^-16 of a
 // usual one of T.  The scales therefore follow what is measured: Y_mu per mode, since
 // the strong couplings inside a molecule cancel for the modes that move it as a whole,
 // and the atoms, since a mode may extend over parts whose Phi3 differs by orders of
 // magnitude.  With one exponent for the whole Phi3 the modes of the weaker part lost
 // 3e-4 of gamma where its Phi3 is 2^-16 of the stronger part's, 4e-3 at 2^-20 and 0.3
 // at 2^-24; 4e-7 now, as in a uniform cell, and 2e-6 for modes mixed of the two parts
-// at 2^-24 (216 modes).  The passes this takes: 256 atoms 2.88 -> 3.14 ms.
+// at 2^-24 (216 modes).  What this takes: 256 atoms 2.88 -> 3.05 ms (3.14 with Y_mu
+// built in FP32 first and scaled by its mode's largest element in a second pass).
 constexpr int kEBits = 15, kYBits = 15, kTBits = 15;
 struct Scales {
     const int *e, *h;         // [nb] e_m, h_m
-    const int *ymax;          // [nb] bits of the largest |Y^_mu| (FP32)
+    const int *ymax;          // [nb] y_mu (far below any exponent: no element)
     int hR;
     __device__ __forceinline__ int y(int mu) const {
-        int x;
-        frexpf(__int_as_float(__ldg(ymax + mu)), &x);
-        return x;
+        const int x = __ldg(ymax + mu);
+        return x < -1000000 ? 0 : x;
     }
     // what takes an accumulator of the second contraction to phi, for row m of mode mu
     // and for column n
@@ -198,7 +201,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
     __shared__ __align__(8) uint64_t full[kStages], empty[kStages], done;
     __shared__ uint32_t tmem_base_sm;
     __shared__ int fail_sm;
-    __shared__ float wn_sm[kBN], wl_sm[kBN], nn_sm[kBN], nl_sm[kBN], cf_sm[kBN];
+    __shared__ float wn_sm[kBN], wl_sm[kBN], nn_sm[kBN], nl_sm[kBN];
+    __shared__ __align__(16) float cf_sm[kBN];
     __shared__ double red[gemm_threads(EPI) / 32];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -266,8 +270,18 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
             mma_commit(&empty[s]);               // stage free once these MMAs finish
         }
         mma_commit(&done);                       // accumulator complete
+    } else if (EPI == EPI_SPLIT && warp >= 2) {
+        // what takes T's columns to the mode's y
+        const int y = sc.y(es.mu0 + bz);
+        for (int x = threadIdx.x - 64; x < kBN; x += 64) {
+            const int c = tn * kBN + x;
+            cf_sm[x] = c < N ? ldexpf(1.0f, __ldg(es.yk + (size_t)bz * (N / 3) + c / 3) - y) : 0.0f;
+        }
     }
     __syncwarp();
+    const int row = (warp & 3) * 32 + lane;      // accumulator lane = tile row
+    const int m = tm * kBM + row;
+    const int hm = EPI == EPI_SPLIT && m < M ? __ldg(sc.h + m) : 0;
     // ---- epilogue: wait for the accumulator (bounded)
     bool ok = mbar_wait(&done, 0, wait_limit);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -276,8 +290,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
         if (threadIdx.x == 0) atomicOr(err, 1);
     }
     const int quad = warp & 3;                   // the 32 lanes a warp may read
-    const int row = quad * 32 + lane;            // accumulator lane = tile row
-    const int m = tm * kBM + row;
     const uint32_t taddr = tmem + ((uint32_t)(quad * 32) << 16);
     if (EPI == EPI_SPLIT) {
         // whole tile: rows and columns past M, N hold exact zeros (their A rows
@@ -285,8 +297,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
         // size (ld a multiple of 128).  The lanes of a warp hold consecutive
         // rows, so each lane pair writes two whole 64-byte row segments per
         // chunk with 32-byte stores (st_rowpair_v8).
+        __syncthreads();                         // (cf_sm)
         const bool okw = __all_sync(0xffffffffu, ok);
-        const float tsc = ldexpf(1.0f, kTBits - (m < M ? __ldg(sc.h + m) : 0) - sc.hR - kEBits - kYBits);
+        const float tsc = ldexpf(1.0f, kTBits - hm - sc.hR - kEBits - kYBits);
         const size_t orow = (size_t)bz * es.b_rows + m;
         char *ph = reinterpret_cast<char *>(es.hi + orow * es.ld + tn * kBN);
         char *pl = reinterpret_cast<char *>(es.lo + orow * es.ld + tn * kBN);
@@ -299,9 +312,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ 
             uint32_t hw[16], lw[16];
 #pragma unroll
             for (int x = 0; x < 16; ++x) {
-                const float a = v[2 * x] * tsc, b = v[2 * x + 1] * tsc;
-                const __half2 h = __floats2half2_rn(a, b);
-                const __half2 l = __floats2half2_rn(a - __low2float(h), b - __high2float(h));
+                const float2 s = __fmul2_rn(*reinterpret_cast<const float2 *>(cf_sm + c0 + 2 * x), make_float2(tsc, tsc));
+                const float2 u = __fmul2_rn(make_float2(v[2 * x], v[2 * x + 1]), s);
+                const __half2 h = __floats2half2_rn(u.x, u.y);
+                const __half2 l = __floats2half2_rn(u.x - __low2float(h), u.y - __high2float(h));
                 hw[x] = *reinterpret_cast<const uint32_t *>(&h);
                 lw[x] = *reinterpret_cast<const uint32_t *>(&l);
             }
@@ -644,44 +658,53 @@ __device__ __forceinline__ void pair_fma(F2 &acc, float2 a, float2 b) {
     acc.l = __fadd_rn(acc.l, __fadd_rn(r, e));
 }
 
-// Y^_mu(c, b) of modes mu0 .. mu0 + nm - 1, in FP32 by entry: out[m][9 group + 3 (b % 3) +
-// c % 3], groups in `order`, and the bits of each mode's largest one in ymax.  Sums of
-// FP32 pairs (about 46 bits), rounded once.  y_store_kernel makes the planes:
-// their scale is known when the whole Y_mu is.
+// The rows c = 3 k .. 3 k + 2 of Y^_mu(c, b) of modes mu0 .. mu0 + nm - 1, scaled, in
+// their FP16 hi/lo planes (plane stride plane_elems); CTA = (k, MT modes).  Sums of FP32
+// pairs (about 46 bits), rounded once to FP32 and, when the rows' largest element is
+// known (its exponent goes to yk[mode][k], the mode's to ymax), split.  The other
+// elements of the planes are zero and stay so.
 //
-// Bound: FP64 units.  As plain FP64 sums (one thread per output and mode, 2
+// Bound: FP32 issue (a batch of 34 modes of 768 branches 74 us, of 22 modes 34 us; 65
+// and 33 without the largest elements, which a CTA of any groups can do).  As plain FP64
+// sums (one thread per output and mode, 2
 // FP64 FMA per clock and SM) this build took 173 us per launch of 18 modes of a 768-mode
 // cell, three times both GEMMs together; a pair FMA is 12 FP32 operations
 // against the 64 that one FP64 FMA costs here.  A thread takes MT modes
 // of one output, so a block's values are read once for all of them and the
-// modes of an eigenvector component are contiguous.  Groups come longest
-// first (order): the n_long longest -- the atoms paired with themselves hold
+// modes of an eigenvector component are contiguous.  The groups of k come longest
+// first: the k_start[k].y longest -- the atoms paired with themselves hold
 // one block per neighbour where the others hold two or three -- take a warp
-// each, three lanes per output, so that they do not serialise the launch.
+// each, three lanes per output, or the whole CTA; the warps take the others from a
+// counter.
+constexpr int kYAll = 24;
+constexpr int kNoRow = -100000;                        // exponent of rows without an element
 template <int MT>
-__global__ void __launch_bounds__(256)
-ybuild_pair_kernel(int n_groups, int n_long, const int *__restrict__ order, const int *__restrict__ group_jk,
-                   const int *__restrict__ group_start, const int *__restrict__ blk_i,
+__global__ void __launch_bounds__(256, 6)
+ybuild_rows_kernel(const int2 *__restrict__ k_start, const int4 *__restrict__ k_grp, const int *__restrict__ blk_i,
                    const float2 *__restrict__ fc3, const float2 *__restrict__ Et, int ldm, int mu0, int nm,
-                   const int *__restrict__ kx, float *__restrict__ out, unsigned *ymax) {
+                   const int *__restrict__ kx, int ld, size_t plane_elems, int n_val, __half *__restrict__ hi,
+                   __half *__restrict__ lo, int *__restrict__ yk, int *ymax) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float *val = reinterpret_cast<float *>(smem_raw);            // [MT][n_val]
     __shared__ unsigned top_sm[8][MT];
-    const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    const int m0 = blockIdx.y * MT;
-    const bool lng = gw < n_long;                      // uniform over the warp
-    const int t = lng ? 0 : (gw - n_long) * 32 + lane;
-    const int gi = lng ? gw : n_long + t / 9;
-    const int bg = lng ? lane % 9 : t % 9;
-    const bool act = gi < n_groups && (!lng || lane < 27);
-    const int g = act ? order[gi] : 0;
-    const bool put = act && !(lng && lane >= 9);
-    const int ks = put ? __ldg(kx + __ldg(group_jk + 2 * g)) + __ldg(kx + __ldg(group_jk + 2 * g + 1)) : 0;
-    F2 acc[MT];
+    __shared__ float2 part_sm[8][MT][9];
+    __shared__ int next;
+    const int k = blockIdx.x, m0 = blockIdx.y * MT, n_m = min(MT, nm - m0);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int2 ks = k_start[k];
+    const int n_g = k_start[k + 1].x - ks.x, n_w = ks.y + (9 * (n_g - ks.y) + 31) / 32;
+    const int kk = __ldg(kx + k);
+    if (threadIdx.x == 0) next = 0;
+    __syncthreads();
+    unsigned top[MT];
 #pragma unroll
-    for (int m = 0; m < MT; ++m) acc[m] = F2{0.f, 0.f};
-    if (act) {
-        const int b1 = group_start[g + 1], step = lng ? 3 : 1;
+    for (int m = 0; m < MT; ++m) top[m] = 0;
+    // sum of the blocks b0, b0 + step .. b1 - 1 of a group for output bg
+    auto blocks = [&](F2(&acc)[MT], int b0, int b1, int step, int bg) {
+#pragma unroll
+        for (int m = 0; m < MT; ++m) acc[m] = F2{0.f, 0.f};
 #pragma unroll 2
-        for (int bl = group_start[g] + (lng ? lane / 9 : 0); bl < b1; bl += step) {
+        for (int bl = b0; bl < b1; bl += step) {
             const float2 *e = Et + (size_t)(3 * __ldg(blk_i + bl)) * ldm + mu0 + m0;
             const float2 *f = fc3 + (size_t)27 * bl + bg;
 #pragma unroll
@@ -691,85 +714,98 @@ ybuild_pair_kernel(int n_groups, int n_long, const int *__restrict__ order, cons
                 for (int m = 0; m < MT; ++m) pair_fma(acc[m], v, __ldg(e + (size_t)a * ldm + m));
             }
         }
-    }
-    if (lng) {
-        // the three lanes of an output, in order
+    };
+    // the three lanes of an output (lane / 9), in order, to lanes 0 .. 8
+    auto lanes3 = [&](F2(&acc)[MT]) {
 #pragma unroll
         for (int m = 0; m < MT; ++m) {
             F2 p[2];
 #pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                p[k].h = __shfl_down_sync(0xffffffffu, acc[m].h, 9 * (k + 1));
-                p[k].l = __shfl_down_sync(0xffffffffu, acc[m].l, 9 * (k + 1));
+            for (int z = 0; z < 2; ++z) {
+                p[z].h = __shfl_down_sync(0xffffffffu, acc[m].h, 9 * (z + 1));
+                p[z].l = __shfl_down_sync(0xffffffffu, acc[m].l, 9 * (z + 1));
             }
             acc[m] = f2_add(f2_add(acc[m], p[0]), p[1]);
         }
+    };
+    auto put = [&](const F2 &s, int m, int e, int sh) {
+        const float v = ldexpf(__fadd_rn(s.h, s.l), -sh);
+        val[m * n_val + e] = v;
+        top[m] = max(top[m], __float_as_uint(fabsf(v)));
+    };
+    F2 acc[MT];
+    // groups of more than kYAll blocks by all warps, three lanes per output each
+    for (int gi = 0; gi < ks.y; ++gi) {
+        const int4 g = __ldg(k_grp + ks.x + gi);       // (first block, end, j)
+        if (g.y - g.x <= kYAll) continue;              // uniform
+        const int sh = kk + __ldg(kx + g.z);
+        blocks(acc, lane < 27 ? g.x + 3 * warp + lane / 9 : g.y, g.y, 24, lane % 9);
+        lanes3(acc);
+        __syncthreads();                               // (part_sm has been read)
+        if (lane < 9)
+#pragma unroll
+            for (int m = 0; m < MT; ++m) part_sm[warp][m][lane] = make_float2(acc[m].h, acc[m].l);
+        __syncthreads();
+        if (threadIdx.x < 9) {
+#pragma unroll
+            for (int m = 0; m < MT; ++m) {
+                F2 s{part_sm[0][m][threadIdx.x].x, part_sm[0][m][threadIdx.x].y};
+                for (int w = 1; w < 8; ++w) s = f2_add(s, F2{part_sm[w][m][threadIdx.x].x, part_sm[w][m][threadIdx.x].y});
+                put(s, m, 9 * gi + threadIdx.x, sh);
+            }
+        }
+    }
+    for (;;) {
+        int w = 0;
+        if (lane == 0) w = atomicAdd(&next, 1);
+        w = __shfl_sync(0xffffffffu, w, 0);
+        if (w >= n_w) break;
+        const bool lng = w < ks.y;                     // uniform over the warp
+        const int t = lng ? 0 : (w - ks.y) * 32 + lane;
+        const int gi = lng ? w : ks.y + t / 9, bg = lng ? lane % 9 : t % 9;
+        const bool act = gi < n_g && (!lng || lane < 27);
+        const int4 g = act ? __ldg(k_grp + ks.x + gi) : make_int4(0, 0, 0, 0);
+        if (lng && __shfl_sync(0xffffffffu, g.y - g.x, 0) > kYAll) continue;       // (done above)
+        const int sh = kk + __ldg(kx + g.z);
+        blocks(acc, g.x + (lng ? lane / 9 : 0), g.y, lng ? 3 : 1, bg);
+        if (lng) lanes3(acc);
+        if (act && !(lng && lane >= 9))
+#pragma unroll
+            for (int m = 0; m < MT; ++m) put(acc[m], m, 9 * gi + bg, sh);
     }
 #pragma unroll
     for (int m = 0; m < MT; ++m) {
-        const float v = put ? ldexpf(__fadd_rn(acc[m].h, acc[m].l), -ks) : 0.0f;
-        if (put && m0 + m < nm) out[(size_t)(m0 + m) * 9 * n_groups + 9 * gi + bg] = v;
-        const unsigned t1 = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(v)));
+        const unsigned t1 = __reduce_max_sync(0xffffffffu, top[m]);
         if (lane == 0) top_sm[threadIdx.x >> 5][m] = t1;
     }
     __syncthreads();
-    if (threadIdx.x < MT && m0 + (int)threadIdx.x < nm) {
+    int ex[MT];
+#pragma unroll
+    for (int m = 0; m < MT; ++m) {
         unsigned t1 = 0;
-        for (int w = 0; w < 8; ++w) t1 = max(t1, top_sm[w][threadIdx.x]);
-        atomicMax(ymax + mu0 + m0 + threadIdx.x, t1);
-    }
-}
-
-// The rows c = 3 k .. 3 k + 2 of the scaled Y of up to kYStoreModes modes, hi/lo planes
-// (plane stride plane_elems): CTA = (k, modes), its groups (place in `order`, j) at
-// k_at[k_start[k]] ..
-//
-// Bound: the writes, 80 MB per batch of 34 modes of 768 branches in 18 us.  Whole rows,
-// assembled in shared memory, zeros and all: storing the entries where they belong, two
-// bytes each, made the memory fetch and write back a 32-byte sector for every three of
-// them (30 us from a cold cache where this takes 22).
-constexpr int kYStoreModes = 4, kYStoreCols = 768;
-__global__ void __launch_bounds__(256)
-y_store_kernel(int n_groups, const int *__restrict__ k_start, const int2 *__restrict__ k_at,
-               const float *__restrict__ y, int mu0, int nm, int ld, size_t plane_elems, Scales sc,
-               __half *__restrict__ hi, __half *__restrict__ lo) {
-    __shared__ __align__(16) __half row[kYStoreModes][2][3][kYStoreCols];
-    const int k = blockIdx.x, m0 = blockIdx.y * kYStoreModes, n_m = min(kYStoreModes, nm - m0);
-    const int s0 = k_start[k], n_e = 9 * (k_start[k + 1] - s0);
-    int sh[kYStoreModes];
-#pragma unroll
-    for (int m = 0; m < kYStoreModes; ++m) sh[m] = kYBits - sc.y(mu0 + m0 + min(m, n_m - 1));
-    for (int c0 = 0; c0 < ld; c0 += kYStoreCols) {
-        const int w8 = min(kYStoreCols, ld - c0) / 8;             // (ld is a multiple of 128)
-        __syncthreads();
-        for (int x = threadIdx.x; x < (int)sizeof(row) / 16; x += 256)
-            reinterpret_cast<uint4 *>(row)[x] = make_uint4(0, 0, 0, 0);
-        __syncthreads();
-        for (int x = threadIdx.x; x < n_e; x += 256) {
-            const int p = x / 9, bg = x - 9 * p;
-            const int2 a = __ldg(k_at + s0 + p);
-            const int c = 3 * a.y + bg / 3 - c0;
-            if (c < 0 || c >= kYStoreCols) continue;
-            float v[kYStoreModes];
-#pragma unroll
-            for (int m = 0; m < kYStoreModes; ++m)
-                v[m] = __ldg(y + (size_t)(m0 + min(m, n_m - 1)) * 9 * n_groups + 9 * a.x + bg);
-#pragma unroll
-            for (int m = 0; m < kYStoreModes; ++m) {
-                const float s = ldexpf(v[m], sh[m]);
-                const __half h = __float2half_rn(s);
-                row[m][0][bg % 3][c] = h;
-                row[m][1][bg % 3][c] = __float2half_rn(s - __half2float(h));
-            }
+        for (int w = 0; w < 8; ++w) t1 = max(t1, top_sm[w][m]);
+        frexpf(__uint_as_float(t1), &ex[m]);
+        if (threadIdx.x == 0 && m < n_m) {
+            yk[(size_t)(m0 + m) * gridDim.x + k] = t1 ? ex[m] : kNoRow;
+            if (t1) atomicMax(ymax + mu0 + m0 + m, ex[m]);
         }
-        __syncthreads();
-        for (int x = threadIdx.x; x < n_m * 6 * w8; x += 256) {
-            const int r = x / w8, z = x - r * w8, m = r / 6, pl = r / 3 % 2, g = r % 3;
-            __half *out = (pl ? lo : hi) + (size_t)(m0 + m) * plane_elems + (size_t)(3 * k + g) * ld + c0;
-            reinterpret_cast<uint4 *>(out)[z] = reinterpret_cast<const uint4 *>(row[m][pl][g])[z];
+    }
+    for (int x = threadIdx.x; x < 9 * n_g; x += 256) {
+        const int bg = x % 9;
+        const size_t off = (size_t)(3 * k + bg % 3) * ld + 3 * __ldg(k_grp + ks.x + x / 9).z + bg / 3;
+#pragma unroll
+        for (int m = 0; m < MT; ++m) {
+            if (m >= n_m) break;
+            const float s = ldexpf(val[m * n_val + x], kYBits - ex[m]);
+            const __half h = __float2half_rn(s);
+            const size_t o = (size_t)(m0 + m) * plane_elems + off;
+            hi[o] = h;
+            lo[o] = __float2half_rn(s - __half2float(h));
         }
     }
 }
+// Shared memory of the Y build for mt modes and at most n_val entries of a k.
+size_t ybuild_smem(int mt, int n_val) { return sizeof(float) * mt * (size_t)n_val; }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
@@ -831,8 +867,9 @@ static int tc_ldm(int nb) { return (nb + 3 + 31) / 32 * 32; }
 static size_t tc_gsym_bytes(size_t n_tiles) { return ws_round(sizeof(double) * kBM * std::max<size_t>(n_tiles, 1)); }
 static int tc_gsym_parts(int nb) { return (nb + kSumModes - 1) / kSumModes; }
 
-// e, h and ymax of the modes, the strengths and the exponents of the atoms.
-static size_t tc_scale_ints(int nb) { return 3 * (size_t)nb + 2 * (size_t)((nb + 2) / 3); }
+// e, h and ymax of the modes, the strengths and the exponents of the atoms, those of the
+// rows of Y of a batch.
+static size_t tc_scale_ints(int nb, int mb_max) { return 3 * (size_t)nb + (2 + (size_t)mb_max) * ((nb + 2) / 3); }
 
 size_t tc_gamma_scratch_bytes(int nb, int mb_max, size_t n_fc3, int sym3, size_t n_tiles) {
     const int ld = (nb + kBN - 1) / kBN * kBN;     // whole 128-column tiles per row
@@ -842,7 +879,7 @@ size_t tc_gamma_scratch_bytes(int nb, int mb_max, size_t n_fc3, int sym3, size_t
     // then the FP32 pairs of Phi3 and of the eigenvectors and the scales, then (Phi3 symmetric under
     // every permutation) the tiles' sums and the modes' sums
     return (2 + 4 * (size_t)mb_max) * plane + ws_round(sizeof(float2) * 27 * std::max<size_t>(n_fc3, 1)) +
-           ws_round(sizeof(float2) * (size_t)nb * tc_ldm(nb)) + ws_round(sizeof(int) * tc_scale_ints(nb)) +
+           ws_round(sizeof(float2) * (size_t)nb * tc_ldm(nb)) + ws_round(sizeof(int) * tc_scale_ints(nb, mb_max)) +
            (sym3 ? 2 * tc_gsym_bytes(n_tiles) + ws_round(sizeof(double) * (size_t)nb * (1 + tc_gsym_parts(nb))) : 0);
 }
 
@@ -873,7 +910,7 @@ cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const L
     float2 *fc3p = reinterpret_cast<float2 *>(pairs);
     float2 *Et = reinterpret_cast<float2 *>(pairs + ws_round(sizeof(float2) * 27 * std::max<size_t>(gp.n_fc3, 1)));
     char *sums = reinterpret_cast<char *>(Et) + ws_round(sizeof(float2) * (size_t)nb * ldm);
-    char *gsums = sums + ws_round(sizeof(int) * tc_scale_ints(nb));
+    char *gsums = sums + ws_round(sizeof(int) * tc_scale_ints(nb, gp.mb_max));
     double *rowp = nullptr, *colp = nullptr, *gacc = nullptr;
     // tile_start follows the tiles (same allocation)
     int *ts = reinterpret_cast<int *>(tiles_dev + std::max<size_t>(tiles.size(), 1));
@@ -892,7 +929,8 @@ cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const L
     const int n_at = nb / 3;
     int *em = reinterpret_cast<int *>(sums), *hm = em + nb, *ymax = hm + nb, *kx = ymax + nb;
     unsigned *strength = reinterpret_cast<unsigned *>(kx + n_at);
-    e = cudaMemsetAsync(ymax, 0, sizeof(int) * (size_t)nb, st);
+    int *yk = reinterpret_cast<int *>(strength + n_at);
+    e = cudaMemsetAsync(ymax, 0x80, sizeof(int) * (size_t)nb, st);          // (no element yet)
     if (e == cudaSuccess) e = cudaMemsetAsync(strength, 0, sizeof(int) * (size_t)n_at, st);
     if (e != cudaSuccess) return e;
     if (gp.n_groups)
@@ -903,6 +941,7 @@ cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const L
     int hR = 0;
     while ((1LL << (2 * hR)) < gp.row_entries) ++hR;
     const Scales sc{em, hm, ymax, hR};
+    const int n_val = 3 * gp.row_entries;          // entries of the three rows of one k
     split_kernel<<<counted(4096), 256, 0, st>>>(nb, reinterpret_cast<const double2 *>(d.eig), kx, em, ld, Eh, El);
     // the planes of one stack are contiguous: plane_elems = plane / 2 elements apart
     const size_t plane_elems = plane / sizeof(__half);
@@ -933,28 +972,26 @@ cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const L
         const int nm = std::min(mb, nb - mu0);
         const int t0 = tile_start[mu0], t1 = tile_start[mu0 + nm];
         if (t1 == t0) continue;                     // no delta-band tile (masked modes)
-        // the entries of Y stand in the T planes before they are scaled (9 n_groups <=
-        // nb^2 FP32 values per mode there, and the first contraction writes every tile
-        // that the second reads)
-        float *yf = reinterpret_cast<float *>(Th);
-        const long long yth = 32LL * gp.n_long + 9LL * (gp.n_groups - gp.n_long);
-        const unsigned ygx = (unsigned)((yth + 255) / 256);
         auto ybuild = [&](auto kern, int mt) {
-            kern<<<counted(dim3(ygx, (nm + mt - 1) / mt)), 256, 0, st>>>(gp.n_groups, gp.n_long, d.group_order,
-                                                                         d.group_jk, d.group_start, d.blk_i, fc3p, Et,
-                                                                         ldm, mu0, nm, kx, yf,
-                                                                         reinterpret_cast<unsigned *>(ymax));
+            const size_t smem = ybuild_smem(mt, n_val);
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e == cudaSuccess)
+                kern<<<counted(dim3(n_at, (nm + mt - 1) / mt)), 256, smem, st>>>(d.k_start, d.k_grp, d.blk_i, fc3p, Et, ldm,
+                                                                               mu0, nm, kx, ld, plane_elems, n_val, Yh,
+                                                                               Yl, yk, ymax);
         };
-        // modes per thread: 4, or 3 where that leaves fewer of them unused
-        if (nm == 1) ybuild(ybuild_pair_kernel<1>, 1);
-        else if (nm == 2) ybuild(ybuild_pair_kernel<2>, 2);
-        else if ((nm + 2) / 3 * 3 < (nm + 3) / 4 * 4) ybuild(ybuild_pair_kernel<3>, 3);
-        else ybuild(ybuild_pair_kernel<4>, 4);
-        y_store_kernel<<<counted(dim3(n_at, (nm + kYStoreModes - 1) / kYStoreModes)), 256, 0, st>>>(
-            gp.n_groups, d.k_start, d.k_at, yf, mu0, nm, ld, plane_elems, sc, Yh, Yl);
+        // modes per CTA: 4, or 3 where that leaves fewer of them unused, and fewer where
+        // their entries do not fit
+        int mt = nm < 3 ? nm : (nm + 2) / 3 * 3 < (nm + 3) / 4 * 4 ? 3 : 4;
+        while (mt > 1 && ybuild_smem(mt, n_val) > (size_t)96 << 10) --mt;
+        if (mt == 1) ybuild(ybuild_rows_kernel<1>, 1);
+        else if (mt == 2) ybuild(ybuild_rows_kernel<2>, 2);
+        else if (mt == 3) ybuild(ybuild_rows_kernel<3>, 3);
+        else ybuild(ybuild_rows_kernel<4>, 4);
+        if (e != cudaSuccess) return e;
         // (with sym3 the tiles of a mode start at its own row tile)
         const int tm0 = gp.sym3 ? mu0 / kBM : 0;
-        EpiSplit es{Th, Tl, ld, prow, tm0};
+        EpiSplit es{Th, Tl, ld, prow, tm0, mu0, yk};
         EpiGamma eg{};
         ProfMark p1(p.prof, KALD_PROF_TC_GEMM1, st);
         k1<<<counted(dim3(nt, nt - tm0, nm)), 128, kSmemBytes, st>>>(mEh, mEl, mYh, mYl, nb, nb, ld, sc, es, eg, err,
@@ -963,7 +1000,7 @@ cudaError_t launch_gamma_only_tc(const GammaPlan &gp, const GammaDev &d, const L
         EpiGamma eg2{d.omega, d.occ, mu0, prow, sig2inv, p.cut_w, p.shape, partial_tc + t0, d.allowed,
                      tiles_dev + t0, symmetric, rowp ? rowp + (size_t)t0 * kBM : nullptr,
                      colp ? colp + (size_t)t0 * kBM : nullptr};
-        EpiSplit es0{nullptr, nullptr, 0, 0, 0};
+        EpiSplit es0{nullptr, nullptr, 0, 0, 0, 0, nullptr};
         ProfMark p2(p.prof, KALD_PROF_TC_GEMM2, st);
         k2<<<counted(t1 - t0), gp.sym3 ? gemm_threads(EPI_GSYM) : 128, kSmemBytes, st>>>(mTh, mTl, mEh, mEl, nb, nb, ld, sc, es0, eg2, err, p.wait_limit);
         p2.end();

@@ -783,3 +783,19 @@ def test_crystal_split_of_unlike_parts(k, log_ratio, phase_sum, monkeypatch):
     ref, got = (np.asarray(kk.kald_linewidths(ctx, s, mesh, nu, eig, opt)[0]).ravel() for s in (alike, unlike))
     assert _rel(got[weak] * 4.0 ** log_ratio, ref[weak]) < 1e-6
     assert _rel(got[~weak], ref[~weak]) < 1e-6
+
+
+@pytest.mark.parametrize("cell,extra", [((3, 3, 1), 12000), ((9, 1, 1), 40000), ((13, 1, 1), 2500)])
+def test_gamma_only_y_build_of_dense_cells(k, cell, extra):
+    """Atom pairs of 1 to some 45 blocks each, all pairs of the cell in use: outputs of a
+    lane, of three lanes of a warp and of all warps of a CTA in one set of rows (108 and
+    156 modes; a Phi3 without symmetry)."""
+    kk, ctx = k
+    s = ki.random_fc3_system(ki.fcc_supercell_system(cell, seed=5), extra, seed=3)
+    nu, eig = ph.phonons(s, (1, 1, 1))
+    out = {}
+    for prec in ("fp64", "bf16split"):
+        opt = kk.Options(temperature_K=300.0, sigma_thz=0.1, precision=prec)
+        out[prec] = kk.kald_linewidths(ctx, [s], (1, 1, 1), nu.ravel(), eig.ravel(), opt)
+    assert abs(out["fp64"][1][1] - out["bf16split"][1][1]) <= 1e-5 * out["fp64"][1][1]
+    assert _rel(out["bf16split"][0], out["fp64"][0]) < 1e-5
