@@ -9,8 +9,9 @@
 // error of gamma from that, 1e-5 for the smallest cells, grows when each triple of
 // modes is projected once instead of three times).  FP16's narrow range is met by
 // powers of two (Scales): each atom by how strongly Phi3 holds it, each mode's
-// eigenvector by its largest component, Y_mu by its largest element as built, T by
-// the norms of its two factors; the epilogues take them out exactly.
+// eigenvector by its largest component, the rows of Y_mu of one atom by their largest
+// element as built, T by the norms of its two factors; the epilogues take them out
+// exactly.
 //
 // Several modes go through each launch (a batch of MB modes, so that small
 // systems still fill the GPU): the Y and T planes of the batch are stacked
